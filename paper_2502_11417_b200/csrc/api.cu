@@ -403,7 +403,24 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     // ---- per class: 32-bit range proof and histogram windows of the regular TBTs
     const HostReadback& rb = *c->rb;
     const int64_t n_max = rb.max_n;
-    for (ClassConst& cc : classes) {
+    std::vector<char> paced(classes.size());       // no interval of any stream can exceed the pace tau
+    std::vector<uint32_t> search(classes.size());  // ... then: tokens the search for the hand-off may look at
+    for (size_t k = 0; k < classes.size(); ++k) {
+        ClassConst& cc = classes[k];
+        bool never_clamps = cc.pacing != 0;
+        for (int g = 0; g < G; ++g)
+            never_clamps = never_clamps && (int64_t)c->gc[g].T_srv + c->gc[g].J_srv <= cc.tau &&
+                           (int64_t)c->gc[g].T_dev + c->gc[g].J_dev <= cc.tau;
+        paced[k] = never_clamps;
+        for (int g = 0; g < G && never_clamps; ++g) {
+            const GroupConst& gc = c->gc[g];
+            const int64_t gain = cc.tau - (gc.candidate == 2 ? (int64_t)gc.T_dev + gc.J_dev : (int64_t)gc.T_srv + gc.J_srv);
+            const int64_t fill = (int64_t)std::max(cc.B - 1, 0) * cc.tau;
+            int64_t need = gain > 0 ? fill / gain + 1 : (int64_t)kMaxOutput;
+            if (cc.B == 0 || !cc.mig_any || gc.candidate == 0) need = 1;       // nothing to search for
+            cc.search[g] = (uint32_t)std::min<int64_t>(need, kMaxOutput);
+            if (rb.ng[g]) search[k] = std::max(search[k], cc.search[g]);
+        }
         int Wmax[3] = {1, 1, 1};
         for (int g = 0; g < G; ++g) {
             const GroupConst& gc = c->gc[g];
@@ -426,6 +443,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             }
         }
         for (int k = 0; k < 3; ++k) cc.W[k] = Wmax[k];
+        if (never_clamps) continue;                // its windows are not stored
         const size_t win_bytes = (size_t)n * (Wmax[0] + Wmax[1] + Wmax[2]) * 4;
         if (win_bytes > (48ull << 30)) return fail(DISCO_ENOMEM, "per-request TBT windows would exceed 48 GB");
     }
@@ -434,7 +452,12 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     cudaError_t e;
     const size_t N1 = n ? n : 1;
     size_t wmax[3] = {1, 1, 1};
-    for (const ClassConst& cc : classes) for (int k = 0; k < 3; ++k) wmax[k] = std::max<size_t>(wmax[k], cc.W[k]);
+    bool stored = false;                  // some class stores sums, maxima and windows
+    for (size_t k = 0; k < classes.size(); ++k) {
+        if (paced[k]) continue;
+        stored = true;
+        for (int s = 0; s < 3; ++s) wmax[s] = std::max<size_t>(wmax[s], classes[k].W[s]);
+    }
 #define R(buf, bytes) if ((e = c->buf.reserve(bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation")
     R(d_prep, (size_t)G * P * sizeof(Prep));
     const size_t acc_bytes = (size_t)P * G * kNAcc * 8, hist_bytes = (size_t)P * kNBins * 8;
@@ -443,13 +466,16 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const size_t cls_cnt_bytes = (classes.size() * 8 + 15) / 16 * 16;
     const size_t cnt_bytes = cls_cnt_bytes + 32 + (classes.size() * 4 + 15) / 16 * 16;
     R(d_accum, acc_bytes + 2 * hist_bytes + cnt_bytes);
-    R(d_todo, N1 * 4);
     c->d_acc.p = c->d_accum.p; c->d_hist_ttft.p = (char*)c->d_accum.p + acc_bytes;
     c->d_hist_tbt.p = (char*)c->d_accum.p + acc_bytes + hist_bytes;
     R(d_stats, P * sizeof(disco_policy_stats_t) + 16);
-    for (int k = 0; k < 7; ++k) R(rec_u32[k], N1 * 4);
+    R(rec_u32[6], N1 * 4);
     for (int k = 0; k < 2; ++k) R(rec_u16[k], N1 * 2);
-    for (int k = 0; k < 3; ++k) R(rec_win[k], N1 * wmax[k] * 4);
+    if (stored) {
+        R(d_todo, N1 * 4);
+        for (int k = 0; k < 6; ++k) R(rec_u32[k], N1 * 4);
+        for (int k = 0; k < 3; ++k) R(rec_win[k], N1 * wmax[k] * 4);
+    }
 
     if (c->fin_imported) {            // an import replaced the totals the final reductions refer to: back to the trace's own
         c->fin_own.assign((size_t)2 * G, 0);
@@ -595,12 +621,10 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         const ClassConst* dcc = c->d_classes.as<ClassConst>() + k;
         if (timed) CU(cudaEventRecord(c->ev[0], st));
         // with pacing on, a stream whose slowest interval T + J is within tau never falls behind its reader
-        bool never_clamps = classes[k].pacing != 0;
-        for (int g = 0; g < G; ++g)
-            never_clamps = never_clamps && (int64_t)c->gc[g].T_srv + c->gc[g].J_srv <= classes[k].tau &&
-                           (int64_t)c->gc[g].T_dev + c->gc[g].J_dev <= classes[k].tau;
+        const bool never_clamps = paced[k] != 0;
+        rec.tau = never_clamps ? (uint32_t)classes[k].tau : 0u;
         CU(launch_timeline(tr, c->d_gc.as<GroupConst>(), dcc, classes[k].pacing != 0, c->knots.as<int32_t>(), k0, rec,
-                           c->err, c->d_todo.as<uint32_t>(), todo_counts + 2 * k, never_clamps, long_outputs,
+                           c->err, c->d_todo.as<uint32_t>(), todo_counts + 2 * k, never_clamps, search[k], long_outputs,
                            timed ? c->ev[1] : nullptr, c->sms, st));
         if (timed) CU(cudaEventRecord(c->ev[2], st));
         CU(launch_pairs(tr, c->d_gc.as<GroupConst>(), dcc, c->d_prep.as<Prep>(), P,

@@ -63,10 +63,16 @@ struct ClassConst {
     int32_t W[3];                // bins per request for the server, device and migrated timelines
     int32_t lo[kMaxGroups][3];   // first bin of each window, per group
     int32_t ktau[kMaxGroups][3]; // index of bin(tau) inside the window, or -1
+    // Tokens the search for the hand-off may have to look at, per group, when no interval can exceed tau: every
+    // token then adds at least tau - (T + J) to the delivery lag, so (B-1) tau is passed within that many tokens.
+    uint32_t search[kMaxGroups];
 };
 
 // Per-request summaries of the up to three distinct decode timelines of a class.
 struct TimelineRec {
+    uint32_t tau;                // not 0: every stream is delivered at this pace (no interval can exceed it), and sums, maxima
+                                 // and windows are not stored: they follow from the lengths, m and the stall
+
     uint32_t *sum[3], *max[3];   // d_n - d_1 and the largest TBT, ticks ([n] each)
     uint32_t* stall;             // TBT of the first token after a hand-off
     uint16_t *m, *delayed;       // hand-off index (0 = buffer never fills) and delayed tokens
@@ -202,6 +208,7 @@ cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const Clas
                             TimelineRec rec, int32_t* err, uint32_t* todo,
                             uint32_t* todo_count /* two words, zero on entry: length of the list, batch tickets */,
                             bool never_clamps /* pacing on and tau >= T + J for both endpoints of every group */,
+                            uint32_t search /* then: largest ClassConst::search of a group with requests */,
                             bool long_outputs /* mean output length of 512 tokens or more */,
                             cudaEvent_t mid /* recorded between its two kernels, or null */,
                             int sms /* multiprocessors of the device */, cudaStream_t st);

@@ -173,9 +173,14 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
         Raw q;
         q.l = tr.l[kk]; q.n = tr.nout[kk]; q.S = (uint32_t)tr.S[kk];
         q.m = rec.m[kk]; q.dly = rec.delayed[kk]; q.stall = rec.stall[kk];
-        q.nt0 = kt0 >= 0 ? rec.win[0][(size_t)kk * W0 + kt0] : 0u;
-        q.nt1 = kt1 >= 0 ? rec.win[1][(size_t)kk * W1 + kt1] : 0u;
-        q.nt2 = kt2 >= 0 ? rec.win[2][(size_t)kk * W2 + kt2] : 0u;
+        if (rec.tau) {                                           // every interval but a hand-off's equals tau
+            q.nt0 = q.nt1 = q.n - 1;
+            q.nt2 = q.m ? q.n - 2 : 0u;
+        } else {
+            q.nt0 = kt0 >= 0 ? rec.win[0][(size_t)kk * W0 + kt0] : 0u;
+            q.nt1 = kt1 >= 0 ? rec.win[1][(size_t)kk * W1 + kt1] : 0u;
+            q.nt2 = kt2 >= 0 ? rec.win[2][(size_t)kk * W2 + kt2] : 0u;
+        }
         q.orig = EXT ? tr.orig[kk] : 0u;
         return q;
     };
@@ -545,7 +550,18 @@ k_pairs_rows(TraceDev tr, const GroupConst* __restrict__ gcs, const Prep* __rest
         const float inv_cnt = q.n > 1 ? 1e-6f / (float)(q.n - 1) : 0.0f;
         float mean[3], mx[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) { mean[c] = (float)rec.sum[c][k] * inv_cnt; mx[c] = (float)rec.max[c][k] * 1e-6f; }
+        for (int c = 0; c < 3; ++c) {
+            uint32_t sum, most;
+            if (rec.tau) {                            // every interval equals tau, but the one after a hand-off (stream 2)
+                const uint32_t nI = q.n - 1;
+                const uint32_t stall = (c == 2 && q.m) ? rec.stall[k] : 0u;
+                sum = c < 2 ? nI * rec.tau : (q.m ? (nI - 1) * rec.tau + stall : 0u);
+                most = c < 2 ? (nI ? rec.tau : 0u) : stall;
+            } else {
+                sum = rec.sum[c][k]; most = rec.max[c][k];
+            }
+            mean[c] = (float)sum * inv_cnt; mx[c] = (float)most * 1e-6f;
+        }
         const uint32_t l = q.l, n = q.n, m = q.m, lm = l + m;
         auto put = [&](int oc, uint32_t pre_srv, uint32_t pre_dev, uint32_t tok_dev, int stream) {
             const uint32_t tok_srv = n - tok_dev;

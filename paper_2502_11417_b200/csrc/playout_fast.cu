@@ -88,12 +88,14 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
         // ---- one request per lane: inputs
         const uint32_t kk = batch0 + lane;
         const bool live = lane < rpw && kk < tr.n;
-        uint32_t n_l = 1, l_l = 1, key_l = 0;
+        uint32_t n_l = 1, l_l = 1, key_l = 0, nI_l = 0;          // nI_l: tokens to draw
         int g_l = 0;
         if (live) {
             n_l = tr.nout[kk]; l_l = tr.l[kk];
             key_l = mix32(k0 + tr.orig[kk] * kHashReq);
             while (g_l + 1 < tr.n_groups && kk >= tr.grp_off[g_l + 1]) ++g_l;
+            nI_l = n_l - 1;
+            if (LEAN && DBG_OK(g_l, kMaxGroups, DBG_K_PLAYOUT_FAST, DBG_GROUP)) nI_l = min(nI_l, cc.search[g_l]);
         }
         // ---- one request per lane: results (bit 31 of o_md: played here; bits 0-15 m, 16-30 late tokens)
         uint32_t o_md = 0, o_stall = 0;
@@ -104,7 +106,7 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
             //      a lane is valid; the rounding only moves load.  Every group of PER lanes holds the same
             //      PER values here, lane s of a group standing for request r0 + s.
             const int r0 = it * PER, s8 = lane & (PER - 1);
-            const uint32_t nI_s = __shfl_sync(FULL, n_l, r0 + s8) - 1;
+            const uint32_t nI_s = __shfl_sync(FULL, nI_l, r0 + s8);
             uint32_t inc = nI_s;
 #pragma unroll
             for (int off = 1; off < PER; off <<= 1) {
@@ -139,7 +141,8 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
                 G.cand = mig_any ? gc.candidate : 0;
                 G.K = knots + g * kNKnots;
             }
-            const uint32_t nI = tot ? n - 1 : 0u;                      // inter-token intervals, tokens 2..n
+            const uint32_t nI_r = __shfl_sync(FULL, nI_l, r);
+            const uint32_t nI = tot ? nI_r : 0u;                       // tokens to draw, from token 2 on
             // tokens per lane, ceil(nI / lanes) or one more (lanes >= 1 here); all that matters is lanes * L >= nI
             uint32_t L = __float2uint_ru(__fdividef((float)nI, (float)lanes));
             if (L * (uint32_t)lanes < nI) ++L;
@@ -276,10 +279,11 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
         if (live && (o_md >> 31) && DBG_OK(kk, tr.n, DBG_K_PLAYOUT_FAST, DBG_REQUEST) &&
             DBG_OK(g_l, kMaxGroups, DBG_K_PLAYOUT_FAST, DBG_GROUP)) {
             const uint32_t nI = n_l - 1, ut = (uint32_t)tau, m = o_md & 0xFFFFu, dl = (o_md >> 16) & 0x7FFFu;
+            rec.stall[kk] = m ? o_stall : 0u; rec.m[kk] = (uint16_t)m; rec.delayed[kk] = (uint16_t)(m ? dl : 0u);
+            if (LEAN) continue;                                        // the rest follows from these (TimelineRec::tau)
             rec.sum[0][kk] = nI * ut; rec.max[0][kk] = nI ? ut : 0u;
             rec.sum[1][kk] = nI * ut; rec.max[1][kk] = nI ? ut : 0u;
             rec.sum[2][kk] = m ? (nI - 1) * ut + o_stall : 0u; rec.max[2][kk] = m ? o_stall : 0u;
-            rec.stall[kk] = m ? o_stall : 0u; rec.m[kk] = (uint16_t)m; rec.delayed[kk] = (uint16_t)(m ? dl : 0u);
             const int kt0 = cc.ktau[g_l][0], kt1 = cc.ktau[g_l][1], kt2 = cc.ktau[g_l][2];
             for (int i = 0; i < W0; ++i) rec.win[0][(size_t)kk * W0 + i] = i == kt0 ? nI : 0u;
             for (int i = 0; i < W1; ++i) rec.win[1][(size_t)kk * W1 + i] = i == kt1 ? nI : 0u;
@@ -288,14 +292,100 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
     }
 }
 
+// The same for classes whose buffer fills within a few tokens and whose streams cannot clamp (the host has checked
+// that tau >= T + J everywhere and that no group's search looks at more than kShortSearch tokens): a thread plays a
+// request.  It draws the candidate's tokens until their lag passes (B-1) tau, then, after a hand-off that stalls, the
+// target's tokens until the lag is made up; no later token can change anything.
+constexpr uint32_t kShortSearch = 64;
+constexpr int kShortThreads = 256;
+
+struct ShortGroup {                      // a group under the class
+    uint32_t mulC, mulT;                 // candidate's and target's jitter ranges
+    int32_t cC, cT;                      // c = base - ((h * mul) >> 32)
+    uint32_t kappa, c0;
+    int cand;
+    uint32_t end;                        // where the group's requests end
+};
+
+__global__ void __launch_bounds__(kShortThreads)
+k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
+                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec) {
+    __shared__ ShortGroup groups[kMaxGroups];
+    grid_dependency_wait();
+    const int32_t tau = ccp->tau;
+    const uint32_t B = (uint32_t)ccp->B;
+    const long long thr64 = (long long)(B ? B - 1 : 0) * tau;
+    const int32_t thr = thr64 > 0x7FFFFFFFLL ? 0x7FFFFFFF : (int32_t)thr64;
+    for (int g = threadIdx.x; g < tr.n_groups; g += kShortThreads) {
+        const GroupConst& gc = gcs[g];
+        ShortGroup G;
+        G.cand = ccp->mig_any ? gc.candidate : 0;
+        const uint32_t mulS = 2u * (uint32_t)gc.J_srv + 1u, mulD = 2u * (uint32_t)gc.J_dev + 1u;
+        const int32_t cS = tau - (gc.T_srv - gc.J_srv), cD = tau - (gc.T_dev - gc.J_dev);
+        G.mulC = G.cand == 2 ? mulD : mulS; G.mulT = G.cand == 2 ? mulS : mulD;
+        G.cC = G.cand == 2 ? cD : cS; G.cT = G.cand == 2 ? cS : cD;
+        G.kappa = (uint32_t)gc.kappa; G.c0 = (uint32_t)gc.c0;
+        G.end = tr.grp_off[g + 1];
+        groups[g] = G;
+    }
+    __syncthreads();
+    const uint32_t kk = blockIdx.x * kShortThreads + threadIdx.x;
+    if (kk >= tr.n) return;
+    int g = 0;
+    while (g + 1 < tr.n_groups && kk >= groups[g].end) ++g;
+    const ShortGroup& G = groups[g];
+    const uint32_t n = tr.nout[kk], l = tr.l[kk];
+    uint32_t m = 0, stall = 0, delayed = 0;
+    if (G.cand != 0 && n > 1) {
+        const uint32_t key = mix32(k0 + tr.orig[kk] * kHashReq);
+        int32_t e_m = 0;
+        if (B == 0) m = 1;                                             // nothing to fill: hand off after token 1
+        else {
+            uint32_t hin = key + kHashTok;
+            for (uint32_t j = 2; j < n; ++j) {                         // (the hand-off needs a token left to generate)
+                hin += kHashTok;
+                e_m += G.cC - (int32_t)__umulhi(mix32(hin), G.mulC);
+                if (e_m > thr) { m = j; break; }
+            }
+        }
+        if (m) {
+            uint32_t M;
+            if (G.cand == 1) M = G.kappa * (l + m) + G.c0;             // device re-prefills prompt + m tokens
+            else {
+                const uint32_t u = mix32(key);                         // a server TTFT drawn from F by its knots
+                const uint32_t ki = u >> 24, fr = (u >> 8) & 0xFFFFu;
+                const int32_t* K = knots + g * kNKnots;
+                M = 0;
+                if (DBG_OK(ki + 1, kNKnots, DBG_K_PLAYOUT_FAST, DBG_KNOT))
+                    M = (uint32_t)(K[ki] + (int32_t)(((int64_t)(K[ki + 1] - K[ki]) * (int64_t)fr) >> 16));
+            }
+            const int32_t need = -(e_m + (tau - (int32_t)M));          // how late token m+1 is
+            stall = (uint32_t)tau + (uint32_t)max(need, 0);
+            if (need > 0) {
+                // tokens m+2.. stay late while the target's sum of c from there on is below the lag (c >= 0: a prefix)
+                int32_t run = 0;
+                uint32_t j = m + 2;
+                for (uint32_t hin = key + j * kHashTok; j <= n; ++j, hin += kHashTok) {
+                    run += G.cT - (int32_t)__umulhi(mix32(hin), G.mulT);
+                    if (run >= need) break;
+                }
+                delayed = j - m - 1;                                   // tokens m+1 .. j-1
+            }
+        }
+    }
+    rec.stall[kk] = stall; rec.m[kk] = (uint16_t)m; rec.delayed[kk] = (uint16_t)delayed;
+}
+
 }  // namespace
 
 DBG_TRANSLATION_UNIT()
 
 cudaError_t launch_playout_fast(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const int32_t* knots,
                                 uint32_t k0, TimelineRec rec, uint32_t* todo, uint32_t* todo_count,
-                                bool never_clamps, bool long_outputs, int sms, cudaStream_t st) {
+                                bool never_clamps, uint32_t search, bool long_outputs, int sms, cudaStream_t st) {
     if (tr.n == 0) return cudaSuccess;
+    if (never_clamps && search <= kShortSearch)
+        return launch_after(k_playout_short, (tr.n + kShortThreads - 1) / kShortThreads, kShortThreads, 0, st, tr, gc, cc, knots, k0, rec);
     // requests per ticket: small batches spread the end of the launch evenly; large traces amortise the ticket
     int rpw = 8;
     while (rpw < 32 && (uint64_t)tr.n / (2 * rpw) >= (uint64_t)sms * 48u * 4u) rpw *= 2;
