@@ -11,7 +11,6 @@
 
 #include "disco_internal.cuh"
 #include "load.cuh"
-#include "tile.cuh"
 
 using namespace disco;
 
@@ -98,8 +97,8 @@ struct disco_ctx {
     const void* gc_dev_at = nullptr;
     // trace
     DevBuf in_prompt, in_out, in_ttft, in_sp, in_dp;      // staging of host inputs
-    DevBuf keys_a, keys_b, tmp_idx, tmp_ln, cursors, inv, placed;
-    DevBuf S, l, nout, orig, sorted;
+    DevBuf keys_a, keys_b, tmp_idx, tmp_ln, cursors, inv;
+    DevBuf req, sorted;
     DevBuf zero, cum_mass, ng_exact, grp_off, knots, d_gc;   // `zero`: every table a load must clear, contiguous
     DevBuf fin_totals;                 // [2G] u64: output tokens and requests per group that the accumulators cover
     uint64_t first_index = 0;          // index of request 0 in the whole trace (hash key base)
@@ -121,11 +120,11 @@ struct disco_ctx {
     uint32_t P = 0;
     bool evaluated = false, reduced = false;
     std::vector<PolicyConst> pol;
-    DevBuf d_prep, d_accum, d_stats, d_tables, d_todo, d_left;
+    DevBuf d_prep, d_accum, d_stats, d_tables, d_grid, d_left;
     struct View { void* p = nullptr; template <class T> T* as() const { return (T*)p; } };
     View d_acc, d_hist_ttft, d_hist_tbt, d_work;       // regions of d_accum (cleared by one memset)
-    View d_pol, d_classes, d_pol_list, d_chunks;       // four regions of d_tables (filled by one copy)
-    DevBuf rec_u32[7], rec_u16[2], rec_win[3];
+    View d_pol, d_classes, d_tab, d_slabs, d_chunks, d_pair_chunks;    // regions of d_tables (filled by one copy)
+    DevBuf rec_hand, rec_u32[6], rec_win[3];
     void* stage = nullptr;       // pinned staging for the small host->device tables
     size_t stage_cap = 0;
     cudaEvent_t stage_free = nullptr;
@@ -138,12 +137,11 @@ struct disco_ctx {
     bool timing_valid = false;
 
     ~disco_ctx() {
-        DevBuf* all[] = {&in_prompt, &in_out, &in_ttft, &in_sp, &in_dp, &keys_a, &keys_b, &tmp_idx, &tmp_ln, &cursors, &inv, &placed,
-                         &S, &l, &nout, &orig, &sorted, &zero, &cum_mass, &ng_exact, &grp_off, &knots, &d_gc, &d_prep, &d_accum, &d_stats, &d_tables, &d_todo,
+        DevBuf* all[] = {&in_prompt, &in_out, &in_ttft, &in_sp, &in_dp, &keys_a, &keys_b, &tmp_idx, &tmp_ln, &cursors, &inv,
+                         &req, &sorted, &zero, &cum_mass, &ng_exact, &grp_off, &knots, &d_gc, &d_prep, &d_accum, &d_stats, &d_tables, &d_grid, &rec_hand,
                          &fin_totals, &F_sorted_imp, &F_off_imp, &d_left};
         for (DevBuf* b : all) b->release();
         for (auto& b : rec_u32) b.release();
-        for (auto& b : rec_u16) b.release();
         for (auto& b : rec_win) b.release();
         if (rb) cudaFreeHost(rb);
         if (stage) cudaFreeHost(stage);
@@ -206,8 +204,7 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, bool host_inputs, bool has_s
         if (has_dp) R(in_dp, N);
     }
     R(keys_a, N * 8); R(keys_b, N * 8);
-    R(tmp_ln, N * 4); R(cursors, (size_t)G * (kMaxPrompt + 1) * 4); R(inv, N * 4); R(placed, N * 16);
-    R(S, N * 4); R(l, N * 2); R(nout, N * 2); R(orig, N * 4); R(sorted, N * 4);
+    R(tmp_ln, N * 4); R(cursors, (size_t)G * (kMaxPrompt + 1) * 4); R(inv, N * 4); R(req, N * 16); R(sorted, N * 4);
     // one block for everything a load clears: cnt | grp_sum_n | ng | max_n | err | first radix counter buffer,
     // followed by the second counter buffer
     const size_t cnt_bytes = ((size_t)G * (kMaxPrompt + 1) * 4 + 15) / 16 * 16;
@@ -311,11 +308,10 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         a.prompt = d->prompt_len; a.outlen = d->output_len; a.ttft = d->server_ttft_s;
         a.sp = d->server_profile; a.dp = d->device_profile;
     }
-    a.keys_a = c->keys_a.as<uint64_t>(); a.keys_b = c->keys_b.as<uint64_t>(); a.cursors = c->cursors.as<uint32_t>(); a.inv = c->inv.as<uint32_t>(); a.placed = c->placed.as<uint4>();
+    a.keys_a = c->keys_a.as<uint64_t>(); a.keys_b = c->keys_b.as<uint64_t>(); a.cursors = c->cursors.as<uint32_t>(); a.inv = c->inv.as<uint32_t>(); a.req = c->req.as<uint4>();
     a.l_tmp = c->tmp_ln.as<uint16_t>(); a.n_tmp = c->tmp_ln.as<uint16_t>() + (n ? n : 1);
     a.radix_counts = c->radix_counts; a.zero_block = c->zero.p; a.zero_bytes = c->zero_bytes;
     a.ng_exact = c->ng_exact.as<uint32_t>(); a.readback = c->rb;     // pinned host memory, written by the last kernel
-    a.S = c->S.as<int32_t>(); a.l = c->l.as<uint16_t>(); a.nout = c->nout.as<uint16_t>(); a.orig = c->orig.as<uint32_t>();
     a.sorted = c->sorted.as<int32_t>(); a.cnt = c->cnt; a.cum_mass = c->cum_mass.as<int64_t>();
     a.ng = c->ng; a.grp_off = c->grp_off.as<uint32_t>(); a.knots = c->knots.as<int32_t>();
     a.grp_sum_n = c->grp_sum_n; a.max_n = c->max_n; a.err = c->err;
@@ -361,7 +357,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     std::vector<PolicyConst> pc(P);
     std::vector<ClassConst> classes;
     bool any_beta = false;                // some policy uses the Eq. 1-2 wait rule
-    bool cls_extras_pending = false;      // some policy routes at random or triggers on an expected length
+    bool extras = false;                  // some policy routes at random or triggers on an expected length
     for (uint32_t p = 0; p < P; ++p) {
         const disco_policy_t& q = pol[p];
         auto at = [p] { return " (policy " + std::to_string(p) + ")"; };
@@ -386,7 +382,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         if (q.flags & DISCO_FLAG_BETA_RULE) any_beta = true;
         o.route_all = q.budget >= 1.0f ? 1 : 0;
         o.route_thr = o.route_all ? 0xFFFFFFFFu : (uint32_t)std::floor((double)q.budget * 4294967296.0);
-        if ((q.flags & (DISCO_FLAG_STOCHASTIC | DISCO_FLAG_BETA_RULE)) || q.expected_len) cls_extras_pending = true;
+        if ((q.flags & (DISCO_FLAG_STOCHASTIC | DISCO_FLAG_BETA_RULE)) || q.expected_len) extras = true;
         int cls = -1;
         for (size_t k = 0; k < classes.size(); ++k)
             if (classes[k].tau == o.tau && classes[k].B == o.B && classes[k].pacing == (int)pacing) { cls = (int)k; break; }
@@ -400,27 +396,16 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         classes[cls].mig_any |= mig ? 1 : 0;
         o.cls = cls;
     }
-    // ---- per class: 32-bit range proof and histogram windows of the regular TBTs
+    // ---- per class: 32-bit range proof, how each group's streams behave, histogram windows of the regular TBTs
     const HostReadback& rb = *c->rb;
     const int64_t n_max = rb.max_n;
-    std::vector<char> paced(classes.size());       // no interval of any stream can exceed the pace tau
-    std::vector<uint32_t> search(classes.size());  // ... then: tokens the search for the hand-off may look at
+    struct ClassPlan { uint32_t kinds = 0, batches[3] = {0, 0, 0}, search = 0; };
+    std::vector<ClassPlan> plan(classes.size());
+    size_t wmax[3] = {1, 1, 1};
+    bool stored = false;                  // some class stores sums, maxima and windows
     for (size_t k = 0; k < classes.size(); ++k) {
         ClassConst& cc = classes[k];
-        bool never_clamps = cc.pacing != 0;
-        for (int g = 0; g < G; ++g)
-            never_clamps = never_clamps && (int64_t)c->gc[g].T_srv + c->gc[g].J_srv <= cc.tau &&
-                           (int64_t)c->gc[g].T_dev + c->gc[g].J_dev <= cc.tau;
-        paced[k] = never_clamps;
-        for (int g = 0; g < G && never_clamps; ++g) {
-            const GroupConst& gc = c->gc[g];
-            const int64_t gain = cc.tau - (gc.candidate == 2 ? (int64_t)gc.T_dev + gc.J_dev : (int64_t)gc.T_srv + gc.J_srv);
-            const int64_t fill = (int64_t)std::max(cc.B - 1, 0) * cc.tau;
-            int64_t need = gain > 0 ? fill / gain + 1 : (int64_t)kMaxOutput;
-            if (cc.B == 0 || !cc.mig_any || gc.candidate == 0) need = 1;       // nothing to search for
-            cc.search[g] = (uint32_t)std::min<int64_t>(need, kMaxOutput);
-            if (rb.ng[g]) search[k] = std::max(search[k], cc.search[g]);
-        }
+        ClassPlan& pl = plan[k];
         int Wmax[3] = {1, 1, 1};
         for (int g = 0; g < G; ++g) {
             const GroupConst& gc = c->gc[g];
@@ -431,51 +416,227 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 if ((n_max - 1) * step + Mmax >= (1LL << 31))
                     return fail(DISCO_EINVAL, "a decode stream could outlast 2^31 ticks (about 35 minutes)");
             }
+            // which streams keep the pace at every token, and which wait for every token
+            const int cand = cc.mig_any ? gc.candidate : 0;
+            const bool even_s = cc.pacing && xs <= cc.tau, even_d = cc.pacing && xd <= cc.tau;
+            const bool free_s = gc.T_srv - (int64_t)gc.J_srv >= cc.tau, free_d = gc.T_dev - (int64_t)gc.J_dev >= cc.tau;
+            cc.even[g] = (uint8_t)((even_s ? 1 : 0) | (even_d ? 2 : 0));
+            if (even_s && even_d) { cc.kind[g] = G_EXACT; cc.even[g] = 7; }
+            else if (!cc.pacing) cc.kind[g] = G_FREE;
+            else if ((even_s || free_s) && (even_d || free_d) &&
+                     (cand == 0 || (cc.B > 0 && !(cand == 1 ? even_s : even_d)))) cc.kind[g] = G_FREE;   // (its buffer never fills)
+            else cc.kind[g] = G_GENERAL;
+            if (cc.kind[g] == G_EXACT) {
+                const int64_t gain = cc.tau - (gc.candidate == 2 ? xd : xs), fill = (int64_t)std::max(cc.B - 1, 0) * cc.tau;
+                int64_t need = gain > 0 ? fill / gain + 1 : (int64_t)kMaxOutput;
+                if (cc.B == 0 || cand == 0) need = 1;                         // nothing to search for
+                cc.search[g] = (uint32_t)std::min<int64_t>(need, kMaxOutput);
+            }
+            if (rb.ng[g]) {
+                pl.kinds |= 1u << cc.kind[g];
+                pl.batches[cc.kind[g]] += (rb.ng[g] + 31) / 32;
+                if (cc.kind[g] == G_EXACT) pl.search = std::max(pl.search, cc.search[g]);
+            }
             int64_t lo_v[3], hi_v[3];
             lo_v[0] = cc.pacing ? cc.tau : gc.T_srv - (int64_t)gc.J_srv; hi_v[0] = cc.pacing ? std::max<int64_t>(cc.tau, xs) : xs;
             lo_v[1] = cc.pacing ? cc.tau : gc.T_dev - (int64_t)gc.J_dev; hi_v[1] = cc.pacing ? std::max<int64_t>(cc.tau, xd) : xd;
             lo_v[2] = std::min(lo_v[0], lo_v[1]); hi_v[2] = std::max(hi_v[0], hi_v[1]);
-            for (int k = 0; k < 3; ++k) {
-                const int lo = host_bin_of_ticks(lo_v[k]), hi = host_bin_of_ticks(hi_v[k]);
-                cc.lo[g][k] = lo;
-                cc.ktau[g][k] = cc.pacing ? host_bin_of_ticks(cc.tau) - lo : -1;
-                Wmax[k] = std::max(Wmax[k], hi - lo + 1);
+            for (int s = 0; s < 3; ++s) {
+                const int lo = host_bin_of_ticks(lo_v[s]), hi = host_bin_of_ticks(hi_v[s]);
+                cc.lo[g][s] = lo;
+                cc.ktau[g][s] = cc.pacing ? host_bin_of_ticks(cc.tau) - lo : -1;
+                Wmax[s] = std::max(Wmax[s], hi - lo + 1);
             }
         }
-        for (int k = 0; k < 3; ++k) cc.W[k] = Wmax[k];
-        if (never_clamps) continue;                // its windows are not stored
-        const size_t win_bytes = (size_t)n * (Wmax[0] + Wmax[1] + Wmax[2]) * 4;
-        if (win_bytes > (48ull << 30)) return fail(DISCO_ENOMEM, "per-request TBT windows would exceed 48 GB");
+        for (int s = 0; s < 3; ++s) cc.W[s] = Wmax[s];
+        if (!(pl.kinds & ~(1u << G_EXACT))) continue;                        // nothing but the hand-offs is stored
+        stored = true;
+        for (int s = 0; s < 3; ++s) wmax[s] = std::max<size_t>(wmax[s], Wmax[s]);
+        if ((size_t)n * (Wmax[0] + Wmax[1] + Wmax[2]) * 2 > (48ull << 30))
+            return fail(DISCO_ENOMEM, "per-request TBT windows would exceed 48 GB");
+    }
+
+    // ---- the policies of a class: plain ones form grids of budgets by overheads (grid.cu), at most kGridCols by kGridRows
+    //      to a slab; random routing and the Eq. 1-2 rule go pair by pair
+    std::vector<uint32_t> tab;                     // lists of policy indices, one after the other
+    std::vector<Slab> slabs;
+    std::vector<uint32_t> mixed_pols;              // per slab: where its policies are listed for the pair kernel (mixed slabs)
+    struct ClassLists { size_t all, n_all, ext, n_ext, slab0, slab1; };
+    std::vector<ClassLists> lists(classes.size());
+    bool any_mixed = false, any_pairs = false;
+    for (size_t k = 0; k < classes.size(); ++k) {
+        ClassLists& L = lists[k];
+        L.all = tab.size();
+        for (uint32_t p = 0; p < P; ++p) if (pc[p].cls == (int)k) tab.push_back(p);
+        L.n_all = tab.size() - L.all;
+        auto is_ext = [&](uint32_t p) { return (pc[p].flags & (DISCO_FLAG_STOCHASTIC | DISCO_FLAG_BETA_RULE)) != 0; };
+        L.ext = tab.size();
+        std::vector<uint32_t> plain;
+        for (size_t i = L.all; i < L.all + L.n_all; ++i) { const uint32_t p = tab[i]; if (is_ext(p)) tab.push_back(p); else plain.push_back(p); }
+        L.n_ext = tab.size() - L.ext;
+        any_pairs = any_pairs || L.n_ext != 0;
+        L.slab0 = slabs.size();
+        auto theta_of = [&](uint32_t p) { return (pc[p].flags & DISCO_FLAG_MIGRATION) ? pc[p].theta : 0.0f; };   // (else it does not matter)
+        auto same_grid = [&](uint32_t x, uint32_t y) {
+            return pc[x].flags == pc[y].flags && pc[x].expected_len == pc[y].expected_len && pc[x].alpha == pc[y].alpha;
+        };
+        std::sort(plain.begin(), plain.end(), [&](uint32_t x, uint32_t y) {
+            const PolicyConst &a = pc[x], &b = pc[y];
+            if (a.flags != b.flags) return a.flags < b.flags;
+            if (a.expected_len != b.expected_len) return a.expected_len < b.expected_len;
+            if (a.alpha != b.alpha) return a.alpha < b.alpha;
+            if (a.budget != b.budget) return a.budget < b.budget;
+            const float tx = theta_of(x), ty = theta_of(y);
+            return tx != ty ? tx < ty : x < y;
+        });
+        for (size_t i = 0; i < plain.size();) {
+            size_t end = i;
+            while (end < plain.size() && same_grid(plain[i], plain[end])) ++end;
+            std::vector<float> th;
+            size_t budgets = 0;
+            for (size_t x = i; x < end; ++x) {
+                th.push_back(theta_of(plain[x]));
+                if (x == i || pc[plain[x]].budget != pc[plain[x - 1]].budget) ++budgets;
+            }
+            std::sort(th.begin(), th.end());
+            th.erase(std::unique(th.begin(), th.end()), th.end());
+            auto open = [&](int T, bool mixed) {
+                Slab sl;
+                std::memset(&sl, 0, sizeof sl);
+                sl.T = T; sl.expected_len = pc[plain[i]].expected_len; sl.mixed = mixed ? 1 : 0;
+                sl.mig = (pc[plain[i]].flags & DISCO_FLAG_MIGRATION) ? 1 : 0;
+                return sl;
+            };
+            // closes a slab of the columns `cols` (a policy per row, ~0 for none)
+            auto close = [&](Slab sl, const std::vector<std::vector<uint32_t>>& cols, size_t c0, size_t c1, uint32_t listed) {
+                sl.K = (int32_t)(c1 - c0);
+                sl.cols = (uint32_t)tab.size();
+                for (size_t x = c0; x < c1; ++x)
+                    for (uint32_t p : cols[x]) if (p != 0xFFFFFFFFu) { tab.push_back(p); break; }
+                sl.cells = (uint32_t)tab.size();
+                for (size_t x = c0; x < c1; ++x)
+                    for (uint32_t p : cols[x]) { tab.push_back(p); sl.policies += p != 0xFFFFFFFFu; }
+                slabs.push_back(sl);
+                mixed_pols.push_back(listed);
+            };
+            if (th.size() > 1 && 2 * (end - i) <= budgets * th.size()) {
+                // Most (budget, overhead) combinations are no policy: a column per policy instead, and what the overheads
+                // of a slab's policies do not agree on goes pair by pair.
+                for (size_t x0 = i; x0 < end; x0 += kGridCols) {
+                    const size_t x1 = std::min(end, x0 + (size_t)kGridCols);
+                    Slab sl = open(1, true);
+                    std::vector<std::vector<uint32_t>> cols;
+                    float lo = theta_of(plain[x0]), hi = lo;
+                    const uint32_t listed = (uint32_t)tab.size();
+                    for (size_t x = x0; x < x1; ++x) {
+                        cols.push_back({plain[x]});
+                        tab.push_back(plain[x]);
+                        lo = std::min(lo, theta_of(plain[x])); hi = std::max(hi, theta_of(plain[x]));
+                    }
+                    sl.theta[0] = lo; sl.theta[1] = hi;
+                    close(sl, cols, 0, cols.size(), listed);
+                    any_mixed = any_pairs = true;
+                }
+            } else {
+                for (size_t r0 = 0; r0 < th.size(); r0 += kGridRows) {
+                    const size_t r1 = std::min(th.size(), r0 + (size_t)kGridRows);
+                    Slab sl = open((int)(r1 - r0), false);
+                    for (size_t r = r0; r < r1; ++r) sl.theta[r - r0] = th[r];
+                    // columns in ascending order of budget; a policy given twice takes a further column of its budget
+                    std::vector<std::vector<uint32_t>> cols;
+                    for (size_t x = i; x < end;) {
+                        const size_t c_first = cols.size();
+                        const float b = pc[plain[x]].budget;
+                        for (; x < end && pc[plain[x]].budget == b; ++x) {
+                            const size_t r = std::lower_bound(th.begin(), th.end(), theta_of(plain[x])) - th.begin();
+                            if (r < r0 || r >= r1) continue;
+                            size_t at = c_first;
+                            while (at < cols.size() && cols[at][r - r0] != 0xFFFFFFFFu) ++at;
+                            if (at == cols.size()) cols.push_back(std::vector<uint32_t>(r1 - r0, 0xFFFFFFFFu));
+                            cols[at][r - r0] = plain[x];
+                        }
+                    }
+                    for (size_t c0 = 0; c0 < cols.size(); c0 += kGridCols)
+                        close(sl, cols, c0, std::min(cols.size(), c0 + (size_t)kGridCols), 0u);
+                }
+            }
+            i = end;
+        }
+        L.slab1 = slabs.size();
+    }
+
+    // ---- request chunks, of one group each: of the grid kernel, about three to each block that fits the GPU at once, 256
+    //      requests (one a thread) or more; of the pair kernel, two to a multiprocessor, 2,048 requests or more
+    const uint32_t sms = (uint32_t)c->sms, kMaxChunk = 65280;
+    const size_t N1 = n ? n : 1;
+    bool tall = false;
+    for (const Slab& sl : slabs) tall = tall || sl.T > 1;
+    auto chunk_size = [&](size_t want, uint32_t least) {
+        const size_t ch = ((N1 + want - 1) / want + 255) / 256 * 256;
+        return (uint32_t)std::min<size_t>(std::max<size_t>(ch, least), kMaxChunk);
+    };
+    // the chunks of the groups that Algorithm 1 finds device-constrained come first: Algorithm 2's wait map costs the
+    // grid kernel more sweeps per chunk, and its blocks draw their work in list order, so the items drawn last (when
+    // some blocks already idle) should be the cheap ones
+    auto make_chunks = [&](uint32_t CH) {
+        std::vector<Chunk> v;
+        for (int dear = 1; dear >= 0; --dear)
+            for (int g = 0; g < G; ++g) {
+                if ((c->gc[g].auto_device_constrained != 0) != (dear != 0)) continue;
+                for (uint32_t s = rb.grp_off[g]; s < rb.grp_off[g + 1]; s += CH)
+                    v.push_back({s, std::min(CH, rb.grp_off[g + 1] - s), g, 0});
+            }
+        return v;
+    };
+    const std::vector<Chunk> chunks = make_chunks(chunk_size((size_t)3 * sms * grid_blocks_per_sm(tall ? 2 : 1), 256));
+    std::vector<Chunk> pair_chunks;
+    if (any_pairs) pair_chunks = make_chunks(chunk_size((size_t)2 * sms, 2048));
+
+    // ---- the difference tables of the slabs, laid out batch by batch: a batch's slabs have like numbers of rows and share
+    //      one class; its tables are cleared, filled, added up and then belong to the next batch
+    struct Batch { size_t first, count; int K, T; uint64_t ttft, tbt, sums; };
+    std::vector<std::vector<Batch>> batches(classes.size());
+    uint64_t grid_bytes = 0;
+    auto wide_class = [&](size_t k) { return (plan[k].kinds & ~(1u << G_EXACT)) != 0; };
+    uint32_t n_tickets = (uint32_t)classes.size();
+    for (size_t k = 0; k < classes.size(); ++k) {
+        const uint64_t tbt_word = wide_class(k) ? 8 : 4;
+        for (size_t x = lists[k].slab0; x < lists[k].slab1; ++x) {
+            Slab& sl = slabs[x];
+            auto bytes = [&](const Batch& b) { return b.ttft * 4 + b.tbt * tbt_word + b.sums * 8; };
+            auto rows = [](int T) { return T == 1 ? 1 : T <= 4 ? 4 : 8; };
+            std::vector<Batch>& bs = batches[k];
+            if (bs.empty() || bytes(bs.back()) > (256ull << 20) || rows(bs.back().T) != rows(sl.T) || sl.mixed || slabs[x - 1].mixed)
+                bs.push_back(Batch{x, 0, 1, 1, 0, 0, 0});
+            Batch& b = bs.back();
+            sl.ttft = b.ttft; sl.tbt = b.tbt; sl.sums = b.sums;
+            b.ttft += grid_ttft_words(sl.K); b.tbt += grid_tbt_words(sl.K, sl.T); b.sums += grid_sum_words(sl.K, sl.T, G);
+            ++b.count;
+            b.K = std::max(b.K, sl.K); b.T = std::max(b.T, sl.T);
+            grid_bytes = std::max(grid_bytes, bytes(b) + 64);
+        }
+        n_tickets += (uint32_t)batches[k].size();
     }
 
     // ---- device buffers
     cudaError_t e;
-    const size_t N1 = n ? n : 1;
-    size_t wmax[3] = {1, 1, 1};
-    bool stored = false;                  // some class stores sums, maxima and windows
-    for (size_t k = 0; k < classes.size(); ++k) {
-        if (paced[k]) continue;
-        stored = true;
-        for (int s = 0; s < 3; ++s) wmax[s] = std::max<size_t>(wmax[s], classes[k].W[s]);
-    }
 #define R(buf, bytes) if ((e = c->buf.reserve(bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation")
     R(d_prep, (size_t)G * P * sizeof(Prep));
     const size_t acc_bytes = (size_t)P * G * kNAcc * 8, hist_bytes = (size_t)P * kNBins * 8;
-    // a to-do counter and a ticket counter per class, the work counters of the pair kernels (four words), and a
-    // ticket counter per class for the zone kernel
-    const size_t cls_cnt_bytes = (classes.size() * 8 + 15) / 16 * 16;
-    const size_t cnt_bytes = cls_cnt_bytes + 32 + (classes.size() * 4 + 15) / 16 * 16;
+    const size_t cnt_bytes = 32 + ((size_t)n_tickets * 4 + 15) / 16 * 16;     // four work counters, then the tickets
     R(d_accum, acc_bytes + 2 * hist_bytes + cnt_bytes);
     c->d_acc.p = c->d_accum.p; c->d_hist_ttft.p = (char*)c->d_accum.p + acc_bytes;
     c->d_hist_tbt.p = (char*)c->d_accum.p + acc_bytes + hist_bytes;
+    c->d_work.p = (char*)c->d_accum.p + acc_bytes + 2 * hist_bytes;
+    uint32_t* tickets = (uint32_t*)((char*)c->d_work.p + 32);
     R(d_stats, P * sizeof(disco_policy_stats_t) + 16);
-    R(rec_u32[6], N1 * 4);
-    for (int k = 0; k < 2; ++k) R(rec_u16[k], N1 * 2);
+    R(rec_hand, N1 * 8);
     if (stored) {
-        R(d_todo, N1 * 4);
         for (int k = 0; k < 6; ++k) R(rec_u32[k], N1 * 4);
-        for (int k = 0; k < 3; ++k) R(rec_win[k], N1 * wmax[k] * 4);
+        for (int k = 0; k < 3; ++k) R(rec_win[k], N1 * wmax[k] * 2);
     }
+    R(d_grid, grid_bytes);
+    if (any_mixed) R(d_left, (N1 + kMaxGroups) * 4);
 
     if (c->fin_imported) {            // an import replaced the totals the final reductions refer to: back to the trace's own
         c->fin_own.assign((size_t)2 * G, 0);
@@ -483,77 +644,11 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         CU(cudaMemcpyAsync(c->fin_totals.p, c->fin_own.data(), c->fin_own.size() * 8, cudaMemcpyHostToDevice, st));
         c->fin_imported = false;
     }
-    // the accumulators are cleared while the host lays out the chunks and tables below
     CU(cudaMemsetAsync(c->d_accum.p, 0, acc_bytes + 2 * hist_bytes + cnt_bytes, st));
 
-    // ---- policies grouped by class; request chunks (one group each) sized so that chunks x policy tiles
-    //      fill the GPU about once
-    std::vector<uint32_t> pol_list;
-    std::vector<std::pair<uint32_t, uint32_t>> cls_range;       // [begin, end) in pol_list per class
-    for (size_t k = 0; k < classes.size(); ++k) {
-        const uint32_t b = (uint32_t)pol_list.size();
-        for (uint32_t p = 0; p < P; ++p) if (pc[p].cls == (int)k) pol_list.push_back(p);
-        // Within a class the policies are taken in an order that puts like policies side by side with their budgets
-        // ascending, whatever order the caller gave them in: along such a run Algorithm 3's l_th does not increase
-        // and Algorithm 2's l* does not decrease, which is what the zone-by-zone reduction needs of a tile.
-        std::stable_sort(pol_list.begin() + b, pol_list.end(), [&](uint32_t x, uint32_t y) {
-            const PolicyConst &a = pc[x], &c2 = pc[y];
-            if (a.flags != c2.flags) return a.flags < c2.flags;
-            if (a.expected_len != c2.expected_len) return a.expected_len < c2.expected_len;
-            if (a.l_immediate != c2.l_immediate) return a.l_immediate < c2.l_immediate;
-            if (a.alpha != c2.alpha) return a.alpha < c2.alpha;
-            if (a.theta != c2.theta) return a.theta < c2.theta;
-            return a.budget < c2.budget;
-        });
-        cls_range.push_back({b, (uint32_t)pol_list.size()});
-    }
-    const uint32_t tiles = (P + 31) / 32;
-    // the zone kernel's blocks take (chunk, family of four policy tiles) items; the pair kernel works a chunk in
-    // passes of at most 65,280 requests
-    const uint32_t kMaxChunk = 65280;
-    const uint32_t sms = (uint32_t)c->sms;
-    const uint32_t fams = (tiles + 3) / 4;
-    // about two items a block (the blocks draw them from a counter, so uneven items even out), chunks of 2,048
-    // requests or more
-    uint32_t want_chunks = std::max<uint32_t>(1, (2 * sms + fams - 1) / fams);
-    const uint32_t min_chunks = (uint32_t)((N1 + kMaxChunk - 1) / kMaxChunk);
-    if (min_chunks > want_chunks) {
-        // several waves of blocks: the fewest chunks whose last wave is nearly full (long chunks spread a block's
-        // set-up and flush over more requests), else the count near the minimum whose last wave is fullest
-        double best = 0.0;
-        for (uint32_t k = min_chunks; k < min_chunks + sms; ++k) {
-            const uint64_t blocks = (uint64_t)k * fams, waves = (blocks + sms - 1) / sms;
-            const double fill = (double)blocks / (double)(waves * sms);
-            if (fill > best + 1e-9) { best = fill; want_chunks = k; }
-            if (fill >= 0.94) break;
-        }
-    }
-    uint32_t CH = (uint32_t)((N1 + want_chunks - 1) / want_chunks);
-    CH = (CH + 255) / 256 * 256;
-    CH = std::min<uint32_t>(std::max<uint32_t>(CH, 2048), kMaxChunk);
-    // the chunks of the groups that Algorithm 1 finds device-constrained come first: Algorithm 2's wait map costs the
-    // zone kernel more sweeps per chunk, and its blocks draw their work in list order, so the items drawn last (when
-    // some blocks already idle) should be the cheap ones
-    std::vector<Chunk> chunks;
-    for (int dear = 1; dear >= 0; --dear)
-        for (int g = 0; g < G; ++g) {
-            if ((c->gc[g].auto_device_constrained != 0) != (dear != 0)) continue;
-            for (uint32_t s = rb.grp_off[g]; s < rb.grp_off[g + 1]; s += CH)
-                chunks.push_back({s, std::min(CH, rb.grp_off[g + 1] - s), g, 0});
-        }
-#undef R
-
-    // scratch of the pair kernels: a bit per (request, policy tile), a counter per (chunk, policy tile)
-    const size_t left_mask_words = (size_t)N1 * ((tiles + 31) / 32);
-    // ... and, while that stays below 1 GB, a short list of flagged requests per (chunk, tile)
-    const size_t left_cells = chunks.size() * (size_t)tiles;
-    const size_t left_list_words = left_cells * kLeftList * 4 <= (1ull << 30) ? left_cells * kLeftList : 0;
-    if ((e = c->d_left.reserve((left_mask_words + left_cells + left_list_words + 4) * 4)) != cudaSuccess)
-        return fail_cuda(e, "device allocation for the evaluation");
-
-    // ---- small tables to the device through pinned staging
-    const size_t need = P * sizeof(PolicyConst) + classes.size() * sizeof(ClassConst) + P * 4 +
-                        chunks.size() * sizeof(Chunk) + 64;
+    // ---- small tables to the device through pinned staging: one staging block, one copy (16-byte aligned regions)
+    const size_t need = P * sizeof(PolicyConst) + classes.size() * sizeof(ClassConst) + tab.size() * 4 + slabs.size() * sizeof(Slab) +
+                        (chunks.size() + pair_chunks.size()) * sizeof(Chunk) + 128;
     if (c->stage_free) CU(cudaEventSynchronize(c->stage_free));     // an earlier call's copies may still read it
     else CU(cudaEventCreateWithFlags(&c->stage_free, cudaEventDisableTiming));
     if (need > c->stage_cap) {
@@ -562,32 +657,32 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         CU(cudaMallocHost(&c->stage, need));
         c->stage_cap = need;
     }
-    // one staging block, one copy: policies | classes | policy list | chunks (16-byte aligned regions)
     char* sp = (char*)c->stage;
     size_t off = 0;
     auto put = [&](DevBufView& v, const void* src, size_t bytes) {
-        std::memcpy(sp + off, src, bytes);
+        if (bytes) std::memcpy(sp + off, src, bytes);
         v.off = off;
         off += (bytes + 15) / 16 * 16;
     };
-    DevBufView v_pol, v_cls, v_list, v_chunks;
+    DevBufView v_pol, v_cls, v_tab, v_slabs, v_chunks, v_pair;
     put(v_pol, pc.data(), P * sizeof(PolicyConst));
     put(v_cls, classes.data(), classes.size() * sizeof(ClassConst));
-    put(v_list, pol_list.data(), P * 4);
+    put(v_tab, tab.data(), tab.size() * 4);
+    put(v_slabs, slabs.data(), slabs.size() * sizeof(Slab));
     put(v_chunks, chunks.data(), chunks.size() * sizeof(Chunk));
+    put(v_pair, pair_chunks.data(), pair_chunks.size() * sizeof(Chunk));
     if ((e = c->d_tables.reserve(off + 16)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
+#undef R
     char* dt = (char*)c->d_tables.p;
-    c->d_pol.p = dt + v_pol.off; c->d_classes.p = dt + v_cls.off; c->d_pol_list.p = dt + v_list.off;
-    c->d_chunks.p = dt + v_chunks.off;
+    c->d_pol.p = dt + v_pol.off; c->d_classes.p = dt + v_cls.off; c->d_tab.p = dt + v_tab.off; c->d_slabs.p = dt + v_slabs.off;
+    c->d_chunks.p = dt + v_chunks.off; c->d_pair_chunks.p = dt + v_pair.off;
     CU(cudaMemcpyAsync(dt, sp, off, cudaMemcpyHostToDevice, st));
     CU(cudaEventRecord(c->stage_free, st));
-
-    uint32_t* todo_counts = (uint32_t*)((char*)c->d_accum.p + acc_bytes + 2 * hist_bytes);
-    c->d_work.p = (char*)c->d_accum.p + acc_bytes + 2 * hist_bytes + cls_cnt_bytes;
 
     // ---- Algorithms 1-3 for every (group, policy)
     CU(launch_prep(c->d_pol.as<PolicyConst>(), P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
                    c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), st));
+    g_launches += 1;
     if (any_beta) {
         CU(launch_prep_beta(c->d_pol.as<PolicyConst>(), P, G, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
                             c->F_off, c->d_prep.as<Prep>(), st));
@@ -595,51 +690,82 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     }
 
     TraceDev tr;
-    tr.n = n; tr.n_groups = G; tr.S = c->S.as<int32_t>(); tr.l = c->l.as<uint16_t>(); tr.nout = c->nout.as<uint16_t>();
-    tr.orig = c->orig.as<uint32_t>(); tr.inv = c->inv.as<uint32_t>(); tr.len_end = c->cursors.as<uint32_t>(); tr.grp_off = c->grp_off.as<uint32_t>();
+    tr.n = n; tr.n_groups = G; tr.req = c->req.as<uint4>(); tr.inv = c->inv.as<uint32_t>();
+    tr.len_end = c->cursors.as<uint32_t>(); tr.grp_off = c->grp_off.as<uint32_t>();
     TimelineRec rec;
+    rec.hand = c->rec_hand.as<uint2>();
     for (int k = 0; k < 3; ++k) {
         rec.sum[k] = c->rec_u32[2 * k].as<uint32_t>(); rec.max[k] = c->rec_u32[2 * k + 1].as<uint32_t>();
-        rec.win[k] = c->rec_win[k].as<uint32_t>();
+        rec.win[k] = c->rec_win[k].as<uint16_t>();
     }
-    rec.stall = c->rec_u32[6].as<uint32_t>();
-    rec.m = c->rec_u16[0].as<uint16_t>(); rec.delayed = c->rec_u16[1].as<uint16_t>();
     disco_pair_out_t po;
     std::memset(&po, 0, sizeof po);
     if (out) po = *out;
+    const bool rows = po.ttft_s || po.tbt_mean_s || po.tbt_max_s || po.cost || po.tok_server || po.tok_device || po.mig_at ||
+                      po.delayed || po.decision;
 
     uint64_t out_tokens = 0;
     for (int g = 0; g < G; ++g) out_tokens += rb.grp_sum_n[g];
     const bool long_outputs = out_tokens >= 512ull * n;
     // the hash is keyed by the request's index in the whole trace: key = mix(k0 + (first_index + i) * C_REQ)
     const uint32_t k0 = seed_key(seed) + (uint32_t)c->first_index * kHashReq;
-    // ---- per timeline class: play every request out, then evaluate the class's policies on the summaries
-    g_launches += 1;
     c->timing_valid = false;
     const bool timed = c->timing && classes.size() == 1;
-    for (size_t k = 0; k < classes.size(); ++k) {
+    uint32_t ticket = (uint32_t)classes.size();
+    const Prep* prep = c->d_prep.as<Prep>();
+    const GroupConst* gc = c->d_gc.as<GroupConst>();
+    const uint32_t* d_tab = c->d_tab.as<uint32_t>();
+    uint64_t *acc = c->d_acc.as<uint64_t>(), *h_ttft = c->d_hist_ttft.as<uint64_t>(), *h_tbt = c->d_hist_tbt.as<uint64_t>(),
+             *work = c->d_work.as<uint64_t>();
+    // ---- per timeline class: play every request out, then evaluate the class's policies on the summaries
+    for (size_t k = 0; k < classes.size() && n != 0; ++k) {
         const ClassConst* dcc = c->d_classes.as<ClassConst>() + k;
+        const bool wide = wide_class(k);
         if (timed) CU(cudaEventRecord(c->ev[0], st));
-        // with pacing on, a stream whose slowest interval T + J is within tau never falls behind its reader
-        const bool never_clamps = paced[k] != 0;
-        rec.tau = never_clamps ? (uint32_t)classes[k].tau : 0u;
-        CU(launch_timeline(tr, c->d_gc.as<GroupConst>(), dcc, classes[k].pacing != 0, c->knots.as<int32_t>(), k0, rec,
-                           c->err, c->d_todo.as<uint32_t>(), todo_counts + 2 * k, never_clamps, search[k], long_outputs,
-                           timed ? c->ev[1] : nullptr, c->sms, st));
+        CU(launch_timeline(tr, gc, dcc, classes[k], c->knots.as<int32_t>(), k0, rec, c->err, tickets + k, plan[k].kinds,
+                           plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, c->sms, st));
+        g_launches += timeline_launches(plan[k].kinds);
         if (timed) CU(cudaEventRecord(c->ev[2], st));
-        CU(launch_pairs(tr, c->d_gc.as<GroupConst>(), dcc, c->d_prep.as<Prep>(), P,
-                        c->d_pol_list.as<uint32_t>() + cls_range[k].first, cls_range[k].second - cls_range[k].first,
-                        c->d_chunks.as<Chunk>(), (uint32_t)chunks.size(), rec, po, c->d_acc.as<uint64_t>(),
-                        c->d_hist_ttft.as<uint64_t>(), c->d_hist_tbt.as<uint64_t>(), c->d_left.as<uint32_t>(),
-                        c->d_left.as<uint32_t>() + left_mask_words,
-                        left_list_words ? c->d_left.as<uint32_t>() + left_mask_words + left_cells : nullptr,
-                        sms, (uint32_t*)(c->d_work.as<uint64_t>() + 4) + k, c->d_work.as<uint64_t>(), k0, cls_extras_pending,
-                        !classes[k].pacing || classes[k].W[0] > 1 || classes[k].W[1] > 1 || classes[k].W[2] > 1,
-                        timed ? c->ev[3] : nullptr, st));
+        for (const Batch& b : batches[k]) {
+            GridTables gt;
+            const size_t tbt_word = wide ? 8 : 4;
+            char* base = (char*)c->d_grid.p;
+            gt.sums = (unsigned long long*)base;
+            gt.tbt = base + b.sums * 8;
+            gt.ttft = (uint32_t*)(base + b.sums * 8 + b.tbt * tbt_word);
+            CU(cudaMemsetAsync(base, 0, b.sums * 8 + b.tbt * tbt_word + b.ttft * 4, st));
+            const Slab* dsl = c->d_slabs.as<Slab>() + b.first;
+            const bool mixed = slabs[b.first].mixed != 0;
+            LeftLists left = {nullptr, nullptr};
+            if (mixed) {
+                left.list = c->d_left.as<uint32_t>(); left.count = left.list + N1;
+                CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
+            }
+            CU(launch_grid(tr, gc, dcc, prep, P, dsl, (uint32_t)b.count, b.T, wide, classes[k].pacing != 0, d_tab,
+                           c->d_chunks.as<Chunk>(), (uint32_t)chunks.size(), rec, gt, left, tickets + ticket++, work, c->sms, st));
+            CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.K, b.T, wide, host_bin_of_ticks(classes[k].tau), d_tab, gt, acc,
+                             h_ttft, h_tbt, st));
+            g_launches += 2;
+            if (mixed) {
+                const Slab& sl = slabs[b.first];
+                CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + mixed_pols[b.first], sl.policies, c->d_pair_chunks.as<Chunk>(),
+                                    (uint32_t)pair_chunks.size(), left.list, left.count, rec, acc, h_ttft, h_tbt, work, k0,
+                                    sl.expected_len != 0, wide, st));
+                g_launches += 1;
+            }
+        }
+        if (lists[k].n_ext) {
+            CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + lists[k].ext, (uint32_t)lists[k].n_ext,
+                                c->d_pair_chunks.as<Chunk>(), (uint32_t)pair_chunks.size(), nullptr, nullptr, rec, acc, h_ttft, h_tbt,
+                                work, k0, true, wide, st));
+            g_launches += 1;
+        }
+        if (timed) CU(cudaEventRecord(c->ev[3], st));
+        if (rows) {
+            CU(launch_pairs_rows(tr, gc, dcc, prep, P, d_tab + lists[k].all, (uint32_t)lists[k].n_all, rec, po, k0, extras, st));
+            g_launches += 1;
+        }
         if (timed) CU(cudaEventRecord(c->ev[4], st));
-        const bool wide_k = !classes[k].pacing || classes[k].W[0] > 1 || classes[k].W[1] > 1 || classes[k].W[2] > 1;
-        g_launches += (n ? ((classes[k].pacing && !never_clamps) ? 2 : 1) : 0) +
-                      ((n && !chunks.empty()) ? (out ? 2 : 1) + (wide_k ? 0 : 1) : 0);
     }
     c->timing_valid = timed && n != 0;
     c->P = P; c->pol = pc;

@@ -54,6 +54,13 @@ struct Prep {
 };
 
 // ---- a timeline class: the parameters a play-out depends on besides the request ----
+// How the streams of a group behave under a class, which decides the kernel that plays its requests:
+//   G_EXACT    no interval of either stream can exceed tau: everything is delivered at the pace, but the token after a
+//              hand-off.  Only the hand-off is played; sums, maxima and windows follow from the lengths.
+//   G_FREE     a stream either cannot clamp, as above, or clamps at every token (or pacing is off): it is delivered as
+//              it is generated, TBT = x_j.
+//   G_GENERAL  anything else.
+enum GroupKind { G_EXACT = 0, G_FREE = 1, G_GENERAL = 2 };
 struct ClassConst {
     int32_t tau_eff;             // tau when pacing is on, else 0 (then delivery = generation)
     int32_t tau;                 // tau of the policies (for the "equals tau" fast count)
@@ -63,28 +70,26 @@ struct ClassConst {
     int32_t W[3];                // bins per request for the server, device and migrated timelines
     int32_t lo[kMaxGroups][3];   // first bin of each window, per group
     int32_t ktau[kMaxGroups][3]; // index of bin(tau) inside the window, or -1
-    // Tokens the search for the hand-off may have to look at, per group, when no interval can exceed tau: every
-    // token then adds at least tau - (T + J) to the delivery lag, so (B-1) tau is passed within that many tokens.
+    // G_EXACT: tokens the search for the hand-off may have to look at.  Every token adds at least tau - (T + J) to the
+    // delivery lag, so (B-1) tau is passed within that many.
     uint32_t search[kMaxGroups];
+    uint8_t kind[kMaxGroups];    // GroupKind
+    uint8_t even[kMaxGroups];    // bit s: every regular interval of stream s equals tau, and its windows are not stored
 };
 
 // Per-request summaries of the up to three distinct decode timelines of a class.
 struct TimelineRec {
-    uint32_t tau;                // not 0: every stream is delivered at this pace (no interval can exceed it), and sums, maxima
-                                 // and windows are not stored: they follow from the lengths, m and the stall
-
-    uint32_t *sum[3], *max[3];   // d_n - d_1 and the largest TBT, ticks ([n] each)
-    uint32_t* stall;             // TBT of the first token after a hand-off
-    uint16_t *m, *delayed;       // hand-off index (0 = buffer never fills) and delayed tokens
-    uint32_t* win[3];            // [n][W[c]] counts per window bin
+    uint2* hand;                 // [n]: hand-off index (0 = buffer never fills) | delayed tokens << 16, and the TBT of the
+                                 // first token after the hand-off
+    uint32_t *sum[3], *max[3];   // d_n - d_1 and the largest TBT, ticks ([n] each; not of G_EXACT groups)
+    uint16_t* win[3];            // [n][W[c]] counts per window bin (not of streams that are even)
 };
 
 struct TraceDev {
     uint32_t n;
     int32_t n_groups;
-    const int32_t* S;            // server TTFT ticks, internal order: by group, inside a group by prompt length
-    const uint16_t *l, *nout;
-    const uint32_t* orig;        // caller's index of each request
+    const uint4* req;            // internal order (by group, inside a group by prompt length): server TTFT ticks,
+                                 // prompt length | output length << 16, caller's index, unused
     const uint32_t* inv;         // place of each of the caller's requests in the internal order
     const uint32_t* len_end;     // [G][4097]: where the group's requests of each prompt length end (the next length starts)
     const uint32_t* grp_off;     // [G+1]
@@ -150,6 +155,18 @@ inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block,
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The batch-th batch of 32 requests among the groups of one kind: its group, first request and length.
+__device__ __forceinline__ bool batch_of_kind(const TraceDev& tr, const ClassConst& cc, int kind, uint32_t batch, int& g,
+                                              uint32_t& k_lo, uint32_t& count) {
+    for (g = 0; g < tr.n_groups; ++g) {
+        if (cc.kind[g] != kind) continue;
+        const uint32_t lo = tr.grp_off[g], len = tr.grp_off[g + 1] - lo, here = (len + 31u) / 32u;
+        if (batch < here) { k_lo = lo + batch * 32u; count = min(32u, len - batch * 32u); return true; }
+        batch -= here;
+    }
+    return false;
+}
 #endif
 
 // Records the calling thread's error message (read back by disco_last_error) and returns `code`.
@@ -203,36 +220,55 @@ cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupCo
                         cudaStream_t st);
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, int G, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off, Prep* prep, cudaStream_t st);
-cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, bool pacing,
+// Plays every request under one class.  `kinds`: bit k set if some group with requests is of GroupKind k; `batches[k]`:
+// batches of 32 requests of the groups of kind k.
+cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const ClassConst& host_cc,
                             const int32_t* knots, uint32_t k0 /* hash key base: seed_key(seed) + first_index * kHashReq */,
-                            TimelineRec rec, int32_t* err, uint32_t* todo,
-                            uint32_t* todo_count /* two words, zero on entry: length of the list, batch tickets */,
-                            bool never_clamps /* pacing on and tau >= T + J for both endpoints of every group */,
-                            uint32_t search /* then: largest ClassConst::search of a group with requests */,
+                            TimelineRec rec, int32_t* err, uint32_t* ticket /* one word, zero */, uint32_t kinds,
+                            const uint32_t* batches, uint32_t search /* largest ClassConst::search of a group with requests */,
                             bool long_outputs /* mean output length of 512 tokens or more */,
-                            cudaEvent_t mid /* recorded between its two kernels, or null */,
+                            cudaEvent_t mid /* recorded between the kernels of exact groups and the others, or null */,
                             int sms /* multiprocessors of the device */, cudaStream_t st);
-cudaError_t launch_pairs(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
-                         const uint32_t* pol_list, uint32_t n_list, const Chunk* chunks, uint32_t n_chunks,
-                         TimelineRec rec, disco_pair_out_t out, uint64_t* acc, uint64_t* hist_ttft,
-                         uint64_t* hist_tbt,
-                         uint32_t* left_mask /* [n][ceil(tiles / 32)] scratch for the requests the zone kernel leaves to
-                         the pair kernel, or null: every pair is evaluated one by one */,
-                         uint32_t* left_count /* [n_chunks][tiles] scratch */,
-                         uint32_t* left_lists /* [n_chunks][tiles][kLeftList] scratch, or null */,
-                         uint32_t zone_blocks /* blocks the zone kernel may run: one per multiprocessor */,
-                         uint32_t* zone_ticket /* one word, zero: the zone kernel's blocks draw their work from it */,
-                         uint64_t* work /* [4], added to: pairs settled zone by zone, pairs evaluated one by one,
-                         requests settled per policy family, sweeps over segments of a chunk */,
-                         uint32_t k0, bool extras /* some policy routes at random or uses an
-                         expected length */, bool wide /* some window W of the class spans several bins */,
-                         cudaEvent_t mid /* recorded between its two kernels, or null */,
-                         cudaStream_t st);
-cudaError_t launch_pairs_zones(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep,
-                               uint32_t P, const uint32_t* pol_list, uint32_t n_list, int PL, const Chunk* chunks,
-                               uint32_t n_chunks, TimelineRec rec, uint64_t* acc, uint64_t* hist_ttft,
-                               uint64_t* hist_tbt, uint32_t* left_mask, uint32_t* left_count, uint32_t* left_lists,
-                               uint32_t max_blocks, uint32_t* ticket, uint64_t* work, cudaStream_t st);
+uint32_t timeline_launches(uint32_t kinds);
+
+// Reductions over a grid of plain policies, budget by overhead (grid.cu).
+constexpr int kGridRows = 8;     // overheads a slab may have
+constexpr int kGridCols = 256;   // budgets a slab may have
+struct Slab {
+    int32_t K, T;                // distinct budgets (columns, ascending), distinct overheads (rows, ascending)
+    uint32_t cols;               // index into the tables: policy whose preparation stands for each column, [K]
+    uint32_t cells;              // index into the tables: policy of (column, row), [K][T], ~0 where there is none
+    uint32_t expected_len;
+    int32_t mig;                 // the policies migrate
+    uint32_t policies;           // how many they are
+    int32_t mixed;               // a column per policy, whose overheads lie between theta[0] and theta[1] (T = 1):
+                                 // requests whose saving lies between the two are left to the pair kernel
+    float theta[kGridRows];
+    // 32- or 64-bit words in front of the slab's difference tables, see grid.cu
+    uint64_t ttft, tbt, sums;
+};
+struct GridTables { uint32_t* ttft; void* tbt; unsigned long long* sums; };
+struct LeftLists { uint32_t* list; uint32_t* count; };   // [slabs][n] places in the internal order, [slabs][G]
+uint64_t grid_ttft_words(int K), grid_tbt_words(int K, int T), grid_sum_words(int K, int T, int G);
+uint32_t grid_blocks_per_sm(int T);
+cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
+                        const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide, bool count_pairs,
+                        const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt,
+                        LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t* ticket /* zero */,
+                        uint64_t* work /* [4], added to */, int sms, cudaStream_t st);
+cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int K, int T,
+                          bool wide, int bin_tau, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
+                          uint64_t* hist_tbt, cudaStream_t st);
+// Pair by pair: `n_list` policies under the chunks' requests, or (list not null) under the listed ones.
+cudaError_t launch_pairs_acc(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
+                             const uint32_t* pol_list, uint32_t n_list, const Chunk* chunks, uint32_t n_chunks,
+                             const uint32_t* list /* [n] */, const uint32_t* list_count /* [G] */, TimelineRec rec,
+                             uint64_t* acc, uint64_t* hist_ttft, uint64_t* hist_tbt, uint64_t* work, uint32_t k0,
+                             bool extras /* some policy routes at random or waits by Eq. 1-2 */,
+                             bool wide /* some window W of the class spans several bins */, cudaStream_t st);
+cudaError_t launch_pairs_rows(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
+                              const uint32_t* pol_list, uint32_t n_list, TimelineRec rec, const disco_pair_out_t& out,
+                              uint32_t k0, bool extras, cudaStream_t st);
 cudaError_t launch_finalize(uint32_t P, int G, const GroupConst* gc, const uint64_t* acc, const uint64_t* hist_ttft,
                             const uint64_t* hist_tbt,
                             const uint64_t* fin_totals /* [2G]: output tokens per group, then requests per group */,

@@ -1,0 +1,646 @@
+// Per-policy reductions over a grid of plain policies, budgets by migration overheads: dispatch decision (Algorithms 2-3,
+// wait-then-race), TTFT, which decode stream applies (migration trigger, Eq. 4), tokens per endpoint.
+//
+// The distinct budgets of the policies are the grid's COLUMNS (ascending), the distinct overheads its ROWS.  What a
+// request comes to under a policy, but for the hand-off, depends on the column alone, and along the columns thresholds
+// are ordered: Algorithm 3's l_th does not increase, Algorithm 2's l* does not decrease, its w_tail does not increase.
+// So a request falls into at most three runs of columns that dispatch it alike:
+//   Algorithm 3:  columns [0, k) have l_th > l  -> device only;     [k, K) race at once (wait 0);
+//   Algorithm 2:  columns [0, k1) have l* < l   -> wait w_tail;     [k1, k2) have l* = l -> wait their own w*;
+//                 [k2, K) have l* > l           -> wait 0.
+// k, k1, k2 depend on the prompt length alone, and the requests of a group are stored by prompt length: a chunk of
+// requests splits into a few SEGMENTS of consecutive requests that share them.  A block sweeps a segment once per run
+// with a lane per request, sums up what the requests come to in registers and shared-memory histograms, and enters the
+// run's totals ONCE: into row k2 of a table of differences that is carried to the columns from k2 on, or into row k1 of
+// one that is carried to the columns below k1.  k_spread adds the rows up and writes every policy's sums and histograms.
+// Under Algorithm 2 the first columns (budgets below the tail ratio) may wait longer than the others: for the few
+// requests that the common w_tail does not cover (at most a share alpha of them) the block keeps a list, and each of
+// those columns gets the list's totals under its own wait in place of the common one.
+//
+// The rows differ in the hand-off alone: a race won by the endpoint that may hand over migrates in the rows whose
+// overhead is below the request's saving.  Every sweep adds what migration changes to each row whose overhead it passes
+// (three additions a row); the hand-off stall is counted at the level of the last such row, and the levels are summed
+// up when the run is entered.
+//
+// Bound: integer issue.  Against one sweep per 128 policies of one overhead, with what differs between neighbouring
+// policies entered into their histograms one by one, a request is visited once per run instead of once per run and
+// overhead (figures at launch_grid).
+#include <algorithm>
+#include <cstddef>
+#include <type_traits>
+
+#include "tile.cuh"
+
+namespace disco {
+
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kListCap = 8192;           // requests a block lists for the columns with longer waits
+constexpr int kListStep = 4096;          // ... and looks after the list's room every so many requests
+constexpr int kMaxSeg = 2 * kGridCols + 2;
+constexpr uint32_t FULL = 0xFFFFFFFFu;
+constexpr uint32_t kNoPolicy = 0xFFFFFFFFu;
+
+// Sums of a run: what every row gets, and per row what migration changes.
+enum Base { B_TD = 0, B_PS, B_PD, B_DO, B_RACE, B_DW, B_TAU, B_TT, kBase };
+enum Lev { V_A = 0, V_B, V_C, V_N, V_TAU, kLev };      // tokens handed over, prefill of the target, delayed, count, TBTs in tau's bin
+__host__ __device__ constexpr int sum_fields(int T) { return kBase + T * kLev; }
+
+struct Seg { uint16_t pa, pb, k1, k2; };               // requests [pa, pb) of the chunk
+
+struct Smem {                                          // fixed part; the TBT histograms [T][kNBins] follow, and one more for
+                                                       // the device-only run where windows are counted
+    uint32_t sum[kBase + kGridRows * kLev];            // totals of the run in work
+    uint32_t only_sum[4];                              // ... of the device-only run: requests, tokens, prompt tokens, TBTs in tau's bin
+    unsigned long long tt, only_tt;                    // ... and the sums of TTFTs
+    uint32_t ttft[kNBins], only_ttft[kNBins];
+    uint32_t n_seg, n_list, flagged, ticket;
+    int32_t key[kGridCols];                            // the columns' length thresholds
+    uint32_t w_star[kGridCols], w_tail[kGridCols];
+    Seg seg[kMaxSeg];
+    uint16_t list[kListCap];
+};
+
+template <int NT>
+struct Acc {                                           // a lane's share of a run
+    uint32_t td, ps, pd, tau, race, dw;
+    unsigned long long tt;
+    uint32_t a[NT], b[NT], cn[NT], tx[NT];             // cn: delayed tokens | requests << 22 (at most 255 requests a lane)
+};
+
+struct Only { uint32_t cnt, n, l, tau; unsigned long long tt; };   // ... of a device-only run
+
+struct Ctx {                                           // a (chunk, slab)
+    uint32_t start, len;
+    uint32_t kappa, c0;
+    float delta_c;
+    int cand, g;
+    int K, T;
+    bool may_migrate, mixed;
+    float th_lo;                                       // mixed: smallest overhead
+    int E0;
+    uint32_t even;
+};
+
+struct Args {
+    TraceDev tr;
+    TimelineRec rec;
+    const GroupConst* gcs;
+    const ClassConst* cc;
+    const Prep* prep;
+    uint32_t P;
+    const Slab* slabs;
+    uint32_t n_slabs;
+    const uint32_t* tab;
+    const Chunk* chunks;
+    uint32_t n_chunks;
+    GridTables gt;
+    LeftLists left;
+    uint32_t* ticket;
+    unsigned long long* work;
+    int count_pairs;
+};
+
+__device__ __forceinline__ void hist_add(uint32_t* h, int bin) {
+    if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicAdd(&h[bin], 1u);
+}
+
+// Adds the rows of window counts of the lanes' requests to the TBT histograms (streams whose intervals are not all tau).
+// hist_all: the histogram that every row gets.  need_x: the stream after a hand-off, at level t (1 .. T).
+__device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_t* tbt, uint32_t* hist_all, bool need_base,
+                                            bool need_x, uint32_t kk, int stream, int t) {
+    const ClassConst& cc = *a.cc;
+    const int lane = threadIdx.x & 31;
+    uint32_t pend = __ballot_sync(FULL, need_base || need_x);
+    const uint32_t mine = (uint32_t)stream | (need_base ? 2u : 0u) | (need_x ? 4u : 0u) | ((uint32_t)t << 3);
+    while (pend) {
+        const int r = __ffs(pend) - 1;
+        pend &= pend - 1u;
+        const uint32_t code = __shfl_sync(FULL, mine, r), k = __shfl_sync(FULL, kk, r);
+        const int level = (int)(code >> 3);
+        if (code & 2u) {
+            const int s = (int)(code & 1u), W = cc.W[s], lo = cc.lo[c.g][s];
+            const uint16_t* row = a.rec.win[s] + (size_t)k * W;
+            for (int b = lane; b < W; b += 32) {
+                const uint32_t v = row[b];
+                if (v == 0u || !DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) continue;
+                if (level < c.T || !tbt) atomicAdd(&hist_all[lo + b], v);
+                if (level > 0 && level < c.T) atomicSub(&tbt[(level - 1) * kNBins + lo + b], v);
+            }
+        }
+        if (code & 4u) {
+            const int W = cc.W[2], lo = cc.lo[c.g][2];
+            const uint16_t* row = a.rec.win[2] + (size_t)k * W;
+            for (int b = lane; b < W; b += 32) {
+                const uint32_t v = row[b];
+                if (v && DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicAdd(&tbt[(level - 1) * kNBins + lo + b], v);
+            }
+        }
+    }
+}
+
+// One sweep over the requests [pa, pb) of the chunk, or (list) of the block's list: what they come to when the device
+// starts after the wait w, added up in `s` and in the shared histograms.  push: requests with S > w go on the list.
+// ONLY: the segment is Algorithm 3's; `race` says whether some columns race (w = 0), `only` whether some run the device
+// alone, which is added up in `o` and histograms of its own.
+template <int NT, bool WIDE, bool ONLY>
+__device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (&th)[NT], Smem& sm, uint32_t* tbt, uint32_t pa,
+                                      uint32_t pb, uint32_t w, bool list, bool push, bool race, bool only, Acc<NT>& s, Only& o) {
+    const int lane = threadIdx.x & 31;
+    for (uint32_t i0 = pa + (threadIdx.x & ~31u); i0 < pb; i0 += kThreads) {          // a warp's lanes iterate together
+        const uint32_t i = min(i0 + lane, pb - 1);
+        const uint32_t pos = list ? (uint32_t)sm.list[i] : i;
+        const uint32_t kk = c.start + pos;
+        bool valid = i0 + lane < pb && DBG_OK(kk, a.tr.n, DBG_K_PAIRS_ZONES, DBG_REQUEST);
+        const uint4 q = a.tr.req[kk];
+        const uint2 hand = c.may_migrate ? a.rec.hand[kk] : make_uint2(0u, 0u);
+        const uint32_t S = q.x, l = q.y & 0xFFFFu, n = q.y >> 16, m = hand.x & 0xFFFFu, dly = hand.x >> 16;
+        const uint32_t Td = c.kappa * l + c.c0;
+        // Eq. 4's projected saving, on the true remainder or on what is left of the expected length; a request may only
+        // hand over if its buffer filled (m != 0)
+        float saving = m ? c.delta_c * (float)(c.E0 ? max(c.E0 - (int)m, 0) : (int)(n - m)) : -1.0f;
+        if (c.mixed) valid = valid && !(saving > c.th_lo && !(saving > th[0]));       // left to the pair kernel
+        if (ONLY) {
+            if (only) {
+                const int bin = bin_of_ticks(Td);
+                const uint32_t live = __ballot_sync(FULL, valid);
+                // requests of one prompt length share the device's TTFT: mostly the whole warp counts in one bin
+                if (__shfl_sync(FULL, l, 0) == __shfl_sync(FULL, l, 31)) {
+                    if (lane == 0 && live && DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicAdd(&sm.only_ttft[bin], (uint32_t)__popc(live));
+                } else if (valid) hist_add(sm.only_ttft, bin);
+                if (valid) { o.cnt += 1u; o.n += n; o.l += l; o.tt += Td; o.tau += (!WIDE || (c.even & 2u)) ? n - 1u : 0u; }
+                if (WIDE && !(c.even & 2u)) add_windows(a, c, nullptr, tbt + NT * kNBins, valid, false, kk, 1, 0);
+            }
+            if (!race) continue;
+        }
+        const bool started = S > w, dev_wins = S > w + Td;            // the device starts after the wait; a tie goes to the server
+        const uint32_t tt = min(S, w + Td);
+        const bool pace = ((c.even >> (dev_wins ? 1 : 0)) & 1u) != 0; // the base stream's intervals are all tau
+        if (valid) {
+            s.td += dev_wins ? n : 0u; s.ps += l; s.pd += started ? l : 0u;
+            s.race += started ? 1u : 0u; s.dw += dev_wins ? 1u : 0u;
+            s.tt += tt;
+            s.tau += (!WIDE || pace) ? n - 1u : 0u;
+            hist_add(sm.ttft, bin_of_ticks(tt));
+        }
+        if (!ONLY && push) {
+            const bool mine = valid && S > w;
+            const uint32_t all = __ballot_sync(FULL, mine);
+            if (all) {
+                uint32_t at = 0;
+                if (lane == 0) at = atomicAdd(&sm.n_list, (uint32_t)__popc(all));
+                at = __shfl_sync(FULL, at, 0) + __popc(all & ((1u << lane) - 1u));
+                if (mine && DBG_OK(at, kListCap, DBG_K_PAIRS_ZONES, DBG_SLOT)) sm.list[at] = (uint16_t)pos;
+            }
+        }
+        if (!(valid && started && (dev_wins ? 2 : 1) == c.cand)) saving = -1.0f;      // not won by the endpoint that may hand over
+        const uint32_t handed = n - m, refill = l + m, cn = dly | 1u << 22;
+        const uint32_t tx = WIDE ? ((c.even & 4u) ? n - 2u : 0u) - (pace ? n - 1u : 0u) : 0u;
+        int t = 0;                                                    // rows that migrate: [0, t)
+#pragma unroll
+        for (int r = 0; r < NT; ++r)
+            if (saving > th[r]) {
+                s.a[r] += handed; s.b[r] += refill; s.cn[r] += cn; ++t;
+                if (WIDE) s.tx[r] += tx;
+            }
+        if (t > 0) hist_add(tbt + (t - 1) * kNBins, bin_of_ticks(hand.y));
+        if (WIDE) add_windows(a, c, tbt, tbt + (c.T - 1) * kNBins, valid && !pace, t > 0 && !(c.even & 4u), kk, dev_wins ? 1 : 0, t);
+    }
+}
+
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+    return v;
+}
+
+// The lanes' shares of a run go to the block's totals (32-bit: at most 65,280 requests of at most 12,288 tokens).  Lane f
+// of a warp adds field f.
+template <int NT, bool WIDE>
+__device__ __forceinline__ void share_out(Smem& sm, const Acc<NT>& s, int T) {
+    const int lane = threadIdx.x & 31;
+    uint32_t lo = 0, hi = 0;
+    auto put = [&](int f, uint32_t v) {
+        v = __reduce_add_sync(FULL, v);
+        if (f < 32) { if (lane == f) lo = v; } else if (lane == f - 32) hi = v;
+    };
+    put(B_TD, s.td); put(B_PS, s.ps); put(B_PD, s.pd); put(B_RACE, s.race); put(B_DW, s.dw); put(B_TAU, s.tau);
+#pragma unroll
+    for (int r = 0; r < NT; ++r) {
+        const int f = kBase + r * kLev;
+        put(f + V_A, s.a[r]); put(f + V_B, s.b[r]); put(f + V_C, s.cn[r] & 0x3FFFFFu); put(f + V_N, s.cn[r] >> 22);
+        if (WIDE) put(f + V_TAU, s.tx[r]);
+    }
+    if (lo) atomicAdd(&sm.sum[lane], lo);
+    if (NT * kLev + kBase > 32 && hi) atomicAdd(&sm.sum[32 + lane], hi);
+    const unsigned long long tt = warp_sum(s.tt);
+    if (lane == 0 && tt) atomicAdd(&sm.tt, tt);
+}
+__device__ __forceinline__ void share_only(Smem& sm, const Only& o) {
+    const uint32_t c = __reduce_add_sync(FULL, o.cnt), n = __reduce_add_sync(FULL, o.n), l = __reduce_add_sync(FULL, o.l),
+                   tau = __reduce_add_sync(FULL, o.tau);
+    const unsigned long long tt = warp_sum(o.tt);
+    if ((threadIdx.x & 31) == 0 && c) {
+        atomicAdd(&sm.only_sum[0], c); atomicAdd(&sm.only_sum[1], n); atomicAdd(&sm.only_sum[2], l); atomicAdd(&sm.only_sum[3], tau);
+        atomicAdd(&sm.only_tt, tt);
+    }
+}
+
+// A slab's difference tables.  U row q is carried to the columns below q, V row q to the columns from q on (q = 0 .. K).
+template <bool WIDE>
+struct Tables {
+    using word = typename std::conditional<WIDE, unsigned long long, unsigned int>::type;   // windows hold more than 2^32 TBTs
+    uint32_t* ttft;                      // [2][K + 1][kNBins]
+    word* tbt;                           // [2][K + 1][T][kNBins]
+    unsigned long long* sums;            // [2][G][K + 1][fields]
+    int K, T, G;
+    __device__ Tables(const GridTables& gt, const Slab& sl, int G_)
+        : ttft(gt.ttft + sl.ttft), tbt((word*)gt.tbt + sl.tbt), sums(gt.sums + sl.sums), K(sl.K), T(sl.T), G(G_) {}
+    __device__ uint32_t* ttft_row(int v, int q) const { return ttft + (size_t)(v * (K + 1) + q) * kNBins; }
+    __device__ word* tbt_row(int v, int q, int r) const { return tbt + ((size_t)(v * (K + 1) + q) * T + r) * kNBins; }
+    __device__ unsigned long long* sum_row(int v, int g, int q) const { return sums + ((size_t)(v * G + g) * (K + 1) + q) * sum_fields(T); }
+};
+
+// Where a run's totals are entered: V row `row` (from), U row `row` (below, negated or not), or one column alone.
+enum Enter { E_FROM, E_BELOW, E_BELOW_NEG, E_ALONE };
+
+// Enters what the block has totalled for a run and clears it.  All threads call; barriers before and after.
+template <bool WIDE>
+__device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE>& tb, int g, Enter how, int row) {
+    using word = typename Tables<WIDE>::word;
+    const int v = how == E_FROM ? 1 : 0, q = how == E_ALONE ? row + 1 : row;
+    const bool neg = how == E_BELOW_NEG, second = how == E_ALONE && row > 0;    // (row 0 is carried to nobody)
+    for (int b = threadIdx.x; b < kNBins; b += kThreads) {
+        const uint32_t x = sm.ttft[b];
+        if (x) {
+            sm.ttft[b] = 0;
+            atomicAdd(&tb.ttft_row(v, q)[b], neg ? 0u - x : x);
+            if (second) atomicAdd(&tb.ttft_row(0, row)[b], 0u - x);
+        }
+        int32_t level = 0;                                             // counts at a level go to every row below it
+        for (int r = tb.T - 1; r >= 0; --r) {
+            const int32_t y = (int32_t)tbt[r * kNBins + b];
+            if (y) { tbt[r * kNBins + b] = 0; level += y; }
+            if (level) {
+                const word z = (word)(long long)level;
+                atomicAdd(&tb.tbt_row(v, q, r)[b], neg ? (word)0 - z : z);
+                if (second) atomicAdd(&tb.tbt_row(0, row, r)[b], (word)0 - z);
+            }
+        }
+    }
+    const int F = sum_fields(tb.T);
+    for (int f = threadIdx.x; f < F; f += kThreads) {
+        unsigned long long x = (f >= kBase && (f - kBase) % kLev == V_TAU) ? (unsigned long long)(long long)(int32_t)sm.sum[f] : sm.sum[f];
+        sm.sum[f] = 0;
+        if (f == B_TT) { x = sm.tt; sm.tt = 0; }
+        if (!x) continue;
+        atomicAdd(&tb.sum_row(v, g, q)[f], neg ? 0ull - x : x);
+        if (second) atomicAdd(&tb.sum_row(0, g, row)[f], 0ull - x);
+    }
+}
+
+// The same for a device-only run, columns below `row`.
+template <bool WIDE>
+__device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const Tables<WIDE>& tb, int g, int row) {
+    using word = typename Tables<WIDE>::word;
+    for (int b = threadIdx.x; b < kNBins; b += kThreads) {
+        const uint32_t x = sm.only_ttft[b];
+        if (x) { sm.only_ttft[b] = 0; atomicAdd(&tb.ttft_row(0, row)[b], x); }
+        if (WIDE) {
+            const uint32_t y = only_tbt[b];
+            if (y) {
+                only_tbt[b] = 0;
+                for (int r = 0; r < tb.T; ++r) atomicAdd(&tb.tbt_row(0, row, r)[b], (word)y);
+            }
+        }
+    }
+    if (threadIdx.x < 5) {
+        const int k = threadIdx.x;
+        const unsigned long long x = k < 4 ? (unsigned long long)sm.only_sum[k] : sm.only_tt;
+        if (k < 4) sm.only_sum[k] = 0; else sm.only_tt = 0;
+        const int f = k == 0 ? B_DO : k == 1 ? B_TD : k == 2 ? B_PD : k == 3 ? B_TAU : B_TT;
+        if (x) atomicAdd(&tb.sum_row(0, g, row)[f], x);
+    }
+}
+
+template <int NT, bool WIDE>
+__global__ void __launch_bounds__(kThreads, NT == 1 ? 4 : 2)
+k_grid(const __grid_constant__ Args a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+    uint32_t* tbt = (uint32_t*)(smem_raw + sizeof(Smem));
+    grid_dependency_wait();
+    for (int i = threadIdx.x; i < (int)(offsetof(Smem, key) / 4); i += kThreads) ((uint32_t*)&sm)[i] = 0;
+    for (int i = threadIdx.x; i < (NT + (WIDE ? 1 : 0)) * kNBins; i += kThreads) tbt[i] = 0;
+
+    // the blocks draw (chunk, slab) items from a counter (zero at launch): items differ in cost
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) { sm.ticket = atomicAdd(a.ticket, 1u); sm.n_seg = 0; sm.n_list = 0; sm.flagged = 0; }
+        __syncthreads();
+        const uint32_t item = sm.ticket;
+        if (item >= a.n_chunks * a.n_slabs) break;
+        const uint32_t slab_id = item % a.n_slabs;
+        const Slab& sl = a.slabs[slab_id];
+        const Chunk ch = a.chunks[item / a.n_slabs];
+        const int g = ch.g;
+        if (!DBG_OK(g, a.tr.n_groups, DBG_K_PAIRS_ZONES, DBG_GROUP) ||
+            (ch.len && !DBG_OK((unsigned long long)ch.start + ch.len - 1, a.tr.n, DBG_K_PAIRS_ZONES, DBG_REQUEST)))
+            continue;
+        const GroupConst& gc = a.gcs[g];
+        const Tables<WIDE> tb(a.gt, sl, a.tr.n_groups);
+        Ctx c;
+        c.start = ch.start; c.len = ch.len; c.kappa = (uint32_t)gc.kappa; c.c0 = (uint32_t)gc.c0;
+        c.delta_c = gc.delta_c; c.cand = gc.candidate; c.g = g; c.K = sl.K; c.T = sl.T;
+        c.may_migrate = sl.mig && gc.candidate != 0;
+        c.mixed = sl.mixed && c.may_migrate;
+        c.E0 = (int)sl.expected_len; c.even = a.cc->even[g];
+        float th[NT];                                                  // rows beyond the slab's never migrate
+#pragma unroll
+        for (int r = 0; r < NT; ++r) th[r] = (c.may_migrate && r < c.T) ? sl.theta[sl.mixed ? 1 : r] : __int_as_float(0x7F800000);
+        c.th_lo = sl.theta[0];
+        bool waits = false;
+        {
+            const Prep& pr = a.prep[(size_t)g * a.P + a.tab[sl.cols]];
+            waits = pr.device_constrained != 0;
+        }
+        for (int p = threadIdx.x; p < c.K; p += kThreads) {
+            if (!DBG_OK(a.tab[sl.cols + p], a.P, DBG_K_PAIRS_ZONES, DBG_POLICY)) continue;
+            const Prep& pr = a.prep[(size_t)g * a.P + a.tab[sl.cols + p]];
+            sm.key[p] = waits ? pr.l_star : pr.l_th;
+            sm.w_star[p] = (uint32_t)pr.w_star; sm.w_tail[p] = (uint32_t)pr.w_tail;
+        }
+        if (c.mixed) {
+            // ---- requests whose saving lies between the policies' overheads: to the pair kernel's list
+            const uint32_t first = a.tr.grp_off[g];
+            uint32_t mine = 0;
+            for (uint32_t i0 = threadIdx.x & ~31u; i0 < ch.len; i0 += kThreads) {
+                const uint32_t i = min(i0 + (threadIdx.x & 31), ch.len - 1), kk = ch.start + i;
+                const uint4 q = a.tr.req[kk];
+                const uint32_t m = a.rec.hand[kk].x & 0xFFFFu, n = q.y >> 16;
+                const float saving = m ? c.delta_c * (float)(c.E0 ? max(c.E0 - (int)m, 0) : (int)(n - m)) : -1.0f;
+                const bool out = i0 + (threadIdx.x & 31) < ch.len && saving > c.th_lo && !(saving > th[0]);
+                const uint32_t all = __ballot_sync(FULL, out);
+                if (!all) continue;
+                uint32_t at = 0;
+                if ((threadIdx.x & 31) == 0) at = atomicAdd(&a.left.count[slab_id * a.tr.n_groups + g], (uint32_t)__popc(all));
+                at = first + __shfl_sync(FULL, at, 0) + __popc(all & ((1u << (threadIdx.x & 31)) - 1u));
+                if (out && DBG_OK(at, a.tr.n, DBG_K_PAIRS_ZONES, DBG_REQUEST)) a.left.list[(size_t)slab_id * a.tr.n + at] = kk;
+                mine += (uint32_t)__popc(all);
+            }
+            if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&sm.flagged, mine);
+        }
+        __syncthreads();
+
+        // ---- the segments: stretches of prompt lengths between two thresholds and (Algorithm 2) the thresholds
+        //      themselves; a thread per candidate looks up where its lengths lie in the chunk
+        const int K = c.K;
+        for (int q = threadIdx.x; q < (waits ? 2 * K + 1 : K + 1); q += kThreads) {
+            auto cl = [](int x) { return min(max(x, 0), kMaxPrompt + 1); };
+            int la, lb, k1, k2;
+            bool any = true;
+            if (waits) {                                             // thresholds ascend
+                const int p = q >> 1;
+                k1 = k2 = p;
+                if (q == 2 * K) { la = cl(sm.key[K - 1] + 1); lb = kMaxPrompt + 1; }
+                else if (q & 1) {
+                    la = cl(sm.key[p]); lb = cl(sm.key[p] + 1); any = p == 0 || sm.key[p] != sm.key[p - 1];
+                    if (any && la < lb) while (k2 < K && sm.key[k2] == sm.key[p]) ++k2;
+                }
+                else { la = p ? cl(sm.key[p - 1] + 1) : 0; lb = cl(sm.key[p]); }
+            } else {                                                 // thresholds descend
+                la = q ? cl(sm.key[K - q]) : 0;
+                lb = q < K ? cl(sm.key[K - 1 - q]) : kMaxPrompt + 1;
+                k1 = k2 = K - q;
+            }
+            if (any && la < lb) {
+                // first request of the group with a prompt of at least L tokens: where the shorter ones end
+                const uint32_t* ends = a.tr.len_end + (size_t)g * (kMaxPrompt + 1);
+                const uint32_t at_a = la ? ends[la - 1] : a.tr.grp_off[g], at_b = ends[lb - 1];
+                const uint32_t lo = ch.start, hi = ch.start + ch.len;
+                const uint32_t pa = min(max(at_a, lo), hi) - lo, pb = min(max(at_b, lo), hi) - lo;
+                if (pa < pb) {
+                    const uint32_t at = atomicAdd(&sm.n_seg, 1u);
+                    if (DBG_OK(at, kMaxSeg, DBG_K_PAIRS_ZONES, DBG_SLOT))
+                        sm.seg[at] = Seg{(uint16_t)pa, (uint16_t)pb, (uint16_t)k1, (uint16_t)k2};
+                }
+            }
+        }
+        const uint32_t wt_min = waits ? sm.w_tail[K - 1] : 0u;
+        int n_low = 0;                                                // columns that wait longer than the others: the first ones
+        for (int p0 = 0; waits && p0 < K; p0 += kThreads) {
+            const int p = p0 + (int)threadIdx.x;
+            n_low += __syncthreads_count(p < K && sm.w_tail[p] > wt_min);
+        }
+        __syncthreads();
+        const int n_seg = (int)min(sm.n_seg, (uint32_t)kMaxSeg);
+        uint32_t passes = 0;
+
+        // one run: sweep and enter; `list` and `push` as in sweep
+        auto run = [&](uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, Enter how, int row) {
+            Acc<NT> s = {};
+            Only none = {};
+            sweep<NT, WIDE, false>(a, c, th, sm, tbt, pa, pb, w, list, push, true, false, s, none);
+            share_out<NT, WIDE>(sm, s, c.T);
+            __syncthreads();
+            enter<WIDE>(sm, tbt, tb, g, how, row);
+            __syncthreads();
+            ++passes;
+        };
+        if (!waits) {
+            for (int si = 0; si < n_seg; ++si) {
+                const Seg sg = sm.seg[si];
+                const bool race = (int)sg.k2 < K, only = sg.k1 > 0;
+                Acc<NT> s = {};
+                Only o = {};
+                sweep<NT, WIDE, true>(a, c, th, sm, tbt, sg.pa, sg.pb, 0u, false, false, race, only, s, o);
+                if (race) share_out<NT, WIDE>(sm, s, c.T);
+                if (only) share_only(sm, o);
+                __syncthreads();
+                if (race) enter<WIDE>(sm, tbt, tb, g, E_FROM, sg.k2);
+                if (only) enter_only<WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1);
+                __syncthreads();
+                ++passes;
+            }
+        } else {
+            // segment by segment, run by run: [k2, K) waits 0, each column of [k1, k2) its own w*, [0, k1) w_tail -- and,
+            // when the list is full or the chunk is done, the list for the columns that wait longer
+            uint32_t pa = 0;                                          // (of the segment in work: where the sweep goes on)
+            int si = 0, ri = 0;
+            for (;;) {
+                uint32_t from, to, w;
+                bool list = false, push = false, last = false;
+                Enter how;
+                int row;
+                if (si < n_seg) {
+                    const Seg sg = sm.seg[si];
+                    const int n_pts = (int)sg.k2 - (int)sg.k1;
+                    if (ri == 0) { pa = sg.pa; }
+                    if (ri == 0 && (int)sg.k2 >= K) { ++ri; continue; }
+                    if (ri > n_pts && sg.k1 == 0) { ri = 0; ++si; continue; }
+                    from = pa; to = sg.pb;
+                    if (ri == 0) { w = 0u; how = E_FROM; row = sg.k2; ++ri; }
+                    else if (ri <= n_pts) { row = (int)sg.k1 + ri - 1; w = sm.w_star[row]; how = E_ALONE; ++ri; }
+                    else {
+                        w = wt_min; how = E_BELOW; row = sg.k1; push = n_low > 0;
+                        if (push && to - from > (uint32_t)kListStep) { to = from + kListStep; pa = to; }
+                        else { ri = 0; ++si; }
+                    }
+                } else if (sm.n_list > 0) { from = to = 0; w = 0; how = E_FROM; row = 0; last = true; }
+                else break;
+                if (!last) run(from, to, w, list, push, how, row);
+                if (last || (push && sm.n_list > (uint32_t)(kListCap - kListStep))) {
+                    const uint32_t k = sm.n_list;                     // (barriers inside run: all threads agree)
+                    __syncthreads();
+                    if (threadIdx.x == 0) sm.n_list = 0;
+                    for (int p = -1; p < n_low; ++p)
+                        run(0u, k, p < 0 ? wt_min : sm.w_tail[p], true, false, p < 0 ? E_BELOW_NEG : E_ALONE, p < 0 ? n_low : p);
+                }
+            }
+        }
+        if (threadIdx.x == 0 && a.work) {
+            const unsigned long long settled = ch.len - sm.flagged;
+            atomicAdd(&a.work[a.count_pairs ? 0 : 1], settled * (unsigned long long)sl.policies);
+            atomicAdd(&a.work[2], settled);                            // requests settled, per slab
+            atomicAdd(&a.work[3], (unsigned long long)passes);         // sweeps over segments
+        }
+    }
+}
+
+// Adds up the difference rows: what a policy gets is the sum of U's rows above its column and V's rows up to it.  A
+// thread takes one histogram bin (or one sum) of one row of the grid and 32 columns: it adds the rows up for the first
+// column and goes on to the next by two.  Bound: L2 (the tables are read once per 32 columns, every policy's histograms
+// are written once).
+constexpr int kSpreadThreads = 128;
+constexpr int kSpreadCols = 32;
+
+template <class T, class F>
+__device__ __forceinline__ T first_column(int c0, int K, F at) {       // at(v, q)
+    T v = 0;
+#pragma unroll 8
+    for (int q = c0 + 1; q <= K; ++q) v += at(0, q);
+#pragma unroll 8
+    for (int q = 0; q <= c0; ++q) v += at(1, q);
+    return v;
+}
+
+template <bool WIDE>
+__global__ void __launch_bounds__(kSpreadThreads)
+k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict__ slabs, int bin_tau,
+         const uint32_t* __restrict__ tab, GridTables gt, unsigned long long* __restrict__ acc,
+         unsigned long long* __restrict__ hist_ttft, unsigned long long* __restrict__ hist_tbt) {
+    grid_dependency_wait();
+    const Slab& sl = slabs[blockIdx.z];
+    const int K = sl.K, T = sl.T, c0 = blockIdx.y * kSpreadCols, c1 = min(K, c0 + kSpreadCols);
+    if (c0 >= K) return;
+    const Tables<WIDE> tb(gt, sl, tr.n_groups);
+    using word = typename Tables<WIDE>::word;
+    const uint32_t* cells = tab + sl.cells;
+    int k = blockIdx.x * kSpreadThreads + threadIdx.x;
+    if (k < kNBins) {                                                  // TTFT: the same for every row
+        auto at = [&](int v, int q) { return tb.ttft_row(v, q)[k]; };
+        uint32_t x = first_column<uint32_t>(c0, K, at);
+        for (int c = c0; c < c1; ++c) {
+            for (int r = 0; r < T; ++r) {
+                const uint32_t p = cells[c * T + r];
+                if (p != kNoPolicy) hist_ttft[(size_t)p * kNBins + k] = x;
+            }
+            if (c + 1 < c1) x += at(1, c + 1) - at(0, c + 1);
+        }
+        return;
+    }
+    k -= kNBins;
+    if (k < T * kNBins) {                                              // TBT
+        const int r = k / kNBins, b = k - r * kNBins;
+        auto at = [&](int v, int q) { return tb.tbt_row(v, q, r)[b]; };
+        word x = first_column<word>(c0, K, at);
+        for (int c = c0; c < c1; ++c) {
+            const uint32_t p = cells[c * T + r];
+            if (p != kNoPolicy) {
+                unsigned long long* h = &hist_tbt[(size_t)p * kNBins + b];
+                if (b == bin_tau) atomicAdd(h, (unsigned long long)x); else *h = x;      // (the regular TBTs join tau's bin below)
+            }
+            if (c + 1 < c1) x += at(1, c + 1) - at(0, c + 1);
+        }
+        return;
+    }
+    k -= T * kNBins;
+    if (k < tr.n_groups * T * kNAcc) {                                 // sums
+        const int s = k % kNAcc, r = (k / kNAcc) % T, g = k / (kNAcc * T);
+        const int cand = gcs[g].candidate;
+        const int fb = s == A_DEVICE_ONLY ? B_DO : s == A_RACE ? B_RACE : s == A_DEVICE_WON ? B_DW : s == A_TOK_DEVICE ? B_TD
+                     : s == A_PRE_SERVER ? B_PS : s == A_PRE_DEVICE ? B_PD : s == A_TTFT_SUM ? B_TT : s == A_TAU_CNT ? B_TAU : -1;
+        int fl = -1;
+        bool minus = false;
+        if (s == A_TOK_DEVICE) { fl = V_A; minus = cand == 2; }        // the server's tokens go to the device, or the device's to the server
+        else if (s == A_PRE_SERVER && cand == 2) fl = V_B;
+        else if (s == A_PRE_DEVICE && cand == 1) fl = V_B;
+        else if (s == A_DELAYED) fl = V_C;
+        else if (s == A_MIGR) fl = V_N;
+        else if (s == A_TAU_CNT) { fl = WIDE ? V_TAU : V_N; minus = !WIDE; }
+        const int f2 = fl < 0 ? -1 : kBase + r * kLev + fl;
+        auto at = [&](int v, int q) {
+            const unsigned long long* row = tb.sum_row(v, g, q);
+            unsigned long long y = fb >= 0 ? row[fb] : 0ull;
+            if (f2 >= 0) y += minus ? 0ull - row[f2] : row[f2];
+            return y;
+        };
+        unsigned long long x = (fb < 0 && f2 < 0) ? 0ull : first_column<unsigned long long>(c0, K, at);
+        for (int c = c0; c < c1; ++c) {
+            const uint32_t p = cells[c * T + r];
+            if (p != kNoPolicy) {
+                unsigned long long* to = acc + ((size_t)p * tr.n_groups + g) * kNAcc + s;
+                if (s == A_TAU_CNT) { *to = 0; if (x) atomicAdd(&hist_tbt[(size_t)p * kNBins + bin_tau], x); }
+                else *to = x;
+            }
+            if (c + 1 < c1) x += at(1, c + 1) - at(0, c + 1);
+        }
+    }
+}
+
+size_t grid_smem(int NT, bool wide) { return sizeof(Smem) + (size_t)(NT + (wide ? 1 : 0)) * kNBins * 4; }
+
+template <int NT, bool WIDE>
+cudaError_t launch_one(const Args& a, int sms, cudaStream_t st) {
+    const size_t smem = grid_smem(NT, WIDE);
+    cudaError_t e = cudaFuncSetAttribute(k_grid<NT, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e) return e;
+    const uint64_t items = (uint64_t)a.n_chunks * a.n_slabs;
+    const uint32_t blocks = (uint32_t)std::min<uint64_t>(items, (uint64_t)sms * (NT == 1 ? 4 : 2));
+    return launch_after(k_grid<NT, WIDE>, dim3(blocks), kThreads, smem, st, a);
+}
+
+}  // namespace
+
+DBG_TRANSLATION_UNIT()
+
+uint64_t grid_ttft_words(int K) { return 2ull * (K + 1) * kNBins; }
+uint64_t grid_tbt_words(int K, int T) { return 2ull * (K + 1) * T * kNBins; }
+uint64_t grid_sum_words(int K, int T, int G) { return 2ull * G * (K + 1) * sum_fields(T); }
+uint32_t grid_blocks_per_sm(int T) { return T == 1 ? 4 : 2; }
+
+cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
+                        const Slab* slabs, uint32_t n_slabs, int T, bool wide, bool count_pairs, const uint32_t* tab,
+                        const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt, LeftLists left,
+                        uint32_t* ticket, uint64_t* work, int sms, cudaStream_t st) {
+    if (n_chunks == 0 || n_slabs == 0) return cudaSuccess;
+    if ((uint64_t)n_chunks * n_slabs > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    const Args a = {tr, rec, gc, cc, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, ticket,
+                    (unsigned long long*)work, count_pairs ? 1 : 0};
+    if (wide) return T == 1 ? launch_one<1, true>(a, sms, st) : T <= 4 ? launch_one<4, true>(a, sms, st) : launch_one<8, true>(a, sms, st);
+    return T == 1 ? launch_one<1, false>(a, sms, st) : T <= 4 ? launch_one<4, false>(a, sms, st) : launch_one<8, false>(a, sms, st);
+}
+
+cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int K, int T,
+                          bool wide, int bin_tau, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
+                          uint64_t* hist_tbt, cudaStream_t st) {
+    if (n_slabs == 0) return cudaSuccess;
+    const uint32_t per = (uint32_t)(kNBins * (1 + T) + tr.n_groups * T * kNAcc);
+    const dim3 grid((per + kSpreadThreads - 1) / kSpreadThreads, (K + kSpreadCols - 1) / kSpreadCols, n_slabs);
+    auto* kernel = wide ? k_spread<true> : k_spread<false>;
+    return launch_after(kernel, grid, kSpreadThreads, 0, st, tr, gc, slabs, bin_tau, tab, gt, (unsigned long long*)acc,
+                        (unsigned long long*)hist_ttft, (unsigned long long*)hist_tbt);
+}
+
+}  // namespace disco

@@ -271,14 +271,13 @@ k_length_cursors(const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ 
 }
 
 // The internal request order: each request takes the next free place of its (group, prompt length).  Requests of
-// one group and length keep no particular order among themselves (nothing downstream depends on it: orig and inv
+// one group and length keep no particular order among themselves (nothing downstream depends on it: req[].z and inv
 // map between the two orders).  The lanes of a warp that share a bucket take their places with one add.  A
-// request goes to its place as one 16-byte record (ticks, lengths, caller's index): one scattered store instead
-// of four; k_unpack_requests then writes the arrays side by side.
+// request goes to its place as one 16-byte record (ticks, lengths, caller's index), which is what the later kernels read.
 __global__ void k_scatter_by_length(uint32_t n, int G, const uint64_t* __restrict__ keys,
                                     const uint16_t* __restrict__ prompt, const uint16_t* __restrict__ outlen,
                                     const int32_t* __restrict__ err, uint32_t* __restrict__ cursor,
-                                    uint4* __restrict__ placed, uint32_t* __restrict__ inv) {
+                                    uint4* __restrict__ req, uint32_t* __restrict__ inv) {
     if (err[0] != 0) return;                          // a rejected trace: its lengths were not all written
     const int lane = threadIdx.x & 31;
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -297,7 +296,7 @@ __global__ void k_scatter_by_length(uint32_t n, int G, const uint64_t* __restric
         if (lane == leader) at = atomicAdd(&cursor[bucket], (uint32_t)__popc(peers));
         at = __shfl_sync(peers, at, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
         if (!DBG_OK(at, n, DBG_K_GATHER, DBG_REQUEST)) continue;
-        placed[at] = make_uint4((uint32_t)key, len | ((uint32_t)outlen[i] << 16), i, 0u);
+        req[at] = make_uint4((uint32_t)key, len | ((uint32_t)outlen[i] << 16), i, 0u);
         inv[i] = at;
     }
 }
@@ -313,7 +312,7 @@ __global__ void __launch_bounds__(kSliceThreads)
 k_scatter_by_length_slices(uint32_t n, int G, const uint64_t* __restrict__ keys,
                            const uint16_t* __restrict__ prompt, const uint16_t* __restrict__ outlen,
                            const int32_t* __restrict__ err, uint32_t* __restrict__ cursor,
-                           uint4* __restrict__ placed, uint32_t* __restrict__ inv) {
+                           uint4* __restrict__ req, uint32_t* __restrict__ inv) {
     extern __shared__ uint32_t s_at[];               // [G][kMaxPrompt + 1]: counts, then next free places
     if (err[0] != 0) return;                         // a rejected trace: its lengths were not all written
     const uint32_t buckets = (uint32_t)G * (uint32_t)(kMaxPrompt + 1);
@@ -338,23 +337,10 @@ k_scatter_by_length_slices(uint32_t n, int G, const uint64_t* __restrict__ keys,
             if (!DBG_OK(g, G, DBG_K_GATHER, DBG_GROUP) || !DBG_OK(len, kMaxPrompt + 1, DBG_K_GATHER, DBG_TABLE)) continue;
             const uint32_t at = atomicAdd(&s_at[g * (uint32_t)(kMaxPrompt + 1) + len], 1u);
             if (!DBG_OK(at, n, DBG_K_GATHER, DBG_REQUEST)) continue;
-            placed[at] = make_uint4((uint32_t)key, len | ((uint32_t)outlen[i] << 16), i, 0u);
+            req[at] = make_uint4((uint32_t)key, len | ((uint32_t)outlen[i] << 16), i, 0u);
             inv[i] = at;
         }
         __syncthreads();
-    }
-}
-
-__global__ void k_unpack_requests(uint32_t n, const uint4* __restrict__ placed, const int32_t* __restrict__ err,
-                                  int32_t* __restrict__ S, uint16_t* __restrict__ l, uint16_t* __restrict__ nout,
-                                  uint32_t* __restrict__ orig) {
-    if (err[0] != 0) return;
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const uint4 r = placed[k];
-        S[k] = (int32_t)r.x;
-        l[k] = (uint16_t)(r.y & 0xFFFFu);
-        nout[k] = (uint16_t)(r.y >> 16);
-        orig[k] = r.z;
     }
 }
 
@@ -469,10 +455,10 @@ DBG_TRANSLATION_UNIT()
 
 uint32_t load_kernel_launches(uint32_t n, int G) {
     if (n == 0) return 1;
-    // ingest, cursors, scatter by length, unpack; (row scan, scatter) x 4, two histograms; group tables
-    if (G == 1 && n <= (1u << 20)) return 4 + 2 * 4 + 2 + 1;
+    // ingest, cursors, scatter by length; (row scan, scatter) x 4, two histograms; group tables
+    if (G == 1 && n <= (1u << 20)) return 3 + 2 * 4 + 2 + 1;
     const uint32_t passes = G > 1 ? 5 : 4;                  // radix passes over (group, ticks)
-    return 4 + 3 * passes + 1 + 1;                          // ..., passes, low words, group tables
+    return 3 + 3 * passes + 1 + 1;                          // ..., passes, low words, group tables
 }
 
 cudaError_t run_load(const LoadArgs& a, cudaStream_t st) {
@@ -507,12 +493,11 @@ cudaError_t run_load(const LoadArgs& a, cudaStream_t st) {
             if ((e = cudaFuncSetAttribute(k_scatter_by_length_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024))) return e;
             const uint32_t slices = (n + kSliceRequests - 1) / kSliceRequests;
             k_scatter_by_length_slices<<<std::min<uint32_t>(slices, 2u * (uint32_t)a.sms), kSliceThreads, cursor_bytes, st>>>(
-                n, G, a.keys_a, a.l_tmp, a.n_tmp, a.err, a.cursors, a.placed, a.inv);
+                n, G, a.keys_a, a.l_tmp, a.n_tmp, a.err, a.cursors, a.req, a.inv);
         } else {
             k_scatter_by_length<<<grid_for(n, 256, a.sms), 256, 0, st>>>(n, G, a.keys_a, a.l_tmp, a.n_tmp, a.err, a.cursors,
-                                                                         a.placed, a.inv);
+                                                                         a.req, a.inv);
         }
-        k_unpack_requests<<<grid_for(n, 256, a.sms), 256, 0, st>>>(n, a.placed, a.err, a.S, a.l, a.nout, a.orig);
         // sort (group, ticks): four byte passes over the ticks, one over the group id
         uint64_t *src = a.keys_a, *dst = a.keys_b;
         const int passes = G > 1 ? 5 : 4;

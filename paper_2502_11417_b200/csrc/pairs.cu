@@ -69,9 +69,8 @@ __device__ __forceinline__ PairOut decide(const PairIn& q, const Prep& pr, uint3
 // outcome only.  The lane that loads a request therefore writes, once, one row of addends per outcome into
 // shared memory; a policy lane decides the outcome and adds the row it selects.
 //
-// Tiles whose policies can be evaluated zone by zone (tile.cuh, zones.cu) have been through that kernel first:
-// this one then takes only the requests it flagged for the tile in the bit mask, packed to the front of the
-// staging area, and returns at once where nothing was flagged.
+// It takes the policies that no grid can (random routing, the Eq. 1-2 wait rule) under every request, and those of a
+// mixed grid (grid.cu) under the requests that kernel listed.
 // ------------------------------------------------------------------------------------------------------
 constexpr int kAccThreads = 512;         // one block per SM: histograms and staging fill its shared memory
 constexpr int kAccWarps = kAccThreads / 32;
@@ -90,11 +89,10 @@ template <bool EXT, bool WIDE>
 __global__ void __launch_bounds__(kAccThreads, 1)
 k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
             const Prep* __restrict__ prep, uint32_t P, const uint32_t* __restrict__ pol_list, uint32_t n_list,
-            int PL, const Chunk* __restrict__ chunks, uint32_t n_tiles, TimelineRec rec, uint32_t k0,
+            int PL, const Chunk* __restrict__ chunks, uint32_t n_tiles, const uint32_t* __restrict__ list,
+            const uint32_t* __restrict__ list_count, TimelineRec rec, uint32_t k0,
             unsigned long long* __restrict__ acc, unsigned long long* __restrict__ hist_ttft,
-            unsigned long long* __restrict__ hist_tbt, const uint32_t* __restrict__ left_mask,
-            const uint32_t* __restrict__ left_count, const uint32_t* __restrict__ left_lists,
-            unsigned long long* __restrict__ work) {
+            unsigned long long* __restrict__ hist_tbt, unsigned long long* __restrict__ work) {
     extern __shared__ uint32_t smem[];
     uint32_t* h_ttft = smem;                                  // [PL][kHWords]
     uint32_t* h_stall = smem + PL * kHWords;                  // [PL][kHWords]
@@ -116,10 +114,13 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
         return;
     const Prep pr = prep[(size_t)g * P + p];
     const int pols_here = (int)min((uint32_t)PL, n_list - tile * PL);
-    // a tile that went through the zone kernel: only the requests it flagged are left (block-uniform)
-    const bool flagged_only = left_mask != nullptr && left_count[(size_t)chunk_id * n_tiles + tile] != kNotByZones;
-    if (flagged_only && left_count[(size_t)chunk_id * n_tiles + tile] == 0u) return;
-    const uint32_t mask_words = left_words_per_request(n_tiles), mask_bit = 1u << (tile & 31u);
+    // with a list: its entries lie where the group's requests do, and the chunk stands for as many of them
+    uint32_t r_hi = ch.len;
+    if (list) {
+        const uint32_t at = ch.start - tr.grp_off[g], have = list_count[g];
+        r_hi = have > at ? min(ch.len, have - at) : 0u;
+        if (r_hi == 0u) return;                               // (block-uniform)
+    }
     const GroupConst& gc = gcs[g];
     const ClassConst& cc = *ccp;
     const uint32_t kappa = (uint32_t)gc.kappa, c0 = (uint32_t)gc.c0;
@@ -127,7 +128,7 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
     const float delta_c = gc.delta_c;
     const int W0 = cc.W[0], W1 = cc.W[1], W2 = cc.W[2];
     const int kt0 = cc.ktau[g][0], kt1 = cc.ktau[g][1], kt2 = cc.ktau[g][2];
-    const uint32_t tau = (uint32_t)cc.tau;
+    const uint32_t tau = (uint32_t)cc.tau, even = cc.even[g];
 
     // With no waits in the tile (Algorithm 3, random routing) a TTFT is the request's S or its T_d, whose
     // histogram increments are staged; otherwise the bin is worked out per pair.
@@ -138,12 +139,7 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
     uint32_t* my_ttft = h_ttft + pol_in_tile * kHWords;
     uint32_t* my_stall = h_stall + pol_in_tile * kHWords;
 
-    // The block-private histogram counters are 16 bits wide: at most 65,280 requests are evaluated between two
-    // flushes.  A longer chunk (one that the zone kernel left more than that of, or took nothing of) goes in passes.
-    const uint32_t to_do = flagged_only ? left_count[(size_t)chunk_id * n_tiles + tile] : ch.len;
-    const uint32_t pass_len = to_do <= 65280u ? ch.len : 65280u;
-    for (uint32_t r_lo = 0; r_lo < ch.len; r_lo += pass_len) {
-    const uint32_t r_hi = min(ch.len, r_lo + pass_len);
+    // (the block-private histogram counters are 16 bits wide: a chunk holds at most 65,280 requests)
     for (int i = threadIdx.x; i < 2 * PL * kHWords + 2 * PL * kNAcc; i += kAccThreads) smem[i] = 0;   // (staging needs no clearing)
     __syncthreads();
 
@@ -167,34 +163,30 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
     const uint32_t lth16 = (uint32_t)max(l_th, 0) << 4;      // against a staged (l << 4 | outcome at w = 0)
 
     // One request per lane, fetched a batch ahead so that the loads fly while the previous batch is evaluated.
-    struct Raw { uint32_t l, n, S, m, dly, stall, nt0, nt1, nt2, orig; };   // as loaded: nothing may consume a load early
+    struct Raw { uint4 q; uint2 hand; uint32_t nt0, nt1, nt2, kk; };   // as loaded: nothing may consume a load early
     auto fetch = [&](uint32_t at) {                              // the request at position `at` of the chunk
-        const uint32_t kk = ch.start + min(at, r_hi - 1);
-        Raw q;
-        q.l = tr.l[kk]; q.n = tr.nout[kk]; q.S = (uint32_t)tr.S[kk];
-        q.m = rec.m[kk]; q.dly = rec.delayed[kk]; q.stall = rec.stall[kk];
-        if (rec.tau) {                                           // every interval but a hand-off's equals tau
-            q.nt0 = q.nt1 = q.n - 1;
-            q.nt2 = q.m ? q.n - 2 : 0u;
-        } else {
-            q.nt0 = kt0 >= 0 ? rec.win[0][(size_t)kk * W0 + kt0] : 0u;
-            q.nt1 = kt1 >= 0 ? rec.win[1][(size_t)kk * W1 + kt1] : 0u;
-            q.nt2 = kt2 >= 0 ? rec.win[2][(size_t)kk * W2 + kt2] : 0u;
-        }
-        q.orig = EXT ? tr.orig[kk] : 0u;
-        return q;
+        Raw x;
+        x.kk = ch.start + min(at, r_hi - 1);
+        if (list) x.kk = list[x.kk];
+        if (!DBG_OK(x.kk, tr.n, DBG_K_PAIRS_ACC, DBG_REQUEST)) x.kk = ch.start;
+        x.q = tr.req[x.kk]; x.hand = rec.hand[x.kk];
+        x.nt0 = (!(even & 1u) && kt0 >= 0) ? rec.win[0][(size_t)x.kk * W0 + kt0] : 0u;
+        x.nt1 = (!(even & 2u) && kt1 >= 0) ? rec.win[1][(size_t)x.kk * W1 + kt1] : 0u;
+        x.nt2 = (!(even & 4u) && kt2 >= 0) ? rec.win[2][(size_t)x.kk * W2 + kt2] : 0u;
+        return x;
     };
     // Stages the requests of the lanes in `taken`, packed to the front of the staging area, and evaluates them under
-    // the tile's policies.  b0: chunk position of lane 0's request when the lanes hold a batch in order.
-    auto run_batch = [&](const Raw& cur, uint32_t taken, uint32_t b0) {
+    // the tile's policies.
+    auto run_batch = [&](const Raw& cur, uint32_t taken) {
         const int n_here = __popc(taken);
         staged += (uint32_t)n_here;
         if (((taken >> lane) & 1u) && DBG_OK(__popc(taken & ((1u << lane) - 1u)), kStageReq, DBG_K_PAIRS_ACC, DBG_SLOT)) {
             const int at = __popc(taken & ((1u << lane) - 1u));
-            const uint32_t l = cur.l, n = cur.n, S = cur.S, m = cur.m;
-            const uint32_t stall = cur.stall, dly = cur.dly;
-            const uint32_t nt0 = cur.nt0, nt1 = cur.nt1;
-            uint32_t nt2 = cur.nt2;
+            const uint32_t l = cur.q.y & 0xFFFFu, n = cur.q.y >> 16, S = cur.q.x, m = cur.hand.x & 0xFFFFu;
+            const uint32_t stall = cur.hand.y, dly = cur.hand.x >> 16;
+            // TBTs in tau's bin; of a stream that keeps the pace, all of them (but a hand-off's)
+            const uint32_t nt0 = (even & 1u) ? n - 1u : cur.nt0, nt1 = (even & 2u) ? n - 1u : cur.nt1;
+            uint32_t nt2 = (even & 4u) ? n - 2u : cur.nt2;
             uint32_t stall_code = 0u;                          // the token after a hand-off: counted with tau's bin,
             if (stall == tau) ++nt2; else stall_code = hist16_code(bin_of_ticks(stall));   // else an increment of its own
             // a request may only migrate if its buffer filled (m != 0); fold that into the saving (Eq. 4)
@@ -228,7 +220,7 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
             b[O_RACE_DEV] = make_uint4(0u, 0x00010100u, oT, iT);
             b[O_MIGR_TO_DEV] = make_uint4(dly << 17 | stall_code, 0x01000100u, oS, iS);
             b[O_MIGR_TO_SRV] = make_uint4(dly << 17 | stall_code, 0x01010100u, oT, iT);
-            b[6] = make_uint4(0u, EXT ? routing_draw(k0, cur.orig) : 0u, m, n);
+            b[6] = make_uint4(cur.kk, EXT ? routing_draw(k0, cur.q.z) : 0u, m, n);
         }
         __syncwarp();
         // kIlp requests at a time per lane, phase by phase, so that the shared-memory loads of one do not
@@ -315,9 +307,9 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
                 for (int k = 0; k < kIlp; ++k) {
                     if (!kAllOk && !ok[k]) continue;
                     const int c = migr[k] ? 2 : (dev_wins[k] ? 1 : 0);
+                    if ((even >> c) & 1u) continue;
                     const int W = c == 2 ? W2 : (c == 1 ? W1 : W0), kt = c == 2 ? kt2 : (c == 1 ? kt1 : kt0);
-                    // (no bit mask with wide windows: the staged requests are the batch's first ones, in order)
-                    const uint32_t* wp = rec.win[c] + (size_t)(ch.start + b0 + rr[k]) * W;
+                    const uint16_t* wp = rec.win[c] + (size_t)stB[rr[k] * kStageVec + 6].x * W;
                     unsigned long long* hp = hist_tbt + (size_t)p * kNBins + cc.lo[g][c];
                     for (int j = 0; j < W; ++j) {
                         const uint32_t v = j == kt ? 0u : wp[j];
@@ -355,60 +347,13 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
         }
         cnt_a += __byte_perm(cnt8, 0u, 0x4140); cnt_b += __byte_perm(cnt8, 0u, 0x4342); cnt8 = 0;
     };
-    if (!flagged_only) {
-        // ---- every request of the range: one per lane, fetched a batch ahead so that the loads fly while the
-        //      previous batch is evaluated
-        Raw nx = fetch(r_lo + wib * kStageReq + lane);
-        for (uint32_t b0 = r_lo + wib * kStageReq; b0 < r_hi; b0 += kAccWarps * kStageReq) {
-            const Raw cur = nx;
-            if (b0 + kAccWarps * kStageReq < r_hi) nx = fetch(b0 + kAccWarps * kStageReq + lane);
-            __syncwarp();
-            run_batch(cur, __ballot_sync(0xFFFFFFFFu, b0 + lane < r_hi), b0);
-        }
-    } else {
-        // ---- only the requests the zone kernel flagged for this tile: the warp reads the flags of 32 requests at a
-        //      time and collects the flagged ones, one per lane, until it holds (nearly) a full batch
-        uint32_t held = 0;                                       // chunk position of the request this lane holds
-        int n_held = 0;                                          // warp-uniform
-        auto work_off = [&]() {
-            const Raw d = fetch(held);                           // (lanes beyond n_held fetch a valid request and drop it)
-            __syncwarp();
-            run_batch(d, n_held == 32 ? 0xFFFFFFFFu : (1u << n_held) - 1u, 0u);
-            n_held = 0;
-        };
-        if (left_lists && to_do <= kLeftList) {
-            // few enough to be listed by position: no scan
-            const uint32_t* list = left_lists + ((size_t)chunk_id * n_tiles + tile) * kLeftList;
-            for (uint32_t k0l = wib * 32u; k0l < to_do; k0l += kAccWarps * 32u) {
-                n_held = (int)min(32u, to_do - k0l);
-                if (lane < n_held) held = list[k0l + lane];
-                work_off();
-            }
-        } else {
-        constexpr int kScan = 4;                                 // flag words a lane has in flight
-        constexpr uint32_t kStride = kAccWarps * kStageReq;
-        auto flags_at = [&](uint32_t at) {
-            return at < r_hi ? left_mask[(size_t)(ch.start + at) * mask_words + (tile >> 5)] & mask_bit : 0u;
-        };
-        for (uint32_t c0 = r_lo + wib * kStageReq; c0 < r_hi; c0 += kScan * kStride) {
-            const uint32_t f0 = flags_at(c0 + lane), f1 = flags_at(c0 + kStride + lane);
-            const uint32_t f2 = flags_at(c0 + 2 * kStride + lane), f3 = flags_at(c0 + 3 * kStride + lane);
-            static_assert(kScan == 4, "four flag words are loaded by name");
-#pragma unroll 1
-            for (int j = 0; j < kScan; ++j) {                    // (not unrolled: the batch evaluation is long code)
-                const uint32_t b0 = c0 + j * kStride;
-                const uint32_t taken = __ballot_sync(0xFFFFFFFFu, (j == 0 ? f0 : j == 1 ? f1 : j == 2 ? f2 : f3) != 0u);
-                if (taken == 0u) continue;
-                const int n_new = __popc(taken);
-                if (n_held + n_new > 32) work_off();
-                const int want = lane - n_held;                  // lane n_held + j takes the j-th flagged request
-                if (want >= 0 && want < n_new) held = b0 + __fns(taken, 0, want + 1);
-                n_held += n_new;
-                if (n_held >= 28) work_off();
-            }
-        }
-        if (n_held > 0) work_off();
-        }
+    // ---- one request per lane, fetched a batch ahead so that the loads fly while the previous batch is evaluated
+    Raw nx = fetch(wib * kStageReq + lane);
+    for (uint32_t b0 = wib * kStageReq; b0 < r_hi; b0 += kAccWarps * kStageReq) {
+        const Raw cur = nx;
+        if (b0 + kAccWarps * kStageReq < r_hi) nx = fetch(b0 + kAccWarps * kStageReq + lane);
+        __syncwarp();
+        run_batch(cur, __ballot_sync(0xFFFFFFFFu, b0 + lane < r_hi));
     }
     // ---- block totals, then one flush per block.  With fewer than 32 policies in the tile several lanes of a warp
     //      hold sums of the same policy: they are added up by shuffles first, so that one lane per policy and warp
@@ -454,8 +399,6 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
         if (s == A_TAU_CNT) atomicAdd(&hist_tbt[(size_t)pp * kNBins + bin_tau], v);   // TBTs equal to tau
         else atomicAdd(&acc[((size_t)pp * tr.n_groups + g) * kNAcc + s], v);
     }
-    __syncthreads();
-    }   // next pass
 }
 
 size_t acc_smem_bytes(int PL) {
@@ -497,7 +440,8 @@ __device__ __forceinline__ RowPol row_pol(const Prep& pr, int candidate, uint32_
 // IDX32: every element index p * N + i fits 32 bits, so a store address is one widening multiply-add.
 template <bool EXT, bool IDX32>
 __global__ void __launch_bounds__(kRowThreads)
-k_pairs_rows(TraceDev tr, const GroupConst* __restrict__ gcs, const Prep* __restrict__ prep, uint32_t P,
+k_pairs_rows(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
+             const Prep* __restrict__ prep, uint32_t P,
              const uint32_t* __restrict__ pol_list, uint32_t n_list, TimelineRec rec, uint32_t k0,
              disco_pair_out_t out) {
     using idx_t = typename std::conditional<IDX32, uint32_t, size_t>::type;
@@ -526,9 +470,11 @@ k_pairs_rows(TraceDev tr, const GroupConst* __restrict__ gcs, const Prep* __rest
     // one group: a thread per request in the caller's order, so that the rows are written side by side (the reads
     // are scattered instead, once per request); several groups: the block's policies depend on the group, a thread
     // per request in the internal order
-    uint32_t orig = k;
-    if (tr.n_groups == 1) k = tr.inv[k]; else orig = tr.orig[k];
+    if (tr.n_groups == 1) k = tr.inv[k];
     if (!DBG_OK(k, tr.n, DBG_K_PAIRS_ROWS, DBG_REQUEST)) return;
+    const uint4 rq = tr.req[k];
+    const uint2 hand = rec.hand[k];
+    const uint32_t orig = rq.z;
     int g = g_lo;
     while (g < g_hi && k >= tr.grp_off[g + 1]) ++g;
     const GroupConst& gc = gcs[g];
@@ -538,25 +484,27 @@ k_pairs_rows(TraceDev tr, const GroupConst* __restrict__ gcs, const Prep* __rest
     const idx_t N = (idx_t)tr.n;
 
     PairIn q;
-    q.l = tr.l[k]; q.n = tr.nout[k]; q.S = (uint32_t)tr.S[k]; q.m = rec.m[k];
+    q.l = rq.y & 0xFFFFu; q.n = rq.y >> 16; q.S = rq.x; q.m = hand.x & 0xFFFFu;
     q.saving = delta_c * (float)(q.n - q.m);
     q.delta_c = delta_c;
     q.u = EXT ? routing_draw(k0, orig) : 0u;
-    const uint32_t Td = (uint32_t)gc.kappa * q.l + (uint32_t)gc.c0, dly = rec.delayed[k];
+    const uint32_t Td = (uint32_t)gc.kappa * q.l + (uint32_t)gc.c0, dly = hand.x >> 16;
     const float saving_m = q.m ? q.saving : -1.0f;        // a request migrates only if its buffer filled (m != 0)
     const uint4* row = s_rows + threadIdx.x * kRowVec;
     {
         uint4* wrow = s_rows + threadIdx.x * kRowVec;
         const float inv_cnt = q.n > 1 ? 1e-6f / (float)(q.n - 1) : 0.0f;
+        const bool exact = ccp->kind[g] == G_EXACT;
+        const uint32_t tau = (uint32_t)ccp->tau;
         float mean[3], mx[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             uint32_t sum, most;
-            if (rec.tau) {                            // every interval equals tau, but the one after a hand-off (stream 2)
+            if (exact) {                              // every interval equals tau, but the one after a hand-off (stream 2)
                 const uint32_t nI = q.n - 1;
-                const uint32_t stall = (c == 2 && q.m) ? rec.stall[k] : 0u;
-                sum = c < 2 ? nI * rec.tau : (q.m ? (nI - 1) * rec.tau + stall : 0u);
-                most = c < 2 ? (nI ? rec.tau : 0u) : stall;
+                const uint32_t stall = (c == 2 && q.m) ? hand.y : 0u;
+                sum = c < 2 ? nI * tau : (q.m ? (nI - 1) * tau + stall : 0u);
+                most = c < 2 ? (nI ? tau : 0u) : stall;
             } else {
                 sum = rec.sum[c][k]; most = rec.max[c][k];
             }
@@ -624,13 +572,12 @@ k_pairs_rows(TraceDev tr, const GroupConst* __restrict__ gcs, const Prep* __rest
 
 DBG_TRANSLATION_UNIT()
 
-cudaError_t launch_pairs(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
-                         const uint32_t* pol_list, uint32_t n_list, const Chunk* chunks, uint32_t n_chunks,
-                         TimelineRec rec, disco_pair_out_t out, uint64_t* acc, uint64_t* hist_ttft,
-                         uint64_t* hist_tbt, uint32_t* left_mask, uint32_t* left_count, uint32_t* left_lists,
-                         uint32_t zone_blocks, uint32_t* zone_ticket, uint64_t* work, uint32_t k0,
-                         bool extras, bool wide, cudaEvent_t mid, cudaStream_t st) {
-    if (n_chunks == 0 || n_list == 0) return mid ? cudaEventRecord(mid, st) : cudaSuccess;
+cudaError_t launch_pairs_acc(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
+                             const uint32_t* pol_list, uint32_t n_list, const Chunk* chunks, uint32_t n_chunks,
+                             const uint32_t* list, const uint32_t* list_count, TimelineRec rec, uint64_t* acc,
+                             uint64_t* hist_ttft, uint64_t* hist_tbt, uint64_t* work, uint32_t k0, bool extras, bool wide,
+                             cudaStream_t st) {
+    if (n_chunks == 0 || n_list == 0) return cudaSuccess;
     int PL = 1;
     while (PL < 32 && (uint32_t)PL < n_list) PL <<= 1;
     auto* acc_kernel = extras ? (wide ? k_pairs_acc<true, true> : k_pairs_acc<true, false>)
@@ -640,32 +587,19 @@ cudaError_t launch_pairs(const TraceDev& tr, const GroupConst* gc, const ClassCo
     if (e) return e;
     const uint32_t n_tiles = (n_list + PL - 1) / PL;
     if ((uint64_t)n_chunks * n_tiles > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    // zone by zone first (tiles it cannot take return at once), then pair by pair what is left
-    const bool zones = !wide && left_mask != nullptr;
-    if (zones) {
-        const size_t mask_bytes = (size_t)tr.n * left_words_per_request(n_tiles) * 4;
-        if ((e = cudaMemsetAsync(left_mask, 0, mask_bytes, st))) return e;
-        if ((e = launch_pairs_zones(tr, gc, cc, prep, P, pol_list, n_list, PL, chunks, n_chunks, rec, acc, hist_ttft,
-                                    hist_tbt, left_mask, left_count, left_lists, zone_blocks, zone_ticket, work, st)))
-            return e;
-    }
-    if ((e = launch_after(acc_kernel, dim3(n_chunks * n_tiles), kAccThreads, acc_smem_bytes(PL), st, tr, gc, cc, prep, P,
-                          pol_list, n_list, PL, chunks, n_tiles, rec, k0, (unsigned long long*)acc,
-                          (unsigned long long*)hist_ttft, (unsigned long long*)hist_tbt,
-                          (const uint32_t*)(zones ? left_mask : nullptr), (const uint32_t*)left_count,
-                          (const uint32_t*)left_lists, (unsigned long long*)work)))
-        return e;
-    if (mid && (e = cudaEventRecord(mid, st))) return e;
-    const bool rows = out.ttft_s || out.tbt_mean_s || out.tbt_max_s || out.cost || out.tok_server || out.tok_device ||
-                      out.mig_at || out.delayed || out.decision;
-    if (rows) {
-        const bool idx32 = (uint64_t)P * tr.n <= 0xFFFFFFFFull;
-        auto* row_kernel = extras ? (idx32 ? k_pairs_rows<true, true> : k_pairs_rows<true, false>)
-                                  : (idx32 ? k_pairs_rows<false, true> : k_pairs_rows<false, false>);
-        dim3 grid_r((tr.n + kRowThreads - 1) / kRowThreads, (n_list + kRowPols - 1) / kRowPols);
-        e = launch_after(row_kernel, grid_r, kRowThreads, 0, st, tr, gc, prep, P, pol_list, n_list, rec, k0, out);
-    }
-    return e;
+    return launch_after(acc_kernel, dim3(n_chunks * n_tiles), kAccThreads, acc_smem_bytes(PL), st, tr, gc, cc, prep, P,
+                        pol_list, n_list, PL, chunks, n_tiles, list, list_count, rec, k0, (unsigned long long*)acc,
+                        (unsigned long long*)hist_ttft, (unsigned long long*)hist_tbt, (unsigned long long*)work);
+}
+
+cudaError_t launch_pairs_rows(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
+                              const uint32_t* pol_list, uint32_t n_list, TimelineRec rec, const disco_pair_out_t& out,
+                              uint32_t k0, bool extras, cudaStream_t st) {
+    const bool idx32 = (uint64_t)P * tr.n <= 0xFFFFFFFFull;
+    auto* row_kernel = extras ? (idx32 ? k_pairs_rows<true, true> : k_pairs_rows<true, false>)
+                              : (idx32 ? k_pairs_rows<false, true> : k_pairs_rows<false, false>);
+    dim3 grid_r((tr.n + kRowThreads - 1) / kRowThreads, (n_list + kRowPols - 1) / kRowPols);
+    return launch_after(row_kernel, grid_r, kRowThreads, 0, st, tr, gc, cc, prep, P, pol_list, n_list, rec, k0, out);
 }
 
 }  // namespace disco

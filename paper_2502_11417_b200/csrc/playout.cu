@@ -1,4 +1,5 @@
-// Decode play-out (Sec. 4.3): warps play requests cooperatively, every token of every stream.
+// Decode play-out (Sec. 4.3) of the groups whose streams may clamp at some tokens and not at others (G_GENERAL, paced):
+// warps play requests cooperatively, every token of every stream.
 //
 // A stream's delivery times follow d_1 = 0, d_j = max(g_j, d_{j-1} + tau) over generation times
 // g_j = g_{j-1} + x_j, x_j = T + jitter(hash(seed, request, j)).  With e_j = d_j - g_j (how far delivery lags
@@ -14,8 +15,9 @@
 // it; while nothing clamps it follows from the two streams' prefix sums, otherwise it is played out in a
 // second pass.
 //
-// A warp takes 32 consecutive requests at a time: their inputs are loaded and their results stored one
-// request per lane, so the per-request memory traffic is coalesced and paid once per 32 requests.
+// A warp takes 32 consecutive requests of one group at a time: their inputs are loaded and their results stored one
+// request per lane, so the per-request memory traffic is coalesced and paid once per 32 requests.  TBTs other than
+// tau are counted in windows of histogram bins in shared memory of the warp's own and written once per request.
 #include <algorithm>
 #include <climits>
 
@@ -43,7 +45,6 @@ struct Round {                           // what a lane knows about the current 
     uint32_t j0, last_j, n;              // lane's first token, round's last valid token, output length
     uint32_t round_valid;                // valid tokens in the round
     int32_t tau_eff;
-    bool pacing;
     int32_t* err;
 };
 
@@ -118,7 +119,7 @@ __device__ __forceinline__ void play_round(WS& st, uint32_t& mxl, uint32_t& ntl,
                                            bool nonneg, const Round& rd, uint32_t* win, int lo, int W, bool search,
                                            uint32_t B, int32_t thr, uint32_t& clean_until, uint32_t* ring,
                                            uint32_t& m_out, int32_t& em_out) {
-    if (rd.pacing && nonneg && !(search && !st.clean)) {   // no clamp: every TBT of the round equals tau
+    if (nonneg && !(search && !st.clean)) {   // no clamp: every TBT of the round equals tau
         const int32_t tot = __reduce_add_sync(FULL, s);
         if (search) {
             // clean stream: d_q = (q-1) tau, so d_{j-B+1} > g_j  <=>  S_j > (B-1) tau, and S is non-decreasing
@@ -153,7 +154,7 @@ __device__ __forceinline__ void play_round(WS& st, uint32_t& mxl, uint32_t& ntl,
             e = max(v, 0);
             const uint32_t ex = (uint32_t)(e - v);                                 // TBT - tau
             mxl = max(mxl, ex);
-            if (rd.pacing && ex == 0) ++ntl; else count_slow((uint32_t)rd.tau_eff + ex, win, lo, W, rd.err);
+            if (ex == 0) ++ntl; else count_slow((uint32_t)rd.tau_eff + ex, win, lo, W, rd.err);
             if (search) {
                 run += c[t];
                 const uint32_t j = rd.j0 + t;
@@ -198,7 +199,6 @@ __device__ __forceinline__ uint32_t handoff_latency(const GroupClass& G, uint32_
 __device__ __noinline__ void play_x(const GroupClass& G, Round rd, uint32_t key, uint32_t nI, uint32_t m, uint32_t M,
                                     uint32_t* win2, int W2, XResult* out) {
     const int32_t tau_eff = rd.tau_eff;
-    const bool pacing = rd.pacing;
     const int32_t cM = tau_eff - (int32_t)M;
     const uint32_t mulC = G.cand == 1 ? G.mulS : G.mulD, mulT = G.cand == 1 ? G.mulD : G.mulS;
     const int32_t cC_base = G.cand == 1 ? G.cS_base : G.cD_base, cT_base = G.cand == 1 ? G.cD_base : G.cS_base;
@@ -234,9 +234,9 @@ __device__ __noinline__ void play_x(const GroupClass& G, Round rd, uint32_t key,
             }
         }
         const bool special = base + 2 <= m + 1 && rd.last_j >= m;        // round holds token m or m+1
-        const bool late = pacing && D0_known && D0 + sX.S < 0;           // tokens may still miss their slots
+        const bool late = D0_known && D0 + sX.S < 0;           // tokens may still miss their slots
         const bool nonneg = !__any_sync(FULL, neg < 0);
-        if (pacing && !special && !late && nonneg) {
+        if (!special && !late && nonneg) {
             const int32_t tot = __reduce_add_sync(FULL, s);
             sX.e += tot; sX.S += tot; sX.nt += rd.round_valid;
             continue;
@@ -254,7 +254,7 @@ __device__ __noinline__ void play_x(const GroupClass& G, Round rd, uint32_t key,
                 mxX = max(mxX, ex);
                 run += cx[t];
                 if (j == m + 1) stall = (uint32_t)tau_eff + ex;          // kept apart from the regular TBTs
-                else if (pacing && ex == 0) ++ntX;
+                else if (ex == 0) ++ntX;
                 else count_slow((uint32_t)tau_eff + ex, win2, G.lo2, W2, rd.err);
                 if (j == m) em_minus_Sm = e - run;
             }
@@ -265,7 +265,7 @@ __device__ __noinline__ void play_x(const GroupClass& G, Round rd, uint32_t key,
         } else if (m == 1 && base == 0) {
             D0 = 0; D0_known = true;                                     // e_1 = S_1 = 0
         }
-        if (pacing && D0_known) {                                        // generated after d_m + (j-m) tau ?
+        if (D0_known) {                                        // generated after d_m + (j-m) tau ?
             run = S_in;
 #pragma unroll
             for (int t = 0; t < kR; ++t)
@@ -285,70 +285,73 @@ __device__ __noinline__ void play_x(const GroupClass& G, Round rd, uint32_t key,
 
 __global__ void __launch_bounds__(kWarps * 32)
 k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
-          const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int32_t* err,
-          const uint32_t* __restrict__ todo, const uint32_t* __restrict__ todo_count, uint32_t count_imm) {
-    // Requests to play: todo[0 .. *todo_count), or 0 .. count_imm when there is no list.
+          const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int32_t* err) {
     __shared__ uint32_t ring_s[kWarps][kRing];
     __shared__ XResult xres_s[kWarps];
+    extern __shared__ uint32_t s_win[];                                // [warps][W0 + W1 + W2]
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     grid_dependency_wait();
-    const uint32_t count = todo_count ? *todo_count : count_imm;
-    for (uint32_t batch0 = (blockIdx.x * kWarps + wib) * 32u; batch0 < count; batch0 += gridDim.x * kWarps * 32u) {
-    uint32_t* ring = ring_s[wib];
     const ClassConst& cc = *ccp;
     const int32_t tau_eff = cc.tau_eff, tau = cc.tau;
-    const bool pacing = cc.pacing != 0;
     const int W0 = cc.W[0], W1 = cc.W[1], W2 = cc.W[2];
     const uint32_t B = (uint32_t)cc.B;
     const long long thr64 = (long long)(B ? B - 1 : 0) * tau;
     const int32_t thr = thr64 > INT_MAX ? INT_MAX : (int32_t)thr64;
+    uint32_t* ring = ring_s[wib];
+    uint32_t* win0 = s_win + wib * (W0 + W1 + W2);
+    uint32_t* win1 = win0 + W0;
+    uint32_t* win2 = win1 + W1;
+    for (int i = lane; i < W0 + W1 + W2; i += 32) win0[i] = 0;
+    __syncwarp();
+    for (uint32_t batch = blockIdx.x * kWarps + wib;; batch += gridDim.x * kWarps) {
+    int g;
+    uint32_t k_lo, n_here;
+    if (!batch_of_kind(tr, cc, G_GENERAL, batch, g, k_lo, n_here)) break;
 
     // ---- one request per lane: inputs
-    bool live = batch0 + lane < count;
-    const uint32_t kk = !live ? 0u : (todo ? todo[batch0 + lane] : batch0 + lane);
-    if (live && !DBG_OK(kk, tr.n, DBG_K_PLAYOUT, DBG_REQUEST)) live = false;
+    const bool live = lane < (int)n_here;
+    const uint32_t kk = k_lo + lane;
     uint32_t n_l = 1, l_l = 1, key_l = 0;
-    int g_l = 0;
     if (live) {
-        n_l = tr.nout[kk]; l_l = tr.l[kk];
-        key_l = mix32(k0 + tr.orig[kk] * kHashReq);
-        while (g_l + 1 < tr.n_groups && kk >= tr.grp_off[g_l + 1]) ++g_l;
-        for (int i = 0; i < W0; ++i) rec.win[0][(size_t)kk * W0 + i] = 0;
-        for (int i = 0; i < W1; ++i) rec.win[1][(size_t)kk * W1 + i] = 0;
-        for (int i = 0; i < W2; ++i) rec.win[2][(size_t)kk * W2 + i] = 0;
+        const uint4 q = tr.req[kk];
+        n_l = q.y >> 16; l_l = q.y & 0xFFFFu;
+        key_l = mix32(k0 + q.z * kHashReq);
     }
-    __syncwarp();
     // ---- one request per lane: results
     uint32_t o_sumS = 0, o_maxS = 0, o_sumD = 0, o_maxD = 0, o_sumX = 0, o_maxX = 0, o_stall = 0, o_m = 0, o_dl = 0;
-    uint32_t o_ntS = 0, o_ntD = 0, o_ntX = 0;
 
     GroupClass G;
-    int cur_g = -1;
+    {
+        const GroupConst& gc = gcs[g];
+        G.mulS = 2u * (uint32_t)gc.J_srv + 1u; G.mulD = 2u * (uint32_t)gc.J_dev + 1u;
+        G.cS_base = tau_eff - (gc.T_srv - gc.J_srv); G.cD_base = tau_eff - (gc.T_dev - gc.J_dev);
+        G.kappa = gc.kappa; G.c0 = gc.c0;
+        G.cand = cc.mig_any ? gc.candidate : 0;
+        G.lo0 = cc.lo[g][0]; G.lo1 = cc.lo[g][1]; G.lo2 = cc.lo[g][2];
+        G.kt0 = cc.ktau[g][0]; G.kt1 = cc.ktau[g][1]; G.kt2 = cc.ktau[g][2];
+        G.K = knots + g * kNKnots;
+    }
+    const bool evenS = (cc.even[g] & 1u) != 0, evenD = (cc.even[g] & 2u) != 0;
     Round rd;
-    rd.lane = lane; rd.tau_eff = tau_eff; rd.pacing = pacing; rd.err = err;
-    const int n_here = (int)min(32u, count - batch0);
+    rd.lane = lane; rd.tau_eff = tau_eff; rd.err = err;
 
-    for (int r = 0; r < n_here; ++r) {
+    for (int r = 0; r < (int)n_here; ++r) {
         const uint32_t n = __shfl_sync(FULL, n_l, r), l = __shfl_sync(FULL, l_l, r);
         const uint32_t key = __shfl_sync(FULL, key_l, r);
-        const int g = __shfl_sync(FULL, g_l, r);
-        const uint32_t k = __shfl_sync(FULL, kk, r);
-        if (g != cur_g && DBG_OK(g, tr.n_groups, DBG_K_PLAYOUT, DBG_GROUP)) {
-            cur_g = g;
-            const GroupConst& gc = gcs[g];
-            G.mulS = 2u * (uint32_t)gc.J_srv + 1u; G.mulD = 2u * (uint32_t)gc.J_dev + 1u;
-            G.cS_base = tau_eff - (gc.T_srv - gc.J_srv); G.cD_base = tau_eff - (gc.T_dev - gc.J_dev);
-            G.kappa = gc.kappa; G.c0 = gc.c0;
-            G.cand = cc.mig_any ? gc.candidate : 0;
-            G.lo0 = cc.lo[g][0]; G.lo1 = cc.lo[g][1]; G.lo2 = cc.lo[g][2];
-            G.kt0 = cc.ktau[g][0]; G.kt1 = cc.ktau[g][1]; G.kt2 = cc.ktau[g][2];
-            G.K = knots + g * kNKnots;
-        }
+        const uint32_t k = k_lo + (uint32_t)r;
         const uint32_t nI = n - 1;                                     // inter-token intervals, tokens 2..n
-        if (nI == 0) continue;                                         // a single token: all results stay 0
-        uint32_t* win0 = rec.win[0] + (size_t)k * W0;
-        uint32_t* win1 = rec.win[1] + (size_t)k * W1;
-        uint32_t* win2 = rec.win[2] + (size_t)k * W2;
+        // the request's windows go out (streams that keep the pace store none) and are cleared for the next one
+        auto windows_out = [&](uint32_t tS, uint32_t tD, uint32_t tX, bool has_x) {
+            __syncwarp();
+            if (!evenS)
+                for (int i = lane; i < W0; i += 32) { rec.win[0][(size_t)k * W0 + i] = (uint16_t)(win0[i] + (i == G.kt0 ? tS : 0u)); win0[i] = 0; }
+            if (!evenD)
+                for (int i = lane; i < W1; i += 32) { rec.win[1][(size_t)k * W1 + i] = (uint16_t)(win1[i] + (i == G.kt1 ? tD : 0u)); win1[i] = 0; }
+            if (has_x)
+                for (int i = lane; i < W2; i += 32) { rec.win[2][(size_t)k * W2 + i] = (uint16_t)(win2[i] + (i == G.kt2 ? tX : 0u)); win2[i] = 0; }
+            __syncwarp();
+        };
+        if (nI == 0) { windows_out(0u, 0u, 0u, false); continue; }     // a single token: all results stay 0
         const int cand = G.cand;
         rd.n = n;
         WS sS = {0, 0, 0, true}, sD = {0, 0, 0, true};
@@ -362,7 +365,7 @@ k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __r
         uint32_t M = 0, dl_clean = 0;
         int32_t v_m1 = 0, need = 0, carry = 0;
         bool counting = false;
-        if (m && pacing) {
+        if (m) {
             M = handoff_latency(G, key, l, m);
             v_m1 = tau_eff - (int32_t)M;
             if (v_m1 < 0) { counting = true; need = -v_m1; dl_clean = 1; }
@@ -396,7 +399,7 @@ k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __r
             const bool searching = cand != 0 && m == 0;
             const bool cand_clean = cand == 1 ? sS.clean : sD.clean;
             const int32_t cand_after = cand == 1 ? sS.S + totS : sD.S + totD;
-            if (pacing && posS && posD && !counting && !(searching && (!cand_clean || cand_after > thr))) {
+            if (posS && posD && !counting && !(searching && (!cand_clean || cand_after > thr))) {
                 // nothing clamps, the buffer does not fill in this round: every TBT equals tau
                 sS.e += totS; sS.S += totS; sS.nt += rd.round_valid;
                 sD.e += totD; sD.S += totD; sD.nt += rd.round_valid;
@@ -472,7 +475,7 @@ k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __r
         XResult xr = {0, 0, 0, 0, 0};
         if (m) {
             const bool target_clean = cand == 1 ? sD.clean : sS.clean;
-            if (pacing && m_clean && target_clean) {
+            if (m_clean && target_clean) {
                 // nothing clamps but the hand-off itself: tokens up to m and after m+1 are delivered tau apart
                 xr.stall = (uint32_t)tau_eff + (uint32_t)max(-v_m1, 0);
                 xr.nt = nI - 1;
@@ -480,16 +483,17 @@ k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __r
                 xr.mx = xr.stall;
                 xr.delayed = v_m1 < 0 ? dl_clean : 0u;
             } else {
-                if (!(pacing && m_clean)) M = handoff_latency(G, key, l, m);
+                if (!m_clean) M = handoff_latency(G, key, l, m);
                 play_x(G, rd, key, nI, m, M, win2, W2, &xres_s[wib]);
                 __syncwarp();
                 xr = xres_s[wib];
                 __syncwarp();
             }
         }
+        windows_out(tS, tD, xr.nt, m != 0);
         if (lane == r) {
-            o_sumS = r_sumS; o_maxS = r_maxS; o_sumD = r_sumD; o_maxD = r_maxD; o_ntS = tS; o_ntD = tD;
-            o_sumX = xr.sum; o_maxX = xr.mx; o_stall = xr.stall; o_m = m; o_dl = xr.delayed; o_ntX = xr.nt;
+            o_sumS = r_sumS; o_maxS = r_maxS; o_sumD = r_sumD; o_maxD = r_maxD;
+            o_sumX = xr.sum; o_maxX = xr.mx; o_stall = xr.stall; o_m = m; o_dl = xr.delayed;
         }
     }
     __syncwarp();
@@ -498,11 +502,7 @@ k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __r
         rec.sum[0][kk] = o_sumS; rec.max[0][kk] = o_maxS;
         rec.sum[1][kk] = o_sumD; rec.max[1][kk] = o_maxD;
         rec.sum[2][kk] = o_sumX; rec.max[2][kk] = o_maxX;
-        rec.stall[kk] = o_stall; rec.m[kk] = (uint16_t)o_m; rec.delayed[kk] = (uint16_t)o_dl;
-        const int kt0 = cc.ktau[g_l][0], kt1 = cc.ktau[g_l][1], kt2 = cc.ktau[g_l][2];
-        if (kt0 >= 0 && o_ntS) rec.win[0][(size_t)kk * W0 + kt0] += o_ntS;
-        if (kt1 >= 0 && o_ntD) rec.win[1][(size_t)kk * W1 + kt1] += o_ntD;
-        if (kt2 >= 0 && o_ntX) rec.win[2][(size_t)kk * W2 + kt2] += o_ntX;
+        rec.hand[kk] = make_uint2(o_m | o_dl << 16, o_stall);
     }
     __syncwarp();
     }   // next batch
@@ -512,31 +512,32 @@ k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __r
 
 DBG_TRANSLATION_UNIT()
 
-cudaError_t launch_playout_fast(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const int32_t* knots,
-                                uint32_t k0, TimelineRec rec, uint32_t* todo, uint32_t* todo_count, bool never_clamps,
-                                uint32_t search, bool long_outputs, int sms, cudaStream_t st);
+cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const int32_t* knots,
+                                 uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, int sms,
+                                 cudaStream_t st);
+cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const ClassConst& host_cc,
+                                const int32_t* knots, uint32_t k0, TimelineRec rec, int32_t* err, uint32_t batches, int sms,
+                                cudaStream_t st);
 
-// pacing: with the delivery buffer on, the clamp-free kernel plays every request it can and lists the rest
-// in todo[0 .. *todo_count) (todo_count must be zero on entry); the general kernel then plays the list.
-cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, bool pacing,
-                            const int32_t* knots, uint32_t k0, TimelineRec rec, int32_t* err, uint32_t* todo,
-                            uint32_t* todo_count, bool never_clamps, uint32_t search, bool long_outputs, cudaEvent_t mid, int sms,
-                            cudaStream_t st) {
-    if (tr.n == 0) return cudaSuccess;
-    const uint32_t per_block = kWarps * 32;
-    if (!pacing) {
-        if (mid) { cudaError_t e0 = cudaEventRecord(mid, st); if (e0) return e0; }
-        const uint32_t blocks = std::min<uint32_t>((tr.n + per_block - 1) / per_block, (uint32_t)sms * 16u);
-        return launch_after(k_playout, blocks, kWarps * 32, 0, st, tr, gc, cc, knots, k0, rec, err, nullptr,
-                            nullptr, tr.n);
-    }
-    cudaError_t e = launch_playout_fast(tr, gc, cc, knots, k0, rec, todo, todo_count, never_clamps, search, long_outputs, sms, st);
-    if (e) return e;
+uint32_t timeline_launches(uint32_t kinds) { return (kinds & 1u) + ((kinds >> 1) & 1u) + ((kinds >> 2) & 1u); }
+
+cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const ClassConst& host_cc,
+                            const int32_t* knots, uint32_t k0, TimelineRec rec, int32_t* err, uint32_t* ticket,
+                            uint32_t kinds, const uint32_t* batches, uint32_t search, bool long_outputs, cudaEvent_t mid,
+                            int sms, cudaStream_t st) {
+    cudaError_t e;
+    if (kinds & (1u << G_EXACT))
+        if ((e = launch_playout_exact(tr, gc, cc, knots, k0, rec, ticket, search, long_outputs, sms, st))) return e;
     if (mid && (e = cudaEventRecord(mid, st))) return e;
-    if (never_clamps) return cudaSuccess;             // no interval can exceed tau: the list stays empty
-    const uint32_t blocks = std::min<uint32_t>((tr.n + per_block - 1) / per_block, (uint32_t)sms * 2u);
-    return launch_after(k_playout, blocks, kWarps * 32, 0, st, tr, gc, cc, knots, k0, rec, err, todo, todo_count,
-                        0u);
+    if (kinds & (1u << G_FREE))
+        if ((e = launch_playout_free(tr, gc, cc, host_cc, knots, k0, rec, err, batches[G_FREE], sms, st))) return e;
+    if (kinds & (1u << G_GENERAL)) {
+        const size_t smem = (size_t)kWarps * (host_cc.W[0] + host_cc.W[1] + host_cc.W[2]) * 4;
+        if ((e = cudaFuncSetAttribute(k_playout, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024))) return e;
+        const uint32_t blocks = std::min<uint32_t>((batches[G_GENERAL] + kWarps - 1) / kWarps, (uint32_t)sms * 32u);
+        return launch_after(k_playout, blocks, kWarps * 32, smem, st, tr, gc, cc, knots, k0, rec, err);
+    }
+    return cudaSuccess;
 }
 
 }  // namespace disco

@@ -1,6 +1,4 @@
-// What the two reduction kernels over (request, policy) pairs share: the six outcomes of a pair, the 16-bit
-// block-private histogram counters, and how the zone-by-zone kernel (zones.cu) tells the pair-by-pair kernel
-// (pairs.cu) what it left over.
+// The six outcomes of a (request, policy) pair and the 16-bit block-private histogram counters of the pair kernel.
 #pragma once
 
 #include "disco_internal.cuh"
@@ -19,11 +17,6 @@ __device__ __forceinline__ uint32_t hist16_code(int bin) { return ((uint32_t)(bi
 __device__ __forceinline__ void hist16_apply(uint32_t* row, uint32_t code) {
     atomicAdd((uint32_t*)((char*)row + (code & 0xFFCu)), code & 0x10001u);
 }
-// The same increment taken away again (the word is read as two signed sixteen-bit counts, see zones.cu).
-__device__ __forceinline__ void hist16_retract(uint32_t* row, uint32_t code) {
-    atomicAdd((uint32_t*)((char*)row + (code & 0xFFCu)), 0u - (code & 0x10001u));
-}
-
 // One more TTFT of t ticks, t < 2^31 (so its bin is below kNBins): the counter pair and the half come straight
 // from the float's exponent and leading mantissa bits, 32 bins per octave as in bin_of_ticks.
 __device__ __forceinline__ void hist16_add_ticks(uint32_t* row, uint32_t t) {
@@ -31,18 +24,5 @@ __device__ __forceinline__ void hist16_add_ticks(uint32_t* row, uint32_t t) {
     const uint32_t fb = __float_as_uint(__uint2float_rz(t));
     atomicAdd((uint32_t*)((char*)row - 4 * (((127 + 4) << 5) >> 1) + ((fb >> 17) & 0x3FFCu)), 1u << ((fb >> 14) & 16u));
 }
-
-// A word that holds two signed sixteen-bit counts, W = hi * 65536 + lo (mod 2^32), each within +-32767.
-__device__ __forceinline__ int32_t packed_lo(uint32_t w) { return (int32_t)(int16_t)(w & 0xFFFFu); }
-__device__ __forceinline__ int32_t packed_hi(uint32_t w) { return (int32_t)(w - (uint32_t)packed_lo(w)) >> 16; }
-
-// Requests a zone-by-zone kernel could not settle for a tile are flagged in a bit mask: word
-// request * words_per_request + tile / 32, bit tile % 32.
-__host__ __device__ __forceinline__ uint32_t left_words_per_request(uint32_t n_tiles) { return (n_tiles + 31u) / 32u; }
-// The first kLeftList of them per (chunk, tile) are also listed by chunk position, so that the pair kernel need not
-// scan the flags of a chunk for a handful of requests.
-constexpr uint32_t kLeftList = 2048;
-// The count of a (chunk, tile) whose policies the zone-by-zone kernel could not take at all.
-constexpr uint32_t kNotByZones = 0xFFFFFFFFu;
 
 }  // namespace disco
