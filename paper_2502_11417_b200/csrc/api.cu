@@ -594,7 +594,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
 
     // ---- the difference tables of the slabs, laid out batch by batch: a batch's slabs have like numbers of rows and share
     //      one class; its tables are cleared, filled, added up and then belong to the next batch
-    struct Batch { size_t first, count; int K, T; uint64_t ttft, tbt, sums; };
+    struct Batch { size_t first, count; int T; uint64_t ttft, tbt, sums; };
     std::vector<std::vector<Batch>> batches(classes.size());
     uint64_t grid_bytes = 0;
     auto wide_class = [&](size_t k) { return (plan[k].kinds & ~(1u << G_EXACT)) != 0; };
@@ -607,12 +607,12 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             auto rows = [](int T) { return T == 1 ? 1 : T <= 4 ? 4 : 8; };
             std::vector<Batch>& bs = batches[k];
             if (bs.empty() || bytes(bs.back()) > (256ull << 20) || rows(bs.back().T) != rows(sl.T) || sl.mixed || slabs[x - 1].mixed)
-                bs.push_back(Batch{x, 0, 1, 1, 0, 0, 0});
+                bs.push_back(Batch{x, 0, 1, 0, 0, 0});
             Batch& b = bs.back();
             sl.ttft = b.ttft; sl.tbt = b.tbt; sl.sums = b.sums;
             b.ttft += grid_ttft_words(sl.K); b.tbt += grid_tbt_words(sl.K, sl.T); b.sums += grid_sum_words(sl.K, sl.T, G);
             ++b.count;
-            b.K = std::max(b.K, sl.K); b.T = std::max(b.T, sl.T);
+            b.T = std::max(b.T, sl.T);
             grid_bytes = std::max(grid_bytes, bytes(b) + 64);
         }
         n_tickets += (uint32_t)batches[k].size();
@@ -743,7 +743,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             }
             CU(launch_grid(tr, gc, dcc, prep, P, dsl, (uint32_t)b.count, b.T, wide, classes[k].pacing != 0, d_tab,
                            c->d_chunks.as<Chunk>(), (uint32_t)chunks.size(), rec, gt, left, tickets + ticket++, work, c->sms, st));
-            CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.K, b.T, wide, host_bin_of_ticks(classes[k].tau), d_tab, gt, acc,
+            CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, wide, host_bin_of_ticks(classes[k].tau), d_tab, gt, acc,
                              h_ttft, h_tbt, st));
             g_launches += 2;
             if (mixed) {

@@ -156,13 +156,13 @@ inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block,
 }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// The batch-th batch of 32 requests among the groups of one kind: its group, first request and length.
-__device__ __forceinline__ bool batch_of_kind(const TraceDev& tr, const ClassConst& cc, int kind, uint32_t batch, int& g,
-                                              uint32_t& k_lo, uint32_t& count) {
+// The batch-th batch of `size` requests among the groups of one kind: its group, first request and length.
+__device__ __forceinline__ bool batch_of_kind(const TraceDev& tr, const ClassConst& cc, int kind, uint32_t size, uint32_t batch,
+                                              int& g, uint32_t& k_lo, uint32_t& count) {
     for (g = 0; g < tr.n_groups; ++g) {
         if (cc.kind[g] != kind) continue;
-        const uint32_t lo = tr.grp_off[g], len = tr.grp_off[g + 1] - lo, here = (len + 31u) / 32u;
-        if (batch < here) { k_lo = lo + batch * 32u; count = min(32u, len - batch * 32u); return true; }
+        const uint32_t lo = tr.grp_off[g], len = tr.grp_off[g + 1] - lo, here = (len + size - 1u) / size;
+        if (batch < here) { k_lo = lo + batch * size; count = min(size, len - batch * size); return true; }
         batch -= here;
     }
     return false;
@@ -256,7 +256,7 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
                         const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt,
                         LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t* ticket /* zero */,
                         uint64_t* work /* [4], added to */, int sms, cudaStream_t st);
-cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int K, int T,
+cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
                           bool wide, int bin_tau, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
                           uint64_t* hist_tbt, cudaStream_t st);
 // Pair by pair: `n_list` policies under the chunks' requests, or (list not null) under the listed ones.

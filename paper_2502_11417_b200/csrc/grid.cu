@@ -11,8 +11,9 @@
 // k, k1, k2 depend on the prompt length alone, and the requests of a group are stored by prompt length: a chunk of
 // requests splits into a few SEGMENTS of consecutive requests that share them.  A block sweeps a segment once per run
 // with a lane per request, sums up what the requests come to in registers and shared-memory histograms, and enters the
-// run's totals ONCE: into row k2 of a table of differences that is carried to the columns from k2 on, or into row k1 of
-// one that is carried to the columns below k1.  k_spread adds the rows up and writes every policy's sums and histograms.
+// run's totals ONCE into a table of differences along the columns (row q is carried to the columns from q on: a run of the
+// columns [a, b) is entered into row a and taken back in row b).  k_spread adds the rows up and writes every policy's
+// sums and histograms.
 // Under Algorithm 2 the first columns (budgets below the tail ratio) may wait longer than the others: for the few
 // requests that the common w_tail does not cover (at most a share alpha of them) the block keeps a list, and each of
 // those columns gets the list's totals under its own wait in place of the common one.
@@ -106,38 +107,49 @@ __device__ __forceinline__ void hist_add(uint32_t* h, int bin) {
     if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicAdd(&h[bin], 1u);
 }
 
-// Adds the rows of window counts of the lanes' requests to the TBT histograms (streams whose intervals are not all tau).
-// hist_all: the histogram that every row gets.  need_x: the stream after a hand-off, at level t (1 .. T).
-__device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_t* tbt, uint32_t* hist_all, bool need_base,
-                                            bool need_x, uint32_t kk, int stream, int t) {
-    const ClassConst& cc = *a.cc;
+// Adds (or, sub, takes) the rows of window counts of the lanes' requests that are in the mask: a lane sums up a bin over
+// the requests, with eight loads in flight, and adds once.
+__device__ __forceinline__ void add_rows(const uint16_t* __restrict__ win, int W, int lo, uint32_t mask, uint32_t kk, bool sub,
+                                         uint32_t* hist) {
+    if (mask == 0u) return;
     const int lane = threadIdx.x & 31;
-    uint32_t pend = __ballot_sync(FULL, need_base || need_x);
-    const uint32_t mine = (uint32_t)stream | (need_base ? 2u : 0u) | (need_x ? 4u : 0u) | ((uint32_t)t << 3);
-    while (pend) {
-        const int r = __ffs(pend) - 1;
-        pend &= pend - 1u;
-        const uint32_t code = __shfl_sync(FULL, mine, r), k = __shfl_sync(FULL, kk, r);
-        const int level = (int)(code >> 3);
-        if (code & 2u) {
-            const int s = (int)(code & 1u), W = cc.W[s], lo = cc.lo[c.g][s];
-            const uint16_t* row = a.rec.win[s] + (size_t)k * W;
-            for (int b = lane; b < W; b += 32) {
-                const uint32_t v = row[b];
-                if (v == 0u || !DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) continue;
-                if (level < c.T || !tbt) atomicAdd(&hist_all[lo + b], v);
-                if (level > 0 && level < c.T) atomicSub(&tbt[(level - 1) * kNBins + lo + b], v);
+    for (int b0 = 0; b0 < W; b0 += 32) {
+        const int b = b0 + lane;
+        const bool in = b < W && DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN);
+        uint32_t sum = 0;
+#pragma unroll 1
+        for (int r0 = 0; r0 < 32; r0 += 8) {
+            if (((mask >> r0) & 255u) == 0u) continue;
+            uint32_t v[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const uint32_t k = __shfl_sync(FULL, kk, r0 + r);
+                v[r] = (in && ((mask >> (r0 + r)) & 1u)) ? win[(size_t)k * W + b] : 0u;
             }
+#pragma unroll
+            for (int r = 0; r < 8; ++r) sum += v[r];
         }
-        if (code & 4u) {
-            const int W = cc.W[2], lo = cc.lo[c.g][2];
-            const uint16_t* row = a.rec.win[2] + (size_t)k * W;
-            for (int b = lane; b < W; b += 32) {
-                const uint32_t v = row[b];
-                if (v && DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicAdd(&tbt[(level - 1) * kNBins + lo + b], v);
-            }
-        }
+        if (sum) atomicAdd(&hist[lo + b], sub ? 0u - sum : sum);
     }
+}
+
+// The windows of the lanes' requests whose streams' intervals are not all tau: the base stream (device or server) goes to
+// every row of the grid but those that migrate, [0, t), which get the stream after the hand-off.
+__device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_t* tbt, bool valid, uint32_t kk, bool device, int t) {
+    const ClassConst& cc = *a.cc;
+    uint32_t* all = tbt + (c.T - 1) * kNBins;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        if ((c.even >> s) & 1u) continue;
+        const bool mine = valid && (int)device == s;
+        const int W = cc.W[s], lo = cc.lo[c.g][s];
+        add_rows(a.rec.win[s], W, lo, __ballot_sync(FULL, mine && t < c.T), kk, false, all);
+        for (int r = 1; r < c.T; ++r)
+            add_rows(a.rec.win[s], W, lo, __ballot_sync(FULL, mine && t == r), kk, true, tbt + (r - 1) * kNBins);
+    }
+    if (c.even & 4u) return;
+    for (int r = 1; r <= c.T; ++r)
+        add_rows(a.rec.win[2], cc.W[2], cc.lo[c.g][2], __ballot_sync(FULL, valid && t == r), kk, false, tbt + (r - 1) * kNBins);
 }
 
 // One sweep over the requests [pa, pb) of the chunk, or (list) of the block's list: what they come to when the device
@@ -170,7 +182,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                     if (lane == 0 && live && DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicAdd(&sm.only_ttft[bin], (uint32_t)__popc(live));
                 } else if (valid) hist_add(sm.only_ttft, bin);
                 if (valid) { o.cnt += 1u; o.n += n; o.l += l; o.tt += Td; o.tau += (!WIDE || (c.even & 2u)) ? n - 1u : 0u; }
-                if (WIDE && !(c.even & 2u)) add_windows(a, c, nullptr, tbt + NT * kNBins, valid, false, kk, 1, 0);
+                if (WIDE && !(c.even & 2u)) add_rows(a.rec.win[1], a.cc->W[1], a.cc->lo[c.g][1], live, kk, false, tbt + NT * kNBins);
             }
             if (!race) continue;
         }
@@ -205,7 +217,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                 if (WIDE) s.tx[r] += tx;
             }
         if (t > 0) hist_add(tbt + (t - 1) * kNBins, bin_of_ticks(hand.y));
-        if (WIDE) add_windows(a, c, tbt, tbt + (c.T - 1) * kNBins, valid && !pace, t > 0 && !(c.even & 4u), kk, dev_wins ? 1 : 0, t);
+        if (WIDE) add_windows(a, c, tbt, valid, kk, dev_wins, t);
     }
 }
 
@@ -247,45 +259,43 @@ __device__ __forceinline__ void share_only(Smem& sm, const Only& o) {
     }
 }
 
-// A slab's difference tables.  U row q is carried to the columns below q, V row q to the columns from q on (q = 0 .. K).
+// A slab's difference tables: row q is carried to the columns from q on.
 template <bool WIDE>
 struct Tables {
     using word = typename std::conditional<WIDE, unsigned long long, unsigned int>::type;   // windows hold more than 2^32 TBTs
-    uint32_t* ttft;                      // [2][K + 1][kNBins]
-    word* tbt;                           // [2][K + 1][T][kNBins]
-    unsigned long long* sums;            // [2][G][K + 1][fields]
+    uint32_t* ttft;                      // [K][kNBins]
+    word* tbt;                           // [T][K][kNBins]
+    unsigned long long* sums;            // [G][K][fields]
     int K, T, G;
     __device__ Tables(const GridTables& gt, const Slab& sl, int G_)
         : ttft(gt.ttft + sl.ttft), tbt((word*)gt.tbt + sl.tbt), sums(gt.sums + sl.sums), K(sl.K), T(sl.T), G(G_) {}
-    __device__ uint32_t* ttft_row(int v, int q) const { return ttft + (size_t)(v * (K + 1) + q) * kNBins; }
-    __device__ word* tbt_row(int v, int q, int r) const { return tbt + ((size_t)(v * (K + 1) + q) * T + r) * kNBins; }
-    __device__ unsigned long long* sum_row(int v, int g, int q) const { return sums + ((size_t)(v * G + g) * (K + 1) + q) * sum_fields(T); }
+    __device__ uint32_t* ttft_row(int q) const { return ttft + (size_t)q * kNBins; }
+    __device__ word* tbt_row(int q, int r) const { return tbt + ((size_t)r * K + q) * kNBins; }
+    __device__ unsigned long long* sum_row(int g, int q) const { return sums + ((size_t)g * K + q) * sum_fields(T); }
 };
 
-// Where a run's totals are entered: V row `row` (from), U row `row` (below, negated or not), or one column alone.
-enum Enter { E_FROM, E_BELOW, E_BELOW_NEG, E_ALONE };
-
-// Enters what the block has totalled for a run and clears it.  All threads call; barriers before and after.
+// Enters what the block has totalled for a run of the columns [q0, q1), or takes it from them (neg), and clears it.  All
+// threads call; barriers before and after.
 template <bool WIDE>
-__device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE>& tb, int g, Enter how, int row) {
+__device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE>& tb, int g, int q0, int q1, bool neg) {
     using word = typename Tables<WIDE>::word;
-    const int v = how == E_FROM ? 1 : 0, q = how == E_ALONE ? row + 1 : row;
-    const bool neg = how == E_BELOW_NEG, second = how == E_ALONE && row > 0;    // (row 0 is carried to nobody)
+    const bool back = q1 < tb.K;
     for (int b = threadIdx.x; b < kNBins; b += kThreads) {
         const uint32_t x = sm.ttft[b];
         if (x) {
             sm.ttft[b] = 0;
-            atomicAdd(&tb.ttft_row(v, q)[b], neg ? 0u - x : x);
-            if (second) atomicAdd(&tb.ttft_row(0, row)[b], 0u - x);
+            const uint32_t y = neg ? 0u - x : x;
+            atomicAdd(&tb.ttft_row(q0)[b], y);
+            if (back) atomicAdd(&tb.ttft_row(q1)[b], 0u - y);
         }
         int32_t level = 0;                                             // counts at a level go to every row below it
         for (int r = tb.T - 1; r >= 0; --r) {
             const int32_t y = (int32_t)tbt[r * kNBins + b];
             if (y) { tbt[r * kNBins + b] = 0; level += y; }
             if (level) {
-                const word z = (word)(long long)level;
-                atomicAdd(&tb.tbt_row(v, q, r)[b], neg ? (word)0 - z : z);
-                if (second) atomicAdd(&tb.tbt_row(0, row, r)[b], (word)0 - z);
+                const word z = (word)(long long)(neg ? -level : level);
+                atomicAdd(&tb.tbt_row(q0, r)[b], z);
+                if (back) atomicAdd(&tb.tbt_row(q1, r)[b], (word)0 - z);
             }
         }
     }
@@ -295,23 +305,32 @@ __device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE
         sm.sum[f] = 0;
         if (f == B_TT) { x = sm.tt; sm.tt = 0; }
         if (!x) continue;
-        atomicAdd(&tb.sum_row(v, g, q)[f], neg ? 0ull - x : x);
-        if (second) atomicAdd(&tb.sum_row(0, g, row)[f], 0ull - x);
+        if (neg) x = 0ull - x;
+        atomicAdd(&tb.sum_row(g, q0)[f], x);
+        if (back) atomicAdd(&tb.sum_row(g, q1)[f], 0ull - x);
     }
 }
 
-// The same for a device-only run, columns below `row`.
+// The same for a device-only run of the columns below q1.
 template <bool WIDE>
-__device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const Tables<WIDE>& tb, int g, int row) {
+__device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const Tables<WIDE>& tb, int g, int q1) {
     using word = typename Tables<WIDE>::word;
+    const bool back = q1 < tb.K;
     for (int b = threadIdx.x; b < kNBins; b += kThreads) {
         const uint32_t x = sm.only_ttft[b];
-        if (x) { sm.only_ttft[b] = 0; atomicAdd(&tb.ttft_row(0, row)[b], x); }
+        if (x) {
+            sm.only_ttft[b] = 0;
+            atomicAdd(&tb.ttft_row(0)[b], x);
+            if (back) atomicAdd(&tb.ttft_row(q1)[b], 0u - x);
+        }
         if (WIDE) {
-            const uint32_t y = only_tbt[b];
+            const word y = only_tbt[b];
             if (y) {
                 only_tbt[b] = 0;
-                for (int r = 0; r < tb.T; ++r) atomicAdd(&tb.tbt_row(0, row, r)[b], (word)y);
+                for (int r = 0; r < tb.T; ++r) {
+                    atomicAdd(&tb.tbt_row(0, r)[b], y);
+                    if (back) atomicAdd(&tb.tbt_row(q1, r)[b], (word)0 - y);
+                }
             }
         }
     }
@@ -320,7 +339,10 @@ __device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const T
         const unsigned long long x = k < 4 ? (unsigned long long)sm.only_sum[k] : sm.only_tt;
         if (k < 4) sm.only_sum[k] = 0; else sm.only_tt = 0;
         const int f = k == 0 ? B_DO : k == 1 ? B_TD : k == 2 ? B_PD : k == 3 ? B_TAU : B_TT;
-        if (x) atomicAdd(&tb.sum_row(0, g, row)[f], x);
+        if (x) {
+            atomicAdd(&tb.sum_row(g, 0)[f], x);
+            if (back) atomicAdd(&tb.sum_row(g, q1)[f], 0ull - x);
+        }
     }
 }
 
@@ -438,13 +460,13 @@ k_grid(const __grid_constant__ Args a) {
         uint32_t passes = 0;
 
         // one run: sweep and enter; `list` and `push` as in sweep
-        auto run = [&](uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, Enter how, int row) {
+        auto run = [&](uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, int q0, int q1, bool neg) {
             Acc<NT> s = {};
             Only none = {};
             sweep<NT, WIDE, false>(a, c, th, sm, tbt, pa, pb, w, list, push, true, false, s, none);
             share_out<NT, WIDE>(sm, s, c.T);
             __syncthreads();
-            enter<WIDE>(sm, tbt, tb, g, how, row);
+            enter<WIDE>(sm, tbt, tb, g, q0, q1, neg);
             __syncthreads();
             ++passes;
         };
@@ -458,7 +480,7 @@ k_grid(const __grid_constant__ Args a) {
                 if (race) share_out<NT, WIDE>(sm, s, c.T);
                 if (only) share_only(sm, o);
                 __syncthreads();
-                if (race) enter<WIDE>(sm, tbt, tb, g, E_FROM, sg.k2);
+                if (race) enter<WIDE>(sm, tbt, tb, g, sg.k2, K, false);
                 if (only) enter_only<WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1);
                 __syncthreads();
                 ++passes;
@@ -469,33 +491,32 @@ k_grid(const __grid_constant__ Args a) {
             uint32_t pa = 0;                                          // (of the segment in work: where the sweep goes on)
             int si = 0, ri = 0;
             for (;;) {
-                uint32_t from, to, w;
-                bool list = false, push = false, last = false;
-                Enter how;
-                int row;
-                if (si < n_seg) {
+                uint32_t from = 0, to = 0, w = 0;
+                int q0 = 0, q1 = 0;
+                bool push = false;
+                const bool done = si >= n_seg;
+                if (!done) {
                     const Seg sg = sm.seg[si];
                     const int n_pts = (int)sg.k2 - (int)sg.k1;
-                    if (ri == 0) { pa = sg.pa; }
+                    if (ri == 0) pa = sg.pa;
                     if (ri == 0 && (int)sg.k2 >= K) { ++ri; continue; }
                     if (ri > n_pts && sg.k1 == 0) { ri = 0; ++si; continue; }
                     from = pa; to = sg.pb;
-                    if (ri == 0) { w = 0u; how = E_FROM; row = sg.k2; ++ri; }
-                    else if (ri <= n_pts) { row = (int)sg.k1 + ri - 1; w = sm.w_star[row]; how = E_ALONE; ++ri; }
+                    if (ri == 0) { q0 = sg.k2; q1 = K; ++ri; }
+                    else if (ri <= n_pts) { q0 = (int)sg.k1 + ri - 1; q1 = q0 + 1; w = sm.w_star[q0]; ++ri; }
                     else {
-                        w = wt_min; how = E_BELOW; row = sg.k1; push = n_low > 0;
+                        w = wt_min; q1 = sg.k1; push = n_low > 0;
                         if (push && to - from > (uint32_t)kListStep) { to = from + kListStep; pa = to; }
                         else { ri = 0; ++si; }
                     }
-                } else if (sm.n_list > 0) { from = to = 0; w = 0; how = E_FROM; row = 0; last = true; }
-                else break;
-                if (!last) run(from, to, w, list, push, how, row);
-                if (last || (push && sm.n_list > (uint32_t)(kListCap - kListStep))) {
+                    run(from, to, w, false, push, q0, q1, false);
+                } else if (sm.n_list == 0) break;
+                if (done || (push && sm.n_list > (uint32_t)(kListCap - kListStep))) {
                     const uint32_t k = sm.n_list;                     // (barriers inside run: all threads agree)
                     __syncthreads();
                     if (threadIdx.x == 0) sm.n_list = 0;
-                    for (int p = -1; p < n_low; ++p)
-                        run(0u, k, p < 0 ? wt_min : sm.w_tail[p], true, false, p < 0 ? E_BELOW_NEG : E_ALONE, p < 0 ? n_low : p);
+                    for (int p = -1; p < n_low; ++p)                  // the common wait's totals go, each column's own come
+                        run(0u, k, p < 0 ? wt_min : sm.w_tail[p], true, false, max(p, 0), p < 0 ? n_low : p + 1, p < 0);
                 }
             }
         }
@@ -508,95 +529,105 @@ k_grid(const __grid_constant__ Args a) {
     }
 }
 
-// Adds up the difference rows: what a policy gets is the sum of U's rows above its column and V's rows up to it.  A
-// thread takes one histogram bin (or one sum) of one row of the grid and 32 columns: it adds the rows up for the first
-// column and goes on to the next by two.  Bound: L2 (the tables are read once per 32 columns, every policy's histograms
-// are written once).
-constexpr int kSpreadThreads = 128;
-constexpr int kSpreadCols = 32;
+// Adds up the difference rows: what a policy gets is the sum of the rows up to its column.  A block takes 32 histogram
+// bins (or sums) of one row of the grid, a lane each, and all columns, a few consecutive ones a warp: the warps add up
+// their own rows, the totals meet in shared memory, and every warp writes its columns' policies.  Bound: L2 and the
+// stores (the tables are read once, every policy's histograms written once).  (One thread a bin, walking the columns:
+// 202 us at 256 x 4 policies.)
+constexpr int kSpreadWarps = 32;
+constexpr int kSpreadPer = kGridCols / kSpreadWarps;                   // columns a warp may have
+static_assert(kNBins % 32 == 0, "a block's bins");
 
-template <class T, class F>
-__device__ __forceinline__ T first_column(int c0, int K, F at) {       // at(v, q)
-    T v = 0;
-#pragma unroll 8
-    for (int q = c0 + 1; q <= K; ++q) v += at(0, q);
-#pragma unroll 8
-    for (int q = 0; q <= c0; ++q) v += at(1, q);
-    return v;
+template <class W, class F, class E>
+__device__ __forceinline__ void spread_columns(unsigned long long* s_part, int K, F at /* (q) */, E emit /* (column, value) */) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int per = (K + kSpreadWarps - 1) / kSpreadWarps, q0 = min(K, w * per), q1 = min(K, q0 + per);
+    W x[kSpreadPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kSpreadPer; ++k) x[k] = q0 + k < q1 ? (W)at(q0 + k) : (W)0;
+#pragma unroll
+    for (int k = 0; k < kSpreadPer; ++k) { sum += x[k]; x[k] = sum; }
+    s_part[w * 33 + lane] = sum;
+    __syncthreads();
+    // the warps' totals in front of each: a warp scans one bin's 32 totals
+    {
+        unsigned long long v = s_part[lane * 33 + w];
+        const unsigned long long own = v;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned long long up = __shfl_up_sync(FULL, v, off);
+            if (lane >= off) v += up;
+        }
+        s_part[lane * 33 + w] = v - own;
+    }
+    __syncthreads();
+    const W before = (W)s_part[w * 33 + lane];
+#pragma unroll
+    for (int k = 0; k < kSpreadPer; ++k) if (q0 + k < q1) emit(q0 + k, (W)(before + x[k]));
 }
 
 template <bool WIDE>
-__global__ void __launch_bounds__(kSpreadThreads)
+__global__ void __launch_bounds__(kSpreadWarps * 32)
 k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict__ slabs, int bin_tau,
          const uint32_t* __restrict__ tab, GridTables gt, unsigned long long* __restrict__ acc,
          unsigned long long* __restrict__ hist_ttft, unsigned long long* __restrict__ hist_tbt) {
+    __shared__ unsigned long long s_part[kSpreadWarps * 33];
     grid_dependency_wait();
-    const Slab& sl = slabs[blockIdx.z];
-    const int K = sl.K, T = sl.T, c0 = blockIdx.y * kSpreadCols, c1 = min(K, c0 + kSpreadCols);
-    if (c0 >= K) return;
+    const Slab& sl = slabs[blockIdx.y];
+    const int K = sl.K, T = sl.T, lane = threadIdx.x & 31;
     const Tables<WIDE> tb(gt, sl, tr.n_groups);
     using word = typename Tables<WIDE>::word;
     const uint32_t* cells = tab + sl.cells;
-    int k = blockIdx.x * kSpreadThreads + threadIdx.x;
-    if (k < kNBins) {                                                  // TTFT: the same for every row
-        auto at = [&](int v, int q) { return tb.ttft_row(v, q)[k]; };
-        uint32_t x = first_column<uint32_t>(c0, K, at);
-        for (int c = c0; c < c1; ++c) {
-            for (int r = 0; r < T; ++r) {
-                const uint32_t p = cells[c * T + r];
-                if (p != kNoPolicy) hist_ttft[(size_t)p * kNBins + k] = x;
-            }
-            if (c + 1 < c1) x += at(1, c + 1) - at(0, c + 1);
-        }
+    constexpr int kParts = kNBins / 32;
+    int part = blockIdx.x;
+    if (part < T * kParts) {                                           // TTFT: the same for every row
+        const int r = part / kParts, b = (part - r * kParts) * 32 + lane;
+        spread_columns<uint32_t>(s_part, K, [&](int q) { return tb.ttft_row(q)[b]; }, [&](int c, uint32_t x) {
+            const uint32_t p = cells[c * T + r];
+            if (p != kNoPolicy) hist_ttft[(size_t)p * kNBins + b] = x;
+        });
         return;
     }
-    k -= kNBins;
-    if (k < T * kNBins) {                                              // TBT
-        const int r = k / kNBins, b = k - r * kNBins;
-        auto at = [&](int v, int q) { return tb.tbt_row(v, q, r)[b]; };
-        word x = first_column<word>(c0, K, at);
-        for (int c = c0; c < c1; ++c) {
+    part -= T * kParts;
+    if (part < T * kParts) {                                           // TBT
+        const int r = part / kParts, b = (part - r * kParts) * 32 + lane;
+        spread_columns<word>(s_part, K, [&](int q) { return tb.tbt_row(q, r)[b]; }, [&](int c, word x) {
             const uint32_t p = cells[c * T + r];
-            if (p != kNoPolicy) {
-                unsigned long long* h = &hist_tbt[(size_t)p * kNBins + b];
-                if (b == bin_tau) atomicAdd(h, (unsigned long long)x); else *h = x;      // (the regular TBTs join tau's bin below)
-            }
-            if (c + 1 < c1) x += at(1, c + 1) - at(0, c + 1);
-        }
+            if (p == kNoPolicy) return;
+            unsigned long long* h = &hist_tbt[(size_t)p * kNBins + b];
+            if (b == bin_tau) atomicAdd(h, (unsigned long long)x); else *h = x;      // (the regular TBTs join tau's bin below)
+        });
         return;
     }
-    k -= T * kNBins;
-    if (k < tr.n_groups * T * kNAcc) {                                 // sums
-        const int s = k % kNAcc, r = (k / kNAcc) % T, g = k / (kNAcc * T);
-        const int cand = gcs[g].candidate;
-        const int fb = s == A_DEVICE_ONLY ? B_DO : s == A_RACE ? B_RACE : s == A_DEVICE_WON ? B_DW : s == A_TOK_DEVICE ? B_TD
-                     : s == A_PRE_SERVER ? B_PS : s == A_PRE_DEVICE ? B_PD : s == A_TTFT_SUM ? B_TT : s == A_TAU_CNT ? B_TAU : -1;
-        int fl = -1;
-        bool minus = false;
-        if (s == A_TOK_DEVICE) { fl = V_A; minus = cand == 2; }        // the server's tokens go to the device, or the device's to the server
-        else if (s == A_PRE_SERVER && cand == 2) fl = V_B;
-        else if (s == A_PRE_DEVICE && cand == 1) fl = V_B;
-        else if (s == A_DELAYED) fl = V_C;
-        else if (s == A_MIGR) fl = V_N;
-        else if (s == A_TAU_CNT) { fl = WIDE ? V_TAU : V_N; minus = !WIDE; }
-        const int f2 = fl < 0 ? -1 : kBase + r * kLev + fl;
-        auto at = [&](int v, int q) {
-            const unsigned long long* row = tb.sum_row(v, g, q);
-            unsigned long long y = fb >= 0 ? row[fb] : 0ull;
-            if (f2 >= 0) y += minus ? 0ull - row[f2] : row[f2];
-            return y;
-        };
-        unsigned long long x = (fb < 0 && f2 < 0) ? 0ull : first_column<unsigned long long>(c0, K, at);
-        for (int c = c0; c < c1; ++c) {
-            const uint32_t p = cells[c * T + r];
-            if (p != kNoPolicy) {
-                unsigned long long* to = acc + ((size_t)p * tr.n_groups + g) * kNAcc + s;
-                if (s == A_TAU_CNT) { *to = 0; if (x) atomicAdd(&hist_tbt[(size_t)p * kNBins + bin_tau], x); }
-                else *to = x;
-            }
-            if (c + 1 < c1) x += at(1, c + 1) - at(0, c + 1);
-        }
-    }
+    part -= T * kParts;
+    const int k = part * 32 + lane;                                    // sums
+    if (part * 32 >= tr.n_groups * T * kNAcc) return;
+    const bool mine = k < tr.n_groups * T * kNAcc;
+    const int s = mine ? k % kNAcc : 0, r = mine ? (k / kNAcc) % T : 0, g = mine ? k / (kNAcc * T) : 0;
+    const int cand = gcs[g].candidate;
+    const int fb = s == A_DEVICE_ONLY ? B_DO : s == A_RACE ? B_RACE : s == A_DEVICE_WON ? B_DW : s == A_TOK_DEVICE ? B_TD
+                 : s == A_PRE_SERVER ? B_PS : s == A_PRE_DEVICE ? B_PD : s == A_TTFT_SUM ? B_TT : s == A_TAU_CNT ? B_TAU : -1;
+    int fl = -1;
+    bool minus = false;
+    if (s == A_TOK_DEVICE) { fl = V_A; minus = cand == 2; }            // the server's tokens go to the device, or the device's to the server
+    else if (s == A_PRE_SERVER && cand == 2) fl = V_B;
+    else if (s == A_PRE_DEVICE && cand == 1) fl = V_B;
+    else if (s == A_DELAYED) fl = V_C;
+    else if (s == A_MIGR) fl = V_N;
+    else if (s == A_TAU_CNT) { fl = WIDE ? V_TAU : V_N; minus = !WIDE; }
+    const int f2 = fl < 0 ? -1 : kBase + r * kLev + fl;
+    spread_columns<unsigned long long>(s_part, K, [&](int q) {
+        const unsigned long long* row = tb.sum_row(g, q);
+        unsigned long long y = fb >= 0 ? row[fb] : 0ull;
+        if (f2 >= 0) y += minus ? 0ull - row[f2] : row[f2];
+        return y;
+    }, [&](int c, unsigned long long x) {
+        const uint32_t p = mine ? cells[c * T + r] : kNoPolicy;
+        if (p == kNoPolicy) return;
+        unsigned long long* to = acc + ((size_t)p * tr.n_groups + g) * kNAcc + s;
+        if (s == A_TAU_CNT) { *to = 0; if (x) atomicAdd(&hist_tbt[(size_t)p * kNBins + bin_tau], x); }
+        else *to = x;
+    });
 }
 
 size_t grid_smem(int NT, bool wide) { return sizeof(Smem) + (size_t)(NT + (wide ? 1 : 0)) * kNBins * 4; }
@@ -615,9 +646,9 @@ cudaError_t launch_one(const Args& a, int sms, cudaStream_t st) {
 
 DBG_TRANSLATION_UNIT()
 
-uint64_t grid_ttft_words(int K) { return 2ull * (K + 1) * kNBins; }
-uint64_t grid_tbt_words(int K, int T) { return 2ull * (K + 1) * T * kNBins; }
-uint64_t grid_sum_words(int K, int T, int G) { return 2ull * G * (K + 1) * sum_fields(T); }
+uint64_t grid_ttft_words(int K) { return (uint64_t)K * kNBins; }
+uint64_t grid_tbt_words(int K, int T) { return (uint64_t)K * T * kNBins; }
+uint64_t grid_sum_words(int K, int T, int G) { return (uint64_t)G * K * sum_fields(T); }
 uint32_t grid_blocks_per_sm(int T) { return T == 1 ? 4 : 2; }
 
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
@@ -632,14 +663,13 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
     return T == 1 ? launch_one<1, false>(a, sms, st) : T <= 4 ? launch_one<4, false>(a, sms, st) : launch_one<8, false>(a, sms, st);
 }
 
-cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int K, int T,
+cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
                           bool wide, int bin_tau, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
                           uint64_t* hist_tbt, cudaStream_t st) {
     if (n_slabs == 0) return cudaSuccess;
-    const uint32_t per = (uint32_t)(kNBins * (1 + T) + tr.n_groups * T * kNAcc);
-    const dim3 grid((per + kSpreadThreads - 1) / kSpreadThreads, (K + kSpreadCols - 1) / kSpreadCols, n_slabs);
+    const dim3 grid((uint32_t)(2 * T * (kNBins / 32) + (tr.n_groups * T * kNAcc + 31) / 32), n_slabs);
     auto* kernel = wide ? k_spread<true> : k_spread<false>;
-    return launch_after(kernel, grid, kSpreadThreads, 0, st, tr, gc, slabs, bin_tau, tab, gt, (unsigned long long*)acc,
+    return launch_after(kernel, grid, kSpreadWarps * 32, 0, st, tr, gc, slabs, bin_tau, tab, gt, (unsigned long long*)acc,
                         (unsigned long long*)hist_ttft, (unsigned long long*)hist_tbt);
 }
 

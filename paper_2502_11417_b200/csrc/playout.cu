@@ -306,7 +306,7 @@ k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __r
     for (uint32_t batch = blockIdx.x * kWarps + wib;; batch += gridDim.x * kWarps) {
     int g;
     uint32_t k_lo, n_here;
-    if (!batch_of_kind(tr, cc, G_GENERAL, batch, g, k_lo, n_here)) break;
+    if (!batch_of_kind(tr, cc, G_GENERAL, 32u, batch, g, k_lo, n_here)) break;
 
     // ---- one request per lane: inputs
     const bool live = lane < (int)n_here;
@@ -516,7 +516,7 @@ cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const
                                  uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, int sms,
                                  cudaStream_t st);
 cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const ClassConst& host_cc,
-                                const int32_t* knots, uint32_t k0, TimelineRec rec, int32_t* err, uint32_t batches, int sms,
+                                const int32_t* knots, uint32_t k0, TimelineRec rec, uint32_t batches, int sms,
                                 cudaStream_t st);
 
 uint32_t timeline_launches(uint32_t kinds) { return (kinds & 1u) + ((kinds >> 1) & 1u) + ((kinds >> 2) & 1u); }
@@ -530,7 +530,7 @@ cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const Clas
         if ((e = launch_playout_exact(tr, gc, cc, knots, k0, rec, ticket, search, long_outputs, sms, st))) return e;
     if (mid && (e = cudaEventRecord(mid, st))) return e;
     if (kinds & (1u << G_FREE))
-        if ((e = launch_playout_free(tr, gc, cc, host_cc, knots, k0, rec, err, batches[G_FREE], sms, st))) return e;
+        if ((e = launch_playout_free(tr, gc, cc, host_cc, knots, k0, rec, batches[G_FREE], sms, st))) return e;
     if (kinds & (1u << G_GENERAL)) {
         const size_t smem = (size_t)kWarps * (host_cc.W[0] + host_cc.W[1] + host_cc.W[2]) * 4;
         if ((e = cudaFuncSetAttribute(k_playout, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024))) return e;

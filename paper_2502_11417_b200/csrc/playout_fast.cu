@@ -227,11 +227,18 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
     }
 }
 
-// Buffers that fill within a few tokens (no group's search looks at more than kShortSearch of them): a thread plays a
-// request.  The lanes of a warp hold requests of one prompt length or nearly so, whose searches and, where the device
-// takes over, lags are alike; beyond some 64 tokens the longest of 32 requests would keep the others waiting.
+// Buffers that fill within a few tokens (no group's search looks at more than kShortSearch of them).  A thread plays a
+// request up to the hand-off: the lanes of a warp hold requests whose searches take about the same number of tokens;
+// beyond some 64 tokens the longest of 32 requests would keep the others waiting.  The lag after a hand-off is another
+// matter: a few requests in ten have one, and where the server takes over it is as widely spread as its TTFT.  Those
+// requests are therefore collected in shared memory first.  A thread each, in full warps, draws the first tokens of a lag;
+// what is left of the longer ones is made up by a warp each, 32 tokens at a time, so that the longest (thousands of
+// tokens) does not hold the block for as many dependent steps.  A thread draws 32 tokens, or 256 where most of the block's
+// requests have longer lags (prompts that take a device long to read: those lags are alike).  (Without the collection:
+// 513 us for the 16 M requests of three server profiles and two devices, 43 us for 250,000 of them; now 245 and 12.)
 constexpr uint32_t kShortSearch = 64;
 constexpr int kShortThreads = 256;
+constexpr int kShortPer = 4;             // requests a thread may play
 
 struct ShortGroup {                      // a group under the class
     uint32_t mulC, mulT;                 // candidate's and target's jitter ranges
@@ -240,17 +247,22 @@ struct ShortGroup {                      // a group under the class
     int cand;
     uint32_t end;                        // where the group's requests end
     int exact;                           // played here
+    int32_t cT_mean;
 };
 
 __global__ void __launch_bounds__(kShortThreads)
 k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
-                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec) {
+                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int per) {
     __shared__ ShortGroup groups[kMaxGroups];
+    __shared__ uint4 lag[kShortThreads * kShortPer];         // hash key, lag, output length | hand-off << 16, place | group << 16
+    __shared__ uint16_t rest[kShortThreads * kShortPer];     // lags that a thread has not made up
+    __shared__ int n_lag, n_long, n_rest;
     grid_dependency_wait();
     const int32_t tau = ccp->tau;
     const uint32_t B = (uint32_t)ccp->B;
     const long long thr64 = (long long)(B ? B - 1 : 0) * tau;
     const int32_t thr = thr64 > 0x7FFFFFFFLL ? 0x7FFFFFFF : (int32_t)thr64;
+    if (threadIdx.x == 0) { n_lag = 0; n_long = 0; n_rest = 0; }
     for (int g = threadIdx.x; g < tr.n_groups; g += kShortThreads) {
         const GroupConst& gc = gcs[g];
         ShortGroup G;
@@ -262,56 +274,95 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassCons
         G.kappa = (uint32_t)gc.kappa; G.c0 = (uint32_t)gc.c0;
         G.end = tr.grp_off[g + 1];
         G.exact = ccp->kind[g] == G_EXACT;
+        G.cT_mean = G.cT - (int32_t)(G.mulT >> 1);
         groups[g] = G;
     }
     __syncthreads();
-    const uint32_t kk = blockIdx.x * kShortThreads + threadIdx.x;
-    if (kk >= tr.n) return;
-    int g = 0;
-    while (g + 1 < tr.n_groups && kk >= groups[g].end) ++g;
-    const ShortGroup& G = groups[g];
-    if (!G.exact) return;
-    const uint4 q = tr.req[kk];
-    const uint32_t n = q.y >> 16, l = q.y & 0xFFFFu;
-    uint32_t m = 0, stall = 0, delayed = 0;
-    if (G.cand != 0 && n > 1) {
-        const uint32_t key = mix32(k0 + q.z * kHashReq);
-        int32_t e_m = 0;
-        if (B == 0) m = 1;                                             // nothing to fill: hand off after token 1
-        else {
-            uint32_t hin = key + kHashTok;
-            for (uint32_t j = 2; j < n; ++j) {                         // (the hand-off needs a token left to generate)
-                hin += kHashTok;
-                e_m += G.cC - (int32_t)__umulhi(mix32(hin), G.mulC);
-                if (e_m > thr) { m = j; break; }
-            }
-        }
-        if (m) {
-            uint32_t M;
-            if (G.cand == 1) M = G.kappa * (l + m) + G.c0;             // device re-prefills prompt + m tokens
+    const uint32_t first = blockIdx.x * (uint32_t)(kShortThreads * per);
+    for (int k = 0; k < per; ++k) {
+        const uint32_t kk = first + k * kShortThreads + threadIdx.x;
+        if (kk >= tr.n) break;
+        int g = 0;
+        while (g + 1 < tr.n_groups && kk >= groups[g].end) ++g;
+        const ShortGroup& G = groups[g];
+        if (!G.exact) continue;
+        const uint4 q = tr.req[kk];
+        const uint32_t n = q.y >> 16, l = q.y & 0xFFFFu;
+        uint32_t m = 0, stall = 0;
+        if (G.cand != 0 && n > 1) {
+            const uint32_t key = mix32(k0 + q.z * kHashReq);
+            int32_t e_m = 0;
+            if (B == 0) m = 1;                                         // nothing to fill: hand off after token 1
             else {
-                const uint32_t u = mix32(key);                         // a server TTFT drawn from F by its knots
-                const uint32_t ki = u >> 24, fr = (u >> 8) & 0xFFFFu;
-                const int32_t* K = knots + g * kNKnots;
-                M = 0;
-                if (DBG_OK(ki + 1, kNKnots, DBG_K_PLAYOUT_FAST, DBG_KNOT))
-                    M = (uint32_t)(K[ki] + (int32_t)(((int64_t)(K[ki + 1] - K[ki]) * (int64_t)fr) >> 16));
-            }
-            const int32_t need = -(e_m + (tau - (int32_t)M));          // how late token m+1 is
-            stall = (uint32_t)tau + (uint32_t)max(need, 0);
-            if (need > 0) {
-                // tokens m+2.. stay late while the target's sum of c from there on is below the lag (c >= 0: a prefix)
-                int32_t run = 0;
-                uint32_t j = m + 2;
-                for (uint32_t hin = key + j * kHashTok; j <= n; ++j, hin += kHashTok) {
-                    run += G.cT - (int32_t)__umulhi(mix32(hin), G.mulT);
-                    if (run >= need) break;
+                uint32_t hin = key + kHashTok;
+                for (uint32_t j = 2; j < n; ++j) {                     // (the hand-off needs a token left to generate)
+                    hin += kHashTok;
+                    e_m += G.cC - (int32_t)__umulhi(mix32(hin), G.mulC);
+                    if (e_m > thr) { m = j; break; }
                 }
-                delayed = j - m - 1;                                   // tokens m+1 .. j-1
+            }
+            if (m) {
+                uint32_t M;
+                if (G.cand == 1) M = G.kappa * (l + m) + G.c0;         // device re-prefills prompt + m tokens
+                else {
+                    const uint32_t u = mix32(key);                     // a server TTFT drawn from F by its knots
+                    const uint32_t ki = u >> 24, fr = (u >> 8) & 0xFFFFu;
+                    const int32_t* K = knots + g * kNKnots;
+                    M = 0;
+                    if (DBG_OK(ki + 1, kNKnots, DBG_K_PLAYOUT_FAST, DBG_KNOT))
+                        M = (uint32_t)(K[ki] + (int32_t)(((int64_t)(K[ki + 1] - K[ki]) * (int64_t)fr) >> 16));
+                }
+                const int32_t need = -(e_m + (tau - (int32_t)M));      // how late token m+1 is
+                stall = (uint32_t)tau + (uint32_t)max(need, 0);
+                if (need > 0) {
+                    if (n - m > 33u && (need >> 5) > G.cT_mean) atomicAdd(&n_long, 1);
+                    const int at = atomicAdd(&n_lag, 1);
+                    if (DBG_OK(at, kShortThreads * kShortPer, DBG_K_PLAYOUT_FAST, DBG_SLOT))
+                        lag[at] = make_uint4(key, (uint32_t)need, n | m << 16, (uint32_t)(k * kShortThreads) + threadIdx.x | (uint32_t)g << 16);
+                }
             }
         }
+        rec.hand[kk] = make_uint2(m, stall);
     }
-    rec.hand[kk] = make_uint2(m | delayed << 16, stall);
+    __syncthreads();
+    // ---- tokens m+2.. stay late while the target's sum of c from there on is below the lag (c >= 0: a prefix)
+    const uint32_t most = n_long > kShortThreads / 4 ? 256u : 32u;
+    for (int i = threadIdx.x; i < n_lag; i += kShortThreads) {
+        const uint4 x = lag[i];
+        const ShortGroup& G = groups[x.w >> 16];
+        const int32_t need = (int32_t)x.y, cT = G.cT;
+        const uint32_t n = x.z & 0xFFFFu, m = x.z >> 16, mulT = G.mulT, end = min(n, m + 1 + most);
+        int32_t run = 0;
+        uint32_t j = m + 2;
+        for (uint32_t hin = x.x + j * kHashTok; j <= end; ++j, hin += kHashTok) {
+            run += cT - (int32_t)__umulhi(mix32(hin), mulT);
+            if (run >= need) break;
+        }
+        if (run < need && j <= n) { lag[i].y = (uint32_t)(need - run); rest[atomicAdd(&n_rest, 1)] = (uint16_t)i; continue; }
+        rec.hand[first + (x.w & 0xFFFFu)].x = m | (j - m - 1) << 16;           // tokens m+1 .. j-1 are late
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < n_rest; i += kShortThreads / 32) {
+        const uint4 x = lag[rest[i]];
+        const ShortGroup& G = groups[x.w >> 16];
+        const int32_t need = (int32_t)x.y, cT = G.cT;
+        const uint32_t n = x.z & 0xFFFFu, m = x.z >> 16, mulT = G.mulT;
+        int32_t run = 0;
+        uint32_t jb = m + 2 + most;
+        for (; jb <= n; jb += 32) {
+            const uint32_t j = jb + lane;
+            const int32_t c = j <= n ? cT - (int32_t)__umulhi(mix32(x.x + j * kHashTok), mulT) : 0;
+            const int32_t all = __reduce_add_sync(FULL, c);
+            if (run + all >= need) {
+                const int32_t R = run + team_inclusive_sum(c, lane);
+                jb += __popc(__ballot_sync(FULL, R < need && j <= n));
+                break;
+            }
+            run += all;
+        }
+        if (lane == 0) rec.hand[first + (x.w & 0xFFFFu)].x = m | (min(jb, n + 1) - m - 1) << 16;
+    }
 }
 
 }  // namespace
@@ -321,8 +372,12 @@ DBG_TRANSLATION_UNIT()
 cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const int32_t* knots,
                                  uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, int sms,
                                  cudaStream_t st) {
-    if (search <= kShortSearch)
-        return launch_after(k_playout_short, (tr.n + kShortThreads - 1) / kShortThreads, kShortThreads, 0, st, tr, gc, cc, knots, k0, rec);
+    if (search <= kShortSearch) {
+        // four requests a thread (fuller warps of lags) once that leaves several blocks to every multiprocessor
+        const int per = tr.n >= (uint32_t)sms * 8u * kShortThreads * kShortPer ? kShortPer : 1;
+        const uint32_t per_block = (uint32_t)(kShortThreads * per);
+        return launch_after(k_playout_short, (tr.n + per_block - 1) / per_block, kShortThreads, 0, st, tr, gc, cc, knots, k0, rec, per);
+    }
     // requests per ticket: small batches spread the end of the launch evenly; large traces amortise the ticket
     int rpw = 8;
     while (rpw < 32 && (uint64_t)tr.n / (2 * rpw) >= (uint64_t)sms * 48u * 4u) rpw *= 2;

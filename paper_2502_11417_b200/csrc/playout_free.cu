@@ -4,9 +4,10 @@
 // histogram bins.
 //
 // Bound: integer issue (a hash, a range map and a bin per token and stream).  A warp plays a request, a lane every 32nd
-// token; the windows are counted in shared memory of the warp's own (increments of one, which the hardware merges
-// where lanes meet) and written once, as rows of 16-bit counts.  200,000 requests of 200 tokens, two streams:
-// see the figure at launch_playout_free.
+// token.  Every lane counts in counters of its own, [bin][lane] in shared memory: no atomics and no bank conflicts, where
+// 32 lanes would meet in the few bins of a stream; two requests share a counter's halves before the lanes' counts are
+// added up (step k of lane b reads counter (k + b) mod 32, again without conflicts) and written as rows of 16-bit counts.
+// 200,000 requests of 200 tokens, two streams: 204 us with one window a warp and atomics.
 #include <algorithm>
 
 #include "disco_internal.cuh"
@@ -17,46 +18,46 @@ namespace {
 
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr int kFreeWarps = 8;
+constexpr int kFreeBatch = 8;             // requests a warp takes at a time
 
-struct FreeStream {                      // one stream of a group
-    uint32_t mul;
-    int32_t base;                        // x = base + ((h * mul) >> 32), base = T - J
-    int lo, W;                           // its window of bins
-    bool on;                             // played here (else it keeps the pace)
-};
+// Where a stream's window of counters starts for this lane, and the bin in front of it.
+struct Counters { uint32_t* at; int lo, W; };
 
-// One interval more in a window that starts at bin lo.
-__device__ __forceinline__ void count_in(uint32_t* win, int lo, int W, uint32_t x, int32_t* err) {
-    const int b = bin_of_ticks(x) - lo;
-    if (b >= 0 && b < W) atomicAdd(&win[b], 1u); else atomicExch(&err[2], 1);
+// One interval of x ticks more.  SMALL: intervals below 32 ticks occur, which have bins of their own (bin_of_ticks).
+template <bool SMALL>
+__device__ __forceinline__ void count_in(const Counters& c, uint32_t x, uint32_t inc) {
+    const int b = (SMALL ? bin_of_ticks(x) : (int)(__float_as_uint(__uint2float_rz(x)) >> 18) - ((127 + 4) << 5)) - c.lo;
+    if (DBG_OK(b, c.W, DBG_K_PLAYOUT, DBG_WINDOW)) c.at[b * 32] += inc;
 }
 
-__global__ void __launch_bounds__(kFreeWarps * 32)
+// BOTH: pacing is off, both streams are played and a hand-off may follow the first token.  Otherwise pacing is on, a
+// stream or two clamp at every token and no buffer fills: each is played for itself.  (Kernels of their own: in one
+// kernel for all cases the warps waited for instructions four cycles of every ten.)
+template <bool BOTH, bool SMALL>
+__global__ void __launch_bounds__(kFreeWarps * 32, 4)
 k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
-               const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int32_t* __restrict__ err) {
-    extern __shared__ uint32_t s_win[];                       // [warps][W0 + W1]
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+               const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec) {
+    extern __shared__ uint32_t s_win[];                       // per warp: [W0 + W1][32] counters, [W0 + W1] their sums
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warps = blockDim.x >> 5;
     grid_dependency_wait();
     const ClassConst& cc = *ccp;
-    const int W0 = cc.W[0], W1 = cc.W[1], W2 = cc.W[2];
-    uint32_t* win0 = s_win + wib * (W0 + W1);
-    uint32_t* win1 = win0 + W0;
-    for (int b = lane; b < W0 + W1; b += 32) win0[b] = 0;
+    const int W0 = cc.W[0], W1 = cc.W[1], W2 = cc.W[2], WW = W0 + W1;
+    uint32_t* win = s_win + wib * (WW * 33);
+    uint32_t* red = win + WW * 32;
+    for (int b = lane; b < WW * 32; b += 32) win[b] = 0;
     __syncwarp();
-    const uint32_t tau = (uint32_t)cc.tau;
-    for (uint32_t batch = blockIdx.x * kFreeWarps + wib;; batch += gridDim.x * kFreeWarps) {
+    for (uint32_t batch = blockIdx.x * warps + wib;; batch += gridDim.x * warps) {
         int g;
         uint32_t k_lo, n_here;
-        if (!batch_of_kind(tr, cc, G_FREE, batch, g, k_lo, n_here)) break;
+        if (!batch_of_kind(tr, cc, G_FREE, kFreeBatch, batch, g, k_lo, n_here)) break;
         const GroupConst& gc = gcs[g];
-        FreeStream st[2];
-        st[0].mul = 2u * (uint32_t)gc.J_srv + 1u; st[0].base = gc.T_srv - gc.J_srv; st[0].lo = cc.lo[g][0]; st[0].W = W0;
-        st[1].mul = 2u * (uint32_t)gc.J_dev + 1u; st[1].base = gc.T_dev - gc.J_dev; st[1].lo = cc.lo[g][1]; st[1].W = W1;
-        st[0].on = !(cc.even[g] & 1u); st[1].on = !(cc.even[g] & 2u);
-        // without pacing the buffer is empty and the dearer winner hands over after its first token; with pacing such a
-        // stream never fills a buffer
-        const int cand = (cc.mig_any && !cc.pacing) ? gc.candidate : 0;
-        const int tgt = cand == 1 ? 1 : 0;
+        const uint32_t mul0 = 2u * (uint32_t)gc.J_srv + 1u, mul1 = 2u * (uint32_t)gc.J_dev + 1u;
+        const uint32_t base0 = (uint32_t)(gc.T_srv - gc.J_srv), base1 = (uint32_t)(gc.T_dev - gc.J_dev);   // x = base + ((h * mul) >> 32)
+        const Counters ct0 = {win + lane, cc.lo[g][0], W0}, ct1 = {win + W0 * 32 + lane, cc.lo[g][1], W1};
+        const bool on0 = BOTH || !(cc.even[g] & 1u), on1 = BOTH || !(cc.even[g] & 2u);
+        // without pacing the buffer is empty and the dearer winner hands over after its first token
+        const int cand = (BOTH && cc.mig_any) ? gc.candidate : 0;
+        const bool to_dev = cand == 1;
         // ---- one request per lane: inputs, results
         uint32_t n_l = 1, l_l = 1, key_l = 0;
         if (lane < n_here) {
@@ -64,67 +65,117 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
             n_l = q.y >> 16; l_l = q.y & 0xFFFFu;
             key_l = mix32(k0 + q.z * kHashReq);
         }
-        uint32_t o_sum[3] = {0, 0, 0}, o_max[3] = {0, 0, 0}, o_m = 0, o_stall = 0;
-        for (int r = 0; r < (int)n_here; ++r) {
-            const uint32_t n = __shfl_sync(FULL, n_l, r), key = __shfl_sync(FULL, key_l, r), k = k_lo + r;
-            uint32_t sum[2] = {0, 0}, most[2] = {0, 0}, first[2] = {0, 0}, most_later[2] = {0, 0};
-            for (uint32_t j = 2 + lane; j <= n; j += 32) {
-                const uint32_t h = mix32(key + j * kHashTok);
+        // sums and maxima of the jitter u = (h * (2J + 1)) >> 32, and of the target's from token 3 on
+        uint32_t o_s0 = 0, o_s1 = 0, o_m0 = 0, o_m1 = 0, o_later = 0;
+        for (int r0 = 0; r0 < (int)n_here; r0 += 2) {
+            const int pair = min(2, (int)n_here - r0);
+#pragma unroll 1
+            for (int half = 0; half < pair; ++half) {
+                const int r = r0 + half;
+                const uint32_t n = __shfl_sync(FULL, n_l, r), key = __shfl_sync(FULL, key_l, r), inc = half ? 65536u : 1u;
+                uint32_t s0 = 0, s1 = 0, m0 = 0, m1 = 0;
+                if (BOTH) {
+                    uint32_t later = 0;                       // the target's largest jitter from token 3 on
+                    uint32_t hin = key + (2u + lane) * kHashTok;
+#pragma unroll 2
+                    for (uint32_t j = 2u + lane; j <= n; j += 32u) {
+                        const uint32_t h = mix32(hin);
+                        hin += 32u * kHashTok;
+                        const uint32_t u = __umulhi(h, mul0), v = __umulhi(h, mul1);
+                        s0 += u; m0 = max(m0, u);
+                        count_in<SMALL>(ct0, base0 + u, inc);
+                        s1 += v; m1 = max(m1, v);
+                        count_in<SMALL>(ct1, base1 + v, inc);
+                        if (j != 2u) later = max(later, to_dev ? v : u);
+                    }
+                    later = __reduce_max_sync(FULL, later);
+                    if (lane == r) o_later = later;
+                } else {
+                    if (on0) {
+                        uint32_t hin = key + (2u + lane) * kHashTok;
+#pragma unroll 2
+                        for (uint32_t j = 2u + lane; j <= n; j += 32u) {
+                            const uint32_t u = __umulhi(mix32(hin), mul0);
+                            hin += 32u * kHashTok;
+                            s0 += u; m0 = max(m0, u);
+                            count_in<SMALL>(ct0, base0 + u, inc);
+                        }
+                    }
+                    if (on1) {
+                        uint32_t hin = key + (2u + lane) * kHashTok;
+#pragma unroll 2
+                        for (uint32_t j = 2u + lane; j <= n; j += 32u) {
+                            const uint32_t v = __umulhi(mix32(hin), mul1);
+                            hin += 32u * kHashTok;
+                            s1 += v; m1 = max(m1, v);
+                            count_in<SMALL>(ct1, base1 + v, inc);
+                        }
+                    }
+                }
+                s0 = __reduce_add_sync(FULL, s0); m0 = __reduce_max_sync(FULL, m0);
+                s1 = __reduce_add_sync(FULL, s1); m1 = __reduce_max_sync(FULL, m1);
+                if (lane == r) { o_s0 = s0; o_s1 = s1; o_m0 = m0; o_m1 = m1; }
+            }
+            __syncwarp();
+            // the lanes' counts are added up and go out; the counters are cleared for the next pair
+            const size_t k = k_lo + r0;
+#pragma unroll 1
+            for (int b = lane; b < WW; b += 32) {
+                uint32_t t = 0;
+                uint32_t* row = win + b * 32;
 #pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    if (!st[s].on) continue;                  // (uniform over the batch)
-                    const uint32_t x = (uint32_t)st[s].base + __umulhi(h, st[s].mul);
-                    sum[s] += x;
-                    if (j == 2) first[s] = x; else most_later[s] = max(most_later[s], x);
-                    count_in(s ? win1 : win0, st[s].lo, st[s].W, x, err);
+                for (int c = 0; c < 32; ++c) t += row[(c + b) & 31];
+                if (BOTH) red[b] = t;
+                const bool first = b < W0;
+                if (first ? on0 : on1) {
+                    uint16_t* to = first ? rec.win[0] + k * W0 + b : rec.win[1] + k * W1 + (b - W0);
+                    to[0] = (uint16_t)t;
+                    if (pair > 1) to[first ? W0 : W1] = (uint16_t)(t >> 16);
                 }
             }
             __syncwarp();
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                if (!st[s].on) { sum[s] = (n - 1) * tau; most[s] = n > 1 ? tau : 0u; continue; }
-                sum[s] = __reduce_add_sync(FULL, sum[s]);
-                most_later[s] = __reduce_max_sync(FULL, most_later[s]);
-                first[s] = __shfl_sync(FULL, first[s], 0);
-                most[s] = max(first[s], most_later[s]);
+#pragma unroll 4
+            for (int b = 0; b < WW; ++b) win[b * 32 + lane] = 0;
+            if (BOTH && cand) {
+                // stream X: one token of the candidate, then the target's from token 3 on
+                const int lo_t = to_dev ? ct1.lo : ct0.lo, Wt = to_dev ? W1 : W0, shift = cc.lo[g][2] - lo_t;
+                const uint32_t* wt = red + (to_dev ? W0 : 0);
+#pragma unroll 1
+                for (int half = 0; half < pair; ++half) {
+                    const uint32_t h2 = mix32(__shfl_sync(FULL, key_l, r0 + half) + 2u * kHashTok);
+                    const int skip = bin_of_ticks(to_dev ? base1 + __umulhi(h2, mul1) : base0 + __umulhi(h2, mul0)) - lo_t;
+                    for (int b = lane; b < W2; b += 32) {
+                        const int t = b + shift;
+                        uint32_t v = (t >= 0 && t < Wt) ? wt[t] >> (16 * half) : 0u;
+                        if (t == skip) --v;
+                        rec.win[2][(k + half) * W2 + b] = (uint16_t)v;
+                    }
+                }
+                __syncwarp();
             }
+        }
+        if (lane < n_here) {
+            const uint32_t k = k_lo + lane, nI = n_l - 1u, tau = (uint32_t)cc.tau;
             uint32_t m = 0, M = 0, sumX = 0, maxX = 0;
-            if (cand && n > 1) {                              // stream X: one token of the candidate, then the target
+            const uint32_t sum0 = on0 ? o_s0 + nI * base0 : nI * tau, sum1 = on1 ? o_s1 + nI * base1 : nI * tau;
+            if (BOTH && cand && nI) {
                 m = 1;
-                if (cand == 1) M = (uint32_t)gc.kappa * (__shfl_sync(FULL, l_l, r) + 1u) + (uint32_t)gc.c0;
+                if (to_dev) M = (uint32_t)gc.kappa * (l_l + 1u) + (uint32_t)gc.c0;
                 else {
-                    const uint32_t u = mix32(key);            // a server TTFT drawn from F by its knots
+                    const uint32_t u = mix32(key_l);          // a server TTFT drawn from F by its knots
                     const uint32_t ki = u >> 24, fr = (u >> 8) & 0xFFFFu;
                     const int32_t* K = knots + g * kNKnots;
                     if (DBG_OK(ki + 1, kNKnots, DBG_K_PLAYOUT, DBG_KNOT))
                         M = (uint32_t)(K[ki] + (int32_t)(((int64_t)(K[ki + 1] - K[ki]) * (int64_t)fr) >> 16));
                 }
-                sumX = M + (sum[tgt] - first[tgt]);
-                maxX = max(M, most_later[tgt]);
-                const int shift = cc.lo[g][2] - st[tgt].lo, skip = bin_of_ticks(first[tgt]) - st[tgt].lo;
-                const uint32_t* wt = tgt ? win1 : win0;
-                for (int b = lane; b < W2; b += 32) {
-                    const int t = b + shift;
-                    uint32_t v = (t >= 0 && t < st[tgt].W) ? wt[t] : 0u;
-                    if (t == skip) --v;
-                    rec.win[2][(size_t)k * W2 + b] = (uint16_t)v;
-                }
-                __syncwarp();
+                const uint32_t base = to_dev ? base1 : base0;
+                sumX = M + (to_dev ? sum1 : sum0) - (base + __umulhi(mix32(key_l + 2u * kHashTok), to_dev ? mul1 : mul0));
+                maxX = max(M, nI > 1u ? base + o_later : 0u);
             }
-            // the windows go out and are cleared for the next request
-            if (st[0].on) for (int b = lane; b < W0; b += 32) { rec.win[0][(size_t)k * W0 + b] = (uint16_t)win0[b]; win0[b] = 0; }
-            if (st[1].on) for (int b = lane; b < W1; b += 32) { rec.win[1][(size_t)k * W1 + b] = (uint16_t)win1[b]; win1[b] = 0; }
-            __syncwarp();
-            if (lane == r) {
-                o_sum[0] = sum[0]; o_sum[1] = sum[1]; o_sum[2] = sumX; o_max[0] = most[0]; o_max[1] = most[1]; o_max[2] = maxX;
-                o_m = m; o_stall = M;
-            }
-        }
-        if (lane < n_here) {
-            const uint32_t k = k_lo + lane;
-            rec.hand[k] = make_uint2(o_m, o_stall);
-#pragma unroll
-            for (int s = 0; s < 3; ++s) { rec.sum[s][k] = o_sum[s]; rec.max[s][k] = o_max[s]; }
+            rec.hand[k] = make_uint2(m, M);
+            rec.sum[0][k] = sum0; rec.sum[1][k] = sum1; rec.sum[2][k] = sumX;
+            rec.max[0][k] = nI ? (on0 ? o_m0 + base0 : tau) : 0u; rec.max[1][k] = nI ? (on1 ? o_m1 + base1 : tau) : 0u;
+            rec.max[2][k] = maxX;
         }
         __syncwarp();
     }
@@ -135,14 +186,21 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
 DBG_TRANSLATION_UNIT()
 
 cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const ClassConst& host_cc,
-                                const int32_t* knots, uint32_t k0, TimelineRec rec, int32_t* err, uint32_t batches, int sms,
+                                const int32_t* knots, uint32_t k0, TimelineRec rec, uint32_t batches, int sms,
                                 cudaStream_t st) {
-    const size_t smem = (size_t)kFreeWarps * (host_cc.W[0] + host_cc.W[1]) * 4;
+    // as many warps to a block as the windows leave room for (wide jitter: up to 114 KB of counters a stream and warp)
+    const size_t per_warp = (size_t)(host_cc.W[0] + host_cc.W[1]) * 33 * 4;
+    const uint32_t warps = std::max<uint32_t>(1u, std::min<uint32_t>(kFreeWarps, (uint32_t)(100 * 1024 / per_warp)));
+    const size_t smem = per_warp * warps;
+    bool small = false;                                       // intervals below 32 ticks occur
+    for (int g = 0; g < tr.n_groups; ++g) small = small || host_cc.lo[g][0] < 32 || host_cc.lo[g][1] < 32;
+    auto* kernel = host_cc.pacing ? (small ? k_playout_free<false, true> : k_playout_free<false, false>)
+                                  : (small ? k_playout_free<true, true> : k_playout_free<true, false>);
     cudaError_t e;
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(k_playout_free, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-    const uint32_t blocks = std::min<uint32_t>((batches + kFreeWarps - 1) / kFreeWarps, (uint32_t)sms * 32u);
-    return launch_after(k_playout_free, blocks, kFreeWarps * 32, smem, st, tr, gc, cc, knots, k0, rec, err);
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024))) return e;
+    // (batches counts 32 requests each; four blocks of eight warps fit a multiprocessor)
+    const uint32_t blocks = std::min<uint32_t>((batches * (32 / kFreeBatch) + warps - 1) / warps, (uint32_t)sms * 4u * kFreeWarps / warps);
+    return launch_after(kernel, blocks, warps * 32, smem, st, tr, gc, cc, knots, k0, rec);
 }
 
 }  // namespace disco
