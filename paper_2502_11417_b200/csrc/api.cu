@@ -97,9 +97,10 @@ struct disco_ctx {
     const void* gc_dev_at = nullptr;
     // trace
     DevBuf in_prompt, in_out, in_ttft, in_sp, in_dp;      // staging of host inputs
-    DevBuf keys_a, keys_b, tmp_idx, tmp_ln, cursors, inv;
-    DevBuf req, sorted;
-    DevBuf zero, cum_mass, ng_exact, grp_off, knots, d_gc;   // `zero`: every table a load must clear, contiguous
+    DevBuf st_ticks, st_ln, st_g;                         // the trace as the ingestion leaves it when it reads host memory
+    DevBuf binned, tick_start, len_end, inv, req, sorted;
+    DevBuf keys_a, keys_b, radix_counts, sort_in;         // radix sort (fallback) and the sort of imported ticks
+    DevBuf zero, cum_mass, grp_off, knots, d_gc;          // `zero`: what a load must clear, contiguous
     DevBuf fin_totals;                 // [2G] u64: output tokens and requests per group that the accumulators cover
     uint64_t first_index = 0;          // index of request 0 in the whole trace (hash key base)
     int sms = 0;                       // multiprocessors of the context's device
@@ -111,8 +112,8 @@ struct disco_ctx {
     std::vector<uint64_t> F_n;         // requests per group behind F (the group's own count unless imported)
     bool fin_imported = false;         // fin_totals holds a caller's merged totals, not this trace's
     std::vector<uint64_t> fin_own;     // this trace's totals, to put back before the next evaluation
-    uint32_t *cnt = nullptr, *ng = nullptr, *max_n = nullptr, *radix_counts = nullptr;
-    uint64_t* grp_sum_n = nullptr;
+    LoadZero* z = nullptr;
+    uint32_t *cnt = nullptr, *tick_cnt = nullptr;
     int32_t* err = nullptr;
     size_t zero_bytes = 0;
     HostReadback* rb = nullptr;
@@ -137,8 +138,8 @@ struct disco_ctx {
     bool timing_valid = false;
 
     ~disco_ctx() {
-        DevBuf* all[] = {&in_prompt, &in_out, &in_ttft, &in_sp, &in_dp, &keys_a, &keys_b, &tmp_idx, &tmp_ln, &cursors, &inv,
-                         &req, &sorted, &zero, &cum_mass, &ng_exact, &grp_off, &knots, &d_gc, &d_prep, &d_accum, &d_stats, &d_tables, &d_grid, &rec_hand,
+        DevBuf* all[] = {&in_prompt, &in_out, &in_ttft, &in_sp, &in_dp, &st_ticks, &st_ln, &st_g, &binned, &tick_start, &len_end, &inv,
+                         &req, &sorted, &keys_a, &keys_b, &radix_counts, &sort_in, &zero, &cum_mass, &grp_off, &knots, &d_gc, &d_prep, &d_accum, &d_stats, &d_tables, &d_grid, &rec_hand,
                          &fin_totals, &F_sorted_imp, &F_off_imp, &d_left};
         for (DevBuf* b : all) b->release();
         for (auto& b : rec_u32) b.release();
@@ -193,7 +194,7 @@ int check_profiles(const disco_trace_desc_t* d, std::vector<GroupConst>* out) {
     return 0;
 }
 
-cudaError_t reserve_trace(disco_ctx* c, uint32_t n, bool host_inputs, bool has_sp, bool has_dp) {
+cudaError_t reserve_trace(disco_ctx* c, uint32_t n, bool host_inputs, bool in_place, bool has_sp, bool has_dp) {
     cudaError_t e;
     const size_t N = n ? n : 1;
     const int G = c->G;
@@ -203,25 +204,36 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, bool host_inputs, bool has_s
         if (has_sp) R(in_sp, N);
         if (has_dp) R(in_dp, N);
     }
-    R(keys_a, N * 8); R(keys_b, N * 8);
-    R(tmp_ln, N * 4); R(cursors, (size_t)G * (kMaxPrompt + 1) * 4); R(inv, N * 4); R(req, N * 16); R(sorted, N * 4);
-    // one block for everything a load clears: cnt | grp_sum_n | ng | max_n | err | first radix counter buffer,
-    // followed by the second counter buffer
-    const size_t cnt_bytes = ((size_t)G * (kMaxPrompt + 1) * 4 + 15) / 16 * 16;
-    const size_t counts_bytes = (size_t)256 * kRadixMaxBlocks * 4;
-    const size_t head = cnt_bytes + kMaxGroups * 8 + kMaxGroups * 4 + 16 + 16;
-    R(zero, head + 5 * counts_bytes + 1024);                    // + the 256 digit totals
-    char* z = (char*)c->zero.p;
-    c->cnt = (uint32_t*)z; c->grp_sum_n = (uint64_t*)(z + cnt_bytes); c->ng = (uint32_t*)(z + cnt_bytes + kMaxGroups * 8);
-    c->max_n = (uint32_t*)(z + cnt_bytes + kMaxGroups * 12); c->err = (int32_t*)(z + cnt_bytes + kMaxGroups * 12 + 16);
-    c->radix_counts = (uint32_t*)(z + head);
-    c->zero_bytes = head;
-    R(cum_mass, (size_t)G * (kMaxPrompt + 2) * 8); R(ng_exact, kMaxGroups * 4);
+    if (in_place) { R(st_ticks, N * 4); R(st_ln, N * 4); R(st_g, N); }
+    R(binned, N * 4); R(req, N * 16); R(sorted, N * 4);
+    if (G == 1) R(inv, N * 4);
+    R(tick_start, (size_t)2 * G * kTickBins * 4); R(len_end, (size_t)G * (kMaxPrompt + 1) * 4);
+    // one block for everything a load clears: the flags and sums, the two histograms
+    const size_t tick_bytes = (size_t)G * kTickBins * 4, cnt_bytes = ((size_t)G * (kMaxPrompt + 1) * 4 + 15) / 16 * 16;
+    R(zero, sizeof(LoadZero) + tick_bytes + cnt_bytes);
+    c->z = (LoadZero*)c->zero.p;
+    c->tick_cnt = (uint32_t*)(c->z + 1);
+    c->cnt = (uint32_t*)((char*)c->tick_cnt + tick_bytes);
+    c->err = c->z->err;
+    c->zero_bytes = sizeof(LoadZero) + tick_bytes + cnt_bytes;
+    R(cum_mass, (size_t)G * (kMaxPrompt + 2) * 8);
     R(grp_off, (kMaxGroups + 1) * 4); R(knots, (size_t)G * kNKnots * 4);
     R(d_gc, (size_t)G * sizeof(GroupConst));
     R(fin_totals, (size_t)2 * kMaxGroups * 8);
 #undef R
     return cudaSuccess;
+}
+
+// The fallback sort: ticks stored group after group (off: [G + 1], device memory) ascending within each group into out.
+int radix_sort(disco_ctx* c, const int32_t* ticks, const uint32_t* off, uint32_t total, int32_t* out, cudaStream_t st) {
+    cudaError_t e;
+    if ((e = c->keys_a.reserve((size_t)total * 8)) != cudaSuccess || (e = c->keys_b.reserve((size_t)total * 8)) != cudaSuccess ||
+        (e = c->radix_counts.reserve(((size_t)256 * kRadixMaxBlocks + 256) * 4)) != cudaSuccess)
+        return fail_cuda(e, "device allocation for the radix sort");
+    if ((e = radix_sort_ticks(ticks, off, c->G, total, c->keys_a.as<uint64_t>(), c->keys_b.as<uint64_t>(),
+                              c->radix_counts.as<uint32_t>(), out, c->sms, st)) != cudaSuccess) return fail_cuda(e, "radix sort");
+    g_launches += radix_sort_launches(c->G);
+    return 0;
 }
 
 }  // namespace
@@ -285,12 +297,12 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     if (zero_copy) host_in = false;
     if (!c->rb && (e = cudaMallocHost((void**)&c->rb, sizeof(HostReadback))) != cudaSuccess)
         return bail(fail_cuda(e, "cudaMallocHost"));
-    if ((e = reserve_trace(c, n, host_in, d->server_profile != nullptr, d->device_profile != nullptr)) != cudaSuccess)
+    if ((e = reserve_trace(c, n, host_in, zero_copy, d->server_profile != nullptr, d->device_profile != nullptr)) != cudaSuccess)
         return bail(fail_cuda(e, "device allocation for the trace"));
 
     LoadArgs a;
     std::memset(&a, 0, sizeof a);
-    a.n = n; a.ns = c->ns; a.nd = c->nd;
+    a.n = n; a.G = c->G; a.ns = c->ns; a.nd = c->nd;
     if (host_in && n) {
 #define H2D(dst, src, bytes) if ((e = cudaMemcpyAsync(c->dst.p, src, bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess) return bail(fail_cuda(e, "host to device copy"))
         H2D(in_prompt, d->prompt_len, (size_t)n * 4); H2D(in_out, d->output_len, (size_t)n * 4);
@@ -308,14 +320,14 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         a.prompt = d->prompt_len; a.outlen = d->output_len; a.ttft = d->server_ttft_s;
         a.sp = d->server_profile; a.dp = d->device_profile;
     }
-    a.keys_a = c->keys_a.as<uint64_t>(); a.keys_b = c->keys_b.as<uint64_t>(); a.cursors = c->cursors.as<uint32_t>(); a.inv = c->inv.as<uint32_t>(); a.req = c->req.as<uint4>();
-    a.l_tmp = c->tmp_ln.as<uint16_t>(); a.n_tmp = c->tmp_ln.as<uint16_t>() + (n ? n : 1);
-    a.radix_counts = c->radix_counts; a.zero_block = c->zero.p; a.zero_bytes = c->zero_bytes;
-    a.ng_exact = c->ng_exact.as<uint32_t>(); a.readback = c->rb;     // pinned host memory, written by the last kernel
-    a.sorted = c->sorted.as<int32_t>(); a.cnt = c->cnt; a.cum_mass = c->cum_mass.as<int64_t>();
-    a.ng = c->ng; a.grp_off = c->grp_off.as<uint32_t>(); a.knots = c->knots.as<int32_t>();
-    a.grp_sum_n = c->grp_sum_n; a.max_n = c->max_n; a.err = c->err;
-    a.fin_totals = c->fin_totals.as<uint64_t>(); a.sms = c->sms;
+    if (zero_copy) { a.st_ticks = c->st_ticks.as<uint32_t>(); a.st_ln = c->st_ln.as<uint32_t>(); a.st_g = c->st_g.as<uint8_t>(); }
+    a.z = c->z; a.cnt = c->cnt; a.tick_cnt = c->tick_cnt;
+    a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)c->G * kTickBins;
+    a.binned = c->binned.as<uint32_t>();
+    a.req = c->req.as<uint4>(); a.inv = c->G == 1 ? c->inv.as<uint32_t>() : nullptr; a.sorted = c->sorted.as<int32_t>();
+    a.len_end = c->len_end.as<uint32_t>(); a.cum_mass = c->cum_mass.as<int64_t>(); a.grp_off = c->grp_off.as<uint32_t>();
+    a.knots = c->knots.as<int32_t>(); a.fin_totals = c->fin_totals.as<uint64_t>();
+    a.readback = c->rb;                                             // pinned host memory, written by the kernel
     // the profile table is read from pageable memory: this copy returns once it has been staged
     const bool same_profiles = c->gc_dev_at == c->d_gc.p && c->gc_dev.size() == c->gc.size() &&
                                std::memcmp(c->gc_dev.data(), c->gc.data(), c->gc.size() * sizeof(GroupConst)) == 0;
@@ -324,8 +336,9 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         if ((e = cudaMemcpyAsync(c->d_gc.p, c->gc.data(), c->gc.size() * sizeof(GroupConst), cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return bail(fail_cuda(e, "profile copy"));
     }
-    if ((e = run_load(a, st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion kernels"));
-    g_launches += load_kernel_launches(n, c->G);
+    if ((e = cudaMemsetAsync(c->zero.p, 0, c->zero_bytes, st)) != cudaSuccess ||
+        (e = run_load(a, c->sms, st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion kernel"));
+    g_launches += 1;
     // the few numbers the host needs (error word, group sizes, longest output, largest TTFT per group) are in rb
     HostReadback* rb = c->rb;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion"));
@@ -335,6 +348,19 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         static const char* what[] = {"", "prompt length outside 1..4096", "output length outside 1..8192",
                                      "server TTFT not finite, not positive or above 2000 s", "profile id out of range"};
         return bail(fail(DISCO_EINVAL, std::string(what[rb->err[0]]) + " at request " + std::to_string(rb->err[1])));
+    }
+    if (rb->err[3] == 2) return bail(fail(DISCO_ECUDA, "internal error: the blocks of the ingestion kernel lost each other"));
+    if (rb->err[3] == 1) {
+        // a sample that the bin-wise sort gives up on: radix sort, then the knots of the sorted sample
+        if (int rc = radix_sort(c, c->binned.as<int32_t>(), c->grp_off.as<uint32_t>(), n, c->sorted.as<int32_t>(), st)) return bail(rc);
+        if ((e = launch_tables_imported(c->G, c->cnt, c->cum_mass.as<int64_t>(), c->sorted.as<int32_t>(), c->grp_off.as<uint32_t>(),
+                                        c->knots.as<int32_t>(), st)) != cudaSuccess) return bail(fail_cuda(e, "group tables"));
+        g_launches += 1;
+        for (int g = 0; g < c->G; ++g)
+            if (rb->ng[g] && (e = cudaMemcpyAsync(&rb->knot_max[g], c->sorted.as<int32_t>() + rb->grp_off[g + 1] - 1, 4,
+                                                  cudaMemcpyDeviceToHost, st)) != cudaSuccess) return bail(fail_cuda(e, "group tables"));
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion"));
+        if (int rc = debug_check()) return bail(rc);
     }
     c->F_sorted = c->sorted.as<int32_t>(); c->F_off = c->grp_off.as<uint32_t>();
     c->F_n.assign(rb->ng, rb->ng + c->G);
@@ -691,7 +717,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
 
     TraceDev tr;
     tr.n = n; tr.n_groups = G; tr.req = c->req.as<uint4>(); tr.inv = c->inv.as<uint32_t>();
-    tr.len_end = c->cursors.as<uint32_t>(); tr.grp_off = c->grp_off.as<uint32_t>();
+    tr.len_end = c->len_end.as<uint32_t>(); tr.grp_off = c->grp_off.as<uint32_t>();
     TimelineRec rec;
     rec.hand = c->rec_hand.as<uint2>();
     for (int k = 0; k < 3; ++k) {
@@ -944,21 +970,22 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     if (total && !ticks) return fail(DISCO_EINVAL, "null argument");
     cudaError_t e;
     const size_t T1 = (size_t)std::max<uint64_t>(total, 1);
-    // the sort's scratch: the key buffers of the load (free between loads), grown if the whole trace is larger
+    const size_t tick_bytes = (size_t)G * kTickBins * 4;
     if ((e = c->F_sorted_imp.reserve(T1 * 4)) != cudaSuccess || (e = c->F_off_imp.reserve((size_t)(kMaxGroups + 1) * 4)) != cudaSuccess ||
-        (e = c->keys_a.reserve(T1 * 8)) != cudaSuccess || (e = c->keys_b.reserve(T1 * 8)) != cudaSuccess ||
-        (e = c->tmp_idx.reserve(T1 * 4)) != cudaSuccess)
+        (e = c->sort_in.reserve(2 * T1 * 4)) != cudaSuccess)
         return fail_cuda(e, "device allocation for the tables");
-    CU(cudaMemsetAsync(c->err, 0, 16, st));
-    if (total) CU(cudaMemcpyAsync(c->tmp_idx.p, ticks, (size_t)total * 4, cudaMemcpyDefault, st));
+    int32_t* in = c->sort_in.as<int32_t>();
+    CU(cudaMemsetAsync(c->z, 0, sizeof(LoadZero) + tick_bytes, st));
+    if (total) CU(cudaMemcpyAsync(in, ticks, (size_t)total * 4, cudaMemcpyDefault, st));
     CU(cudaMemcpyAsync(c->F_off_imp.p, off.data(), (size_t)(G + 1) * 4, cudaMemcpyHostToDevice, st));
     CU(cudaMemcpyAsync(c->cnt, cnt32.data(), cnt32.size() * 4, cudaMemcpyHostToDevice, st));
-    uint32_t* counts = c->radix_counts + (size_t)4 * 256u * kRadixMaxBlocks;
-    CU(sort_grouped_ticks(c->tmp_idx.as<int32_t>(), c->F_off_imp.as<uint32_t>(), G, (uint32_t)total, c->keys_a.as<uint64_t>(),
-                          c->keys_b.as<uint64_t>(), counts, c->err, c->F_sorted_imp.as<int32_t>(), c->sms, st));
-    CU(launch_tables_imported(G, c->cnt, c->cum_mass.as<int64_t>(), c->ng_exact.as<uint32_t>(),
-                              c->F_sorted_imp.as<int32_t>(), c->F_off_imp.as<uint32_t>(), c->knots.as<int32_t>(), st));
-    if (total) g_launches += 2 + 3 * (G > 1 ? 5 : 4);
+    LoadArgs a = {};
+    a.n = (uint32_t)total; a.G = G; a.ticks = in; a.off = c->F_off_imp.as<uint32_t>();
+    a.z = c->z; a.tick_cnt = c->tick_cnt; a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)G * kTickBins;
+    a.binned = (uint32_t*)in + T1; a.sorted = c->F_sorted_imp.as<int32_t>();
+    if (total) { CU(run_sort_ticks(a, c->sms, st)); g_launches += 1; }
+    CU(launch_tables_imported(G, c->cnt, c->cum_mass.as<int64_t>(), c->F_sorted_imp.as<int32_t>(), c->F_off_imp.as<uint32_t>(),
+                              c->knots.as<int32_t>(), st));
     g_launches += 1;
     // error word and each group's largest tick (the largest hand-off latency a draw from F can give)
     int32_t err_host[4] = {0, 0, 0, 0};
@@ -969,6 +996,17 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     CU(cudaStreamSynchronize(st));          // the host vectors above are read by the copies until here
     if (int rc = debug_check()) { c->loaded = false; return rc; }
     c->evaluated = c->reduced = false;
+    if (err_host[3] == 2) { c->loaded = false; return fail(DISCO_ECUDA, "internal error: the blocks of the sort lost each other"); }
+    if (!err_host[0] && err_host[3] == 1) {
+        if (int rc = radix_sort(c, in, c->F_off_imp.as<uint32_t>(), (uint32_t)total, c->F_sorted_imp.as<int32_t>(), st)) { c->loaded = false; return rc; }
+        CU(launch_tables_imported(G, c->cnt, c->cum_mass.as<int64_t>(), c->F_sorted_imp.as<int32_t>(), c->F_off_imp.as<uint32_t>(),
+                                  c->knots.as<int32_t>(), st));
+        g_launches += 1;
+        for (int g = 0; g < G; ++g)
+            if (n_ticks[g]) CU(cudaMemcpyAsync(&top[g], c->F_sorted_imp.as<int32_t>() + off[g + 1] - 1, 4, cudaMemcpyDeviceToHost, st));
+        CU(cudaStreamSynchronize(st));
+        if (int rc = debug_check()) { c->loaded = false; return rc; }
+    }
     if (err_host[0]) {
         c->loaded = false;                  // the length counts have been overwritten: the context must be reloaded
         return fail(DISCO_EINVAL, "negative TTFT tick at position " + std::to_string(err_host[1]) + "; reload the trace");

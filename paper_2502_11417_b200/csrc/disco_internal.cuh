@@ -278,13 +278,8 @@ cudaError_t launch_finalize(uint32_t P, int G, const GroupConst* gc, const uint6
 cudaError_t launch_select(const disco_policy_stats_t* stats, uint32_t P, double cost_cap, float tbt_slo_s,
                           int32_t* result /* [2]: status, index; may be pinned host memory */, cudaStream_t st);
 // Cumulative token mass and knots from tables given by the caller (F_off[g] .. F_off[g+1] delimit group g's ticks).
-cudaError_t launch_tables_imported(int G, const uint32_t* cnt, int64_t* cum_mass, uint32_t* ng_exact,
-                                   const int32_t* F_sorted, const uint32_t* F_off, int32_t* knots, cudaStream_t st);
-// Sorts ticks stored group after group (off[g] .. off[g+1], device memory) ascending within each group into `out`;
-// keys_a / keys_b: scratch of `total` 64-bit words each, counts: 256 * 1024 + 256 words; err[0..1]: set to (3, index) on
-// a negative tick.  Launches 2 + 3 * (G > 1 ? 5 : 4) kernels.
-cudaError_t sort_grouped_ticks(const int32_t* ticks, const uint32_t* off, int G, uint32_t total, uint64_t* keys_a,
-                               uint64_t* keys_b, uint32_t* counts, int32_t* err, int32_t* out, int sms, cudaStream_t st);
+cudaError_t launch_tables_imported(int G, const uint32_t* cnt, int64_t* cum_mass, const int32_t* F_sorted,
+                                   const uint32_t* F_off, int32_t* knots, cudaStream_t st);
 // Checked build: 0, or DISCO_ECUDA (error string set) if a kernel refused an index since the last call.  Always 0 in
 // an ordinary build.  To be called after the stream has been synchronised.
 int check_debug_record();

@@ -1,574 +1,573 @@
-// Trace ingestion on the device: tick conversion and validation, per-group prompt-length histogram,
-// internal request order (by group, then by prompt length), radix sort of the server-TTFT ticks (the empirical F of
+// Trace ingestion on the device in one kernel: tick conversion and validation, per-group prompt-length histogram,
+// internal request order (by group, then by prompt length), sort of the server-TTFT ticks (the empirical F of
 // Algorithm 1), cumulative input-token mass (Eq. 3) and the quantile knots of F.
+//
+// One block of 1024 threads per multiprocessor, all resident at once (a cooperative launch), works in three passes with a
+// wait for all blocks between them:
+//   1. count: every request is checked and counted by (group, prompt length) and by (group, bin of its ticks), 128 bins an
+//      octave, in counters of the block's own.  The block adds its counters to the global ones and keeps what was there
+//      before: where its own requests of each bucket go within the bucket.
+//   2. place: from the totals every block works out where the buckets start, then sends its requests to their places: one
+//      16-byte record into the internal order and the ticks into their bin.
+//   3. sort: the bins in order, about 4,096 ticks at a time, are sorted in shared memory (all ticks of a window differ in
+//      few low bits), each window by one block.  A bin of more than 8,192 ticks that spans at most 2^18 values is sorted by
+//      counting them; a trace that has a denser and wider one goes to the radix sort (radix.cu) instead.
+//
+// Bound: latency at 10^5 requests (one launch instead of eighteen), memory at 10^7: the columns are read twice (once when
+// they are in host memory: then the first pass leaves a copy), 20 bytes a request are written to scattered places, the
+// ticks are read and written once more.
 #include "load.cuh"
 
 #include <algorithm>
 #include <mutex>
 
+#include "scan.cuh"
+
 namespace disco {
 
 namespace {
 
-constexpr int kIngestThreads = 1024;
+constexpr int kThreads = 1024;
+constexpr int kLens = kMaxPrompt + 1;
+constexpr uint32_t FULL = 0xFFFFFFFFu;
+constexpr uint32_t kWindow = 4096;        // a window starts with the first bin behind every 4,096th tick of its group
+constexpr uint32_t kSortCap = 8192;       // ticks sorted at a time
+constexpr uint32_t kCounters = 16384;     // values counted at a time
+constexpr uint32_t kMaxRange = 1u << 18;  // values a dense bin may span
+constexpr uint32_t kMaxCount = 1u << 24;  // ticks a dense bin may hold
+constexpr int kPrivateGroups = 7;         // groups whose counters fit in shared memory (29 KB each)
+constexpr int kPrivateTickGroups = 16;    // the same, counters of tick bins alone
+constexpr int kUnroll = 4;                // requests a thread has in flight
 
-__global__ void k_ingest(uint32_t n, const int32_t* __restrict__ prompt, const int32_t* __restrict__ outlen,
-                         const float* __restrict__ ttft, const uint8_t* __restrict__ sp,
-                         const uint8_t* __restrict__ dp, uint32_t ns, uint32_t nd, uint64_t* __restrict__ keys,
-                         uint32_t* __restrict__ cnt, unsigned long long* __restrict__ grp_sum_n,
-                         uint32_t* __restrict__ grp_n, uint32_t* __restrict__ max_n, int32_t* __restrict__ err,
-                         uint16_t* __restrict__ l_out, uint16_t* __restrict__ n_out,
-                         uint32_t* __restrict__ counts0, uint32_t per_block0,
-                         uint32_t blocks0, int hist_groups) {
-    // l_out, n_out: packed copies of the lengths in the caller's order, for the scatter into the internal order;
-    // counts0: first radix digit counted per sort block (small traces; large ones use the histogram kernel)
-    __shared__ unsigned long long s_sum[kMaxGroups];
-    __shared__ uint32_t s_cnt[kMaxGroups];
-    __shared__ uint32_t s_max, s_max_ticks;         // longest output, largest TTFT ticks (max_n[0], max_n[1])
-    // hist_groups: groups whose length histograms this block keeps in shared memory (all of them, or none when they
-    // do not fit: then the counts go to global memory one by one)
-    extern __shared__ uint32_t s_len[];              // [hist_groups][kMaxPrompt + 1]
-    const int G = (int)(ns * nd);
-    const bool one = G == 1;
-    for (int g = threadIdx.x; g < G; g += blockDim.x) { s_sum[g] = 0; s_cnt[g] = 0; }
-    for (int i = threadIdx.x; i < hist_groups * (kMaxPrompt + 1); i += blockDim.x) s_len[i] = 0;
-    if (threadIdx.x == 0) { s_max = 0; s_max_ticks = 0; }
+enum Source { S_TRACE, S_TICKS, S_TTFT };
+
+__device__ __forceinline__ int tick_bin(uint32_t t) {
+    return t < 128u ? (int)t : (int)(__float_as_uint(__uint2float_rz(t)) >> 16) - ((127 + 7) << 7) + 128;
+}
+__device__ __forceinline__ uint32_t tick_bin_edge(int b) {     // smallest ticks of the bin (2^31 behind the last)
+    return b < 128 ? (uint32_t)b : (uint32_t)(128 + (b & 127)) << ((b >> 7) - 1);
+}
+
+struct SortSmem {
+    uint32_t a[kSortCap], b[kSortCap];                 // ticks of a window, twice; or kCounters counters
+    uint16_t wcnt[kThreads / 32][256];                 // keys of each digit per warp; or the list of frequent values
+    uint32_t dig[256];
+    uint32_t wtot[32];
+    uint32_t lo, hi, n_list;
+    int bin0, bin1;
+};
+static_assert(kCounters == 2 * kSortCap, "the counters lie over the two key arrays");
+
+// Waits until every block of the grid has come here `times` times.  The wait is bounded: a block that gives up sets the
+// flag and goes on (the host refuses the results).
+__device__ __forceinline__ void grid_barrier(LoadZero* z, uint32_t times) {
     __syncthreads();
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t i0 = blockIdx.x * blockDim.x; i0 < n; i0 += stride) {       // whole warps iterate together
-        const uint32_t i = i0 + threadIdx.x;
-        const bool in = i < n;
-        const int32_t l = in ? prompt[i] : 1, o = in ? outlen[i] : 1;
-        const float t = in ? ttft[i] : 1.0f;
-        const uint32_t s = (in && sp) ? sp[i] : 0u, d = (in && dp) ? dp[i] : 0u;
-        int bad = 0;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&z->barrier, 1u);
+        const uint32_t want = times * gridDim.x;
+        uint32_t seen, tries = 0;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&z->barrier) : "memory");
+        } while (seen < want && ++tries < (1u << 22));
+        if (seen < want) atomicExch(&z->err[3], 2);
+        __threadfence();
+    }
+    __syncthreads();
+}
+
+// A request of the trace (or a tick of a sample) as the two passes see it.
+struct Item { uint32_t g, S, l, o; bool in; };
+
+// First pass: reads and checks item i.
+template <int SRC>
+__device__ __forceinline__ Item check_item(const LoadArgs& a, uint32_t i, const uint32_t* s_off) {
+    Item x = {0u, 0u, 1u, 1u, i < a.n};
+    if (!x.in) return x;
+    int bad = 0;
+    if (SRC == S_TICKS) {
+        while ((int)x.g + 1 < a.G && i >= s_off[x.g + 1]) ++x.g;
+        const int32_t t = a.ticks[i];
+        if (t < 0) bad = 3;
+        x.S = (uint32_t)t;
+    } else {
+        const float t = a.ttft[i];
+        uint32_t s = 0, d = 0;
+        int32_t l = 1, o = 1;
+        if (SRC == S_TRACE) { l = a.prompt[i]; o = a.outlen[i]; s = a.sp ? a.sp[i] : 0u; d = a.dp ? a.dp[i] : 0u; }
         if (l < 1 || l > kMaxPrompt) bad = 1;
         else if (o < 1 || o > kMaxOutput) bad = 2;
         else if (!(t > 0.0f) || !(t <= 2000.0f)) bad = 3;      // NaN fails both comparisons
-        else if (s >= ns || d >= nd) bad = 4;
-        const bool ok = in && !bad;
-        if (in && bad) {
-            if (atomicCAS(&err[0], 0, bad) == 0) err[1] = (int32_t)i;
-            keys[i] = 0;
-        }
+        else if (SRC == S_TRACE && (s >= a.ns || d >= a.nd)) bad = 4;
         // ticks = nearest integer (ties to even) of the fp64 product, as a host llrint would give
-        const long long S = __double2ll_rn(__dmul_rn((double)t, 1e6));
-        const uint32_t g = ok ? s * nd + d : 0u;
-        if (ok && DBG_OK(g, G, DBG_K_INGEST, DBG_GROUP) && DBG_OK(l, kMaxPrompt + 1, DBG_K_INGEST, DBG_TABLE)) {
-            keys[i] = ((uint64_t)g << 32) | (uint32_t)S;
-            if (hist_groups) atomicAdd(&s_len[g * (kMaxPrompt + 1) + l], 1u); else atomicAdd(&cnt[g * (kMaxPrompt + 1) + l], 1u);
-            l_out[i] = (uint16_t)l; n_out[i] = (uint16_t)o;
-            if (counts0 && DBG_OK(i / per_block0, blocks0, DBG_K_INGEST, DBG_COUNTER))
-                atomicAdd(&counts0[((uint32_t)S & 255u) * blocks0 + i / per_block0], 1u);
-        }
-        if (one) {                                             // one group: sums by warp reduction
-            const uint32_t so = __reduce_add_sync(0xFFFFFFFFu, ok ? (uint32_t)o : 0u);
-            const uint32_t mo = __reduce_max_sync(0xFFFFFFFFu, ok ? (uint32_t)o : 0u);
-            const uint32_t co = __popc(__ballot_sync(0xFFFFFFFFu, ok));
-            const uint32_t mt = __reduce_max_sync(0xFFFFFFFFu, ok ? (uint32_t)S : 0u);
-            if ((threadIdx.x & 31) == 0 && co) {
-                atomicAdd(&s_sum[0], (unsigned long long)so); atomicAdd(&s_cnt[0], co); atomicMax(&s_max, mo);
-                atomicMax(&s_max_ticks, mt);
-            }
-        } else {
-            // several groups: the lanes of each group present in the warp add up among themselves, one lane adds
-            const uint32_t mo = __reduce_max_sync(0xFFFFFFFFu, ok ? (uint32_t)o : 0u);
-            const uint32_t mt = __reduce_max_sync(0xFFFFFFFFu, ok ? (uint32_t)S : 0u);
-            uint32_t rest = __ballot_sync(0xFFFFFFFFu, ok);
-            const int lane = threadIdx.x & 31;
-            if (lane == 0 && rest) { atomicMax(&s_max, mo); atomicMax(&s_max_ticks, mt); }
-            while (rest) {
-                const int first = __ffs(rest) - 1;
-                const uint32_t g1 = __shfl_sync(0xFFFFFFFFu, g, first);
-                const bool mine = ok && g == g1;
-                const uint32_t same = __ballot_sync(0xFFFFFFFFu, mine);
-                const uint32_t so = __reduce_add_sync(0xFFFFFFFFu, mine ? (uint32_t)o : 0u);
-                if (lane == first) { atomicAdd(&s_sum[g1], (unsigned long long)so); atomicAdd(&s_cnt[g1], (uint32_t)__popc(same)); }
-                rest &= ~same;
-            }
-        }
+        x.S = (uint32_t)__double2ll_rn(__dmul_rn((double)t, 1e6));
+        x.g = s * a.nd + d; x.l = (uint32_t)l; x.o = (uint32_t)o;
+        if (SRC == S_TTFT) x.g = 0;
     }
-    __syncthreads();
-    for (int g = threadIdx.x; g < G; g += blockDim.x)
-        if (s_cnt[g]) { atomicAdd(&grp_sum_n[g], s_sum[g]); atomicAdd(&grp_n[g], s_cnt[g]); }
-    for (int i = threadIdx.x; i < hist_groups * (kMaxPrompt + 1); i += blockDim.x) if (s_len[i]) atomicAdd(&cnt[i], s_len[i]);
-    if (threadIdx.x == 0 && s_max) { atomicMax(max_n, s_max); atomicMax(max_n + 1, s_max_ticks); }
+    if (bad) {
+        if (atomicCAS(&a.z->err[0], 0, bad) == 0) a.z->err[1] = (int32_t)i;
+        x.in = false;
+    }
+    return x;
 }
 
-// Inclusive prefix sum over the threads of a block (blockDim.x a multiple of 32, at most 1024): shuffles inside
-// the warps, one pass over the warp totals, two barriers.  `wtot` is shared scratch of 32 entries; every thread
-// of the block must call.  Returns this thread's inclusive sum; *total receives the block's sum.
-template <class T>
-__device__ __forceinline__ T block_inclusive_scan(T v, T* wtot, T* total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const T up = __shfl_up_sync(0xFFFFFFFFu, v, off);
-        if (lane >= off) v += up;
-    }
-    if (lane == 31) wtot[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        T t = lane < nw ? wtot[lane] : T(0);
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const T up = __shfl_up_sync(0xFFFFFFFFu, t, off);
-            if (lane >= off) t += up;
+// Second pass: the same item, known to be good.
+template <int SRC, bool STAGE>
+__device__ __forceinline__ Item read_item(const LoadArgs& a, uint32_t i, const uint32_t* s_off) {
+    Item x = {0u, 0u, 1u, 1u, i < a.n};
+    if (!x.in) return x;
+    if (STAGE) {
+        const uint32_t ln = a.st_ln[i];
+        x.S = a.st_ticks[i]; x.l = ln & 0xFFFFu; x.o = ln >> 16; x.g = a.st_g[i];
+    } else if (SRC == S_TICKS) {
+        while ((int)x.g + 1 < a.G && i >= s_off[x.g + 1]) ++x.g;
+        x.S = (uint32_t)a.ticks[i];
+    } else {
+        x.S = (uint32_t)__double2ll_rn(__dmul_rn((double)a.ttft[i], 1e6));
+        if (SRC == S_TRACE) {
+            x.l = (uint32_t)a.prompt[i]; x.o = (uint32_t)a.outlen[i];
+            x.g = (a.sp ? a.sp[i] : 0u) * a.nd + (a.dp ? a.dp[i] : 0u);
         }
-        wtot[lane] = t;                                   // inclusive over the warps
     }
-    __syncthreads();
-    if (total) *total = wtot[nw - 1];
-    return w ? v + wtot[w - 1] : v;
+    return x;
 }
 
-// ---- one stable LSD radix pass over 64-bit keys (8-bit digit), optional 32-bit payload -------------------
-constexpr int kRadixThreads = 256;
-constexpr int kRadixWarps = kRadixThreads / 32;
-
-__global__ void k_radix_hist(const uint64_t* __restrict__ keys, uint32_t n, uint32_t per_block, int shift,
-                             uint32_t* __restrict__ counts /* [256][gridDim.x] */,
-                             const uint32_t* __restrict__ max_key = nullptr, uint32_t skip_below = 0) {
-    // max_key, skip_below: the pass is not needed (every key has this digit zero, the order is final) when the
-    // largest key is below skip_below; the kernels of such a pass return at once
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
-    grid_dependency_wait();
-    if (max_key && *max_key < skip_below) return;
+// Exclusive prefix sums of L <= 5 * kThreads counters, `base` added; emit(k, count, start).  All threads call.
+template <class E>
+__device__ __forceinline__ void scan_counts(const uint32_t* cnt, int L, uint32_t base, uint32_t* wtot, E emit) {
+    constexpr int kPer = 5;
+    const int k0 = (int)threadIdx.x * kPer;
+    uint32_t c[kPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) { c[k] = k0 + k < L ? __ldcg(&cnt[k0 + k]) : 0u; sum += c[k]; }
+    uint32_t run = base + block_inclusive_scan(sum, wtot, (uint32_t*)nullptr) - sum;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) { if (k0 + k < L) emit(k0 + k, c[k], run); run += c[k]; }
     __syncthreads();
-    const uint32_t lo = min(n, blockIdx.x * per_block), hi = min(n, lo + per_block);
-    for (uint32_t i = lo + threadIdx.x; i < hi; i += kRadixThreads)
-        atomicAdd(&h[(uint32_t)(keys[i] >> shift) & 255u], 1u);
-    __syncthreads();
-    counts[threadIdx.x * gridDim.x + blockIdx.x] = h[threadIdx.x];
 }
 
-// One block per digit: exclusive scan of the digit's per-block counts, in place, and the digit's total.
-__global__ void k_radix_rowscan(uint32_t* __restrict__ counts /* [256][blocks] */, uint32_t blocks,
-                                uint32_t* __restrict__ totals /* [256] */,
-                                const uint32_t* __restrict__ max_key = nullptr, uint32_t skip_below = 0) {
-    __shared__ uint32_t wtot[32];
-    grid_dependency_wait();
-    if (max_key && *max_key < skip_below) return;
-    uint32_t* row = counts + (size_t)blockIdx.x * blocks;
-    const uint32_t per = (blocks + 127u) / 128u;
-    const uint32_t lo = min(blocks, threadIdx.x * per), hi = min(blocks, lo + per);
-    uint32_t s = 0;
-    for (uint32_t i = lo; i < hi; ++i) s += row[i];
-    uint32_t total;
-    uint32_t run = block_inclusive_scan(s, wtot, &total) - s;
-    for (uint32_t i = lo; i < hi; ++i) { const uint32_t c = row[i]; row[i] = run; run += c; }
-    if (threadIdx.x == 0) totals[blockIdx.x] = total;
+// Cumulative input-token mass cum[L] = sum_{l<L} l cnt[l], L = 0 .. 4097.  All threads call.
+__device__ __forceinline__ void group_mass(const uint32_t* cnt, int64_t* cum, unsigned long long* wm) {
+    constexpr int kPer = 5;
+    const int k0 = (int)threadIdx.x * kPer;
+    uint32_t c[kPer];
+    unsigned long long m = 0, total;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) { c[k] = k0 + k < kLens ? __ldcg(&cnt[k0 + k]) : 0u; m += (unsigned long long)(k0 + k) * c[k]; }
+    unsigned long long run = block_inclusive_scan(m, wm, &total) - m;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) { if (k0 + k < kLens) cum[k0 + k] = (int64_t)run; run += (unsigned long long)(k0 + k) * c[k]; }
+    if (threadIdx.x == 0) cum[kLens] = (int64_t)total;
+    __syncthreads();
 }
 
-__global__ void k_radix_scatter(const uint64_t* __restrict__ keys_in, uint64_t* __restrict__ keys_out,
-                                const uint32_t* __restrict__ pay_in, uint32_t* __restrict__ pay_out, uint32_t n,
-                                uint32_t per_block, int shift, const uint32_t* __restrict__ offsets,
-                                const uint32_t* __restrict__ totals, uint32_t* __restrict__ counts_next = nullptr,
-                                int32_t* __restrict__ low_out = nullptr,
-                                const uint32_t* __restrict__ max_key = nullptr, uint32_t skip_below = 0,
-                                int32_t* __restrict__ low_out_if_last = nullptr, uint32_t last_below = 0) {
-    // low_out: the last pass writes the low words (the sorted ticks) instead of the keys.  low_out_if_last: this
-    // pass writes them as well when the largest key is below last_below (the later passes then skip themselves).
-    __shared__ uint32_t run[256];                 // next output slot of each digit for this block
-    __shared__ uint32_t wcnt[kRadixWarps][256];   // keys of each digit per warp in the current slab
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    grid_dependency_wait();
-    if (max_key && *max_key < skip_below) return;
-    if (low_out_if_last && *max_key >= last_below) low_out_if_last = nullptr;
-    {
-        // offsets[d][b]: keys of digit d in earlier blocks (k_radix_rowscan); totals[d]: keys of digit d.
-        // This block's first slot for digit d = keys of smaller digits + keys of d in earlier blocks.
-        uint32_t* wtot = wcnt[0];                                    // scratch of the scan (32 words)
-        const uint32_t total = totals[threadIdx.x], before = offsets[threadIdx.x * gridDim.x + blockIdx.x];
-        const uint32_t incl = block_inclusive_scan(total, wtot, (uint32_t*)nullptr);
-        run[threadIdx.x] = incl - total + before;
-        __syncthreads();
+// Sorts `count` <= kSortCap ticks from src (all of them in [lo, lo + 2^bits)) into out: stable counting passes of at most
+// eight bits in shared memory, a warp's 256 keys at a time with the ranks from ballots.
+__device__ __forceinline__ void sort_window(SortSmem& sm, const uint32_t* src, uint32_t count, uint32_t lo, int bits, int32_t* out) {
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    if (bits == 0) {
+        for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)lo;
+        return;
     }
-    const uint32_t lo = min(n, blockIdx.x * per_block), hi = min(n, lo + per_block);
-    constexpr int kPer = 4;                                   // keys per thread and tile
-    constexpr uint32_t kTile = kRadixThreads * kPer;          // a warp owns 128 consecutive keys of a tile
-    for (uint32_t base = lo; base < hi; base += kTile) {
-        for (int k = 0; k < kRadixWarps; ++k) wcnt[k][threadIdx.x] = 0;
-        uint64_t key[kPer];
-        uint32_t dig[kPer], peers[kPer];
-        bool live[kPer];
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const uint32_t i = base + w * (32 * kPer) + j * 32 + lane;
-            live[j] = i < hi;
-            key[j] = live[j] ? keys_in[i] : 0;
-            dig[j] = (uint32_t)(key[j] >> shift) & 255u;
-            // lanes holding the same digit, from eight ballots over the digit's bits
-            uint32_t m = __ballot_sync(0xFFFFFFFFu, live[j]);
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, (dig[j] >> b) & 1u);
-                m &= ((dig[j] >> b) & 1u) ? bal : ~bal;
-            }
-            peers[j] = m;
-        }
+    uint32_t *from = sm.a, *to = sm.b;
+    for (uint32_t i = tid; i < count; i += kThreads) from[i] = __ldcg(&src[i]) - lo;
+    const int passes = (bits + 7) / 8, d_bits = (bits + passes - 1) / passes, digits = 1 << d_bits;
+    const int rounds = (int)((min(count, 256u) + 31u) / 32u), warps = (int)((count + 255u) / 256u);
+    for (int p = 0; p < passes; ++p) {
+        const int shift = p * d_bits;
+        for (int i = tid; i < warps * 256; i += kThreads) (&sm.wcnt[0][0])[i] = 0;
         __syncthreads();
-        // keys of each digit in each warp (a warp's row is its own: plain adds, rounds in order)
+        uint32_t key[8], place[8];                    // place: digit | rank among the warp's equal digits so far << 8
+        if (w < warps) {
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            if (live[j] && (peers[j] & ((1u << lane) - 1u)) == 0) wcnt[w][dig[j]] += __popc(peers[j]);
-            __syncwarp();
-        }
-        __syncthreads();
-        {   // turn the counts into each warp's first slot per digit; advance the block's running slots
-            uint32_t at = run[threadIdx.x];
-            for (int k = 0; k < kRadixWarps; ++k) { const uint32_t c = wcnt[k][threadIdx.x]; wcnt[k][threadIdx.x] = at; at += c; }
-            run[threadIdx.x] = at;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            uint32_t nxt = 0xFFFFFFFFu;                          // next pass's counter for this key (none: dead lane)
-            if (live[j]) {
-                const uint32_t rank = __popc(peers[j] & ((1u << lane) - 1u));
-                const uint32_t pos = wcnt[w][dig[j]] + rank;
-                if (DBG_OK(pos, n, DBG_K_RADIX, DBG_ELEMENT)) {
-                    if (low_out) low_out[pos] = (int32_t)(uint32_t)key[j]; else keys_out[pos] = key[j];
-                    if (low_out_if_last) low_out_if_last[pos] = (int32_t)(uint32_t)key[j];
-                    if (pay_out) {
-                        const uint32_t i = base + w * (32 * kPer) + j * 32 + lane;
-                        pay_out[pos] = pay_in ? pay_in[i] : i;
-                    }
+            for (int j = 0; j < 8; ++j) {
+                if (j >= rounds) break;
+                const uint32_t i = w * 256u + j * 32u + lane;
+                const bool live = i < count;
+                key[j] = live ? from[i] : 0u;
+                const uint32_t d = (key[j] >> shift) & (uint32_t)(digits - 1);
+                uint32_t peers = __ballot_sync(FULL, live);
+                for (int b = 0; b < d_bits; ++b) {
+                    const uint32_t bal = __ballot_sync(FULL, (d >> b) & 1u);
+                    peers &= ((d >> b) & 1u) ? bal : ~bal;
                 }
-                if (DBG_OK(pos / per_block, gridDim.x, DBG_K_RADIX, DBG_COUNTER))
-                    nxt = ((uint32_t)(key[j] >> (shift + 8)) & 255u) * gridDim.x + pos / per_block;
+                const uint32_t below = __popc(peers & ((1u << lane) - 1u));
+                uint32_t before = 0;
+                if (live) before = sm.wcnt[w][d];
+                __syncwarp();
+                if (live && below == 0) sm.wcnt[w][d] = (uint16_t)(before + __popc(peers));
+                __syncwarp();
+                place[j] = d | (before + below) << 8;
             }
-            __syncwarp();
-            if (counts_next) {
-                // lanes bound for the same counter add once: high digits take few values, and one add per key
-                // would queue every key of the trace on a handful of addresses
-                const uint32_t same = __match_any_sync(0xFFFFFFFFu, nxt);
-                if (live[j] && (same & ((1u << lane) - 1u)) == 0) atomicAdd(&counts_next[nxt], (uint32_t)__popc(same));
+        }
+        __syncthreads();
+        // where each digit starts, and each warp's keys of it
+        uint32_t total = 0;
+        if (tid < digits) for (int k = 0; k < warps; ++k) { const uint32_t c = sm.wcnt[k][tid]; sm.wcnt[k][tid] = (uint16_t)total; total += c; }
+        const uint32_t incl = block_inclusive_scan(tid < digits ? total : 0u, sm.wtot, (uint32_t*)nullptr);
+        if (tid < digits) sm.dig[tid] = incl - total;
+        __syncthreads();
+        if (w < warps) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (j >= rounds) break;
+                const uint32_t i = w * 256u + j * 32u + lane;
+                if (i < count) {
+                    const uint32_t d = place[j] & 255u, at = sm.dig[d] + sm.wcnt[w][d] + (place[j] >> 8);
+                    if (DBG_OK(at, count, DBG_K_RADIX, DBG_ELEMENT)) to[at] = key[j];
+                }
             }
-            if (live[j] && (peers[j] & ((1u << lane) - 1u)) == 0) wcnt[w][dig[j]] += __popc(peers[j]);
-            __syncwarp();
         }
+        __syncthreads();
+        uint32_t* t = from; from = to; to = t;
+    }
+    for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)(from[i] + lo);
+}
+
+// Sorts a dense bin by counting its values.  Returns false where that would take too long.
+__device__ __forceinline__ bool sort_dense(SortSmem& sm, const uint32_t* src, uint32_t count, int32_t* out) {
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    if (tid == 0) { sm.lo = 0xFFFFFFFFu; sm.hi = 0u; }
+    __syncthreads();
+    uint32_t mn = 0xFFFFFFFFu, mx = 0u;
+    for (uint32_t i = tid; i < count; i += kThreads) { const uint32_t t = __ldcg(&src[i]); mn = min(mn, t); mx = max(mx, t); }
+    mn = __reduce_min_sync(FULL, mn); mx = __reduce_max_sync(FULL, mx);
+    if (lane == 0) { atomicMin(&sm.lo, mn); atomicMax(&sm.hi, mx); }
+    __syncthreads();
+    const uint32_t lo = sm.lo, range = sm.hi - lo + 1u;
+    if (range == 1u) {
+        for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)lo;
+        return true;
+    }
+    if (range > kMaxRange || count > kMaxCount) return false;
+    uint32_t* n_of = sm.a;                                            // kCounters of them
+    uint16_t* list = &sm.wcnt[0][0];
+    constexpr uint32_t kOften = 4096;                                 // such values are written by the whole block
+    uint32_t done = 0;
+    for (uint32_t r0 = 0; r0 < range; r0 += kCounters) {
+        for (uint32_t i = tid; i < kCounters; i += kThreads) n_of[i] = 0;
+        if (tid == 0) sm.n_list = 0;
+        __syncthreads();
+        for (uint32_t i = tid; i < count; i += kThreads) {
+            const uint32_t v = __ldcg(&src[i]) - lo - r0;
+            if (v < kCounters) atomicAdd(&n_of[v], 1u);
+        }
+        __syncthreads();
+        // a thread's sixteen values, then where they start
+        constexpr uint32_t kPer = kCounters / kThreads;
+        uint32_t sum = 0, total;
+        for (uint32_t k = 0; k < kPer; ++k) sum += n_of[tid * kPer + k];
+        uint32_t run = done + block_inclusive_scan(sum, sm.wtot, &total) - sum;
+        // a warp writes its threads' values one thread after another, 32 copies at a time
+        for (int t = 0; t < 32; ++t) {
+            uint32_t at = __shfl_sync(FULL, run, t);
+            if (__shfl_sync(FULL, sum, t) == 0u) continue;
+            for (uint32_t k = 0; k < kPer; ++k) {
+                const uint32_t v = (uint32_t)(w * 32 + t) * kPer + k, c = n_of[v];
+                if (c > kOften) {
+                    if (lane == 0) { const uint32_t e = atomicAdd(&sm.n_list, 1u); if (DBG_OK(e, 8192, DBG_K_RADIX, DBG_SLOT)) list[e] = (uint16_t)v; }
+                } else {
+                    for (uint32_t j = lane; j < c; j += 32) out[at + j] = (int32_t)(lo + r0 + v);
+                }
+                at += c;
+            }
+        }
+        __syncthreads();
+        for (uint32_t e = 0; e < sm.n_list; ++e) {                    // (at most kMaxCount / kOften of them)
+            const uint32_t v = list[e];
+            // where it starts: the counters in front of it
+            uint32_t part = 0;
+            for (uint32_t k = tid; k < v; k += kThreads) part += n_of[k];
+            uint32_t before;
+            block_inclusive_scan(part, sm.wtot, &before);
+            const uint32_t c = n_of[v];
+            for (uint32_t j = tid; j < c; j += kThreads) out[done + before + j] = (int32_t)(lo + r0 + v);
+            __syncthreads();
+        }
+        done += total;
         __syncthreads();
     }
+    return true;
 }
 
-// Where the requests of each (group, prompt length) start in the internal order: the groups one after another,
-// inside a group the prompt lengths ascending.  One block of 1024 threads per group.
-__global__ void __launch_bounds__(1024)
-k_length_cursors(const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ ng, uint32_t* __restrict__ cursor) {
-    constexpr int NT = 1024, L = kMaxPrompt + 1;
-    __shared__ uint32_t wc[32];
-    const int g = blockIdx.x;
-    uint32_t base = 0;
-    for (int h = 0; h < g; ++h) base += ng[h];
-    const int per = (L + NT - 1) / NT;
-    const int lo = min(L, (int)threadIdx.x * per), hi = min(L, lo + per);
-    uint32_t k = 0;
-    for (int l = lo; l < hi; ++l) k += cnt[(size_t)g * L + l];
-    uint32_t run = base + block_inclusive_scan(k, wc, (uint32_t*)nullptr) - k;
-    for (int l = lo; l < hi; ++l) { cursor[(size_t)g * L + l] = run; run += cnt[(size_t)g * L + l]; }
-}
+template <int SRC, bool PRIV, bool STAGE>
+__global__ void __launch_bounds__(kThreads, 1)
+k_load(const __grid_constant__ LoadArgs a) {
+    constexpr bool kTrace = SRC == S_TRACE;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_off[kMaxGroups + 1];        // group offsets in the internal order
+    __shared__ unsigned long long s_wide[32];
+    __shared__ uint32_t s_wtot[32];
+    __shared__ unsigned long long s_sum[kMaxGroups];
+    __shared__ uint32_t s_max, s_item;
+    const int G = a.G, tid = threadIdx.x, lane = tid & 31;
+    LoadZero* z = a.z;
+    uint32_t* s_len = (uint32_t*)smem_raw;                             // [G][kLens]
+    uint32_t* s_tick = s_len + (kTrace ? G * kLens : 0);               // [G][kTickBins]
+    uint32_t waits = 0;
 
-// The internal request order: each request takes the next free place of its (group, prompt length).  Requests of
-// one group and length keep no particular order among themselves (nothing downstream depends on it: req[].z and inv
-// map between the two orders).  The lanes of a warp that share a bucket take their places with one add.  A
-// request goes to its place as one 16-byte record (ticks, lengths, caller's index), which is what the later kernels read.
-__global__ void k_scatter_by_length(uint32_t n, int G, const uint64_t* __restrict__ keys,
-                                    const uint16_t* __restrict__ prompt, const uint16_t* __restrict__ outlen,
-                                    const int32_t* __restrict__ err, uint32_t* __restrict__ cursor,
-                                    uint4* __restrict__ req, uint32_t* __restrict__ inv) {
-    if (err[0] != 0) return;                          // a rejected trace: its lengths were not all written
-    const int lane = threadIdx.x & 31;
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t i0 = blockIdx.x * blockDim.x; i0 < n; i0 += stride) {       // whole warps iterate together
-        const uint32_t i = i0 + threadIdx.x;
-        bool in = i < n;
-        const uint64_t key = in ? keys[i] : 0ull;
-        const uint32_t g = (uint32_t)(key >> 32), len = in ? prompt[i] : 0u;
-        in = in && DBG_OK(g, G, DBG_K_GATHER, DBG_GROUP) && DBG_OK(len, kMaxPrompt + 1, DBG_K_GATHER, DBG_TABLE);
-        const uint32_t live = __ballot_sync(0xFFFFFFFFu, in);
-        if (!in) continue;
-        const uint32_t bucket = g * (uint32_t)(kMaxPrompt + 1) + len;
-        const uint32_t peers = __match_any_sync(live, bucket);
-        const int leader = __ffs(peers) - 1;
-        uint32_t at = 0;
-        if (lane == leader) at = atomicAdd(&cursor[bucket], (uint32_t)__popc(peers));
-        at = __shfl_sync(peers, at, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
-        if (!DBG_OK(at, n, DBG_K_GATHER, DBG_REQUEST)) continue;
-        req[at] = make_uint4((uint32_t)key, len | ((uint32_t)outlen[i] << 16), i, 0u);
-        inv[i] = at;
+    // ---- 1. count
+    if (PRIV) for (int i = tid; i < (kTrace ? G * kLens : 0) + G * kTickBins; i += kThreads) s_len[i] = 0;
+    if (SRC == S_TICKS) for (int g = tid; g <= G; g += kThreads) s_off[g] = a.off[g];
+    for (int g = tid; g < G; g += kThreads) s_sum[g] = 0;
+    if (tid == 0) s_max = 0;
+    __syncthreads();
+    const uint32_t stride = gridDim.x * kThreads, i_first = blockIdx.x * kThreads + tid;
+    uint32_t tok[kPrivateGroups] = {};                                 // output tokens per group
+    uint32_t longest = 0;
+    for (uint32_t i0 = i_first; i0 < a.n; i0 += kUnroll * stride) {
+        Item x[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const uint32_t i = i0 + u * stride;
+            x[u] = check_item<SRC>(a, i, s_off);
+        }
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const Item& y = x[u];
+            if (!y.in || !DBG_OK(y.g, G, DBG_K_INGEST, DBG_GROUP) || !DBG_OK(y.l, kLens, DBG_K_INGEST, DBG_TABLE)) continue;
+            const int tb = tick_bin(y.S);
+            if (!DBG_OK(tb, kTickBins, DBG_K_INGEST, DBG_BIN)) continue;
+            if (STAGE) {
+                const uint32_t i = i0 + u * stride;
+                a.st_ticks[i] = y.S; a.st_ln[i] = y.l | y.o << 16; a.st_g[i] = (uint8_t)y.g;
+            }
+            if (PRIV) {
+                if (kTrace) atomicAdd(&s_len[y.g * kLens + y.l], 1u);
+                atomicAdd(&s_tick[y.g * kTickBins + tb], 1u);
+            } else {
+                if (kTrace) { atomicAdd(&a.cnt[(size_t)y.g * kLens + y.l], 1u); atomicAdd(&s_sum[y.g], (unsigned long long)y.o); }
+                atomicAdd(&a.tick_cnt[(size_t)y.g * kTickBins + tb], 1u);
+            }
+            if (kTrace) {
+                longest = max(longest, y.o);
+                if (PRIV) {
+#pragma unroll
+                    for (int g = 0; g < kPrivateGroups; ++g) tok[g] += (int)y.g == g ? y.o : 0u;    // (at most 2^21 requests a thread)
+                }
+            }
+        }
     }
-}
-
-// The same for traces whose length histograms fit in shared memory (up to six groups).  A block takes slices of
-// kSliceRequests requests: it counts the slice's requests per bucket in shared memory, reserves each bucket's places
-// with ONE add to the global cursor, and hands the places out from shared memory.  A popular bucket's cursor then
-// sees one add per slice instead of one per warp (adds to one address are served one after another).
-constexpr uint32_t kSliceRequests = 16384;
-constexpr int kSliceThreads = 1024;
-
-__global__ void __launch_bounds__(kSliceThreads)
-k_scatter_by_length_slices(uint32_t n, int G, const uint64_t* __restrict__ keys,
-                           const uint16_t* __restrict__ prompt, const uint16_t* __restrict__ outlen,
-                           const int32_t* __restrict__ err, uint32_t* __restrict__ cursor,
-                           uint4* __restrict__ req, uint32_t* __restrict__ inv) {
-    extern __shared__ uint32_t s_at[];               // [G][kMaxPrompt + 1]: counts, then next free places
-    if (err[0] != 0) return;                         // a rejected trace: its lengths were not all written
-    const uint32_t buckets = (uint32_t)G * (uint32_t)(kMaxPrompt + 1);
-    for (uint32_t lo = blockIdx.x * kSliceRequests; lo < n; lo += gridDim.x * kSliceRequests) {
-        const uint32_t hi = min(n, lo + kSliceRequests);
-        for (uint32_t b = threadIdx.x; b < buckets; b += kSliceThreads) s_at[b] = 0;
-        __syncthreads();
-        for (uint32_t i = lo + threadIdx.x; i < hi; i += kSliceThreads) {
-            const uint32_t g = (uint32_t)(keys[i] >> 32), len = prompt[i];
-            if (DBG_OK(g, G, DBG_K_GATHER, DBG_GROUP) && DBG_OK(len, kMaxPrompt + 1, DBG_K_GATHER, DBG_TABLE))
-                atomicAdd(&s_at[g * (uint32_t)(kMaxPrompt + 1) + len], 1u);
+    if (kTrace) {
+        longest = __reduce_max_sync(FULL, longest);
+        if (lane == 0 && longest) atomicMax(&s_max, longest);
+        if (PRIV) {
+#pragma unroll
+            for (int g = 0; g < kPrivateGroups; ++g) {
+                if (g >= G) break;
+                unsigned long long v = tok[g];
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+                if (lane == 0 && v) atomicAdd(&s_sum[g], v);
+            }
         }
-        __syncthreads();
-        for (uint32_t b = threadIdx.x; b < buckets; b += kSliceThreads) {
-            const uint32_t c = s_at[b];
-            if (c) s_at[b] = atomicAdd(&cursor[b], c);
-        }
-        __syncthreads();
-        for (uint32_t i = lo + threadIdx.x; i < hi; i += kSliceThreads) {
-            const uint64_t key = keys[i];
-            const uint32_t g = (uint32_t)(key >> 32), len = prompt[i];
-            if (!DBG_OK(g, G, DBG_K_GATHER, DBG_GROUP) || !DBG_OK(len, kMaxPrompt + 1, DBG_K_GATHER, DBG_TABLE)) continue;
-            const uint32_t at = atomicAdd(&s_at[g * (uint32_t)(kMaxPrompt + 1) + len], 1u);
-            if (!DBG_OK(at, n, DBG_K_GATHER, DBG_REQUEST)) continue;
-            req[at] = make_uint4((uint32_t)key, len | ((uint32_t)outlen[i] << 16), i, 0u);
-            inv[i] = at;
-        }
-        __syncthreads();
-    }
-}
-
-__global__ void k_low_words(uint32_t n, const uint64_t* __restrict__ keys, int32_t* __restrict__ out) {
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-        out[k] = (int32_t)(uint32_t)keys[k];
-}
-
-// One block of 1024 threads per group: cumulative input-token mass cum[L] = sum_{l<L} l*cnt[l], L = 0..4097, and N_g.
-__device__ __forceinline__ void group_mass(const uint32_t* __restrict__ cnt, int64_t* __restrict__ cum,
-                                           uint32_t* __restrict__ ng) {
-    constexpr int NT = 1024, L = kMaxPrompt + 1;      // 4097 lengths
-    __shared__ unsigned long long wm[32];
-    __shared__ uint32_t wc[32];
-    const int g = blockIdx.x;
-    const uint32_t* c = cnt + (size_t)g * L;
-    int64_t* out = cum + (size_t)g * (L + 1);
-    const int per = (L + NT - 1) / NT;                 // 5
-    const int lo = min(L, (int)threadIdx.x * per), hi = min(L, lo + per);
-    unsigned long long m = 0; uint32_t k = 0;
-    for (int l = lo; l < hi; ++l) { m += (unsigned long long)l * c[l]; k += c[l]; }
-    unsigned long long m_total; uint32_t k_total;
-    unsigned long long run = block_inclusive_scan(m, wm, &m_total) - m;
-    block_inclusive_scan(k, wc, &k_total);
-    for (int l = lo; l < hi; ++l) { out[l] = (int64_t)run; run += (unsigned long long)l * c[l]; }
-    if (threadIdx.x == 0) { out[L] = (int64_t)m_total; ng[g] = k_total; }
-}
-
-// Group offsets in the partitioned order, the 257 knots K_g[k] = sorted_g[(k (N_g - 1)) / 256] and the few
-// numbers the host reads back.  One block per group (ng: the group sizes counted at ingestion).
-__device__ __forceinline__ void group_knots(int G, const uint32_t* __restrict__ ng, const int32_t* __restrict__ sorted,
-                                            uint32_t* __restrict__ grp_off, int32_t* __restrict__ knots,
-                                            const int32_t* __restrict__ err, const uint32_t* __restrict__ max_n,
-                                            const unsigned long long* __restrict__ grp_sum_n,
-                                            unsigned long long* __restrict__ fin_totals,
-                                            LoadReadback* __restrict__ rb) {
-    __shared__ uint32_t off[kMaxGroups + 1];
-    const int g = blockIdx.x;
-    if (threadIdx.x == 0) {
-        uint32_t r = 0;
-        for (int k = 0; k < G; ++k) { off[k] = r; r += ng[k]; }
-        off[G] = r;
     }
     __syncthreads();
-    const uint32_t N = off[g + 1] - off[g];
-    for (int k = threadIdx.x; k < kNKnots; k += blockDim.x) {
-        const uint32_t at = N ? (uint32_t)(((uint64_t)k * (N - 1)) / 256u) : 0u;
-        knots[g * kNKnots + k] = (N && DBG_OK(at, N, DBG_K_TABLES, DBG_ELEMENT)) ? sorted[off[g] + at] : 0;
+    if (kTrace) {
+        for (int g = tid; g < G; g += kThreads) if (s_sum[g]) atomicAdd((unsigned long long*)&z->grp_sum_n[g], s_sum[g]);
+        if (tid == 0 && s_max) atomicMax(&z->max_n, s_max);
     }
-    if (threadIdx.x == 0) {
-        rb->knot_max[g] = N ? sorted[off[g] + N - 1] : 0;
-        rb->ng[g] = N; rb->grp_sum_n[g] = grp_sum_n[g];
-        fin_totals[g] = grp_sum_n[g]; fin_totals[G + g] = N;      // what the final reductions' totals refer to
-        if (g == 0) {
-            for (int k = 0; k <= G; ++k) { grp_off[k] = off[k]; rb->grp_off[k] = off[k]; }
-            for (int k = 0; k < 4; ++k) rb->err[k] = err[k];
-            rb->max_n = *max_n;
+    // the block's counters join the global ones; what it finds there is where its own requests go within the bucket
+    if (PRIV) {
+        auto join = [&](uint32_t* mine, uint32_t* all, int count) {
+            for (int i0 = tid; i0 < count; i0 += 4 * kThreads) {
+                uint32_t c[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) { const int i = i0 + u * kThreads; c[u] = i < count ? mine[i] : 0u; }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) if (c[u]) c[u] = atomicAdd(&all[i0 + u * kThreads], c[u]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) { const int i = i0 + u * kThreads; if (i < count) mine[i] = c[u]; }
+            }
+        };
+        if (kTrace) join(s_len, a.cnt, G * kLens);
+        join(s_tick, a.tick_cnt, G * kTickBins);
+    }
+    grid_barrier(z, ++waits);
+
+    // ---- 2. place
+    const int32_t bad = __ldcg(&z->err[0]);
+    // group sizes: the sum of their tick counts
+    uint32_t base = 0;
+    for (int g = 0; g < G; ++g) {
+        if (SRC != S_TICKS && tid == 0) s_off[g] = base;
+        const bool mine = (int)(blockIdx.x % (uint32_t)G) == g || gridDim.x < (uint32_t)G;    // the blocks that write the group's tables
+        uint32_t in_group = 0;
+        auto ticks_at = [&](int k, uint32_t c, uint32_t start) {
+            const size_t at = (size_t)g * kTickBins + k;
+            if (PRIV) s_tick[at] += start;
+            if (mine) { a.tick_start[at] = start; if (!PRIV && blockIdx.x < (uint32_t)G) a.tick_at[at] = start; }
+            if (k == kTickBins - 1) s_item = start + c - base;
+        };
+        scan_counts(a.tick_cnt + (size_t)g * kTickBins, kTickBins, base, s_wtot, ticks_at);
+        in_group = s_item;
+        if (kTrace) {
+            scan_counts(a.cnt + (size_t)g * kLens, kLens, base, s_wtot, [&](int k, uint32_t c, uint32_t start) {
+                const size_t at = (size_t)g * kLens + k;
+                if (PRIV) { s_len[at] += start; if (mine) a.len_end[at] = start + c; }
+                else if (mine && blockIdx.x < (uint32_t)G) a.len_end[at] = start;      // the cursor, which ends up there
+            });
+            if (mine) group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
         }
+        base += in_group;
+        __syncthreads();
+    }
+    if (SRC != S_TICKS && tid == 0) s_off[G] = base;
+    __syncthreads();
+    if (kTrace && blockIdx.x == 0) {
+        for (int g = tid; g < G; g += kThreads) {
+            const uint32_t N = s_off[g + 1] - s_off[g];
+            const uint64_t sum = __ldcg((const unsigned long long*)&z->grp_sum_n[g]);
+            a.readback->ng[g] = N; a.readback->grp_sum_n[g] = sum; a.readback->grp_off[g] = s_off[g];
+            a.grp_off[g] = s_off[g];
+            a.fin_totals[g] = sum; a.fin_totals[G + g] = N;            // what the final reductions' totals refer to
+            if (N == 0) a.readback->knot_max[g] = 0;
+        }
+        if (tid == 0) { a.grp_off[G] = s_off[G]; a.readback->grp_off[G] = s_off[G]; a.readback->max_n = __ldcg(&z->max_n); }
+        for (int k = tid; k < G * kNKnots; k += kThreads)
+            if (s_off[k / kNKnots + 1] == s_off[k / kNKnots]) a.knots[k] = 0;
+    }
+    if (bad) {                                         // a rejected trace: nothing is placed
+        if (kTrace && blockIdx.x == 0 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
+        return;
+    }
+    if (!PRIV) grid_barrier(z, ++waits);               // the cursors are complete
+    for (uint32_t i0 = i_first; i0 < a.n; i0 += kUnroll * stride) {
+        Item x[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const uint32_t i = i0 + u * stride;
+            x[u] = read_item<SRC, STAGE>(a, i, s_off);
+        }
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const Item& y = x[u];
+            const uint32_t i = i0 + u * stride;
+            if (!y.in || !DBG_OK(y.g, G, DBG_K_GATHER, DBG_GROUP) || !DBG_OK(y.l, kLens, DBG_K_GATHER, DBG_TABLE)) continue;
+            const uint32_t tb = y.g * kTickBins + (uint32_t)tick_bin(y.S);
+            const uint32_t tp = atomicAdd(PRIV ? &s_tick[tb] : &a.tick_at[tb], 1u);
+            if (DBG_OK(tp, a.n, DBG_K_GATHER, DBG_ELEMENT)) a.binned[tp] = y.S;
+            if (kTrace) {
+                const uint32_t lb = y.g * kLens + y.l;
+                const uint32_t at = atomicAdd(PRIV ? &s_len[lb] : &a.len_end[lb], 1u);
+                if (!DBG_OK(at, a.n, DBG_K_GATHER, DBG_REQUEST)) continue;
+                a.req[at] = make_uint4(y.S, y.l | y.o << 16, i, 0u);
+                if (a.inv) a.inv[i] = at;
+            }
+        }
+    }
+    grid_barrier(z, ++waits);
+
+    // ---- 3. sort
+    SortSmem& sm = *reinterpret_cast<SortSmem*>(smem_raw);
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) s_item = atomicAdd(&z->ticket, 1u);
+        __syncthreads();
+        uint32_t win = s_item;
+        int g = 0;
+        for (; g < G; ++g) {
+            const uint32_t here = (s_off[g + 1] - s_off[g] + kWindow - 1) / kWindow;
+            if (win < here) break;
+            win -= here;
+        }
+        if (g == G) break;
+        const uint32_t first = s_off[g], N = s_off[g + 1] - first;
+        const uint32_t* start = a.tick_start + (size_t)g * kTickBins;
+        // the window's bins: those that hold ticks and start in [first + win * kWindow, ... + kWindow)
+        if (tid == 0) { sm.bin0 = kTickBins; sm.bin1 = -1; }
+        __syncthreads();
+        const uint32_t x0 = first + win * kWindow, x1 = x0 + kWindow;
+        const uint32_t* counts = a.tick_cnt + (size_t)g * kTickBins;
+        int b_min = kTickBins, b_max = -1;
+        for (int b = tid; b < kTickBins; b += kThreads) {
+            const uint32_t s = __ldcg(&start[b]), c = __ldcg(&counts[b]);
+            if (c && s >= x0 && s < x1) { b_min = min(b_min, b); b_max = max(b_max, b); }
+        }
+        if (b_max >= 0) { atomicMin(&sm.bin0, b_min); atomicMax(&sm.bin1, b_max); }
+        __syncthreads();
+        const int b0 = sm.bin0, b1 = sm.bin1;
+        if (b1 < 0) continue;                                          // (inside a large bin)
+        const uint32_t k0 = __ldcg(&start[b0]), k2 = __ldcg(&start[b1]), k1 = k2 + __ldcg(&counts[b1]);
+        const uint32_t lo = tick_bin_edge(b0);
+        auto bits_of = [](uint32_t range) { return range <= 1u ? 0 : 32 - __clz((int)(range - 1u)); };
+        if (k1 - k0 <= kSortCap) {
+            sort_window(sm, a.binned + k0, k1 - k0, lo, bits_of(tick_bin_edge(b1 + 1) - lo), a.sorted + k0);
+        } else {                                                       // the last bin is a large one: the others first
+            if (k2 > k0) {
+                sort_window(sm, a.binned + k0, k2 - k0, lo, bits_of(tick_bin_edge(b1) - lo), a.sorted + k0);
+                __syncthreads();
+            }
+            if (!sort_dense(sm, a.binned + k2, k1 - k2, a.sorted + k2) && tid == 0) atomicExch(&z->err[3], 1);
+        }
+        __syncthreads();
+        if (kTrace) {
+            // the knots K_g[k] = sorted_g[(k (N_g - 1)) / 256] that lie in the window
+            for (int k = tid; k < kNKnots; k += kThreads) {
+                const uint32_t at = first + (uint32_t)(((uint64_t)k * (N - 1)) / 256u);
+                if (at >= k0 && at < k1) {
+                    const int32_t v = __ldcg(&a.sorted[at]);
+                    a.knots[g * kNKnots + k] = v;
+                    if (k == kNKnots - 1) a.readback->knot_max[g] = v;
+                }
+            }
+        }
+    }
+    if (kTrace) {
+        // the last block to come here reports the flags
+        if (tid == 0) { __threadfence(); s_item = atomicAdd(&z->pad, 1u); }
+        __syncthreads();
+        if (s_item == gridDim.x - 1 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
     }
 }
 
-// The group tables in one launch: one block of 1024 threads per group.
-__global__ void __launch_bounds__(1024)
-k_group_tables(int G, const uint32_t* __restrict__ cnt, int64_t* __restrict__ cum, uint32_t* __restrict__ ng_exact,
-               const uint32_t* __restrict__ ng, const int32_t* __restrict__ sorted, uint32_t* __restrict__ grp_off,
-               int32_t* __restrict__ knots, const int32_t* __restrict__ err, const uint32_t* __restrict__ max_n,
-               const unsigned long long* __restrict__ grp_sum_n, unsigned long long* __restrict__ fin_totals,
-               LoadReadback* __restrict__ rb) {
-    grid_dependency_wait();
-    group_knots(G, ng, sorted, grp_off, knots, err, max_n, grp_sum_n, fin_totals, rb);
-    group_mass(cnt, cum, ng_exact);
+template <int SRC, bool STAGE>
+cudaError_t launch_load(const LoadArgs& a, int sms, cudaStream_t st) {
+    const bool priv = a.G <= (SRC == S_TRACE ? kPrivateGroups : kPrivateTickGroups);
+    const size_t counters = priv ? (size_t)a.G * ((SRC == S_TRACE ? kLens : 0) + kTickBins) * 4 : 0;
+    const size_t smem = std::max(counters, sizeof(SortSmem));
+    auto* kernel = priv ? k_load<SRC, true, STAGE> : k_load<SRC, false, STAGE>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    if (e) return e;
+    // a request a thread until the multiprocessors are full
+    const uint32_t blocks = std::max<uint32_t>(1u, std::min<uint32_t>((a.n + kThreads - 1) / kThreads, (uint32_t)sms));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = blocks; cfg.blockDim = kThreads; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
 // The same tables from a length histogram and a sorted sample given by the caller (a whole trace's, of which
 // the context holds a shard): one block of 1024 threads per group.
-__global__ void __launch_bounds__(1024)
-k_tables_imported(const uint32_t* __restrict__ cnt, int64_t* __restrict__ cum, uint32_t* __restrict__ ng_exact,
-                  const int32_t* __restrict__ F_sorted, const uint32_t* __restrict__ F_off, int32_t* __restrict__ knots) {
+__global__ void __launch_bounds__(kThreads)
+k_tables_imported(const uint32_t* __restrict__ cnt, int64_t* __restrict__ cum, const int32_t* __restrict__ F_sorted,
+                  const uint32_t* __restrict__ F_off, int32_t* __restrict__ knots) {
+    __shared__ unsigned long long wm[32];
     const int g = blockIdx.x;
     const uint32_t off = F_off[g], N = F_off[g + 1] - off;
     for (int k = threadIdx.x; k < kNKnots; k += blockDim.x) {
         const uint32_t at = N ? (uint32_t)(((uint64_t)k * (N - 1)) / 256u) : 0u;
         knots[g * kNKnots + k] = (N && DBG_OK(at, N, DBG_K_TABLES, DBG_ELEMENT)) ? F_sorted[off + at] : 0;
     }
-    group_mass(cnt, cum, ng_exact);
-}
-
-int grid_for(uint32_t n, int threads, int sms) {
-    long long b = ((long long)n + threads - 1) / threads;
-    if (b < 1) b = 1;
-    if (b > (long long)sms * 16) b = (long long)sms * 16;
-    return (int)b;
-}
-
-cudaError_t radix_pass(const uint64_t* kin, uint64_t* kout, const uint32_t* pin, uint32_t* pout, uint32_t n,
-                       int shift, uint32_t* counts, cudaStream_t st) {
-    uint32_t blocks = (n + 1023u) / 1024u;
-    if (blocks < 1) blocks = 1;
-    if (blocks > kRadixMaxBlocks) blocks = kRadixMaxBlocks;
-    uint32_t per_block = (n + blocks - 1) / blocks;
-    per_block = (per_block + kRadixThreads - 1) / kRadixThreads * kRadixThreads;
-    uint32_t* totals = counts + (size_t)256u * blocks;       // the caller's buffer has room for these 256 words
-    k_radix_hist<<<blocks, kRadixThreads, 0, st>>>(kin, n, per_block, shift, counts);
-    k_radix_rowscan<<<256, 128, 0, st>>>(counts, blocks, totals);
-    k_radix_scatter<<<blocks, kRadixThreads, 0, st>>>(kin, kout, pin, pout, n, per_block, shift, counts, totals);
-    return cudaGetLastError();
+    group_mass(cnt + (size_t)g * kLens, cum + (size_t)g * (kLens + 1), wm);
 }
 
 }  // namespace
 
 DBG_TRANSLATION_UNIT()
 
-uint32_t load_kernel_launches(uint32_t n, int G) {
-    if (n == 0) return 1;
-    // ingest, cursors, scatter by length; (row scan, scatter) x 4, two histograms; group tables
-    if (G == 1 && n <= (1u << 20)) return 3 + 2 * 4 + 2 + 1;
-    const uint32_t passes = G > 1 ? 5 : 4;                  // radix passes over (group, ticks)
-    return 3 + 3 * passes + 1 + 1;                          // ..., passes, low words, group tables
+cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st) {
+    return a.st_ticks ? launch_load<S_TRACE, true>(a, sms, st) : launch_load<S_TRACE, false>(a, sms, st);
 }
+cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st) { return launch_load<S_TICKS, false>(a, sms, st); }
+cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st) { return launch_load<S_TTFT, false>(a, sms, st); }
 
-cudaError_t run_load(const LoadArgs& a, cudaStream_t st) {
-    const uint32_t n = a.n;
-    const int G = (int)(a.ns * a.nd);
-    cudaError_t e;
-    // radix geometry (as in radix_pass)
-    uint32_t blocks = (n + 1023u) / 1024u;
-    if (blocks < 1) blocks = 1;
-    if (blocks > kRadixMaxBlocks) blocks = kRadixMaxBlocks;
-    uint32_t per_block = (n + blocks - 1) / blocks;
-    per_block = (per_block + kRadixThreads - 1) / kRadixThreads * kRadixThreads;
-    const bool small = G == 1 && n <= (1u << 20);      // fused histograms pay off while launches dominate
-    // everything that must start at zero lies in one block: cnt, grp_sum_n, grp_n, max_n, err, counts A
-    // (zero_bytes covers the tables; the per-pass digit counters of the small path follow them)
-    if ((e = cudaMemsetAsync(a.zero_block, 0, a.zero_bytes + (small ? (size_t)2 * 256u * blocks * 4u : 0u), st))) return e;
-    if (n) {
-        uint32_t* counts_a = a.radix_counts;                                   // small path: pass p uses slice p
-        uint32_t* counts_b = a.radix_counts + (size_t)4 * 256u * kRadixMaxBlocks;  // large path: one scanned buffer
-        // block-private length histograms while they fit two blocks to a multiprocessor (up to six groups)
-        const int hist_groups = (size_t)G * (kMaxPrompt + 1) * 4 <= 100 * 1024 ? G : 0;
-        const size_t hist_bytes = (size_t)hist_groups * (kMaxPrompt + 1) * 4;
-        if ((e = cudaFuncSetAttribute(k_ingest, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024))) return e;
-        k_ingest<<<std::min(grid_for(n, 4 * kIngestThreads, a.sms), 2 * a.sms), kIngestThreads, hist_bytes, st>>>(
-            n, a.prompt, a.outlen, a.ttft, a.sp, a.dp, a.ns, a.nd, a.keys_a, a.cnt,
-            (unsigned long long*)a.grp_sum_n, a.ng, a.max_n, a.err,
-            a.l_tmp, a.n_tmp, small ? counts_a : nullptr, per_block, blocks, hist_groups);
-        // internal request order: by group, then by prompt length
-        k_length_cursors<<<G, 1024, 0, st>>>(a.cnt, a.ng, a.cursors);
-        const size_t cursor_bytes = (size_t)G * (kMaxPrompt + 1) * 4;
-        if (cursor_bytes <= 100 * 1024) {
-            if ((e = cudaFuncSetAttribute(k_scatter_by_length_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024))) return e;
-            const uint32_t slices = (n + kSliceRequests - 1) / kSliceRequests;
-            k_scatter_by_length_slices<<<std::min<uint32_t>(slices, 2u * (uint32_t)a.sms), kSliceThreads, cursor_bytes, st>>>(
-                n, G, a.keys_a, a.l_tmp, a.n_tmp, a.err, a.cursors, a.req, a.inv);
-        } else {
-            k_scatter_by_length<<<grid_for(n, 256, a.sms), 256, 0, st>>>(n, G, a.keys_a, a.l_tmp, a.n_tmp, a.err, a.cursors,
-                                                                         a.req, a.inv);
-        }
-        // sort (group, ticks): four byte passes over the ticks, one over the group id
-        uint64_t *src = a.keys_a, *dst = a.keys_b;
-        const int passes = G > 1 ? 5 : 4;
-        if (small) {
-            uint32_t* totals = a.radix_counts + (size_t)5 * 256u * kRadixMaxBlocks;
-            for (int p = 0; p < passes; ++p) {
-                // The first scatter also counts the second pass's digits (the low bytes of the ticks are spread
-                // evenly, so its adds meet little contention).  High bytes take few values: those passes count
-                // with the block-private histogram kernel instead.
-                const bool last = p == passes - 1, fused_next = p == 0;
-                uint32_t* cur = a.radix_counts + (size_t)p * 256u * blocks;
-                // Ticks below 2^24 (16.7 s) leave the fourth byte zero: the third pass then also writes the sorted
-                // ticks and the kernels of the fourth return at once (a.max_n[1]: the largest tick, from ingestion).
-                const uint32_t* max_key = a.max_n + 1;
-                const uint32_t skip_below = p == 3 ? (1u << 24) : 0u;
-                if (p >= 2 && (e = launch_after(k_radix_hist, blocks, kRadixThreads, 0, st, (const uint64_t*)src, n, per_block,
-                                                8 * p, cur, max_key, skip_below))) return e;
-                if ((e = launch_after(k_radix_rowscan, 256, 128, 0, st, cur, blocks, totals, max_key, skip_below))) return e;
-                if ((e = launch_after(k_radix_scatter, blocks, kRadixThreads, 0, st, src, dst, nullptr, nullptr, n, per_block,
-                                      8 * p, cur, totals, fused_next ? cur + 256u * blocks : nullptr,
-                                      last ? a.sorted : nullptr, max_key, skip_below,
-                                      p == 2 ? a.sorted : nullptr, 1u << 24))) return e;
-                uint64_t* t = src; src = dst; dst = t;
-            }
-        } else {
-            for (int p = 0; p < passes; ++p) {
-                if ((e = radix_pass(src, dst, nullptr, nullptr, n, 8 * p, counts_b, st))) return e;
-                uint64_t* t = src; src = dst; dst = t;
-            }
-            k_low_words<<<grid_for(n, 256, a.sms), 256, 0, st>>>(n, src, a.sorted);
-        }
-    }
-    if ((e = launch_after(k_group_tables, G, 1024, 0, st, G, a.cnt, a.cum_mass, a.ng_exact, a.ng, a.sorted, a.grp_off,
-                          a.knots, a.err, a.max_n, (const unsigned long long*)a.grp_sum_n,
-                          (unsigned long long*)a.fin_totals, a.readback))) return e;
-    return cudaGetLastError();
-}
-
-cudaError_t launch_tables_imported(int G, const uint32_t* cnt, int64_t* cum_mass, uint32_t* ng_exact,
-                                   const int32_t* F_sorted, const uint32_t* F_off, int32_t* knots, cudaStream_t st) {
-    k_tables_imported<<<G, 1024, 0, st>>>(cnt, cum_mass, ng_exact, F_sorted, F_off, knots);
-    return cudaGetLastError();
-}
-
-namespace {
-// Sort keys (group << 32 | ticks) for ticks stored group after group; a negative tick sets the error word.
-__global__ void k_keys_of_grouped_ticks(uint32_t total, const int32_t* __restrict__ ticks, const uint32_t* __restrict__ off,
-                                        int G, uint64_t* __restrict__ keys, int32_t* __restrict__ err) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        int g = 0;
-        while (g + 1 < G && i >= off[g + 1]) ++g;
-        const int32_t t = ticks[i];
-        if (t < 0 && atomicCAS(&err[0], 0, 3) == 0) err[1] = (int32_t)i;
-        keys[i] = ((uint64_t)(uint32_t)g << 32) | (uint32_t)max(t, 0);
-    }
-}
-}  // namespace
-
-cudaError_t sort_grouped_ticks(const int32_t* ticks, const uint32_t* off, int G, uint32_t total, uint64_t* keys_a,
-                               uint64_t* keys_b, uint32_t* counts, int32_t* err, int32_t* out, int sms, cudaStream_t st) {
-    if (total == 0) return cudaSuccess;
-    cudaError_t e;
-    k_keys_of_grouped_ticks<<<grid_for(total, 256, sms), 256, 0, st>>>(total, ticks, off, G, keys_a, err);
-    if ((e = cudaGetLastError())) return e;
-    uint64_t *src = keys_a, *dst = keys_b;
-    const int passes = G > 1 ? 5 : 4;                   // the ticks' four bytes, then the group id
-    for (int p = 0; p < passes; ++p) {
-        if ((e = radix_pass(src, dst, nullptr, nullptr, total, 8 * p, counts, st))) return e;
-        uint64_t* t = src; src = dst; dst = t;
-    }
-    k_low_words<<<grid_for(total, 256, sms), 256, 0, st>>>(total, src, out);
+cudaError_t launch_tables_imported(int G, const uint32_t* cnt, int64_t* cum_mass, const int32_t* F_sorted,
+                                   const uint32_t* F_off, int32_t* knots, cudaStream_t st) {
+    k_tables_imported<<<G, kThreads, 0, st>>>(cnt, cum_mass, F_sorted, F_off, knots);
     return cudaGetLastError();
 }
 
@@ -576,33 +575,24 @@ cudaError_t sort_grouped_ticks(const int32_t* ticks, const uint32_t* off, int G,
 
 
 // -----------------------------------------------------------------------------------------------------
-// Sorting server TTFTs without allocating.  The scratch the radix sort needs (two key buffers, the digit
-// counters, an error word) lives in a fixed array inside the library image instead of in cudaMalloc'd
-// memory.  Every GPU that loads the library carries these bytes until the process exits, and every call
-// on a GPU uses the same bytes.
+// Sorting server TTFTs without allocating.  The scratch the sort needs (the ticks by bin, the bins' counters,
+// and the radix sort's keys and counters, should it be needed) lives in a fixed array inside the library image
+// instead of in cudaMalloc'd memory.  Every GPU that loads the library carries these bytes until the process
+// exits, and every call on a GPU uses the same bytes.
 // -----------------------------------------------------------------------------------------------------
 namespace disco {
 namespace {
 
 constexpr uint32_t kNoAllocMaxN = DISCO_NOALLOC_MAX_N;
 constexpr size_t kNaKeysBytes = (size_t)kNoAllocMaxN * sizeof(uint64_t);
-constexpr size_t kNaCountsBytes = (256u * ((kNoAllocMaxN + 1023u) / 1024u) + 256u) * sizeof(uint32_t);   // as radix_pass sizes its grid, plus the digit totals
-constexpr size_t kNaErrOff = 2 * kNaKeysBytes + kNaCountsBytes;
+constexpr size_t kNaCountsBytes = (256u * ((kNoAllocMaxN + 1023u) / 1024u) + 256u) * sizeof(uint32_t);   // as radix_sort_ticks sizes its grid, plus the digit totals
+// words that must start at zero: the flags and the bins' counters; then the bins' starts and the offsets of the one group
+constexpr size_t kNaZeroOff = 2 * kNaKeysBytes + kNaCountsBytes;
+constexpr size_t kNaZeroBytes = sizeof(LoadZero) + kTickBins * 4;
+constexpr size_t kNaStartOff = kNaZeroOff + kNaZeroBytes;
+constexpr size_t kNaOffOff = kNaStartOff + kTickBins * 4;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaErrOff + 256];
-
-__global__ void k_ttft_keys(uint32_t n, const float* __restrict__ ttft, uint64_t* __restrict__ keys,
-                            int32_t* __restrict__ err) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float t = ttft[i];
-        if (!(t > 0.0f) || !(t <= 2000.0f)) {
-            if (atomicCAS(&err[0], 0, 3) == 0) err[1] = (int32_t)i;
-            keys[i] = 0;
-            continue;
-        }
-        keys[i] = (uint64_t)(uint32_t)__double2ll_rn(__dmul_rn((double)t, 1e6));
-    }
-}
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaOffOff + 256];
 
 std::mutex g_na_mutex;
 unsigned char* g_na_base[64] = {};        // device address of the scratch array, per device ordinal
@@ -640,32 +630,40 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
         base = g_na_base[dev];
         sms = g_na_sms[dev];
     }
-    uint64_t* keys_a = (uint64_t*)base;
-    uint64_t* keys_b = (uint64_t*)(base + kNaKeysBytes);
-    uint32_t* counts = (uint32_t*)(base + 2 * kNaKeysBytes);
-    int32_t* err = (int32_t*)(base + kNaErrOff);
-    // the array still holds the previous call's data: the error word must start at zero; keys and counters
-    // are fully rewritten for the first n entries before they are read
-    if ((e = cudaMemsetAsync(err, 0, 16, st)) != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
+    LoadArgs a = {};
+    a.n = n; a.G = 1; a.ns = a.nd = 1;
+    a.ttft = server_ttft_s;
+    a.z = (LoadZero*)(base + kNaZeroOff); a.tick_cnt = (uint32_t*)(base + kNaZeroOff + sizeof(LoadZero));
+    a.tick_start = (uint32_t*)(base + kNaStartOff);
+    a.binned = (uint32_t*)base; a.sorted = sorted_ticks;
+    // the array still holds the previous call's data: flags and counters must start at zero
+    if ((e = cudaMemsetAsync(a.z, 0, kNaZeroBytes, st)) != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
     // Once a kernel has been queued the shared array is in use: every way out below, failures included, first
     // waits for the stream, so that a caller who retries cannot overlap kernels still writing the array.
     auto fail_after_launch = [&](cudaError_t err_code) {
         cudaStreamSynchronize(st);
         return set_error(DISCO_ECUDA, cudaGetErrorString(err_code));
     };
-    k_ttft_keys<<<grid_for(n, 256, sms), 256, 0, st>>>(n, server_ttft_s, keys_a, err);
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail_after_launch(e);
-    uint64_t *src = keys_a, *dst = keys_b;
-    for (int p = 0; p < 4; ++p) {
-        if ((e = radix_pass(src, dst, nullptr, nullptr, n, 8 * p, counts, st)) != cudaSuccess) return fail_after_launch(e);
-        uint64_t* t = src; src = dst; dst = t;
-    }
-    k_low_words<<<grid_for(n, 256, sms), 256, 0, st>>>(n, src, sorted_ticks);
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail_after_launch(e);
-    int32_t h_err[2] = {0, 0};
-    if ((e = cudaMemcpyAsync(h_err, err, sizeof h_err, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return fail_after_launch(e);
+    if ((e = run_sort_ttft(a, sms, st)) != cudaSuccess) return fail_after_launch(e);
+    int32_t h_err[4] = {0, 0, 0, 0};
+    if ((e = cudaMemcpyAsync(h_err, a.z->err, sizeof h_err, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return fail_after_launch(e);
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
     if (int rc = check_debug_record()) return rc;
     if (h_err[0]) return set_error(DISCO_EINVAL, "server TTFT not finite, not positive or above 2000 s");
+    if (h_err[3] == 2) return set_error(DISCO_ECUDA, "internal error: the blocks of the sort lost each other");
+    if (h_err[3] == 1) {
+        // a sample the bin-wise sort gives up on: radix sort, by way of the caller's output array
+        uint64_t* keys_a = (uint64_t*)base;
+        uint64_t* keys_b = (uint64_t*)(base + kNaKeysBytes);
+        uint32_t* counts = (uint32_t*)(base + 2 * kNaKeysBytes);
+        uint32_t* off = (uint32_t*)(base + kNaOffOff);
+        const uint32_t h_off[2] = {0, n};
+        if ((e = cudaMemcpyAsync(sorted_ticks, a.binned, (size_t)n * 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(off, h_off, sizeof h_off, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+            (e = radix_sort_ticks(sorted_ticks, off, 1, n, keys_a, keys_b, counts, sorted_ticks, sms, st)) != cudaSuccess)
+            return fail_after_launch(e);
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
+        if (int rc = check_debug_record()) return rc;
+    }
     return 0;
 }

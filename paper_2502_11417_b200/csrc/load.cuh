@@ -1,13 +1,14 @@
-// Arguments of the device-side trace ingestion (all pointers are device memory).
+// Trace ingestion and the sort of server-TTFT ticks (load.cu).
 #pragma once
 
 #include "disco_internal.cuh"
 
 namespace disco {
 
-constexpr uint32_t kRadixMaxBlocks = 1024;
+// Ticks fall into 3,200 bins a group: their value below 128, then 128 bins an octave up to 2^31.
+constexpr int kTickBins = 128 + 24 * 128;
 
-struct LoadReadback {            // what the host needs after a load, gathered for one copy
+struct LoadReadback {            // what the host needs after a load; pinned host memory, written by the kernel
     int32_t err[4];
     uint32_t max_n;
     uint32_t ng[kMaxGroups];
@@ -16,36 +17,57 @@ struct LoadReadback {            // what the host needs after a load, gathered f
     uint64_t grp_sum_n[kMaxGroups];
 };
 
+// Words that a load or a sort must find zero, contiguous.
+struct LoadZero {
+    uint64_t grp_sum_n[kMaxGroups];       // output tokens per group
+    uint32_t ng[kMaxGroups];              // requests per group
+    uint32_t max_n;                       // longest output
+    uint32_t barrier, ticket, pad;
+    int32_t err[4];                       // code, request index, window flag, sort flag (1: some bin needs the fallback, 2: a
+                                          // wait between blocks ran out)
+};
+
 struct LoadArgs {
-    uint32_t n, ns, nd;
-    // inputs in the caller's order
+    uint32_t n;
+    int G;
+    uint32_t ns, nd;
+    // inputs in the caller's order: a trace's columns ...
     const int32_t *prompt, *outlen;
     const float* ttft;
     const uint8_t *sp, *dp;               // may be null
-    // scratch
-    uint64_t *keys_a, *keys_b;            // [n] (group << 32 | ticks)
-    uint16_t *l_tmp, *n_tmp;              // [n] each: lengths in the caller's order
-    uint32_t* cursors;                    // [G][4097]: next free place of each (group, prompt length)
-    uint32_t* radix_counts;               // [5][256 * kRadixMaxBlocks], directly after zero_block's tables
-    void* zero_block; size_t zero_bytes;  // cnt, grp_sum_n, ng, max_n, err, contiguous
-    uint32_t* ng_exact;                   // [G] group sizes recounted from the length histogram
-    LoadReadback* readback;               // device copy of what the host reads back
+    // ... or ticks stored group after group (off[g] .. off[g + 1])
+    const int32_t* ticks;
+    const uint32_t* off;
+    // where the kernel leaves a trace it reads from host memory, for its second pass (null: the columns are read twice)
+    uint32_t *st_ticks, *st_ln;
+    uint8_t* st_g;
+    LoadZero* z;
+    uint32_t* cnt;                        // [G][4097] requests per prompt length (zero on entry)
+    uint32_t* tick_cnt;                   // [G][kTickBins] (zero on entry)
+    uint32_t* tick_start;                 // [G][kTickBins]
+    uint32_t* tick_at;                    // [G][kTickBins] cursors, used when the groups' counters do not fit in shared memory
+    uint32_t* binned;                     // [n] ticks bin by bin
     // outputs
     uint4* req;                           // [n] internal order (by group, then by prompt length): see TraceDev
-    uint32_t* inv;                        // [n]: place of each of the caller's requests in the internal order
+    uint32_t* inv;                        // [n] place of each of the caller's requests (one group), or null
     int32_t* sorted;                      // [n] ticks ascending within each group
-    uint32_t* cnt;                        // [G][4097] requests per prompt length
+    uint32_t* len_end;                    // [G][4097]
     int64_t* cum_mass;                    // [G][4098]
-    uint32_t *ng, *grp_off;               // [G], [G+1]
+    uint32_t* grp_off;                    // [G + 1]
     int32_t* knots;                       // [G][257]
-    uint64_t* grp_sum_n;                  // [kMaxGroups] output tokens per group
-    uint32_t* max_n;                      // longest output
-    int32_t* err;                         // [4]: code, request index, window flag
     uint64_t* fin_totals;                 // [2G]: output tokens per group, then requests per group
-    int sms;                              // multiprocessors of the device (grid sizing)
+    LoadReadback* readback;
 };
 
-cudaError_t run_load(const LoadArgs& a, cudaStream_t st);
-uint32_t load_kernel_launches(uint32_t n, int G);   // kernels run_load launches for such a trace
+cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st);          // one kernel; z, cnt and tick_cnt cleared by the caller
+cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st);    // ticks, off, G, n -> sorted
+cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st);     // ttft, n (one group) -> sorted
+
+// The least-significant-digit radix sort, for samples that the kernels above give up on (err[3] = 1: more than 8,192 ticks
+// in one bin, spread over more than 2^18 values).  keys_a, keys_b: n words each; counts: 256 * kRadixMaxBlocks + 256.
+constexpr uint32_t kRadixMaxBlocks = 1024;
+cudaError_t radix_sort_ticks(const int32_t* ticks, const uint32_t* off, int G, uint32_t total, uint64_t* keys_a, uint64_t* keys_b,
+                             uint32_t* counts, int32_t* out, int sms, cudaStream_t st);
+uint32_t radix_sort_launches(int G);
 
 }  // namespace disco

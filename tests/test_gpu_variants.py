@@ -1,5 +1,6 @@
 """Variants of the kernels that the library chooses by sizes and types: parity with the oracle where each one's range
 begins and ends."""
+import numpy as np
 import pytest
 
 from paper_2502_11417_b200 import synth
@@ -23,3 +24,56 @@ def test_handoff_search_by_one_thread_and_by_a_warp(n, buffer_tokens):
         w.devices = devices
         full_parity(w, [synth.policy(b, r_c=20.0, t_m_s=buffer_tokens * 0.05, mig_threshold=th, flags=PACED)
                         for b in (0.3, 1.0) for th in (0.0, 0.1)], select=False, tag=f"search {buffer_tokens}")
+
+
+def _sample(kind, n, rng):
+    if kind == "spread":                       # windows of many bins, up to the largest TTFT
+        return np.exp(rng.uniform(np.log(1e-6), np.log(2000.0), n))
+    if kind == "ties":                         # one value, and another in every sixteenth place
+        return np.where(np.arange(n) % 16 == 3, 0.5, 600.0)
+    if kind == "dense":                        # bins of more than 8,192 ticks spread over few values: counted
+        return np.round(0.25 + 0.004 * rng.random(n), 6)
+    if kind == "often":                        # ... a few of them very often
+        return np.where(rng.random(n) < 0.9, 0.25, 0.25 + 1e-6 * rng.integers(0, 900, n))
+    return 1000.0 + 100.0 * rng.random(n)      # "wide": bins of more than 8,192 ticks and 2^18 values: the radix sort
+
+
+@pytest.mark.parametrize("kind", ["spread", "ties", "dense", "often", "wide"])
+@pytest.mark.parametrize("n", [1, 33, 4096, 4097, 8193, 70001, 260000])
+def test_sorted_samples(kind, n):
+    import torch
+    from paper_2502_11417_b200 import Trace
+    from paper_2502_11417_b200.api import sort_ttft_ticks_noalloc
+    rng = np.random.default_rng(n)
+    x = np.clip(_sample(kind, n, rng), 1e-6, 2000.0).astype(np.float32)
+    ticks = np.rint(x.astype(np.float64) * 1e6).astype(np.int64)
+    want = np.sort(ticks)
+    out = torch.empty(n, dtype=torch.int32, device="cuda")
+    assert (sort_ttft_ticks_noalloc(torch.from_numpy(x).cuda(), out).cpu().numpy() == want).all()
+    # two groups, loaded; then imported as a whole trace's tables would be
+    dp = (np.arange(n) % 3 == 0).astype(np.uint8)
+    devices = [synth.device(500.0, 20.0), synth.device(400.0, 20.0)]
+    tr = Trace().load_trace(np.full(n, 7, np.int32), np.full(n, 5, np.int32), x, None, dp, [synth.server()], devices)
+    groups = [ticks[dp == 0], ticks[dp == 1]]
+    for _ in range(2):
+        for g in range(2):
+            cnt, knots, got = tr.group_tables(g)
+            srt = np.sort(groups[g])
+            assert got.shape == srt.shape and (got == srt).all()
+            if len(srt):
+                assert (knots == srt[np.arange(257, dtype=np.int64) * (len(srt) - 1) // 256]).all() and cnt[7] == len(srt)
+        lengths = np.zeros((2, 4097), dtype=np.int64)
+        lengths[:, 7] = [len(g) for g in groups]
+        tr.set_group_tables(lengths, np.concatenate(groups).astype(np.int32), lengths[:, 7].astype(np.uint64))
+    tr.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 7), (2, 4), (4, 5)])
+@pytest.mark.parametrize("where", ["host", "pinned"])
+def test_groups_whose_counters_fit_a_block_or_do_not(shape, where):
+    import torch
+    w = synth.tiny_workload(91, 5003, n_servers=shape[0], n_devices=shape[1], max_prompt=4096, max_out=60)
+    if where == "pinned":
+        for f in ("prompt_len", "output_len", "server_ttft_s", "server_profile", "device_profile"):
+            setattr(w, f, torch.from_numpy(getattr(w, f)).pin_memory().numpy())
+    full_parity(w, [synth.policy(b) for b in synth.budget_grid(9)], tag=f"{shape} groups")
