@@ -114,6 +114,7 @@ struct disco_ctx {
     std::vector<uint64_t> fin_own;     // this trace's totals, to put back before the next evaluation
     LoadZero* z = nullptr;
     uint32_t *cnt = nullptr, *tick_cnt = nullptr;
+    uint2* windows = nullptr;
     int32_t* err = nullptr;
     size_t zero_bytes = 0;
     HostReadback* rb = nullptr;
@@ -204,18 +205,20 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, bool host_inputs, bool in_pl
         if (has_sp) R(in_sp, N);
         if (has_dp) R(in_dp, N);
     }
-    if (in_place) { R(st_ticks, N * 4); R(st_ln, N * 4); R(st_g, N); }
+    if (in_place) { R(st_ticks, (N + 3) * 4); R(st_ln, (N + 3) * 4); R(st_g, N + 3); }      // (whole vectors of four)
     R(binned, N * 4); R(req, N * 16); R(sorted, N * 4);
     if (G == 1) R(inv, N * 4);
     R(tick_start, (size_t)2 * G * kTickBins * 4); R(len_end, (size_t)G * (kMaxPrompt + 1) * 4);
     // one block for everything a load clears: the flags and sums, the two histograms
     const size_t tick_bytes = (size_t)G * kTickBins * 4, cnt_bytes = ((size_t)G * (kMaxPrompt + 1) * 4 + 15) / 16 * 16;
-    R(zero, sizeof(LoadZero) + tick_bytes + cnt_bytes);
+    const size_t win_bytes = (size_t)sort_windows(n, G) * 8;
+    R(zero, sizeof(LoadZero) + tick_bytes + cnt_bytes + win_bytes);
     c->z = (LoadZero*)c->zero.p;
     c->tick_cnt = (uint32_t*)(c->z + 1);
     c->cnt = (uint32_t*)((char*)c->tick_cnt + tick_bytes);
     c->err = c->z->err;
-    c->zero_bytes = sizeof(LoadZero) + tick_bytes + cnt_bytes;
+    c->windows = (uint2*)((char*)c->cnt + cnt_bytes);
+    c->zero_bytes = sizeof(LoadZero) + tick_bytes + cnt_bytes + win_bytes;
     R(cum_mass, (size_t)G * (kMaxPrompt + 2) * 8);
     R(grp_off, (kMaxGroups + 1) * 4); R(knots, (size_t)G * kNKnots * 4);
     R(d_gc, (size_t)G * sizeof(GroupConst));
@@ -327,6 +330,8 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     a.req = c->req.as<uint4>(); a.inv = c->G == 1 ? c->inv.as<uint32_t>() : nullptr; a.sorted = c->sorted.as<int32_t>();
     a.len_end = c->len_end.as<uint32_t>(); a.cum_mass = c->cum_mass.as<int64_t>(); a.grp_off = c->grp_off.as<uint32_t>();
     a.knots = c->knots.as<int32_t>(); a.fin_totals = c->fin_totals.as<uint64_t>();
+    a.windows = c->windows;
+    a.rounds = (n + 3000000u - 1) / 3000000u;                       // (3 million records and ticks take 60 MB)
     a.readback = c->rb;                                             // pinned host memory, written by the kernel
     // the profile table is read from pageable memory: this copy returns once it has been staged
     const bool same_profiles = c->gc_dev_at == c->d_gc.p && c->gc_dev.size() == c->gc.size() &&
@@ -972,9 +977,10 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     const size_t T1 = (size_t)std::max<uint64_t>(total, 1);
     const size_t tick_bytes = (size_t)G * kTickBins * 4;
     if ((e = c->F_sorted_imp.reserve(T1 * 4)) != cudaSuccess || (e = c->F_off_imp.reserve((size_t)(kMaxGroups + 1) * 4)) != cudaSuccess ||
-        (e = c->sort_in.reserve(2 * T1 * 4)) != cudaSuccess)
+        (e = c->sort_in.reserve(2 * ((T1 + 3) / 4 * 4) * 4 + (size_t)sort_windows((uint32_t)total, G) * 8)) != cudaSuccess)
         return fail_cuda(e, "device allocation for the tables");
-    int32_t* in = c->sort_in.as<int32_t>();
+    int32_t* in = c->sort_in.as<int32_t>();                           // the ticks, the same by bin, the windows
+    const size_t T4 = (T1 + 3) / 4 * 4, win_bytes = (size_t)sort_windows((uint32_t)total, G) * 8;
     CU(cudaMemsetAsync(c->z, 0, sizeof(LoadZero) + tick_bytes, st));
     if (total) CU(cudaMemcpyAsync(in, ticks, (size_t)total * 4, cudaMemcpyDefault, st));
     CU(cudaMemcpyAsync(c->F_off_imp.p, off.data(), (size_t)(G + 1) * 4, cudaMemcpyHostToDevice, st));
@@ -982,7 +988,8 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     LoadArgs a = {};
     a.n = (uint32_t)total; a.G = G; a.ticks = in; a.off = c->F_off_imp.as<uint32_t>();
     a.z = c->z; a.tick_cnt = c->tick_cnt; a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)G * kTickBins;
-    a.binned = (uint32_t*)in + T1; a.sorted = c->F_sorted_imp.as<int32_t>();
+    a.binned = (uint32_t*)in + T4; a.windows = (uint2*)(in + 2 * T4); a.rounds = 1; a.sorted = c->F_sorted_imp.as<int32_t>();
+    CU(cudaMemsetAsync(a.windows, 0, win_bytes, st));
     if (total) { CU(run_sort_ticks(a, c->sms, st)); g_launches += 1; }
     CU(launch_tables_imported(G, c->cnt, c->cum_mass.as<int64_t>(), c->F_sorted_imp.as<int32_t>(), c->F_off_imp.as<uint32_t>(),
                               c->knots.as<int32_t>(), st));

@@ -34,10 +34,9 @@ constexpr uint32_t kWindow = 4096;        // a window starts with the first bin 
 constexpr uint32_t kSortCap = 8192;       // ticks sorted at a time
 constexpr uint32_t kCounters = 16384;     // values counted at a time
 constexpr uint32_t kMaxRange = 1u << 18;  // values a dense bin may span
-constexpr uint32_t kMaxCount = 1u << 24;  // ticks a dense bin may hold
+constexpr uint32_t kMaxCount = 1u << 22;  // ticks a dense bin may hold
 constexpr int kPrivateGroups = 7;         // groups whose counters fit in shared memory (29 KB each)
 constexpr int kPrivateTickGroups = 16;    // the same, counters of tick bins alone
-constexpr int kUnroll = 4;                // requests a thread has in flight
 
 enum Source { S_TRACE, S_TICKS, S_TTFT };
 
@@ -50,11 +49,11 @@ __device__ __forceinline__ uint32_t tick_bin_edge(int b) {     // smallest ticks
 
 struct SortSmem {
     uint32_t a[kSortCap], b[kSortCap];                 // ticks of a window, twice; or kCounters counters
-    uint16_t wcnt[kThreads / 32][256];                 // keys of each digit per warp; or the list of frequent values
+    uint16_t wcnt[kThreads / 32][256];                 // keys of each digit per warp (radix sort)
     uint32_t dig[256];
     uint32_t wtot[32];
     uint32_t lo, hi, n_list;
-    int bin0, bin1;
+    uint32_t bin[kTickBins];                           // of a window's bins: first place | count << 16; or the frequent values
 };
 static_assert(kCounters == 2 * kSortCap, "the counters lie over the two key arrays");
 
@@ -76,73 +75,118 @@ __device__ __forceinline__ void grid_barrier(LoadZero* z, uint32_t times) {
     __syncthreads();
 }
 
-// A request of the trace (or a tick of a sample) as the two passes see it.
+// Four neighbouring requests of the trace (or ticks of a sample) as the two passes see them.
 struct Item { uint32_t g, S, l, o; bool in; };
 
-// First pass: reads and checks item i.
-template <int SRC>
-__device__ __forceinline__ Item check_item(const LoadArgs& a, uint32_t i, const uint32_t* s_off) {
-    Item x = {0u, 0u, 1u, 1u, i < a.n};
-    if (!x.in) return x;
-    int bad = 0;
+// (LAST: read for the last time, so that the lines need not stay in L2)
+template <class T4, bool LAST, class T>
+__device__ __forceinline__ void load4(const T* p, uint32_t i0, uint32_t n, bool wide, T (&v)[4], T fill) {
+    if (wide && i0 + 4u <= n) {
+        const T4 x = LAST ? __ldcs(reinterpret_cast<const T4*>(p + i0)) : *reinterpret_cast<const T4*>(p + i0);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i0 + u < n ? p[i0 + u] : fill;
+    }
+}
+
+// Reads the items i0 .. i0 + 3, and in the first pass checks them.  wide: the columns are aligned for vector loads.
+// AGAIN: for counting; it will be read once more.
+template <int SRC, bool STAGE, bool CHECK, bool AGAIN = false>
+__device__ __forceinline__ void read_items(const LoadArgs& a, uint32_t i0, bool wide, const uint32_t* s_off, Item (&x)[4]) {
+    if (STAGE && !CHECK) {
+        uint32_t ln[4], S[4];
+        uint8_t g[4];
+        load4<uint4, !CHECK && !AGAIN>(a.st_ln, i0, a.n, true, ln, 0u);
+        load4<uint4, !CHECK && !AGAIN>(a.st_ticks, i0, a.n, true, S, 0u);
+        load4<uchar4, !CHECK && !AGAIN>(a.st_g, i0, a.n, true, g, (uint8_t)0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = Item{g[u], S[u], ln[u] & 0xFFFFu, ln[u] >> 16, i0 + u < a.n};
+        return;
+    }
     if (SRC == S_TICKS) {
-        while ((int)x.g + 1 < a.G && i >= s_off[x.g + 1]) ++x.g;
-        const int32_t t = a.ticks[i];
-        if (t < 0) bad = 3;
-        x.S = (uint32_t)t;
-    } else {
-        const float t = a.ttft[i];
-        uint32_t s = 0, d = 0;
-        int32_t l = 1, o = 1;
-        if (SRC == S_TRACE) { l = a.prompt[i]; o = a.outlen[i]; s = a.sp ? a.sp[i] : 0u; d = a.dp ? a.dp[i] : 0u; }
-        if (l < 1 || l > kMaxPrompt) bad = 1;
-        else if (o < 1 || o > kMaxOutput) bad = 2;
-        else if (!(t > 0.0f) || !(t <= 2000.0f)) bad = 3;      // NaN fails both comparisons
-        else if (SRC == S_TRACE && (s >= a.ns || d >= a.nd)) bad = 4;
-        // ticks = nearest integer (ties to even) of the fp64 product, as a host llrint would give
-        x.S = (uint32_t)__double2ll_rn(__dmul_rn((double)t, 1e6));
-        x.g = s * a.nd + d; x.l = (uint32_t)l; x.o = (uint32_t)o;
-        if (SRC == S_TTFT) x.g = 0;
-    }
-    if (bad) {
-        if (atomicCAS(&a.z->err[0], 0, bad) == 0) a.z->err[1] = (int32_t)i;
-        x.in = false;
-    }
-    return x;
-}
-
-// Second pass: the same item, known to be good.
-template <int SRC, bool STAGE>
-__device__ __forceinline__ Item read_item(const LoadArgs& a, uint32_t i, const uint32_t* s_off) {
-    Item x = {0u, 0u, 1u, 1u, i < a.n};
-    if (!x.in) return x;
-    if (STAGE) {
-        const uint32_t ln = a.st_ln[i];
-        x.S = a.st_ticks[i]; x.l = ln & 0xFFFFu; x.o = ln >> 16; x.g = a.st_g[i];
-    } else if (SRC == S_TICKS) {
-        while ((int)x.g + 1 < a.G && i >= s_off[x.g + 1]) ++x.g;
-        x.S = (uint32_t)a.ticks[i];
-    } else {
-        x.S = (uint32_t)__double2ll_rn(__dmul_rn((double)a.ttft[i], 1e6));
-        if (SRC == S_TRACE) {
-            x.l = (uint32_t)a.prompt[i]; x.o = (uint32_t)a.outlen[i];
-            x.g = (a.sp ? a.sp[i] : 0u) * a.nd + (a.dp ? a.dp[i] : 0u);
+        int32_t t[4];
+        load4<int4, !CHECK>(a.ticks, i0, a.n, wide, t, 0);
+        uint32_t g = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            x[u] = Item{0u, (uint32_t)t[u], 1u, 1u, i0 + u < a.n};
+            while ((int)g + 1 < a.G && i0 + u >= s_off[g + 1]) ++g;
+            x[u].g = g;
+            if (CHECK && t[u] < 0) {
+                if (atomicCAS(&a.z->err[0], 0, 3) == 0) a.z->err[1] = (int32_t)(i0 + u);
+                x[u].in = false;
+            }
         }
+        return;
     }
-    return x;
+    float t[4];
+    int32_t l[4] = {1, 1, 1, 1}, o[4] = {1, 1, 1, 1};
+    uint8_t sp[4] = {0, 0, 0, 0}, dp[4] = {0, 0, 0, 0};
+    constexpr bool kLast = !CHECK && !AGAIN;
+    load4<float4, kLast>(a.ttft, i0, a.n, wide, t, 1.0f);
+    if (SRC == S_TRACE) {
+        load4<int4, kLast>(a.prompt, i0, a.n, wide, l, 1);
+        if (!AGAIN) load4<int4, kLast>(a.outlen, i0, a.n, wide, o, 1);
+        if (a.sp) load4<uchar4, kLast>(a.sp, i0, a.n, wide, sp, (uint8_t)0);
+        if (a.dp) load4<uchar4, kLast>(a.dp, i0, a.n, wide, dp, (uint8_t)0);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        bool in = i0 + u < a.n;
+        if (CHECK && in) {
+            int bad = 0;
+            if (l[u] < 1 || l[u] > kMaxPrompt) bad = 1;
+            else if (o[u] < 1 || o[u] > kMaxOutput) bad = 2;
+            else if (!(t[u] > 0.0f) || !(t[u] <= 2000.0f)) bad = 3;      // NaN fails both comparisons
+            else if (SRC == S_TRACE && (sp[u] >= a.ns || dp[u] >= a.nd)) bad = 4;
+            if (bad) {
+                if (atomicCAS(&a.z->err[0], 0, bad) == 0) a.z->err[1] = (int32_t)(i0 + u);
+                in = false;
+            }
+        }
+        // ticks = nearest integer (ties to even) of the fp64 product, as a host llrint would give
+        const uint32_t S = (uint32_t)__double2ll_rn(__dmul_rn((double)t[u], 1e6));
+        x[u] = Item{SRC == S_TRACE ? (uint32_t)sp[u] * a.nd + dp[u] : 0u, S, (uint32_t)l[u], (uint32_t)o[u], in};
+    }
 }
 
-// Exclusive prefix sums of L <= 5 * kThreads counters, `base` added; emit(k, count, start).  All threads call.
+// Exclusive prefix sums over L counters (16-byte aligned) by the whole block: a warp takes a run of them, sums it up, and
+// goes through it again with the sum of the runs in front (read from L2 both times, four a lane).  emit(k, counts, starts):
+// the counters k .. k + 3, those from L on empty.
 template <class E>
-__device__ __forceinline__ void scan_counts(const uint32_t* cnt, int L, uint32_t base, uint32_t* wtot, E emit) {
-    constexpr int kPer = 5;
-    const int k0 = (int)threadIdx.x * kPer;
-    uint32_t c[kPer], sum = 0;
+__device__ __forceinline__ void scan_counts(const uint32_t* cnt, int L, uint32_t* wtot, E emit) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int per = ((L + 31) / 32 + 127) / 128 * 128, k0 = w * per + lane * 4, k1 = min(L, (w + 1) * per);
+    auto four = [&](int k) {
+        if (k + 4 <= k1) return __ldcg(reinterpret_cast<const uint4*>(cnt + k));
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (k < k1) v.x = __ldcg(&cnt[k]);
+        if (k + 1 < k1) v.y = __ldcg(&cnt[k + 1]);
+        if (k + 2 < k1) v.z = __ldcg(&cnt[k + 2]);
+        return v;
+    };
+    uint32_t sum = 0;
+#pragma unroll 2
+    for (int k = k0; k < k1; k += 128) { const uint4 v = four(k); sum += v.x + v.y + v.z + v.w; }
+    sum = __reduce_add_sync(FULL, sum);
+    if (lane == 0) wtot[w] = sum;
+    __syncthreads();
+    uint32_t run = __reduce_add_sync(FULL, lane < w ? wtot[lane] : 0u);
+#pragma unroll 1
+    for (int k = w * per; k < k1; k += 128) {
+        const uint4 c = four(k + lane * 4);
+        const uint32_t own = c.x + c.y + c.z + c.w;
+        uint32_t v = own;
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) { c[k] = k0 + k < L ? __ldcg(&cnt[k0 + k]) : 0u; sum += c[k]; }
-    uint32_t run = base + block_inclusive_scan(sum, wtot, (uint32_t*)nullptr) - sum;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) { if (k0 + k < L) emit(k0 + k, c[k], run); run += c[k]; }
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t up = __shfl_up_sync(FULL, v, off);
+            if (lane >= off) v += up;
+        }
+        const uint32_t at = run + v - own;
+        if (k + lane * 4 < k1) emit(k + lane * 4, c, make_uint4(at, at + c.x, at + c.x + c.y, at + c.x + c.y + c.z));
+        run += __shfl_sync(FULL, v, 31);
+    }
     __syncthreads();
 }
 
@@ -161,9 +205,90 @@ __device__ __forceinline__ void group_mass(const uint32_t* cnt, int64_t* cum, un
     __syncthreads();
 }
 
-// Sorts `count` <= kSortCap ticks from src (all of them in [lo, lo + 2^bits)) into out: stable counting passes of at most
-// eight bits in shared memory, a warp's 256 keys at a time with the ranks from ballots.
-__device__ __forceinline__ void sort_window(SortSmem& sm, const uint32_t* src, uint32_t count, uint32_t lo, int bits, int32_t* out) {
+// Sorts the `count` <= kSortCap ticks of the bins [b0, b1] of a group from src into out: every bin has as many cells (or
+// twice as many) as ticks, evenly over its values, so that a cell holds a tick or so whatever the distribution; the ticks
+// are counted by cell, placed, and those that share a cell put in order by insertion.  Returns false, with nothing
+// written, if more than kCellCap different ticks may share a cell.
+constexpr uint32_t kCells = 8192, kCellCap = 64;
+
+__device__ __forceinline__ bool sort_window(SortSmem& sm, const uint32_t* src, uint32_t count, const uint32_t* bin_start,
+                                            const uint32_t* bin_count, int b0, int b1, int32_t* out) {
+    const int tid = threadIdx.x;
+    constexpr int kPer = kSortCap / kThreads, kCellsPer = kCells / kThreads;
+    uint32_t* cell = sm.b;                                             // counts, then starts
+    const uint32_t k0 = __ldcg(&bin_start[b0]), f = count <= kCells / 2 ? 1u : 0u, cells = count << f;
+    for (uint32_t i = tid; i < (cells + 7u) / 8u * 8u; i += kThreads) cell[i] = 0;
+    for (int b = b0 + tid; b <= b1; b += kThreads) {
+        const uint32_t c = __ldcg(&bin_count[b]);
+        sm.bin[b - b0] = (__ldcg(&bin_start[b]) - k0) | c << 16;       // (an empty bin's is not used)
+    }
+    if (tid == 0) sm.n_list = 0;
+    uint32_t key[kPer], at[kPer];                                      // at: cell | rank in it << 16
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const uint32_t i = k * kThreads + tid;
+        if (i < count) key[k] = __ldcg(&src[i]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if ((uint32_t)k * kThreads + tid >= count) continue;
+        const int b = tick_bin(key[k]);
+        if (!DBG_OK(b - b0, b1 - b0 + 1, DBG_K_RADIX, DBG_BIN)) { at[k] = 0; continue; }
+        const uint32_t sc = sm.bin[b - b0], w = b < 128 ? 0u : (uint32_t)(b >> 7) - 1u, in = key[k] - tick_bin_edge(b);
+        const uint32_t sh = min(w, 16u);                               // (a bin spans 2^w values; 16 leading bits of the place in it)
+        uint32_t c = ((sc & 0xFFFFu) << f) + (((in >> (w - sh)) * ((sc >> 16) << f)) >> sh);
+        if (!DBG_OK(c, cells, DBG_K_RADIX, DBG_BIN)) c = 0;
+        at[k] = c | atomicAdd(&cell[c], 1u) << 16;
+    }
+    __syncthreads();
+    // the cells' starts; a thread's eight neighbouring cells (as vectors: single words would meet in four banks)
+    static_assert(kCellsPer == 8, "two vectors");
+    uint4* cell4 = reinterpret_cast<uint4*>(cell) + tid * 2;
+    uint4 u = make_uint4(0u, 0u, 0u, 0u), v = u;
+    if (tid * 8u < cells) { u = cell4[0]; v = cell4[1]; }              // (those beyond `cells` are zero)
+    const uint32_t sum = u.x + u.y + u.z + u.w + v.x + v.y + v.z + v.w;
+    uint32_t run = block_inclusive_scan(sum, sm.wtot, (uint32_t*)nullptr) - sum;
+    if (tid * 8u < cells) {
+        uint32_t t;
+        t = u.x; u.x = run; run += t; t = u.y; u.y = run; run += t; t = u.z; u.z = run; run += t; t = u.w; u.w = run; run += t;
+        t = v.x; v.x = run; run += t; t = v.y; v.y = run; run += t; t = v.z; v.z = run; run += t; t = v.w; v.w = run; run += t;
+        cell4[0] = u; cell4[1] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if ((uint32_t)k * kThreads + tid >= count) continue;
+        const uint32_t p = cell[at[k] & 0xFFFFu] + (at[k] >> 16);
+        if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) sm.a[p] = key[k];
+    }
+    __syncthreads();
+    // a thread every 1,024th cell
+    for (uint32_t x = tid; x < cells; x += kThreads) {
+        const uint32_t from = cell[x], to = x + 1u < cells ? cell[x + 1u] : count;
+        if (to - from < 2u) continue;
+        if (to - from > 8u) {
+            // a cell of a bin with at least as many cells as values holds one value
+            const int b = tick_bin(sm.a[from]);
+            if (b < 128 || 1u << ((b >> 7) - 1) <= (sm.bin[b - b0] >> 16) << f) continue;
+            if (to - from > kCellCap) { sm.n_list = 1; continue; }
+        }
+        for (uint32_t y = from + 1u; y < to; ++y) {
+            const uint32_t v = sm.a[y];
+            uint32_t p = y;
+            while (p > from && sm.a[p - 1u] > v) { sm.a[p] = sm.a[p - 1u]; --p; }
+            sm.a[p] = v;
+        }
+    }
+    __syncthreads();
+    if (sm.n_list) return false;
+    for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)sm.a[i];
+    return true;
+}
+
+// The same whatever the ticks (all of them in [lo, lo + 2^bits)): stable counting passes of at most eight bits, a warp's 256
+// keys at a time with the ranks from ballots.  Four to six times slower.
+__device__ __noinline__ void sort_window_radix(SortSmem& sm, const uint32_t* src, uint32_t count, uint32_t lo, int bits, int32_t* out) {
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     if (bits == 0) {
         for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)lo;
@@ -226,7 +351,7 @@ __device__ __forceinline__ void sort_window(SortSmem& sm, const uint32_t* src, u
 
 // Sorts a dense bin by counting its values.  Returns false where that would take too long.
 __device__ __forceinline__ bool sort_dense(SortSmem& sm, const uint32_t* src, uint32_t count, int32_t* out) {
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) { sm.lo = 0xFFFFFFFFu; sm.hi = 0u; }
     __syncthreads();
     uint32_t mn = 0xFFFFFFFFu, mx = 0u;
@@ -240,50 +365,45 @@ __device__ __forceinline__ bool sort_dense(SortSmem& sm, const uint32_t* src, ui
         return true;
     }
     if (range > kMaxRange || count > kMaxCount) return false;
-    uint32_t* n_of = sm.a;                                            // kCounters of them
-    uint16_t* list = &sm.wcnt[0][0];
-    constexpr uint32_t kOften = 4096;                                 // such values are written by the whole block
+    uint32_t* at = sm.a;                                              // kCounters of them: counts, then places
+    uint32_t* often = sm.bin;                                         // values that the whole block writes: value, place, count
+    constexpr uint32_t kOften = 4096;
+    static_assert(3 * (kMaxCount / kOften) <= kTickBins, "room for the frequent values");
     uint32_t done = 0;
     for (uint32_t r0 = 0; r0 < range; r0 += kCounters) {
-        for (uint32_t i = tid; i < kCounters; i += kThreads) n_of[i] = 0;
+        // a thread's neighbouring values, as few as the range needs
+        const uint32_t here = min(range - r0, kCounters), per = (here + kThreads - 1) / kThreads;
+        for (uint32_t i = tid; i < per * kThreads; i += kThreads) at[i] = 0;
         if (tid == 0) sm.n_list = 0;
         __syncthreads();
+#pragma unroll 4
         for (uint32_t i = tid; i < count; i += kThreads) {
             const uint32_t v = __ldcg(&src[i]) - lo - r0;
-            if (v < kCounters) atomicAdd(&n_of[v], 1u);
+            if (v < here) atomicAdd(&at[v], 1u);
         }
         __syncthreads();
-        // a thread's sixteen values, then where they start
-        constexpr uint32_t kPer = kCounters / kThreads;
         uint32_t sum = 0, total;
-        for (uint32_t k = 0; k < kPer; ++k) sum += n_of[tid * kPer + k];
+        for (uint32_t k = 0; k < per; ++k) sum += at[tid * per + k];
         uint32_t run = done + block_inclusive_scan(sum, sm.wtot, &total) - sum;
-        // a warp writes its threads' values one thread after another, 32 copies at a time
-        for (int t = 0; t < 32; ++t) {
-            uint32_t at = __shfl_sync(FULL, run, t);
-            if (__shfl_sync(FULL, sum, t) == 0u) continue;
-            for (uint32_t k = 0; k < kPer; ++k) {
-                const uint32_t v = (uint32_t)(w * 32 + t) * kPer + k, c = n_of[v];
-                if (c > kOften) {
-                    if (lane == 0) { const uint32_t e = atomicAdd(&sm.n_list, 1u); if (DBG_OK(e, 8192, DBG_K_RADIX, DBG_SLOT)) list[e] = (uint16_t)v; }
-                } else {
-                    for (uint32_t j = lane; j < c; j += 32) out[at + j] = (int32_t)(lo + r0 + v);
-                }
-                at += c;
+        for (uint32_t k = 0; k < per; ++k) {
+            const uint32_t v = tid * per + k, c = at[v];
+            at[v] = run;
+            if (c > kOften) {
+                const uint32_t e = atomicAdd(&sm.n_list, 1u);
+                if (DBG_OK(e, kMaxCount / kOften, DBG_K_RADIX, DBG_SLOT)) { often[3 * e] = v; often[3 * e + 1] = run; often[3 * e + 2] = c; at[v] = 0xFFFFFFFFu; }
             }
+            run += c;
         }
         __syncthreads();
-        for (uint32_t e = 0; e < sm.n_list; ++e) {                    // (at most kMaxCount / kOften of them)
-            const uint32_t v = list[e];
-            // where it starts: the counters in front of it
-            uint32_t part = 0;
-            for (uint32_t k = tid; k < v; k += kThreads) part += n_of[k];
-            uint32_t before;
-            block_inclusive_scan(part, sm.wtot, &before);
-            const uint32_t c = n_of[v];
-            for (uint32_t j = tid; j < c; j += kThreads) out[done + before + j] = (int32_t)(lo + r0 + v);
-            __syncthreads();
+#pragma unroll 4
+        for (uint32_t i = tid; i < count; i += kThreads) {
+            const uint32_t t = __ldcg(&src[i]), v = t - lo - r0;
+            if (v >= here || *(volatile uint32_t*)&at[v] == 0xFFFFFFFFu) continue;
+            const uint32_t p = atomicAdd(&at[v], 1u);                 // equal ticks in any order
+            if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) out[p] = (int32_t)t;
         }
+        for (uint32_t e = 0; e < sm.n_list; ++e)
+            for (uint32_t j = tid; j < often[3 * e + 2]; j += kThreads) out[often[3 * e + 1] + j] = (int32_t)(lo + r0 + often[3 * e]);
         done += total;
         __syncthreads();
     }
@@ -302,36 +422,48 @@ k_load(const __grid_constant__ LoadArgs a) {
     __shared__ uint32_t s_max, s_item;
     const int G = a.G, tid = threadIdx.x, lane = tid & 31;
     LoadZero* z = a.z;
-    uint32_t* s_len = (uint32_t*)smem_raw;                             // [G][kLens]
-    uint32_t* s_tick = s_len + (kTrace ? G * kLens : 0);               // [G][kTickBins]
+    uint32_t* s_tick = (uint32_t*)smem_raw;                            // [G][kTickBins]
+    uint32_t* s_len = s_tick + G * kTickBins;                          // [G][kLens]
     uint32_t waits = 0;
 
+    // the block's counters join the global ones; what it finds there is where its own requests go within the bucket
+    auto join = [&](uint32_t* mine, uint32_t* all, int count) {
+#pragma unroll 1
+        for (int i0 = tid; i0 < count; i0 += 4 * kThreads) {
+            uint32_t c[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { const int i = i0 + u * kThreads; c[u] = i < count ? mine[i] : 0u; }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) if (c[u]) c[u] = atomicAdd(&all[i0 + u * kThreads], c[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { const int i = i0 + u * kThreads; if (i < count) mine[i] = c[u]; }
+        }
+    };
+
     // ---- 1. count
-    if (PRIV) for (int i = tid; i < (kTrace ? G * kLens : 0) + G * kTickBins; i += kThreads) s_len[i] = 0;
+    if (PRIV) for (int i = tid; i < (kTrace ? G * kLens : 0) + G * kTickBins; i += kThreads) s_tick[i] = 0;
     if (SRC == S_TICKS) for (int g = tid; g <= G; g += kThreads) s_off[g] = a.off[g];
     for (int g = tid; g < G; g += kThreads) s_sum[g] = 0;
     if (tid == 0) s_max = 0;
     __syncthreads();
-    const uint32_t stride = gridDim.x * kThreads, i_first = blockIdx.x * kThreads + tid;
+    // a thread takes four neighbouring requests at a time, as vectors where the columns are aligned
+    const auto aligned = [](const void* p, uintptr_t k) { return ((uintptr_t)p & (k - 1)) == 0; };
+    const bool wide = SRC == S_TICKS ? aligned(a.ticks, 16)
+                                     : aligned(a.ttft, 16) && (!kTrace || (aligned(a.prompt, 16) && aligned(a.outlen, 16) && aligned(a.sp, 4) && aligned(a.dp, 4)));
+    const uint32_t stride = gridDim.x * kThreads * 4u, i_first = (blockIdx.x * kThreads + tid) * 4u;
+    uint32_t i_next = i_first;                                         // (second pass)
     uint32_t tok[kPrivateGroups] = {};                                 // output tokens per group
     uint32_t longest = 0;
-    for (uint32_t i0 = i_first; i0 < a.n; i0 += kUnroll * stride) {
-        Item x[kUnroll];
+#pragma unroll 1
+    for (uint32_t i0 = i_first; i0 < a.n; i0 += stride) {
+        Item x[4];
+        read_items<SRC, STAGE, true>(a, i0, wide, s_off, x);
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            const uint32_t i = i0 + u * stride;
-            x[u] = check_item<SRC>(a, i, s_off);
-        }
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+        for (int u = 0; u < 4; ++u) {
             const Item& y = x[u];
             if (!y.in || !DBG_OK(y.g, G, DBG_K_INGEST, DBG_GROUP) || !DBG_OK(y.l, kLens, DBG_K_INGEST, DBG_TABLE)) continue;
             const int tb = tick_bin(y.S);
             if (!DBG_OK(tb, kTickBins, DBG_K_INGEST, DBG_BIN)) continue;
-            if (STAGE) {
-                const uint32_t i = i0 + u * stride;
-                a.st_ticks[i] = y.S; a.st_ln[i] = y.l | y.o << 16; a.st_g[i] = (uint8_t)y.g;
-            }
             if (PRIV) {
                 if (kTrace) atomicAdd(&s_len[y.g * kLens + y.l], 1u);
                 atomicAdd(&s_tick[y.g * kTickBins + tb], 1u);
@@ -346,6 +478,11 @@ k_load(const __grid_constant__ LoadArgs a) {
                     for (int g = 0; g < kPrivateGroups; ++g) tok[g] += (int)y.g == g ? y.o : 0u;    // (at most 2^21 requests a thread)
                 }
             }
+        }
+        if (STAGE) {                                                   // (the staging arrays hold whole vectors)
+            *reinterpret_cast<uint4*>(a.st_ticks + i0) = make_uint4(x[0].S, x[1].S, x[2].S, x[3].S);
+            *reinterpret_cast<uint4*>(a.st_ln + i0) = make_uint4(x[0].l | x[0].o << 16, x[1].l | x[1].o << 16, x[2].l | x[2].o << 16, x[3].l | x[3].o << 16);
+            *reinterpret_cast<uchar4*>(a.st_g + i0) = make_uchar4((uint8_t)x[0].g, (uint8_t)x[1].g, (uint8_t)x[2].g, (uint8_t)x[3].g);
         }
     }
     if (kTrace) {
@@ -367,19 +504,7 @@ k_load(const __grid_constant__ LoadArgs a) {
         for (int g = tid; g < G; g += kThreads) if (s_sum[g]) atomicAdd((unsigned long long*)&z->grp_sum_n[g], s_sum[g]);
         if (tid == 0 && s_max) atomicMax(&z->max_n, s_max);
     }
-    // the block's counters join the global ones; what it finds there is where its own requests go within the bucket
     if (PRIV) {
-        auto join = [&](uint32_t* mine, uint32_t* all, int count) {
-            for (int i0 = tid; i0 < count; i0 += 4 * kThreads) {
-                uint32_t c[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) { const int i = i0 + u * kThreads; c[u] = i < count ? mine[i] : 0u; }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) if (c[u]) c[u] = atomicAdd(&all[i0 + u * kThreads], c[u]);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) { const int i = i0 + u * kThreads; if (i < count) mine[i] = c[u]; }
-            }
-        };
         if (kTrace) join(s_len, a.cnt, G * kLens);
         join(s_tick, a.tick_cnt, G * kTickBins);
     }
@@ -387,33 +512,52 @@ k_load(const __grid_constant__ LoadArgs a) {
 
     // ---- 2. place
     const int32_t bad = __ldcg(&z->err[0]);
-    // group sizes: the sum of their tick counts
-    uint32_t base = 0;
-    for (int g = 0; g < G; ++g) {
-        if (SRC != S_TICKS && tid == 0) s_off[g] = base;
-        const bool mine = (int)(blockIdx.x % (uint32_t)G) == g || gridDim.x < (uint32_t)G;    // the blocks that write the group's tables
-        uint32_t in_group = 0;
-        auto ticks_at = [&](int k, uint32_t c, uint32_t start) {
-            const size_t at = (size_t)g * kTickBins + k;
-            if (PRIV) s_tick[at] += start;
-            if (mine) { a.tick_start[at] = start; if (!PRIV && blockIdx.x < (uint32_t)G) a.tick_at[at] = start; }
-            if (k == kTickBins - 1) s_item = start + c - base;
-        };
-        scan_counts(a.tick_cnt + (size_t)g * kTickBins, kTickBins, base, s_wtot, ticks_at);
-        in_group = s_item;
-        if (kTrace) {
-            scan_counts(a.cnt + (size_t)g * kLens, kLens, base, s_wtot, [&](int k, uint32_t c, uint32_t start) {
-                const size_t at = (size_t)g * kLens + k;
-                if (PRIV) { s_len[at] += start; if (mine) a.len_end[at] = start + c; }
-                else if (mine && blockIdx.x < (uint32_t)G) a.len_end[at] = start;      // the cursor, which ends up there
-            });
-            if (mine) group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
+    // where every bucket starts: the groups one after another, so one running sum over all groups' counters each; the
+    // blocks share the writing of the tables
+    const bool writer = (uint32_t)(tid >> 5) % gridDim.x == blockIdx.x;
+    const bool cursors = !PRIV || a.rounds > 1;                        // places are handed out by global cursors
+    scan_counts(a.tick_cnt, G * kTickBins, s_wtot, [&](int k, const uint4& c, const uint4& start) {
+        // (kTickBins is a multiple of four: the four bins belong to one group)
+        if (PRIV) {
+            uint4& mine = *reinterpret_cast<uint4*>(s_tick + k);
+            mine = make_uint4(mine.x + start.x, mine.y + start.y, mine.z + start.z, mine.w + start.w);
         }
-        base += in_group;
-        __syncthreads();
+        if (SRC != S_TICKS) {
+            if (k % kTickBins == 0) s_off[k / kTickBins] = start.x;
+            if (k == G * kTickBins - 4) s_off[G] = start.w + c.w;
+        }
+        if (writer) {
+            *reinterpret_cast<uint4*>(a.tick_start + k) = start;
+            if (cursors) *reinterpret_cast<uint4*>(a.tick_at + k) = start;
+        }
+    });
+    if (kTrace) {
+        scan_counts(a.cnt, G * kLens, s_wtot, [&](int k, const uint4& c, const uint4& start) {
+            const uint32_t cs[4] = {c.x, c.y, c.z, c.w}, st[4] = {start.x, start.y, start.z, start.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (k + u >= G * kLens) break;
+                if (PRIV) s_len[k + u] += st[u];
+                if (writer) a.len_end[k + u] = cursors ? st[u] : st[u] + cs[u];    // (a cursor ends up where its bucket does)
+            }
+        });
+        for (int g = 0; g < G; ++g)
+            if ((uint32_t)(G - 1 - g) % gridDim.x == gridDim.x - 1 - blockIdx.x)
+                group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
     }
-    if (SRC != S_TICKS && tid == 0) s_off[G] = base;
-    __syncthreads();
+    // the windows' first and last bins: a thread a bin of those this block writes
+    if (writer) {
+        const int L = G * kTickBins, w = tid >> 5, per = ((L + 31) / 32 + 127) / 128 * 128;
+#pragma unroll 1
+        for (int k = w * per + lane; k < min(L, (w + 1) * per); k += 32) {
+            if (__ldcg(&a.tick_cnt[k]) == 0u) continue;
+            const int g = k / kTickBins;
+            uint32_t win = (a.tick_start[k] - s_off[g]) / kWindow;      // (written by this warp)
+            for (int h = 0; h < g; ++h) win += (s_off[h + 1] - s_off[h] + kWindow - 1) / kWindow;
+            atomicMax(&a.windows[win].x, 0xFFFFFFFFu - (uint32_t)k);
+            atomicMax(&a.windows[win].y, (uint32_t)k + 1u);
+        }
+    }
     if (kTrace && blockIdx.x == 0) {
         for (int g = tid; g < G; g += kThreads) {
             const uint32_t N = s_off[g + 1] - s_off[g];
@@ -431,73 +575,107 @@ k_load(const __grid_constant__ LoadArgs a) {
         if (kTrace && blockIdx.x == 0 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
         return;
     }
-    if (!PRIV) grid_barrier(z, ++waits);               // the cursors are complete
-    for (uint32_t i0 = i_first; i0 < a.n; i0 += kUnroll * stride) {
-        Item x[kUnroll];
+    if (cursors) grid_barrier(z, ++waits);             // the cursors are complete
+    auto place = [&](uint32_t i_end) {
+#pragma unroll 1
+        for (; i_next < i_end; i_next += stride) {
+            const uint32_t i0 = i_next;
+            Item x[4];
+            read_items<SRC, STAGE, false>(a, i0, wide, s_off, x);
+            uint32_t at[4] = {0, 0, 0, 0}, tp[4];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            const uint32_t i = i0 + u * stride;
-            x[u] = read_item<SRC, STAGE>(a, i, s_off);
-        }
+            for (int u = 0; u < 4; ++u) {
+                const Item& y = x[u];
+                if (!y.in || !DBG_OK(y.g, G, DBG_K_GATHER, DBG_GROUP) || !DBG_OK(y.l, kLens, DBG_K_GATHER, DBG_TABLE)) { x[u].in = false; continue; }
+                if (kTrace) { const uint32_t lb = y.g * kLens + y.l; at[u] = atomicAdd(PRIV ? &s_len[lb] : &a.len_end[lb], 1u); }
+                const uint32_t tb = y.g * kTickBins + (uint32_t)tick_bin(y.S);
+                tp[u] = atomicAdd(PRIV ? &s_tick[tb] : &a.tick_at[tb], 1u);
+            }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            const Item& y = x[u];
-            const uint32_t i = i0 + u * stride;
-            if (!y.in || !DBG_OK(y.g, G, DBG_K_GATHER, DBG_GROUP) || !DBG_OK(y.l, kLens, DBG_K_GATHER, DBG_TABLE)) continue;
-            const uint32_t tb = y.g * kTickBins + (uint32_t)tick_bin(y.S);
-            const uint32_t tp = atomicAdd(PRIV ? &s_tick[tb] : &a.tick_at[tb], 1u);
-            if (DBG_OK(tp, a.n, DBG_K_GATHER, DBG_ELEMENT)) a.binned[tp] = y.S;
-            if (kTrace) {
-                const uint32_t lb = y.g * kLens + y.l;
-                const uint32_t at = atomicAdd(PRIV ? &s_len[lb] : &a.len_end[lb], 1u);
-                if (!DBG_OK(at, a.n, DBG_K_GATHER, DBG_REQUEST)) continue;
-                a.req[at] = make_uint4(y.S, y.l | y.o << 16, i, 0u);
-                if (a.inv) a.inv[i] = at;
+            for (int u = 0; u < 4; ++u) {
+                const Item& y = x[u];
+                if (!y.in) continue;
+                if (DBG_OK(tp[u], a.n, DBG_K_GATHER, DBG_ELEMENT)) a.binned[tp[u]] = y.S;
+                if (kTrace && DBG_OK(at[u], a.n, DBG_K_GATHER, DBG_REQUEST)) a.req[at[u]] = make_uint4(y.S, y.l | y.o << 16, i0 + u, 0u);
+            }
+            if (kTrace && a.inv) {
+                if (i0 + 4u <= a.n) *reinterpret_cast<uint4*>(a.inv + i0) = make_uint4(at[0], at[1], at[2], at[3]);
+                else for (uint32_t u = 0; i0 + u < a.n; ++u) a.inv[i0 + u] = at[u];
             }
         }
+    };
+    if (kTrace && PRIV && a.rounds > 1) {
+        // a round of the trace at a time: its requests are counted once more, and the blocks take their shares of each bucket
+        // and bin from the global cursors
+        const uint32_t per_round = (a.n + a.rounds - 1) / a.rounds;
+#pragma unroll 1
+        for (uint32_t r = 0; r < a.rounds; ++r) {
+            const uint32_t i_end = r + 1 == a.rounds ? a.n : (r + 1) * per_round;
+            for (int i = tid; i < G * (kTickBins + kLens); i += kThreads) s_tick[i] = 0;
+            __syncthreads();
+#pragma unroll 1
+            for (uint32_t i0 = i_next; i0 < i_end; i0 += stride) {
+                Item x[4];
+                read_items<SRC, STAGE, false, true>(a, i0, wide, s_off, x);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (x[u].in && DBG_OK(x[u].g, G, DBG_K_GATHER, DBG_GROUP) && DBG_OK(x[u].l, kLens, DBG_K_GATHER, DBG_TABLE)) {
+                        atomicAdd(&s_len[x[u].g * kLens + x[u].l], 1u);
+                        atomicAdd(&s_tick[x[u].g * kTickBins + tick_bin(x[u].S)], 1u);
+                    }
+            }
+            __syncthreads();
+            join(s_len, a.len_end, G * kLens);
+            join(s_tick, a.tick_at, G * kTickBins);
+            __syncthreads();
+            place(i_end);
+            __syncthreads();
+        }
+    } else {
+        place(a.n);
     }
     grid_barrier(z, ++waits);
 
     // ---- 3. sort
     SortSmem& sm = *reinterpret_cast<SortSmem*>(smem_raw);
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_item = atomicAdd(&z->ticket, 1u);
-        __syncthreads();
-        uint32_t win = s_item;
-        int g = 0;
-        for (; g < G; ++g) {
-            const uint32_t here = (s_off[g + 1] - s_off[g] + kWindow - 1) / kWindow;
-            if (win < here) break;
-            win -= here;
-        }
-        if (g == G) break;
-        const uint32_t first = s_off[g], N = s_off[g + 1] - first;
-        const uint32_t* start = a.tick_start + (size_t)g * kTickBins;
-        // the window's bins: those that hold ticks and start in [first + win * kWindow, ... + kWindow)
-        if (tid == 0) { sm.bin0 = kTickBins; sm.bin1 = -1; }
-        __syncthreads();
-        const uint32_t x0 = first + win * kWindow, x1 = x0 + kWindow;
-        const uint32_t* counts = a.tick_cnt + (size_t)g * kTickBins;
-        int b_min = kTickBins, b_max = -1;
-        for (int b = tid; b < kTickBins; b += kThreads) {
-            const uint32_t s = __ldcg(&start[b]), c = __ldcg(&counts[b]);
-            if (c && s >= x0 && s < x1) { b_min = min(b_min, b); b_max = max(b_max, b); }
-        }
-        if (b_max >= 0) { atomicMin(&sm.bin0, b_min); atomicMax(&sm.bin1, b_max); }
-        __syncthreads();
-        const int b0 = sm.bin0, b1 = sm.bin1;
-        if (b1 < 0) continue;                                          // (inside a large bin)
-        const uint32_t k0 = __ldcg(&start[b0]), k2 = __ldcg(&start[b1]), k1 = k2 + __ldcg(&counts[b1]);
-        const uint32_t lo = tick_bin_edge(b0);
-        auto bits_of = [](uint32_t range) { return range <= 1u ? 0 : 32 - __clz((int)(range - 1u)); };
-        if (k1 - k0 <= kSortCap) {
-            sort_window(sm, a.binned + k0, k1 - k0, lo, bits_of(tick_bin_edge(b1 + 1) - lo), a.sorted + k0);
-        } else {                                                       // the last bin is a large one: the others first
-            if (k2 > k0) {
-                sort_window(sm, a.binned + k0, k2 - k0, lo, bits_of(tick_bin_edge(b1) - lo), a.sorted + k0);
-                __syncthreads();
+    __shared__ uint32_t s_win[5][32];                 // of the block's next windows: first tick, last bin's first tick, end, bins
+    uint32_t n_win = 0;
+    for (int g = 0; g < G; ++g) n_win += (s_off[g + 1] - s_off[g] + kWindow - 1) / kWindow;
+#pragma unroll 1
+    for (uint32_t j = 0;; ++j) {
+        const uint32_t win = blockIdx.x + j * gridDim.x;
+        if (win >= n_win) break;
+        if ((j & 31u) == 0u) {
+            __syncthreads();
+            if (tid < 32) {
+                const uint32_t mine = blockIdx.x + (j + tid) * gridDim.x;
+                uint2 bins = make_uint2(0u, 0u);
+                if (mine < n_win) bins = __ldcg(&a.windows[mine]);
+                if (bins.y) {
+                    const uint32_t first_bin = 0xFFFFFFFFu - bins.x, last_bin = bins.y - 1u;
+                    const uint32_t k2 = __ldcg(&a.tick_start[last_bin]);
+                    s_win[0][tid] = __ldcg(&a.tick_start[first_bin]); s_win[1][tid] = k2;
+                    s_win[2][tid] = k2 + __ldcg(&a.tick_cnt[last_bin]); s_win[3][tid] = first_bin; s_win[4][tid] = last_bin;
+                } else s_win[0][tid] = s_win[2][tid] = 0u;
             }
+        }
+        __syncthreads();
+        const uint32_t k0 = s_win[0][j & 31u], k2 = s_win[1][j & 31u], k1 = s_win[2][j & 31u];
+        if (k0 >= k1) continue;                                        // (inside a large bin)
+        const int g = (int)s_win[3][j & 31u] / kTickBins, b0 = (int)s_win[3][j & 31u] - g * kTickBins, b1 = (int)s_win[4][j & 31u] - g * kTickBins;
+        const uint32_t first = s_off[g], N = s_off[g + 1] - first, lo = tick_bin_edge(b0);
+        auto bits_of = [](uint32_t range) { return range <= 1u ? 0 : 32 - __clz((int)(range - 1u)); };
+        const uint32_t *starts = a.tick_start + (size_t)g * kTickBins, *counts = a.tick_cnt + (size_t)g * kTickBins;
+        // up to kSortCap ticks; otherwise the last bin is a large one: the others first
+        const bool large = k1 - k0 > kSortCap;
+        const uint32_t to = large ? k2 : k1;
+        const int last = large ? b1 - 1 : b1;
+        if (to > k0 && !sort_window(sm, a.binned + k0, to - k0, starts, counts, b0, last, a.sorted + k0)) {
+            __syncthreads();
+            sort_window_radix(sm, a.binned + k0, to - k0, lo, bits_of(tick_bin_edge(last + 1) - lo), a.sorted + k0);
+        }
+        if (large) {
+            __syncthreads();
             if (!sort_dense(sm, a.binned + k2, k1 - k2, a.sorted + k2) && tid == 0) atomicExch(&z->err[3], 1);
         }
         __syncthreads();
@@ -515,7 +693,7 @@ k_load(const __grid_constant__ LoadArgs a) {
     }
     if (kTrace) {
         // the last block to come here reports the flags
-        if (tid == 0) { __threadfence(); s_item = atomicAdd(&z->pad, 1u); }
+        if (tid == 0) { __threadfence(); s_item = atomicAdd(&z->done, 1u); }
         __syncthreads();
         if (s_item == gridDim.x - 1 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
     }
@@ -526,11 +704,13 @@ cudaError_t launch_load(const LoadArgs& a, int sms, cudaStream_t st) {
     const bool priv = a.G <= (SRC == S_TRACE ? kPrivateGroups : kPrivateTickGroups);
     const size_t counters = priv ? (size_t)a.G * ((SRC == S_TRACE ? kLens : 0) + kTickBins) * 4 : 0;
     const size_t smem = std::max(counters, sizeof(SortSmem));
+    static_assert(kTickBins % 4 == 0 && sizeof(LoadZero) % 16 == 0, "vector loads of the counters");
     auto* kernel = priv ? k_load<SRC, true, STAGE> : k_load<SRC, false, STAGE>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     if (e) return e;
-    // a request a thread until the multiprocessors are full
-    const uint32_t blocks = std::max<uint32_t>(1u, std::min<uint32_t>((a.n + kThreads - 1) / kThreads, (uint32_t)sms));
+    // four requests a thread (and about a window a block) until the multiprocessors are full
+    const uint32_t per_block = 4u * kThreads;
+    const uint32_t blocks = std::max<uint32_t>(1u, std::min<uint32_t>((a.n + per_block - 1) / per_block, (uint32_t)sms));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = blocks; cfg.blockDim = kThreads; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -588,7 +768,7 @@ constexpr size_t kNaKeysBytes = (size_t)kNoAllocMaxN * sizeof(uint64_t);
 constexpr size_t kNaCountsBytes = (256u * ((kNoAllocMaxN + 1023u) / 1024u) + 256u) * sizeof(uint32_t);   // as radix_sort_ticks sizes its grid, plus the digit totals
 // words that must start at zero: the flags and the bins' counters; then the bins' starts and the offsets of the one group
 constexpr size_t kNaZeroOff = 2 * kNaKeysBytes + kNaCountsBytes;
-constexpr size_t kNaZeroBytes = sizeof(LoadZero) + kTickBins * 4;
+constexpr size_t kNaZeroBytes = (sizeof(LoadZero) + kTickBins * 4 + sort_windows(kNoAllocMaxN, 1) * 8 + 15) / 16 * 16;
 constexpr size_t kNaStartOff = kNaZeroOff + kNaZeroBytes;
 constexpr size_t kNaOffOff = kNaStartOff + kTickBins * 4;
 
@@ -634,6 +814,7 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
     a.n = n; a.G = 1; a.ns = a.nd = 1;
     a.ttft = server_ttft_s;
     a.z = (LoadZero*)(base + kNaZeroOff); a.tick_cnt = (uint32_t*)(base + kNaZeroOff + sizeof(LoadZero));
+    a.windows = (uint2*)(a.tick_cnt + kTickBins); a.rounds = 1;
     a.tick_start = (uint32_t*)(base + kNaStartOff);
     a.binned = (uint32_t*)base; a.sorted = sorted_ticks;
     // the array still holds the previous call's data: flags and counters must start at zero

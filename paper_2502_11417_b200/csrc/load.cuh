@@ -22,10 +22,12 @@ struct LoadZero {
     uint64_t grp_sum_n[kMaxGroups];       // output tokens per group
     uint32_t ng[kMaxGroups];              // requests per group
     uint32_t max_n;                       // longest output
-    uint32_t barrier, ticket, pad;
+    uint32_t barrier, done, pad;
     int32_t err[4];                       // code, request index, window flag, sort flag (1: some bin needs the fallback, 2: a
                                           // wait between blocks ran out)
 };
+
+constexpr uint32_t sort_windows(uint32_t n, int G) { return n / 4096u + (uint32_t)G; }
 
 struct LoadArgs {
     uint32_t n;
@@ -41,11 +43,15 @@ struct LoadArgs {
     // where the kernel leaves a trace it reads from host memory, for its second pass (null: the columns are read twice)
     uint32_t *st_ticks, *st_ln;
     uint8_t* st_g;
+    // Parts of the trace placed one after another (1: all at once), for traces whose records do not fit in L2: the blocks'
+    // shares of all buckets are open at once, and what leaves L2 in parts is written twice.
+    uint32_t rounds;
     LoadZero* z;
     uint32_t* cnt;                        // [G][4097] requests per prompt length (zero on entry)
     uint32_t* tick_cnt;                   // [G][kTickBins] (zero on entry)
     uint32_t* tick_start;                 // [G][kTickBins]
     uint32_t* tick_at;                    // [G][kTickBins] cursors, used when the groups' counters do not fit in shared memory
+    uint2* windows;                       // [n / 4096 + G] of the sort: first and last bin (zero on entry)
     uint32_t* binned;                     // [n] ticks bin by bin
     // outputs
     uint4* req;                           // [n] internal order (by group, then by prompt length): see TraceDev
@@ -59,7 +65,7 @@ struct LoadArgs {
     LoadReadback* readback;
 };
 
-cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st);          // one kernel; z, cnt and tick_cnt cleared by the caller
+cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st);          // one kernel; z, cnt, tick_cnt and windows cleared by the caller
 cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st);    // ticks, off, G, n -> sorted
 cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st);     // ttft, n (one group) -> sorted
 
