@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import Dict, Optional, Sequence
 
 import numpy as np
@@ -140,11 +141,20 @@ def _check(rc: int, allow=()):
     return rc
 
 
-def _stream_ptr(stream) -> Optional[int]:
-    if stream is None:
+_torch = None
+
+
+def _t():
+    """torch, imported at the first use of a GPU."""
+    global _torch
+    if _torch is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        _torch = torch
+    return _torch
+
+
+def _stream_ptr(stream) -> Optional[int]:
+    return (_t().cuda.current_stream() if stream is None else stream).cuda_stream
 
 
 _cuda_ok = None
@@ -153,8 +163,7 @@ _cuda_ok = None
 def _require_cuda():
     global _cuda_ok
     if _cuda_ok is None:
-        import torch
-        _cuda_ok = bool(torch.cuda.is_available())
+        _cuda_ok = bool(_t().cuda.is_available())
     if not _cuda_ok:
         raise DiscoError(ECUDA, "no CUDA device: libdisco has no CPU path")
 
@@ -172,22 +181,24 @@ def stats_view(stats):
 
 
 def _torch_dtype(name):
-    import torch
-    return getattr(torch, name)
+    return getattr(_t(), name)
+
+
+_SERVER, _DEVICE = struct.Struct("4f"), struct.Struct("7f")
 
 
 def server_array(servers: Sequence[Dict[str, float]]):
     arr = (ServerProfile * len(servers))()
     for k, s in enumerate(servers):
-        arr[k] = ServerProfile(s["tbt_s"], s["jitter"], s["c_prefill"], s["c_decode"])
+        _SERVER.pack_into(arr, 16 * k, s["tbt_s"], s["jitter"], s["c_prefill"], s["c_decode"])
     return arr
 
 
 def device_array(devices: Sequence[Dict[str, float]]):
     arr = (DeviceProfile * len(devices))()
     for k, d in enumerate(devices):
-        arr[k] = DeviceProfile(d["prefill_tps"], d["ttft_intercept_s"], d["decode_tps"], d["jitter"],
-                               d["c_prefill"], d["c_decode"], d["lam"])
+        _DEVICE.pack_into(arr, 28 * k, d["prefill_tps"], d["ttft_intercept_s"], d["decode_tps"], d["jitter"],
+                          d["c_prefill"], d["c_decode"], d["lam"])
     return arr
 
 
@@ -203,7 +214,7 @@ def select_policy(stats, cost_cap: float, tbt_slo_s: float):
     """disco_select_policy over a (PolicyStats * P) array in host memory (the records of reduce_stats, or
     merged ones).  Returns (status, index): status 0, or EINFEASIBLE with the cheapest policy's index."""
     best = C.c_int32(-1)
-    rc = _check(lib().disco_select_policy(C.cast(stats, C.c_void_p), len(stats), cost_cap, tbt_slo_s, C.byref(best)),
+    rc = _check(lib().disco_select_policy(C.addressof(stats), len(stats), cost_cap, tbt_slo_s, C.byref(best)),
                 allow=(EINFEASIBLE,))
     return rc, best.value
 
@@ -254,36 +265,34 @@ class Trace:
         all of the same kind.  Reloading reuses the context's device memory.  first_index: position of these
         arrays' first request in the whole trace when they are a shard of it.  staged_copy: host arrays are copied
         by the copy engine even when they are page-locked (instead of being read in place by the ingestion kernel)."""
-        import torch
+        torch = _t()
         _require_cuda()
-        arrs = [prompt_len, output_len, server_ttft_s, server_profile, device_profile]
         on_dev = isinstance(prompt_len, torch.Tensor) and prompt_len.is_cuda
-        want = [("int32", np.int32), ("int32", np.int32), ("float32", np.float32), ("uint8", np.uint8),
-                ("uint8", np.uint8)]
         ptrs, keep = [], []
-        for a, (tname, npdt) in zip(arrs, want):
+        for a, want, npdt in ((prompt_len, torch.int32, np.int32), (output_len, torch.int32, np.int32),
+                              (server_ttft_s, torch.float32, np.float32), (server_profile, torch.uint8, np.uint8),
+                              (device_profile, torch.uint8, np.uint8)):
             if a is None:
                 ptrs.append(None)
-                continue
-            if isinstance(a, torch.Tensor):
+            elif isinstance(a, torch.Tensor):
                 if a.is_cuda != on_dev:
                     raise ValueError("all trace arrays must live on the same side")
-                t = a.contiguous()
-                if t.dtype != _torch_dtype(tname):
-                    raise TypeError(f"expected {tname}, got {t.dtype}")
-                keep.append(t)
-                ptrs.append(t.data_ptr())
+                if a.dtype != want:
+                    raise TypeError(f"expected {want}, got {a.dtype}")
+                if not a.is_contiguous():
+                    a = a.contiguous()
+                    keep.append(a)
+                ptrs.append(a.data_ptr())
             else:
                 if on_dev:
                     raise ValueError("all trace arrays must live on the same side")
                 x = np.ascontiguousarray(a, dtype=npdt)
                 keep.append(x)
-                ptrs.append(x.ctypes.data)
+                ptrs.append(x.__array_interface__["data"][0])
         n = int(len(prompt_len))
         sv, dv = server_array(servers), device_array(devices)
-        desc = TraceDesc(n, ptrs[0], ptrs[1], ptrs[2], ptrs[3], ptrs[4], C.cast(sv, C.c_void_p), len(servers),
-                         C.cast(dv, C.c_void_p), len(devices), 1 if on_dev else (2 if staged_copy else 0),
-                         int(first_index))
+        desc = TraceDesc(n, *ptrs, C.addressof(sv), len(servers), C.addressof(dv), len(devices),
+                         1 if on_dev else (2 if staged_copy else 0), int(first_index))
         _check(lib().disco_load_trace(C.byref(self._h), C.byref(desc), _stream_ptr(stream)))
         self.n = n
         self.n_groups = len(servers) * len(devices)
@@ -307,25 +316,31 @@ class Trace:
         P = len(arr)
         po = None
         if out is not None:
-            vals = {}
+            shape = (P, self.n)
+            vals = []
             for f, dt in PAIR_FIELDS:
                 t = out.get(f)
                 if t is not None:
-                    if not t.is_cuda or t.dtype != _torch_dtype(dt) or tuple(t.shape) != (P, self.n) \
-                            or not t.is_contiguous():
+                    if not t.is_cuda or t.dtype != _torch_dtype(dt) or t.shape != shape or not t.is_contiguous():
                         raise ValueError(f"output '{f}' must be a contiguous CUDA tensor [P, n] of {dt}")
-                    vals[f] = t.data_ptr()
-            po = PairOut(*[vals.get(f) for f, _ in PAIR_FIELDS])
-        _check(lib().disco_eval_policies(self._h, C.cast(arr, C.c_void_p), P, seed,
-                                         C.byref(po) if po is not None else None, _stream_ptr(stream)))
+                    t = t.data_ptr()
+                vals.append(t)
+            po = C.byref(PairOut(*vals))
+        _check(lib().disco_eval_policies(self._h, C.addressof(arr), P, seed, po, _stream_ptr(stream)))
         self.P = P
         self._keep = (arr, out)
         return self
 
     # -- disco_reduce_stats --------------------------------------------------------------------------------
     def reduce_stats(self, stream=None):
-        stats = (PolicyStats * self.P)()
-        _check(lib().disco_reduce_stats(self._h, C.cast(stats, C.c_void_p), _stream_ptr(stream)))
+        if self.P < 64:
+            stats = (PolicyStats * self.P)()
+        else:
+            # page-locked memory, which the kernel writes straight into: no copy, no fresh pages to fault in
+            mem = _t().empty(self.P * C.sizeof(PolicyStats), dtype=_t().uint8, pin_memory=True)
+            stats = (PolicyStats * self.P).from_address(mem.data_ptr())
+            stats._memory = mem                          # lives as long as the records
+        _check(lib().disco_reduce_stats(self._h, C.addressof(stats), _stream_ptr(stream)))
         return stats
 
     # -- disco_select_policy -------------------------------------------------------------------------------

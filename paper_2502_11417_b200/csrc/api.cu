@@ -5,12 +5,14 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
 
 #include "disco_internal.cuh"
 #include "load.cuh"
+#include "pack.cuh"
 
 using namespace disco;
 
@@ -42,7 +44,11 @@ struct DevBuf {
     template <class T> T* as() const { return (T*)p; }
 };
 
-struct DevBufView { size_t off = 0; };
+// Places several arrays in one buffer, each on a 256-byte boundary.
+struct Layout {
+    size_t bytes = 0;
+    size_t take(size_t n) { const size_t at = bytes; bytes += (n + 255) / 256 * 256; return at; }
+};
 
 int64_t ticks_of_seconds(float s) { return llrint((double)s * 1e6); }
 int64_t ticks_of_rate(float per_s) { return llrint(1e6 / (double)per_s); }
@@ -53,6 +59,19 @@ using HostReadback = LoadReadback;   // pinned host mirror of the load's read-ba
 
 namespace disco {
 int set_error(int code, const char* msg) { return fail(code, msg); }
+
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+    // (kernel, device, size) that have been allowed: a few dozen at most
+    struct Allowed { const void* kernel; int device; size_t bytes; };
+    static thread_local std::vector<Allowed> seen;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e) return e;
+    for (const Allowed& x : seen) if (x.kernel == kernel && x.device == dev && x.bytes >= bytes) return cudaSuccess;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes))) return e;
+    seen.push_back({kernel, dev, bytes});
+    return cudaSuccess;
+}
 
 #ifdef DISCO_DEBUG
 namespace {
@@ -95,13 +114,16 @@ struct disco_ctx {
     std::vector<GroupConst> gc;
     std::vector<GroupConst> gc_dev;   // what d_gc holds (a reload with the same profiles skips the copy)
     const void* gc_dev_at = nullptr;
-    // trace
-    DevBuf in_prompt, in_out, in_ttft, in_sp, in_dp;      // staging of host inputs
-    DevBuf st_ticks, st_ln, st_g;                         // the trace as the ingestion leaves it when it reads host memory
-    DevBuf binned, tick_start, len_end, inv, req, sorted;
+    struct View { void* p = nullptr; template <class T> T* as() const { return (T*)p; } };
+    // trace: one buffer for everything a load writes, and what a load needs in between
+    DevBuf trace_mem, d_gc;
+    View req, inv, sorted, len_end, tick_start, binned, zero, cum_mass, grp_off, knots;   // `zero`: what a load must clear
+    View in_prompt, in_out, in_ttft, in_sp, in_dp;        // copies of host inputs
+    View packed;                                          // ... or the same packed (pack.cuh)
+    View st_ticks, st_ln, st_g;                           // ... or what the ingestion leaves when it reads host memory in place
+    View fin_totals;                   // [2G] u64: output tokens and requests per group that the accumulators cover
+    std::unique_ptr<Packer> packer;
     DevBuf keys_a, keys_b, radix_counts, sort_in;         // radix sort (fallback) and the sort of imported ticks
-    DevBuf zero, cum_mass, grp_off, knots, d_gc;          // `zero`: what a load must clear, contiguous
-    DevBuf fin_totals;                 // [2G] u64: output tokens and requests per group that the accumulators cover
     uint64_t first_index = 0;          // index of request 0 in the whole trace (hash key base)
     int sms = 0;                       // multiprocessors of the context's device
     // F as Algorithms 1-3 read it: the trace's own sorted ticks, or a whole trace's given by the caller
@@ -122,15 +144,14 @@ struct disco_ctx {
     uint32_t P = 0;
     bool evaluated = false, reduced = false;
     std::vector<PolicyConst> pol;
-    DevBuf d_prep, d_accum, d_stats, d_tables, d_grid, d_left;
-    struct View { void* p = nullptr; template <class T> T* as() const { return (T*)p; } };
-    View d_acc, d_hist_ttft, d_hist_tbt, d_work;       // regions of d_accum (cleared by one memset)
-    View d_pol, d_classes, d_tab, d_slabs, d_chunks, d_pair_chunks;    // regions of d_tables (filled by one copy)
-    DevBuf rec_hand, rec_u32[6], rec_win[3];
+    DevBuf eval_mem;             // one buffer for everything an evaluation writes
+    View d_prep, d_accum, d_stats, d_tables, d_grid, d_left;
+    View d_acc, d_hist_ttft, d_hist_tbt, d_work;          // regions of d_accum; d_work: the counters in front of d_grid
+    View rec_hand, rec_u32[6], rec_win[3];
     void* stage = nullptr;       // pinned staging for the small host->device tables
     size_t stage_cap = 0;
     cudaEvent_t stage_free = nullptr;
-    int32_t* sel_host = nullptr; // pinned [2]
+    int32_t* sel_host = nullptr; // [2], in the pinned block of rb
     void* stats_host = nullptr;  // pinned mirror of the statistics
     size_t stats_host_cap = 0;
     bool timing = false;         // record events around the play-out and pair kernels
@@ -139,15 +160,10 @@ struct disco_ctx {
     bool timing_valid = false;
 
     ~disco_ctx() {
-        DevBuf* all[] = {&in_prompt, &in_out, &in_ttft, &in_sp, &in_dp, &st_ticks, &st_ln, &st_g, &binned, &tick_start, &len_end, &inv,
-                         &req, &sorted, &keys_a, &keys_b, &radix_counts, &sort_in, &zero, &cum_mass, &grp_off, &knots, &d_gc, &d_prep, &d_accum, &d_stats, &d_tables, &d_grid, &rec_hand,
-                         &fin_totals, &F_sorted_imp, &F_off_imp, &d_left};
+        DevBuf* all[] = {&trace_mem, &d_gc, &keys_a, &keys_b, &radix_counts, &sort_in, &F_sorted_imp, &F_off_imp, &eval_mem};
         for (DevBuf* b : all) b->release();
-        for (auto& b : rec_u32) b.release();
-        for (auto& b : rec_win) b.release();
         if (rb) cudaFreeHost(rb);
         if (stage) cudaFreeHost(stage);
-        if (sel_host) cudaFreeHost(sel_host);
         if (stats_host) cudaFreeHost(stats_host);
         if (stage_free) cudaEventDestroy(stage_free);
         for (auto& e : ev) if (e) cudaEventDestroy(e);
@@ -195,36 +211,45 @@ int check_profiles(const disco_trace_desc_t* d, std::vector<GroupConst>* out) {
     return 0;
 }
 
-cudaError_t reserve_trace(disco_ctx* c, uint32_t n, bool host_inputs, bool in_place, bool has_sp, bool has_dp) {
-    cudaError_t e;
-    const size_t N = n ? n : 1;
+// How a load's inputs reach the ingestion kernel.
+enum Inputs { IN_DEVICE, IN_COPIED, IN_PLACE, IN_PACKED };
+
+cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool has_dp) {
+    const size_t N = n ? n : 1, N4 = N + 3;
     const int G = c->G;
-#define R(buf, bytes) if ((e = c->buf.reserve(bytes)) != cudaSuccess) return e
-    if (host_inputs) {
-        R(in_prompt, N * 4); R(in_out, N * 4); R(in_ttft, N * 4);
-        if (has_sp) R(in_sp, N);
-        if (has_dp) R(in_dp, N);
-    }
-    if (in_place) { R(st_ticks, (N + 3) * 4); R(st_ln, (N + 3) * 4); R(st_g, N + 3); }      // (whole vectors of four)
-    R(binned, N * 4); R(req, N * 16); R(sorted, N * 4);
-    if (G == 1) R(inv, N * 4);
-    R(tick_start, (size_t)2 * G * kTickBins * 4); R(len_end, (size_t)G * (kMaxPrompt + 1) * 4);
-    // one block for everything a load clears: the flags and sums, the two histograms
+    Layout lay;
+    const size_t o_req = lay.take(N * 16), o_sorted = lay.take(N * 4), o_binned = lay.take(N * 4), o_inv = lay.take(G == 1 ? N * 4 : 0);
+    // one block for everything a load clears: the flags and sums, the two histograms, the windows of the sort
     const size_t tick_bytes = (size_t)G * kTickBins * 4, cnt_bytes = ((size_t)G * (kMaxPrompt + 1) * 4 + 15) / 16 * 16;
-    const size_t win_bytes = (size_t)sort_windows(n, G) * 8;
-    R(zero, sizeof(LoadZero) + tick_bytes + cnt_bytes + win_bytes);
+    c->zero_bytes = sizeof(LoadZero) + tick_bytes + cnt_bytes + (size_t)sort_windows(n, G) * 8;
+    const size_t o_zero = lay.take(c->zero_bytes), o_ends = lay.take((size_t)G * (kMaxPrompt + 1) * 4), o_starts = lay.take(2 * tick_bytes);
+    const size_t o_mass = lay.take((size_t)G * (kMaxPrompt + 2) * 8), o_off = lay.take((kMaxGroups + 1) * 4);
+    const size_t o_knots = lay.take((size_t)G * kNKnots * 4), o_fin = lay.take((size_t)2 * kMaxGroups * 8);
+    size_t o_in[5] = {0, 0, 0, 0, 0};
+    if (in == IN_COPIED) {
+        for (int k = 0; k < 3; ++k) o_in[k] = lay.take(N * 4);
+        o_in[3] = lay.take(has_sp ? N : 0); o_in[4] = lay.take(has_dp ? N : 0);
+    } else if (in == IN_PLACE) {
+        o_in[0] = lay.take(N4 * 4); o_in[1] = lay.take(N4 * 4); o_in[2] = lay.take(N4);      // (whole vectors of four)
+    } else if (in == IN_PACKED) {
+        o_in[0] = lay.take(n > kPackInPlace ? packed_bytes(n) : 0);
+    }
+    const cudaError_t e = c->trace_mem.reserve(lay.bytes);
+    if (e) return e;
+    char* base = (char*)c->trace_mem.p;
+    c->req.p = base + o_req; c->sorted.p = base + o_sorted; c->binned.p = base + o_binned; c->inv.p = base + o_inv;
+    c->zero.p = base + o_zero; c->len_end.p = base + o_ends; c->tick_start.p = base + o_starts; c->cum_mass.p = base + o_mass;
+    c->grp_off.p = base + o_off; c->knots.p = base + o_knots; c->fin_totals.p = base + o_fin;
+    c->in_prompt.p = c->st_ticks.p = c->packed.p = base + o_in[0];
+    c->in_out.p = c->st_ln.p = base + o_in[1];
+    c->in_ttft.p = c->st_g.p = base + o_in[2];
+    c->in_sp.p = base + o_in[3]; c->in_dp.p = base + o_in[4];
     c->z = (LoadZero*)c->zero.p;
     c->tick_cnt = (uint32_t*)(c->z + 1);
     c->cnt = (uint32_t*)((char*)c->tick_cnt + tick_bytes);
-    c->err = c->z->err;
     c->windows = (uint2*)((char*)c->cnt + cnt_bytes);
-    c->zero_bytes = sizeof(LoadZero) + tick_bytes + cnt_bytes + win_bytes;
-    R(cum_mass, (size_t)G * (kMaxPrompt + 2) * 8);
-    R(grp_off, (kMaxGroups + 1) * 4); R(knots, (size_t)G * kNKnots * 4);
-    R(d_gc, (size_t)G * sizeof(GroupConst));
-    R(fin_totals, (size_t)2 * kMaxGroups * 8);
-#undef R
-    return cudaSuccess;
+    c->err = c->z->err;
+    return c->d_gc.reserve((size_t)kMaxGroups * sizeof(GroupConst));
 }
 
 // The fallback sort: ticks stored group after group (off: [G + 1], device memory) ascending within each group into out.
@@ -280,33 +305,32 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         if (e0 != cudaSuccess || c->sms < 1) return bail(fail_cuda(e0, "multiprocessor count of the current device"));
     }
     const uint32_t n = c->n;
-    bool host_in = d->arrays_on_device != 1;
     cudaError_t e;
     // Host arrays that are page-locked and mapped (cudaHostAlloc, cudaHostRegister, a pinned tensor) are read by
     // the ingestion kernel in place (it reads every element exactly once): no staging copies.  Pageable arrays are
-    // copied first.
+    // packed and copied by several threads.
     const void* in_place[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    bool zero_copy = host_in && n != 0 && d->arrays_on_device == 0;
-    if (zero_copy) {
+    Inputs in = d->arrays_on_device == 1 ? IN_DEVICE : (d->arrays_on_device == 2 || n == 0) ? IN_COPIED : IN_PLACE;
+    if (in == IN_PLACE) {
         const void* host[5] = {d->prompt_len, d->output_len, d->server_ttft_s, d->server_profile, d->device_profile};
-        for (int k = 0; k < 5 && zero_copy; ++k) {
+        for (int k = 0; k < 5 && in == IN_PLACE; ++k) {
             if (!host[k]) continue;
             cudaPointerAttributes attr;
-            if (cudaPointerGetAttributes(&attr, host[k]) != cudaSuccess) { cudaGetLastError(); zero_copy = false; break; }
-            if (attr.type != cudaMemoryTypeHost || !attr.devicePointer) zero_copy = false;
+            if (cudaPointerGetAttributes(&attr, host[k]) != cudaSuccess) { cudaGetLastError(); in = IN_PACKED; break; }
+            if (attr.type != cudaMemoryTypeHost || !attr.devicePointer) in = IN_PACKED;
             else in_place[k] = attr.devicePointer;
         }
     }
-    if (zero_copy) host_in = false;
-    if (!c->rb && (e = cudaMallocHost((void**)&c->rb, sizeof(HostReadback))) != cudaSuccess)
+    if (!c->rb && (e = cudaMallocHost((void**)&c->rb, sizeof(HostReadback) + 256)) != cudaSuccess)    // (the selection's pair behind it)
         return bail(fail_cuda(e, "cudaMallocHost"));
-    if ((e = reserve_trace(c, n, host_in, zero_copy, d->server_profile != nullptr, d->device_profile != nullptr)) != cudaSuccess)
+    c->sel_host = (int32_t*)((char*)c->rb + (sizeof(HostReadback) + 15) / 16 * 16);
+    if ((e = reserve_trace(c, n, in, d->server_profile != nullptr, d->device_profile != nullptr)) != cudaSuccess)
         return bail(fail_cuda(e, "device allocation for the trace"));
 
     LoadArgs a;
     std::memset(&a, 0, sizeof a);
     a.n = n; a.G = c->G; a.ns = c->ns; a.nd = c->nd;
-    if (host_in && n) {
+    if (in == IN_COPIED && n) {
 #define H2D(dst, src, bytes) if ((e = cudaMemcpyAsync(c->dst.p, src, bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess) return bail(fail_cuda(e, "host to device copy"))
         H2D(in_prompt, d->prompt_len, (size_t)n * 4); H2D(in_out, d->output_len, (size_t)n * 4);
         H2D(in_ttft, d->server_ttft_s, (size_t)n * 4);
@@ -316,14 +340,18 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         a.prompt = c->in_prompt.as<int32_t>(); a.outlen = c->in_out.as<int32_t>(); a.ttft = c->in_ttft.as<float>();
         a.sp = d->server_profile ? c->in_sp.as<uint8_t>() : nullptr;
         a.dp = d->device_profile ? c->in_dp.as<uint8_t>() : nullptr;
-    } else if (zero_copy) {
+    } else if (in == IN_PACKED) {
+        if (!c->packer) c->packer.reset(new (std::nothrow) Packer);
+        if (!c->packer) return bail(fail(DISCO_ENOMEM, "out of host memory"));
+        if ((e = c->packer->pack(*d, c->packed.as<char>(), st, &a.packed)) != cudaSuccess) return bail(fail_cuda(e, "packing the trace"));
+    } else if (in == IN_PLACE) {
         a.prompt = (const int32_t*)in_place[0]; a.outlen = (const int32_t*)in_place[1]; a.ttft = (const float*)in_place[2];
         a.sp = (const uint8_t*)in_place[3]; a.dp = (const uint8_t*)in_place[4];
+        a.st_ticks = c->st_ticks.as<uint32_t>(); a.st_ln = c->st_ln.as<uint32_t>(); a.st_g = c->st_g.as<uint8_t>();
     } else {
         a.prompt = d->prompt_len; a.outlen = d->output_len; a.ttft = d->server_ttft_s;
         a.sp = d->server_profile; a.dp = d->device_profile;
     }
-    if (zero_copy) { a.st_ticks = c->st_ticks.as<uint32_t>(); a.st_ln = c->st_ln.as<uint32_t>(); a.st_g = c->st_g.as<uint8_t>(); }
     a.z = c->z; a.cnt = c->cnt; a.tick_cnt = c->tick_cnt;
     a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)c->G * kTickBins;
     a.binned = c->binned.as<uint32_t>();
@@ -333,7 +361,8 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     a.windows = c->windows;
     a.rounds = (n + 3000000u - 1) / 3000000u;                       // (3 million records and ticks take 60 MB)
     a.readback = c->rb;                                             // pinned host memory, written by the kernel
-    // the profile table is read from pageable memory: this copy returns once it has been staged
+    // the profile table is read from pageable memory: this copy returns once it has been staged (a reload with the same
+    // profiles skips it)
     const bool same_profiles = c->gc_dev_at == c->d_gc.p && c->gc_dev.size() == c->gc.size() &&
                                std::memcmp(c->gc_dev.data(), c->gc.data(), c->gc.size() * sizeof(GroupConst)) == 0;
     if (!same_profiles) {
@@ -490,108 +519,115 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     // ---- the policies of a class: plain ones form grids of budgets by overheads (grid.cu), at most kGridCols by kGridRows
     //      to a slab; random routing and the Eq. 1-2 rule go pair by pair
     std::vector<uint32_t> tab;                     // lists of policy indices, one after the other
+    tab.reserve((size_t)4 * P + 64);
     std::vector<Slab> slabs;
     std::vector<uint32_t> mixed_pols;              // per slab: where its policies are listed for the pair kernel (mixed slabs)
     struct ClassLists { size_t all, n_all, ext, n_ext, slab0, slab1; };
     std::vector<ClassLists> lists(classes.size());
     bool any_mixed = false, any_pairs = false;
+    constexpr uint32_t kNone = 0xFFFFFFFFu;
+    auto theta_of = [&](uint32_t p) { return (pc[p].flags & DISCO_FLAG_MIGRATION) ? pc[p].theta : 0.0f; };   // (else it does not matter)
+    // The place of x in an ascending list of distinct values, entered if it is new; `at`: where the last one was.  Grids are
+    // given budget by budget or overhead by overhead: the next value mostly follows the last one.
+    auto place_of = [](std::vector<float>& v, float x, size_t& at) {
+        for (size_t k = at; k < v.size() && k < at + 2; ++k) if (v[k] == x) { at = k; return; }
+        const auto it = std::lower_bound(v.begin(), v.end(), x);
+        at = it - v.begin();
+        if (it == v.end() || *it != x) v.insert(it, x);
+    };
+    struct Grid { uint32_t flags, expected_len; float alpha; std::vector<uint32_t> pols; std::vector<float> budgets, thetas; size_t b_at, t_at; };
+    std::vector<Grid> grids;
+    std::vector<uint32_t> cells, used;
     for (size_t k = 0; k < classes.size(); ++k) {
         ClassLists& L = lists[k];
         L.all = tab.size();
         for (uint32_t p = 0; p < P; ++p) if (pc[p].cls == (int)k) tab.push_back(p);
         L.n_all = tab.size() - L.all;
-        auto is_ext = [&](uint32_t p) { return (pc[p].flags & (DISCO_FLAG_STOCHASTIC | DISCO_FLAG_BETA_RULE)) != 0; };
         L.ext = tab.size();
-        std::vector<uint32_t> plain;
-        for (size_t i = L.all; i < L.all + L.n_all; ++i) { const uint32_t p = tab[i]; if (is_ext(p)) tab.push_back(p); else plain.push_back(p); }
+        L.slab0 = slabs.size();
+        grids.clear();
+        for (size_t i = L.all; i < L.all + L.n_all; ++i) {
+            const uint32_t p = tab[i];
+            const PolicyConst& q = pc[p];
+            if (q.flags & (DISCO_FLAG_STOCHASTIC | DISCO_FLAG_BETA_RULE)) { tab.push_back(p); continue; }
+            Grid* at = nullptr;
+            for (size_t x = grids.size(); x-- > 0 && !at;)
+                if (grids[x].flags == q.flags && grids[x].expected_len == q.expected_len && grids[x].alpha == q.alpha) at = &grids[x];
+            if (!at) {
+                grids.push_back(Grid{q.flags, q.expected_len, q.alpha, {}, {}, {}, 0, 0});
+                at = &grids.back();
+                at->pols.reserve(L.n_all);
+            }
+            at->pols.push_back(p);
+            place_of(at->budgets, q.budget, at->b_at);
+            place_of(at->thetas, theta_of(p), at->t_at);
+        }
         L.n_ext = tab.size() - L.ext;
         any_pairs = any_pairs || L.n_ext != 0;
-        L.slab0 = slabs.size();
-        auto theta_of = [&](uint32_t p) { return (pc[p].flags & DISCO_FLAG_MIGRATION) ? pc[p].theta : 0.0f; };   // (else it does not matter)
-        auto same_grid = [&](uint32_t x, uint32_t y) {
-            return pc[x].flags == pc[y].flags && pc[x].expected_len == pc[y].expected_len && pc[x].alpha == pc[y].alpha;
-        };
-        std::sort(plain.begin(), plain.end(), [&](uint32_t x, uint32_t y) {
-            const PolicyConst &a = pc[x], &b = pc[y];
-            if (a.flags != b.flags) return a.flags < b.flags;
-            if (a.expected_len != b.expected_len) return a.expected_len < b.expected_len;
-            if (a.alpha != b.alpha) return a.alpha < b.alpha;
-            if (a.budget != b.budget) return a.budget < b.budget;
-            const float tx = theta_of(x), ty = theta_of(y);
-            return tx != ty ? tx < ty : x < y;
-        });
-        for (size_t i = 0; i < plain.size();) {
-            size_t end = i;
-            while (end < plain.size() && same_grid(plain[i], plain[end])) ++end;
-            std::vector<float> th;
-            size_t budgets = 0;
-            for (size_t x = i; x < end; ++x) {
-                th.push_back(theta_of(plain[x]));
-                if (x == i || pc[plain[x]].budget != pc[plain[x - 1]].budget) ++budgets;
-            }
-            std::sort(th.begin(), th.end());
-            th.erase(std::unique(th.begin(), th.end()), th.end());
+        for (Grid& gr : grids) {
+            const size_t n_b = gr.budgets.size(), n_t = gr.thetas.size(), n_p = gr.pols.size();
             auto open = [&](int T, bool mixed) {
                 Slab sl;
                 std::memset(&sl, 0, sizeof sl);
-                sl.T = T; sl.expected_len = pc[plain[i]].expected_len; sl.mixed = mixed ? 1 : 0;
-                sl.mig = (pc[plain[i]].flags & DISCO_FLAG_MIGRATION) ? 1 : 0;
+                sl.T = T; sl.expected_len = gr.expected_len; sl.mixed = mixed ? 1 : 0;
+                sl.mig = (gr.flags & DISCO_FLAG_MIGRATION) ? 1 : 0;
                 return sl;
             };
-            // closes a slab of the columns `cols` (a policy per row, ~0 for none)
-            auto close = [&](Slab sl, const std::vector<std::vector<uint32_t>>& cols, size_t c0, size_t c1, uint32_t listed) {
+            // closes a slab of the columns [c0, c1) of `cells` (T policies each, kNone for none)
+            auto close = [&](Slab sl, size_t c0, size_t c1, uint32_t listed) {
+                const size_t T = (size_t)sl.T;
                 sl.K = (int32_t)(c1 - c0);
                 sl.cols = (uint32_t)tab.size();
                 for (size_t x = c0; x < c1; ++x)
-                    for (uint32_t p : cols[x]) if (p != 0xFFFFFFFFu) { tab.push_back(p); break; }
+                    for (size_t r = 0; r < T; ++r) if (cells[x * T + r] != kNone) { tab.push_back(cells[x * T + r]); break; }
                 sl.cells = (uint32_t)tab.size();
-                for (size_t x = c0; x < c1; ++x)
-                    for (uint32_t p : cols[x]) { tab.push_back(p); sl.policies += p != 0xFFFFFFFFu; }
+                for (size_t x = c0 * T; x < c1 * T; ++x) sl.policies += cells[x] != kNone;
+                tab.insert(tab.end(), cells.begin() + c0 * T, cells.begin() + c1 * T);
                 slabs.push_back(sl);
                 mixed_pols.push_back(listed);
             };
-            if (th.size() > 1 && 2 * (end - i) <= budgets * th.size()) {
+            if (n_t > 1 && 2 * n_p <= n_b * n_t) {
                 // Most (budget, overhead) combinations are no policy: a column per policy instead, and what the overheads
                 // of a slab's policies do not agree on goes pair by pair.
-                for (size_t x0 = i; x0 < end; x0 += kGridCols) {
-                    const size_t x1 = std::min(end, x0 + (size_t)kGridCols);
+                cells = gr.pols;
+                std::sort(cells.begin(), cells.end(), [&](uint32_t x, uint32_t y) { return pc[x].budget != pc[y].budget ? pc[x].budget < pc[y].budget : x < y; });
+                for (size_t x0 = 0; x0 < n_p; x0 += kGridCols) {
+                    const size_t x1 = std::min(n_p, x0 + (size_t)kGridCols);
                     Slab sl = open(1, true);
-                    std::vector<std::vector<uint32_t>> cols;
-                    float lo = theta_of(plain[x0]), hi = lo;
                     const uint32_t listed = (uint32_t)tab.size();
+                    tab.insert(tab.end(), cells.begin() + x0, cells.begin() + x1);
+                    sl.theta[0] = sl.theta[1] = theta_of(cells[x0]);
                     for (size_t x = x0; x < x1; ++x) {
-                        cols.push_back({plain[x]});
-                        tab.push_back(plain[x]);
-                        lo = std::min(lo, theta_of(plain[x])); hi = std::max(hi, theta_of(plain[x]));
+                        sl.theta[0] = std::min(sl.theta[0], theta_of(cells[x])); sl.theta[1] = std::max(sl.theta[1], theta_of(cells[x]));
                     }
-                    sl.theta[0] = lo; sl.theta[1] = hi;
-                    close(sl, cols, 0, cols.size(), listed);
+                    close(sl, x0, x1, listed);
                     any_mixed = any_pairs = true;
                 }
-            } else {
-                for (size_t r0 = 0; r0 < th.size(); r0 += kGridRows) {
-                    const size_t r1 = std::min(th.size(), r0 + (size_t)kGridRows);
-                    Slab sl = open((int)(r1 - r0), false);
-                    for (size_t r = r0; r < r1; ++r) sl.theta[r - r0] = th[r];
-                    // columns in ascending order of budget; a policy given twice takes a further column of its budget
-                    std::vector<std::vector<uint32_t>> cols;
-                    for (size_t x = i; x < end;) {
-                        const size_t c_first = cols.size();
-                        const float b = pc[plain[x]].budget;
-                        for (; x < end && pc[plain[x]].budget == b; ++x) {
-                            const size_t r = std::lower_bound(th.begin(), th.end(), theta_of(plain[x])) - th.begin();
-                            if (r < r0 || r >= r1) continue;
-                            size_t at = c_first;
-                            while (at < cols.size() && cols[at][r - r0] != 0xFFFFFFFFu) ++at;
-                            if (at == cols.size()) cols.push_back(std::vector<uint32_t>(r1 - r0, 0xFFFFFFFFu));
-                            cols[at][r - r0] = plain[x];
-                        }
-                    }
-                    for (size_t c0 = 0; c0 < cols.size(); c0 += kGridCols)
-                        close(sl, cols, c0, std::min(cols.size(), c0 + (size_t)kGridCols), 0u);
-                }
+                continue;
             }
-            i = end;
+            for (size_t r0 = 0; r0 < n_t; r0 += kGridRows) {
+                const size_t r1 = std::min(n_t, r0 + (size_t)kGridRows), T = r1 - r0;
+                Slab sl = open((int)T, false);
+                for (size_t r = r0; r < r1; ++r) sl.theta[r - r0] = gr.thetas[r];
+                // how many policies share a (budget, overhead): those after the first take further columns of their budget
+                used.assign(n_b * T, 0);
+                size_t b_at = 0, t_at = 0;
+                std::vector<uint32_t> wide(n_b, 0);
+                for (uint32_t p : gr.pols) {
+                    place_of(gr.budgets, pc[p].budget, b_at); place_of(gr.thetas, theta_of(p), t_at);
+                    if (t_at >= r0 && t_at < r1) wide[b_at] = std::max(wide[b_at], ++used[b_at * T + (t_at - r0)]);
+                }
+                size_t cols = 0;
+                for (uint32_t& w : wide) { const uint32_t here = w; w = (uint32_t)cols; cols += here; }
+                cells.assign(cols * T, kNone);
+                used.assign(n_b * T, 0);
+                b_at = t_at = 0;
+                for (uint32_t p : gr.pols) {
+                    place_of(gr.budgets, pc[p].budget, b_at); place_of(gr.thetas, theta_of(p), t_at);
+                    if (t_at >= r0 && t_at < r1) cells[(wide[b_at] + used[b_at * T + (t_at - r0)]++) * T + (t_at - r0)] = p;
+                }
+                for (size_t c0 = 0; c0 < cols; c0 += kGridCols) close(sl, c0, std::min(cols, c0 + (size_t)kGridCols), 0u);
+            }
         }
         L.slab1 = slabs.size();
     }
@@ -649,25 +685,43 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         n_tickets += (uint32_t)batches[k].size();
     }
 
-    // ---- device buffers
+    // ---- device memory: what must be clear comes first and together -- the work counters and tickets, the difference
+    //      tables of the first batch, and the accumulators if some pairs are added to them one by one (k_spread writes those
+    //      of all other policies)
     cudaError_t e;
-#define R(buf, bytes) if ((e = c->buf.reserve(bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation")
-    R(d_prep, (size_t)G * P * sizeof(Prep));
     const size_t acc_bytes = (size_t)P * G * kNAcc * 8, hist_bytes = (size_t)P * kNBins * 8;
-    const size_t cnt_bytes = 32 + ((size_t)n_tickets * 4 + 15) / 16 * 16;     // four work counters, then the tickets
-    R(d_accum, acc_bytes + 2 * hist_bytes + cnt_bytes);
+    auto batch_bytes = [&](const Batch& b, bool wide) { return b.sums * 8 + b.tbt * (wide ? 8 : 4) + b.ttft * 4; };
+    size_t first_bytes = 0;
+    for (size_t k = 0; k < classes.size() && first_bytes == 0; ++k)
+        if (!batches[k].empty()) first_bytes = batch_bytes(batches[k][0], wide_class(k));
+    const bool clear_accum = any_pairs || n == 0;
+    Layout lay;
+    const size_t o_work = lay.take(32 + (size_t)n_tickets * 4), o_accum = clear_accum ? lay.take(acc_bytes + 2 * hist_bytes) : 0;
+    const size_t o_grid = lay.bytes;
+    lay.take(grid_bytes);
+    const size_t clear_bytes = n == 0 ? o_grid : o_grid + first_bytes;
+    const size_t o_prep = lay.take((size_t)G * P * sizeof(Prep)), o_stats = lay.take(P * sizeof(disco_policy_stats_t) + 16);
+    const size_t o_accum2 = clear_accum ? o_accum : lay.take(acc_bytes + 2 * hist_bytes);
+    const size_t o_left = lay.take(any_mixed ? (N1 + kMaxGroups) * 4 : 0), o_hand = lay.take(N1 * 8);
+    size_t o_rec[6] = {}, o_win[3] = {};
+    if (stored) {
+        for (int k = 0; k < 6; ++k) o_rec[k] = lay.take(N1 * 4);
+        for (int k = 0; k < 3; ++k) o_win[k] = lay.take(N1 * wmax[k] * 2);
+    }
+    const size_t table_bytes = ((size_t)P * sizeof(PolicyConst) + 15) / 16 * 16 + (classes.size() * sizeof(ClassConst) + 15) / 16 * 16 +
+                               (tab.size() * 4 + 15) / 16 * 16 + (slabs.size() * sizeof(Slab) + 15) / 16 * 16 +
+                               (chunks.size() + pair_chunks.size()) * sizeof(Chunk);
+    const size_t o_tables = lay.take(table_bytes);
+    if ((e = c->eval_mem.reserve(lay.bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
+    char* mem = (char*)c->eval_mem.p;
+    c->d_prep.p = mem + o_prep; c->d_accum.p = mem + o_accum2; c->d_stats.p = mem + o_stats; c->d_grid.p = mem + o_grid;
+    c->d_left.p = mem + o_left; c->d_tables.p = mem + o_tables; c->rec_hand.p = mem + o_hand;
+    for (int k = 0; k < 6; ++k) c->rec_u32[k].p = mem + o_rec[k];
+    for (int k = 0; k < 3; ++k) c->rec_win[k].p = mem + o_win[k];
     c->d_acc.p = c->d_accum.p; c->d_hist_ttft.p = (char*)c->d_accum.p + acc_bytes;
     c->d_hist_tbt.p = (char*)c->d_accum.p + acc_bytes + hist_bytes;
-    c->d_work.p = (char*)c->d_accum.p + acc_bytes + 2 * hist_bytes;
+    c->d_work.p = mem + o_work;
     uint32_t* tickets = (uint32_t*)((char*)c->d_work.p + 32);
-    R(d_stats, P * sizeof(disco_policy_stats_t) + 16);
-    R(rec_hand, N1 * 8);
-    if (stored) {
-        for (int k = 0; k < 6; ++k) R(rec_u32[k], N1 * 4);
-        for (int k = 0; k < 3; ++k) R(rec_win[k], N1 * wmax[k] * 2);
-    }
-    R(d_grid, grid_bytes);
-    if (any_mixed) R(d_left, (N1 + kMaxGroups) * 4);
 
     if (c->fin_imported) {            // an import replaced the totals the final reductions refer to: back to the trace's own
         c->fin_own.assign((size_t)2 * G, 0);
@@ -675,47 +729,40 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         CU(cudaMemcpyAsync(c->fin_totals.p, c->fin_own.data(), c->fin_own.size() * 8, cudaMemcpyHostToDevice, st));
         c->fin_imported = false;
     }
-    CU(cudaMemsetAsync(c->d_accum.p, 0, acc_bytes + 2 * hist_bytes + cnt_bytes, st));
+    CU(cudaMemsetAsync(mem, 0, clear_bytes, st));
 
     // ---- small tables to the device through pinned staging: one staging block, one copy (16-byte aligned regions)
-    const size_t need = P * sizeof(PolicyConst) + classes.size() * sizeof(ClassConst) + tab.size() * 4 + slabs.size() * sizeof(Slab) +
-                        (chunks.size() + pair_chunks.size()) * sizeof(Chunk) + 128;
     if (c->stage_free) CU(cudaEventSynchronize(c->stage_free));     // an earlier call's copies may still read it
     else CU(cudaEventCreateWithFlags(&c->stage_free, cudaEventDisableTiming));
-    if (need > c->stage_cap) {
+    if (table_bytes > c->stage_cap) {
         if (c->stage) cudaFreeHost(c->stage);
         c->stage = nullptr; c->stage_cap = 0;
-        CU(cudaMallocHost(&c->stage, need));
-        c->stage_cap = need;
+        CU(cudaMallocHost(&c->stage, table_bytes));
+        c->stage_cap = table_bytes;
     }
-    char* sp = (char*)c->stage;
+    char *sp = (char*)c->stage, *dt = mem + o_tables;
     size_t off = 0;
-    auto put = [&](DevBufView& v, const void* src, size_t bytes) {
+    auto put = [&](const void* src, size_t bytes) {
         if (bytes) std::memcpy(sp + off, src, bytes);
-        v.off = off;
+        char* at = dt + off;
         off += (bytes + 15) / 16 * 16;
+        return at;
     };
-    DevBufView v_pol, v_cls, v_tab, v_slabs, v_chunks, v_pair;
-    put(v_pol, pc.data(), P * sizeof(PolicyConst));
-    put(v_cls, classes.data(), classes.size() * sizeof(ClassConst));
-    put(v_tab, tab.data(), tab.size() * 4);
-    put(v_slabs, slabs.data(), slabs.size() * sizeof(Slab));
-    put(v_chunks, chunks.data(), chunks.size() * sizeof(Chunk));
-    put(v_pair, pair_chunks.data(), pair_chunks.size() * sizeof(Chunk));
-    if ((e = c->d_tables.reserve(off + 16)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
-#undef R
-    char* dt = (char*)c->d_tables.p;
-    c->d_pol.p = dt + v_pol.off; c->d_classes.p = dt + v_cls.off; c->d_tab.p = dt + v_tab.off; c->d_slabs.p = dt + v_slabs.off;
-    c->d_chunks.p = dt + v_chunks.off; c->d_pair_chunks.p = dt + v_pair.off;
+    const PolicyConst* d_pol = (const PolicyConst*)put(pc.data(), P * sizeof(PolicyConst));
+    const ClassConst* d_classes = (const ClassConst*)put(classes.data(), classes.size() * sizeof(ClassConst));
+    const uint32_t* d_tab = (const uint32_t*)put(tab.data(), tab.size() * 4);
+    const Slab* d_slabs = (const Slab*)put(slabs.data(), slabs.size() * sizeof(Slab));
+    const Chunk* d_chunks = (const Chunk*)put(chunks.data(), chunks.size() * sizeof(Chunk));
+    const Chunk* d_pair_chunks = (const Chunk*)put(pair_chunks.data(), pair_chunks.size() * sizeof(Chunk));
     CU(cudaMemcpyAsync(dt, sp, off, cudaMemcpyHostToDevice, st));
     CU(cudaEventRecord(c->stage_free, st));
 
     // ---- Algorithms 1-3 for every (group, policy)
-    CU(launch_prep(c->d_pol.as<PolicyConst>(), P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
+    CU(launch_prep(d_pol, P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
                    c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), st));
     g_launches += 1;
     if (any_beta) {
-        CU(launch_prep_beta(c->d_pol.as<PolicyConst>(), P, G, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
+        CU(launch_prep_beta(d_pol, P, G, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
                             c->F_off, c->d_prep.as<Prep>(), st));
         g_launches += 1;
     }
@@ -745,12 +792,12 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     uint32_t ticket = (uint32_t)classes.size();
     const Prep* prep = c->d_prep.as<Prep>();
     const GroupConst* gc = c->d_gc.as<GroupConst>();
-    const uint32_t* d_tab = c->d_tab.as<uint32_t>();
     uint64_t *acc = c->d_acc.as<uint64_t>(), *h_ttft = c->d_hist_ttft.as<uint64_t>(), *h_tbt = c->d_hist_tbt.as<uint64_t>(),
              *work = c->d_work.as<uint64_t>();
+    bool first_batch = true;
     // ---- per timeline class: play every request out, then evaluate the class's policies on the summaries
     for (size_t k = 0; k < classes.size() && n != 0; ++k) {
-        const ClassConst* dcc = c->d_classes.as<ClassConst>() + k;
+        const ClassConst* dcc = d_classes + k;
         const bool wide = wide_class(k);
         if (timed) CU(cudaEventRecord(c->ev[0], st));
         CU(launch_timeline(tr, gc, dcc, classes[k], c->knots.as<int32_t>(), k0, rec, c->err, tickets + k, plan[k].kinds,
@@ -764,8 +811,9 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             gt.sums = (unsigned long long*)base;
             gt.tbt = base + b.sums * 8;
             gt.ttft = (uint32_t*)(base + b.sums * 8 + b.tbt * tbt_word);
-            CU(cudaMemsetAsync(base, 0, b.sums * 8 + b.tbt * tbt_word + b.ttft * 4, st));
-            const Slab* dsl = c->d_slabs.as<Slab>() + b.first;
+            if (!first_batch) CU(cudaMemsetAsync(base, 0, batch_bytes(b, wide), st));
+            first_batch = false;
+            const Slab* dsl = d_slabs + b.first;
             const bool mixed = slabs[b.first].mixed != 0;
             LeftLists left = {nullptr, nullptr};
             if (mixed) {
@@ -773,13 +821,13 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
             }
             CU(launch_grid(tr, gc, dcc, prep, P, dsl, (uint32_t)b.count, b.T, wide, classes[k].pacing != 0, d_tab,
-                           c->d_chunks.as<Chunk>(), (uint32_t)chunks.size(), rec, gt, left, tickets + ticket++, work, c->sms, st));
+                           d_chunks, (uint32_t)chunks.size(), rec, gt, left, tickets + ticket++, work, c->sms, st));
             CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, wide, host_bin_of_ticks(classes[k].tau), d_tab, gt, acc,
                              h_ttft, h_tbt, st));
             g_launches += 2;
             if (mixed) {
                 const Slab& sl = slabs[b.first];
-                CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + mixed_pols[b.first], sl.policies, c->d_pair_chunks.as<Chunk>(),
+                CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + mixed_pols[b.first], sl.policies, d_pair_chunks,
                                     (uint32_t)pair_chunks.size(), left.list, left.count, rec, acc, h_ttft, h_tbt, work, k0,
                                     sl.expected_len != 0, wide, st));
                 g_launches += 1;
@@ -787,7 +835,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         }
         if (lists[k].n_ext) {
             CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + lists[k].ext, (uint32_t)lists[k].n_ext,
-                                c->d_pair_chunks.as<Chunk>(), (uint32_t)pair_chunks.size(), nullptr, nullptr, rec, acc, h_ttft, h_tbt,
+                                d_pair_chunks, (uint32_t)pair_chunks.size(), nullptr, nullptr, rec, acc, h_ttft, h_tbt,
                                 work, k0, true, wide, st));
             g_launches += 1;
         }
@@ -799,7 +847,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         if (timed) CU(cudaEventRecord(c->ev[4], st));
     }
     c->timing_valid = timed && n != 0;
-    c->P = P; c->pol = pc;
+    c->P = P; c->pol.swap(pc);
     c->evaluated = true;
     return 0;
 }
@@ -808,9 +856,16 @@ int disco_reduce_stats(disco_ctx_t* c, disco_policy_stats_t* stats, void* stream
     if (!c || !stats) return fail(DISCO_EINVAL, "null argument");
     if (!c->evaluated) return fail(DISCO_EINVAL, "no evaluation to reduce");
     cudaStream_t st = (cudaStream_t)stream;
-    // statistics and the error word land in pinned host memory straight from the kernel
-    const size_t bytes = c->P * sizeof(disco_policy_stats_t) + 16;
-    if (bytes > c->stats_host_cap) {
+    // Statistics and the error word land in pinned host memory straight from the kernel: in the caller's array if it is
+    // page-locked (from a few dozen records on, where the copy would count), else in the context's.
+    const size_t bytes = c->P * sizeof(disco_policy_stats_t);
+    disco_policy_stats_t* to = nullptr;
+    if (c->P >= 64) {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, stats) != cudaSuccess) cudaGetLastError();
+        else if (attr.type == cudaMemoryTypeHost && attr.devicePointer) to = (disco_policy_stats_t*)attr.devicePointer;
+    }
+    if (!to && bytes > c->stats_host_cap) {
         if (c->stats_host) cudaFreeHost(c->stats_host);
         c->stats_host = nullptr; c->stats_host_cap = 0;
         CU(cudaMallocHost(&c->stats_host, bytes));
@@ -818,11 +873,10 @@ int disco_reduce_stats(disco_ctx_t* c, disco_policy_stats_t* stats, void* stream
     }
     CU(launch_finalize(c->P, c->G, c->d_gc.as<GroupConst>(), c->d_acc.as<uint64_t>(), c->d_hist_ttft.as<uint64_t>(),
                        c->d_hist_tbt.as<uint64_t>(), c->fin_totals.as<uint64_t>(),
-                       c->d_stats.as<disco_policy_stats_t>(), (disco_policy_stats_t*)c->stats_host, c->err, st));
+                       c->d_stats.as<disco_policy_stats_t>(), to ? to : (disco_policy_stats_t*)c->stats_host, c->err, c->rb->err, st));
     CU(cudaStreamSynchronize(st));
     if (int rc = debug_check()) return rc;
-    std::memcpy(stats, c->stats_host, c->P * sizeof(disco_policy_stats_t));
-    std::memcpy(c->rb->err, (char*)c->stats_host + c->P * sizeof(disco_policy_stats_t), 16);
+    if (!to) std::memcpy(stats, c->stats_host, bytes);
     g_launches += 1;
     if (c->timing_valid) {
         for (int k = 0; k < 4; ++k) CU(cudaEventElapsedTime(&c->ms[k], c->ev[k], c->ev[k + 1]));
@@ -869,7 +923,6 @@ int disco_select_policy_device(disco_ctx_t* c, double cost_cap, float tbt_slo_s,
     if (!c || !best) return fail(DISCO_EINVAL, "null argument");
     if (!c->reduced) return fail(DISCO_EINVAL, "reduce the statistics before selecting");
     cudaStream_t st = (cudaStream_t)stream;
-    if (!c->sel_host) CU(cudaMallocHost((void**)&c->sel_host, 8));
     g_launches += 1;
     CU(launch_select(c->d_stats.as<disco_policy_stats_t>(), c->P, cost_cap, tbt_slo_s, c->sel_host, st));   // writes the pinned pair
     CU(cudaStreamSynchronize(st));

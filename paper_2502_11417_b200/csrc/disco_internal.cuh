@@ -169,6 +169,9 @@ __device__ __forceinline__ bool batch_of_kind(const TraceDev& tr, const ClassCon
 }
 #endif
 
+// Lets a kernel use that much dynamic shared memory, once per kernel and device.
+cudaError_t allow_smem(const void* kernel, size_t bytes);
+
 // Records the calling thread's error message (read back by disco_last_error) and returns `code`.
 int set_error(int code, const char* msg);
 
@@ -272,9 +275,9 @@ cudaError_t launch_pairs_rows(const TraceDev& tr, const GroupConst* gc, const Cl
 cudaError_t launch_finalize(uint32_t P, int G, const GroupConst* gc, const uint64_t* acc, const uint64_t* hist_ttft,
                             const uint64_t* hist_tbt,
                             const uint64_t* fin_totals /* [2G]: output tokens per group, then requests per group */,
-                            disco_policy_stats_t* stats /* [P] + 16 bytes */,
-                            disco_policy_stats_t* stats_host /* pinned host mirror of the same size, written by the kernel */,
-                            const int32_t* err, cudaStream_t st);
+                            disco_policy_stats_t* stats /* [P] */,
+                            disco_policy_stats_t* stats_host /* [P], pinned host memory, written by the kernel */,
+                            const int32_t* err, int32_t* err_host /* pinned: a copy of err */, cudaStream_t st);
 cudaError_t launch_select(const disco_policy_stats_t* stats, uint32_t P, double cost_cap, float tbt_slo_s,
                           int32_t* result /* [2]: status, index; may be pinned host memory */, cudaStream_t st);
 // Cumulative token mass and knots from tables given by the caller (F_off[g] .. F_off[g+1] delimit group g's ticks).

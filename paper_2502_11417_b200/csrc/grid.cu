@@ -591,11 +591,20 @@ k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict
     part -= T * kParts;
     if (part < T * kParts) {                                           // TBT
         const int r = part / kParts, b = (part - r * kParts) * 32 + lane;
-        spread_columns<word>(s_part, K, [&](int q) { return tb.tbt_row(q, r)[b]; }, [&](int c, word x) {
+        // (in 64 bits: tau's bin holds all regular TBTs; a 32-bit row is a difference of at most 2^31 requests)
+        using big = unsigned long long;
+        spread_columns<big>(s_part, K, [&](int q) {
+            const word y = tb.tbt_row(q, r)[b];
+            big x = WIDE ? (big)y : (big)(long long)(int32_t)y;
+            if (b == bin_tau)                                          // the regular TBTs of streams that keep the pace
+                for (int g = 0; g < tr.n_groups; ++g) {
+                    const unsigned long long* row = tb.sum_row(g, q);
+                    x += row[B_TAU] + (WIDE ? row[kBase + r * kLev + V_TAU] : 0ull - row[kBase + r * kLev + V_N]);
+                }
+            return x;
+        }, [&](int c, big x) {
             const uint32_t p = cells[c * T + r];
-            if (p == kNoPolicy) return;
-            unsigned long long* h = &hist_tbt[(size_t)p * kNBins + b];
-            if (b == bin_tau) atomicAdd(h, (unsigned long long)x); else *h = x;      // (the regular TBTs join tau's bin below)
+            if (p != kNoPolicy) hist_tbt[(size_t)p * kNBins + b] = x;
         });
         return;
     }
@@ -606,7 +615,7 @@ k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict
     const int s = mine ? k % kNAcc : 0, r = mine ? (k / kNAcc) % T : 0, g = mine ? k / (kNAcc * T) : 0;
     const int cand = gcs[g].candidate;
     const int fb = s == A_DEVICE_ONLY ? B_DO : s == A_RACE ? B_RACE : s == A_DEVICE_WON ? B_DW : s == A_TOK_DEVICE ? B_TD
-                 : s == A_PRE_SERVER ? B_PS : s == A_PRE_DEVICE ? B_PD : s == A_TTFT_SUM ? B_TT : s == A_TAU_CNT ? B_TAU : -1;
+                 : s == A_PRE_SERVER ? B_PS : s == A_PRE_DEVICE ? B_PD : s == A_TTFT_SUM ? B_TT : -1;
     int fl = -1;
     bool minus = false;
     if (s == A_TOK_DEVICE) { fl = V_A; minus = cand == 2; }            // the server's tokens go to the device, or the device's to the server
@@ -614,7 +623,6 @@ k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict
     else if (s == A_PRE_DEVICE && cand == 1) fl = V_B;
     else if (s == A_DELAYED) fl = V_C;
     else if (s == A_MIGR) fl = V_N;
-    else if (s == A_TAU_CNT) { fl = WIDE ? V_TAU : V_N; minus = !WIDE; }
     const int f2 = fl < 0 ? -1 : kBase + r * kLev + fl;
     spread_columns<unsigned long long>(s_part, K, [&](int q) {
         const unsigned long long* row = tb.sum_row(g, q);
@@ -624,9 +632,7 @@ k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict
     }, [&](int c, unsigned long long x) {
         const uint32_t p = mine ? cells[c * T + r] : kNoPolicy;
         if (p == kNoPolicy) return;
-        unsigned long long* to = acc + ((size_t)p * tr.n_groups + g) * kNAcc + s;
-        if (s == A_TAU_CNT) { *to = 0; if (x) atomicAdd(&hist_tbt[(size_t)p * kNBins + bin_tau], x); }
-        else *to = x;
+        acc[((size_t)p * tr.n_groups + g) * kNAcc + s] = x;
     });
 }
 
@@ -635,7 +641,7 @@ size_t grid_smem(int NT, bool wide) { return sizeof(Smem) + (size_t)(NT + (wide 
 template <int NT, bool WIDE>
 cudaError_t launch_one(const Args& a, int sms, cudaStream_t st) {
     const size_t smem = grid_smem(NT, WIDE);
-    cudaError_t e = cudaFuncSetAttribute(k_grid<NT, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)k_grid<NT, WIDE>, smem);
     if (e) return e;
     const uint64_t items = (uint64_t)a.n_chunks * a.n_slabs;
     const uint32_t blocks = (uint32_t)std::min<uint64_t>(items, (uint64_t)sms * (NT == 1 ? 4 : 2));

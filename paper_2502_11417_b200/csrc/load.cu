@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "pack.cuh"
 #include "scan.cuh"
 
 namespace disco {
@@ -39,6 +40,7 @@ constexpr int kPrivateGroups = 7;         // groups whose counters fit in shared
 constexpr int kPrivateTickGroups = 16;    // the same, counters of tick bins alone
 
 enum Source { S_TRACE, S_TICKS, S_TTFT };
+enum Form { F_COLUMNS, F_STAGE, F_PACKED };   // a trace's columns; the same, with a copy left for the second pass; packed
 
 __device__ __forceinline__ int tick_bin(uint32_t t) {
     return t < 128u ? (int)t : (int)(__float_as_uint(__uint2float_rz(t)) >> 16) - ((127 + 7) << 7) + 128;
@@ -92,9 +94,9 @@ __device__ __forceinline__ void load4(const T* p, uint32_t i0, uint32_t n, bool 
 
 // Reads the items i0 .. i0 + 3, and in the first pass checks them.  wide: the columns are aligned for vector loads.
 // AGAIN: for counting; it will be read once more.
-template <int SRC, bool STAGE, bool CHECK, bool AGAIN = false>
+template <int SRC, int FORM, bool CHECK, bool AGAIN = false>
 __device__ __forceinline__ void read_items(const LoadArgs& a, uint32_t i0, bool wide, const uint32_t* s_off, Item (&x)[4]) {
-    if (STAGE && !CHECK) {
+    if (FORM == F_STAGE && !CHECK) {
         uint32_t ln[4], S[4];
         uint8_t g[4];
         load4<uint4, !CHECK && !AGAIN>(a.st_ln, i0, a.n, true, ln, 0u);
@@ -124,12 +126,26 @@ __device__ __forceinline__ void read_items(const LoadArgs& a, uint32_t i0, bool 
     int32_t l[4] = {1, 1, 1, 1}, o[4] = {1, 1, 1, 1};
     uint8_t sp[4] = {0, 0, 0, 0}, dp[4] = {0, 0, 0, 0};
     constexpr bool kLast = !CHECK && !AGAIN;
-    load4<float4, kLast>(a.ttft, i0, a.n, wide, t, 1.0f);
-    if (SRC == S_TRACE) {
+    if (FORM == F_PACKED) {
+        // (chunks are whole vectors, and a vector lies in one chunk; what lies behind item n is not used)
+        const char* c = a.packed + (size_t)(i0 / kPackChunk) * kPackBytes;
+        const uint32_t k = i0 % kPackChunk;
+        const uint4 ln = *reinterpret_cast<const uint4*>(c + (size_t)k * 4);
+        const float4 tt = *reinterpret_cast<const float4*>(c + (size_t)kPackChunk * 4 + (size_t)k * 4);
+        const uchar4 gg = *reinterpret_cast<const uchar4*>(c + (size_t)kPackChunk * 8 + k);
+        const uint32_t lns[4] = {ln.x, ln.y, ln.z, ln.w};
+        t[0] = tt.x; t[1] = tt.y; t[2] = tt.z; t[3] = tt.w;
+        dp[0] = gg.x; dp[1] = gg.y; dp[2] = gg.z; dp[3] = gg.w;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { l[u] = (int32_t)(lns[u] & 0xFFFFu); o[u] = (int32_t)(lns[u] >> 16); }
+    } else if (SRC == S_TRACE) {
+        load4<float4, kLast>(a.ttft, i0, a.n, wide, t, 1.0f);
         load4<int4, kLast>(a.prompt, i0, a.n, wide, l, 1);
         if (!AGAIN) load4<int4, kLast>(a.outlen, i0, a.n, wide, o, 1);
         if (a.sp) load4<uchar4, kLast>(a.sp, i0, a.n, wide, sp, (uint8_t)0);
         if (a.dp) load4<uchar4, kLast>(a.dp, i0, a.n, wide, dp, (uint8_t)0);
+    } else {
+        load4<float4, kLast>(a.ttft, i0, a.n, wide, t, 1.0f);
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -139,7 +155,7 @@ __device__ __forceinline__ void read_items(const LoadArgs& a, uint32_t i0, bool 
             if (l[u] < 1 || l[u] > kMaxPrompt) bad = 1;
             else if (o[u] < 1 || o[u] > kMaxOutput) bad = 2;
             else if (!(t[u] > 0.0f) || !(t[u] <= 2000.0f)) bad = 3;      // NaN fails both comparisons
-            else if (SRC == S_TRACE && (sp[u] >= a.ns || dp[u] >= a.nd)) bad = 4;
+            else if (FORM == F_PACKED ? (int)dp[u] >= a.G : SRC == S_TRACE && (sp[u] >= a.ns || dp[u] >= a.nd)) bad = 4;
             if (bad) {
                 if (atomicCAS(&a.z->err[0], 0, bad) == 0) a.z->err[1] = (int32_t)(i0 + u);
                 in = false;
@@ -410,7 +426,7 @@ __device__ __forceinline__ bool sort_dense(SortSmem& sm, const uint32_t* src, ui
     return true;
 }
 
-template <int SRC, bool PRIV, bool STAGE>
+template <int SRC, bool PRIV, int FORM>
 __global__ void __launch_bounds__(kThreads, 1)
 k_load(const __grid_constant__ LoadArgs a) {
     constexpr bool kTrace = SRC == S_TRACE;
@@ -457,7 +473,7 @@ k_load(const __grid_constant__ LoadArgs a) {
 #pragma unroll 1
     for (uint32_t i0 = i_first; i0 < a.n; i0 += stride) {
         Item x[4];
-        read_items<SRC, STAGE, true>(a, i0, wide, s_off, x);
+        read_items<SRC, FORM, true>(a, i0, wide, s_off, x);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const Item& y = x[u];
@@ -479,7 +495,7 @@ k_load(const __grid_constant__ LoadArgs a) {
                 }
             }
         }
-        if (STAGE) {                                                   // (the staging arrays hold whole vectors)
+        if (FORM == F_STAGE) {                                                   // (the staging arrays hold whole vectors)
             *reinterpret_cast<uint4*>(a.st_ticks + i0) = make_uint4(x[0].S, x[1].S, x[2].S, x[3].S);
             *reinterpret_cast<uint4*>(a.st_ln + i0) = make_uint4(x[0].l | x[0].o << 16, x[1].l | x[1].o << 16, x[2].l | x[2].o << 16, x[3].l | x[3].o << 16);
             *reinterpret_cast<uchar4*>(a.st_g + i0) = make_uchar4((uint8_t)x[0].g, (uint8_t)x[1].g, (uint8_t)x[2].g, (uint8_t)x[3].g);
@@ -581,7 +597,7 @@ k_load(const __grid_constant__ LoadArgs a) {
         for (; i_next < i_end; i_next += stride) {
             const uint32_t i0 = i_next;
             Item x[4];
-            read_items<SRC, STAGE, false>(a, i0, wide, s_off, x);
+            read_items<SRC, FORM, false>(a, i0, wide, s_off, x);
             uint32_t at[4] = {0, 0, 0, 0}, tp[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -616,7 +632,7 @@ k_load(const __grid_constant__ LoadArgs a) {
 #pragma unroll 1
             for (uint32_t i0 = i_next; i0 < i_end; i0 += stride) {
                 Item x[4];
-                read_items<SRC, STAGE, false, true>(a, i0, wide, s_off, x);
+                read_items<SRC, FORM, false, true>(a, i0, wide, s_off, x);
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (x[u].in && DBG_OK(x[u].g, G, DBG_K_GATHER, DBG_GROUP) && DBG_OK(x[u].l, kLens, DBG_K_GATHER, DBG_TABLE)) {
@@ -699,14 +715,14 @@ k_load(const __grid_constant__ LoadArgs a) {
     }
 }
 
-template <int SRC, bool STAGE>
+template <int SRC, int FORM>
 cudaError_t launch_load(const LoadArgs& a, int sms, cudaStream_t st) {
     const bool priv = a.G <= (SRC == S_TRACE ? kPrivateGroups : kPrivateTickGroups);
     const size_t counters = priv ? (size_t)a.G * ((SRC == S_TRACE ? kLens : 0) + kTickBins) * 4 : 0;
     const size_t smem = std::max(counters, sizeof(SortSmem));
     static_assert(kTickBins % 4 == 0 && sizeof(LoadZero) % 16 == 0, "vector loads of the counters");
-    auto* kernel = priv ? k_load<SRC, true, STAGE> : k_load<SRC, false, STAGE>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    auto* kernel = priv ? k_load<SRC, true, FORM> : k_load<SRC, false, FORM>;
+    cudaError_t e = allow_smem((const void*)kernel, 220 * 1024);
     if (e) return e;
     // four requests a thread (and about a window a block) until the multiprocessors are full
     const uint32_t per_block = 4u * kThreads;
@@ -740,10 +756,11 @@ k_tables_imported(const uint32_t* __restrict__ cnt, int64_t* __restrict__ cum, c
 DBG_TRANSLATION_UNIT()
 
 cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st) {
-    return a.st_ticks ? launch_load<S_TRACE, true>(a, sms, st) : launch_load<S_TRACE, false>(a, sms, st);
+    if (a.packed) return launch_load<S_TRACE, F_PACKED>(a, sms, st);
+    return a.st_ticks ? launch_load<S_TRACE, F_STAGE>(a, sms, st) : launch_load<S_TRACE, F_COLUMNS>(a, sms, st);
 }
-cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st) { return launch_load<S_TICKS, false>(a, sms, st); }
-cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st) { return launch_load<S_TTFT, false>(a, sms, st); }
+cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st) { return launch_load<S_TICKS, F_COLUMNS>(a, sms, st); }
+cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st) { return launch_load<S_TTFT, F_COLUMNS>(a, sms, st); }
 
 cudaError_t launch_tables_imported(int G, const uint32_t* cnt, int64_t* cum_mass, const int32_t* F_sorted,
                                    const uint32_t* F_off, int32_t* knots, cudaStream_t st) {

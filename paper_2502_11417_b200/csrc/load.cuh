@@ -37,6 +37,8 @@ struct LoadArgs {
     const int32_t *prompt, *outlen;
     const float* ttft;
     const uint8_t *sp, *dp;               // may be null
+    // ... or packed (pack.cuh) ...
+    const char* packed;
     // ... or ticks stored group after group (off[g] .. off[g + 1])
     const int32_t* ticks;
     const uint32_t* off;

@@ -1,0 +1,54 @@
+// Traces in pageable host memory on their way to the device (pack.cu).
+#pragma once
+
+#include <atomic>
+#include <condition_variable>
+#include <mutex>
+#include <thread>
+#include <vector>
+
+#include "disco_internal.cuh"
+
+namespace disco {
+
+// Packed requests, a chunk of 32,768 after another: lengths (prompt | output << 16), TTFTs, groups (a byte each).  A length
+// or profile out of range is packed as 0 or 255, which the ingestion kernel refuses with the same error.
+constexpr uint32_t kPackChunk = 32768;
+constexpr size_t kPackBytes = (size_t)kPackChunk * 9;
+constexpr uint32_t kPackInPlace = 8192;       // traces up to this size are read from the pinned slot, without a copy
+inline size_t packed_bytes(uint32_t n) { return ((size_t)n + kPackChunk - 1) / kPackChunk * kPackBytes; }
+
+// Packs and copies with a few threads of its own.  One per context: its threads and its page-locked slots live as long.
+class Packer {
+public:
+    Packer() = default;
+    ~Packer();
+    Packer(const Packer&) = delete;
+    Packer& operator=(const Packer&) = delete;
+    // Packs the trace into `dev` (packed_bytes(n) of it) by copies on the stream, or, up to kPackInPlace requests, into
+    // page-locked memory of its own; *at receives where.  Must not be called again before the kernel that reads the result
+    // has run.
+    cudaError_t pack(const disco_trace_desc_t& d, char* dev, cudaStream_t st, const char** at);
+
+private:
+    struct Lane { char* slot[2] = {nullptr, nullptr}; cudaEvent_t free[2] = {nullptr, nullptr}; int next = 0; };
+    cudaError_t open_lane(Lane& l, bool both);
+    cudaError_t work(Lane& l);
+    void run(size_t lane);
+
+    std::vector<Lane> lanes_;                 // the caller's, then the threads'
+    std::vector<std::thread> threads_;
+    std::mutex m_;
+    std::condition_variable wake_, done_;
+    uint64_t job_ = 0;
+    size_t running_ = 0;
+    bool stop_ = false;
+    int device_ = 0;
+    const disco_trace_desc_t* d_ = nullptr;   // the job in work
+    char* dev_ = nullptr;
+    cudaStream_t st_ = nullptr;
+    std::atomic<uint32_t> chunk_{0};
+    std::atomic<int> error_{0};
+};
+
+}  // namespace disco

@@ -582,8 +582,7 @@ cudaError_t launch_pairs_acc(const TraceDev& tr, const GroupConst* gc, const Cla
     while (PL < 32 && (uint32_t)PL < n_list) PL <<= 1;
     auto* acc_kernel = extras ? (wide ? k_pairs_acc<true, true> : k_pairs_acc<true, false>)
                               : (wide ? k_pairs_acc<false, true> : k_pairs_acc<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(acc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)acc_smem_bytes(32));
+    cudaError_t e = allow_smem((const void*)acc_kernel, acc_smem_bytes(32));
     if (e) return e;
     const uint32_t n_tiles = (n_list + PL - 1) / PL;
     if ((uint64_t)n_chunks * n_tiles > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;

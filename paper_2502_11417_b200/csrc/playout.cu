@@ -533,7 +533,7 @@ cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const Clas
         if ((e = launch_playout_free(tr, gc, cc, host_cc, knots, k0, rec, batches[G_FREE], sms, st))) return e;
     if (kinds & (1u << G_GENERAL)) {
         const size_t smem = (size_t)kWarps * (host_cc.W[0] + host_cc.W[1] + host_cc.W[2]) * 4;
-        if ((e = cudaFuncSetAttribute(k_playout, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024))) return e;
+        if ((e = allow_smem((const void*)k_playout, 100 * 1024))) return e;
         const uint32_t blocks = std::min<uint32_t>((batches[G_GENERAL] + kWarps - 1) / kWarps, (uint32_t)sms * 32u);
         return launch_after(k_playout, blocks, kWarps * 32, smem, st, tr, gc, cc, knots, k0, rec, err);
     }

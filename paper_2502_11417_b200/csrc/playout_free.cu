@@ -197,7 +197,7 @@ cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const 
     auto* kernel = host_cc.pacing ? (small ? k_playout_free<false, true> : k_playout_free<false, false>)
                                   : (small ? k_playout_free<true, true> : k_playout_free<true, false>);
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024))) return e;
+    if ((e = allow_smem((const void*)kernel, 227 * 1024))) return e;
     // (batches counts 32 requests each; four blocks of eight warps fit a multiprocessor)
     const uint32_t blocks = std::min<uint32_t>((batches * (32 / kFreeBatch) + warps - 1) / warps, (uint32_t)sms * 4u * kFreeWarps / warps);
     return launch_after(kernel, blocks, warps * 32, smem, st, tr, gc, cc, knots, k0, rec);
