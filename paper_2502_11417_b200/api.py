@@ -421,28 +421,30 @@ class Trace:
         return int(ng)
 
     def group_tables(self, g: int, n_sorted: Optional[int] = None, stream=None):
-        cnt = np.zeros(4097, dtype=np.int64)
-        kn = np.zeros(257, dtype=np.int32)
-        ng = lib().disco_get_group_tables(self._h, g, None, None, None, 0, _stream_ptr(stream))
+        cnt = np.empty(4097, dtype=np.int64)
+        kn = np.empty(257, dtype=np.int32)
+        call, st = lib().disco_get_group_tables, _stream_ptr(stream)
+        ng = call(self._h, g, cnt.ctypes.data, kn.ctypes.data, None, 0, st)
         if ng < 0:
             _check(int(ng))
         k = int(ng) if n_sorted is None else min(int(ng), n_sorted)
-        srt = np.zeros(max(k, 1), dtype=np.int32)
-        rc = lib().disco_get_group_tables(self._h, g, cnt.ctypes.data, kn.ctypes.data, srt.ctypes.data, k,
-                                          _stream_ptr(stream))
-        if rc < 0:
-            _check(int(rc))
-        return cnt, kn, srt[:k]
+        srt = np.empty(k, dtype=np.int32)
+        if k:
+            rc = call(self._h, g, None, None, srt.ctypes.data, k, st)
+            if rc < 0:
+                _check(int(rc))
+        return cnt, kn, srt
 
     def sorted_ticks_device(self, g: int, stream=None):
         """Group g's ascending server-TTFT ticks as a CUDA int32 tensor (a device-to-device copy)."""
-        import torch
-        ng = lib().disco_get_group_tables(self._h, g, None, None, None, 0, _stream_ptr(stream))
+        torch = _t()
+        call, st = lib().disco_get_group_tables, _stream_ptr(stream)
+        ng = call(self._h, g, None, None, None, 0, st)
         if ng < 0:
             _check(int(ng))
         out = torch.empty(int(ng), dtype=torch.int32, device="cuda")
         if ng:
-            rc = lib().disco_get_group_tables(self._h, g, None, None, out.data_ptr(), int(ng), _stream_ptr(stream))
+            rc = call(self._h, g, None, None, out.data_ptr(), int(ng), st)
             if rc < 0:
                 _check(int(rc))
         return out

@@ -152,6 +152,9 @@ struct disco_ctx {
     size_t stage_cap = 0;
     cudaEvent_t stage_free = nullptr;
     int32_t* sel_host = nullptr; // [2], in the pinned block of rb
+    uint32_t* tab_host = nullptr;   // pinned copy of the group tables: [G][4097] length counts, then [G][257] knots
+    int tab_host_groups = 0;        // groups it has room for
+    bool tab_host_now = false;      // it holds the current tables
     void* stats_host = nullptr;  // pinned mirror of the statistics
     size_t stats_host_cap = 0;
     bool timing = false;         // record events around the play-out and pair kernels
@@ -164,6 +167,7 @@ struct disco_ctx {
         for (DevBuf* b : all) b->release();
         if (rb) cudaFreeHost(rb);
         if (stage) cudaFreeHost(stage);
+        if (tab_host) cudaFreeHost(tab_host);
         if (stats_host) cudaFreeHost(stats_host);
         if (stage_free) cudaEventDestroy(stage_free);
         for (auto& e : ev) if (e) cudaEventDestroy(e);
@@ -252,6 +256,36 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     return c->d_gc.reserve((size_t)kMaxGroups * sizeof(GroupConst));
 }
 
+// The pinned copy of the group tables; fetch_knots brings the knots alone (copies queued on the stream).
+constexpr size_t kLengths = kMaxPrompt + 1;
+int32_t* host_knots(disco_ctx* c, int g) { return (int32_t*)c->tab_host + c->G * kLengths + (size_t)g * kNKnots; }
+int reserve_tab_host(disco_ctx* c) {
+    if (c->tab_host_groups >= c->G) return 0;
+    if (c->tab_host) cudaFreeHost(c->tab_host);
+    c->tab_host = nullptr; c->tab_host_groups = 0;
+    CU(cudaMallocHost((void**)&c->tab_host, (size_t)c->G * (kLengths + kNKnots) * 4));
+    c->tab_host_groups = c->G;
+    return 0;
+}
+int fetch_knots(disco_ctx* c, cudaStream_t st) {
+    if (int rc = reserve_tab_host(c)) return rc;
+    CU(cudaMemcpyAsync(host_knots(c, 0), c->knots.p, (size_t)c->G * kNKnots * 4, cudaMemcpyDeviceToHost, st));
+    return 0;
+}
+
+// Pinned staging of at least that many bytes, once the copies of an earlier call no longer read it.
+int reserve_stage(disco_ctx* c, size_t bytes) {
+    if (c->stage_free) CU(cudaEventSynchronize(c->stage_free));
+    else CU(cudaEventCreateWithFlags(&c->stage_free, cudaEventDisableTiming));
+    if (bytes > c->stage_cap) {
+        if (c->stage) cudaFreeHost(c->stage);
+        c->stage = nullptr; c->stage_cap = 0;
+        CU(cudaMallocHost(&c->stage, bytes));
+        c->stage_cap = bytes;
+    }
+    return 0;
+}
+
 // The fallback sort: ticks stored group after group (off: [G + 1], device memory) ascending within each group into out.
 int radix_sort(disco_ctx* c, const int32_t* ticks, const uint32_t* off, uint32_t total, int32_t* out, cudaStream_t st) {
     cudaError_t e;
@@ -296,7 +330,7 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     c->loaded = c->evaluated = c->reduced = false;
     c->n = (uint32_t)d->n; c->ns = d->n_servers; c->nd = d->n_devices; c->G = (int)gc.size(); c->gc = gc;
     c->first_index = d->first_index;
-    c->tables_imported = false;
+    c->tables_imported = c->tab_host_now = false;
     c->fin_imported = false;
     if (!c->sms) {
         int dev = 0;
@@ -390,11 +424,10 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         if ((e = launch_tables_imported(c->G, c->cnt, c->cum_mass.as<int64_t>(), c->sorted.as<int32_t>(), c->grp_off.as<uint32_t>(),
                                         c->knots.as<int32_t>(), st)) != cudaSuccess) return bail(fail_cuda(e, "group tables"));
         g_launches += 1;
-        for (int g = 0; g < c->G; ++g)
-            if (rb->ng[g] && (e = cudaMemcpyAsync(&rb->knot_max[g], c->sorted.as<int32_t>() + rb->grp_off[g + 1] - 1, 4,
-                                                  cudaMemcpyDeviceToHost, st)) != cudaSuccess) return bail(fail_cuda(e, "group tables"));
+        if (int rc = fetch_knots(c, st)) return bail(rc);
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion"));
         if (int rc = debug_check()) return bail(rc);
+        for (int g = 0; g < c->G; ++g) rb->knot_max[g] = host_knots(c, g)[kNKnots - 1];      // (the last knot is the largest tick)
     }
     c->F_sorted = c->sorted.as<int32_t>(); c->F_off = c->grp_off.as<uint32_t>();
     c->F_n.assign(rb->ng, rb->ng + c->G);
@@ -732,14 +765,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     CU(cudaMemsetAsync(mem, 0, clear_bytes, st));
 
     // ---- small tables to the device through pinned staging: one staging block, one copy (16-byte aligned regions)
-    if (c->stage_free) CU(cudaEventSynchronize(c->stage_free));     // an earlier call's copies may still read it
-    else CU(cudaEventCreateWithFlags(&c->stage_free, cudaEventDisableTiming));
-    if (table_bytes > c->stage_cap) {
-        if (c->stage) cudaFreeHost(c->stage);
-        c->stage = nullptr; c->stage_cap = 0;
-        CU(cudaMallocHost(&c->stage, table_bytes));
-        c->stage_cap = table_bytes;
-    }
+    if (int rc = reserve_stage(c, table_bytes)) return rc;
     char *sp = (char*)c->stage, *dt = mem + o_tables;
     size_t off = 0;
     auto put = [&](const void* src, size_t bytes) {
@@ -763,7 +789,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     g_launches += 1;
     if (any_beta) {
         CU(launch_prep_beta(d_pol, P, G, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
-                            c->F_off, c->d_prep.as<Prep>(), st));
+                            c->F_off, c->tick_start.as<uint32_t>(), c->tick_cnt, c->d_prep.as<Prep>(), st));
         g_launches += 1;
     }
 
@@ -988,16 +1014,27 @@ int64_t disco_get_group_tables(disco_ctx_t* c, uint32_t g, int64_t* cnt, int32_t
     const uint64_t ng = c->F_n[g];
     uint64_t off = c->rb->grp_off[g];
     if (c->tables_imported) { off = 0; for (uint32_t k = 0; k < g; ++k) off += c->F_n[k]; }
-    if (cnt) {
-        std::vector<uint32_t> tmp(kMaxPrompt + 1);
-        CU(cudaMemcpyAsync(tmp.data(), c->cnt + (size_t)g * (kMaxPrompt + 1), tmp.size() * 4, cudaMemcpyDeviceToHost, st));
-        CU(cudaStreamSynchronize(st));
-        for (size_t i = 0; i < tmp.size(); ++i) cnt[i] = tmp[i];
+    // The length counts and knots of all groups come over together, with the first group's that is asked for after a load;
+    // those of the others are then read from the copy.
+    bool knots_on_host = true;
+    if (knots) {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, knots) != cudaSuccess) cudaGetLastError();
+        else knots_on_host = attr.type == cudaMemoryTypeHost || attr.type == cudaMemoryTypeUnregistered;
     }
-    if (knots) CU(cudaMemcpyAsync(knots, c->knots.as<int32_t>() + (size_t)g * kNKnots, kNKnots * 4, cudaMemcpyDefault, st));
+    const bool fetch = (cnt || (knots && knots_on_host)) && !c->tab_host_now;
+    if (fetch) {
+        if (int rc = fetch_knots(c, st)) return rc;
+        CU(cudaMemcpyAsync(c->tab_host, c->cnt, (size_t)c->G * kLengths * 4, cudaMemcpyDeviceToHost, st));
+    }
+    if (knots && !knots_on_host)
+        CU(cudaMemcpyAsync(knots, c->knots.as<int32_t>() + (size_t)g * kNKnots, kNKnots * 4, cudaMemcpyDefault, st));
     const uint64_t k = std::min<uint64_t>(n_sorted, ng);
     if (sorted_ticks && k) CU(cudaMemcpyAsync(sorted_ticks, c->F_sorted + off, k * 4, cudaMemcpyDefault, st));
     CU(cudaStreamSynchronize(st));
+    if (fetch) c->tab_host_now = true;
+    if (cnt) for (size_t i = 0; i < kLengths; ++i) cnt[i] = c->tab_host[g * kLengths + i];
+    if (knots && knots_on_host) std::memcpy(knots, host_knots(c, (int)g), kNKnots * 4);
     return (int64_t)ng;
 }
 
@@ -1007,18 +1044,21 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     if (!c->loaded) return fail(DISCO_EINVAL, "no trace loaded");
     cudaStream_t st = (cudaStream_t)stream;
     const int G = c->G;
-    const size_t L = kMaxPrompt + 1;
+    const size_t L = kLengths;
     uint64_t total = 0;
-    std::vector<uint32_t> off(G + 1, 0), cnt32((size_t)G * L);
+    if (int rc = reserve_stage(c, ((size_t)G * L + kMaxGroups + 1) * 4)) return rc;
+    uint32_t *cnt32 = (uint32_t*)c->stage, *off = cnt32 + (size_t)G * L;      // counts of all groups, then the groups' offsets
+    off[0] = 0;
     for (int g = 0; g < G; ++g) {
-        uint64_t by_length = 0;
+        const int64_t* from = cnt + (size_t)g * L;
+        uint64_t by_length = 0, high = 0;
         for (size_t l = 0; l < L; ++l) {
-            const int64_t v = cnt[(size_t)g * L + l];
-            if (v < 0 || v > 0xFFFFFFFFll || (l == 0 && v != 0))
-                return fail(DISCO_EINVAL, "length count negative, above 2^32 - 1 or at length 0 (group " + std::to_string(g) + ")");
-            by_length += (uint64_t)v;
+            const uint64_t v = (uint64_t)from[l];
+            high |= v >> 32; by_length += v;
             cnt32[(size_t)g * L + l] = (uint32_t)v;
         }
+        if (high || from[0] != 0)
+            return fail(DISCO_EINVAL, "length count negative, above 2^32 - 1 or at length 0 (group " + std::to_string(g) + ")");
         if (by_length != n_ticks[g])
             return fail(DISCO_EINVAL, "length counts do not add up to the number of TTFT ticks (group " + std::to_string(g) + ")");
         total += n_ticks[g];
@@ -1032,28 +1072,36 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     if ((e = c->F_sorted_imp.reserve(T1 * 4)) != cudaSuccess || (e = c->F_off_imp.reserve((size_t)(kMaxGroups + 1) * 4)) != cudaSuccess ||
         (e = c->sort_in.reserve(2 * ((T1 + 3) / 4 * 4) * 4 + (size_t)sort_windows((uint32_t)total, G) * 8)) != cudaSuccess)
         return fail_cuda(e, "device allocation for the tables");
-    int32_t* in = c->sort_in.as<int32_t>();                           // the ticks, the same by bin, the windows
+    // ticks in device memory are read where they are; sort_in: a copy of others, the same by bin, the windows
+    bool on_device = false;
+    if (total) {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, ticks) != cudaSuccess) cudaGetLastError();
+        else on_device = attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
+    }
+    int32_t* copy = c->sort_in.as<int32_t>();
+    const int32_t* in = on_device ? ticks : copy;
     const size_t T4 = (T1 + 3) / 4 * 4, win_bytes = (size_t)sort_windows((uint32_t)total, G) * 8;
     CU(cudaMemsetAsync(c->z, 0, sizeof(LoadZero) + tick_bytes, st));
-    if (total) CU(cudaMemcpyAsync(in, ticks, (size_t)total * 4, cudaMemcpyDefault, st));
-    CU(cudaMemcpyAsync(c->F_off_imp.p, off.data(), (size_t)(G + 1) * 4, cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(c->cnt, cnt32.data(), cnt32.size() * 4, cudaMemcpyHostToDevice, st));
+    if (total && !on_device) CU(cudaMemcpyAsync(copy, ticks, (size_t)total * 4, cudaMemcpyDefault, st));
+    CU(cudaMemcpyAsync(c->F_off_imp.p, off, (size_t)(G + 1) * 4, cudaMemcpyHostToDevice, st));
+    CU(cudaMemcpyAsync(c->cnt, cnt32, (size_t)G * L * 4, cudaMemcpyHostToDevice, st));
+    CU(cudaEventRecord(c->stage_free, st));
+    c->tab_host_now = false;
     LoadArgs a = {};
     a.n = (uint32_t)total; a.G = G; a.ticks = in; a.off = c->F_off_imp.as<uint32_t>();
     a.z = c->z; a.tick_cnt = c->tick_cnt; a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)G * kTickBins;
-    a.binned = (uint32_t*)in + T4; a.windows = (uint2*)(in + 2 * T4); a.rounds = 1; a.sorted = c->F_sorted_imp.as<int32_t>();
+    a.binned = (uint32_t*)copy + T4; a.windows = (uint2*)(copy + 2 * T4); a.rounds = 1; a.sorted = c->F_sorted_imp.as<int32_t>();
     CU(cudaMemsetAsync(a.windows, 0, win_bytes, st));
     if (total) { CU(run_sort_ticks(a, c->sms, st)); g_launches += 1; }
     CU(launch_tables_imported(G, c->cnt, c->cum_mass.as<int64_t>(), c->F_sorted_imp.as<int32_t>(), c->F_off_imp.as<uint32_t>(),
                               c->knots.as<int32_t>(), st));
     g_launches += 1;
-    // error word and each group's largest tick (the largest hand-off latency a draw from F can give)
-    int32_t err_host[4] = {0, 0, 0, 0};
-    std::vector<int32_t> top(G, 0);
+    // error word and each group's largest tick, the last of its knots (the largest hand-off latency a draw from F can give)
+    if (int rc = fetch_knots(c, st)) return rc;
+    int32_t* err_host = c->rb->err;
     CU(cudaMemcpyAsync(err_host, c->err, 16, cudaMemcpyDeviceToHost, st));
-    for (int g = 0; g < G; ++g)
-        if (n_ticks[g]) CU(cudaMemcpyAsync(&top[g], c->F_sorted_imp.as<int32_t>() + off[g + 1] - 1, 4, cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));          // the host vectors above are read by the copies until here
+    CU(cudaStreamSynchronize(st));
     if (int rc = debug_check()) { c->loaded = false; return rc; }
     c->evaluated = c->reduced = false;
     if (err_host[3] == 2) { c->loaded = false; return fail(DISCO_ECUDA, "internal error: the blocks of the sort lost each other"); }
@@ -1062,8 +1110,7 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
         CU(launch_tables_imported(G, c->cnt, c->cum_mass.as<int64_t>(), c->F_sorted_imp.as<int32_t>(), c->F_off_imp.as<uint32_t>(),
                                   c->knots.as<int32_t>(), st));
         g_launches += 1;
-        for (int g = 0; g < G; ++g)
-            if (n_ticks[g]) CU(cudaMemcpyAsync(&top[g], c->F_sorted_imp.as<int32_t>() + off[g + 1] - 1, 4, cudaMemcpyDeviceToHost, st));
+        if (int rc = fetch_knots(c, st)) return rc;
         CU(cudaStreamSynchronize(st));
         if (int rc = debug_check()) { c->loaded = false; return rc; }
     }
@@ -1073,7 +1120,7 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     }
     c->F_sorted = c->F_sorted_imp.as<int32_t>(); c->F_off = c->F_off_imp.as<uint32_t>();
     c->tables_imported = true;
-    for (int g = 0; g < G; ++g) { c->F_n[g] = n_ticks[g]; c->rb->knot_max[g] = top[g]; }
+    for (int g = 0; g < G; ++g) { c->F_n[g] = n_ticks[g]; c->rb->knot_max[g] = host_knots(c, g)[kNKnots - 1]; }
     return 0;
 }
 

@@ -222,7 +222,9 @@ cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupCo
                         const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep,
                         cudaStream_t st);
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, int G, const int64_t* cum_mass, const uint32_t* cnt,
-                             const int32_t* sorted, const uint32_t* grp_off, Prep* prep, cudaStream_t st);
+                             const int32_t* sorted, const uint32_t* grp_off,
+                             const uint32_t* tick_start, const uint32_t* tick_cnt /* [G][kTickBins], of the sorted ticks */,
+                             Prep* prep, cudaStream_t st);
 // Plays every request under one class.  `kinds`: bit k set if some group with requests is of GroupKind k; `batches[k]`:
 // batches of 32 requests of the groups of kind k.
 cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const ClassConst& host_cc,

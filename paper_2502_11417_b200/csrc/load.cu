@@ -42,9 +42,6 @@ constexpr int kPrivateTickGroups = 16;    // the same, counters of tick bins alo
 enum Source { S_TRACE, S_TICKS, S_TTFT };
 enum Form { F_COLUMNS, F_STAGE, F_PACKED };   // a trace's columns; the same, with a copy left for the second pass; packed
 
-__device__ __forceinline__ int tick_bin(uint32_t t) {
-    return t < 128u ? (int)t : (int)(__float_as_uint(__uint2float_rz(t)) >> 16) - ((127 + 7) << 7) + 128;
-}
 __device__ __forceinline__ uint32_t tick_bin_edge(int b) {     // smallest ticks of the bin (2^31 behind the last)
     return b < 128 ? (uint32_t)b : (uint32_t)(128 + (b & 127)) << ((b >> 7) - 1);
 }

@@ -7,6 +7,11 @@ namespace disco {
 
 // Ticks fall into 3,200 bins a group: their value below 128, then 128 bins an octave up to 2^31.
 constexpr int kTickBins = 128 + 24 * 128;
+#ifdef __CUDACC__
+__device__ __forceinline__ int tick_bin(uint32_t t) {
+    return t < 128u ? (int)t : (int)(__float_as_uint(__uint2float_rz(t)) >> 16) - ((127 + 7) << 7) + 128;
+}
+#endif
 
 struct LoadReadback {            // what the host needs after a load; pinned host memory, written by the kernel
     int32_t err[4];

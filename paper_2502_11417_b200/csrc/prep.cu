@@ -1,13 +1,16 @@
 // Policy preparation: Algorithms 1-3 for every (group, policy).
-#include "disco_internal.cuh"
+#include "load.cuh"
 
 namespace disco {
 
 namespace {
 
+constexpr uint32_t FULL = 0xFFFFFFFFu;
+
 // ------------------------------------------------------------------------------------------------------
-// Algorithms 1-3, one thread per (group, policy).  All fp64 steps use explicit round-to-nearest
-// operations so that no multiply-add is contracted.
+// Algorithms 1-3, one warp per (group, policy).  All fp64 steps use explicit round-to-nearest
+// operations so that no multiply-add is contracted.  Bound: the latency of a dozen dependent loads.  (A thread per pair
+// with fifteen probes a round took 10 us for one policy and 23 us where the lanes of a warp held groups of both kinds.)
 // ------------------------------------------------------------------------------------------------------
 __device__ int32_t inverse_cdf(const int32_t* sorted, uint32_t N, double q) {
     if (N == 0) return 0;
@@ -19,36 +22,32 @@ __device__ int32_t inverse_cdf(const int32_t* sorted, uint32_t N, double q) {
 }
 
 // Smallest x in [lo, hi) with pred(x), or hi if there is none; pred is false up to some point and true from
-// there on.  Fifteen probes a round instead of one: the probes of a round are independent loads, so the search
-// over the 4098 cumulative masses takes four rounds of memory latency instead of thirteen.
+// there on.  The lanes probe 32 places a round: the search over the 4098 cumulative masses takes three rounds.
 template <class F>
 __device__ __forceinline__ int first_true(int lo, int hi, F pred) {
-    while (hi - lo > 16) {
-        const int step = (hi - lo + 15) >> 4;
-        bool f[15];
-#pragma unroll
-        for (int k = 0; k < 15; ++k) { const int x = lo + (k + 1) * step; f[k] = x < hi ? pred(x) : true; }
-        int k0 = 15;                                                  // first probe that holds
-#pragma unroll
-        for (int k = 14; k >= 0; --k) if (f[k]) k0 = k;
-        const int nlo = k0 == 0 ? lo : lo + k0 * step + 1;            // the probe before it failed
-        const int nhi = k0 == 15 ? hi : min(hi, lo + (k0 + 1) * step);
-        lo = nlo; hi = nhi;
+    const int lane = threadIdx.x & 31;
+    while (hi > lo) {
+        const int step = (hi - lo + 31) >> 5;                         // the last places of 32 pieces
+        const int x = min(lo + (lane + 1) * step, hi) - 1;
+        const uint32_t holds = __ballot_sync(FULL, pred(x));
+        if (holds == 0u) return hi;
+        const int k = __ffs(holds) - 1;                               // the answer lies in piece k
+        hi = min(lo + (k + 1) * step, hi) - 1;                        // ... or is its last place
+        lo += k * step;
+        if (step == 1) return lo;
     }
-    bool f[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) { const int x = lo + k; f[k] = x < hi ? pred(x) : true; }
-    int k0 = 16;
-#pragma unroll
-    for (int k = 15; k >= 0; --k) if (f[k]) k0 = k;
-    return min(lo + k0, hi);
+    return lo;
 }
 
-__global__ void k_prep(const PolicyConst* __restrict__ pol, uint32_t P, int G, const GroupConst* __restrict__ gc,
+constexpr int kPrepThreads = 128;
+
+__global__ void __launch_bounds__(kPrepThreads)
+k_prep(const PolicyConst* __restrict__ pol, uint32_t P, int G, const GroupConst* __restrict__ gc,
                        const int64_t* __restrict__ cum_mass, const uint32_t* __restrict__ cnt,
                        const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
                        Prep* __restrict__ prep) {
-    const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dependency_wait();
+    const uint32_t idx = (blockIdx.x * kPrepThreads + threadIdx.x) >> 5;
     if (idx >= P * (uint32_t)G) return;
     const int g = (int)(idx / P);
     const uint32_t p = idx % P;
@@ -99,64 +98,124 @@ __global__ void k_prep(const PolicyConst* __restrict__ pol, uint32_t P, int G, c
             }
         }
     }
-    prep[(size_t)g * P + p] = r;
+    if ((threadIdx.x & 31) == 0) prep[(size_t)g * P + p] = r;
 }
 
 // Eq. 1-2 variant of phase 2, one block per (group, policy): the smallest whole slope beta (ticks per prompt
 // token) with  sum_l l cnt[l] #{S > w(l)} <= b Total N,  w(l) = 0 for l <= l_immediate, min(beta l, w_tail) above.
-// The sum is exact (it is below Total N < 2^63); it does not grow with beta, so beta is found by bisection.
-__global__ void __launch_bounds__(256)
+// The sum is exact (it is below Total N < 2^63); it does not grow with beta, so beta is found by search: three slopes a
+// round, which cut the range to a quarter.  A thread keeps four prompt lengths and, for each, the two positions in the
+// sorted ticks that belong to the ends of the range, between which the positions of the slopes in between lie; the first
+// and last positions come from the bins' starts in shared memory.  Bound: latency (two barriers and a few dependent loads a
+// round, eleven rounds).  (A bisection whose every step searched all the ticks for every length: 437 us.)
+constexpr int kBetaThreads = 1024;
+constexpr int kBetaLens = kMaxPrompt / kBetaThreads;                  // prompt lengths a thread has
+static_assert(kBetaLens * kBetaThreads == kMaxPrompt, "lengths 1 .. 4096");
+
+__global__ void __launch_bounds__(kBetaThreads)
 k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __restrict__ cum_mass,
             const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
-            Prep* __restrict__ prep) {
-    __shared__ long long part[8];
-    __shared__ long long total_s;
+            const uint32_t* __restrict__ tick_start, const uint32_t* __restrict__ tick_cnt, Prep* __restrict__ prep) {
+    __shared__ uint32_t s_end[kTickBins];                             // ticks of the group up to the bin's last
+    __shared__ long long part[3][32];
+    grid_dependency_wait();
     const int g = (int)(blockIdx.x / P);
     const uint32_t p = blockIdx.x % P;
     Prep& out = prep[(size_t)g * P + p];
     const Prep pr = out;
     const PolicyConst pc = pol[p];
     if (!pr.beta_rule || !pr.device_constrained || (double)pc.budget <= (double)pc.alpha) return;   // block-uniform
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const uint32_t off = grp_off[g], N = grp_off[g + 1] - off;
     const int32_t* srt = sorted + off;
-    const uint32_t* c = cnt + (size_t)g * (kMaxPrompt + 1);
     const double Total = (double)cum_mass[(size_t)g * (kMaxPrompt + 2) + kMaxPrompt + 1];
     const double limit = __dmul_rn(__dmul_rn((double)pc.budget, Total), (double)N);
     const long long w_tail = pr.w_tail, l_imm = pr.l_star;
+    for (int k = threadIdx.x; k < kTickBins; k += kBetaThreads)
+        s_end[k] = tick_start[(size_t)g * kTickBins + k] + tick_cnt[(size_t)g * kTickBins + k] - off;
+    __syncthreads();
 
-    auto started_tokens = [&](long long beta) -> long long {
-        long long acc = 0;
-        for (int l = 1 + (int)threadIdx.x; l <= kMaxPrompt; l += 256) {
-            const uint32_t k = c[l];
-            if (k == 0) continue;
-            const long long w = l <= l_imm ? 0 : min(beta * (long long)l, w_tail);
-            uint32_t lo = 0, hi = N;                                  // requests with S <= w
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (!DBG_OK(mid, N, DBG_K_PREP, DBG_ELEMENT)) break;
-                if ((long long)srt[mid] <= w) lo = mid + 1; else hi = mid;
-            }
-            acc += (long long)l * (long long)k * (long long)(N - lo);
+    // ticks at or below w, known to be between lo and hi of them
+    auto position = [&](long long w, uint32_t lo, uint32_t hi) {
+        if (lo < hi) {
+            const int bin = tick_bin((uint32_t)w);
+            if (bin > 0) lo = max(lo, s_end[bin - 1]);
+            hi = min(hi, s_end[bin]);
         }
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (!DBG_OK(mid, N, DBG_K_PREP, DBG_ELEMENT)) break;
+            if ((long long)srt[mid] <= w) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    };
+    uint32_t k[kBetaLens], at_lo[kBetaLens], at_hi[kBetaLens];        // requests of the length; positions at the range's ends
+    int len[kBetaLens];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+    for (int i = 0; i < kBetaLens; ++i) {
+        len[i] = 1 + (int)threadIdx.x + i * kBetaThreads;
+        k[i] = cnt[(size_t)g * (kMaxPrompt + 1) + len[i]];
+        at_lo[i] = at_hi[i] = 0;
+        if (k[i] == 0) continue;
+        at_lo[i] = position(0, 0u, N);
+        at_hi[i] = len[i] <= l_imm ? at_lo[i] : position(min((w_tail + 1) * (long long)len[i], w_tail), 0u, N);
+    }
+    // the block's sums of three values, the same to all threads
+    auto totals = [&](long long (&v)[3]) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(FULL, v[j], o);
+            if (lane == 0) part[j][wi] = v[j];
+        }
         __syncthreads();
-        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            v[j] = part[j][lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(FULL, v[j], o);
+        }
         __syncthreads();
-        if (threadIdx.x == 0) { long long t = 0; for (int k = 0; k < 8; ++k) t += part[k]; total_s = t; }
-        __syncthreads();
-        return total_s;
     };
     long long lo = 0, hi = w_tail + 1;                                // beyond hi every wait is w_tail
-    if ((double)started_tokens(hi) <= limit) {
-        while (lo < hi) {
-            const long long mid = lo + (hi - lo) / 2;
-            if ((double)started_tokens(mid) <= limit) hi = mid; else lo = mid + 1;
+    {
+        long long v[3] = {0, 0, 0};                                   // device's tokens at the range's ends
+#pragma unroll
+        for (int i = 0; i < kBetaLens; ++i) {
+            v[0] += (long long)len[i] * (long long)k[i] * (long long)(N - at_lo[i]);
+            v[1] += (long long)len[i] * (long long)k[i] * (long long)(N - at_hi[i]);
         }
-    } else {
-        lo = hi;                                                      // not even the longest waits fit
+        totals(v);
+        if ((double)v[0] <= limit) hi = lo;                           // (no waits at all fit)
+        else if ((double)v[1] > limit) lo = hi;                       // not even the longest waits fit
     }
-    if (threadIdx.x == 0) out.w_star = (int32_t)lo;
+    // the slope at lo is too small, that at hi fits
+    while (hi - lo > 1) {
+        const long long d = hi - lo;
+        const long long m[3] = {lo + (d + 3) / 4, lo + (d + 1) / 2, lo + (3 * d + 3) / 4};     // (ascending, above lo, at most hi)
+        uint32_t at[3][kBetaLens];
+        long long v[3] = {0, 0, 0};
+#pragma unroll
+        for (int i = 0; i < kBetaLens; ++i) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                at[j][i] = at_lo[i];
+                if (k[i] != 0 && at_lo[i] < at_hi[i]) at[j][i] = position(min(m[j] * (long long)len[i], w_tail), at_lo[i], at_hi[i]);
+                v[j] += (long long)len[i] * (long long)k[i] * (long long)(N - at[j][i]);
+            }
+        }
+        totals(v);
+        const int fit = (double)v[0] <= limit ? 0 : (double)v[1] <= limit ? 1 : (double)v[2] <= limit ? 2 : 3;   // first slope that fits
+        const long long old_lo = lo;
+        lo = fit == 0 ? old_lo : fit == 1 ? m[0] : fit == 2 ? m[1] : m[2];
+        hi = fit == 0 ? m[0] : fit == 1 ? m[1] : fit == 2 ? m[2] : hi;
+#pragma unroll
+        for (int i = 0; i < kBetaLens; ++i) {
+            if (fit < 3) at_hi[i] = fit == 0 ? at[0][i] : fit == 1 ? at[1][i] : at[2][i];
+            if (fit > 0) at_lo[i] = fit == 1 ? at[0][i] : fit == 2 ? at[1][i] : at[2][i];
+        }
+    }
+    if (threadIdx.x == 0) out.w_star = (int32_t)hi;
 }
 
 }  // namespace
@@ -166,15 +225,16 @@ DBG_TRANSLATION_UNIT()
 cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupConst* gc, const int64_t* cum_mass,
                         const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep,
                         cudaStream_t st) {
-    const uint32_t total = P * (uint32_t)G;
-    k_prep<<<(total + 127) / 128, 128, 0, st>>>(pol, P, G, gc, cum_mass, cnt, sorted, grp_off, prep);
-    return cudaGetLastError();
+    const uint32_t per = kPrepThreads / 32;
+    return launch_after(k_prep, (P * (uint32_t)G + per - 1) / per, kPrepThreads, 0, st, pol, P, G, gc, cum_mass, cnt, sorted,
+                        grp_off, prep);
 }
 
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, int G, const int64_t* cum_mass, const uint32_t* cnt,
-                             const int32_t* sorted, const uint32_t* grp_off, Prep* prep, cudaStream_t st) {
-    k_prep_beta<<<P * (uint32_t)G, 256, 0, st>>>(pol, P, cum_mass, cnt, sorted, grp_off, prep);
-    return cudaGetLastError();
+                             const int32_t* sorted, const uint32_t* grp_off, const uint32_t* tick_start,
+                             const uint32_t* tick_cnt, Prep* prep, cudaStream_t st) {
+    return launch_after(k_prep_beta, P * (uint32_t)G, kBetaThreads, 0, st, pol, P, cum_mass, cnt, sorted, grp_off, tick_start,
+                        tick_cnt, prep);
 }
 
 }  // namespace disco

@@ -77,3 +77,24 @@ def test_groups_whose_counters_fit_a_block_or_do_not(shape, where):
         for f in ("prompt_len", "output_len", "server_ttft_s", "server_profile", "device_profile"):
             setattr(w, f, torch.from_numpy(getattr(w, f)).pin_memory().numpy())
     full_parity(w, [synth.policy(b) for b in synth.budget_grid(9)], tag=f"{shape} groups")
+
+
+@pytest.mark.parametrize("kind", ["spread", "ties", "dense", "wide"])
+@pytest.mark.parametrize("n", [1, 2, 700, 40000])
+def test_linear_wait_rule_on_samples(kind, n):
+    # the slope of Eq. 1-2 is searched between positions in the sorted ticks: one tick, equal ticks, crowded bins
+    rng = np.random.default_rng(n + 5)
+    w = synth.tiny_workload(95, n, max_prompt=4096, max_out=20, device_dearer=True)
+    w.server_ttft_s = np.clip(_sample(kind, n, rng) / (4.0 if kind == "wide" else 1.0), 1e-6, 500.0).astype(np.float32)
+    flags = PACED | synth.FLAG_BETA_RULE | synth.MODE_DEVICE_CONSTRAINED
+    pols = [synth.policy(b, flags=flags, l_immediate=li) for b in (0.0, 0.06, 0.3, 0.9, 1.0) for li in (0, 100, 4096)]
+    if n <= 700:
+        full_parity(w, pols, select=False, tag=f"{kind} {n}")
+        return
+    from oracle import Oracle
+    from paper_2502_11417_b200 import Trace
+    from parity import check_prep
+    tr = Trace.from_workload(w)
+    tr.eval_policies(pols, 1)
+    check_prep(tr, Oracle.from_workload(w), pols, f"{kind} {n}")
+    tr.close()
