@@ -85,6 +85,8 @@ PAIR_FIELDS = [("ttft_s", "float32"), ("tbt_mean_s", "float32"), ("tbt_max_s", "
                ("tok_server", "uint32"), ("tok_device", "uint32"), ("mig_at", "uint32"), ("delayed", "uint16"),
                ("decision", "uint8")]
 
+_I32, _F32, _U8 = np.dtype(np.int32), np.dtype(np.float32), np.dtype(np.uint8)
+
 _lib = None
 
 
@@ -142,19 +144,37 @@ def _check(rc: int, allow=()):
 
 
 _torch = None
+_raw_stream = None      # () -> the current stream of the current device as an integer
 
 
 def _t():
     """torch, imported at the first use of a GPU."""
-    global _torch
+    global _torch, _raw_stream
     if _torch is None:
         import torch
         _torch = torch
+        get, dev = (getattr(torch._C, f, None) for f in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        if get and dev:                                   # (without the Stream object that torch.cuda builds around it)
+            _raw_stream = lambda: get(dev())              # noqa: E731
+        else:
+            _raw_stream = lambda: torch.cuda.current_stream().cuda_stream   # noqa: E731
     return _torch
 
 
 def _stream_ptr(stream) -> Optional[int]:
-    return (_t().cuda.current_stream() if stream is None else stream).cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        _t()
+    return _raw_stream()
+
+
+def _address(a) -> int:
+    """Where a C-contiguous numpy array's elements lie."""
+    try:
+        return C.addressof(C.c_char.from_buffer(a))       # (a.ctypes.data builds several objects on the way)
+    except (TypeError, ValueError, BufferError):          # read-only or empty
+        return a.ctypes.data
 
 
 _cuda_ok = None
@@ -184,38 +204,53 @@ def _torch_dtype(name):
     return getattr(_t(), name)
 
 
-_SERVER, _DEVICE = struct.Struct("4f"), struct.Struct("7f")
+_SERVER, _DEVICE, _POLICY = struct.Struct("4f"), struct.Struct("7f"), struct.Struct("5f3I")
+_pair_dtype_list = None
+
+
+def _pair_dtypes():
+    """PAIR_FIELDS with torch's dtypes."""
+    global _pair_dtype_list
+    if _pair_dtype_list is None:
+        _pair_dtype_list = [(f, _torch_dtype(dt)) for f, dt in PAIR_FIELDS]
+    return _pair_dtype_list
+
+
+def _fill(arr, layout, rows):
+    """Fills an array of plain structures (struct is several times faster here than setting ctypes fields; what it refuses,
+    such as a number beyond the field's range, is left to ctypes' conversions)."""
+    for k, row in enumerate(rows):
+        try:
+            layout.pack_into(arr, layout.size * k, *row)
+        except (struct.error, OverflowError):
+            arr[k] = type(arr)._type_(*row)
+    return arr
 
 
 def server_array(servers: Sequence[Dict[str, float]]):
-    arr = (ServerProfile * len(servers))()
-    for k, s in enumerate(servers):
-        _SERVER.pack_into(arr, 16 * k, s["tbt_s"], s["jitter"], s["c_prefill"], s["c_decode"])
-    return arr
+    return _fill((ServerProfile * len(servers))(), _SERVER,
+                 [(s["tbt_s"], s["jitter"], s["c_prefill"], s["c_decode"]) for s in servers])
 
 
 def device_array(devices: Sequence[Dict[str, float]]):
-    arr = (DeviceProfile * len(devices))()
-    for k, d in enumerate(devices):
-        _DEVICE.pack_into(arr, 28 * k, d["prefill_tps"], d["ttft_intercept_s"], d["decode_tps"], d["jitter"],
-                          d["c_prefill"], d["c_decode"], d["lam"])
-    return arr
+    return _fill((DeviceProfile * len(devices))(), _DEVICE,
+                 [(d["prefill_tps"], d["ttft_intercept_s"], d["decode_tps"], d["jitter"], d["c_prefill"], d["c_decode"],
+                   d["lam"]) for d in devices])
 
 
 def policy_array(policies: Sequence[Dict[str, float]]):
-    arr = (Policy * len(policies))()
-    for k, p in enumerate(policies):
-        arr[k] = Policy(p["budget"], p["alpha"], p["mig_threshold"], p["t_m_s"], p["r_c"], p["flags"],
-                        p.get("expected_len", 0), p.get("l_immediate", 0))
-    return arr
+    return _fill((Policy * len(policies))(), _POLICY,
+                 [(p["budget"], p["alpha"], p["mig_threshold"], p["t_m_s"], p["r_c"], p["flags"], p.get("expected_len", 0),
+                   p.get("l_immediate", 0)) for p in policies])
 
 
 def select_policy(stats, cost_cap: float, tbt_slo_s: float):
     """disco_select_policy over a (PolicyStats * P) array in host memory (the records of reduce_stats, or
     merged ones).  Returns (status, index): status 0, or EINFEASIBLE with the cheapest policy's index."""
     best = C.c_int32(-1)
-    rc = _check(lib().disco_select_policy(C.addressof(stats), len(stats), cost_cap, tbt_slo_s, C.byref(best)),
-                allow=(EINFEASIBLE,))
+    rc = lib().disco_select_policy(C.addressof(stats), len(stats), cost_cap, tbt_slo_s, C.byref(best))
+    if rc != 0:
+        _check(rc, allow=(EINFEASIBLE,))
     return rc, best.value
 
 
@@ -265,16 +300,16 @@ class Trace:
         all of the same kind.  Reloading reuses the context's device memory.  first_index: position of these
         arrays' first request in the whole trace when they are a shard of it.  staged_copy: host arrays are copied
         by the copy engine even when they are page-locked (instead of being read in place by the ingestion kernel)."""
-        torch = _t()
         _require_cuda()
-        on_dev = isinstance(prompt_len, torch.Tensor) and prompt_len.is_cuda
+        torch = _t()
+        on_dev = type(prompt_len) is not np.ndarray and isinstance(prompt_len, torch.Tensor) and prompt_len.is_cuda
         ptrs, keep = [], []
-        for a, want, npdt in ((prompt_len, torch.int32, np.int32), (output_len, torch.int32, np.int32),
-                              (server_ttft_s, torch.float32, np.float32), (server_profile, torch.uint8, np.uint8),
-                              (device_profile, torch.uint8, np.uint8)):
+        for a, want, npdt in ((prompt_len, torch.int32, _I32), (output_len, torch.int32, _I32),
+                              (server_ttft_s, torch.float32, _F32), (server_profile, torch.uint8, _U8),
+                              (device_profile, torch.uint8, _U8)):
             if a is None:
                 ptrs.append(None)
-            elif isinstance(a, torch.Tensor):
+            elif type(a) is not np.ndarray and isinstance(a, torch.Tensor):
                 if a.is_cuda != on_dev:
                     raise ValueError("all trace arrays must live on the same side")
                 if a.dtype != want:
@@ -288,7 +323,7 @@ class Trace:
                     raise ValueError("all trace arrays must live on the same side")
                 x = np.ascontiguousarray(a, dtype=npdt)
                 keep.append(x)
-                ptrs.append(x.__array_interface__["data"][0])
+                ptrs.append(_address(x))
         n = int(len(prompt_len))
         sv, dv = server_array(servers), device_array(devices)
         desc = TraceDesc(n, *ptrs, C.addressof(sv), len(servers), C.addressof(dv), len(devices),
@@ -318,10 +353,10 @@ class Trace:
         if out is not None:
             shape = (P, self.n)
             vals = []
-            for f, dt in PAIR_FIELDS:
+            for f, dt in _pair_dtypes():
                 t = out.get(f)
                 if t is not None:
-                    if not t.is_cuda or t.dtype != _torch_dtype(dt) or t.shape != shape or not t.is_contiguous():
+                    if not t.is_cuda or t.dtype != dt or t.shape != shape or not t.is_contiguous():
                         raise ValueError(f"output '{f}' must be a contiguous CUDA tensor [P, n] of {dt}")
                     t = t.data_ptr()
                 vals.append(t)

@@ -386,7 +386,7 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         a.prompt = d->prompt_len; a.outlen = d->output_len; a.ttft = d->server_ttft_s;
         a.sp = d->server_profile; a.dp = d->device_profile;
     }
-    a.z = c->z; a.cnt = c->cnt; a.tick_cnt = c->tick_cnt;
+    a.z = c->z; a.zero_bytes = c->zero_bytes; a.cnt = c->cnt; a.tick_cnt = c->tick_cnt;
     a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)c->G * kTickBins;
     a.binned = c->binned.as<uint32_t>();
     a.req = c->req.as<uint4>(); a.inv = c->G == 1 ? c->inv.as<uint32_t>() : nullptr; a.sorted = c->sorted.as<int32_t>();
@@ -404,8 +404,7 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         if ((e = cudaMemcpyAsync(c->d_gc.p, c->gc.data(), c->gc.size() * sizeof(GroupConst), cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return bail(fail_cuda(e, "profile copy"));
     }
-    if ((e = cudaMemsetAsync(c->zero.p, 0, c->zero_bytes, st)) != cudaSuccess ||
-        (e = run_load(a, c->sms, st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion kernel"));
+    if ((e = run_load(a, c->sms, st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion kernel"));
     g_launches += 1;
     // the few numbers the host needs (error word, group sizes, longest output, largest TTFT per group) are in rb
     HostReadback* rb = c->rb;
@@ -1081,8 +1080,7 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     }
     int32_t* copy = c->sort_in.as<int32_t>();
     const int32_t* in = on_device ? ticks : copy;
-    const size_t T4 = (T1 + 3) / 4 * 4, win_bytes = (size_t)sort_windows((uint32_t)total, G) * 8;
-    CU(cudaMemsetAsync(c->z, 0, sizeof(LoadZero) + tick_bytes, st));
+    const size_t T4 = (T1 + 3) / 4 * 4;
     if (total && !on_device) CU(cudaMemcpyAsync(copy, ticks, (size_t)total * 4, cudaMemcpyDefault, st));
     CU(cudaMemcpyAsync(c->F_off_imp.p, off, (size_t)(G + 1) * 4, cudaMemcpyHostToDevice, st));
     CU(cudaMemcpyAsync(c->cnt, cnt32, (size_t)G * L * 4, cudaMemcpyHostToDevice, st));
@@ -1090,9 +1088,9 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     c->tab_host_now = false;
     LoadArgs a = {};
     a.n = (uint32_t)total; a.G = G; a.ticks = in; a.off = c->F_off_imp.as<uint32_t>();
-    a.z = c->z; a.tick_cnt = c->tick_cnt; a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)G * kTickBins;
+    a.z = c->z; a.zero_bytes = sizeof(LoadZero) + tick_bytes; a.tick_cnt = c->tick_cnt; a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)G * kTickBins;
     a.binned = (uint32_t*)copy + T4; a.windows = (uint2*)(copy + 2 * T4); a.rounds = 1; a.sorted = c->F_sorted_imp.as<int32_t>();
-    CU(cudaMemsetAsync(a.windows, 0, win_bytes, st));
+    if (!total) CU(cudaMemsetAsync(c->z, 0, sizeof(LoadZero), st));
     if (total) { CU(run_sort_ticks(a, c->sms, st)); g_launches += 1; }
     CU(launch_tables_imported(G, c->cnt, c->cum_mass.as<int64_t>(), c->F_sorted_imp.as<int32_t>(), c->F_off_imp.as<uint32_t>(),
                               c->knots.as<int32_t>(), st));

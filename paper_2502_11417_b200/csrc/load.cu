@@ -7,8 +7,9 @@
 //   1. count: every request is checked and counted by (group, prompt length) and by (group, bin of its ticks), 128 bins an
 //      octave, in counters of the block's own.  The block adds its counters to the global ones and keeps what was there
 //      before: where its own requests of each bucket go within the bucket.
-//   2. place: from the totals every block works out where the buckets start, then sends its requests to their places: one
-//      16-byte record into the internal order and the ticks into their bin.
+//   2. place: the blocks work out where the buckets start, each for its share of the counters (the blocks tell one another
+//      their totals), then every block sends its requests to their places: one 16-byte record into the internal order and
+//      the ticks into their bin.
 //   3. sort: the bins in order, about 4,096 ticks at a time, are sorted in shared memory (all ticks of a window differ in
 //      few low bits), each window by one block.  A bin of more than 8,192 ticks that spans at most 2^18 values is sorted by
 //      counting them; a trace that has a denser and wider one goes to the radix sort (radix.cu) instead.
@@ -60,6 +61,7 @@ static_assert(kCounters == 2 * kSortCap, "the counters lie over the two key arra
 // flag and goes on (the host refuses the results).
 __device__ __forceinline__ void grid_barrier(LoadZero* z, uint32_t times) {
     __syncthreads();
+    if (gridDim.x == 1) return;
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(&z->barrier, 1u);
@@ -164,43 +166,48 @@ __device__ __forceinline__ void read_items(const LoadArgs& a, uint32_t i0, bool 
     }
 }
 
-// Exclusive prefix sums over L counters (16-byte aligned) by the whole block: a warp takes a run of them, sums it up, and
-// goes through it again with the sum of the runs in front (read from L2 both times, four a lane).  emit(k, counts, starts):
-// the counters k .. k + 3, those from L on empty.
+// Waits (boundedly, as above) for a word that another block writes once.
+__device__ __forceinline__ unsigned long long await_word(LoadZero* z, const unsigned long long* at) {
+    unsigned long long v;
+    uint32_t tries = 0;
+    do {
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(at) : "memory");
+    } while (v == 0ull && ++tries < (1u << 22));
+    if (v == 0ull) atomicExch(&z->err[3], 2);
+    return v;
+}
+
+// Four counters from k on (16-byte aligned), those from k1 on empty.
+__device__ __forceinline__ uint4 four_counters(const uint32_t* cnt, int k, int k1) {
+    if (k + 4 <= k1) return __ldcg(reinterpret_cast<const uint4*>(cnt + k));
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (k < k1) v.x = __ldcg(&cnt[k]);
+    if (k + 1 < k1) v.y = __ldcg(&cnt[k + 1]);
+    if (k + 2 < k1) v.z = __ldcg(&cnt[k + 2]);
+    return v;
+}
+
+// A block's share of L counters: [k0, k1), whole vectors.
+struct Share { int k0, k1; };
+__device__ __forceinline__ Share share_of(int L) {
+    const int per = ((L + (int)gridDim.x - 1) / (int)gridDim.x + 3) / 4 * 4;
+    return Share{min(L, (int)blockIdx.x * per), min(L, ((int)blockIdx.x + 1) * per)};
+}
+
+// Exclusive prefix sums over the block's share, `carry` in front of it, four neighbouring counters a thread at a time.
+// emit(k, counts, starts): the counters k .. k + 3.  first: this thread's counters of the first 4,096.
 template <class E>
-__device__ __forceinline__ void scan_counts(const uint32_t* cnt, int L, uint32_t* wtot, E emit) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int per = ((L + 31) / 32 + 127) / 128 * 128, k0 = w * per + lane * 4, k1 = min(L, (w + 1) * per);
-    auto four = [&](int k) {
-        if (k + 4 <= k1) return __ldcg(reinterpret_cast<const uint4*>(cnt + k));
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (k < k1) v.x = __ldcg(&cnt[k]);
-        if (k + 1 < k1) v.y = __ldcg(&cnt[k + 1]);
-        if (k + 2 < k1) v.z = __ldcg(&cnt[k + 2]);
-        return v;
-    };
-    uint32_t sum = 0;
-#pragma unroll 2
-    for (int k = k0; k < k1; k += 128) { const uint4 v = four(k); sum += v.x + v.y + v.z + v.w; }
-    sum = __reduce_add_sync(FULL, sum);
-    if (lane == 0) wtot[w] = sum;
-    __syncthreads();
-    uint32_t run = __reduce_add_sync(FULL, lane < w ? wtot[lane] : 0u);
-#pragma unroll 1
-    for (int k = w * per; k < k1; k += 128) {
-        const uint4 c = four(k + lane * 4);
+__device__ __forceinline__ void scan_share(const uint32_t* cnt, const Share& sh, const uint4& first, uint32_t carry, uint32_t* wtot, E emit) {
+    for (int k0 = sh.k0; k0 < sh.k1; k0 += 4 * kThreads) {
+        const int k = k0 + (int)threadIdx.x * 4;
+        const uint4 c = k0 == sh.k0 ? first : four_counters(cnt, k, sh.k1);
         const uint32_t own = c.x + c.y + c.z + c.w;
-        uint32_t v = own;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t up = __shfl_up_sync(FULL, v, off);
-            if (lane >= off) v += up;
-        }
-        const uint32_t at = run + v - own;
-        if (k + lane * 4 < k1) emit(k + lane * 4, c, make_uint4(at, at + c.x, at + c.x + c.y, at + c.x + c.y + c.z));
-        run += __shfl_sync(FULL, v, 31);
+        uint32_t total;
+        const uint32_t at = carry + block_inclusive_scan(own, wtot, &total) - own;
+        if (k < sh.k1) emit(k, c, make_uint4(at, at + c.x, at + c.x + c.y, at + c.x + c.y + c.z));
+        carry += total;
+        __syncthreads();
     }
-    __syncthreads();
 }
 
 // Cumulative input-token mass cum[L] = sum_{l<L} l cnt[l], L = 0 .. 4097.  All threads call.
@@ -432,7 +439,7 @@ k_load(const __grid_constant__ LoadArgs a) {
     __shared__ unsigned long long s_wide[32];
     __shared__ uint32_t s_wtot[32];
     __shared__ unsigned long long s_sum[kMaxGroups];
-    __shared__ uint32_t s_max, s_item;
+    __shared__ uint32_t s_max, s_item, s_carry[2];
     const int G = a.G, tid = threadIdx.x, lane = tid & 31;
     LoadZero* z = a.z;
     uint32_t* s_tick = (uint32_t*)smem_raw;                            // [G][kTickBins]
@@ -440,7 +447,11 @@ k_load(const __grid_constant__ LoadArgs a) {
     uint32_t waits = 0;
 
     // the block's counters join the global ones; what it finds there is where its own requests go within the bucket
-    auto join = [&](uint32_t* mine, uint32_t* all, int count) {
+    auto join = [&](uint32_t* mine, uint32_t* all, int count, bool store) {
+        if (store) {
+            for (int i = tid; i < count; i += kThreads) { all[i] = mine[i]; mine[i] = 0; }
+            return;
+        }
 #pragma unroll 1
         for (int i0 = tid; i0 < count; i0 += 4 * kThreads) {
             uint32_t c[4];
@@ -454,6 +465,15 @@ k_load(const __grid_constant__ LoadArgs a) {
     };
 
     // ---- 1. count
+    const bool alone = gridDim.x == 1;                                 // then nothing has been cleared, and nothing is shared
+    if (alone) {
+        for (int i = tid; i < (int)(sizeof(LoadZero) / 4); i += kThreads) ((uint32_t*)z)[i] = 0;
+        for (int i = tid; i < (int)sort_windows(a.n, G); i += kThreads) a.windows[i] = make_uint2(0u, 0u);
+        if (!PRIV) {
+            for (int i = tid; i < G * kTickBins; i += kThreads) a.tick_cnt[i] = 0;
+            if (kTrace) for (int i = tid; i < G * kLens; i += kThreads) a.cnt[i] = 0;
+        }
+    }
     if (PRIV) for (int i = tid; i < (kTrace ? G * kLens : 0) + G * kTickBins; i += kThreads) s_tick[i] = 0;
     if (SRC == S_TICKS) for (int g = tid; g <= G; g += kThreads) s_off[g] = a.off[g];
     for (int g = tid; g < G; g += kThreads) s_sum[g] = 0;
@@ -518,54 +538,83 @@ k_load(const __grid_constant__ LoadArgs a) {
         if (tid == 0 && s_max) atomicMax(&z->max_n, s_max);
     }
     if (PRIV) {
-        if (kTrace) join(s_len, a.cnt, G * kLens);
-        join(s_tick, a.tick_cnt, G * kTickBins);
+        if (kTrace) join(s_len, a.cnt, G * kLens, alone);
+        join(s_tick, a.tick_cnt, G * kTickBins, alone);
     }
     grid_barrier(z, ++waits);
 
     // ---- 2. place
-    const int32_t bad = __ldcg(&z->err[0]);
-    // where every bucket starts: the groups one after another, so one running sum over all groups' counters each; the
-    // blocks share the writing of the tables
-    const bool writer = (uint32_t)(tid >> 5) % gridDim.x == blockIdx.x;
+    if (__ldcg(&z->err[0])) {                          // a rejected trace: nothing is placed
+        if (kTrace && blockIdx.x == 0 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
+        return;
+    }
+    // where every bucket starts: the groups one after another, so one running sum over all groups' counters each
     const bool cursors = !PRIV || a.rounds > 1;                        // places are handed out by global cursors
-    scan_counts(a.tick_cnt, G * kTickBins, s_wtot, [&](int k, const uint4& c, const uint4& start) {
-        // (kTickBins is a multiple of four: the four bins belong to one group)
-        if (PRIV) {
+    {
+        const Share st = share_of(G * kTickBins), sl = share_of(kTrace ? G * kLens : 0);
+        const uint4 ft = four_counters(a.tick_cnt, st.k0 + tid * 4, st.k1);
+        const uint4 fl = kTrace ? four_counters(a.cnt, sl.k0 + tid * 4, sl.k1) : make_uint4(0u, 0u, 0u, 0u);
+        if (!alone) {
+            uint32_t sum[2] = {ft.x + ft.y + ft.z + ft.w, fl.x + fl.y + fl.z + fl.w};
+            for (int k = st.k0 + (tid + kThreads) * 4; k < st.k1; k += 4 * kThreads) { const uint4 c = four_counters(a.tick_cnt, k, st.k1); sum[0] += c.x + c.y + c.z + c.w; }
+            if (kTrace) for (int k = sl.k0 + (tid + kThreads) * 4; k < sl.k1; k += 4 * kThreads) { const uint4 c = four_counters(a.cnt, k, sl.k1); sum[1] += c.x + c.y + c.z + c.w; }
+            if (tid < 2) s_carry[tid] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < (kTrace ? 2 : 1); ++j) {
+                const uint32_t v = __reduce_add_sync(FULL, sum[j]);
+                if (lane == 0 && v) atomicAdd(&s_carry[j], v);
+            }
+            __syncthreads();
+            // a warp for each of the two sums: tells the other blocks, and adds up those in front
+            const int j = tid >> 5;
+            if (j < (kTrace ? 2 : 1)) {
+                if (lane == 0)
+                    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&z->part[j][blockIdx.x]), "l"(((unsigned long long)s_carry[j] << 1) | 1ull) : "memory");
+                uint32_t before = 0;
+                for (uint32_t b = lane; b < blockIdx.x; b += 32) before += (uint32_t)(await_word(z, &z->part[j][b]) >> 1);
+                before = __reduce_add_sync(FULL, before);
+                if (lane == 0) s_carry[j] = before;
+            }
+        } else if (tid < 2) s_carry[tid] = 0;
+        __syncthreads();
+        scan_share(a.tick_cnt, st, ft, s_carry[0], s_wtot, [&](int k, const uint4&, const uint4& start) {
+            *reinterpret_cast<uint4*>(a.tick_start + k) = start;
+            if (cursors) *reinterpret_cast<uint4*>(a.tick_at + k) = start;
+        });
+        if (kTrace)
+            scan_share(a.cnt, sl, fl, s_carry[1], s_wtot, [&](int k, const uint4& c, const uint4& start) {
+                const uint32_t cs[4] = {c.x, c.y, c.z, c.w}, at[4] = {start.x, start.y, start.z, start.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k + u < sl.k1) a.len_end[k + u] = cursors ? at[u] : at[u] + cs[u];    // (a cursor ends up where its bucket does)
+            });
+    }
+    grid_barrier(z, ++waits);
+    if (SRC != S_TICKS) for (int g = tid; g <= G; g += kThreads) s_off[g] = g < G ? __ldcg(&a.tick_start[(size_t)g * kTickBins]) : a.n;
+    __syncthreads();
+    if (!cursors) {
+        // The block's counters, places within the buckets so far, become places: a bucket starts where the one in front ends.
+        // (All of them side by side: read one by one where they are needed, the few lines that most requests need keep L2
+        // busy: 48 us instead of 8 for a million.)
+#pragma unroll 4
+        for (int k = tid * 4; k < G * kTickBins; k += 4 * kThreads) {
+            const uint4 start = __ldcg(reinterpret_cast<const uint4*>(a.tick_start + k));
             uint4& mine = *reinterpret_cast<uint4*>(s_tick + k);
             mine = make_uint4(mine.x + start.x, mine.y + start.y, mine.z + start.z, mine.w + start.w);
         }
-        if (SRC != S_TICKS) {
-            if (k % kTickBins == 0) s_off[k / kTickBins] = start.x;
-            if (k == G * kTickBins - 4) s_off[G] = start.w + c.w;
-        }
-        if (writer) {
-            *reinterpret_cast<uint4*>(a.tick_start + k) = start;
-            if (cursors) *reinterpret_cast<uint4*>(a.tick_at + k) = start;
-        }
-    });
-    if (kTrace) {
-        scan_counts(a.cnt, G * kLens, s_wtot, [&](int k, const uint4& c, const uint4& start) {
-            const uint32_t cs[4] = {c.x, c.y, c.z, c.w}, st[4] = {start.x, start.y, start.z, start.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (k + u >= G * kLens) break;
-                if (PRIV) s_len[k + u] += st[u];
-                if (writer) a.len_end[k + u] = cursors ? st[u] : st[u] + cs[u];    // (a cursor ends up where its bucket does)
-            }
-        });
-        for (int g = 0; g < G; ++g)
-            if ((uint32_t)(G - 1 - g) % gridDim.x == gridDim.x - 1 - blockIdx.x)
-                group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
+        if (kTrace)
+#pragma unroll 8
+            for (int k = tid + 1; k < G * kLens; k += kThreads) s_len[k] += __ldcg(&a.len_end[k - 1]);
     }
-    // the windows' first and last bins: a thread a bin of those this block writes
-    if (writer) {
-        const int L = G * kTickBins, w = tid >> 5, per = ((L + 31) / 32 + 127) / 128 * 128;
+    // the windows' first and last bins
+    {
+        const Share st = share_of(G * kTickBins);
 #pragma unroll 1
-        for (int k = w * per + lane; k < min(L, (w + 1) * per); k += 32) {
+        for (int k = st.k0 + tid; k < st.k1; k += kThreads) {
             if (__ldcg(&a.tick_cnt[k]) == 0u) continue;
             const int g = k / kTickBins;
-            uint32_t win = (a.tick_start[k] - s_off[g]) / kWindow;      // (written by this warp)
+            uint32_t win = (__ldcg(&a.tick_start[k]) - s_off[g]) / kWindow;
             for (int h = 0; h < g; ++h) win += (s_off[h + 1] - s_off[h] + kWindow - 1) / kWindow;
             atomicMax(&a.windows[win].x, 0xFFFFFFFFu - (uint32_t)k);
             atomicMax(&a.windows[win].y, (uint32_t)k + 1u);
@@ -584,11 +633,7 @@ k_load(const __grid_constant__ LoadArgs a) {
         for (int k = tid; k < G * kNKnots; k += kThreads)
             if (s_off[k / kNKnots + 1] == s_off[k / kNKnots]) a.knots[k] = 0;
     }
-    if (bad) {                                         // a rejected trace: nothing is placed
-        if (kTrace && blockIdx.x == 0 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
-        return;
-    }
-    if (cursors) grid_barrier(z, ++waits);             // the cursors are complete
+    __syncthreads();
     auto place = [&](uint32_t i_end) {
 #pragma unroll 1
         for (; i_next < i_end; i_next += stride) {
@@ -638,8 +683,8 @@ k_load(const __grid_constant__ LoadArgs a) {
                     }
             }
             __syncthreads();
-            join(s_len, a.len_end, G * kLens);
-            join(s_tick, a.tick_at, G * kTickBins);
+            join(s_len, a.len_end, G * kLens, false);
+            join(s_tick, a.tick_at, G * kTickBins, false);
             __syncthreads();
             place(i_end);
             __syncthreads();
@@ -705,6 +750,9 @@ k_load(const __grid_constant__ LoadArgs a) {
         }
     }
     if (kTrace) {
+        for (int g = 0; g < G; ++g)                                    // (the last blocks have the fewest windows)
+            if ((uint32_t)(G - 1 - g) % gridDim.x == gridDim.x - 1 - blockIdx.x)
+                group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
         // the last block to come here reports the flags
         if (tid == 0) { __threadfence(); s_item = atomicAdd(&z->done, 1u); }
         __syncthreads();
@@ -723,13 +771,19 @@ cudaError_t launch_load(const LoadArgs& a, int sms, cudaStream_t st) {
     if (e) return e;
     // four requests a thread (and about a window a block) until the multiprocessors are full
     const uint32_t per_block = 4u * kThreads;
-    const uint32_t blocks = std::max<uint32_t>(1u, std::min<uint32_t>((a.n + per_block - 1) / per_block, (uint32_t)sms));
+    const uint32_t blocks = std::max<uint32_t>(1u, std::min<uint32_t>((a.n + per_block - 1) / per_block, std::min<uint32_t>((uint32_t)sms, kLoadBlocks)));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = blocks; cfg.blockDim = kThreads; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (blocks > 1) {
+        // (one block clears its words itself and waits for nobody)
+        if ((e = cudaMemsetAsync(a.z, 0, a.zero_bytes, st))) return e;
+        if (((char*)a.windows < (char*)a.z || (char*)a.windows >= (char*)a.z + a.zero_bytes) &&
+            (e = cudaMemsetAsync(a.windows, 0, sort_windows(a.n, a.G) * sizeof(uint2), st))) return e;
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
@@ -831,8 +885,7 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
     a.windows = (uint2*)(a.tick_cnt + kTickBins); a.rounds = 1;
     a.tick_start = (uint32_t*)(base + kNaStartOff);
     a.binned = (uint32_t*)base; a.sorted = sorted_ticks;
-    // the array still holds the previous call's data: flags and counters must start at zero
-    if ((e = cudaMemsetAsync(a.z, 0, kNaZeroBytes, st)) != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
+    a.zero_bytes = kNaZeroBytes;          // the array still holds the previous call's data: flags and counters must start at zero
     // Once a kernel has been queued the shared array is in use: every way out below, failures included, first
     // waits for the stream, so that a caller who retries cannot overlap kernels still writing the array.
     auto fail_after_launch = [&](cudaError_t err_code) {

@@ -23,7 +23,9 @@ struct LoadReadback {            // what the host needs after a load; pinned hos
 };
 
 // Words that a load or a sort must find zero, contiguous.
+constexpr uint32_t kLoadBlocks = 256;     // blocks of the kernel, at most
 struct LoadZero {
+    unsigned long long part[2][kLoadBlocks];      // sums over the blocks' shares of the counters: sum << 1 | 1
     uint64_t grp_sum_n[kMaxGroups];       // output tokens per group
     uint32_t ng[kMaxGroups];              // requests per group
     uint32_t max_n;                       // longest output
@@ -32,7 +34,7 @@ struct LoadZero {
                                           // wait between blocks ran out)
 };
 
-constexpr uint32_t sort_windows(uint32_t n, int G) { return n / 4096u + (uint32_t)G; }
+__host__ __device__ constexpr uint32_t sort_windows(uint32_t n, int G) { return n / 4096u + (uint32_t)G; }
 
 struct LoadArgs {
     uint32_t n;
@@ -54,11 +56,12 @@ struct LoadArgs {
     // shares of all buckets are open at once, and what leaves L2 in parts is written twice.
     uint32_t rounds;
     LoadZero* z;
-    uint32_t* cnt;                        // [G][4097] requests per prompt length (zero on entry)
-    uint32_t* tick_cnt;                   // [G][kTickBins] (zero on entry)
+    size_t zero_bytes;                    // from z on: what must be zero (cleared by the launch where several blocks need it)
+    uint32_t* cnt;                        // [G][4097] requests per prompt length (cleared)
+    uint32_t* tick_cnt;                   // [G][kTickBins] (cleared)
     uint32_t* tick_start;                 // [G][kTickBins]
     uint32_t* tick_at;                    // [G][kTickBins] cursors, used when the groups' counters do not fit in shared memory
-    uint2* windows;                       // [n / 4096 + G] of the sort: first and last bin (zero on entry)
+    uint2* windows;                       // [n / 4096 + G] of the sort: first and last bin (cleared)
     uint32_t* binned;                     // [n] ticks bin by bin
     // outputs
     uint4* req;                           // [n] internal order (by group, then by prompt length): see TraceDev
@@ -72,7 +75,7 @@ struct LoadArgs {
     LoadReadback* readback;
 };
 
-cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st);          // one kernel; z, cnt, tick_cnt and windows cleared by the caller
+cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st);          // one kernel, after a memset
 cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st);    // ticks, off, G, n -> sorted
 cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st);     // ttft, n (one group) -> sorted
 
