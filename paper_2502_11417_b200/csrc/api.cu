@@ -731,7 +731,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const size_t o_work = lay.take(32 + (size_t)n_tickets * 4), o_accum = clear_accum ? lay.take(acc_bytes + 2 * hist_bytes) : 0;
     const size_t o_grid = lay.bytes;
     lay.take(grid_bytes);
-    const size_t clear_bytes = n == 0 ? o_grid : o_grid + first_bytes;
+    const size_t clear_bytes = n == 0 ? o_grid : (o_grid + first_bytes + 15) / 16 * 16;      // (k_prep clears them)
+    const bool clear_apart = clear_bytes > (64ull << 30);                                     // (beyond its 32-bit index)
     const size_t o_prep = lay.take((size_t)G * P * sizeof(Prep)), o_stats = lay.take(P * sizeof(disco_policy_stats_t) + 16);
     const size_t o_accum2 = clear_accum ? o_accum : lay.take(acc_bytes + 2 * hist_bytes);
     const size_t o_left = lay.take(any_mixed ? (N1 + kMaxGroups) * 4 : 0), o_hand = lay.take(N1 * 8);
@@ -761,7 +762,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         CU(cudaMemcpyAsync(c->fin_totals.p, c->fin_own.data(), c->fin_own.size() * 8, cudaMemcpyHostToDevice, st));
         c->fin_imported = false;
     }
-    CU(cudaMemsetAsync(mem, 0, clear_bytes, st));
+    if (clear_apart) CU(cudaMemsetAsync(mem, 0, clear_bytes, st));
 
     // ---- small tables to the device through pinned staging: one staging block, one copy (16-byte aligned regions)
     if (int rc = reserve_stage(c, table_bytes)) return rc;
@@ -784,7 +785,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
 
     // ---- Algorithms 1-3 for every (group, policy)
     CU(launch_prep(d_pol, P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
-                   c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), st));
+                   c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), mem, clear_apart ? 0 : clear_bytes, c->sms, st));
     g_launches += 1;
     if (any_beta) {
         CU(launch_prep_beta(d_pol, P, G, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,

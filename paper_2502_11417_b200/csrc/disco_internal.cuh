@@ -220,7 +220,7 @@ struct DbgRegistrar { explicit DbgRegistrar(cudaError_t (*r)(int32_t*)) { dbg_re
 // ---- launch wrappers (defined in the kernel translation units) -------------------------------------------
 cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupConst* gc, const int64_t* cum_mass,
                         const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep,
-                        cudaStream_t st);
+                        void* clear, size_t clear_bytes /* a multiple of 16: set to zero on the way */, int sms, cudaStream_t st);
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, int G, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off,
                              const uint32_t* tick_start, const uint32_t* tick_cnt /* [G][kTickBins], of the sorted ticks */,

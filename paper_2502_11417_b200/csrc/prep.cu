@@ -1,4 +1,6 @@
 // Policy preparation: Algorithms 1-3 for every (group, policy).
+#include <algorithm>
+
 #include "load.cuh"
 
 namespace disco {
@@ -45,8 +47,11 @@ __global__ void __launch_bounds__(kPrepThreads)
 k_prep(const PolicyConst* __restrict__ pol, uint32_t P, int G, const GroupConst* __restrict__ gc,
                        const int64_t* __restrict__ cum_mass, const uint32_t* __restrict__ cnt,
                        const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
-                       Prep* __restrict__ prep) {
+                       Prep* __restrict__ prep, uint4* __restrict__ clear, uint32_t clear_vecs) {
     grid_dependency_wait();
+    // what the kernels behind this one must find zero
+    for (uint32_t i = blockIdx.x * kPrepThreads + threadIdx.x; i < clear_vecs; i += gridDim.x * kPrepThreads)
+        clear[i] = make_uint4(0u, 0u, 0u, 0u);
     const uint32_t idx = (blockIdx.x * kPrepThreads + threadIdx.x) >> 5;
     if (idx >= P * (uint32_t)G) return;
     const int g = (int)(idx / P);
@@ -224,10 +229,11 @@ DBG_TRANSLATION_UNIT()
 
 cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupConst* gc, const int64_t* cum_mass,
                         const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep,
-                        cudaStream_t st) {
-    const uint32_t per = kPrepThreads / 32;
-    return launch_after(k_prep, (P * (uint32_t)G + per - 1) / per, kPrepThreads, 0, st, pol, P, G, gc, cum_mass, cnt, sorted,
-                        grp_off, prep);
+                        void* clear, size_t clear_bytes, int sms, cudaStream_t st) {
+    // a warp per pair, and blocks enough to clear at the speed of memory
+    const uint32_t per = kPrepThreads / 32, vecs = (uint32_t)(clear_bytes / 16);
+    const uint32_t blocks = std::max((P * (uint32_t)G + per - 1) / per, std::min((vecs + 4 * kPrepThreads - 1) / (4 * kPrepThreads), (uint32_t)sms * 8u));
+    return launch_after(k_prep, blocks, kPrepThreads, 0, st, pol, P, G, gc, cum_mass, cnt, sorted, grp_off, prep, (uint4*)clear, vecs);
 }
 
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, int G, const int64_t* cum_mass, const uint32_t* cnt,
