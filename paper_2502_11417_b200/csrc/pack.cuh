@@ -15,10 +15,10 @@ namespace disco {
 // or profile out of range is packed as 0 or 255, which the ingestion kernel refuses with the same error.
 constexpr uint32_t kPackChunk = 32768;
 constexpr size_t kPackBytes = (size_t)kPackChunk * 9;
-constexpr uint32_t kPackInPlace = 8192;       // traces up to this size are read from the pinned slot, without a copy
+constexpr uint32_t kPackInPlace = 8192;       // traces up to this size are read from the pinned slots, without a copy
 inline size_t packed_bytes(uint32_t n) { return ((size_t)n + kPackChunk - 1) / kPackChunk * kPackBytes; }
 
-// Packs and copies with a few threads of its own.  One per context: its threads and its page-locked slots live as long.
+// Packs with a few threads of its own.  One per context: its threads and its page-locked slots live as long.
 class Packer {
 public:
     Packer() = default;
@@ -31,24 +31,25 @@ public:
     cudaError_t pack(const disco_trace_desc_t& d, char* dev, cudaStream_t st, const char** at);
 
 private:
-    struct Lane { char* slot[2] = {nullptr, nullptr}; cudaEvent_t free[2] = {nullptr, nullptr}; int next = 0; };
-    cudaError_t open_lane(Lane& l, bool both);
-    cudaError_t work(Lane& l);
-    void run(size_t lane);
+    static constexpr uint32_t kSlots = 32;    // chunks in page-locked memory at a time (9 MB)
+    static constexpr uint32_t kRun = 8;       // chunks that go with one copy, at most
+    cudaError_t reserve_slots(uint32_t slots);
+    cudaError_t copy_runs(uint32_t chunks, char* dev, cudaStream_t st);
+    void run();
 
-    std::vector<Lane> lanes_;                 // the caller's, then the threads'
+    char* slots_ = nullptr;
+    uint32_t have_ = 0;
+    cudaEvent_t copied_[kSlots] = {};         // after the copy that ends with the slot
     std::vector<std::thread> threads_;
     std::mutex m_;
     std::condition_variable wake_, done_;
     uint64_t job_ = 0;
     size_t running_ = 0;
     bool stop_ = false;
-    int device_ = 0;
     const disco_trace_desc_t* d_ = nullptr;   // the job in work
-    char* dev_ = nullptr;
-    cudaStream_t st_ = nullptr;
-    std::atomic<uint32_t> chunk_{0};
-    std::atomic<int> error_{0};
+    std::atomic<uint32_t> chunk_{0};          // next chunk to pack
+    std::atomic<uint32_t> freed_{0};          // chunks whose copies are done: their slots are free
+    std::atomic<uint32_t> packed_[kSlots] = {};   // 1 + the chunk that a slot holds
 };
 
 }  // namespace disco

@@ -98,3 +98,33 @@ def test_linear_wait_rule_on_samples(kind, n):
     tr.eval_policies(pols, 1)
     check_prep(tr, Oracle.from_workload(w), pols, f"{kind} {n}")
     tr.close()
+
+
+@pytest.mark.parametrize("n", [15, 8192, 8193, 32768, 32785, 70001, 1_200_003])
+@pytest.mark.parametrize("profiles", ["both", "server", "device", "none"])
+def test_pageable_traces_are_packed(n, profiles):
+    # ordinary host arrays go to the device packed, chunk by chunk: the same tables and statistics as from device memory;
+    # a value out of range is refused wherever it lies
+    import torch
+    from paper_2502_11417_b200 import DiscoError, Trace
+    w = synth.tiny_workload(97, n, n_servers=3, n_devices=2, max_prompt=4096, max_out=30)
+    sp = w.server_profile if profiles in ("both", "server") else None
+    dp = w.device_profile if profiles in ("both", "device") else None
+    cols = [w.prompt_len, w.output_len, w.server_ttft_s, sp, dp]
+    dev = [None if c is None else torch.from_numpy(c).cuda() for c in cols]
+    got = []
+    for c in (cols, dev):
+        tr = Trace().load_trace(*c, w.servers, w.devices)
+        tr.eval_policies([synth.policy(0.4)], 3)
+        got.append((bytes(tr.reduce_stats()), [t.tobytes() for g in range(tr.n_groups) for t in tr.group_tables(g)]))
+        tr.close()
+    assert got[0] == got[1]
+    for k, bad in ((0, 4097), (0, 0), (1, 8193), (1, -1), (2, 0.0), (3, 3), (4, 2)):
+        if cols[k] is None:
+            continue
+        at = (n * 2) // 3
+        wrong = [None if c is None else c.copy() for c in cols]
+        wrong[k][at] = bad
+        with pytest.raises(DiscoError) as ei:
+            Trace().load_trace(*wrong, w.servers, w.devices)
+        assert ei.value.code == -1 and f"at request {at}" in str(ei.value)
