@@ -197,7 +197,7 @@ int disco_get_prep(disco_ctx_t* ctx, uint32_t g, uint32_t p, disco_prep_t* out, 
 /* Copies group g's tables out (any may be NULL): requests per prompt length
  * cnt[DISCO_MAX_PROMPT+1] (host memory), the 257 equally spaced order statistics
  * of F and up to `n_sorted` of the smallest sorted TTFT ticks (host or device
- * memory, each).  Synchronises `stream`.  Returns the number of
+ * memory, each).  Synchronises `stream` if it has to wait for a copy.  Returns the number of
  * requests behind the group's tables (the group's own requests, or what
  * disco_set_group_tables gave), or a negative status. */
 int64_t disco_get_group_tables(disco_ctx_t* ctx, uint32_t g, int64_t* cnt, int32_t* knots,

@@ -459,13 +459,13 @@ class Trace:
         cnt = np.empty(4097, dtype=np.int64)
         kn = np.empty(257, dtype=np.int32)
         call, st = lib().disco_get_group_tables, _stream_ptr(stream)
-        ng = call(self._h, g, cnt.ctypes.data, kn.ctypes.data, None, 0, st)
+        ng = call(self._h, g, _address(cnt), _address(kn), None, 0, st)
         if ng < 0:
             _check(int(ng))
         k = int(ng) if n_sorted is None else min(int(ng), n_sorted)
         srt = np.empty(k, dtype=np.int32)
         if k:
-            rc = call(self._h, g, None, None, srt.ctypes.data, k, st)
+            rc = call(self._h, g, None, None, _address(srt), k, st)
             if rc < 0:
                 _check(int(rc))
         return cnt, kn, srt

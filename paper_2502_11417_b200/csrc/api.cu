@@ -664,7 +664,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         L.slab1 = slabs.size();
     }
 
-    // ---- request chunks, of one group each: of the grid kernel, about three to each block that fits the GPU at once, 256
+    // ---- request chunks, of one group each: of the grid kernel, about two to each block that fits the GPU at once (three
+    //      where that is more than 16,384 requests: the end of the launch is then worth more than the entering of runs), 256
     //      requests (one a thread) or more; of the pair kernel, two to a multiprocessor, 2,048 requests or more
     const uint32_t sms = (uint32_t)c->sms, kMaxChunk = 65280;
     const size_t N1 = n ? n : 1;
@@ -687,7 +688,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             }
         return v;
     };
-    const std::vector<Chunk> chunks = make_chunks(chunk_size((size_t)3 * sms * grid_blocks_per_sm(tall ? 2 : 1), 256));
+    const size_t at_once = (size_t)sms * grid_blocks_per_sm(tall ? 2 : 1);
+    const std::vector<Chunk> chunks = make_chunks(chunk_size(at_once * (N1 / at_once > 2 * 16384 ? 3 : 2), 256));
     std::vector<Chunk> pair_chunks;
     if (any_pairs) pair_chunks = make_chunks(chunk_size((size_t)2 * sms, 2048));
 
@@ -1031,7 +1033,8 @@ int64_t disco_get_group_tables(disco_ctx_t* c, uint32_t g, int64_t* cnt, int32_t
         CU(cudaMemcpyAsync(knots, c->knots.as<int32_t>() + (size_t)g * kNKnots, kNKnots * 4, cudaMemcpyDefault, st));
     const uint64_t k = std::min<uint64_t>(n_sorted, ng);
     if (sorted_ticks && k) CU(cudaMemcpyAsync(sorted_ticks, c->F_sorted + off, k * 4, cudaMemcpyDefault, st));
-    CU(cudaStreamSynchronize(st));
+    // (what comes from the copy, or is known on the host, waits for nothing)
+    if (fetch || (knots && !knots_on_host) || (sorted_ticks && k)) CU(cudaStreamSynchronize(st));
     if (fetch) c->tab_host_now = true;
     if (cnt) for (size_t i = 0; i < kLengths; ++i) cnt[i] = c->tab_host[g * kLengths + i];
     if (knots && knots_on_host) std::memcpy(knots, host_knots(c, (int)g), kNKnots * 4);

@@ -122,7 +122,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
             const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
             const uint32_t* __restrict__ tick_start, const uint32_t* __restrict__ tick_cnt, Prep* __restrict__ prep) {
     __shared__ uint32_t s_end[kTickBins];                             // ticks of the group up to the bin's last
-    __shared__ long long part[3][32];
+    __shared__ long long part[6][32];
     grid_dependency_wait();
     const int g = (int)(blockIdx.x / P);
     const uint32_t p = blockIdx.x % P;
@@ -160,38 +160,66 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
     for (int i = 0; i < kBetaLens; ++i) {
         len[i] = 1 + (int)threadIdx.x + i * kBetaThreads;
         k[i] = cnt[(size_t)g * (kMaxPrompt + 1) + len[i]];
-        at_lo[i] = at_hi[i] = 0;
-        if (k[i] == 0) continue;
-        at_lo[i] = position(0, 0u, N);
-        at_hi[i] = len[i] <= l_imm ? at_lo[i] : position(min((w_tail + 1) * (long long)len[i], w_tail), 0u, N);
     }
-    // the block's sums of three values, the same to all threads
-    auto totals = [&](long long (&v)[3]) {
+    // the block's sums of the values, the same to all threads
+    auto totals = [&](auto& v) {
+        constexpr int kValues = (int)(sizeof(v) / sizeof(v[0]));
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
+        for (int j = 0; j < kValues; ++j) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(FULL, v[j], o);
             if (lane == 0) part[j][wi] = v[j];
         }
         __syncthreads();
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
+        for (int j = 0; j < kValues; ++j) {
             v[j] = part[j][lane];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(FULL, v[j], o);
         }
         __syncthreads();
     };
+    auto wait = [&](long long beta, int l) { return l <= l_imm ? 0ll : min(beta * (long long)l, w_tail); };
     long long lo = 0, hi = w_tail + 1;                                // beyond hi every wait is w_tail
-    {
-        long long v[3] = {0, 0, 0};                                   // device's tokens at the range's ends
+    // ---- first by whole bins: the ticks up to a bin's first and last bound the sum from both sides, which settles most of
+    //      the range without a look at the ticks
+    while (hi - lo > 1) {
+        const long long d = hi - lo;
+        const long long m[3] = {lo + (d + 3) / 4, lo + (d + 1) / 2, lo + (3 * d + 3) / 4};
+        long long v[6] = {0, 0, 0, 0, 0, 0};                          // at least, at most
 #pragma unroll
         for (int i = 0; i < kBetaLens; ++i) {
+            if (k[i] == 0) continue;
+            const long long mass = (long long)len[i] * (long long)k[i];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int bin = tick_bin((uint32_t)wait(m[j], len[i]));
+                v[j] += mass * (long long)(N - s_end[bin]);
+                v[3 + j] += mass * (long long)(N - (bin ? s_end[bin - 1] : 0u));
+            }
+        }
+        totals(v);
+        const long long old_lo = lo, old_hi = hi;
+#pragma unroll
+        for (int j = 2; j >= 0; --j) if ((double)v[3 + j] <= limit && m[j] < hi) hi = m[j];      // certainly fits
+#pragma unroll
+        for (int j = 0; j < 3; ++j) if ((double)v[j] > limit && m[j] > lo && m[j] < hi) lo = m[j];   // certainly does not
+        if (lo == old_lo && hi == old_hi) break;
+    }
+    // ---- the positions at the ends of what is left
+    {
+        long long v[2] = {0, 0};
+#pragma unroll
+        for (int i = 0; i < kBetaLens; ++i) {
+            at_lo[i] = at_hi[i] = 0;
+            if (k[i] == 0) continue;
+            at_lo[i] = position(wait(lo, len[i]), 0u, N);
+            at_hi[i] = len[i] <= l_imm ? at_lo[i] : position(wait(hi, len[i]), at_lo[i], N);
             v[0] += (long long)len[i] * (long long)k[i] * (long long)(N - at_lo[i]);
             v[1] += (long long)len[i] * (long long)k[i] * (long long)(N - at_hi[i]);
         }
         totals(v);
-        if ((double)v[0] <= limit) hi = lo;                           // (no waits at all fit)
+        if (lo == 0 && (double)v[0] <= limit) hi = lo;                // (no waits at all fit)
         else if ((double)v[1] > limit) lo = hi;                       // not even the longest waits fit
     }
     // the slope at lo is too small, that at hi fits
@@ -205,7 +233,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 at[j][i] = at_lo[i];
-                if (k[i] != 0 && at_lo[i] < at_hi[i]) at[j][i] = position(min(m[j] * (long long)len[i], w_tail), at_lo[i], at_hi[i]);
+                if (k[i] != 0 && at_lo[i] < at_hi[i]) at[j][i] = position(wait(m[j], len[i]), at_lo[i], at_hi[i]);
                 v[j] += (long long)len[i] * (long long)k[i] * (long long)(N - at[j][i]);
             }
         }

@@ -97,11 +97,12 @@ k_finalize(uint32_t P, int G, const GroupConst* __restrict__ gc,
             for (int g = 0; g < G; ++g) s += acc[((size_t)p * G + g) * kNAcc + lane];
             tot[lane] = s;
         }
-        __syncwarp();
-        if (lane == 0) {
-            // Eq. 8 on the exact integer token totals of each group
-            double cost = 0.0;
-            for (int g = 0; g < G; ++g) {
+        // Eq. 8 on the exact integer token totals of each group: a lane per group, added up in the groups' order
+        double cost = 0.0;
+        for (int g0 = 0; g0 < G; g0 += 32) {
+            double x = 0.0;
+            if (g0 + lane < G) {
+                const int g = g0 + lane;
                 const unsigned long long* a = acc + ((size_t)p * G + g) * kNAcc;
                 const unsigned long long dev_tok = a[A_TOK_DEVICE];
                 const double dts = (double)(fin_totals[g] - dev_tok), dtd = (double)dev_tok;
@@ -109,8 +110,12 @@ k_finalize(uint32_t P, int G, const GroupConst* __restrict__ gc,
                 const GroupConst& c = gc[g];
                 const double srv = __dadd_rn(__dmul_rn(c.cps_d, pts), __dmul_rn(c.cds_d, dts));
                 const double dev = __dadd_rn(__dmul_rn(c.cpd_d, ptd), __dmul_rn(c.cdd_d, dtd));
-                cost = __dadd_rn(cost, __dadd_rn(srv, __dmul_rn(c.lambda_d, dev)));
+                x = __dadd_rn(srv, __dmul_rn(c.lambda_d, dev));
             }
+            for (int k = 0; k < min(32, G - g0); ++k) cost = __dadd_rn(cost, __shfl_sync(0xFFFFFFFFu, x, k));
+        }
+        __syncwarp();
+        if (lane == 0) {
             disco_policy_stats_t& s = s_out;
             s.mean_ttft_s = N ? __ddiv_rn(__dmul_rn((double)tot[A_TTFT_SUM], 1e-6), (double)N) : 0.0;
             s.total_cost = cost;
