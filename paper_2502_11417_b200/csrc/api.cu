@@ -529,21 +529,24 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 pl.batches[cc.kind[g]] += (rb.ng[g] + 31) / 32;
                 if (cc.kind[g] == G_EXACT) pl.search = std::max(pl.search, cc.search[g]);
             }
+            // shortest and longest regular interval of the streams: as generated where a stream waits for every token, else from
+            // tau on
+            const bool as_is[2] = {!cc.pacing || (cc.kind[g] == G_FREE && !even_s), !cc.pacing || (cc.kind[g] == G_FREE && !even_d)};
             int64_t lo_v[3], hi_v[3];
-            lo_v[0] = cc.pacing ? cc.tau : gc.T_srv - (int64_t)gc.J_srv; hi_v[0] = cc.pacing ? std::max<int64_t>(cc.tau, xs) : xs;
-            lo_v[1] = cc.pacing ? cc.tau : gc.T_dev - (int64_t)gc.J_dev; hi_v[1] = cc.pacing ? std::max<int64_t>(cc.tau, xd) : xd;
-            lo_v[2] = std::min(lo_v[0], lo_v[1]); hi_v[2] = std::max(hi_v[0], hi_v[1]);
+            lo_v[0] = as_is[0] ? gc.T_srv - (int64_t)gc.J_srv : cc.tau; hi_v[0] = as_is[0] ? xs : std::max<int64_t>(cc.tau, xs);
+            lo_v[1] = as_is[1] ? gc.T_dev - (int64_t)gc.J_dev : cc.tau; hi_v[1] = as_is[1] ? xd : std::max<int64_t>(cc.tau, xd);
+            lo_v[2] = std::min(lo_v[0], lo_v[1]); hi_v[2] = cc.kind[g] == G_GENERAL ? std::max(hi_v[0], hi_v[1]) : lo_v[2];
             for (int s = 0; s < 3; ++s) {
                 const int lo = host_bin_of_ticks(lo_v[s]), hi = host_bin_of_ticks(hi_v[s]);
                 cc.lo[g][s] = lo;
-                cc.ktau[g][s] = cc.pacing ? host_bin_of_ticks(cc.tau) - lo : -1;
+                cc.ktau[g][s] = cc.pacing && !(s < 2 && as_is[s]) ? host_bin_of_ticks(cc.tau) - lo : -1;
                 Wmax[s] = std::max(Wmax[s], hi - lo + 1);
             }
         }
         for (int s = 0; s < 3; ++s) cc.W[s] = Wmax[s];
         if (!(pl.kinds & ~(1u << G_EXACT))) continue;                        // nothing but the hand-offs is stored
         stored = true;
-        for (int s = 0; s < 3; ++s) wmax[s] = std::max<size_t>(wmax[s], Wmax[s]);
+        for (int s = 0; s < ((pl.kinds & (1u << G_GENERAL)) ? 3 : 2); ++s) wmax[s] = std::max<size_t>(wmax[s], Wmax[s]);   // (no other kind stores the third)
         if ((size_t)n * (Wmax[0] + Wmax[1] + Wmax[2]) * 2 > (48ull << 30))
             return fail(DISCO_ENOMEM, "per-request TBT windows would exceed 48 GB");
     }
@@ -849,7 +852,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
             }
             CU(launch_grid(tr, gc, dcc, prep, P, dsl, (uint32_t)b.count, b.T, wide, classes[k].pacing != 0, d_tab,
-                           d_chunks, (uint32_t)chunks.size(), rec, gt, left, tickets + ticket++, work, c->sms, st));
+                           d_chunks, (uint32_t)chunks.size(), rec, gt, left, k0, tickets + ticket++, work, c->sms, st));
             CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, wide, host_bin_of_ticks(classes[k].tau), d_tab, gt, acc,
                              h_ttft, h_tbt, st));
             g_launches += 2;

@@ -156,6 +156,18 @@ inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block,
 }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The stream after a hand-off stores no window of its own where groups are played free without pacing: it is stream
+// x_stream's (0 the server's, 1 the device's) without the interval in front of token 2, whose bin first_bin gives.  -1: it
+// stores one, if it has any.
+__device__ __forceinline__ int x_stream(const ClassConst& cc, const GroupConst& gc) {
+    return cc.pacing ? -1 : (gc.candidate == 1 ? 1 : 0);
+}
+__device__ __forceinline__ int first_bin(const GroupConst& gc, int stream, uint32_t k0, uint32_t orig) {
+    const uint32_t h = mix32(mix32(k0 + orig * kHashReq) + 2u * kHashTok);
+    const int32_t T = stream ? gc.T_dev : gc.T_srv, J = stream ? gc.J_dev : gc.J_srv;
+    return bin_of_ticks((uint32_t)(T - J) + __umulhi(h, 2u * (uint32_t)J + 1u));
+}
+
 // The batch-th batch of `size` requests among the groups of one kind: its group, first request and length.
 __device__ __forceinline__ bool batch_of_kind(const TraceDev& tr, const ClassConst& cc, int kind, uint32_t size, uint32_t batch,
                                               int& g, uint32_t& k_lo, uint32_t& count) {
@@ -259,7 +271,7 @@ uint32_t grid_blocks_per_sm(int T);
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
                         const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide, bool count_pairs,
                         const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt,
-                        LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t* ticket /* zero */,
+                        LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t k0, uint32_t* ticket /* zero */,
                         uint64_t* work /* [4], added to */, int sms, cudaStream_t st);
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
                           bool wide, int bin_tau, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,

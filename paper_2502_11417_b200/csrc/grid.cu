@@ -80,7 +80,7 @@ struct Ctx {                                           // a (chunk, slab)
     int K, T;
     bool may_migrate, mixed;
     float th_lo;                                       // mixed: smallest overhead
-    int E0;
+    int E0, x_from;
     uint32_t even;
 };
 
@@ -98,6 +98,7 @@ struct Args {
     uint32_t n_chunks;
     GridTables gt;
     LeftLists left;
+    uint32_t k0;
     uint32_t* ticket;
     unsigned long long* work;
     int count_pairs;
@@ -113,6 +114,20 @@ __device__ __forceinline__ void add_rows(const uint16_t* __restrict__ win, int W
                                          uint32_t* hist) {
     if (mask == 0u) return;
     const int lane = threadIdx.x & 31;
+    if (W <= 16) {
+        // short rows: several requests' at a time, which mostly lie side by side
+        const int per = 32 / W, mine = lane / W, b = lane - mine * W;
+        const bool in = mine < per && DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN);
+        uint32_t sum = 0;
+#pragma unroll 4
+        for (int r0 = 0; r0 < 32; r0 += per) {
+            const int r = r0 + mine;
+            const uint32_t k = __shfl_sync(FULL, kk, r & 31);
+            if (in && r < 32 && ((mask >> r) & 1u)) sum += win[(size_t)k * W + b];
+        }
+        if (sum) atomicAdd(&hist[lo + b], sub ? 0u - sum : sum);
+        return;
+    }
     for (int b0 = 0; b0 < W; b0 += 32) {
         const int b = b0 + lane;
         const bool in = b < W && DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN);
@@ -135,7 +150,8 @@ __device__ __forceinline__ void add_rows(const uint16_t* __restrict__ win, int W
 
 // The windows of the lanes' requests whose streams' intervals are not all tau: the base stream (device or server) goes to
 // every row of the grid but those that migrate, [0, t), which get the stream after the hand-off.
-__device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_t* tbt, bool valid, uint32_t kk, bool device, int t) {
+__device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_t* tbt, bool valid, uint32_t kk, bool device, int t,
+                                            uint32_t orig) {
     const ClassConst& cc = *a.cc;
     uint32_t* all = tbt + (c.T - 1) * kNBins;
 #pragma unroll
@@ -148,8 +164,13 @@ __device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_
             add_rows(a.rec.win[s], W, lo, __ballot_sync(FULL, mine && t == r), kk, true, tbt + (r - 1) * kNBins);
     }
     if (c.even & 4u) return;
+    const int from = c.x_from >= 0 ? c.x_from : 2;
     for (int r = 1; r <= c.T; ++r)
-        add_rows(a.rec.win[2], cc.W[2], cc.lo[c.g][2], __ballot_sync(FULL, valid && t == r), kk, false, tbt + (r - 1) * kNBins);
+        add_rows(a.rec.win[from], cc.W[from], cc.lo[c.g][from], __ballot_sync(FULL, valid && t == r), kk, false, tbt + (r - 1) * kNBins);
+    if (c.x_from >= 0 && valid && t > 0) {
+        const int bin = first_bin(a.gcs[c.g], c.x_from, a.k0, orig);
+        if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicSub(&tbt[(t - 1) * kNBins + bin], 1u);
+    }
 }
 
 // One sweep over the requests [pa, pb) of the chunk, or (list) of the block's list: what they come to when the device
@@ -217,7 +238,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                 if (WIDE) s.tx[r] += tx;
             }
         if (t > 0) hist_add(tbt + (t - 1) * kNBins, bin_of_ticks(hand.y));
-        if (WIDE) add_windows(a, c, tbt, valid, kk, dev_wins, t);
+        if (WIDE) add_windows(a, c, tbt, valid, kk, dev_wins, t, q.z);
     }
 }
 
@@ -378,6 +399,7 @@ k_grid(const __grid_constant__ Args a) {
         c.may_migrate = sl.mig && gc.candidate != 0;
         c.mixed = sl.mixed && c.may_migrate;
         c.E0 = (int)sl.expected_len; c.even = a.cc->even[g];
+        c.x_from = x_stream(*a.cc, gc);
         float th[NT];                                                  // rows beyond the slab's never migrate
 #pragma unroll
         for (int r = 0; r < NT; ++r) th[r] = (c.may_migrate && r < c.T) ? sl.theta[sl.mixed ? 1 : r] : __int_as_float(0x7F800000);
@@ -660,10 +682,10 @@ uint32_t grid_blocks_per_sm(int T) { return T == 1 ? 4 : 2; }
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
                         const Slab* slabs, uint32_t n_slabs, int T, bool wide, bool count_pairs, const uint32_t* tab,
                         const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt, LeftLists left,
-                        uint32_t* ticket, uint64_t* work, int sms, cudaStream_t st) {
+                        uint32_t k0, uint32_t* ticket, uint64_t* work, int sms, cudaStream_t st) {
     if (n_chunks == 0 || n_slabs == 0) return cudaSuccess;
     if ((uint64_t)n_chunks * n_slabs > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    const Args a = {tr, rec, gc, cc, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, ticket,
+    const Args a = {tr, rec, gc, cc, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, k0, ticket,
                     (unsigned long long*)work, count_pairs ? 1 : 0};
     if (wide) return T == 1 ? launch_one<1, true>(a, sms, st) : T <= 4 ? launch_one<4, true>(a, sms, st) : launch_one<8, true>(a, sms, st);
     return T == 1 ? launch_one<1, false>(a, sms, st) : T <= 4 ? launch_one<4, false>(a, sms, st) : launch_one<8, false>(a, sms, st);

@@ -308,12 +308,18 @@ k_pairs_acc(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* _
                     if (!kAllOk && !ok[k]) continue;
                     const int c = migr[k] ? 2 : (dev_wins[k] ? 1 : 0);
                     if ((even >> c) & 1u) continue;
-                    const int W = c == 2 ? W2 : (c == 1 ? W1 : W0), kt = c == 2 ? kt2 : (c == 1 ? kt1 : kt0);
-                    const uint16_t* wp = rec.win[c] + (size_t)stB[rr[k] * kStageVec + 6].x * W;
-                    unsigned long long* hp = hist_tbt + (size_t)p * kNBins + cc.lo[g][c];
+                    const uint32_t kk = stB[rr[k] * kStageVec + 6].x;
+                    const int x_from = x_stream(cc, gc), from = (c == 2 && x_from >= 0) ? x_from : c;
+                    const int W = from == 2 ? W2 : (from == 1 ? W1 : W0), kt = from == 2 ? kt2 : (from == 1 ? kt1 : kt0);
+                    const uint16_t* wp = rec.win[from] + (size_t)kk * W;
+                    unsigned long long* hp = hist_tbt + (size_t)p * kNBins + cc.lo[g][from];
+                    if (from != c) {
+                        const int bin = first_bin(gc, from, k0, tr.req[kk].z);
+                        if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ACC, DBG_BIN)) atomicAdd(&hist_tbt[(size_t)p * kNBins + bin], ~0ull);
+                    }
                     for (int j = 0; j < W; ++j) {
                         const uint32_t v = j == kt ? 0u : wp[j];
-                        if (v && DBG_OK(cc.lo[g][c] + j, kNBins, DBG_K_PAIRS_ACC, DBG_BIN)) atomicAdd(&hp[j], (unsigned long long)v);
+                        if (v && DBG_OK(cc.lo[g][from] + j, kNBins, DBG_K_PAIRS_ACC, DBG_BIN)) atomicAdd(&hp[j], (unsigned long long)v);
                     }
                 }
             }

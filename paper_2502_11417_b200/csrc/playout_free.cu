@@ -6,8 +6,10 @@
 // Bound: integer issue (a hash, a range map and a bin per token and stream).  A warp plays a request, a lane every 32nd
 // token.  Every lane counts in counters of its own, [bin][lane] in shared memory: no atomics and no bank conflicts, where
 // 32 lanes would meet in the few bins of a stream; two requests share a counter's halves before the lanes' counts are
-// added up (step k of lane b reads counter (k + b) mod 32, again without conflicts) and written as rows of 16-bit counts.
-// 200,000 requests of 200 tokens, two streams: 204 us with one window a warp and atomics.
+// added up (a lane a bin, four counters at a time, lane b starting with the (b mod 8)th four: again without conflicts) and
+// written as rows of 16-bit counts.  The stream after a hand-off stores no window: it is the target's without token 2,
+// which the reductions take away (x_stream in disco_internal.cuh).  200,000 requests of 200 tokens, two streams: 204 us
+// with one window a warp and atomics, 146 us with all three windows stored.
 #include <algorithm>
 
 #include "disco_internal.cuh"
@@ -37,13 +39,12 @@ template <bool BOTH, bool SMALL>
 __global__ void __launch_bounds__(kFreeWarps * 32, 4)
 k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec) {
-    extern __shared__ uint32_t s_win[];                       // per warp: [W0 + W1][32] counters, [W0 + W1] their sums
+    extern __shared__ __align__(16) uint32_t s_win[];         // per warp: [W0 + W1][32] counters
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warps = blockDim.x >> 5;
     grid_dependency_wait();
     const ClassConst& cc = *ccp;
-    const int W0 = cc.W[0], W1 = cc.W[1], W2 = cc.W[2], WW = W0 + W1;
-    uint32_t* win = s_win + wib * (WW * 33);
-    uint32_t* red = win + WW * 32;
+    const int W0 = cc.W[0], W1 = cc.W[1], WW = W0 + W1;
+    uint32_t* win = s_win + wib * (WW * 32);
     for (int b = lane; b < WW * 32; b += 32) win[b] = 0;
     __syncwarp();
     for (uint32_t batch = blockIdx.x * warps + wib;; batch += gridDim.x * warps) {
@@ -65,94 +66,59 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
             n_l = q.y >> 16; l_l = q.y & 0xFFFFu;
             key_l = mix32(k0 + q.z * kHashReq);
         }
-        // sums and maxima of the jitter u = (h * (2J + 1)) >> 32, and of the target's from token 3 on
-        uint32_t o_s0 = 0, o_s1 = 0, o_m0 = 0, o_m1 = 0, o_later = 0;
+        // sums of the jitter u = (h * (2J + 1)) >> 32, its maxima from token 3 on, and token 2's
+        uint32_t o_s0 = 0, o_s1 = 0, o_m0 = 0, o_m1 = 0, o_f0 = 0, o_f1 = 0;
+        const int b_lo = on0 ? 0 : W0, b_hi = on1 ? WW : W0;      // the bins in use
         for (int r0 = 0; r0 < (int)n_here; r0 += 2) {
             const int pair = min(2, (int)n_here - r0);
 #pragma unroll 1
             for (int half = 0; half < pair; ++half) {
                 const int r = r0 + half;
-                const uint32_t n = __shfl_sync(FULL, n_l, r), key = __shfl_sync(FULL, key_l, r), inc = half ? 65536u : 1u;
-                uint32_t s0 = 0, s1 = 0, m0 = 0, m1 = 0;
-                if (BOTH) {
-                    uint32_t later = 0;                       // the target's largest jitter from token 3 on
-                    uint32_t hin = key + (2u + lane) * kHashTok;
+                const uint32_t n = __shfl_sync(FULL, n_l, r), inc = half ? 65536u : 1u;
+                uint32_t hin = __shfl_sync(FULL, key_l, r) + (2u + lane) * kHashTok;
+                uint32_t s0 = 0, s1 = 0, m0 = 0, m1 = 0, f0 = 0, f1 = 0, j = 2u + lane;
+                // one token: its interval in each stream that is played
+                auto token = [&](uint32_t& u, uint32_t& v) {
+                    const uint32_t h = mix32(hin);
+                    hin += 32u * kHashTok;
+                    if (BOTH || on0) { u = __umulhi(h, mul0); s0 += u; count_in<SMALL>(ct0, base0 + u, inc); }
+                    if (BOTH || on1) { v = __umulhi(h, mul1); s1 += v; count_in<SMALL>(ct1, base1 + v, inc); }
+                };
+                if (j <= n) {
+                    token(f0, f1);
+                    if (lane != 0) { m0 = f0; m1 = f1; }          // (lane 0 had token 2)
 #pragma unroll 2
-                    for (uint32_t j = 2u + lane; j <= n; j += 32u) {
-                        const uint32_t h = mix32(hin);
-                        hin += 32u * kHashTok;
-                        const uint32_t u = __umulhi(h, mul0), v = __umulhi(h, mul1);
-                        s0 += u; m0 = max(m0, u);
-                        count_in<SMALL>(ct0, base0 + u, inc);
-                        s1 += v; m1 = max(m1, v);
-                        count_in<SMALL>(ct1, base1 + v, inc);
-                        if (j != 2u) later = max(later, to_dev ? v : u);
-                    }
-                    later = __reduce_max_sync(FULL, later);
-                    if (lane == r) o_later = later;
-                } else {
-                    if (on0) {
-                        uint32_t hin = key + (2u + lane) * kHashTok;
-#pragma unroll 2
-                        for (uint32_t j = 2u + lane; j <= n; j += 32u) {
-                            const uint32_t u = __umulhi(mix32(hin), mul0);
-                            hin += 32u * kHashTok;
-                            s0 += u; m0 = max(m0, u);
-                            count_in<SMALL>(ct0, base0 + u, inc);
-                        }
-                    }
-                    if (on1) {
-                        uint32_t hin = key + (2u + lane) * kHashTok;
-#pragma unroll 2
-                        for (uint32_t j = 2u + lane; j <= n; j += 32u) {
-                            const uint32_t v = __umulhi(mix32(hin), mul1);
-                            hin += 32u * kHashTok;
-                            s1 += v; m1 = max(m1, v);
-                            count_in<SMALL>(ct1, base1 + v, inc);
-                        }
+                    for (j += 32u; j <= n; j += 32u) {
+                        uint32_t u = 0, v = 0;
+                        token(u, v);
+                        if (BOTH || on0) m0 = max(m0, u);
+                        if (BOTH || on1) m1 = max(m1, v);
                     }
                 }
-                s0 = __reduce_add_sync(FULL, s0); m0 = __reduce_max_sync(FULL, m0);
-                s1 = __reduce_add_sync(FULL, s1); m1 = __reduce_max_sync(FULL, m1);
-                if (lane == r) { o_s0 = s0; o_s1 = s1; o_m0 = m0; o_m1 = m1; }
+                if (BOTH || on0) { s0 = __reduce_add_sync(FULL, s0); m0 = __reduce_max_sync(FULL, m0); f0 = __shfl_sync(FULL, f0, 0); }
+                if (BOTH || on1) { s1 = __reduce_add_sync(FULL, s1); m1 = __reduce_max_sync(FULL, m1); f1 = __shfl_sync(FULL, f1, 0); }
+                if (lane == r) { o_s0 = s0; o_s1 = s1; o_m0 = m0; o_m1 = m1; o_f0 = f0; o_f1 = f1; }
             }
             __syncwarp();
             // the lanes' counts are added up and go out; the counters are cleared for the next pair
             const size_t k = k_lo + r0;
 #pragma unroll 1
-            for (int b = lane; b < WW; b += 32) {
+            for (int b = b_lo + lane; b < b_hi; b += 32) {
+                uint4* row = reinterpret_cast<uint4*>(win + b * 32);
                 uint32_t t = 0;
-                uint32_t* row = win + b * 32;
 #pragma unroll
-                for (int c = 0; c < 32; ++c) t += row[(c + b) & 31];
-                if (BOTH) red[b] = t;
-                const bool first = b < W0;
-                if (first ? on0 : on1) {
-                    uint16_t* to = first ? rec.win[0] + k * W0 + b : rec.win[1] + k * W1 + (b - W0);
-                    to[0] = (uint16_t)t;
-                    if (pair > 1) to[first ? W0 : W1] = (uint16_t)(t >> 16);
+                for (int c = 0; c < 8; ++c) {
+                    const int at = (c + b) & 7;
+                    const uint4 x = row[at];
+                    row[at] = make_uint4(0u, 0u, 0u, 0u);
+                    t += x.x + x.y + x.z + x.w;
                 }
+                const bool first = b < W0;
+                uint16_t* to = first ? rec.win[0] + k * W0 + b : rec.win[1] + k * W1 + (b - W0);
+                to[0] = (uint16_t)t;
+                if (pair > 1) to[first ? W0 : W1] = (uint16_t)(t >> 16);
             }
             __syncwarp();
-#pragma unroll 4
-            for (int b = 0; b < WW; ++b) win[b * 32 + lane] = 0;
-            if (BOTH && cand) {
-                // stream X: one token of the candidate, then the target's from token 3 on
-                const int lo_t = to_dev ? ct1.lo : ct0.lo, Wt = to_dev ? W1 : W0, shift = cc.lo[g][2] - lo_t;
-                const uint32_t* wt = red + (to_dev ? W0 : 0);
-#pragma unroll 1
-                for (int half = 0; half < pair; ++half) {
-                    const uint32_t h2 = mix32(__shfl_sync(FULL, key_l, r0 + half) + 2u * kHashTok);
-                    const int skip = bin_of_ticks(to_dev ? base1 + __umulhi(h2, mul1) : base0 + __umulhi(h2, mul0)) - lo_t;
-                    for (int b = lane; b < W2; b += 32) {
-                        const int t = b + shift;
-                        uint32_t v = (t >= 0 && t < Wt) ? wt[t] >> (16 * half) : 0u;
-                        if (t == skip) --v;
-                        rec.win[2][(k + half) * W2 + b] = (uint16_t)v;
-                    }
-                }
-                __syncwarp();
-            }
         }
         if (lane < n_here) {
             const uint32_t k = k_lo + lane, nI = n_l - 1u, tau = (uint32_t)cc.tau;
@@ -169,12 +135,13 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
                         M = (uint32_t)(K[ki] + (int32_t)(((int64_t)(K[ki + 1] - K[ki]) * (int64_t)fr) >> 16));
                 }
                 const uint32_t base = to_dev ? base1 : base0;
-                sumX = M + (to_dev ? sum1 : sum0) - (base + __umulhi(mix32(key_l + 2u * kHashTok), to_dev ? mul1 : mul0));
-                maxX = max(M, nI > 1u ? base + o_later : 0u);
+                sumX = M + (to_dev ? sum1 - o_f1 : sum0 - o_f0) - base;
+                maxX = max(M, nI > 1u ? base + (to_dev ? o_m1 : o_m0) : 0u);
             }
+            const uint32_t most0 = max(o_m0, o_f0) + base0, most1 = max(o_m1, o_f1) + base1;
             rec.hand[k] = make_uint2(m, M);
             rec.sum[0][k] = sum0; rec.sum[1][k] = sum1; rec.sum[2][k] = sumX;
-            rec.max[0][k] = nI ? (on0 ? o_m0 + base0 : tau) : 0u; rec.max[1][k] = nI ? (on1 ? o_m1 + base1 : tau) : 0u;
+            rec.max[0][k] = nI ? (on0 ? most0 : tau) : 0u; rec.max[1][k] = nI ? (on1 ? most1 : tau) : 0u;
             rec.max[2][k] = maxX;
         }
         __syncwarp();
@@ -189,7 +156,7 @@ cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const 
                                 const int32_t* knots, uint32_t k0, TimelineRec rec, uint32_t batches, int sms,
                                 cudaStream_t st) {
     // as many warps to a block as the windows leave room for (wide jitter: up to 114 KB of counters a stream and warp)
-    const size_t per_warp = (size_t)(host_cc.W[0] + host_cc.W[1]) * 33 * 4;
+    const size_t per_warp = (size_t)(host_cc.W[0] + host_cc.W[1]) * 32 * 4;
     const uint32_t warps = std::max<uint32_t>(1u, std::min<uint32_t>(kFreeWarps, (uint32_t)(100 * 1024 / per_warp)));
     const size_t smem = per_warp * warps;
     bool small = false;                                       // intervals below 32 ticks occur
