@@ -672,8 +672,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     //      requests (one a thread) or more; of the pair kernel, two to a multiprocessor, 2,048 requests or more
     const uint32_t sms = (uint32_t)c->sms, kMaxChunk = 65280;
     const size_t N1 = n ? n : 1;
-    bool tall = false;
-    for (const Slab& sl : slabs) tall = tall || sl.T > 1;
+    int tallest = 1;
+    for (const Slab& sl : slabs) tallest = std::max(tallest, sl.T);
     auto chunk_size = [&](size_t want, uint32_t least) {
         const size_t ch = ((N1 + want - 1) / want + 255) / 256 * 256;
         return (uint32_t)std::min<size_t>(std::max<size_t>(ch, least), kMaxChunk);
@@ -691,7 +691,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             }
         return v;
     };
-    const size_t at_once = (size_t)sms * grid_blocks_per_sm(tall ? 2 : 1);
+    const size_t at_once = (size_t)sms * grid_blocks_per_sm(tallest);
     const std::vector<Chunk> chunks = make_chunks(chunk_size(at_once * (N1 / at_once > 2 * 16384 ? 3 : 2), 256));
     std::vector<Chunk> pair_chunks;
     if (any_pairs) pair_chunks = make_chunks(chunk_size((size_t)2 * sms, 2048));
@@ -708,9 +708,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         for (size_t x = lists[k].slab0; x < lists[k].slab1; ++x) {
             Slab& sl = slabs[x];
             auto bytes = [&](const Batch& b) { return b.ttft * 4 + b.tbt * tbt_word + b.sums * 8; };
-            auto rows = [](int T) { return T == 1 ? 1 : T <= 4 ? 4 : 8; };
             std::vector<Batch>& bs = batches[k];
-            if (bs.empty() || bytes(bs.back()) > (256ull << 20) || rows(bs.back().T) != rows(sl.T) || sl.mixed || slabs[x - 1].mixed)
+            if (bs.empty() || bytes(bs.back()) > (256ull << 20) || grid_rows(bs.back().T) != grid_rows(sl.T) || sl.mixed || slabs[x - 1].mixed)
                 bs.push_back(Batch{x, 0, 1, 0, 0, 0});
             Batch& b = bs.back();
             sl.ttft = b.ttft; sl.tbt = b.tbt; sl.sums = b.sums;

@@ -43,6 +43,11 @@ constexpr int kMaxSeg = 2 * kGridCols + 2;
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr uint32_t kNoPolicy = 0xFFFFFFFFu;
 
+// Blocks to a multiprocessor by the rows a kernel is built for: what their registers allow without spilling.
+__host__ __device__ constexpr int blocks_for(int rows, bool wide) { return rows == 1 || (rows == 2 && !wide) ? 4 : rows <= 4 ? 3 : 2; }
+// The rows of the kernel that takes a slab of T.
+constexpr int rows_for(int T) { return T <= 1 ? 1 : T <= 2 ? 2 : T <= 4 ? 4 : 8; }
+
 // Sums of a run: what every row gets, and per row what migration changes.
 enum Base { B_TD = 0, B_PS, B_PD, B_DO, B_RACE, B_DW, B_TAU, B_TT, kBase };
 enum Lev { V_A = 0, V_B, V_C, V_N, V_TAU, kLev };      // tokens handed over, prefill of the target, delayed, count, TBTs in tau's bin
@@ -54,7 +59,7 @@ struct Smem {                                          // fixed part; the TBT hi
                                                        // the device-only run where windows are counted
     uint32_t sum[kBase + kGridRows * kLev];            // totals of the run in work
     uint32_t only_sum[4];                              // ... of the device-only run: requests, tokens, prompt tokens, TBTs in tau's bin
-    unsigned long long tt, only_tt;                    // ... and the sums of TTFTs
+    uint32_t tt[3], only_tt[3];                        // ... and the sums of TTFTs, in parts of 20 bits
     uint32_t ttft[kNBins], only_ttft[kNBins];
     uint32_t n_seg, n_list, flagged, ticket;
     int32_t key[kGridCols];                            // the columns' length thresholds
@@ -242,9 +247,20 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
     }
 }
 
-__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+// Adds the lanes' 64-bit shares (below 2^40 each) to a total kept in parts of 20 bits: three warp sums instead of a tree of
+// shuffles, and 32-bit additions in shared memory, which has no 64-bit ones of its own.
+__device__ __forceinline__ void add_wide(uint32_t (&to)[3], unsigned long long v) {
+    const uint32_t a = __reduce_add_sync(FULL, (uint32_t)v & 0xFFFFFu), b = __reduce_add_sync(FULL, (uint32_t)(v >> 20) & 0xFFFFFu);
+    const int lane = threadIdx.x & 31;
+    const unsigned long long t = (unsigned long long)a + ((unsigned long long)b << 20);
+    if (lane < 3) {
+        const uint32_t part = lane == 0 ? (uint32_t)t & 0xFFFFFu : lane == 1 ? (uint32_t)(t >> 20) & 0xFFFFFu : (uint32_t)(t >> 40);
+        if (part) atomicAdd(&to[lane], part);
+    }
+}
+__device__ __forceinline__ unsigned long long take_wide(uint32_t (&from)[3]) {
+    const unsigned long long v = from[0] + ((unsigned long long)from[1] << 20) + ((unsigned long long)from[2] << 40);
+    from[0] = from[1] = from[2] = 0;
     return v;
 }
 
@@ -267,16 +283,14 @@ __device__ __forceinline__ void share_out(Smem& sm, const Acc<NT>& s, int T) {
     }
     if (lo) atomicAdd(&sm.sum[lane], lo);
     if (NT * kLev + kBase > 32 && hi) atomicAdd(&sm.sum[32 + lane], hi);
-    const unsigned long long tt = warp_sum(s.tt);
-    if (lane == 0 && tt) atomicAdd(&sm.tt, tt);
+    add_wide(sm.tt, s.tt);
 }
 __device__ __forceinline__ void share_only(Smem& sm, const Only& o) {
     const uint32_t c = __reduce_add_sync(FULL, o.cnt), n = __reduce_add_sync(FULL, o.n), l = __reduce_add_sync(FULL, o.l),
                    tau = __reduce_add_sync(FULL, o.tau);
-    const unsigned long long tt = warp_sum(o.tt);
+    add_wide(sm.only_tt, o.tt);
     if ((threadIdx.x & 31) == 0 && c) {
         atomicAdd(&sm.only_sum[0], c); atomicAdd(&sm.only_sum[1], n); atomicAdd(&sm.only_sum[2], l); atomicAdd(&sm.only_sum[3], tau);
-        atomicAdd(&sm.only_tt, tt);
     }
 }
 
@@ -324,7 +338,7 @@ __device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE
     for (int f = threadIdx.x; f < F; f += kThreads) {
         unsigned long long x = (f >= kBase && (f - kBase) % kLev == V_TAU) ? (unsigned long long)(long long)(int32_t)sm.sum[f] : sm.sum[f];
         sm.sum[f] = 0;
-        if (f == B_TT) { x = sm.tt; sm.tt = 0; }
+        if (f == B_TT) x = take_wide(sm.tt);
         if (!x) continue;
         if (neg) x = 0ull - x;
         atomicAdd(&tb.sum_row(g, q0)[f], x);
@@ -357,8 +371,8 @@ __device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const T
     }
     if (threadIdx.x < 5) {
         const int k = threadIdx.x;
-        const unsigned long long x = k < 4 ? (unsigned long long)sm.only_sum[k] : sm.only_tt;
-        if (k < 4) sm.only_sum[k] = 0; else sm.only_tt = 0;
+        const unsigned long long x = k < 4 ? (unsigned long long)sm.only_sum[k] : take_wide(sm.only_tt);
+        if (k < 4) sm.only_sum[k] = 0;
         const int f = k == 0 ? B_DO : k == 1 ? B_TD : k == 2 ? B_PD : k == 3 ? B_TAU : B_TT;
         if (x) {
             atomicAdd(&tb.sum_row(g, 0)[f], x);
@@ -368,7 +382,7 @@ __device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const T
 }
 
 template <int NT, bool WIDE>
-__global__ void __launch_bounds__(kThreads, NT == 1 ? 4 : 2)
+__global__ void __launch_bounds__(kThreads, blocks_for(NT, WIDE))
 k_grid(const __grid_constant__ Args a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
@@ -666,7 +680,7 @@ cudaError_t launch_one(const Args& a, int sms, cudaStream_t st) {
     cudaError_t e = allow_smem((const void*)k_grid<NT, WIDE>, smem);
     if (e) return e;
     const uint64_t items = (uint64_t)a.n_chunks * a.n_slabs;
-    const uint32_t blocks = (uint32_t)std::min<uint64_t>(items, (uint64_t)sms * (NT == 1 ? 4 : 2));
+    const uint32_t blocks = (uint32_t)std::min<uint64_t>(items, (uint64_t)sms * blocks_for(NT, WIDE));
     return launch_after(k_grid<NT, WIDE>, dim3(blocks), kThreads, smem, st, a);
 }
 
@@ -677,7 +691,8 @@ DBG_TRANSLATION_UNIT()
 uint64_t grid_ttft_words(int K) { return (uint64_t)K * kNBins; }
 uint64_t grid_tbt_words(int K, int T) { return (uint64_t)K * T * kNBins; }
 uint64_t grid_sum_words(int K, int T, int G) { return (uint64_t)G * K * sum_fields(T); }
-uint32_t grid_blocks_per_sm(int T) { return T == 1 ? 4 : 2; }
+uint32_t grid_blocks_per_sm(int T) { return (uint32_t)blocks_for(rows_for(T), false); }
+int grid_rows(int T) { return rows_for(T); }
 
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
                         const Slab* slabs, uint32_t n_slabs, int T, bool wide, bool count_pairs, const uint32_t* tab,
@@ -687,8 +702,12 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
     if ((uint64_t)n_chunks * n_slabs > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
     const Args a = {tr, rec, gc, cc, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, k0, ticket,
                     (unsigned long long*)work, count_pairs ? 1 : 0};
-    if (wide) return T == 1 ? launch_one<1, true>(a, sms, st) : T <= 4 ? launch_one<4, true>(a, sms, st) : launch_one<8, true>(a, sms, st);
-    return T == 1 ? launch_one<1, false>(a, sms, st) : T <= 4 ? launch_one<4, false>(a, sms, st) : launch_one<8, false>(a, sms, st);
+    switch (rows_for(T)) {
+        case 1: return wide ? launch_one<1, true>(a, sms, st) : launch_one<1, false>(a, sms, st);
+        case 2: return wide ? launch_one<2, true>(a, sms, st) : launch_one<2, false>(a, sms, st);
+        case 4: return wide ? launch_one<4, true>(a, sms, st) : launch_one<4, false>(a, sms, st);
+        default: return wide ? launch_one<8, true>(a, sms, st) : launch_one<8, false>(a, sms, st);
+    }
 }
 
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
