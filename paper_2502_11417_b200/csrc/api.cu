@@ -144,10 +144,11 @@ struct disco_ctx {
     uint32_t P = 0;
     bool evaluated = false, reduced = false;
     std::vector<PolicyConst> pol;
-    DevBuf eval_mem;             // one buffer for everything an evaluation writes
+    DevBuf rec_mem;              // what the play-out writes
+    DevBuf eval_mem;             // one buffer for everything else an evaluation writes
     View d_prep, d_accum, d_stats, d_tables, d_grid, d_left;
     View d_acc, d_hist_ttft, d_hist_tbt, d_work;          // regions of d_accum; d_work: the counters in front of d_grid
-    View rec_hand, rec_u32[6], rec_win[3];
+    View play_ticket, rec_hand, rec_u32[6], rec_win[3];      // regions of rec_mem
     void* stage = nullptr;       // pinned staging for the small host->device tables
     size_t stage_cap = 0;
     cudaEvent_t stage_free = nullptr;
@@ -163,7 +164,7 @@ struct disco_ctx {
     bool timing_valid = false;
 
     ~disco_ctx() {
-        DevBuf* all[] = {&trace_mem, &d_gc, &keys_a, &keys_b, &radix_counts, &sort_in, &F_sorted_imp, &F_off_imp, &eval_mem};
+        DevBuf* all[] = {&trace_mem, &d_gc, &keys_a, &keys_b, &radix_counts, &sort_in, &F_sorted_imp, &F_off_imp, &rec_mem, &eval_mem};
         for (DevBuf* b : all) b->release();
         if (rb) cudaFreeHost(rb);
         if (stage) cudaFreeHost(stage);
@@ -450,6 +451,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     std::vector<ClassConst> classes;
     bool any_beta = false;                // some policy uses the Eq. 1-2 wait rule
     bool extras = false;                  // some policy routes at random or triggers on an expected length
+    int64_t tau = 0, t_m = 0;
     for (uint32_t p = 0; p < P; ++p) {
         const disco_policy_t& q = pol[p];
         auto at = [p] { return " (policy " + std::to_string(p) + ")"; };
@@ -462,7 +464,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         if (mode == 3 || (q.flags >> 6)) return fail(DISCO_EINVAL, "unknown flags" + at());
         if (q.expected_len > (1u << 20)) return fail(DISCO_EINVAL, "expected length too large" + at());
         if (q.l_immediate > (uint32_t)kMaxPrompt) return fail(DISCO_EINVAL, "l_immediate above the longest prompt" + at());
-        const int64_t tau = ticks_of_rate(q.r_c), t_m = ticks_of_seconds(q.t_m_s);
+        if (p == 0 || q.r_c != pol[p - 1].r_c || q.t_m_s != pol[p - 1].t_m_s) { tau = ticks_of_rate(q.r_c); t_m = ticks_of_seconds(q.t_m_s); }
         if (tau < 1 || tau >= (1 << 30)) return fail(DISCO_EINVAL, "consumption interval outside 1 .. 2^30 ticks" + at());
         const bool pacing = (q.flags & DISCO_FLAG_PACING) != 0, mig = (q.flags & DISCO_FLAG_MIGRATION) != 0;
         int64_t B = pacing ? (t_m + tau - 1) / tau : 0;               // Eq. 6, rounded up
@@ -551,6 +553,47 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             return fail(DISCO_ENOMEM, "per-request TBT windows would exceed 48 GB");
     }
 
+    // ---- the first class's play-out needs no more than this: it runs while the host lays out the policies
+    cudaError_t e;
+    const size_t N1 = n ? n : 1;
+    {
+        Layout lay;
+        const size_t o_ticket = lay.take(4), o_hand = lay.take(N1 * 8);
+        size_t o_rec[6] = {}, o_win[3] = {};
+        if (stored) {
+            for (int k = 0; k < 6; ++k) o_rec[k] = lay.take(N1 * 4);
+            for (int k = 0; k < 3; ++k) o_win[k] = lay.take(N1 * wmax[k] * 2);
+        }
+        if ((e = c->rec_mem.reserve(lay.bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
+        char* mem = (char*)c->rec_mem.p;
+        c->play_ticket.p = mem + o_ticket; c->rec_hand.p = mem + o_hand;
+        for (int k = 0; k < 6; ++k) c->rec_u32[k].p = mem + o_rec[k];
+        for (int k = 0; k < 3; ++k) c->rec_win[k].p = mem + o_win[k];
+    }
+    TraceDev tr;
+    tr.n = n; tr.n_groups = G; tr.req = c->req.as<uint4>(); tr.inv = c->inv.as<uint32_t>();
+    tr.len_end = c->len_end.as<uint32_t>(); tr.grp_off = c->grp_off.as<uint32_t>();
+    TimelineRec rec;
+    rec.hand = c->rec_hand.as<uint2>();
+    for (int k = 0; k < 3; ++k) {
+        rec.sum[k] = c->rec_u32[2 * k].as<uint32_t>(); rec.max[k] = c->rec_u32[2 * k + 1].as<uint32_t>();
+        rec.win[k] = c->rec_win[k].as<uint16_t>();
+    }
+    const GroupConst* gc = c->d_gc.as<GroupConst>();
+    uint64_t out_tokens = 0;
+    for (int g = 0; g < G; ++g) out_tokens += rb.grp_sum_n[g];
+    const bool long_outputs = out_tokens >= 512ull * n;
+    // the hash is keyed by the request's index in the whole trace: key = mix(k0 + (first_index + i) * C_REQ)
+    const uint32_t k0 = seed_key(seed) + (uint32_t)c->first_index * kHashReq;
+    c->timing_valid = false;
+    const bool timed = c->timing && classes.size() == 1;
+    auto play_out = [&](size_t k) {
+        g_launches += timeline_launches(plan[k].kinds);
+        return launch_timeline(tr, gc, classes[k], c->knots.as<int32_t>(), k0, rec, c->err, c->play_ticket.as<uint32_t>(),
+                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, c->sms, st);
+    };
+    if (n != 0 && !timed) CU(play_out(0));
+
     // ---- the policies of a class: plain ones form grids of budgets by overheads (grid.cu), at most kGridCols by kGridRows
     //      to a slab; random routing and the Eq. 1-2 rule go pair by pair
     std::vector<uint32_t> tab;                     // lists of policy indices, one after the other
@@ -572,7 +615,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     };
     struct Grid { uint32_t flags, expected_len; float alpha; std::vector<uint32_t> pols; std::vector<float> budgets, thetas; size_t b_at, t_at; };
     std::vector<Grid> grids;
-    std::vector<uint32_t> cells, used;
+    std::vector<uint32_t> cells, used, wide, cell_of;
     for (size_t k = 0; k < classes.size(); ++k) {
         ClassLists& L = lists[k];
         L.all = tab.size();
@@ -647,20 +690,22 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 // how many policies share a (budget, overhead): those after the first take further columns of their budget
                 used.assign(n_b * T, 0);
                 size_t b_at = 0, t_at = 0;
-                std::vector<uint32_t> wide(n_b, 0);
-                for (uint32_t p : gr.pols) {
+                wide.assign(n_b, 0);
+                cell_of.resize(n_p);
+                for (size_t x = 0; x < n_p; ++x) {
+                    const uint32_t p = gr.pols[x];
                     place_of(gr.budgets, pc[p].budget, b_at); place_of(gr.thetas, theta_of(p), t_at);
-                    if (t_at >= r0 && t_at < r1) wide[b_at] = std::max(wide[b_at], ++used[b_at * T + (t_at - r0)]);
+                    cell_of[x] = kNone;
+                    if (t_at < r0 || t_at >= r1) continue;
+                    cell_of[x] = (uint32_t)(b_at * T + (t_at - r0));
+                    wide[b_at] = std::max(wide[b_at], ++used[cell_of[x]]);
                 }
                 size_t cols = 0;
                 for (uint32_t& w : wide) { const uint32_t here = w; w = (uint32_t)cols; cols += here; }
                 cells.assign(cols * T, kNone);
                 used.assign(n_b * T, 0);
-                b_at = t_at = 0;
-                for (uint32_t p : gr.pols) {
-                    place_of(gr.budgets, pc[p].budget, b_at); place_of(gr.thetas, theta_of(p), t_at);
-                    if (t_at >= r0 && t_at < r1) cells[(wide[b_at] + used[b_at * T + (t_at - r0)]++) * T + (t_at - r0)] = p;
-                }
+                for (size_t x = 0; x < n_p; ++x)
+                    if (cell_of[x] != kNone) cells[(wide[cell_of[x] / T] + used[cell_of[x]]++) * T + cell_of[x] % T] = gr.pols[x];
                 for (size_t c0 = 0; c0 < cols; c0 += kGridCols) close(sl, c0, std::min(cols, c0 + (size_t)kGridCols), 0u);
             }
         }
@@ -671,7 +716,6 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     //      where that is more than 16,384 requests: the end of the launch is then worth more than the entering of runs), 256
     //      requests (one a thread) or more; of the pair kernel, two to a multiprocessor, 2,048 requests or more
     const uint32_t sms = (uint32_t)c->sms, kMaxChunk = 65280;
-    const size_t N1 = n ? n : 1;
     int tallest = 1;
     for (const Slab& sl : slabs) tallest = std::max(tallest, sl.T);
     auto chunk_size = [&](size_t want, uint32_t least) {
@@ -702,7 +746,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     std::vector<std::vector<Batch>> batches(classes.size());
     uint64_t grid_bytes = 0;
     auto wide_class = [&](size_t k) { return (plan[k].kinds & ~(1u << G_EXACT)) != 0; };
-    uint32_t n_tickets = (uint32_t)classes.size();
+    uint32_t n_tickets = 0;
     for (size_t k = 0; k < classes.size(); ++k) {
         const uint64_t tbt_word = wide_class(k) ? 8 : 4;
         for (size_t x = lists[k].slab0; x < lists[k].slab1; ++x) {
@@ -724,7 +768,6 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     // ---- device memory: what must be clear comes first and together -- the work counters and tickets, the difference
     //      tables of the first batch, and the accumulators if some pairs are added to them one by one (k_spread writes those
     //      of all other policies)
-    cudaError_t e;
     const size_t acc_bytes = (size_t)P * G * kNAcc * 8, hist_bytes = (size_t)P * kNBins * 8;
     auto batch_bytes = [&](const Batch& b, bool wide) { return b.sums * 8 + b.tbt * (wide ? 8 : 4) + b.ttft * 4; };
     size_t first_bytes = 0;
@@ -739,12 +782,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const bool clear_apart = clear_bytes > (64ull << 30);                                     // (beyond its 32-bit index)
     const size_t o_prep = lay.take((size_t)G * P * sizeof(Prep)), o_stats = lay.take(P * sizeof(disco_policy_stats_t) + 16);
     const size_t o_accum2 = clear_accum ? o_accum : lay.take(acc_bytes + 2 * hist_bytes);
-    const size_t o_left = lay.take(any_mixed ? (N1 + kMaxGroups) * 4 : 0), o_hand = lay.take(N1 * 8);
-    size_t o_rec[6] = {}, o_win[3] = {};
-    if (stored) {
-        for (int k = 0; k < 6; ++k) o_rec[k] = lay.take(N1 * 4);
-        for (int k = 0; k < 3; ++k) o_win[k] = lay.take(N1 * wmax[k] * 2);
-    }
+    const size_t o_left = lay.take(any_mixed ? (N1 + kMaxGroups) * 4 : 0);
     const size_t table_bytes = ((size_t)P * sizeof(PolicyConst) + 15) / 16 * 16 + (classes.size() * sizeof(ClassConst) + 15) / 16 * 16 +
                                (tab.size() * 4 + 15) / 16 * 16 + (slabs.size() * sizeof(Slab) + 15) / 16 * 16 +
                                (chunks.size() + pair_chunks.size()) * sizeof(Chunk);
@@ -752,9 +790,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     if ((e = c->eval_mem.reserve(lay.bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
     char* mem = (char*)c->eval_mem.p;
     c->d_prep.p = mem + o_prep; c->d_accum.p = mem + o_accum2; c->d_stats.p = mem + o_stats; c->d_grid.p = mem + o_grid;
-    c->d_left.p = mem + o_left; c->d_tables.p = mem + o_tables; c->rec_hand.p = mem + o_hand;
-    for (int k = 0; k < 6; ++k) c->rec_u32[k].p = mem + o_rec[k];
-    for (int k = 0; k < 3; ++k) c->rec_win[k].p = mem + o_win[k];
+    c->d_left.p = mem + o_left; c->d_tables.p = mem + o_tables;
     c->d_acc.p = c->d_accum.p; c->d_hist_ttft.p = (char*)c->d_accum.p + acc_bytes;
     c->d_hist_tbt.p = (char*)c->d_accum.p + acc_bytes + hist_bytes;
     c->d_work.p = mem + o_work;
@@ -797,31 +833,14 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         g_launches += 1;
     }
 
-    TraceDev tr;
-    tr.n = n; tr.n_groups = G; tr.req = c->req.as<uint4>(); tr.inv = c->inv.as<uint32_t>();
-    tr.len_end = c->len_end.as<uint32_t>(); tr.grp_off = c->grp_off.as<uint32_t>();
-    TimelineRec rec;
-    rec.hand = c->rec_hand.as<uint2>();
-    for (int k = 0; k < 3; ++k) {
-        rec.sum[k] = c->rec_u32[2 * k].as<uint32_t>(); rec.max[k] = c->rec_u32[2 * k + 1].as<uint32_t>();
-        rec.win[k] = c->rec_win[k].as<uint16_t>();
-    }
     disco_pair_out_t po;
     std::memset(&po, 0, sizeof po);
     if (out) po = *out;
     const bool rows = po.ttft_s || po.tbt_mean_s || po.tbt_max_s || po.cost || po.tok_server || po.tok_device || po.mig_at ||
                       po.delayed || po.decision;
 
-    uint64_t out_tokens = 0;
-    for (int g = 0; g < G; ++g) out_tokens += rb.grp_sum_n[g];
-    const bool long_outputs = out_tokens >= 512ull * n;
-    // the hash is keyed by the request's index in the whole trace: key = mix(k0 + (first_index + i) * C_REQ)
-    const uint32_t k0 = seed_key(seed) + (uint32_t)c->first_index * kHashReq;
-    c->timing_valid = false;
-    const bool timed = c->timing && classes.size() == 1;
-    uint32_t ticket = (uint32_t)classes.size();
+    uint32_t ticket = 0;
     const Prep* prep = c->d_prep.as<Prep>();
-    const GroupConst* gc = c->d_gc.as<GroupConst>();
     uint64_t *acc = c->d_acc.as<uint64_t>(), *h_ttft = c->d_hist_ttft.as<uint64_t>(), *h_tbt = c->d_hist_tbt.as<uint64_t>(),
              *work = c->d_work.as<uint64_t>();
     bool first_batch = true;
@@ -830,9 +849,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         const ClassConst* dcc = d_classes + k;
         const bool wide = wide_class(k);
         if (timed) CU(cudaEventRecord(c->ev[0], st));
-        CU(launch_timeline(tr, gc, dcc, classes[k], c->knots.as<int32_t>(), k0, rec, c->err, tickets + k, plan[k].kinds,
-                           plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, c->sms, st));
-        g_launches += timeline_launches(plan[k].kinds);
+        if (k != 0 || timed) CU(play_out(k));
         if (timed) CU(cudaEventRecord(c->ev[2], st));
         for (const Batch& b : batches[k]) {
             GridTables gt;

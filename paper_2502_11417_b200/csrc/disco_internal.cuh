@@ -239,9 +239,8 @@ cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, int G, const in
                              Prep* prep, cudaStream_t st);
 // Plays every request under one class.  `kinds`: bit k set if some group with requests is of GroupKind k; `batches[k]`:
 // batches of 32 requests of the groups of kind k.
-cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const ClassConst& host_cc,
-                            const int32_t* knots, uint32_t k0 /* hash key base: seed_key(seed) + first_index * kHashReq */,
-                            TimelineRec rec, int32_t* err, uint32_t* ticket /* one word, zero */, uint32_t kinds,
+cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0 /* hash key base: seed_key(seed) + first_index * kHashReq */,
+                            TimelineRec rec, int32_t* err, uint32_t* ticket /* one word */, uint32_t kinds,
                             const uint32_t* batches, uint32_t search /* largest ClassConst::search of a group with requests */,
                             bool long_outputs /* mean output length of 512 tokens or more */,
                             cudaEvent_t mid /* recorded between the kernels of exact groups and the others, or null */,

@@ -56,12 +56,11 @@ __device__ __forceinline__ uint32_t walk(uint32_t key, uint32_t j0, int cnt, int
 // rpw = requests per ticket (8, 16 or 32): small traces use small batches so that enough warps are in flight.
 template <int PER>
 __global__ void __launch_bounds__(kFastWarps * 32)
-k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
+k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, uint32_t* __restrict__ tickets, int rpw,
                uint32_t one) {
     const int lane = threadIdx.x & 31;
     grid_dependency_wait();
-    const ClassConst& cc = *ccp;
     const int32_t tau = cc.tau;                                   // pacing is on for every launch of this kernel
     const uint32_t B = (uint32_t)cc.B;
     const long long thr64 = (long long)(B ? B - 1 : 0) * tau;
@@ -251,29 +250,29 @@ struct ShortGroup {                      // a group under the class
 };
 
 __global__ void __launch_bounds__(kShortThreads)
-k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
+k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
                 const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int per) {
     __shared__ ShortGroup groups[kMaxGroups];
     __shared__ uint4 lag[kShortThreads * kShortPer];         // hash key, lag, output length | hand-off << 16, place | group << 16
     __shared__ uint16_t rest[kShortThreads * kShortPer];     // lags that a thread has not made up
     __shared__ int n_lag, n_long, n_rest;
     grid_dependency_wait();
-    const int32_t tau = ccp->tau;
-    const uint32_t B = (uint32_t)ccp->B;
+    const int32_t tau = cc.tau;
+    const uint32_t B = (uint32_t)cc.B;
     const long long thr64 = (long long)(B ? B - 1 : 0) * tau;
     const int32_t thr = thr64 > 0x7FFFFFFFLL ? 0x7FFFFFFF : (int32_t)thr64;
     if (threadIdx.x == 0) { n_lag = 0; n_long = 0; n_rest = 0; }
     for (int g = threadIdx.x; g < tr.n_groups; g += kShortThreads) {
         const GroupConst& gc = gcs[g];
         ShortGroup G;
-        G.cand = ccp->mig_any ? gc.candidate : 0;
+        G.cand = cc.mig_any ? gc.candidate : 0;
         const uint32_t mulS = 2u * (uint32_t)gc.J_srv + 1u, mulD = 2u * (uint32_t)gc.J_dev + 1u;
         const int32_t cS = tau - (gc.T_srv - gc.J_srv), cD = tau - (gc.T_dev - gc.J_dev);
         G.mulC = G.cand == 2 ? mulD : mulS; G.mulT = G.cand == 2 ? mulS : mulD;
         G.cC = G.cand == 2 ? cD : cS; G.cT = G.cand == 2 ? cS : cD;
         G.kappa = (uint32_t)gc.kappa; G.c0 = (uint32_t)gc.c0;
         G.end = tr.grp_off[g + 1];
-        G.exact = ccp->kind[g] == G_EXACT;
+        G.exact = cc.kind[g] == G_EXACT;
         G.cT_mean = G.cT - (int32_t)(G.mulT >> 1);
         groups[g] = G;
     }
@@ -369,7 +368,7 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassCons
 
 DBG_TRANSLATION_UNIT()
 
-cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const int32_t* knots,
+cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots,
                                  uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, int sms,
                                  cudaStream_t st) {
     if (search <= kShortSearch) {
@@ -384,6 +383,8 @@ cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const
     const uint32_t per_block = kFastWarps * (uint32_t)rpw;
     // requests per round: eight halve the cost of a round per request; with long outputs the token loop is
     // what counts, and four requests split the lanes more evenly
+    cudaError_t e = cudaMemsetAsync(ticket, 0, 4, st);
+    if (e) return e;
     auto* kernel = long_outputs ? k_playout_fast<4> : k_playout_fast<8>;
     // as many blocks as the GPU holds at once (at most six of these per SM); the ticket counter feeds them
     const uint32_t blocks = std::min<uint32_t>((tr.n + per_block - 1) / per_block, (uint32_t)sms * 6u);

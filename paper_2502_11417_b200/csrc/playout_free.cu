@@ -37,12 +37,11 @@ __device__ __forceinline__ void count_in(const Counters& c, uint32_t x, uint32_t
 // kernel for all cases the warps waited for instructions four cycles of every ten.)
 template <bool BOTH, bool SMALL>
 __global__ void __launch_bounds__(kFreeWarps * 32, 4)
-k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* __restrict__ ccp,
+k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec) {
     extern __shared__ __align__(16) uint32_t s_win[];         // per warp: [W0 + W1][32] counters
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warps = blockDim.x >> 5;
     grid_dependency_wait();
-    const ClassConst& cc = *ccp;
     const int W0 = cc.W[0], W1 = cc.W[1], WW = W0 + W1;
     uint32_t* win = s_win + wib * (WW * 32);
     for (int b = lane; b < WW * 32; b += 32) win[b] = 0;
@@ -152,16 +151,15 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst
 
 DBG_TRANSLATION_UNIT()
 
-cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const ClassConst& host_cc,
-                                const int32_t* knots, uint32_t k0, TimelineRec rec, uint32_t batches, int sms,
+cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0, TimelineRec rec, uint32_t batches, int sms,
                                 cudaStream_t st) {
     // as many warps to a block as the windows leave room for (wide jitter: up to 114 KB of counters a stream and warp)
-    const size_t per_warp = (size_t)(host_cc.W[0] + host_cc.W[1]) * 32 * 4;
+    const size_t per_warp = (size_t)(cc.W[0] + cc.W[1]) * 32 * 4;
     const uint32_t warps = std::max<uint32_t>(1u, std::min<uint32_t>(kFreeWarps, (uint32_t)(100 * 1024 / per_warp)));
     const size_t smem = per_warp * warps;
     bool small = false;                                       // intervals below 32 ticks occur
-    for (int g = 0; g < tr.n_groups; ++g) small = small || host_cc.lo[g][0] < 32 || host_cc.lo[g][1] < 32;
-    auto* kernel = host_cc.pacing ? (small ? k_playout_free<false, true> : k_playout_free<false, false>)
+    for (int g = 0; g < tr.n_groups; ++g) small = small || cc.lo[g][0] < 32 || cc.lo[g][1] < 32;
+    auto* kernel = cc.pacing ? (small ? k_playout_free<false, true> : k_playout_free<false, false>)
                                   : (small ? k_playout_free<true, true> : k_playout_free<true, false>);
     cudaError_t e;
     if ((e = allow_smem((const void*)kernel, 227 * 1024))) return e;
