@@ -7,6 +7,7 @@
 #include <cstring>
 #include <memory>
 #include <new>
+#include <numeric>
 #include <string>
 #include <vector>
 
@@ -619,23 +620,30 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     for (size_t k = 0; k < classes.size(); ++k) {
         ClassLists& L = lists[k];
         L.all = tab.size();
-        for (uint32_t p = 0; p < P; ++p) if (pc[p].cls == (int)k) tab.push_back(p);
+        if (classes.size() == 1) {
+            tab.resize(P);
+            std::iota(tab.begin(), tab.end(), 0u);
+        } else {
+            for (uint32_t p = 0; p < P; ++p) if (pc[p].cls == (int)k) tab.push_back(p);
+        }
         L.n_all = tab.size() - L.all;
         L.ext = tab.size();
         L.slab0 = slabs.size();
         grids.clear();
+        Grid* last = nullptr;
         for (size_t i = L.all; i < L.all + L.n_all; ++i) {
             const uint32_t p = tab[i];
             const PolicyConst& q = pc[p];
             if (q.flags & (DISCO_FLAG_STOCHASTIC | DISCO_FLAG_BETA_RULE)) { tab.push_back(p); continue; }
-            Grid* at = nullptr;
-            for (size_t x = grids.size(); x-- > 0 && !at;)
-                if (grids[x].flags == q.flags && grids[x].expected_len == q.expected_len && grids[x].alpha == q.alpha) at = &grids[x];
+            auto same = [&](const Grid& gr) { return gr.flags == q.flags && gr.expected_len == q.expected_len && gr.alpha == q.alpha; };
+            Grid* at = last && same(*last) ? last : nullptr;           // (mostly the one of the policy before)
+            for (size_t x = grids.size(); x-- > 0 && !at;) if (same(grids[x])) at = &grids[x];
             if (!at) {
                 grids.push_back(Grid{q.flags, q.expected_len, q.alpha, {}, {}, {}, 0, 0});
                 at = &grids.back();
                 at->pols.reserve(L.n_all);
             }
+            last = at;
             at->pols.push_back(p);
             place_of(at->budgets, q.budget, at->b_at);
             place_of(at->thetas, theta_of(p), at->t_at);
@@ -656,11 +664,14 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 const size_t T = (size_t)sl.T;
                 sl.K = (int32_t)(c1 - c0);
                 sl.cols = (uint32_t)tab.size();
-                for (size_t x = c0; x < c1; ++x)
-                    for (size_t r = 0; r < T; ++r) if (cells[x * T + r] != kNone) { tab.push_back(cells[x * T + r]); break; }
+                for (size_t x = c0; x < c1; ++x) {
+                    size_t r = 0;
+                    while (cells[x * T + r] == kNone) ++r;             // (a column has a policy)
+                    tab.push_back(cells[x * T + r]);
+                }
                 sl.cells = (uint32_t)tab.size();
-                for (size_t x = c0 * T; x < c1 * T; ++x) sl.policies += cells[x] != kNone;
                 tab.insert(tab.end(), cells.begin() + c0 * T, cells.begin() + c1 * T);
+                sl.policies = (uint32_t)((c1 - c0) * T - std::count(cells.begin() + c0 * T, cells.begin() + c1 * T, kNone));
                 slabs.push_back(sl);
                 mixed_pols.push_back(listed);
             };
@@ -688,7 +699,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 Slab sl = open((int)T, false);
                 for (size_t r = r0; r < r1; ++r) sl.theta[r - r0] = gr.thetas[r];
                 // how many policies share a (budget, overhead): those after the first take further columns of their budget
-                used.assign(n_b * T, 0);
+                used.assign(n_b * kGridRows, 0);
                 size_t b_at = 0, t_at = 0;
                 wide.assign(n_b, 0);
                 cell_of.resize(n_p);
@@ -697,15 +708,15 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                     place_of(gr.budgets, pc[p].budget, b_at); place_of(gr.thetas, theta_of(p), t_at);
                     cell_of[x] = kNone;
                     if (t_at < r0 || t_at >= r1) continue;
-                    cell_of[x] = (uint32_t)(b_at * T + (t_at - r0));
+                    cell_of[x] = (uint32_t)(b_at * kGridRows + (t_at - r0));                 // (budget, overhead)
                     wide[b_at] = std::max(wide[b_at], ++used[cell_of[x]]);
                 }
                 size_t cols = 0;
                 for (uint32_t& w : wide) { const uint32_t here = w; w = (uint32_t)cols; cols += here; }
                 cells.assign(cols * T, kNone);
-                used.assign(n_b * T, 0);
+                used.assign(n_b * kGridRows, 0);
                 for (size_t x = 0; x < n_p; ++x)
-                    if (cell_of[x] != kNone) cells[(wide[cell_of[x] / T] + used[cell_of[x]]++) * T + cell_of[x] % T] = gr.pols[x];
+                    if (cell_of[x] != kNone) cells[(wide[cell_of[x] / kGridRows] + used[cell_of[x]]++) * T + cell_of[x] % kGridRows] = gr.pols[x];
                 for (size_t c0 = 0; c0 < cols; c0 += kGridCols) close(sl, c0, std::min(cols, c0 + (size_t)kGridCols), 0u);
             }
         }
@@ -727,6 +738,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     // some blocks already idle) should be the cheap ones
     auto make_chunks = [&](uint32_t CH) {
         std::vector<Chunk> v;
+        v.reserve(N1 / CH + (size_t)G + 1);
         for (int dear = 1; dear >= 0; --dear)
             for (int g = 0; g < G; ++g) {
                 if ((c->gc[g].auto_device_constrained != 0) != (dear != 0)) continue;
