@@ -61,7 +61,7 @@ struct Smem {                                          // fixed part; the TBT hi
     uint32_t only_sum[4];                              // ... of the device-only run: requests, tokens, prompt tokens, TBTs in tau's bin
     uint32_t tt[3], only_tt[3];                        // ... and the sums of TTFTs, in parts of 20 bits
     uint32_t ttft[kNBins], only_ttft[kNBins];
-    uint32_t n_seg, n_list, flagged, ticket;
+    uint32_t n_seg, n_runs, n_list, flagged, ticket;
     int32_t key[kGridCols];                            // the columns' length thresholds
     uint32_t w_star[kGridCols], w_tail[kGridCols];
     Seg seg[kMaxSeg];
@@ -381,6 +381,80 @@ __device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const T
     }
 }
 
+// A chunk whose runs have few requests each, request by request: a thread enters what its request comes to in every run by
+// itself.  A run swept by the whole block costs its barriers and a walk over all bins (a microsecond or more), which pays
+// only with enough requests to share it.  Bound: the chain of atomics per request, and, with many of them, the L2 slices
+// that the hottest sums live in (lanes that add up first were tried: shorter there, but longer where the lanes' columns
+// differ).  A step of 1,000 requests under 256 budgets 465 -> 114 us, of 10,000 requests under 256 policies with
+// migration 785 -> 185 us.
+//
+// Taken below so many requests to a run: where every block has at most one item the step waits for the slowest item, and
+// the runs' latency decides (64; nothing changes beyond); with more items than blocks the atomics' rate does, and at 24
+// requests to a run 300,000 requests under 128 policies with migration already lose (286 us against 230, 202 at 16).
+constexpr uint32_t kDirectAlone = 64, kDirectMany = 16;
+
+template <int NT>
+__device__ __noinline__ void enter_requests(const Args& a, const Ctx& c, const float (&th)[NT], const Smem& sm,
+                                            const Tables<false>& tb, bool waits, uint32_t wt_min, int n_low) {
+    const int K = c.K;
+    for (uint32_t i = threadIdx.x; i < c.len; i += kThreads) {
+        const uint32_t kk = c.start + i;
+        const uint4 q = a.tr.req[kk];
+        const uint2 hand = c.may_migrate ? a.rec.hand[kk] : make_uint2(0u, 0u);
+        const uint32_t S = q.x, l = q.y & 0xFFFFu, n = q.y >> 16, m = hand.x & 0xFFFFu, dly = hand.x >> 16;
+        const uint32_t Td = c.kappa * l + c.c0;
+        const float saving = m ? c.delta_c * (float)(c.E0 ? max(c.E0 - (int)m, 0) : (int)(n - m)) : -1.0f;
+        if (c.mixed && saving > c.th_lo && !(saving > th[0])) continue;               // left to the pair kernel
+        // adds (or takes) a count to a histogram of the columns [q0, q1), a value to a sum
+        auto count = [&](uint32_t* at, int q0, int q1) {
+            atomicAdd(at + (size_t)q0 * kNBins, 1u);
+            if (q1 < K) atomicAdd(at + (size_t)q1 * kNBins, ~0u);
+        };
+        const size_t F = sum_fields(c.T);
+        auto add = [&](int f, unsigned long long v, int q0, int q1) {
+            unsigned long long* at = tb.sum_row(c.g, 0) + f;
+            atomicAdd(at + q0 * F, v);
+            if (q1 < K) atomicAdd(at + q1 * F, 0ull - v);
+        };
+        // what the request comes to under the columns [q0, q1), which start the device after w
+        auto enter_run = [&](uint32_t w, int q0, int q1) {
+            const bool started = S > w, dev_wins = S > w + Td;
+            const uint32_t tt = min(S, w + Td);
+            const int bin = bin_of_ticks(tt);
+            if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) count(tb.ttft + bin, q0, q1);
+            if (dev_wins) { add(B_TD, n, q0, q1); add(B_DW, 1ull, q0, q1); }
+            add(B_PS, l, q0, q1);
+            if (started) { add(B_PD, l, q0, q1); add(B_RACE, 1ull, q0, q1); }
+            add(B_TAU, n - 1u, q0, q1); add(B_TT, tt, q0, q1);
+            if (!started || (dev_wins ? 2 : 1) != c.cand) return;
+            const int stall = bin_of_ticks(hand.y);
+#pragma unroll
+            for (int r = 0; r < NT; ++r) {
+                if (!(saving > th[r])) break;                                          // (overheads ascend)
+                const int f = kBase + r * kLev;
+                add(f + V_A, n - m, q0, q1); add(f + V_B, l + m, q0, q1); add(f + V_N, 1ull, q0, q1);
+                if (dly) add(f + V_C, dly, q0, q1);
+                if (DBG_OK(stall, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) count(tb.tbt + (size_t)r * K * kNBins + stall, q0, q1);
+            }
+        };
+        // the columns on either side of the request's length
+        int k1 = 0, k2;
+        for (int hi = K; k1 < hi;) { const int mid = (k1 + hi) >> 1; if (waits ? sm.key[mid] < (int)l : sm.key[mid] > (int)l) k1 = mid + 1; else hi = mid; }
+        k2 = k1;
+        if (waits) {
+            while (k2 < K && sm.key[k2] == (int)l) { enter_run(sm.w_star[k2], k2, k2 + 1); ++k2; }
+            const int low = S > wt_min ? min(n_low, k1) : 0;
+            for (int p = 0; p < low; ++p) enter_run(sm.w_tail[p], p, p + 1);
+            if (low < k1) enter_run(wt_min, low, k1);
+        } else if (k1 > 0) {                                                           // the device alone
+            const int bin = bin_of_ticks(Td);
+            if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) count(tb.ttft + bin, 0, k1);
+            add(B_DO, 1ull, 0, k1); add(B_TD, n, 0, k1); add(B_PD, l, 0, k1); add(B_TAU, n - 1u, 0, k1); add(B_TT, Td, 0, k1);
+        }
+        if (k2 < K) enter_run(0u, k2, K);
+    }
+}
+
 template <int NT, bool WIDE>
 __global__ void __launch_bounds__(kThreads, blocks_for(NT, WIDE))
 k_grid(const __grid_constant__ Args a) {
@@ -391,10 +465,11 @@ k_grid(const __grid_constant__ Args a) {
     for (int i = threadIdx.x; i < (int)(offsetof(Smem, key) / 4); i += kThreads) ((uint32_t*)&sm)[i] = 0;
     for (int i = threadIdx.x; i < (NT + (WIDE ? 1 : 0)) * kNBins; i += kThreads) tbt[i] = 0;
 
+    const uint32_t direct = a.n_chunks * a.n_slabs <= gridDim.x ? kDirectAlone : kDirectMany;
     // the blocks draw (chunk, slab) items from a counter (zero at launch): items differ in cost
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) { sm.ticket = atomicAdd(a.ticket, 1u); sm.n_seg = 0; sm.n_list = 0; sm.flagged = 0; }
+        if (threadIdx.x == 0) { sm.ticket = atomicAdd(a.ticket, 1u); sm.n_seg = 0; sm.n_runs = 0; sm.n_list = 0; sm.flagged = 0; }
         __syncthreads();
         const uint32_t item = sm.ticket;
         if (item >= a.n_chunks * a.n_slabs) break;
@@ -480,6 +555,7 @@ k_grid(const __grid_constant__ Args a) {
                 const uint32_t pa = min(max(at_a, lo), hi) - lo, pb = min(max(at_b, lo), hi) - lo;
                 if (pa < pb) {
                     const uint32_t at = atomicAdd(&sm.n_seg, 1u);
+                    atomicAdd(&sm.n_runs, waits ? (uint32_t)(k2 - k1) + (k1 > 0) + (k2 < K) : 1u);
                     if (DBG_OK(at, kMaxSeg, DBG_K_PAIRS_ZONES, DBG_SLOT))
                         sm.seg[at] = Seg{(uint16_t)pa, (uint16_t)pb, (uint16_t)k1, (uint16_t)k2};
                 }
@@ -506,7 +582,21 @@ k_grid(const __grid_constant__ Args a) {
             __syncthreads();
             ++passes;
         };
-        if (!waits) {
+        bool by_request = false;
+        if constexpr (!WIDE) {
+            by_request = c.len < (sm.n_runs + (n_low ? (uint32_t)n_low + 1u : 0u)) * direct;
+            if (by_request) {
+                const Ctx its = c;                                    // (copies: what is handed over by address lives in memory)
+                const Tables<false> tables = tb;
+                float rows[NT];
+#pragma unroll
+                for (int r = 0; r < NT; ++r) rows[r] = th[r];
+                enter_requests<NT>(a, its, rows, sm, tables, waits, wt_min, n_low);
+                passes = 1;
+            }
+        }
+        if (by_request) {
+        } else if (!waits) {
             for (int si = 0; si < n_seg; ++si) {
                 const Seg sg = sm.seg[si];
                 const bool race = (int)sg.k2 < K, only = sg.k1 > 0;

@@ -128,3 +128,15 @@ def test_pageable_traces_are_packed(n, profiles):
         with pytest.raises(DiscoError) as ei:
             Trace().load_trace(*wrong, w.servers, w.devices)
         assert ei.value.code == -1 and f"at request {at}" in str(ei.value)
+
+
+@pytest.mark.parametrize("dearer", [False, True])
+@pytest.mark.parametrize("n,budgets", [(1, 256), (31, 257), (700, 64), (700, 5), (5003, 256), (5003, 33)])
+def test_few_requests_to_a_run(n, budgets, dearer):
+    # small chunks under many thresholds are entered request by request, others run by run: both against the oracle, with
+    # one overhead and with three, under Algorithm 2 (the device dearer) and 3
+    w = synth.tiny_workload(99, n, n_servers=2, max_prompt=4096, max_out=60, device_dearer=dearer)
+    grid = synth.budget_grid(budgets)
+    full_parity(w, [synth.policy(b) for b in grid], select=False, tag=f"{n} {budgets}")
+    full_parity(w, [synth.policy(b, mig_threshold=t) for b in grid[::3] for t in (0.0, 1e-6, 3e-5)], select=False,
+                tag=f"{n} {budgets} x 3")
