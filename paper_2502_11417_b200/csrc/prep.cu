@@ -122,7 +122,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
             const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
             const uint32_t* __restrict__ tick_start, const uint32_t* __restrict__ tick_cnt, Prep* __restrict__ prep) {
     __shared__ uint32_t s_end[kTickBins];                             // ticks of the group up to the bin's last
-    __shared__ long long part[6][32];
+    __shared__ long long part[8][32], total[6];
     grid_dependency_wait();
     const int g = (int)(blockIdx.x / P);
     const uint32_t p = blockIdx.x % P;
@@ -161,23 +161,32 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
         len[i] = 1 + (int)threadIdx.x + i * kBetaThreads;
         k[i] = cnt[(size_t)g * (kMaxPrompt + 1) + len[i]];
     }
-    // the block's sums of the values, the same to all threads
+    // the block's sums of the values, the same to all threads.  Over a warp the lanes halve what they add up at every step
+    // (nine exchanges for six values, not thirty); a warp then adds up the warps' parts of one value for all.
     auto totals = [&](auto& v) {
-        constexpr int kValues = (int)(sizeof(v) / sizeof(v[0]));
+        constexpr int kValues = (int)(sizeof(v) / sizeof(v[0])), kHold = kValues <= 2 ? 2 : kValues <= 4 ? 4 : 8;
+        long long x[kHold];
 #pragma unroll
-        for (int j = 0; j < kValues; ++j) {
+        for (int j = 0; j < kHold; ++j) x[j] = j < kValues ? v[j] : 0ll;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(FULL, v[j], o);
-            if (lane == 0) part[j][wi] = v[j];
+        for (int s = kHold / 2, o = 16; s > 0; s >>= 1, o >>= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int j = 0; j < s; ++j) x[j] = (up ? x[j + s] : x[j]) + __shfl_xor_sync(FULL, up ? x[j] : x[j + s], o);
+        }
+#pragma unroll
+        for (int o = 16 / kHold; o > 0; o >>= 1) x[0] += __shfl_xor_sync(FULL, x[0], o);
+        if (lane % (32 / kHold) == 0) part[lane / (32 / kHold)][wi] = x[0];
+        __syncthreads();
+        if (wi < kValues) {
+            long long y = part[wi][lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(FULL, y, o);
+            if (lane == 0) total[wi] = y;
         }
         __syncthreads();
 #pragma unroll
-        for (int j = 0; j < kValues; ++j) {
-            v[j] = part[j][lane];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(FULL, v[j], o);
-        }
-        __syncthreads();
+        for (int j = 0; j < kValues; ++j) v[j] = total[j];
     };
     auto wait = [&](long long beta, int l) { return l <= l_imm ? 0ll : min(beta * (long long)l, w_tail); };
     long long lo = 0, hi = w_tail + 1;                                // beyond hi every wait is w_tail
