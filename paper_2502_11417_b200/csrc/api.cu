@@ -617,12 +617,18 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     struct Grid { uint32_t flags, expected_len; float alpha; std::vector<uint32_t> pols; std::vector<float> budgets, thetas; size_t b_at, t_at; };
     std::vector<Grid> grids;
     std::vector<uint32_t> cells, used, wide, cell_of;
+    const size_t beta_at = tab.size();             // (group, policy) pairs whose slope of Eq. 1-2 is searched for
+    for (int g = 0; any_beta && g < G; ++g)
+        for (uint32_t p = 0; p < P; ++p)
+            if ((pc[p].flags & DISCO_FLAG_BETA_RULE) && (pc[p].mode == 1 || (pc[p].mode == 0 && c->gc[g].auto_device_constrained)))
+                tab.push_back((uint32_t)g * P + p);
+    const uint32_t n_beta = (uint32_t)(tab.size() - beta_at);
     for (size_t k = 0; k < classes.size(); ++k) {
         ClassLists& L = lists[k];
         L.all = tab.size();
         if (classes.size() == 1) {
-            tab.resize(P);
-            std::iota(tab.begin(), tab.end(), 0u);
+            tab.resize(L.all + P);
+            std::iota(tab.begin() + L.all, tab.end(), 0u);
         } else {
             for (uint32_t p = 0; p < P; ++p) if (pc[p].cls == (int)k) tab.push_back(p);
         }
@@ -839,9 +845,9 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     CU(launch_prep(d_pol, P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
                    c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), mem, clear_apart ? 0 : clear_bytes, c->sms, st));
     g_launches += 1;
-    if (any_beta) {
-        CU(launch_prep_beta(d_pol, P, G, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
-                            c->F_off, c->tick_start.as<uint32_t>(), c->tick_cnt, c->d_prep.as<Prep>(), st));
+    if (n_beta) {
+        CU(launch_prep_beta(d_pol, P, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
+                            c->F_off, c->tick_start.as<uint32_t>(), c->tick_cnt, d_tab + beta_at, n_beta, c->d_prep.as<Prep>(), st));
         g_launches += 1;
     }
 

@@ -106,13 +106,25 @@ k_prep(const PolicyConst* __restrict__ pol, uint32_t P, int G, const GroupConst*
     if ((threadIdx.x & 31) == 0) prep[(size_t)g * P + p] = r;
 }
 
+// The largest whole x with (double)x <= limit (>= 0): sums are compared as whole numbers, since converting every sum in
+// every thread took most of a round of the search below (4,200 cycles a round with hardly a request to add up).
+__device__ long long last_within(double limit) {
+    if (limit >= 9223372036854774784.0) return 0x7FFFFFFFFFFFFFFFll;  // (the last double below 2^63)
+    const long long x = (long long)limit;                             // (rounded down)
+    if (limit < 9007199254740992.0) return x;                         // below 2^53 every whole number is a double
+    const long long half = 1ll << ((int)(__double_as_longlong(limit) >> 52) - 1023 - 53);    // of the doubles' distance there
+    return (double)(x + half) <= limit ? x + half : x + half - 1;     // (ties go to the even one)
+}
+
 // Eq. 1-2 variant of phase 2, one block per (group, policy): the smallest whole slope beta (ticks per prompt
 // token) with  sum_l l cnt[l] #{S > w(l)} <= b Total N,  w(l) = 0 for l <= l_immediate, min(beta l, w_tail) above.
 // The sum is exact (it is below Total N < 2^63); it does not grow with beta, so beta is found by search: three slopes a
 // round, which cut the range to a quarter.  A thread keeps four prompt lengths and, for each, the two positions in the
 // sorted ticks that belong to the ends of the range, between which the positions of the slopes in between lie; the first
 // and last positions come from the bins' starts in shared memory.  Bound: latency (two barriers and a few dependent loads a
-// round, eleven rounds).  (A bisection whose every step searched all the ticks for every length: 437 us.)
+// round, some fourteen rounds).  (300,000 requests in six groups under sixteen such policies: 437 us with a bisection whose
+// every step searched all the ticks for every length, 85 us now.  Four blocks a pair gave 4 us with few pairs and lost 15
+// once the pairs outnumbered the multiprocessors; three searches in step gave nothing.)
 constexpr int kBetaThreads = 1024;
 constexpr int kBetaLens = kMaxPrompt / kBetaThreads;                  // prompt lengths a thread has
 static_assert(kBetaLens * kBetaThreads == kMaxPrompt, "lengths 1 .. 4096");
@@ -120,12 +132,13 @@ static_assert(kBetaLens * kBetaThreads == kMaxPrompt, "lengths 1 .. 4096");
 __global__ void __launch_bounds__(kBetaThreads)
 k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __restrict__ cum_mass,
             const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
-            const uint32_t* __restrict__ tick_start, const uint32_t* __restrict__ tick_cnt, Prep* __restrict__ prep) {
+            const uint32_t* __restrict__ tick_start, const uint32_t* __restrict__ tick_cnt, const uint32_t* __restrict__ pairs,
+            Prep* __restrict__ prep) {
     __shared__ uint32_t s_end[kTickBins];                             // ticks of the group up to the bin's last
     __shared__ long long part[8][32], total[6];
     grid_dependency_wait();
-    const int g = (int)(blockIdx.x / P);
-    const uint32_t p = blockIdx.x % P;
+    const uint32_t pair = pairs[blockIdx.x], p = pair % P;
+    const int g = (int)(pair / P);
     Prep& out = prep[(size_t)g * P + p];
     const Prep pr = out;
     const PolicyConst pc = pol[p];
@@ -134,7 +147,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
     const uint32_t off = grp_off[g], N = grp_off[g + 1] - off;
     const int32_t* srt = sorted + off;
     const double Total = (double)cum_mass[(size_t)g * (kMaxPrompt + 2) + kMaxPrompt + 1];
-    const double limit = __dmul_rn(__dmul_rn((double)pc.budget, Total), (double)N);
+    const long long limit = last_within(__dmul_rn(__dmul_rn((double)pc.budget, Total), (double)N));
     const long long w_tail = pr.w_tail, l_imm = pr.l_star;
     for (int k = threadIdx.x; k < kTickBins; k += kBetaThreads)
         s_end[k] = tick_start[(size_t)g * kTickBins + k] + tick_cnt[(size_t)g * kTickBins + k] - off;
@@ -210,9 +223,9 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
         totals(v);
         const long long old_lo = lo, old_hi = hi;
 #pragma unroll
-        for (int j = 2; j >= 0; --j) if ((double)v[3 + j] <= limit && m[j] < hi) hi = m[j];      // certainly fits
+        for (int j = 2; j >= 0; --j) if (v[3 + j] <= limit && m[j] < hi) hi = m[j];      // certainly fits
 #pragma unroll
-        for (int j = 0; j < 3; ++j) if ((double)v[j] > limit && m[j] > lo && m[j] < hi) lo = m[j];   // certainly does not
+        for (int j = 0; j < 3; ++j) if (v[j] > limit && m[j] > lo && m[j] < hi) lo = m[j];   // certainly does not
         if (lo == old_lo && hi == old_hi) break;
     }
     // ---- the positions at the ends of what is left
@@ -228,8 +241,8 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
             v[1] += (long long)len[i] * (long long)k[i] * (long long)(N - at_hi[i]);
         }
         totals(v);
-        if (lo == 0 && (double)v[0] <= limit) hi = lo;                // (no waits at all fit)
-        else if ((double)v[1] > limit) lo = hi;                       // not even the longest waits fit
+        if (lo == 0 && v[0] <= limit) hi = lo;                // (no waits at all fit)
+        else if (v[1] > limit) lo = hi;                       // not even the longest waits fit
     }
     // the slope at lo is too small, that at hi fits
     while (hi - lo > 1) {
@@ -247,7 +260,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
             }
         }
         totals(v);
-        const int fit = (double)v[0] <= limit ? 0 : (double)v[1] <= limit ? 1 : (double)v[2] <= limit ? 2 : 3;   // first slope that fits
+        const int fit = v[0] <= limit ? 0 : v[1] <= limit ? 1 : v[2] <= limit ? 2 : 3;   // first slope that fits
         const long long old_lo = lo;
         lo = fit == 0 ? old_lo : fit == 1 ? m[0] : fit == 2 ? m[1] : m[2];
         hi = fit == 0 ? m[0] : fit == 1 ? m[1] : fit == 2 ? m[2] : hi;
@@ -273,11 +286,11 @@ cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupCo
     return launch_after(k_prep, blocks, kPrepThreads, 0, st, pol, P, G, gc, cum_mass, cnt, sorted, grp_off, prep, (uint4*)clear, vecs);
 }
 
-cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, int G, const int64_t* cum_mass, const uint32_t* cnt,
+cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off, const uint32_t* tick_start,
-                             const uint32_t* tick_cnt, Prep* prep, cudaStream_t st) {
-    return launch_after(k_prep_beta, P * (uint32_t)G, kBetaThreads, 0, st, pol, P, cum_mass, cnt, sorted, grp_off, tick_start,
-                        tick_cnt, prep);
+                             const uint32_t* tick_cnt, const uint32_t* pairs, uint32_t n_pairs, Prep* prep, cudaStream_t st) {
+    return launch_after(k_prep_beta, n_pairs, kBetaThreads, 0, st, pol, P, cum_mass, cnt, sorted, grp_off, tick_start,
+                        tick_cnt, pairs, prep);
 }
 
 }  // namespace disco
