@@ -33,43 +33,22 @@ METRIC = "request-policy evaluations/s"
 UNIT = "pairs/s"
 PAIR_OUT_BYTES = 31          # four fp32, three u32, one u16, one u8 per pair
 TRACE_BYTES = 9              # packed request: ticks, prompt, output length, group
-# Lane-instructions one token-step of the play-out needs.  General form (both endpoints' streams share the
-# hash draw): counter add 1, hash finaliser 8, two range maps (multiply-high) 2, tail mask 1, two sums and two
-# maxima 4, loop 1.  When no interval can exceed the consumption interval (tau >= T + J for both endpoints of
-# every group) only the stream of the endpoint that may hand over is summed: counter 1, hash 8, one range map
-# 1, tail test 1, sum 1, loop 1.
+# Bytes a request whose stream cannot fall behind the reader needs of the play-out (one class): its record read, the
+# hand-off written; it is played up to the hand-off only, some buffer's worth of tokens that no count of streams gives.
+PLAYOUT_BYTES = 16 + 8
+# Lane-instructions one token-step of the play-out needs where every token counts (no pacing, or generation slower than
+# consumption; both endpoints' streams share the hash draw): counter add 1, hash finaliser 8, two range maps
+# (multiply-high) 2, tail mask 1, two sums and two maxima 4, loop 1.
 PLAYOUT_INSTR_PER_TOKEN = 17
-PLAYOUT_INSTR_PER_TOKEN_LEAN = 13
-# Lane-instructions one (request, policy) pair needs in the reduction kernel, by the kind of policy.
-# Algorithm 3 (no waits; the race at w = 0 is staged once per request): request vector load 1, length
-# threshold 1, trigger compare and its conjunction 2, outcome index 2, TTFT select 1, row address 1, two row
-# loads 2, six 32-bit sums (tokens on device, two prefills, TBTs in tau's bin, delayed tokens, the four
-# byte-packed counts) and one 64-bit sum 8, staged histogram increment (address, atomic) 2, stall test shared
-# by four pairs 1.
-PAIR_INSTR_NOWAIT = 21
-# Algorithm 2 (waits): load 1, wait map 4, start compare 1, w + T_d 1, win compare 1, minimum 1, trigger 3,
-# outcome index 3, row address 1, two row loads 2, sums 8, histogram increment from the float bits (convert,
-# small-value test and branch, offset 2, increment 3, address, atomic) 10, stall test 1.
-PAIR_INSTR_WAIT = 37
-# Lane-instructions the zone-by-zone reduction needs per request and policy FAMILY (up to 128 policies along a
-# budget axis, whatever their number): request loads 6, device TTFT 1, projected saving 4, race at wait 0 (two
-# compares, select, minimum) 4, trigger against the family's range 3, outcome select 2, the common outcome's
-# addends 14, its ten sums 11, histogram bin and increment 6; the first run's outcome 8, its addends 14, ten
-# differences to the common outcome 20, histogram bin and increment 6; loop 1.  The extra sweeps over requests
-# whose prompt length is some policy's l* are not counted.
-ZONE_INSTR_PER_REQUEST_FAMILY = 100
+# Bytes a request needs of the reductions per slab of a grid of policies (at most 256 budgets by 8 overheads): its record
+# and its hand-off read.
+GRID_BYTES = 16 + 8
 SCHEDULERS, LANES = 4, 32    # warp schedulers per multiprocessor, lanes per warp
 MIN_WARMUP_SECONDS = 0.5     # untimed steps run until this much device time has passed (and at least --warmup)
 MAX_WARMUP_STEPS = 200
-# From the committed ncu captures (profiles/): DRAM bytes per launch of the bench's own launch shape, and the
-# lane-slots the hardware executed per unit of work beside the algorithmic counts above.  None: not captured
+# From the committed ncu captures (profiles/): DRAM bytes per launch of the bench's own launch shape.  None: not captured
 # for the current kernel.
-NCU_TRAFFIC_BYTES = {("k_pairs_rows", 1): 145709568, ("k_playout_fast", 1): 827904}
-# issued lane-slots per token-step (play-out; the workload-3 figure is of a 200,000-request capture of its shape, the
-# workload-4 figure of a 4,000,000-request one) and
-# per request and policy family (zone kernel, workload 2 at full size)
-NCU_EXECUTED_PER_UNIT = {("k_playout_fast", 1): 31.9, ("k_playout_fast", 3): 21.8, ("k_playout_fast", 4): 28.2,
-                         ("k_pairs_zones+k_pairs_acc", 2): 269.0}
+NCU_TRAFFIC_BYTES = {}
 HEADLINE_CONFIG = 4
 ALL_CONFIGS = (0, 1, 2, 3, 4, 5)
 
@@ -457,12 +436,12 @@ class Bench:
         # ---- rooflines of the timed kernels
         hbm_gbs, sm_max_mhz, src = self.peaks
         sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-        names = ["k_playout_fast", "k_playout", "k_pairs_acc", "k_pairs_rows"]
+        names = ["k_playout_short", "k_playout", "k_grid+k_spread+k_pairs_acc", "k_pairs_rows"]
         kms = {nm: statistics.mean(t[i] for t in ktimes) for i, nm in enumerate(names)}
         alu_peak = sms * SCHEDULERS * LANES * sm_max_mhz * 1e6 / 1e12         # T lane-instructions/s
         alu_src = "%d SMs x %d schedulers x %d lanes x %.0f MHz (issue slots)" % (sms, SCHEDULERS, LANES, sm_max_mhz)
         alu_meas = self.alu_measured / 1e12 if self.alu_measured else None
-        per_token = PLAYOUT_INSTR_PER_TOKEN_LEAN if never_clamps(w) else PLAYOUT_INSTR_PER_TOKEN
+        paced = never_clamps(w)
         full_size = not args.requests and not args.budgets
 
         def alu_roof(name, lane_instr, ms, **extra):
@@ -473,45 +452,35 @@ class Bench:
                  # what the GPU sustains on the token loop's own instruction mix with every SM full
                  # (disco_measure_alu_peak, measured in this run)
                  "peak_measured": alu_meas, "frac_of_measured": ach / alu_meas if alu_meas else None,
-                 "executed_lane_slots_per_unit": NCU_EXECUTED_PER_UNIT.get((name, cfg)),
                  "ms_per_launch": ms}
             r.update(extra)
             return r
+
+        def hbm_roof(name, bytes_alg, ms, **extra):
+            ach = bytes_alg / (ms * 1e-3) / 1e9
+            return {"kernel": name, "bound": "hbm", "achieved": ach, "peak": hbm_gbs, "unit": "GB/s",
+                    "frac": ach / hbm_gbs, "traffic": NCU_TRAFFIC_BYTES.get((name, cfg)) if full_size else None,
+                    "peak_source": src, "algorithmic_bytes": bytes_alg, "ms_per_launch": ms, **extra}
 
         def roof_of(name):
             ms = kms[name]
             if ms <= 0.0:
                 return None
             if name == "k_pairs_rows":
-                if not w.materialise:
-                    return None
-                bytes_alg = n * P * PAIR_OUT_BYTES + n * TRACE_BYTES
-                ach = bytes_alg / (ms * 1e-3) / 1e9
-                return {"kernel": name, "bound": "hbm", "achieved": ach, "peak": hbm_gbs, "unit": "GB/s",
-                        "frac": ach / hbm_gbs, "traffic": NCU_TRAFFIC_BYTES.get((name, cfg)) if full_size else None,
-                        "peak_source": src, "algorithmic_bytes": bytes_alg, "ms_per_launch": ms}
-            if name == "k_pairs_acc":
-                # the two reduction kernels together (their events bracket both): requests settled zone by zone per
-                # policy family, and the pairs left to the pair-by-pair kernel, by kind (a (group, policy) waits
-                # when Algorithm 1 made the group device-constrained)
-                zone_pairs, left_pairs, settled, sweeps = tr.work_counts()
-                wait_pairs = 0
-                for g in range(tr.n_groups):
-                    n_g = tr.group_size(g)
-                    wait_pairs += n_g * sum(1 for p in range(P) if tr.prep(g, p).device_constrained)
-                wait_share = wait_pairs / float(max(n * P, 1))
-                per_left_pair = wait_share * PAIR_INSTR_WAIT + (1.0 - wait_share) * PAIR_INSTR_NOWAIT
-                lane_instr = settled * ZONE_INSTR_PER_REQUEST_FAMILY + left_pairs * per_left_pair
-                return alu_roof("k_pairs_zones+k_pairs_acc", lane_instr, ms,
-                                work={"pairs_by_zones": zone_pairs, "pairs_one_by_one": left_pairs,
-                                      "requests_settled_per_family": settled, "segment_sweeps": sweeps},
-                                instr={"per_request_family": ZONE_INSTR_PER_REQUEST_FAMILY,
-                                       "per_pair_one_by_one": per_left_pair},
-                                instr_per_pair_mean=lane_instr / float(max(n * P, 1)))
-            if name == "k_playout_fast":
-                return alu_roof(name, token_steps * per_token * n_classes, ms, token_steps=token_steps * n_classes,
-                                instr_per_token_step=per_token)
-            return None                       # k_playout: only the requests the clamp-free kernel listed
+                return hbm_roof(name, n * P * PAIR_OUT_BYTES + n * TRACE_BYTES, ms) if w.materialise else None
+            if name == "k_grid+k_spread+k_pairs_acc":
+                # the reduction kernels together (their events bracket them): requests settled run by run per slab of
+                # policies, and the pairs left to the pair-by-pair kernel
+                grid_pairs, left_pairs, settled, sweeps = tr.work_counts()
+                return hbm_roof(name, settled * GRID_BYTES, ms, limited_by="issue slots (ncu)",
+                                work={"pairs_by_runs": grid_pairs, "pairs_one_by_one": left_pairs,
+                                      "requests_settled_per_slab": settled, "segment_sweeps": sweeps})
+            if name == "k_playout_short" and paced:
+                return hbm_roof(name, n * n_classes * PLAYOUT_BYTES, ms, limited_by="issue slots (ncu)")
+            if name == "k_playout" and not paced:
+                return alu_roof(name, token_steps * PLAYOUT_INSTR_PER_TOKEN * n_classes, ms,
+                                token_steps=token_steps * n_classes, instr_per_token_step=PLAYOUT_INSTR_PER_TOKEN)
+            return None
 
         roofs = [r for r in (roof_of(nm) for nm in names) if r is not None]
         roof = None
@@ -526,10 +495,11 @@ class Bench:
             cpu = cpu_baseline_of(w, oracle_seconds)
         tr.close()
         res = {"value": value, "ms_per_step": total_ms / steps, "steps": steps, "warmup": warm_dev,
-               # token-steps actually played per second: one play-out per request and timeline class (policies
-               # that share the consumption rate, buffer size and pacing share it), whatever the number of policies
+               # token-steps of the play-outs settled per second: one play-out per request and timeline class (policies
+               # that share the consumption rate, buffer size and pacing share it), whatever the number of policies;
+               # tokens after a hand-off that nothing depends on are settled without being drawn
                "sim_tokens_per_s": job_token_steps * steps / (total_ms * 1e-3),
-               # tokens of all (request, policy) pairs covered per second: each played token counted once for
+               # tokens of all (request, policy) pairs covered per second: each token counted once for
                # every policy that shares its play-out
                "pair_tokens_per_s": job_token_steps / n_classes * P * steps / (total_ms * 1e-3),
                "config": {"workload": w.name, "requests_per_gpu": n, "policies": P, "groups": G,
@@ -580,8 +550,7 @@ def run_ours(args):
             if cfg == args.config:
                 r = main
             else:
-                # enough steps for a stable mean, bounded in time (a workload-3 step takes about 3 ms, a
-                # workload-2 step under 2 ms, the others well under 1 ms)
+                # enough steps for a stable mean, bounded in time (a step of any of the others takes under 1 ms)
                 r = b.run(cfg, max(args.steps, 20), args.warmup, min(args.oracle_seconds, 3.0))
             keep = {k: r[k] for k in ("value", "ms_per_step", "steps", "warmup", "sim_tokens_per_s",
                                       "pair_tokens_per_s", "gpu_launches", "cpu_baseline")}

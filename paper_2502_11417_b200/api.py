@@ -489,13 +489,13 @@ class Trace:
 
     def timing(self):
         """Device milliseconds of the last reduced evaluation's kernels:
-        (clamp-free play-out, general play-out, pair reductions, per-pair rows)."""
+        (clamp-free play-out, other play-outs, reductions, per-pair rows)."""
         ms = (C.c_float * 4)()
         _check(lib().disco_get_timing(self._h, ms))
         return tuple(ms)
 
     def work_counts(self, stream=None):
-        """(pairs settled zone by zone, pairs evaluated one by one, requests settled per policy family, sweeps
+        """(pairs settled run by run, pairs evaluated one by one, requests settled per slab of policies, sweeps
         over chunk segments) of the last evaluation."""
         w = (C.c_uint64 * 4)()
         _check(lib().disco_get_work_counts(self._h, w, _stream_ptr(stream)))

@@ -194,7 +194,7 @@ int set_error(int code, const char* msg);
 // the context stays usable, and the next call that synchronises returns DISCO_ECUDA naming kernel and index.
 // In the ordinary build DBG_OK is the constant true and the checks vanish.
 enum DbgKernel { DBG_K_INGEST = 1, DBG_K_RADIX, DBG_K_GATHER, DBG_K_TABLES, DBG_K_PREP, DBG_K_PLAYOUT_FAST, DBG_K_PLAYOUT,
-                 DBG_K_PAIRS_ACC, DBG_K_PAIRS_ZONES, DBG_K_PAIRS_ROWS, DBG_K_FINALIZE, DBG_K_SELECT, DBG_K_SELFTEST,
+                 DBG_K_PAIRS_ACC, DBG_K_GRID, DBG_K_PAIRS_ROWS, DBG_K_FINALIZE, DBG_K_SELECT, DBG_K_SELFTEST,
                  DBG_K_COUNT };
 enum DbgWhat { DBG_REQUEST = 1, DBG_POLICY, DBG_GROUP, DBG_CHUNK, DBG_KNOT, DBG_BIN, DBG_WINDOW, DBG_SLOT, DBG_TABLE,
                DBG_COUNTER, DBG_ELEMENT, DBG_WHAT_COUNT };

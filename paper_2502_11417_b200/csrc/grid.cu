@@ -25,7 +25,8 @@
 //
 // Bound: integer issue.  Against one sweep per 128 policies of one overhead, with what differs between neighbouring
 // policies entered into their histograms one by one, a request is visited once per run instead of once per run and
-// overhead (figures at launch_grid).
+// overhead: 16 M requests in six groups under 128 budgets by 8 overheads took 2,300 us (and 450 more pair by pair), now
+// 436; a million in one group under 256 by 4 took 220 us, now 36.
 #include <algorithm>
 #include <cstddef>
 #include <type_traits>
@@ -110,7 +111,7 @@ struct Args {
 };
 
 __device__ __forceinline__ void hist_add(uint32_t* h, int bin) {
-    if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicAdd(&h[bin], 1u);
+    if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) atomicAdd(&h[bin], 1u);
 }
 
 // Adds (or, sub, takes) the rows of window counts of the lanes' requests that are in the mask: a lane sums up a bin over
@@ -122,7 +123,7 @@ __device__ __forceinline__ void add_rows(const uint16_t* __restrict__ win, int W
     if (W <= 16) {
         // short rows: several requests' at a time, which mostly lie side by side
         const int per = 32 / W, mine = lane / W, b = lane - mine * W;
-        const bool in = mine < per && DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN);
+        const bool in = mine < per && DBG_OK(lo + b, kNBins, DBG_K_GRID, DBG_BIN);
         uint32_t sum = 0;
 #pragma unroll 4
         for (int r0 = 0; r0 < 32; r0 += per) {
@@ -135,7 +136,7 @@ __device__ __forceinline__ void add_rows(const uint16_t* __restrict__ win, int W
     }
     for (int b0 = 0; b0 < W; b0 += 32) {
         const int b = b0 + lane;
-        const bool in = b < W && DBG_OK(lo + b, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN);
+        const bool in = b < W && DBG_OK(lo + b, kNBins, DBG_K_GRID, DBG_BIN);
         uint32_t sum = 0;
 #pragma unroll 1
         for (int r0 = 0; r0 < 32; r0 += 8) {
@@ -174,7 +175,7 @@ __device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_
         add_rows(a.rec.win[from], cc.W[from], cc.lo[c.g][from], __ballot_sync(FULL, valid && t == r), kk, false, tbt + (r - 1) * kNBins);
     if (c.x_from >= 0 && valid && t > 0) {
         const int bin = first_bin(a.gcs[c.g], c.x_from, a.k0, orig);
-        if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicSub(&tbt[(t - 1) * kNBins + bin], 1u);
+        if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) atomicSub(&tbt[(t - 1) * kNBins + bin], 1u);
     }
 }
 
@@ -190,7 +191,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
         const uint32_t i = min(i0 + lane, pb - 1);
         const uint32_t pos = list ? (uint32_t)sm.list[i] : i;
         const uint32_t kk = c.start + pos;
-        bool valid = i0 + lane < pb && DBG_OK(kk, a.tr.n, DBG_K_PAIRS_ZONES, DBG_REQUEST);
+        bool valid = i0 + lane < pb && DBG_OK(kk, a.tr.n, DBG_K_GRID, DBG_REQUEST);
         const uint4 q = a.tr.req[kk];
         const uint2 hand = c.may_migrate ? a.rec.hand[kk] : make_uint2(0u, 0u);
         const uint32_t S = q.x, l = q.y & 0xFFFFu, n = q.y >> 16, m = hand.x & 0xFFFFu, dly = hand.x >> 16;
@@ -205,7 +206,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                 const uint32_t live = __ballot_sync(FULL, valid);
                 // requests of one prompt length share the device's TTFT: mostly the whole warp counts in one bin
                 if (__shfl_sync(FULL, l, 0) == __shfl_sync(FULL, l, 31)) {
-                    if (lane == 0 && live && DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) atomicAdd(&sm.only_ttft[bin], (uint32_t)__popc(live));
+                    if (lane == 0 && live && DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) atomicAdd(&sm.only_ttft[bin], (uint32_t)__popc(live));
                 } else if (valid) hist_add(sm.only_ttft, bin);
                 if (valid) { o.cnt += 1u; o.n += n; o.l += l; o.tt += Td; o.tau += (!WIDE || (c.even & 2u)) ? n - 1u : 0u; }
                 if (WIDE && !(c.even & 2u)) add_rows(a.rec.win[1], a.cc->W[1], a.cc->lo[c.g][1], live, kk, false, tbt + NT * kNBins);
@@ -229,7 +230,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                 uint32_t at = 0;
                 if (lane == 0) at = atomicAdd(&sm.n_list, (uint32_t)__popc(all));
                 at = __shfl_sync(FULL, at, 0) + __popc(all & ((1u << lane) - 1u));
-                if (mine && DBG_OK(at, kListCap, DBG_K_PAIRS_ZONES, DBG_SLOT)) sm.list[at] = (uint16_t)pos;
+                if (mine && DBG_OK(at, kListCap, DBG_K_GRID, DBG_SLOT)) sm.list[at] = (uint16_t)pos;
             }
         }
         if (!(valid && started && (dev_wins ? 2 : 1) == c.cand)) saving = -1.0f;      // not won by the endpoint that may hand over
@@ -421,7 +422,7 @@ __device__ __noinline__ void enter_requests(const Args& a, const Ctx& c, const f
             const bool started = S > w, dev_wins = S > w + Td;
             const uint32_t tt = min(S, w + Td);
             const int bin = bin_of_ticks(tt);
-            if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) count(tb.ttft + bin, q0, q1);
+            if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) count(tb.ttft + bin, q0, q1);
             if (dev_wins) { add(B_TD, n, q0, q1); add(B_DW, 1ull, q0, q1); }
             add(B_PS, l, q0, q1);
             if (started) { add(B_PD, l, q0, q1); add(B_RACE, 1ull, q0, q1); }
@@ -434,7 +435,7 @@ __device__ __noinline__ void enter_requests(const Args& a, const Ctx& c, const f
                 const int f = kBase + r * kLev;
                 add(f + V_A, n - m, q0, q1); add(f + V_B, l + m, q0, q1); add(f + V_N, 1ull, q0, q1);
                 if (dly) add(f + V_C, dly, q0, q1);
-                if (DBG_OK(stall, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) count(tb.tbt + (size_t)r * K * kNBins + stall, q0, q1);
+                if (DBG_OK(stall, kNBins, DBG_K_GRID, DBG_BIN)) count(tb.tbt + (size_t)r * K * kNBins + stall, q0, q1);
             }
         };
         // the columns on either side of the request's length
@@ -448,7 +449,7 @@ __device__ __noinline__ void enter_requests(const Args& a, const Ctx& c, const f
             if (low < k1) enter_run(wt_min, low, k1);
         } else if (k1 > 0) {                                                           // the device alone
             const int bin = bin_of_ticks(Td);
-            if (DBG_OK(bin, kNBins, DBG_K_PAIRS_ZONES, DBG_BIN)) count(tb.ttft + bin, 0, k1);
+            if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) count(tb.ttft + bin, 0, k1);
             add(B_DO, 1ull, 0, k1); add(B_TD, n, 0, k1); add(B_PD, l, 0, k1); add(B_TAU, n - 1u, 0, k1); add(B_TT, Td, 0, k1);
         }
         if (k2 < K) enter_run(0u, k2, K);
@@ -477,8 +478,8 @@ k_grid(const __grid_constant__ Args a) {
         const Slab& sl = a.slabs[slab_id];
         const Chunk ch = a.chunks[item / a.n_slabs];
         const int g = ch.g;
-        if (!DBG_OK(g, a.tr.n_groups, DBG_K_PAIRS_ZONES, DBG_GROUP) ||
-            (ch.len && !DBG_OK((unsigned long long)ch.start + ch.len - 1, a.tr.n, DBG_K_PAIRS_ZONES, DBG_REQUEST)))
+        if (!DBG_OK(g, a.tr.n_groups, DBG_K_GRID, DBG_GROUP) ||
+            (ch.len && !DBG_OK((unsigned long long)ch.start + ch.len - 1, a.tr.n, DBG_K_GRID, DBG_REQUEST)))
             continue;
         const GroupConst& gc = a.gcs[g];
         const Tables<WIDE> tb(a.gt, sl, a.tr.n_groups);
@@ -499,7 +500,7 @@ k_grid(const __grid_constant__ Args a) {
             waits = pr.device_constrained != 0;
         }
         for (int p = threadIdx.x; p < c.K; p += kThreads) {
-            if (!DBG_OK(a.tab[sl.cols + p], a.P, DBG_K_PAIRS_ZONES, DBG_POLICY)) continue;
+            if (!DBG_OK(a.tab[sl.cols + p], a.P, DBG_K_GRID, DBG_POLICY)) continue;
             const Prep& pr = a.prep[(size_t)g * a.P + a.tab[sl.cols + p]];
             sm.key[p] = waits ? pr.l_star : pr.l_th;
             sm.w_star[p] = (uint32_t)pr.w_star; sm.w_tail[p] = (uint32_t)pr.w_tail;
@@ -519,7 +520,7 @@ k_grid(const __grid_constant__ Args a) {
                 uint32_t at = 0;
                 if ((threadIdx.x & 31) == 0) at = atomicAdd(&a.left.count[slab_id * a.tr.n_groups + g], (uint32_t)__popc(all));
                 at = first + __shfl_sync(FULL, at, 0) + __popc(all & ((1u << (threadIdx.x & 31)) - 1u));
-                if (out && DBG_OK(at, a.tr.n, DBG_K_PAIRS_ZONES, DBG_REQUEST)) a.left.list[(size_t)slab_id * a.tr.n + at] = kk;
+                if (out && DBG_OK(at, a.tr.n, DBG_K_GRID, DBG_REQUEST)) a.left.list[(size_t)slab_id * a.tr.n + at] = kk;
                 mine += (uint32_t)__popc(all);
             }
             if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&sm.flagged, mine);
@@ -556,7 +557,7 @@ k_grid(const __grid_constant__ Args a) {
                 if (pa < pb) {
                     const uint32_t at = atomicAdd(&sm.n_seg, 1u);
                     atomicAdd(&sm.n_runs, waits ? (uint32_t)(k2 - k1) + (k1 > 0) + (k2 < K) : 1u);
-                    if (DBG_OK(at, kMaxSeg, DBG_K_PAIRS_ZONES, DBG_SLOT))
+                    if (DBG_OK(at, kMaxSeg, DBG_K_GRID, DBG_SLOT))
                         sm.seg[at] = Seg{(uint16_t)pa, (uint16_t)pb, (uint16_t)k1, (uint16_t)k2};
                 }
             }

@@ -16,7 +16,8 @@
 //
 // Bound: latency at 10^5 requests (one launch instead of eighteen), memory at 10^7: the columns are read twice (once when
 // they are in host memory: then the first pass leaves a copy), 20 bytes a request are written to scattered places, the
-// ticks are read and written once more.
+// ticks are read and written once more.  16 M requests in six groups: 1,800 us by a chain of kernels, 886 now, over half
+// of it the scattered places (linear stores in their stead: 106 us for that pass instead of 470); a million: 69 us.
 #include "load.cuh"
 
 #include <algorithm>
