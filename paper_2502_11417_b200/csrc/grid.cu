@@ -43,6 +43,7 @@ constexpr int kListStep = 4096;          // ... and looks after the list's room 
 constexpr int kMaxSeg = 2 * kGridCols + 2;
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr uint32_t kNoPolicy = 0xFFFFFFFFu;
+static_assert(kNBins % 32 == 0 && kNBins / 32 < 32, "a bit for each group of bins");
 
 // Blocks to a multiprocessor by the rows a kernel is built for: what their registers allow without spilling.
 __host__ __device__ constexpr int blocks_for(int rows, bool wide) { return rows == 1 || (rows == 2 && !wide) ? 4 : rows <= 4 ? 3 : 2; }
@@ -62,6 +63,7 @@ struct Smem {                                          // fixed part; the TBT hi
     uint32_t only_sum[4];                              // ... of the device-only run: requests, tokens, prompt tokens, TBTs in tau's bin
     uint32_t tt[3], only_tt[3];                        // ... and the sums of TTFTs, in parts of 20 bits
     uint32_t ttft[kNBins], only_ttft[kNBins];
+    uint32_t used[2][3];                               // groups of bins with counts: TTFT, stall, device only; by turns
     uint32_t n_seg, n_runs, n_list, flagged, ticket;
     int32_t key[kGridCols];                            // the columns' length thresholds
     uint32_t w_star[kGridCols], w_tail[kGridCols];
@@ -73,10 +75,11 @@ template <int NT>
 struct Acc {                                           // a lane's share of a run
     uint32_t td, ps, pd, tau, race, dw;
     unsigned long long tt;
+    uint32_t bins, stalls;                             // groups of 32 bins with counts: of the TTFTs, of the hand-off stalls
     uint32_t a[NT], b[NT], cn[NT], tx[NT];             // cn: delayed tokens | requests << 22 (at most 255 requests a lane)
 };
 
-struct Only { uint32_t cnt, n, l, tau; unsigned long long tt; };   // ... of a device-only run
+struct Only { uint32_t cnt, n, l, tau, bins; unsigned long long tt; };   // ... of a device-only run
 
 struct Ctx {                                           // a (chunk, slab)
     uint32_t start, len;
@@ -187,13 +190,31 @@ template <int NT, bool WIDE, bool ONLY>
 __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (&th)[NT], Smem& sm, uint32_t* tbt, uint32_t pa,
                                       uint32_t pb, uint32_t w, bool list, bool push, bool race, bool only, Acc<NT>& s, Only& o) {
     const int lane = threadIdx.x & 31;
-    for (uint32_t i0 = pa + (threadIdx.x & ~31u); i0 < pb; i0 += kThreads) {          // a warp's lanes iterate together
+    // The kernel of eight rows has too few warps a multiprocessor to hide the loads' latency: there they run an iteration
+    // ahead (16 M requests under 128 budgets by 8 overheads 365 us instead of 435; the others have the warps, and no
+    // registers left: 3 % slower).
+    constexpr bool kAhead = NT == 8 && !WIDE;
+    uint32_t pos;
+    uint4 q, q_ahead;
+    uint2 hand, hand_ahead;
+    uint32_t ahead;
+    auto fetch = [&](uint32_t i0, uint32_t& at, uint4& to, uint2& to_hand) {
         const uint32_t i = min(i0 + lane, pb - 1);
-        const uint32_t pos = list ? (uint32_t)sm.list[i] : i;
+        at = list ? (uint32_t)sm.list[i] : i;
+        to = a.tr.req[c.start + at];
+        to_hand = c.may_migrate ? a.rec.hand[c.start + at] : make_uint2(0u, 0u);
+    };
+    const uint32_t first = pa + (threadIdx.x & ~31u);
+    if (kAhead && first < pb) fetch(first, ahead, q_ahead, hand_ahead);
+    for (uint32_t i0 = first; i0 < pb; i0 += kThreads) {              // a warp's lanes iterate together
+        if (kAhead) {
+            pos = ahead; q = q_ahead; hand = hand_ahead;
+            if (i0 + kThreads < pb) fetch(i0 + kThreads, ahead, q_ahead, hand_ahead);
+        } else {
+            fetch(i0, pos, q, hand);
+        }
         const uint32_t kk = c.start + pos;
         bool valid = i0 + lane < pb && DBG_OK(kk, a.tr.n, DBG_K_GRID, DBG_REQUEST);
-        const uint4 q = a.tr.req[kk];
-        const uint2 hand = c.may_migrate ? a.rec.hand[kk] : make_uint2(0u, 0u);
         const uint32_t S = q.x, l = q.y & 0xFFFFu, n = q.y >> 16, m = hand.x & 0xFFFFu, dly = hand.x >> 16;
         const uint32_t Td = c.kappa * l + c.c0;
         // Eq. 4's projected saving, on the true remainder or on what is left of the expected length; a request may only
@@ -208,6 +229,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                 if (__shfl_sync(FULL, l, 0) == __shfl_sync(FULL, l, 31)) {
                     if (lane == 0 && live && DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) atomicAdd(&sm.only_ttft[bin], (uint32_t)__popc(live));
                 } else if (valid) hist_add(sm.only_ttft, bin);
+                if (!WIDE && valid) o.bins |= 1u << (bin >> 5);
                 if (valid) { o.cnt += 1u; o.n += n; o.l += l; o.tt += Td; o.tau += (!WIDE || (c.even & 2u)) ? n - 1u : 0u; }
                 if (WIDE && !(c.even & 2u)) add_rows(a.rec.win[1], a.cc->W[1], a.cc->lo[c.g][1], live, kk, false, tbt + NT * kNBins);
             }
@@ -221,7 +243,9 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
             s.race += started ? 1u : 0u; s.dw += dev_wins ? 1u : 0u;
             s.tt += tt;
             s.tau += (!WIDE || pace) ? n - 1u : 0u;
-            hist_add(sm.ttft, bin_of_ticks(tt));
+            const int bin = bin_of_ticks(tt);
+            hist_add(sm.ttft, bin);
+            if (!WIDE) s.bins |= 1u << (bin >> 5);
         }
         if (!ONLY && push) {
             const bool mine = valid && S > w;
@@ -243,7 +267,11 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                 s.a[r] += handed; s.b[r] += refill; s.cn[r] += cn; ++t;
                 if (WIDE) s.tx[r] += tx;
             }
-        if (t > 0) hist_add(tbt + (t - 1) * kNBins, bin_of_ticks(hand.y));
+        if (t > 0) {
+            const int bin = bin_of_ticks(hand.y);
+            hist_add(tbt + (t - 1) * kNBins, bin);
+            if (!WIDE) s.stalls |= 1u << (bin >> 5);
+        }
         if (WIDE) add_windows(a, c, tbt, valid, kk, dev_wins, t, q.z);
     }
 }
@@ -268,8 +296,13 @@ __device__ __forceinline__ unsigned long long take_wide(uint32_t (&from)[3]) {
 // The lanes' shares of a run go to the block's totals (32-bit: at most 65,280 requests of at most 12,288 tokens).  Lane f
 // of a warp adds field f.
 template <int NT, bool WIDE>
-__device__ __forceinline__ void share_out(Smem& sm, const Acc<NT>& s, int T) {
+__device__ __forceinline__ void share_out(Smem& sm, const Acc<NT>& s, int turn) {
     const int lane = threadIdx.x & 31;
+    if (!WIDE) {
+        const uint32_t bins = __reduce_or_sync(FULL, s.bins), stalls = __reduce_or_sync(FULL, s.stalls);
+        if (lane == 0 && bins) atomicOr(&sm.used[turn][0], bins);
+        if (lane == 0 && stalls) atomicOr(&sm.used[turn][1], stalls);
+    }
     uint32_t lo = 0, hi = 0;
     auto put = [&](int f, uint32_t v) {
         v = __reduce_add_sync(FULL, v);
@@ -286,7 +319,9 @@ __device__ __forceinline__ void share_out(Smem& sm, const Acc<NT>& s, int T) {
     if (NT * kLev + kBase > 32 && hi) atomicAdd(&sm.sum[32 + lane], hi);
     add_wide(sm.tt, s.tt);
 }
-__device__ __forceinline__ void share_only(Smem& sm, const Only& o) {
+__device__ __forceinline__ void share_only(Smem& sm, const Only& o, int turn) {
+    const uint32_t bins = __reduce_or_sync(FULL, o.bins);
+    if ((threadIdx.x & 31) == 0 && bins) atomicOr(&sm.used[turn][2], bins);
     const uint32_t c = __reduce_add_sync(FULL, o.cnt), n = __reduce_add_sync(FULL, o.n), l = __reduce_add_sync(FULL, o.l),
                    tau = __reduce_add_sync(FULL, o.tau);
     add_wide(sm.only_tt, o.tt);
@@ -310,13 +345,26 @@ struct Tables {
     __device__ unsigned long long* sum_row(int g, int q) const { return sums + ((size_t)g * K + q) * sum_fields(T); }
 };
 
+// Calls f(bin) for every bin of the groups of 32 in the mask, a warp a group (ALL: for every bin; windows may lie anywhere).
+template <bool ALL, class F>
+__device__ __forceinline__ void each_bin(uint32_t groups, F f) {
+    if (ALL) {
+        for (int b = threadIdx.x; b < kNBins; b += kThreads) f(b);
+        return;
+    }
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int k = 0; groups; groups &= groups - 1u, ++k)
+        if (k % (kThreads / 32) == w) f((__ffs(groups) - 1) * 32 + lane);
+}
+
 // Enters what the block has totalled for a run of the columns [q0, q1), or takes it from them (neg), and clears it.  All
-// threads call; barriers before and after.
-template <bool WIDE>
-__device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE>& tb, int g, int q0, int q1, bool neg) {
+// threads call; barriers before and after.  Only groups of 32 bins that the run has counts in are looked at (a run over all
+// bins of nine histograms took longer than the sweep of a few hundred requests).
+template <int NT, bool WIDE>
+__device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE>& tb, int g, int q0, int q1, bool neg, int turn) {
     using word = typename Tables<WIDE>::word;
     const bool back = q1 < tb.K;
-    for (int b = threadIdx.x; b < kNBins; b += kThreads) {
+    each_bin<WIDE>(sm.used[turn][0], [&](int b) {
         const uint32_t x = sm.ttft[b];
         if (x) {
             sm.ttft[b] = 0;
@@ -324,17 +372,21 @@ __device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE
             atomicAdd(&tb.ttft_row(q0)[b], y);
             if (back) atomicAdd(&tb.ttft_row(q1)[b], 0u - y);
         }
-        int32_t level = 0;                                             // counts at a level go to every row below it
-        for (int r = tb.T - 1; r >= 0; --r) {
-            const int32_t y = (int32_t)tbt[r * kNBins + b];
-            if (y) { tbt[r * kNBins + b] = 0; level += y; }
+    });
+    each_bin<WIDE>(sm.used[turn][1], [&](int b) {
+        int32_t y[NT], level = 0;                                      // counts at a level go to every row below it
+#pragma unroll
+        for (int r = 0; r < NT; ++r) y[r] = (int32_t)tbt[r * kNBins + b];      // (rows beyond the slab's have none)
+#pragma unroll
+        for (int r = NT - 1; r >= 0; --r) {
+            if (y[r]) { tbt[r * kNBins + b] = 0; level += y[r]; }
             if (level) {
                 const word z = (word)(long long)(neg ? -level : level);
                 atomicAdd(&tb.tbt_row(q0, r)[b], z);
                 if (back) atomicAdd(&tb.tbt_row(q1, r)[b], (word)0 - z);
             }
         }
-    }
+    });
     const int F = sum_fields(tb.T);
     for (int f = threadIdx.x; f < F; f += kThreads) {
         unsigned long long x = (f >= kBase && (f - kBase) % kLev == V_TAU) ? (unsigned long long)(long long)(int32_t)sm.sum[f] : sm.sum[f];
@@ -345,14 +397,15 @@ __device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE
         atomicAdd(&tb.sum_row(g, q0)[f], x);
         if (back) atomicAdd(&tb.sum_row(g, q1)[f], 0ull - x);
     }
+    if (threadIdx.x < 3) sm.used[turn ^ 1][threadIdx.x] = 0;          // (of the run before; all have read them)
 }
 
 // The same for a device-only run of the columns below q1.
 template <bool WIDE>
-__device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const Tables<WIDE>& tb, int g, int q1) {
+__device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const Tables<WIDE>& tb, int g, int q1, int turn) {
     using word = typename Tables<WIDE>::word;
     const bool back = q1 < tb.K;
-    for (int b = threadIdx.x; b < kNBins; b += kThreads) {
+    each_bin<WIDE>(sm.used[turn][2], [&](int b) {
         const uint32_t x = sm.only_ttft[b];
         if (x) {
             sm.only_ttft[b] = 0;
@@ -369,7 +422,8 @@ __device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const T
                 }
             }
         }
-    }
+    });
+    if (threadIdx.x < 3) sm.used[turn ^ 1][threadIdx.x] = 0;
     if (threadIdx.x < 5) {
         const int k = threadIdx.x;
         const unsigned long long x = k < 4 ? (unsigned long long)sm.only_sum[k] : take_wide(sm.only_tt);
@@ -466,6 +520,7 @@ k_grid(const __grid_constant__ Args a) {
     for (int i = threadIdx.x; i < (int)(offsetof(Smem, key) / 4); i += kThreads) ((uint32_t*)&sm)[i] = 0;
     for (int i = threadIdx.x; i < (NT + (WIDE ? 1 : 0)) * kNBins; i += kThreads) tbt[i] = 0;
 
+    int turn = 0;                                                     // which of the two sets of used bins is in use
     const uint32_t direct = a.n_chunks * a.n_slabs <= gridDim.x ? kDirectAlone : kDirectMany;
     // the blocks draw (chunk, slab) items from a counter (zero at launch): items differ in cost
     for (;;) {
@@ -577,11 +632,11 @@ k_grid(const __grid_constant__ Args a) {
             Acc<NT> s = {};
             Only none = {};
             sweep<NT, WIDE, false>(a, c, th, sm, tbt, pa, pb, w, list, push, true, false, s, none);
-            share_out<NT, WIDE>(sm, s, c.T);
+            share_out<NT, WIDE>(sm, s, turn);
             __syncthreads();
-            enter<WIDE>(sm, tbt, tb, g, q0, q1, neg);
+            enter<NT, WIDE>(sm, tbt, tb, g, q0, q1, neg, turn);
             __syncthreads();
-            ++passes;
+            ++passes; turn ^= 1;
         };
         bool by_request = false;
         if constexpr (!WIDE) {
@@ -604,13 +659,13 @@ k_grid(const __grid_constant__ Args a) {
                 Acc<NT> s = {};
                 Only o = {};
                 sweep<NT, WIDE, true>(a, c, th, sm, tbt, sg.pa, sg.pb, 0u, false, false, race, only, s, o);
-                if (race) share_out<NT, WIDE>(sm, s, c.T);
-                if (only) share_only(sm, o);
+                if (race) share_out<NT, WIDE>(sm, s, turn);
+                if (only) share_only(sm, o, turn);
                 __syncthreads();
-                if (race) enter<WIDE>(sm, tbt, tb, g, sg.k2, K, false);
-                if (only) enter_only<WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1);
+                if (race) enter<NT, WIDE>(sm, tbt, tb, g, sg.k2, K, false, turn);
+                if (only) enter_only<WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1, turn);
                 __syncthreads();
-                ++passes;
+                ++passes; turn ^= 1;
             }
         } else {
             // segment by segment, run by run: [k2, K) waits 0, each column of [k1, k2) its own w*, [0, k1) w_tail -- and,

@@ -140,3 +140,13 @@ def test_few_requests_to_a_run(n, budgets, dearer):
     full_parity(w, [synth.policy(b) for b in grid], select=False, tag=f"{n} {budgets}")
     full_parity(w, [synth.policy(b, mig_threshold=t) for b in grid[::3] for t in (0.0, 1e-6, 3e-5)], select=False,
                 tag=f"{n} {budgets} x 3")
+
+
+@pytest.mark.parametrize("dearer", [False, True])
+@pytest.mark.parametrize("n", [257, 9000, 20011])
+def test_eight_overheads(n, dearer):
+    # the kernel of eight rows loads an iteration ahead, and runs are entered by the groups of bins they have counts in:
+    # sweeps of a part of a block, of a whole one and of several, with budgets below the tail ratio (lists) under Algorithm 2
+    w = synth.tiny_workload(101, n, max_prompt=64, max_out=60, device_dearer=dearer)
+    thetas = (0.0, 1e-7, 1e-6, 4e-6, 1e-5, 3e-5, 1e-4, 1.0)
+    full_parity(w, [synth.policy(b, mig_threshold=t) for b in (0.0, 0.01, 0.03, 0.4, 0.8) for t in thetas], select=False, tag=f"{n}")
