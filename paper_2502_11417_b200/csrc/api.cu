@@ -885,7 +885,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 left.list = c->d_left.as<uint32_t>(); left.count = left.list + N1;
                 CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
             }
-            CU(launch_grid(tr, gc, dcc, prep, P, dsl, (uint32_t)b.count, b.T, wide, classes[k].pacing != 0, d_tab,
+            CU(launch_grid(tr, gc, dcc, prep, P, dsl, (uint32_t)b.count, b.T, wide, d_tab,
                            d_chunks, (uint32_t)chunks.size(), rec, gt, left, k0, tickets + ticket++, work, c->sms, st));
             CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, wide, host_bin_of_ticks(classes[k].tau), d_tab, gt, acc,
                              h_ttft, h_tbt, st));

@@ -269,7 +269,7 @@ uint64_t grid_ttft_words(int K), grid_tbt_words(int K, int T), grid_sum_words(in
 uint32_t grid_blocks_per_sm(int T);
 int grid_rows(int T);            // rows the kernel that takes such a slab is built for
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
-                        const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide, bool count_pairs,
+                        const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide,
                         const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt,
                         LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t k0, uint32_t* ticket /* zero */,
                         uint64_t* work /* [4], added to */, int sms, cudaStream_t st);

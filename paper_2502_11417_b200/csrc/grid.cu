@@ -110,7 +110,6 @@ struct Args {
     uint32_t k0;
     uint32_t* ticket;
     unsigned long long* work;
-    int count_pairs;
 };
 
 __device__ __forceinline__ void hist_add(uint32_t* h, int bin) {
@@ -704,7 +703,7 @@ k_grid(const __grid_constant__ Args a) {
         }
         if (threadIdx.x == 0 && a.work) {
             const unsigned long long settled = ch.len - sm.flagged;
-            atomicAdd(&a.work[a.count_pairs ? 0 : 1], settled * (unsigned long long)sl.policies);
+            atomicAdd(&a.work[0], settled * (unsigned long long)sl.policies);      // pairs settled run by run
             atomicAdd(&a.work[2], settled);                            // requests settled, per slab
             atomicAdd(&a.work[3], (unsigned long long)passes);         // sweeps over segments
         }
@@ -841,13 +840,13 @@ uint32_t grid_blocks_per_sm(int T) { return (uint32_t)blocks_for(rows_for(T), fa
 int grid_rows(int T) { return rows_for(T); }
 
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
-                        const Slab* slabs, uint32_t n_slabs, int T, bool wide, bool count_pairs, const uint32_t* tab,
+                        const Slab* slabs, uint32_t n_slabs, int T, bool wide, const uint32_t* tab,
                         const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt, LeftLists left,
                         uint32_t k0, uint32_t* ticket, uint64_t* work, int sms, cudaStream_t st) {
     if (n_chunks == 0 || n_slabs == 0) return cudaSuccess;
     if ((uint64_t)n_chunks * n_slabs > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
     const Args a = {tr, rec, gc, cc, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, k0, ticket,
-                    (unsigned long long*)work, count_pairs ? 1 : 0};
+                    (unsigned long long*)work};
     switch (rows_for(T)) {
         case 1: return wide ? launch_one<1, true>(a, sms, st) : launch_one<1, false>(a, sms, st);
         case 2: return wide ? launch_one<2, true>(a, sms, st) : launch_one<2, false>(a, sms, st);

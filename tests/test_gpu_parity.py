@@ -463,10 +463,11 @@ def test_zone_by_zone_reduction_and_what_it_leaves_to_the_pair_kernel():
         stoch = [synth.policy(b, flags=synth.FLAG_STOCHASTIC | PACE) for b in grid]
         full_parity(w, stoch, tag=f"zones none dear={dear}")
         assert _work(w, stoch)[0] == 0
-        # pacing off: no zone kernel at all
+        # pacing off: settled run by run like the others, and counted so
         nopace = [synth.policy(b, flags=MIG) for b in grid]
         full_parity(w, nopace, tag=f"zones pacing off dear={dear}")
-        assert _work(w, nopace)[0] == 0
+        zone, left, settled, _ = _work(w, nopace)
+        assert (zone, left, settled) == (w.n * len(nopace), 0, w.n)
 
 
 def test_more_than_32_policy_tiles_use_several_flag_words():
