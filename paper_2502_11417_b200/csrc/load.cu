@@ -21,6 +21,7 @@
 #include "load.cuh"
 
 #include <algorithm>
+#include <cstdlib>
 #include <mutex>
 
 #include "pack.cuh"
@@ -58,23 +59,35 @@ struct SortSmem {
 };
 static_assert(kCounters == 2 * kSortCap, "the counters lie over the two key arrays");
 
-// Waits until every block of the grid has come here `times` times.  The wait is bounded: a block that gives up sets the
-// flag and goes on (the host refuses the results).
-__device__ __forceinline__ void grid_barrier(LoadZero* z, uint32_t times) {
+// The waits between blocks are bounded.  Behind one that ran out, tables may hold what an earlier call left in them, and
+// places taken from those could lie anywhere: a block that gives up sets the flag that makes the host refuse the results
+// and kLost in the barriers' word, and leaves the kernel; so does every block that finds kLost where it waits.  A block
+// that passes a barrier has seen every block arrive there, with its part of the work in front of it done.
+constexpr uint32_t kWaitTries = 1u << 22;
+constexpr uint32_t kLost = 1u << 31;              // (the word counts at most 256 blocks three times)
+__device__ __forceinline__ void give_up(LoadZero* z) {
+    atomicMax(&z->err[3], 2);
+    atomicOr(&z->barrier, kLost);
+}
+
+// Waits until every block of the grid has come here `times` times.  False, to all threads: the block has to leave.
+__device__ __forceinline__ bool grid_barrier(LoadZero* z, uint32_t times, uint32_t absent) {
     __syncthreads();
-    if (gridDim.x == 1) return;
+    if (gridDim.x == 1) return true;
+    bool lost = false;
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(&z->barrier, 1u);
-        const uint32_t want = times * gridDim.x;
+        const uint32_t want = times * gridDim.x + absent;
         uint32_t seen, tries = 0;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&z->barrier) : "memory");
-        } while (seen < want && ++tries < (1u << 22));
-        if (seen < want) atomicExch(&z->err[3], 2);
+        } while (seen < want && ++tries < kWaitTries);                 // (with kLost it is above any count)
+        if (seen < want) give_up(z);
+        lost = seen < want || (seen & kLost);
         __threadfence();
     }
-    __syncthreads();
+    return !__syncthreads_or(lost);
 }
 
 // Four neighbouring requests of the trace (or ticks of a sample) as the two passes see them.
@@ -167,16 +180,23 @@ __device__ __forceinline__ void read_items(const LoadArgs& a, uint32_t i0, bool 
     }
 }
 
-// Waits (boundedly, as above) for a word that another block writes once.
+// Waits (boundedly, as above) for a word that another block writes once; 0 if it does not come.
 __device__ __forceinline__ unsigned long long await_word(LoadZero* z, const unsigned long long* at) {
     unsigned long long v;
     uint32_t tries = 0;
     do {
         asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(at) : "memory");
-    } while (v == 0ull && ++tries < (1u << 22));
-    if (v == 0ull) atomicExch(&z->err[3], 2);
+    } while (v == 0ull && ++tries < kWaitTries);
+    if (v == 0ull) give_up(z);
     return v;
 }
+
+// Checked build: a wait for one arrival that nobody makes (LoadArgs::absent).
+#ifdef DISCO_DEBUG
+#define ABSENT(a, wait) ((a).absent == (wait) ? 1u : 0u)
+#else
+#define ABSENT(a, wait) 0u
+#endif
 
 // Four counters from k on (16-byte aligned), those from k1 on empty.
 __device__ __forceinline__ uint4 four_counters(const uint32_t* cnt, int k, int k1) {
@@ -542,7 +562,8 @@ k_load(const __grid_constant__ LoadArgs a) {
         if (kTrace) join(s_len, a.cnt, G * kLens, alone);
         join(s_tick, a.tick_cnt, G * kTickBins, alone);
     }
-    grid_barrier(z, ++waits);
+    ++waits;
+    if (!grid_barrier(z, waits, ABSENT(a, waits))) return;
 
     // ---- 2. place
     if (__ldcg(&z->err[0])) {                          // a rejected trace: nothing is placed
@@ -552,6 +573,7 @@ k_load(const __grid_constant__ LoadArgs a) {
     // where every bucket starts: the groups one after another, so one running sum over all groups' counters each
     const bool cursors = !PRIV || a.rounds > 1;                        // places are handed out by global cursors
     {
+        bool lost = false;
         const Share st = share_of(G * kTickBins), sl = share_of(kTrace ? G * kLens : 0);
         const uint4 ft = four_counters(a.tick_cnt, st.k0 + tid * 4, st.k1);
         const uint4 fl = kTrace ? four_counters(a.cnt, sl.k0 + tid * 4, sl.k1) : make_uint4(0u, 0u, 0u, 0u);
@@ -573,12 +595,17 @@ k_load(const __grid_constant__ LoadArgs a) {
                 if (lane == 0)
                     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&z->part[j][blockIdx.x]), "l"(((unsigned long long)s_carry[j] << 1) | 1ull) : "memory");
                 uint32_t before = 0;
-                for (uint32_t b = lane; b < blockIdx.x; b += 32) before += (uint32_t)(await_word(z, &z->part[j][b]) >> 1);
+                for (uint32_t b = lane; b < blockIdx.x && !lost; b += 32) {
+                    const unsigned long long word = await_word(z, &z->part[j][b]);
+                    lost = word == 0ull;
+                    before += (uint32_t)(word >> 1);
+                }
+                if (ABSENT(a, 4u) && lane == 0) lost = await_word(z, &z->part[j][kLoadBlocks - 1]) == 0ull;
                 before = __reduce_add_sync(FULL, before);
                 if (lane == 0) s_carry[j] = before;
             }
         } else if (tid < 2) s_carry[tid] = 0;
-        __syncthreads();
+        if (__syncthreads_or(lost)) return;                            // (some block's sum did not come)
         scan_share(a.tick_cnt, st, ft, s_carry[0], s_wtot, [&](int k, const uint4&, const uint4& start) {
             *reinterpret_cast<uint4*>(a.tick_start + k) = start;
             if (cursors) *reinterpret_cast<uint4*>(a.tick_at + k) = start;
@@ -591,7 +618,8 @@ k_load(const __grid_constant__ LoadArgs a) {
                     if (k + u < sl.k1) a.len_end[k + u] = cursors ? at[u] : at[u] + cs[u];    // (a cursor ends up where its bucket does)
             });
     }
-    grid_barrier(z, ++waits);
+    ++waits;
+    if (!grid_barrier(z, waits, ABSENT(a, waits))) return;
     if (SRC != S_TICKS) for (int g = tid; g <= G; g += kThreads) s_off[g] = g < G ? __ldcg(&a.tick_start[(size_t)g * kTickBins]) : a.n;
     __syncthreads();
     if (!cursors) {
@@ -693,7 +721,8 @@ k_load(const __grid_constant__ LoadArgs a) {
     } else {
         place(a.n);
     }
-    grid_barrier(z, ++waits);
+    ++waits;
+    if (!grid_barrier(z, waits, ABSENT(a, waits))) return;
 
     // ---- 3. sort
     SortSmem& sm = *reinterpret_cast<SortSmem*>(smem_raw);
@@ -735,7 +764,7 @@ k_load(const __grid_constant__ LoadArgs a) {
         }
         if (large) {
             __syncthreads();
-            if (!sort_dense(sm, a.binned + k2, k1 - k2, a.sorted + k2) && tid == 0) atomicExch(&z->err[3], 1);
+            if (!sort_dense(sm, a.binned + k2, k1 - k2, a.sorted + k2) && tid == 0) atomicMax(&z->err[3], 1);
         }
         __syncthreads();
         if (kTrace) {
@@ -754,7 +783,7 @@ k_load(const __grid_constant__ LoadArgs a) {
         for (int g = 0; g < G; ++g)                                    // (the last blocks have the fewest windows)
             if ((uint32_t)(G - 1 - g) % gridDim.x == gridDim.x - 1 - blockIdx.x)
                 group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
-        // the last block to come here reports the flags
+        // the last block to come here reports the flags (where a block has left, none does: what the host put there stands)
         if (tid == 0) { __threadfence(); s_item = atomicAdd(&z->done, 1u); }
         __syncthreads();
         if (s_item == gridDim.x - 1 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
@@ -788,7 +817,13 @@ cudaError_t launch_load(const LoadArgs& a, int sms, cudaStream_t st) {
         attr[0].val.cooperative = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
     }
+#ifdef DISCO_DEBUG
+    LoadArgs b = a;
+    if (const char* wait = std::getenv("DISCO_DEBUG_ABSENT")) b.absent = (uint32_t)std::atoi(wait);
+    return cudaLaunchKernelEx(&cfg, kernel, b);
+#else
     return cudaLaunchKernelEx(&cfg, kernel, a);
+#endif
 }
 
 // The same tables from a length histogram and a sorted sample given by the caller (a whole trace's, of which

@@ -72,7 +72,10 @@ struct LoadArgs {
     uint32_t* grp_off;                    // [G + 1]
     int32_t* knots;                       // [G][257]
     uint64_t* fin_totals;                 // [2G]: output tokens per group, then requests per group
-    LoadReadback* readback;
+    LoadReadback* readback;               // its err holds 0, 0, 0, 2 (no report) before the launch
+#ifdef DISCO_DEBUG
+    uint32_t absent;                      // the wait that expects one arrival more than comes (from 1; 4: of the other blocks' sums)
+#endif
 };
 
 cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st);          // one kernel, after a memset

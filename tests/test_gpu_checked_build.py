@@ -18,8 +18,8 @@ CASES = ("test_config0_full or test_config1_shape or test_config3_shape or test_
          "or test_one_prompt_length or test_more_groups_than_fit or test_family_whose_first_tile")
 
 
-def _run(args):
-    env = dict(os.environ, DISCO_CHECKED_BUILD="1")
+def _run(args, **more):
+    env = dict(os.environ, DISCO_CHECKED_BUILD="1", **more)
     return subprocess.run([sys.executable] + args, cwd=ROOT, env=env, capture_output=True, text=True, timeout=1500)
 
 
@@ -46,6 +46,60 @@ def test_the_checks_are_live():
         "print('live')\n")
     r = _run(["-c", code])
     assert r.returncode == 0 and "live" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
+
+
+WAITS = """
+import os, sys
+sys.path[:0] = [os.getcwd(), os.path.join(os.getcwd(), "tests")]
+import numpy as np, torch
+from paper_2502_11417_b200 import DiscoError, Trace, synth
+from paper_2502_11417_b200.api import sort_ttft_ticks_noalloc
+from parity import check_tables
+from oracle import Oracle
+
+def lost(call):
+    try:
+        call()
+    except DiscoError as e:
+        assert e.code == -3 and "lost each other" in str(e), str(e)
+        return
+    raise AssertionError("a wait ran out and nobody was told")
+
+def load(t, w):
+    return t.load_trace(w.prompt_len, w.output_len, w.server_ttft_s, w.server_profile, w.device_profile, w.servers, w.devices)
+
+waits = os.environ["WAITS"].split()
+large, small = synth.make_workload(4, n=40000, n_budgets=2), synth.make_workload(4, n=9000, n_budgets=2)
+x = torch.from_numpy(large.server_ttft_s).cuda()
+out = torch.full((large.n,), -7, dtype=torch.int32, device="cuda")
+t, u = load(Trace(), large), load(Trace(), small)
+cnt = np.stack([u.group_tables(g)[0] for g in range(u.n_groups)])
+ticks = torch.cat([u.sorted_ticks_device(g) for g in range(u.n_groups)])
+for wait in waits:
+    os.environ["DISCO_DEBUG_ABSENT"] = wait
+    lost(lambda: load(t, small))
+    lost(lambda: sort_ttft_ticks_noalloc(x, out))
+    assert bool((out == -7).all())
+    lost(lambda: u.set_group_tables(cnt, ticks, cnt.sum(axis=1).astype(np.uint64)))
+    del os.environ["DISCO_DEBUG_ABSENT"]
+    for c in (t, u):
+        try:
+            c.eval_policies(small.policies, 1)
+            raise AssertionError("evaluated a trace that was not loaded")
+        except DiscoError as e:
+            assert e.code == -1
+        load(c, small)
+        check_tables(c, Oracle.from_workload(small), "after wait " + wait)
+assert (sort_ttft_ticks_noalloc(x, out).cpu().numpy() == np.sort(np.rint(large.server_ttft_s.astype(np.float64) * 1e6))).all()
+print("waited")
+"""
+
+
+def test_blocks_leave_when_a_wait_runs_out():
+    # each of the ingestion kernel's waits in turn (three barriers, the blocks' sums) expects an arrival that nobody makes:
+    # the call fails, nothing has been placed or sorted, and the context takes the next load
+    r = _run(["-c", WAITS], WAITS="1 2 3 4")
+    assert r.returncode == 0 and "waited" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
 
 
 def test_the_ordinary_build_has_no_selftest():
