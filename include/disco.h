@@ -213,8 +213,8 @@ int64_t disco_get_group_tables(disco_ctx_t* ctx, uint32_t g, int64_t* cnt, int32
 
 /* Replaces the tables Algorithms 1-3 read by the caller's: cnt[G][DISCO_MAX_PROMPT+1] requests per prompt
  * length (host memory) and, group after group, the server-TTFT ticks behind F: n_ticks[g] (host) of them for
- * group g, in any order within the group, `ticks` in host or device memory (for instance the shards' sorted
- * ticks one after the other).  The library sorts them per group and rebuilds the cumulative token mass
+ * group g, in any order within the group, `ticks` in host or device memory, any device's (for instance the shards'
+ * sorted ticks one after the other).  The library sorts them per group and rebuilds the cumulative token mass
  * (Eq. 3) and the 257 knots of F.  The context keeps its own requests.  DISCO_EINVAL if a group's length
  * counts do not add up to n_ticks[g] or a tick is negative (the context must then be reloaded).  Lasts until
  * the next disco_load_trace.  Synchronises `stream`. */

@@ -1,0 +1,90 @@
+// A CUDA runtime that runs nothing, for tests of the library's host side on a machine without a GPU (preloaded in front of
+// the real one).  Device and page-locked memory is ordinary memory, kernels are not run; the ingestion kernel's launch
+// leaves a report of an accepted trace and is remembered.  A test says what memory a range of addresses is to be taken for.
+#include <cuda_runtime_api.h>
+
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <string>
+#include <vector>
+
+#include "load.cuh"
+
+namespace {
+struct Range { const char* at; size_t bytes; cudaMemoryType type; int device; };
+std::vector<Range> ranges;
+std::map<const void*, std::string> kernels;
+uint64_t copied = 0, loads = 0;                 // bytes copied out of the ranges; ingestion kernels launched
+const void* last_ticks = nullptr;               // what the last of them was given
+
+const Range* range_of(const void* p) {
+    for (const Range& r : ranges) if ((const char*)p >= r.at && (const char*)p < r.at + r.bytes) return &r;
+    return nullptr;
+}
+cudaError_t launch(const void* f, void** args) {
+    if (kernels[f].find("k_load") == std::string::npos) return cudaSuccess;
+    const disco::LoadArgs& a = *(const disco::LoadArgs*)args[0];
+    ++loads;
+    last_ticks = a.ticks;
+    if (a.readback) {
+        std::memset(a.readback, 0, sizeof *a.readback);
+        a.readback->ng[0] = a.readback->grp_off[1] = a.n;
+        a.readback->max_n = 1;
+    }
+    return cudaSuccess;
+}
+}  // namespace
+
+extern "C" {
+// ---- the test's side
+void fake_memory(const void* at, size_t bytes, int type, int device) { ranges.push_back({(const char*)at, bytes, (cudaMemoryType)type, device}); }
+uint64_t fake_copied(void) { return copied; }
+uint64_t fake_loads(void) { return loads; }
+const void* fake_last_ticks(void) { return last_ticks; }
+
+// ---- what the library calls
+void** __cudaRegisterFatBinary(void*) { static void* handle; return &handle; }
+void __cudaRegisterFatBinaryEnd(void**) {}
+void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterFunction(void**, const char* f, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) { kernels[f] = name; }
+void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
+unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, struct CUstream_st*) { return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3*, dim3*, size_t* smem, void* stream) { *smem = 0; *(void**)stream = nullptr; return cudaSuccess; }
+cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t, cudaStream_t) { return launch(f, args); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* f, void** args) { return launch(f, args); }
+cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 1; return cudaSuccess; }
+cudaError_t cudaMalloc(void** p, size_t n) { *p = std::calloc(n, 1); return *p ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaMallocHost(void** p, size_t n) { return cudaMalloc(p, n); }
+cudaError_t cudaFree(void* p) { std::free(p); return cudaSuccess; }
+cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void* to, const void* from, size_t n, cudaMemcpyKind, cudaStream_t) {
+    if (range_of(from)) copied += n;              // (may not be readable here)
+    else std::memcpy(to, from, n);
+    return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) { std::memset(p, v, n); return cudaSuccess; }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
+    std::memset(a, 0, sizeof *a);
+    const Range* r = range_of(p);
+    a->type = r ? r->type : cudaMemoryTypeUnregistered;
+    a->device = r ? r->device : -2;
+    a->devicePointer = r ? (void*)p : nullptr;
+    a->hostPointer = r && r->type != cudaMemoryTypeDevice ? (void*)p : nullptr;
+    return cudaSuccess;
+}
+cudaError_t cudaGetSymbolAddress(void**, const void*) { return cudaErrorInvalidValue; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)&ranges; return cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0.0f; return cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaGetLastError(void) { return cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "an error of the fake runtime"; }
+}

@@ -1,0 +1,81 @@
+"""Which memory the library's host side reads where, against a CUDA runtime that runs nothing (no GPU needed).  Each case
+is a process of its own, with tests/fake_cudart.cpp in front of the real runtime."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+HERE = os.path.join(ROOT, "tests")
+CUDA_INCLUDE = "/usr/local/cuda/include"
+
+PRELUDE = """
+import ctypes as C, mmap, os, sys
+sys.path.insert(0, os.getcwd())
+import numpy as np
+from paper_2502_11417_b200 import api, synth
+L, fake = api.lib(), C.CDLL(os.environ["LD_PRELOAD"])
+fake.fake_memory.argtypes = [C.c_void_p, C.c_size_t, C.c_int, C.c_int]
+fake.fake_copied.restype = fake.fake_loads.restype = C.c_uint64
+fake.fake_last_ticks.restype = C.c_void_p
+HOST, DEVICE, MANAGED = 1, 2, 3                       # cudaMemoryType
+
+libc = C.CDLL(None)
+libc.mmap.restype = C.c_void_p
+libc.mmap.argtypes = [C.c_void_p, C.c_size_t, C.c_int, C.c_int, C.c_int, C.c_long]
+
+def unreadable(count, kind, device=0):
+    # addresses the host cannot read, taken for memory of that kind
+    p = libc.mmap(None, 4 * count, 0, mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS, -1, 0)
+    fake.fake_memory(p, 4 * count, kind, device)
+    return p
+
+def load(ctx, n, columns, arrays_on_device=0):
+    sv, dv = api.server_array([synth.server()]), api.device_array([synth.device(500.0, 20.0)])
+    desc = api.TraceDesc(n, *columns, C.addressof(sv), 1, C.addressof(dv), 1, arrays_on_device, 0)
+    return L.disco_load_trace(C.byref(ctx), C.byref(desc), None)
+
+def host_columns(n):
+    cols = [np.full(n, 7, np.int32), np.full(n, 5, np.int32), np.full(n, 0.5, np.float32), np.zeros(n, np.uint8), np.zeros(n, np.uint8)]
+    return cols, [c.ctypes.data for c in cols]
+
+def set_tables(ctx, n, ticks):
+    cnt = np.zeros((1, 4097), np.int64)
+    cnt[0, 7] = n
+    sizes = np.array([n], np.uint64)
+    return L.disco_set_group_tables(ctx, cnt.ctypes.data, ticks, sizes.ctypes.data, None)
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    if not os.path.exists(os.path.join(CUDA_INCLUDE, "cuda_runtime_api.h")):
+        pytest.skip("no CUDA headers")
+    lib = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I", CUDA_INCLUDE, "-I", os.path.join(ROOT, "include"),
+                           "-I", os.path.join(ROOT, "paper_2502_11417_b200", "csrc"), "-o", lib, os.path.join(HERE, "fake_cudart.cpp")])
+    return lib
+
+
+def _run(fake, code):
+    env = {k: v for k, v in os.environ.items() if k != "DISCO_CHECKED_BUILD"}
+    r = subprocess.run([sys.executable, "-c", PRELUDE + code + "\nprint('as it should')\n"], cwd=ROOT, env=dict(env, LD_PRELOAD=fake),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "as it should" in r.stdout, (r.returncode, r.stdout[-1000:], r.stderr[-2000:])
+
+
+@pytest.mark.parametrize("kind,device,in_place", [("DEVICE", 0, True), ("DEVICE", 1, False), ("MANAGED", 0, True), ("MANAGED", 1, False)])
+def test_ticks_of_another_gpu_are_copied(fake, kind, device, in_place):
+    # a kernel may read this GPU's memory where it is; memory of another one may not be mapped here
+    _run(fake, f"""
+ctx = C.c_void_p(None)
+keep, cols = host_columns(5000)
+assert load(ctx, 5000, cols) == 0, L.disco_last_error()
+ticks = unreadable(9000, {kind}, {device})
+loads = fake.fake_loads()
+assert set_tables(ctx, 9000, ticks) == 0, L.disco_last_error()
+assert fake.fake_loads() == loads + 1
+assert (fake.fake_last_ticks() == ticks) == {in_place}
+assert fake.fake_copied() == {0 if in_place else 4 * 9000}
+""")
