@@ -93,7 +93,8 @@ typedef struct {
     uint32_t n_devices;
     uint32_t arrays_on_device;        /* 0: the five [n] arrays are host memory; 1: device memory.  Host arrays that
                                          are all page-locked (cudaHostAlloc, cudaHostRegister) are read by the
-                                         ingestion kernel in place; pageable ones are copied to the device first.
+                                         ingestion kernel in place; pageable ones are read by the CPU and copied to
+                                         the device first; device memory is refused with DISCO_EINVAL.
                                          Either way they may be reused as soon as disco_load_trace returns.
                                          2: host memory that is always copied first, by the copy engine: the transfer
                                          then leaves the multiprocessors free, so that it can run beside the kernels

@@ -344,15 +344,17 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     cudaError_t e;
     // Host arrays that are page-locked and mapped (cudaHostAlloc, cudaHostRegister, a pinned tensor) are read by
     // the ingestion kernel in place (it reads every element exactly once): no staging copies.  Pageable arrays are
-    // packed and copied by several threads.
+    // packed and copied by several threads, which must not meet device memory.
     const void* in_place[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     Inputs in = d->arrays_on_device == 1 ? IN_DEVICE : (d->arrays_on_device == 2 || n == 0) ? IN_COPIED : IN_PLACE;
     if (in == IN_PLACE) {
         const void* host[5] = {d->prompt_len, d->output_len, d->server_ttft_s, d->server_profile, d->device_profile};
-        for (int k = 0; k < 5 && in == IN_PLACE; ++k) {
+        for (int k = 0; k < 5; ++k) {
             if (!host[k]) continue;
             cudaPointerAttributes attr;
-            if (cudaPointerGetAttributes(&attr, host[k]) != cudaSuccess) { cudaGetLastError(); in = IN_PACKED; break; }
+            if (cudaPointerGetAttributes(&attr, host[k]) != cudaSuccess) { cudaGetLastError(); in = IN_PACKED; continue; }
+            if (attr.type == cudaMemoryTypeDevice)
+                return bail(fail(DISCO_EINVAL, "a trace array is device memory, but arrays_on_device says host memory"));
             if (attr.type != cudaMemoryTypeHost || !attr.devicePointer) in = IN_PACKED;
             else in_place[k] = attr.devicePointer;
         }

@@ -79,3 +79,21 @@ assert fake.fake_loads() == loads + 1
 assert (fake.fake_last_ticks() == ticks) == {in_place}
 assert fake.fake_copied() == {0 if in_place else 4 * 9000}
 """)
+
+
+@pytest.mark.parametrize("column", range(5))
+@pytest.mark.parametrize("others", ["pageable", "pinned"])
+@pytest.mark.parametrize("device", [0, 1])
+def test_device_memory_given_as_host_memory_is_refused(fake, column, others, device):
+    # (ordinary host arrays are packed by the CPU, which must not touch device memory), whichever column it is
+    _run(fake, f"""
+ctx = C.c_void_p(None)
+keep, cols = host_columns(5000)
+if "{others}" == "pinned":
+    for c in keep:
+        fake.fake_memory(c.ctypes.data, c.nbytes, HOST, 0)
+assert load(ctx, 5000, cols) == 0, L.disco_last_error()
+cols[{column}] = unreadable(5000, DEVICE, {device})
+assert load(ctx, 5000, cols) == -1 and b"device memory" in L.disco_last_error()
+assert load(ctx, 0, cols) == 0, L.disco_last_error()         # (of an empty trace nothing is read)
+""")
