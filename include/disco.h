@@ -217,8 +217,8 @@ int64_t disco_get_group_tables(disco_ctx_t* ctx, uint32_t g, int64_t* cnt, int32
  * group g, in any order within the group, `ticks` in host or device memory, any device's (for instance the shards'
  * sorted ticks one after the other).  The library sorts them per group and rebuilds the cumulative token mass
  * (Eq. 3) and the 257 knots of F.  The context keeps its own requests.  DISCO_EINVAL if a group's length
- * counts do not add up to n_ticks[g] or a tick is negative (the context must then be reloaded).  Lasts until
- * the next disco_load_trace.  Synchronises `stream`. */
+ * counts do not add up to n_ticks[g], if there are more than 2^32 - 2^20 ticks in all, or if a tick is negative
+ * (the context must then be reloaded).  Lasts until the next disco_load_trace.  Synchronises `stream`. */
 int disco_set_group_tables(disco_ctx_t* ctx, const int64_t* cnt, const int32_t* ticks, const uint64_t* n_ticks,
                            void* stream);
 

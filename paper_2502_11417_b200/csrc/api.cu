@@ -1106,7 +1106,7 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
         if (by_length != n_ticks[g])
             return fail(DISCO_EINVAL, "length counts do not add up to the number of TTFT ticks (group " + std::to_string(g) + ")");
         total += n_ticks[g];
-        if (total > 0xFFFFFFFFull) return fail(DISCO_EINVAL, "more than 2^32 - 1 requests behind the tables");
+        if (total > kMaxTicks) return fail(DISCO_EINVAL, "more than 2^32 - 2^20 requests behind the tables");
         off[g + 1] = (uint32_t)total;
     }
     if (total && !ticks) return fail(DISCO_EINVAL, "null argument");

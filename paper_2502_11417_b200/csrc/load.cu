@@ -41,6 +41,7 @@ constexpr uint32_t kMaxRange = 1u << 18;  // values a dense bin may span
 constexpr uint32_t kMaxCount = 1u << 22;  // ticks a dense bin may hold
 constexpr int kPrivateGroups = 7;         // groups whose counters fit in shared memory (29 KB each)
 constexpr int kPrivateTickGroups = 16;    // the same, counters of tick bins alone
+static_assert(kMaxTicks + (uint64_t)kLoadBlocks * kThreads * 4 <= 1ull << 32, "a step of the loops over the ticks");
 
 enum Source { S_TRACE, S_TICKS, S_TTFT };
 enum Form { F_COLUMNS, F_STAGE, F_PACKED };   // a trace's columns; the same, with a copy left for the second pass; packed

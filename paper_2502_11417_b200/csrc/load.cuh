@@ -24,6 +24,9 @@ struct LoadReadback {            // what the host needs after a load; pinned hos
 
 // Words that a load or a sort must find zero, contiguous.
 constexpr uint32_t kLoadBlocks = 256;     // blocks of the kernel, at most
+// The ticks that the sorts take, at most.  They are counted in 32 bits by loops that step by up to 2^20 (256 blocks of 1,024
+// threads with four each): an index below this, and one step on, does not wrap.
+constexpr uint64_t kMaxTicks = (1ull << 32) - (1ull << 20);
 struct LoadZero {
     unsigned long long part[2][kLoadBlocks];      // sums over the blocks' shares of the counters: sum << 1 | 1
     uint64_t grp_sum_n[kMaxGroups];       // output tokens per group

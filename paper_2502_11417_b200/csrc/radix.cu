@@ -11,6 +11,10 @@ namespace {
 
 constexpr int kRadixThreads = 256;
 constexpr int kRadixWarps = kRadixThreads / 32;
+constexpr uint32_t kWideBlocks = 4096;            // blocks of the kernels that take a key a thread, at most
+// (a block's share of the keys is rounded up to whole rows of kRadixThreads, and its tiles reach 1,024 keys on)
+static_assert(kMaxTicks + (uint64_t)(kRadixMaxBlocks + 8) * kRadixThreads <= 1ull << 32 &&
+              kMaxTicks + (uint64_t)kWideBlocks * kRadixThreads <= 1ull << 32, "32-bit indices");
 
 __global__ void k_radix_hist(const uint64_t* __restrict__ keys, uint32_t n, uint32_t per_block, int shift,
                              uint32_t* __restrict__ counts /* [256][gridDim.x] */) {
@@ -130,7 +134,7 @@ uint32_t radix_sort_launches(int G) { return 2 + 3 * (G > 1 ? 5 : 4); }
 cudaError_t radix_sort_ticks(const int32_t* ticks, const uint32_t* off, int G, uint32_t total, uint64_t* keys_a, uint64_t* keys_b,
                              uint32_t* counts, int32_t* out, int sms, cudaStream_t st) {
     if (total == 0) return cudaSuccess;
-    const uint32_t wide = std::min<uint32_t>((total + 255u) / 256u, (uint32_t)sms * 16u);
+    const uint32_t wide = std::min<uint32_t>((total + 255u) / 256u, std::min((uint32_t)sms * 16u, kWideBlocks));
     k_keys_of_grouped_ticks<<<wide, 256, 0, st>>>(total, ticks, off, G, keys_a);
     uint32_t blocks = std::min<uint32_t>((total + 1023u) / 1024u, kRadixMaxBlocks);
     uint32_t per_block = (total + blocks - 1) / blocks;

@@ -2,8 +2,8 @@
 // the real one).  Device and page-locked memory is ordinary memory, kernels are not run; the ingestion kernel's launch
 // leaves a report of an accepted trace and is remembered.  A test says what memory a range of addresses is to be taken for.
 #include <cuda_runtime_api.h>
+#include <sys/mman.h>
 
-#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <string>
@@ -57,10 +57,14 @@ cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 1; return cudaSuccess; }
-cudaError_t cudaMalloc(void** p, size_t n) { *p = std::calloc(n, 1); return *p ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaMalloc(void** p, size_t n) {
+    // (a mapping: large sizes cost nothing until they are touched; not given back, a case is a short process)
+    *p = mmap(nullptr, n, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
+    return *p != MAP_FAILED ? cudaSuccess : cudaErrorMemoryAllocation;
+}
 cudaError_t cudaMallocHost(void** p, size_t n) { return cudaMalloc(p, n); }
-cudaError_t cudaFree(void* p) { std::free(p); return cudaSuccess; }
-cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
+cudaError_t cudaFree(void*) { return cudaSuccess; }
+cudaError_t cudaFreeHost(void*) { return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* to, const void* from, size_t n, cudaMemcpyKind, cudaStream_t) {
     if (range_of(from)) copied += n;              // (may not be readable here)
     else std::memcpy(to, from, n);

@@ -97,3 +97,16 @@ cols[{column}] = unreadable(5000, DEVICE, {device})
 assert load(ctx, 5000, cols) == -1 and b"device memory" in L.disco_last_error()
 assert load(ctx, 0, cols) == 0, L.disco_last_error()         # (of an empty trace nothing is read)
 """)
+
+
+@pytest.mark.parametrize("over", [-1, 0, 1, 2**20 - 1])
+def test_more_ticks_than_the_kernels_can_count_are_refused(fake, over):
+    # the kernels' 32-bit loops step by up to 2^20 ticks
+    _run(fake, f"""
+ctx = C.c_void_p(None)
+keep, cols = host_columns(5000)
+assert load(ctx, 5000, cols) == 0, L.disco_last_error()
+loads, total = fake.fake_loads(), 2**32 - 2**20 + {over}
+rc = set_tables(ctx, total, unreadable(total, DEVICE))
+assert (rc, fake.fake_loads() - loads) == {(0, 1) if over <= 0 else (-1, 0)}, (rc, L.disco_last_error())
+""")
