@@ -175,12 +175,12 @@ int prep_group(const orc_trace& tr, const orc_policy_t& p, uint32_t g, orc_prep_
         out->l_immediate = (int32_t)p.l_immediate;
         const double limit = (b * (double)G.Total) * (double)G.N;
         auto started_tokens = [&](int64_t beta) {
-            int64_t acc = 0;
+            __int128 acc = 0;                                /* up to Total N */
             for (int32_t l = 1; l <= ORC_MAX_PROMPT; ++l) {
                 if (G.cnt[l] == 0) continue;
                 const int64_t w = l <= out->l_immediate ? 0 : std::min(beta * (int64_t)l, out->w_tail);
                 const int64_t later = G.N - (std::upper_bound(G.sorted.begin(), G.sorted.end(), w) - G.sorted.begin());
-                acc += (int64_t)l * G.cnt[l] * later;
+                acc += (__int128)((int64_t)l * G.cnt[l]) * later;
             }
             return acc;
         };

@@ -851,7 +851,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     g_launches += 1;
     if (n_beta) {
         CU(launch_prep_beta(d_pol, P, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
-                            c->F_off, c->tick_start.as<uint32_t>(), c->tick_cnt, d_tab + beta_at, n_beta, c->d_prep.as<Prep>(), st));
+                            c->F_off, c->tick_start.as<uint32_t>(), c->tick_cnt, d_tab + beta_at, n_beta,
+                            *std::max_element(c->F_n.begin(), c->F_n.end()), c->d_prep.as<Prep>(), st));
         g_launches += 1;
     }
 

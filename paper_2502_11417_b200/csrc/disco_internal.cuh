@@ -236,7 +236,8 @@ cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupCo
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off,
                              const uint32_t* tick_start, const uint32_t* tick_cnt /* [G][kTickBins], of the sorted ticks */,
-                             const uint32_t* pairs /* [n_pairs]: g P + p */, uint32_t n_pairs, Prep* prep, cudaStream_t st);
+                             const uint32_t* pairs /* [n_pairs]: g P + p */, uint32_t n_pairs,
+                             uint64_t most /* ticks of a group, at most */, Prep* prep, cudaStream_t st);
 // Plays every request under one class.  `kinds`: bit k set if some group with requests is of GroupKind k; `batches[k]`:
 // batches of 32 requests of the groups of kind k.
 cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0 /* hash key base: seed_key(seed) + first_index * kHashReq */,

@@ -1,5 +1,6 @@
 // Policy preparation: Algorithms 1-3 for every (group, policy).
 #include <algorithm>
+#include <type_traits>
 
 #include "load.cuh"
 
@@ -106,19 +107,22 @@ k_prep(const PolicyConst* __restrict__ pol, uint32_t P, int G, const GroupConst*
     if ((threadIdx.x & 31) == 0) prep[(size_t)g * P + p] = r;
 }
 
-// The largest whole x with (double)x <= limit (>= 0): sums are compared as whole numbers, since converting every sum in
-// every thread took most of a round of the search below (4,200 cycles a round with hardly a request to add up).
-__device__ long long last_within(double limit) {
-    if (limit >= 9223372036854774784.0) return 0x7FFFFFFFFFFFFFFFll;  // (the last double below 2^63)
-    const long long x = (long long)limit;                             // (rounded down)
-    if (limit < 9007199254740992.0) return x;                         // below 2^53 every whole number is a double
-    const long long half = 1ll << ((int)(__double_as_longlong(limit) >> 52) - 1023 - 53);    // of the doubles' distance there
-    return (double)(x + half) <= limit ? x + half : x + half - 1;     // (ties go to the even one)
+// The largest whole x with (double)x <= limit (>= 0, and below what Sum holds): sums are compared as whole numbers, since
+// converting every sum in every thread took most of a round of the search below (4,200 cycles a round with hardly a
+// request to add up).
+template <class Sum>
+__device__ Sum last_within(double limit) {
+    if (limit < 9007199254740992.0) return (long long)limit;          // below 2^53 every whole number is a double (rounded down)
+    const long long bits = __double_as_longlong(limit), mantissa = (bits & 0xFFFFFFFFFFFFFll) | 1ll << 52;
+    const int shift = (int)(bits >> 52) - 1023 - 52;                  // limit = mantissa 2^shift, half the doubles' distance 2^(shift - 1)
+    const Sum last = ((Sum)mantissa << shift) + ((Sum)1 << (shift - 1));
+    return (mantissa & 1) ? last - 1 : last;                          // (ties go to the even one)
 }
 
 // Eq. 1-2 variant of phase 2, one block per (group, policy): the smallest whole slope beta (ticks per prompt
 // token) with  sum_l l cnt[l] #{S > w(l)} <= b Total N,  w(l) = 0 for l <= l_immediate, min(beta l, w_tail) above.
-// The sum is exact (it is below Total N < 2^63); it does not grow with beta, so beta is found by search: three slopes a
+// The sum is exact: it is at most Total N <= 4,096 N^2, which 64 bits hold up to kBetaLargeN requests in the group, and 128
+// (LARGE) beyond.  It does not grow with beta, so beta is found by search: three slopes a
 // round, which cut the range to a quarter.  A thread keeps four prompt lengths and, for each, the two positions in the
 // sorted ticks that belong to the ends of the range, between which the positions of the slopes in between lie; the first
 // and last positions come from the bins' starts in shared memory.  Bound: latency (two barriers and a few dependent loads a
@@ -128,7 +132,10 @@ __device__ long long last_within(double limit) {
 constexpr int kBetaThreads = 1024;
 constexpr int kBetaLens = kMaxPrompt / kBetaThreads;                  // prompt lengths a thread has
 static_assert(kBetaLens * kBetaThreads == kMaxPrompt, "lengths 1 .. 4096");
+constexpr uint64_t kBetaLargeN = 47453132;
+static_assert(kMaxPrompt * kBetaLargeN < (1ull << 63) / kBetaLargeN && kMaxPrompt * (kBetaLargeN + 1) >= (1ull << 63) / (kBetaLargeN + 1), "the last N");
 
+template <bool LARGE>
 __global__ void __launch_bounds__(kBetaThreads)
 k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __restrict__ cum_mass,
             const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
@@ -136,6 +143,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
             Prep* __restrict__ prep) {
     __shared__ uint32_t s_end[kTickBins];                             // ticks of the group up to the bin's last
     __shared__ long long part[8][32], total[6];
+    using Sum = typename std::conditional<LARGE, __int128, long long>::type;
     grid_dependency_wait();
     const uint32_t pair = pairs[blockIdx.x], p = pair % P;
     const int g = (int)(pair / P);
@@ -147,7 +155,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
     const uint32_t off = grp_off[g], N = grp_off[g + 1] - off;
     const int32_t* srt = sorted + off;
     const double Total = (double)cum_mass[(size_t)g * (kMaxPrompt + 2) + kMaxPrompt + 1];
-    const long long limit = last_within(__dmul_rn(__dmul_rn((double)pc.budget, Total), (double)N));
+    const Sum limit = last_within<Sum>(__dmul_rn(__dmul_rn((double)pc.budget, Total), (double)N));
     const long long w_tail = pr.w_tail, l_imm = pr.l_star;
     for (int k = threadIdx.x; k < kTickBins; k += kBetaThreads)
         s_end[k] = tick_start[(size_t)g * kTickBins + k] + tick_cnt[(size_t)g * kTickBins + k] - off;
@@ -176,7 +184,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
     }
     // the block's sums of the values, the same to all threads.  Over a warp the lanes halve what they add up at every step
     // (nine exchanges for six values, not thirty); a warp then adds up the warps' parts of one value for all.
-    auto totals = [&](auto& v) {
+    auto add_up = [&](auto& v) {
         constexpr int kValues = (int)(sizeof(v) / sizeof(v[0])), kHold = kValues <= 2 ? 2 : kValues <= 4 ? 4 : 8;
         long long x[kHold];
 #pragma unroll
@@ -201,6 +209,20 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
 #pragma unroll
         for (int j = 0; j < kValues; ++j) v[j] = total[j];
     };
+    auto totals = [&](auto& v) {
+        if constexpr (!LARGE) {
+            add_up(v);
+        } else {
+            constexpr int kValues = (int)(sizeof(v) / sizeof(v[0]));
+            long long low[kValues], high[kValues];                    // 48 bits, and those above (28 at most)
+#pragma unroll
+            for (int j = 0; j < kValues; ++j) { low[j] = (long long)(v[j] & 0xFFFFFFFFFFFFll); high[j] = (long long)(v[j] >> 48); }
+            add_up(low);
+            add_up(high);
+#pragma unroll
+            for (int j = 0; j < kValues; ++j) v[j] = ((Sum)high[j] << 48) + low[j];
+        }
+    };
     auto wait = [&](long long beta, int l) { return l <= l_imm ? 0ll : min(beta * (long long)l, w_tail); };
     long long lo = 0, hi = w_tail + 1;                                // beyond hi every wait is w_tail
     // ---- first by whole bins: the ticks up to a bin's first and last bound the sum from both sides, which settles most of
@@ -208,11 +230,11 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
     while (hi - lo > 1) {
         const long long d = hi - lo;
         const long long m[3] = {lo + (d + 3) / 4, lo + (d + 1) / 2, lo + (3 * d + 3) / 4};
-        long long v[6] = {0, 0, 0, 0, 0, 0};                          // at least, at most
+        Sum v[6] = {0, 0, 0, 0, 0, 0};                                // at least, at most
 #pragma unroll
         for (int i = 0; i < kBetaLens; ++i) {
             if (k[i] == 0) continue;
-            const long long mass = (long long)len[i] * (long long)k[i];
+            const Sum mass = (long long)len[i] * (long long)k[i];
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const int bin = tick_bin((uint32_t)wait(m[j], len[i]));
@@ -230,15 +252,16 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
     }
     // ---- the positions at the ends of what is left
     {
-        long long v[2] = {0, 0};
+        Sum v[2] = {0, 0};
 #pragma unroll
         for (int i = 0; i < kBetaLens; ++i) {
             at_lo[i] = at_hi[i] = 0;
             if (k[i] == 0) continue;
             at_lo[i] = position(wait(lo, len[i]), 0u, N);
             at_hi[i] = len[i] <= l_imm ? at_lo[i] : position(wait(hi, len[i]), at_lo[i], N);
-            v[0] += (long long)len[i] * (long long)k[i] * (long long)(N - at_lo[i]);
-            v[1] += (long long)len[i] * (long long)k[i] * (long long)(N - at_hi[i]);
+            const Sum mass = (long long)len[i] * (long long)k[i];
+            v[0] += mass * (long long)(N - at_lo[i]);
+            v[1] += mass * (long long)(N - at_hi[i]);
         }
         totals(v);
         if (lo == 0 && v[0] <= limit) hi = lo;                // (no waits at all fit)
@@ -249,14 +272,14 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
         const long long d = hi - lo;
         const long long m[3] = {lo + (d + 3) / 4, lo + (d + 1) / 2, lo + (3 * d + 3) / 4};     // (ascending, above lo, at most hi)
         uint32_t at[3][kBetaLens];
-        long long v[3] = {0, 0, 0};
+        Sum v[3] = {0, 0, 0};
 #pragma unroll
         for (int i = 0; i < kBetaLens; ++i) {
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 at[j][i] = at_lo[i];
                 if (k[i] != 0 && at_lo[i] < at_hi[i]) at[j][i] = position(wait(m[j], len[i]), at_lo[i], at_hi[i]);
-                v[j] += (long long)len[i] * (long long)k[i] * (long long)(N - at[j][i]);
+                v[j] += (Sum)((long long)len[i] * (long long)k[i]) * (long long)(N - at[j][i]);
             }
         }
         totals(v);
@@ -288,8 +311,9 @@ cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupCo
 
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off, const uint32_t* tick_start,
-                             const uint32_t* tick_cnt, const uint32_t* pairs, uint32_t n_pairs, Prep* prep, cudaStream_t st) {
-    return launch_after(k_prep_beta, n_pairs, kBetaThreads, 0, st, pol, P, cum_mass, cnt, sorted, grp_off, tick_start,
+                             const uint32_t* tick_cnt, const uint32_t* pairs, uint32_t n_pairs, uint64_t most, Prep* prep, cudaStream_t st) {
+    auto* kernel = most > kBetaLargeN ? k_prep_beta<true> : k_prep_beta<false>;
+    return launch_after(kernel, n_pairs, kBetaThreads, 0, st, pol, P, cum_mass, cnt, sorted, grp_off, tick_start,
                         tick_cnt, pairs, prep);
 }
 

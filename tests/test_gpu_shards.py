@@ -136,3 +136,46 @@ def test_tables_are_checked():
     with pytest.raises(DiscoError):
         Trace().load_trace(w.prompt_len, w.output_len, w.server_ttft_s, None, None, w.servers, w.devices,
                            first_index=(1 << 32) - 100)
+
+
+@pytest.mark.parametrize("n", [1_000_000, 47_453_132, 47_453_133, 60_000_007])
+def test_slope_search_behind_tables_of_many_requests(n):
+    # Eq. 1-2 sums up to (input tokens) x (requests), which 64 bits hold up to 47,453,132 requests of a group; against whole
+    # numbers of any size.  A few waits are shared by most requests, a million are spread between them.
+    import torch
+    often = {150_000: 0.3, 450_000: 0.25, 800_000: 0.2, 1_500_000: 0.15, 9_000_000: 0.1}
+    rng = np.random.default_rng(n)
+    light = np.sort(rng.integers(100_000, 3_000_000, size=min(n // 2, 1_000_000)).astype(np.int64))
+    bins = np.array(sorted(often), dtype=np.float32).view(np.int32) >> 16        # (a value and nothing else in its bin)
+    light = light[~np.isin(light.astype(np.float32).view(np.int32) >> 16, bins)]
+    heavy = {v: int(share * (n - len(light))) for v, share in often.items()}
+    heavy[150_000] += n - len(light) - sum(heavy.values())
+    ticks = torch.cat([torch.full((c,), v, dtype=torch.int32, device="cuda") for v, c in heavy.items()] +
+                      [torch.from_numpy(light.astype(np.int32)).cuda()])
+    cnt = np.zeros((1, 4097), np.int64)
+    cnt[0, [17, 900, 4095]] = n // 50
+    cnt[0, 4096] = n - 3 * (n // 50)
+    w = synth.make_workload(1, n=500, n_budgets=2)
+    tr = Trace.from_workload(w)
+    tr.set_group_tables(cnt, ticks, np.array([n], np.uint64))
+    pols = [synth.policy(b, flags=MIG | PACE | synth.FLAG_BETA_RULE | synth.MODE_DEVICE_CONSTRAINED, l_immediate=li)
+            for b in (0.1, 0.35, 0.8) for li in (0, 64)]
+    tr.eval_policies(pols, 1)
+    total = sum(int(l) * int(cnt[0, l]) for l in np.flatnonzero(cnt[0]))
+    for p, pol in enumerate(pols):
+        got = tr.prep(0, p)
+        limit = (float(np.float32(pol["budget"])) * float(total)) * float(n)
+
+        def started(beta):
+            acc = 0
+            for l in np.flatnonzero(cnt[0]):
+                wait = 0 if l <= pol["l_immediate"] else min(beta * int(l), got.w_tail)
+                above = len(light) - int(np.searchsorted(light, wait, side="right")) + sum(c for v, c in heavy.items() if v > wait)
+                acc += int(l) * int(cnt[0, l]) * above
+            return acc
+        lo, hi = 0, got.w_tail + 1
+        while lo < hi and float(started(hi)) <= limit:
+            mid = (lo + hi) // 2
+            lo, hi = (lo, mid) if float(started(mid)) <= limit else (mid + 1, hi)
+        assert got.beta == hi, (p, got.beta, hi)
+    tr.close()
