@@ -169,7 +169,7 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
             hi = min(hi, s_end[bin]);
         }
         while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
+            const uint32_t mid = LARGE ? lo + ((hi - lo) >> 1) : (lo + hi) >> 1;       // (their sum may pass 2^32)
             if (!DBG_OK(mid, N, DBG_K_PREP, DBG_ELEMENT)) break;
             if ((long long)srt[mid] <= w) lo = mid + 1; else hi = mid;
         }

@@ -138,10 +138,11 @@ def test_tables_are_checked():
                            first_index=(1 << 32) - 100)
 
 
-@pytest.mark.parametrize("n", [1_000_000, 47_453_132, 47_453_133, 60_000_007])
+@pytest.mark.parametrize("n", [1_000_000, 47_453_132, 47_453_133, 60_000_007, 3_221_225_479])
 def test_slope_search_behind_tables_of_many_requests(n):
     # Eq. 1-2 sums up to (input tokens) x (requests), which 64 bits hold up to 47,453,132 requests of a group; against whole
-    # numbers of any size.  A few waits are shared by most requests, a million are spread between them.
+    # numbers of any size.  A few waits are shared by most requests, a million are spread between them.  (The largest: places
+    # whose sum passes 2^32.)
     import torch
     often = {150_000: 0.3, 450_000: 0.25, 800_000: 0.2, 1_500_000: 0.15, 9_000_000: 0.1}
     rng = np.random.default_rng(n)
@@ -179,3 +180,5 @@ def test_slope_search_behind_tables_of_many_requests(n):
             lo, hi = (lo, mid) if float(started(mid)) <= limit else (mid + 1, hi)
         assert got.beta == hi, (p, got.beta, hi)
     tr.close()
+    del ticks
+    torch.cuda.empty_cache()
