@@ -150,3 +150,17 @@ def test_eight_overheads(n, dearer):
     w = synth.tiny_workload(101, n, max_prompt=64, max_out=60, device_dearer=dearer)
     thetas = (0.0, 1e-7, 1e-6, 4e-6, 1e-5, 3e-5, 1e-4, 1.0)
     full_parity(w, [synth.policy(b, mig_threshold=t) for b in (0.0, 0.01, 0.03, 0.4, 0.8) for t in thetas], select=False, tag=f"{n}")
+
+
+@pytest.mark.parametrize("dearer", [False, True])
+@pytest.mark.parametrize("overheads", [3, 4, 5, 8])
+@pytest.mark.parametrize("n", [257, 9000])
+def test_windows_under_several_overheads(n, overheads, dearer):
+    # streams whose intervals are not all tau take their windows to every row of the grid, and the rows that migrate take
+    # them back: without pacing, with a device slower than the reader, with either endpoint slower at times; and, for
+    # comparison, even streams.  The overheads lie between the requests' savings: every level has some.
+    w = synth.tiny_workload(103, n, max_prompt=64, max_out=60, device_dearer=dearer)
+    thetas = (0.0, 0.004, 0.012, 0.02, 0.03, 0.06, 0.12, 1.0)[:overheads]
+    grid = [(b, t) for b in (0.0, 0.01, 0.03, 0.4, 0.8) for t in thetas]
+    for how in (dict(flags=synth.FLAG_MIGRATION), dict(r_c=25.0, t_m_s=0.2), dict(r_c=30.0, t_m_s=0.3), dict(t_m_s=0.4)):
+        full_parity(w, [synth.policy(b, mig_threshold=t, **how) for b, t in grid], select=False, tag=f"{n} x {overheads} {how}")
