@@ -30,7 +30,6 @@ constexpr uint64_t kMaxTicks = (1ull << 32) - (1ull << 20);
 struct LoadZero {
     unsigned long long part[2][kLoadBlocks];      // sums over the blocks' shares of the counters: sum << 1 | 1
     uint64_t grp_sum_n[kMaxGroups];       // output tokens per group
-    uint32_t ng[kMaxGroups];              // requests per group
     uint32_t max_n;                       // longest output
     uint32_t barrier, done, pad;
     int32_t err[4];                       // code, request index, window flag, sort flag (1: some bin needs the fallback, 2: a
