@@ -27,6 +27,10 @@ int fail_cuda(cudaError_t e, const char* what) {
     g_err = std::string(what) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? DISCO_ENOMEM : DISCO_ECUDA;
 }
+// Nothing throws across the C boundary.  (Messages that a string holds without allocating.)
+#define DISCO_CATCH                                                          \
+    catch (const std::bad_alloc&) { return fail(DISCO_ENOMEM, "out of memory"); } \
+    catch (...) { return fail(DISCO_ECUDA, "host exception"); }
 #define CU(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) return fail_cuda(e_, #call); } while (0)
 
 // A growable device buffer.
@@ -59,7 +63,9 @@ using HostReadback = LoadReadback;   // pinned host mirror of the load's read-ba
 }  // namespace
 
 namespace disco {
-int set_error(int code, const char* msg) { return fail(code, msg); }
+int set_error(int code, const char* msg) {
+    try { return fail(code, msg); } catch (...) { g_err.clear(); return code; }
+}
 
 cudaError_t allow_smem(const void* kernel, size_t bytes) {
     // (kernel, device, size) that have been allowed: a few dozen at most
@@ -70,7 +76,7 @@ cudaError_t allow_smem(const void* kernel, size_t bytes) {
     if (e) return e;
     for (const Allowed& x : seen) if (x.kernel == kernel && x.device == dev && x.bytes >= bytes) return cudaSuccess;
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes))) return e;
-    seen.push_back({kernel, dev, bytes});
+    try { seen.push_back({kernel, dev, bytes}); } catch (...) {}       // (asked for again, then)
     return cudaSuccess;
 }
 
@@ -312,7 +318,7 @@ const char* disco_last_error(void) { return g_err.c_str(); }
 
 void disco_free_trace(disco_ctx_t* ctx) { delete ctx; }
 
-int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stream) {
+int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stream) try {
     if (!pctx || !d) return fail(DISCO_EINVAL, "null argument");
     if (d->n >= (1ull << 31)) return fail(DISCO_EINVAL, "too many requests");
     if (d->n && (!d->prompt_len || !d->output_len || !d->server_ttft_s)) return fail(DISCO_EINVAL, "null trace array");
@@ -328,7 +334,8 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
         c = new (std::nothrow) disco_ctx;
         if (!c) return fail(DISCO_ENOMEM, "out of host memory");
     }
-    auto bail = [&](int rc) { if (fresh) delete c; else c->loaded = false; return rc; };
+    std::unique_ptr<disco_ctx> own(fresh ? c : nullptr);              // (until the load has succeeded)
+    auto bail = [&](int rc) { c->loaded = false; return rc; };
     c->loaded = c->evaluated = c->reduced = false;
     c->n = (uint32_t)d->n; c->ns = d->n_servers; c->nd = d->n_devices; c->G = (int)gc.size(); c->gc = gc;
     c->first_index = d->first_index;
@@ -437,12 +444,13 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     c->F_sorted = c->sorted.as<int32_t>(); c->F_off = c->grp_off.as<uint32_t>();
     c->F_n.assign(rb->ng, rb->ng + c->G);
     c->loaded = true;
+    own.release();
     *pctx = c;
     return 0;
-}
+} DISCO_CATCH
 
 int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, uint64_t seed,
-                        const disco_pair_out_t* out, void* stream) {
+                        const disco_pair_out_t* out, void* stream) try {
     if (!c || !pol || P == 0) return fail(DISCO_EINVAL, "null context, null policies or P = 0");
     if (!c->loaded) return fail(DISCO_EINVAL, "no trace loaded");
     if (P > (1u << 19)) return fail(DISCO_EINVAL, "too many policies");
@@ -920,9 +928,9 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     c->P = P; c->pol.swap(pc);
     c->evaluated = true;
     return 0;
-}
+} DISCO_CATCH
 
-int disco_reduce_stats(disco_ctx_t* c, disco_policy_stats_t* stats, void* stream) {
+int disco_reduce_stats(disco_ctx_t* c, disco_policy_stats_t* stats, void* stream) try {
     if (!c || !stats) return fail(DISCO_EINVAL, "null argument");
     if (!c->evaluated) return fail(DISCO_EINVAL, "no evaluation to reduce");
     cudaStream_t st = (cudaStream_t)stream;
@@ -954,10 +962,10 @@ int disco_reduce_stats(disco_ctx_t* c, disco_policy_stats_t* stats, void* stream
     if (c->rb->err[2]) return fail(DISCO_ECUDA, "internal error: an inter-token interval fell outside its histogram window");
     c->reduced = true;
     return 0;
-}
+} DISCO_CATCH
 
 int disco_select_policy(const disco_policy_stats_t* stats, uint32_t P, double cost_cap, float tbt_slo_s,
-                        int32_t* best) {
+                        int32_t* best) try {
     if (!stats || !best || P == 0) return fail(DISCO_EINVAL, "null argument or P = 0");
     if (P > (1u << 19)) return fail(DISCO_EINVAL, "too many policies");
     // lexicographic objective: feasible first; then (P99 TTFT bin, mean TTFT, cost, index); none feasible: cheapest
@@ -987,9 +995,9 @@ int disco_select_policy(const disco_policy_stats_t* stats, uint32_t P, double co
     *best = (int32_t)pick;
     if (!pick_ok) return fail(DISCO_EINFEASIBLE, "no policy meets the cost cap and the TBT objective");
     return 0;
-}
+} DISCO_CATCH
 
-int disco_select_policy_device(disco_ctx_t* c, double cost_cap, float tbt_slo_s, int32_t* best, void* stream) {
+int disco_select_policy_device(disco_ctx_t* c, double cost_cap, float tbt_slo_s, int32_t* best, void* stream) try {
     if (!c || !best) return fail(DISCO_EINVAL, "null argument");
     if (!c->reduced) return fail(DISCO_EINVAL, "reduce the statistics before selecting");
     cudaStream_t st = (cudaStream_t)stream;
@@ -1000,44 +1008,44 @@ int disco_select_policy_device(disco_ctx_t* c, double cost_cap, float tbt_slo_s,
     *best = c->sel_host[1];
     if (c->sel_host[0] != 0) return fail(DISCO_EINFEASIBLE, "no policy meets the cost cap and the TBT objective");
     return 0;
-}
+} DISCO_CATCH
 
 uint64_t disco_kernel_launch_count(void) { return g_launches.load(); }
 
-int disco_set_timing(disco_ctx_t* c, int on) {
+int disco_set_timing(disco_ctx_t* c, int on) try {
     if (!c) return fail(DISCO_EINVAL, "null context");
     if (on) for (auto& e : c->ev) if (!e) CU(cudaEventCreate(&e));
     c->timing = on != 0;
     c->timing_valid = false;
     return 0;
-}
+} DISCO_CATCH
 
-int disco_get_timing(disco_ctx_t* c, float* ms4) {
+int disco_get_timing(disco_ctx_t* c, float* ms4) try {
     if (!c || !ms4) return fail(DISCO_EINVAL, "null argument");
     if (!c->timing_valid || !c->reduced) return fail(DISCO_EINVAL, "no timed evaluation has been reduced");
     for (int k = 0; k < 4; ++k) ms4[k] = c->ms[k];
     return 0;
-}
+} DISCO_CATCH
 
-int disco_get_work_counts(disco_ctx_t* c, uint64_t* counts4, void* stream) {
+int disco_get_work_counts(disco_ctx_t* c, uint64_t* counts4, void* stream) try {
     if (!c || !counts4) return fail(DISCO_EINVAL, "null argument");
     if (!c->evaluated) return fail(DISCO_EINVAL, "no evaluation");
     cudaStream_t st = (cudaStream_t)stream;
     CU(cudaMemcpyAsync(counts4, c->d_work.p, 32, cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
     return 0;
-}
+} DISCO_CATCH
 
-int disco_get_histograms(disco_ctx_t* c, uint32_t p, uint64_t* ttft_hist, uint64_t* tbt_hist, void* stream) {
+int disco_get_histograms(disco_ctx_t* c, uint32_t p, uint64_t* ttft_hist, uint64_t* tbt_hist, void* stream) try {
     if (!c || !c->evaluated || p >= c->P) return fail(DISCO_EINVAL, "no evaluation or policy index out of range");
     cudaStream_t st = (cudaStream_t)stream;
     if (ttft_hist) CU(cudaMemcpyAsync(ttft_hist, c->d_hist_ttft.as<uint64_t>() + (size_t)p * kNBins, kNBins * 8, cudaMemcpyDeviceToHost, st));
     if (tbt_hist) CU(cudaMemcpyAsync(tbt_hist, c->d_hist_tbt.as<uint64_t>() + (size_t)p * kNBins, kNBins * 8, cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
     return 0;
-}
+} DISCO_CATCH
 
-int disco_get_prep(disco_ctx_t* c, uint32_t g, uint32_t p, disco_prep_t* out, void* stream) {
+int disco_get_prep(disco_ctx_t* c, uint32_t g, uint32_t p, disco_prep_t* out, void* stream) try {
     if (!c || !out || !c->evaluated || p >= c->P || g >= (uint32_t)c->G) return fail(DISCO_EINVAL, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
     Prep pr;
@@ -1048,10 +1056,10 @@ int disco_get_prep(disco_ctx_t* c, uint32_t g, uint32_t p, disco_prep_t* out, vo
     out->beta_rule = pr.beta_rule; out->l_immediate = pr.beta_rule ? pr.l_star : 0; out->beta = pr.beta_rule ? pr.w_star : 0;
     if (pr.beta_rule) { out->l_star = 0; out->w_star = 0; }
     return 0;
-}
+} DISCO_CATCH
 
 int64_t disco_get_group_tables(disco_ctx_t* c, uint32_t g, int64_t* cnt, int32_t* knots, int32_t* sorted_ticks,
-                               uint64_t n_sorted, void* stream) {
+                               uint64_t n_sorted, void* stream) try {
     if (!c || !c->loaded || g >= (uint32_t)c->G) return fail(DISCO_EINVAL, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
     // the tables Algorithms 1-3 read: the trace's own, or the whole trace's a caller has set
@@ -1081,10 +1089,10 @@ int64_t disco_get_group_tables(disco_ctx_t* c, uint32_t g, int64_t* cnt, int32_t
     if (cnt) for (size_t i = 0; i < kLengths; ++i) cnt[i] = c->tab_host[g * kLengths + i];
     if (knots && knots_on_host) std::memcpy(knots, host_knots(c, (int)g), kNKnots * 4);
     return (int64_t)ng;
-}
+} DISCO_CATCH
 
 int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ticks, const uint64_t* n_ticks,
-                           void* stream) {
+                           void* stream) try {
     if (!c || !cnt || !n_ticks) return fail(DISCO_EINVAL, "null argument");
     if (!c->loaded) return fail(DISCO_EINVAL, "no trace loaded");
     cudaStream_t st = (cudaStream_t)stream;
@@ -1169,14 +1177,14 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     c->tables_imported = true;
     for (int g = 0; g < G; ++g) { c->F_n[g] = n_ticks[g]; c->rb->knot_max[g] = host_knots(c, g)[kNKnots - 1]; }
     return 0;
-}
+} DISCO_CATCH
 
 uint64_t disco_accumulator_words(disco_ctx_t* c) {
     if (!c || !c->evaluated) return 0;
     return (uint64_t)c->P * c->G * kNAcc + 2ull * c->P * kNBins + 2ull * c->G;
 }
 
-int disco_export_accumulators(disco_ctx_t* c, uint64_t* words, void* stream) {
+int disco_export_accumulators(disco_ctx_t* c, uint64_t* words, void* stream) try {
     if (!c || !words) return fail(DISCO_EINVAL, "null argument");
     if (!c->evaluated) return fail(DISCO_EINVAL, "no evaluation to export");
     cudaStream_t st = (cudaStream_t)stream;
@@ -1185,9 +1193,9 @@ int disco_export_accumulators(disco_ctx_t* c, uint64_t* words, void* stream) {
     CU(cudaMemcpyAsync(words + head, c->fin_totals.p, (size_t)2 * c->G * 8, cudaMemcpyDefault, st));
     CU(cudaStreamSynchronize(st));
     return 0;
-}
+} DISCO_CATCH
 
-int disco_import_accumulators(disco_ctx_t* c, const uint64_t* words, void* stream) {
+int disco_import_accumulators(disco_ctx_t* c, const uint64_t* words, void* stream) try {
     if (!c || !words) return fail(DISCO_EINVAL, "null argument");
     if (!c->evaluated) return fail(DISCO_EINVAL, "evaluate the policies first: the accumulators take their shape from it");
     cudaStream_t st = (cudaStream_t)stream;
@@ -1198,9 +1206,9 @@ int disco_import_accumulators(disco_ctx_t* c, const uint64_t* words, void* strea
     c->reduced = false;
     c->fin_imported = true;
     return 0;
-}
+} DISCO_CATCH
 
-int disco_debug_selftest(void* stream) {
+int disco_debug_selftest(void* stream) try {
 #ifdef DISCO_DEBUG
     // a kernel offers an index beyond its bound to the check: the access is skipped, the record comes back as an error
     CU(run_debug_selftest((cudaStream_t)stream));
@@ -1211,9 +1219,9 @@ int disco_debug_selftest(void* stream) {
     (void)stream;
     return fail(DISCO_EINVAL, "not a checked build (compile with -DDISCO_DEBUG)");
 #endif
-}
+} DISCO_CATCH
 
-int disco_measure_alu_peak(double* lane_instr_per_s, double* token_steps_per_s, void* stream) {
+int disco_measure_alu_peak(double* lane_instr_per_s, double* token_steps_per_s, void* stream) try {
     if (!lane_instr_per_s) return fail(DISCO_EINVAL, "null argument");
     int dev = 0, sms = 0;
     CU(cudaGetDevice(&dev));
@@ -1224,6 +1232,6 @@ int disco_measure_alu_peak(double* lane_instr_per_s, double* token_steps_per_s, 
     *lane_instr_per_s = rate * 13.0;
     if (token_steps_per_s) *token_steps_per_s = rate;
     return 0;
-}
+} DISCO_CATCH
 
 }  // extern "C"

@@ -110,3 +110,21 @@ loads, total = fake.fake_loads(), 2**32 - 2**20 + {over}
 rc = set_tables(ctx, total, unreadable(total, DEVICE))
 assert (rc, fake.fake_loads() - loads) == {(0, 1) if over <= 0 else (-1, 0)}, (rc, L.disco_last_error())
 """)
+
+
+def test_host_memory_that_runs_out_is_an_error_code(fake):
+    # nothing throws across the C boundary: 2^19 policies with 16 MB of address space left, then as much as there was
+    _run(fake, """
+import resource
+ctx = C.c_void_p(None)
+keep, cols = host_columns(5000)
+assert load(ctx, 5000, cols) == 0, L.disco_last_error()
+pols = api.policy_array([synth.policy(0.5)] * (1 << 19))
+before = resource.getrlimit(resource.RLIMIT_AS)
+now = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (now + (16 << 20), before[1]))
+rc = L.disco_eval_policies(ctx, pols, len(pols), 1, None, None)
+resource.setrlimit(resource.RLIMIT_AS, before)
+assert rc == -2 and b"memory" in L.disco_last_error(), (rc, L.disco_last_error())
+assert L.disco_eval_policies(ctx, pols, 2, 1, None, None) == 0, L.disco_last_error()
+""")
