@@ -33,22 +33,26 @@ METRIC = "request-policy evaluations/s"
 UNIT = "pairs/s"
 PAIR_OUT_BYTES = 31          # four fp32, three u32, one u16, one u8 per pair
 TRACE_BYTES = 9              # packed request: ticks, prompt, output length, group
+# Bytes a request needs of the ingestion: its columns read (lengths, TTFT, two profile ids), its record and ticks written.
+LOAD_BYTES = 14 + 16 + 4
 # Bytes a request whose stream cannot fall behind the reader needs of the play-out (one class): its record read, the
-# hand-off written; it is played up to the hand-off only, some buffer's worth of tokens that no count of streams gives.
+# hand-off written.
 PLAYOUT_BYTES = 16 + 8
+# Lane-instructions it needs: it is played up to the hand-off only, one endpoint's draws; per token counter add 1, hash
+# finaliser 8, range map (multiply-high) 1, sum 1, comparison 1, loop 1.
+HANDOFF_INSTR_PER_TOKEN = 13
 # Lane-instructions one token-step of the play-out needs where every token counts (no pacing, or generation slower than
 # consumption; both endpoints' streams share the hash draw): counter add 1, hash finaliser 8, two range maps
 # (multiply-high) 2, tail mask 1, two sums and two maxima 4, loop 1.
 PLAYOUT_INSTR_PER_TOKEN = 17
 # Bytes a request needs of the reductions per slab of a grid of policies (at most 256 budgets by 8 overheads): its record
-# and its hand-off read.
+# and its hand-off read.  Lane-instructions: a dozen for the dispatch, the race and the sums, and per overhead a comparison
+# and three additions.
 GRID_BYTES = 16 + 8
+GRID_INSTR, GRID_INSTR_PER_ROW = 12, 4
 SCHEDULERS, LANES = 4, 32    # warp schedulers per multiprocessor, lanes per warp
 MIN_WARMUP_SECONDS = 0.5     # untimed steps run until this much device time has passed (and at least --warmup)
 MAX_WARMUP_STEPS = 200
-# From the committed ncu captures (profiles/): DRAM bytes per launch of the bench's own launch shape.  None: not captured
-# for the current kernel.
-NCU_TRAFFIC_BYTES = {}
 HEADLINE_CONFIG = 4
 ALL_CONFIGS = (0, 1, 2, 3, 4, 5)
 
@@ -130,6 +134,30 @@ def never_clamps(w):
             if T + int(round(T * float(np.float32(dv["jitter"])))) > tau:
                 return False
     return True
+
+
+def handoff_draws(w, lo, hi):
+    """Tokens that have to be drawn to find the hand-offs of the requests lo .. hi - 1, for paced policies of one rate and
+    buffer: with B buffered tokens a stream that generates a token every T hands over about (B - 1) tau / (tau - T) + 1
+    tokens on, or never if it is shorter.  Only a stream whose endpoint is the dearer decoder hands over."""
+    pol = w.policies[0]
+    tau = 1.0 / float(np.float32(pol["r_c"]))
+    B = math.ceil(float(pol["t_m_s"]) / tau - 1e-9)
+    nd, total = len(w.devices), 0.0
+    group = np.zeros(hi - lo, np.int64)
+    if w.server_profile is not None:
+        group += w.server_profile[lo:hi].astype(np.int64) * nd
+    if w.device_profile is not None:
+        group += w.device_profile[lo:hi]
+    for s, sv in enumerate(w.servers):
+        for d, dv in enumerate(w.devices):
+            device_cost = dv["lam"] * dv["c_decode"]
+            if device_cost == sv["c_decode"]:
+                continue
+            T = 1.0 / dv["decode_tps"] if device_cost > sv["c_decode"] else sv["tbt_s"]
+            draws = (B - 1) * tau / (tau - T) + 1.0 if T < tau else float("inf")
+            total += float(np.minimum(w.output_len[lo:hi][group == s * nd + d] - 1, max(draws, 0.0)).sum())
+    return total
 
 
 def max_over_ranks(total_ms, dist, device):
@@ -346,9 +374,13 @@ class Bench:
         cap_factor, slo = w.select["cost_cap_factor"], w.select["tbt_slo_s"]
         words = None
 
-        def step(arrays):
+        def step(arrays, around_load=None):
             nonlocal words
+            if around_load is not None:
+                around_load[0].record(stream)
             tr.load_trace(*arrays, w.servers, w.devices, stream=stream, first_index=lo)
+            if around_load is not None:
+                around_load[1].record(stream)
             if sharded:
                 # exchange 1: every rank needs the whole trace's p(l) and F before Algorithms 1-3 run
                 cnt = np.stack([tr.group_tables(g, n_sorted=0)[0] for g in range(G)])
@@ -373,15 +405,18 @@ class Bench:
             evs = []
             for _ in range(k):
                 flush.zero_()
+                load = None
                 if collect is not None:
                     tr.set_timing(True)
+                    load = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                 e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                 e0.record(stream)
-                step(arrays)
+                step(arrays, load)
                 e1.record(stream)
                 evs.append((e0, e1))
                 if collect is not None:
-                    collect.append(tr.timing())
+                    load[1].synchronize()
+                    collect.append([load[0].elapsed_time(load[1])] + list(tr.timing()))
             torch.cuda.synchronize()
             return sum(a.elapsed_time(b) for a, b in evs)
 
@@ -436,19 +471,17 @@ class Bench:
         # ---- rooflines of the timed kernels
         hbm_gbs, sm_max_mhz, src = self.peaks
         sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-        names = ["k_playout_short", "k_playout", "k_grid+k_spread+k_pairs_acc", "k_pairs_rows"]
+        names = ["k_load", "k_playout_short", "k_playout", "k_grid+k_spread+k_pairs_acc", "k_pairs_rows"]
         kms = {nm: statistics.mean(t[i] for t in ktimes) for i, nm in enumerate(names)}
         alu_peak = sms * SCHEDULERS * LANES * sm_max_mhz * 1e6 / 1e12         # T lane-instructions/s
         alu_src = "%d SMs x %d schedulers x %d lanes x %.0f MHz (issue slots)" % (sms, SCHEDULERS, LANES, sm_max_mhz)
         alu_meas = self.alu_measured / 1e12 if self.alu_measured else None
         paced = never_clamps(w)
-        full_size = not args.requests and not args.budgets
 
         def alu_roof(name, lane_instr, ms, **extra):
             ach = lane_instr / (ms * 1e-3) / 1e12
             r = {"kernel": name, "bound": "alu", "achieved": ach, "peak": alu_peak, "unit": "Tinstr/s",
-                 "frac": ach / alu_peak, "traffic": NCU_TRAFFIC_BYTES.get((name, cfg)) if full_size else None,
-                 "peak_source": alu_src,
+                 "frac": ach / alu_peak, "traffic": None, "peak_source": alu_src, "lane_instructions": lane_instr,
                  # what the GPU sustains on the token loop's own instruction mix with every SM full
                  # (disco_measure_alu_peak, measured in this run)
                  "peak_measured": alu_meas, "frac_of_measured": ach / alu_meas if alu_meas else None,
@@ -459,24 +492,34 @@ class Bench:
         def hbm_roof(name, bytes_alg, ms, **extra):
             ach = bytes_alg / (ms * 1e-3) / 1e9
             return {"kernel": name, "bound": "hbm", "achieved": ach, "peak": hbm_gbs, "unit": "GB/s",
-                    "frac": ach / hbm_gbs, "traffic": NCU_TRAFFIC_BYTES.get((name, cfg)) if full_size else None,
-                    "peak_source": src, "algorithmic_bytes": bytes_alg, "ms_per_launch": ms, **extra}
+                    "frac": ach / hbm_gbs, "traffic": None, "peak_source": src, "algorithmic_bytes": bytes_alg,
+                    "ms_per_launch": ms, **extra}
+
+        def either_roof(name, bytes_alg, lane_instr, ms, **extra):
+            # what the path needs of both; held against the one that would take longer
+            hbm, alu = hbm_roof(name, bytes_alg, ms), alu_roof(name, lane_instr, ms)
+            r = hbm if hbm["frac"] > alu["frac"] else alu
+            r.update(extra, hbm_frac=hbm["frac"], issue_frac=alu["frac"], algorithmic_bytes=bytes_alg, lane_instructions=lane_instr)
+            return r
 
         def roof_of(name):
             ms = kms[name]
             if ms <= 0.0:
                 return None
+            if name == "k_load":
+                return hbm_roof(name, n * LOAD_BYTES, ms, timed="disco_load_trace: clearing and the kernel")
             if name == "k_pairs_rows":
                 return hbm_roof(name, n * P * PAIR_OUT_BYTES + n * TRACE_BYTES, ms) if w.materialise else None
             if name == "k_grid+k_spread+k_pairs_acc":
                 # the reduction kernels together (their events bracket them): requests settled run by run per slab of
                 # policies, and the pairs left to the pair-by-pair kernel
                 grid_pairs, left_pairs, settled, sweeps = tr.work_counts()
-                return hbm_roof(name, settled * GRID_BYTES, ms, limited_by="issue slots (ncu)",
-                                work={"pairs_by_runs": grid_pairs, "pairs_one_by_one": left_pairs,
-                                      "requests_settled_per_slab": settled, "segment_sweeps": sweeps})
-            if name == "k_playout_short" and paced:
-                return hbm_roof(name, n * n_classes * PLAYOUT_BYTES, ms, limited_by="issue slots (ncu)")
+                rows = min(8, len({float(q["mig_threshold"]) for q in w.policies}))
+                return either_roof(name, settled * GRID_BYTES, settled * (GRID_INSTR + GRID_INSTR_PER_ROW * rows), ms,
+                                   work={"pairs_by_runs": grid_pairs, "pairs_one_by_one": left_pairs,
+                                         "requests_settled_per_slab": settled, "segment_sweeps": sweeps})
+            if name == "k_playout_short" and paced and n_classes == 1:
+                return either_roof(name, n * PLAYOUT_BYTES, handoff_draws(w, lo, hi) * HANDOFF_INSTR_PER_TOKEN, ms)
             if name == "k_playout" and not paced:
                 return alu_roof(name, token_steps * PLAYOUT_INSTR_PER_TOKEN * n_classes, ms,
                                 token_steps=token_steps * n_classes, instr_per_token_step=PLAYOUT_INSTR_PER_TOKEN)
@@ -486,8 +529,8 @@ class Bench:
         roof = None
         if roofs:
             roof = dict(max(roofs, key=lambda r: r["ms_per_launch"]))
-            roof["all_kernels"] = [{k: r.get(k) for k in ("kernel", "bound", "achieved", "peak", "unit", "frac",
-                                                          "frac_of_measured", "ms_per_launch")} for r in roofs]
+            roof["all_kernels"] = [{k: r.get(k) for k in ("kernel", "bound", "achieved", "peak", "unit", "frac", "hbm_frac",
+                                                          "issue_frac", "frac_of_measured", "ms_per_launch")} for r in roofs]
             roof["kernels_ms"] = kms
             roof["kernel_event_samples"] = len(ktimes)
         cpu = None
