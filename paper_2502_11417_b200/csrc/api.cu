@@ -741,9 +741,10 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         L.slab1 = slabs.size();
     }
 
-    // ---- request chunks, of one group each: of the grid kernel, about two to each block that fits the GPU at once (three
-    //      where that is more than 16,384 requests: the end of the launch is then worth more than the entering of runs), 256
-    //      requests (one a thread) or more; of the pair kernel, two to a multiprocessor, 2,048 requests or more
+    // ---- request chunks, of one group each: of the grid kernel, about two to each block that fits the GPU at once, 256
+    //      requests (one a thread) or more (three to a block: k_grid and k_spread for 16 M requests in six groups under 128
+    //      budgets by 8 overheads 369 us either way, under 16 by 2 218 instead of 205, in one group under 64 budgets 139
+    //      instead of 133, a million 34 instead of 30); of the pair kernel, two to a multiprocessor, 2,048 requests or more
     const uint32_t sms = (uint32_t)c->sms, kMaxChunk = 65280;
     int tallest = 1;
     for (const Slab& sl : slabs) tallest = std::max(tallest, sl.T);
@@ -766,7 +767,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         return v;
     };
     const size_t at_once = (size_t)sms * grid_blocks_per_sm(tallest);
-    const std::vector<Chunk> chunks = make_chunks(chunk_size(at_once * (N1 / at_once > 2 * 16384 ? 3 : 2), 256));
+    const std::vector<Chunk> chunks = make_chunks(chunk_size(2 * at_once, 256));
     std::vector<Chunk> pair_chunks;
     if (any_pairs) pair_chunks = make_chunks(chunk_size((size_t)2 * sms, 2048));
 
