@@ -26,7 +26,7 @@
 // Bound: integer issue.  Against one sweep per 128 policies of one overhead, with what differs between neighbouring
 // policies entered into their histograms one by one, a request is visited once per run instead of once per run and
 // overhead: 16 M requests in six groups under 128 budgets by 8 overheads took 2,300 us (and 450 more pair by pair), now
-// 436; a million in one group under 256 by 4 took 220 us, now 36.
+// 349 and k_spread 18; a million in one group under 256 by 4 took 220 us, now 35 and 15.
 #include <algorithm>
 #include <cstddef>
 #include <type_traits>
@@ -45,7 +45,8 @@ constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr uint32_t kNoPolicy = 0xFFFFFFFFu;
 static_assert(kNBins % 32 == 0 && kNBins / 32 < 32, "a bit for each group of bins");
 
-// Blocks to a multiprocessor by the rows a kernel is built for: what their registers allow without spilling.
+// Blocks to a multiprocessor by the rows a kernel is built for: as many as its registers allow with few spills (64 registers:
+// 136 bytes in k_grid<1, true>, 16 in <2, false>; 80: 8 in <2, true>, 20 in <4, true>; the others none).
 __host__ __device__ constexpr int blocks_for(int rows, bool wide) { return rows == 1 || (rows == 2 && !wide) ? 4 : rows <= 4 ? 3 : 2; }
 // The rows of the kernel that takes a slab of T.
 constexpr int rows_for(int T) { return T <= 1 ? 1 : T <= 2 ? 2 : T <= 4 ? 4 : 8; }
@@ -190,8 +191,8 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                                       uint32_t pb, uint32_t w, bool list, bool push, bool race, bool only, Acc<NT>& s, Only& o) {
     const int lane = threadIdx.x & 31;
     // The kernel of eight rows has too few warps a multiprocessor to hide the loads' latency: there they run an iteration
-    // ahead (16 M requests under 128 budgets by 8 overheads 365 us instead of 435; the others have the warps, and no
-    // registers left: 3 % slower).
+    // ahead (16 M requests under 128 budgets by 8 overheads, with k_spread, 369 us instead of 435; the others have the
+    // warps, and no registers left: 3 % slower).
     constexpr bool kAhead = NT == 8 && !WIDE;
     uint32_t pos;
     uint4 q, q_ahead;
@@ -713,8 +714,8 @@ k_grid(const __grid_constant__ Args a) {
 // Adds up the difference rows: what a policy gets is the sum of the rows up to its column.  A block takes 32 histogram
 // bins (or sums) of one row of the grid, a lane each, and all columns, a few consecutive ones a warp: the warps add up
 // their own rows, the totals meet in shared memory, and every warp writes its columns' policies.  Bound: L2 and the
-// stores (the tables are read once, every policy's histograms written once).  (One thread a bin, walking the columns:
-// 202 us at 256 x 4 policies.)
+// stores (the tables are read once, every policy's histograms written once).  (256 x 4 policies: 15 us; one thread a bin,
+// walking the columns, 202.  The 64 registers that 1,024 threads leave spill 204 bytes, 68 with windows.)
 constexpr int kSpreadWarps = 32;
 constexpr int kSpreadPer = kGridCols / kSpreadWarps;                   // columns a warp may have
 static_assert(kNBins % 32 == 0, "a block's bins");

@@ -16,8 +16,9 @@
 //
 // Bound: latency at 10^5 requests (one launch instead of eighteen), memory at 10^7: the columns are read twice (once when
 // they are in host memory: then the first pass leaves a copy), 20 bytes a request are written to scattered places, the
-// ticks are read and written once more.  16 M requests in six groups: 1,800 us by a chain of kernels, 886 now, over half
-// of it the scattered places (linear stores in their stead: 106 us for that pass instead of 470); a million: 69 us.
+// ticks are read and written once more.  16 M requests in six groups: 1,800 us by a chain of kernels, 850 now, over half
+// of it the scattered places (linear stores in their stead: 106 us for that pass instead of 470); a million: 70 us.  (The 64
+// registers that 1,024 threads leave spill 32 bytes.)
 #include "load.cuh"
 
 #include <algorithm>
@@ -507,7 +508,9 @@ k_load(const __grid_constant__ LoadArgs a) {
                                      : aligned(a.ttft, 16) && (!kTrace || (aligned(a.prompt, 16) && aligned(a.outlen, 16) && aligned(a.sp, 4) && aligned(a.dp, 4)));
     const uint32_t stride = gridDim.x * kThreads * 4u, i_first = (blockIdx.x * kThreads + tid) * 4u;
     uint32_t i_next = i_first;                                         // (second pass)
-    uint32_t tok[kPrivateGroups] = {};                                 // output tokens per group
+    // Output tokens per group, of this thread's requests: below 2^32.  (Above 16,384 requests more than four blocks share a
+    // trace, so that of 2^31 a thread has fewer than 2^19, of 8,192 tokens at most.)
+    uint32_t tok[kPrivateGroups] = {};
     uint32_t longest = 0;
 #pragma unroll 1
     for (uint32_t i0 = i_first; i0 < a.n; i0 += stride) {
@@ -530,7 +533,7 @@ k_load(const __grid_constant__ LoadArgs a) {
                 longest = max(longest, y.o);
                 if (PRIV) {
 #pragma unroll
-                    for (int g = 0; g < kPrivateGroups; ++g) tok[g] += (int)y.g == g ? y.o : 0u;    // (at most 2^21 requests a thread)
+                    for (int g = 0; g < kPrivateGroups; ++g) tok[g] += (int)y.g == g ? y.o : 0u;
                 }
             }
         }

@@ -234,7 +234,7 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
 // what is left of the longer ones is made up by a warp each, 32 tokens at a time, so that the longest (thousands of
 // tokens) does not hold the block for as many dependent steps.  A thread draws 32 tokens, or 256 where most of the block's
 // requests have longer lags (prompts that take a device long to read: those lags are alike).  (Without the collection:
-// 513 us for the 16 M requests of three server profiles and two devices, 43 us for 250,000 of them; now 245 and 12.)
+// 513 us for the 16 M requests of three server profiles and two devices, 43 us for 250,000 of them; now 304 and 12.)
 constexpr uint32_t kShortSearch = 64;
 constexpr int kShortThreads = 256;
 constexpr int kShortPer = 4;             // requests a thread may play

@@ -127,7 +127,7 @@ __device__ Sum last_within(double limit) {
 // sorted ticks that belong to the ends of the range, between which the positions of the slopes in between lie; the first
 // and last positions come from the bins' starts in shared memory.  Bound: latency (two barriers and a few dependent loads a
 // round, some fourteen rounds).  (300,000 requests in six groups under sixteen such policies: 437 us with a bisection whose
-// every step searched all the ticks for every length, 85 us now.  Four blocks a pair gave 4 us with few pairs and lost 15
+// every step searched all the ticks for every length, 79 us now.  Four blocks a pair gave 4 us with few pairs and lost 15
 // once the pairs outnumbered the multiprocessors; three searches in step gave nothing.)
 constexpr int kBetaThreads = 1024;
 constexpr int kBetaLens = kMaxPrompt / kBetaThreads;                  // prompt lengths a thread has

@@ -92,7 +92,7 @@ def _oracle_stats_threaded(orc, policies, seed, threads=None):
 
 @pytest.mark.parametrize("cfg,n", [(2, 6000), (4, 9000)])
 def test_whole_policy_grid_against_oracle_on_a_short_trace(cfg, n):
-    # all 1024 policies (32 full policy tiles), no per-pair arrays: every statistic and histogram, and the selection
+    # all 1024 policies (256 budgets by 4 overheads, 128 by 8), no per-pair arrays: every statistic and histogram, and the selection
     from parity import check_stats
     w = synth.make_workload(cfg, n=n)
     assert len(w.policies) == 1024
@@ -232,7 +232,7 @@ def test_pair_arrays_beyond_2_32_elements():
 @pytest.mark.parametrize("cfg,policy_step", [(3, 1), (4, 1)])
 def test_aggregates_on_262144_requests(cfg, policy_step):
     # traces of 2^18 requests with the shape of workloads 3 and 4 under ALL their policies (many chunks, several
-    # waves of blocks, six groups and 32 full policy tiles for workload 4): tables, every statistic and histogram
+    # waves of blocks, six groups and 128 budgets by 8 overheads for workload 4): tables, every statistic and histogram
     # against the oracle run on host threads
     from parity import check_stats, check_tables
     w = synth.make_workload(cfg, n=1 << 18)

@@ -17,7 +17,7 @@ def test_config0_full():
 
 
 def test_config1_shape_ragged_tiles():
-    # several request chunks and policy tiles, none of them full
+    # several request chunks, none of them full, and fewer budgets than a slab has
     w = synth.make_workload(1, n=7013, n_budgets=21)
     full_parity(w, tag="config1-small")
 
@@ -72,8 +72,8 @@ def test_generation_slower_than_consumption():
 
 
 def test_long_outputs_with_and_without_clamping():
-    # mean output above 512 tokens (four requests per warp round); r_c = 5 never clamps, r_c = 30 does for the
-    # phone-class device (10 tok/s), so both forms of the clamp-free kernel and its to-do list run
+    # mean output above 512 tokens; at r_c = 5 no stream falls behind the reader (hand-off kernels, with a shallow and a
+    # deep buffer), at r_c = 30 the server does at times and the phone-class device (10 tok/s) always: the general play-out
     w = synth.make_workload(3, n=1200, n_budgets=3)
     assert w.output_len.mean() >= 512
     pols = [synth.policy(b, r_c=rc, t_m_s=tm) for b in (0.3, 1.0) for rc, tm in ((5.0, 1.0), (30.0, 0.3), (5.0, 4.0))]
@@ -93,8 +93,8 @@ def test_consumption_interval_equal_to_slowest_token():
 
 @pytest.mark.parametrize("top_s", [16.70, 16.80, 1500.0])
 def test_sorted_ticks_around_the_fourth_radix_byte(top_s):
-    # one-group traces whose largest TTFT lies just below 2^24 ticks (the fourth radix pass skips itself), just
-    # above it and far above it: the sorted sample, the knots and everything derived from them
+    # one-group traces whose largest TTFT lies just below 2^24 ticks (an octave of bins ends there, and whole numbers stop
+    # being floats), just above it and far above it: the sorted sample, the knots and everything derived from them
     w = synth.make_workload(1, n=6000, n_budgets=5)
     w.server_ttft_s[::97] *= np.float32(7.0)
     w.server_ttft_s[5] = np.float32(top_s)
@@ -121,7 +121,7 @@ def test_stochastic_baselines_and_expected_length():
         gs, _ = full_parity(w, pols, tag=f"next dear={dear}")
         assert gs[0].n_race == 0 and gs[3].n_race == 0
         assert all(gs[first_both + k].n_race == 0 and gs[first_both + k].n_migrations == 0 for k in range(len(both)))
-        # a tile of such policies alone (staged histogram increments in the reduction kernel)
+        # such policies alone (the pair kernel then stages its histogram increments)
         full_parity(w, both, tag=f"stoch+beta dear={dear}")
 
 
@@ -329,7 +329,7 @@ def test_quantile_rank_reached_at_a_bin_boundary():
 
 def test_pinned_host_inputs_read_in_place_match_pageable_ones():
     # one profile group: page-locked host arrays are read by the ingestion kernel in place, pageable ones are
-    # copied first; both must give the same tables and statistics (and the oracle's)
+    # packed and copied first; both must give the same tables and statistics (and the oracle's)
     import torch
     from parity import check_tables
     from oracle import Oracle
@@ -351,14 +351,14 @@ def test_pinned_host_inputs_read_in_place_match_pageable_ones():
 
 
 def test_pinned_host_inputs_of_several_groups_and_staged_copies():
-    # six groups: page-locked arrays are read in place as well (packed copies of the lengths feed the partition);
+    # six groups: page-locked arrays are read in place as well (the first pass leaves a copy for the second);
     # arrays_on_device = 2 copies them with the copy engine instead.  All three routes give identical records.
     import torch
     from parity import check_tables
     from oracle import Oracle
     w = synth.make_workload(4, n=25013, n_budgets=3)
     cols = (w.prompt_len, w.output_len, w.server_ttft_s, w.server_profile, w.device_profile)
-    a = Trace.from_workload(w)                                  # pageable numpy arrays: copied
+    a = Trace.from_workload(w)                                  # pageable numpy arrays: packed
     a.eval_policies(w.policies, 9)
     sa = a.reduce_stats()
     pinned = [torch.from_numpy(x).pin_memory() for x in cols]
@@ -436,17 +436,17 @@ def _work(w, pols):
 
 
 def test_zone_by_zone_reduction_and_what_it_leaves_to_the_pair_kernel():
-    # ascending budgets: a tile's policies are ordered, so requests are settled against runs of policies; what the
-    # runs cannot express goes pair by pair.  Every variant must give the oracle's numbers.
-    for dear in (False, True):                     # Algorithm 3 tiles, Algorithm 2 tiles
+    # the budgets of like policies are ordered, so requests are settled against runs of neighbouring ones; what the runs
+    # cannot express goes pair by pair.  Every variant must give the oracle's numbers.
+    for dear in (False, True):                     # Algorithm 3, Algorithm 2
         w = synth.tiny_workload(51 + dear, 6000, n_servers=2, n_devices=1, max_prompt=900, max_out=160, device_dearer=dear)
         grid = synth.budget_grid(40)
-        # one overhead per tile: nothing but the odd request is left over
+        # one overhead: nothing is left over
         plain = [synth.policy(b, mig_threshold=0.004) for b in grid]
         full_parity(w, plain, tag=f"zones plain dear={dear}")
         zone, left, _, corr = _work(w, plain)
         assert zone > 0.9 * w.n * len(plain) and corr > 0
-        # overheads that alternate inside a tile: requests whose saving lies between them are left to the pair kernel
+        # an overhead of its own for each budget: requests whose saving lies between them are left to the pair kernel
         mixed = [synth.policy(b, mig_threshold=(0.0, 0.05, synth.INF)[k % 3]) for k, b in enumerate(grid)]
         full_parity(w, mixed, tag=f"zones mixed overheads dear={dear}")
         zone, left, _, _ = _work(w, mixed)
@@ -459,7 +459,7 @@ def test_zone_by_zone_reduction_and_what_it_leaves_to_the_pair_kernel():
         shuffled = [plain[k] for k in rng.permutation(len(plain))]
         full_parity(w, shuffled, tag=f"zones shuffled dear={dear}")
         assert _work(w, shuffled)[0] > 0.9 * w.n * len(plain)
-        # random routing has no ordered thresholds: such tiles go pair by pair
+        # random routing has no ordered thresholds: such policies go pair by pair
         stoch = [synth.policy(b, flags=synth.FLAG_STOCHASTIC | PACE) for b in grid]
         full_parity(w, stoch, tag=f"zones none dear={dear}")
         assert _work(w, stoch)[0] == 0
@@ -471,8 +471,8 @@ def test_zone_by_zone_reduction_and_what_it_leaves_to_the_pair_kernel():
 
 
 def test_more_than_32_policy_tiles_use_several_flag_words():
-    # 1100 policies = 35 tiles: two flag words per request; overheads alternate so that requests are flagged in
-    # tiles of both words
+    # 1100 budgets whose overheads alternate: five slabs of a column per policy, each with requests whose saving lies
+    # between the overheads, which are left to the pair kernel
     w = synth.tiny_workload(61, 1500, n_servers=1, n_devices=2, max_prompt=700, max_out=120, device_dearer=True)
     pols = [synth.policy(b, mig_threshold=(0.0, 0.03)[k % 2]) for k, b in enumerate(synth.budget_grid(1100))]
     full_parity(w, pols, select=False, tag="35 tiles")
@@ -483,7 +483,7 @@ def test_more_than_32_policy_tiles_use_several_flag_words():
 def test_one_prompt_length_and_lengths_at_the_ends():
     # every request in one bucket of the internal order: a chunk is one segment (or a threshold's own), and all
     # lanes of a warp meet in one row and one histogram bin
-    grid = synth.budget_grid(70)                   # three policy tiles: a family of several tiles
+    grid = synth.budget_grid(70)
     for dear in (False, True):
         w = synth.tiny_workload(71 + dear, 5000, n_servers=1, n_devices=1, max_prompt=900, max_out=120, device_dearer=dear)
         w.prompt_len[:] = 300
@@ -494,8 +494,8 @@ def test_one_prompt_length_and_lengths_at_the_ends():
 
 
 def test_more_groups_than_fit_the_scatter_in_shared_memory():
-    # 3 x 3 = 9 groups: the internal request order is built with one add per warp and bucket to the global cursors
-    # (the length histograms of more than six groups do not fit the slice-wise kernel's shared memory)
+    # 3 x 3 = 9 groups: places in the internal request order come from global cursors (the counters of more than seven
+    # groups do not fit a block's shared memory)
     w = synth.tiny_workload(73, 9000, n_servers=3, n_devices=3, max_prompt=600, max_out=100)
     full_parity(w, [synth.policy(b, mig_threshold=0.01) for b in synth.budget_grid(40)], tag="nine groups")
     zone, left, _, _ = _work(w, [synth.policy(b, mig_threshold=0.01) for b in synth.budget_grid(40)])
@@ -503,13 +503,12 @@ def test_more_groups_than_fit_the_scatter_in_shared_memory():
 
 
 def test_family_whose_first_tile_alone_has_longer_waits():
-    # Algorithm 2 along 128 ascending budgets: the lowest budgets wait longest (w_tail falls until it settles), so a
-    # family of four tiles stays whole and requests under which the device wins after such a wait are left to the
-    # pair kernel for the first tile only
+    # Algorithm 2 along 128 ascending budgets: the lowest budgets wait longest (w_tail falls until it settles); the grid
+    # stays whole, and the requests that the common wait does not cover are listed and swept again for those budgets
     w = synth.tiny_workload(74, 20000, n_servers=1, n_devices=1, max_prompt=2000, max_out=200, device_dearer=True)
     pols = [synth.policy(b, mig_threshold=th) for th in (0.0, synth.INF) for b in synth.budget_grid(128)]
     full_parity(w, pols, select=False, tag="four-tile families with waits")
     zone, left, settled, _ = _work(w, pols)
     assert zone + left == w.n * len(pols)
     assert left < 0.1 * zone
-    assert settled <= 2 * w.n                      # one sweep per request and family, not per tile
+    assert settled <= 2 * w.n                      # once per slab
