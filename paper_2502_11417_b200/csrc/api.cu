@@ -388,6 +388,10 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     } else if (in == IN_PACKED) {
         if (!c->packer) c->packer.reset(new (std::nothrow) Packer);
         if (!c->packer) return bail(fail(DISCO_ENOMEM, "out of host memory"));
+        // The CPU reads the columns now, and work on the stream may still write them: page-locked or managed ones by copies and
+        // kernels, any by host functions.  (Asked first: to wait for an idle stream takes 3 us.)
+        if ((e = cudaStreamQuery(st)) == cudaErrorNotReady) { cudaGetLastError(); e = cudaStreamSynchronize(st); }
+        if (e != cudaSuccess) return bail(fail_cuda(e, "work in front of the load"));
         if ((e = c->packer->pack(*d, c->packed.as<char>(), st, &a.packed)) != cudaSuccess) return bail(fail_cuda(e, "packing the trace"));
     } else if (in == IN_PLACE) {
         a.prompt = (const int32_t*)in_place[0]; a.outlen = (const int32_t*)in_place[1]; a.ttft = (const float*)in_place[2];

@@ -17,6 +17,13 @@ std::vector<Range> ranges;
 std::map<const void*, std::string> kernels;
 uint64_t copied = 0, loads = 0;                 // bytes copied out of the ranges; ingestion kernels launched
 const void* last_ticks = nullptr;               // what the last of them was given
+uint32_t first_packed = 0;                      // ... and the lengths of the first request, if it was given a packed trace
+struct Write { void* to; const void* from; size_t bytes; };
+std::vector<Write> pending;                     // work that a stream still holds
+void finish() {
+    for (const Write& w : pending) std::memcpy(w.to, w.from, w.bytes);
+    pending.clear();
+}
 
 const Range* range_of(const void* p) {
     for (const Range& r : ranges) if ((const char*)p >= r.at && (const char*)p < r.at + r.bytes) return &r;
@@ -27,6 +34,7 @@ cudaError_t launch(const void* f, void** args) {
     const disco::LoadArgs& a = *(const disco::LoadArgs*)args[0];
     ++loads;
     last_ticks = a.ticks;
+    if (a.packed) first_packed = *(const uint32_t*)a.packed;
     if (a.readback) {
         std::memset(a.readback, 0, sizeof *a.readback);
         a.readback->ng[0] = a.readback->grp_off[1] = a.n;
@@ -42,6 +50,8 @@ void fake_memory(const void* at, size_t bytes, int type, int device) { ranges.pu
 uint64_t fake_copied(void) { return copied; }
 uint64_t fake_loads(void) { return loads; }
 const void* fake_last_ticks(void) { return last_ticks; }
+uint32_t fake_first_packed(void) { return first_packed; }
+void fake_pending(void* to, const void* from, size_t bytes) { pending.push_back({to, from, bytes}); }
 
 // ---- what the library calls
 void** __cudaRegisterFatBinary(void*) { static void* handle; return &handle; }
@@ -66,6 +76,7 @@ cudaError_t cudaMallocHost(void** p, size_t n) { return cudaMalloc(p, n); }
 cudaError_t cudaFree(void*) { return cudaSuccess; }
 cudaError_t cudaFreeHost(void*) { return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* to, const void* from, size_t n, cudaMemcpyKind, cudaStream_t) {
+    finish();                                     // (in stream order)
     if (range_of(from)) copied += n;              // (may not be readable here)
     else std::memcpy(to, from, n);
     return cudaSuccess;
@@ -81,7 +92,8 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
     return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void**, const void*) { return cudaErrorInvalidValue; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { finish(); return cudaSuccess; }
+cudaError_t cudaStreamQuery(cudaStream_t) { return pending.empty() ? cudaSuccess : cudaErrorNotReady; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)&ranges; return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }

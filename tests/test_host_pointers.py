@@ -128,3 +128,20 @@ resource.setrlimit(resource.RLIMIT_AS, before)
 assert rc == -2 and b"memory" in L.disco_last_error(), (rc, L.disco_last_error())
 assert L.disco_eval_policies(ctx, pols, 2, 1, None, None) == 0, L.disco_last_error()
 """)
+
+
+@pytest.mark.parametrize("lengths", ["pageable", "pinned", "managed"])
+def test_host_arrays_that_the_stream_still_writes(fake, lengths):
+    # what the CPU packs is read in the stream's order, as a copy would: page-locked columns (among pageable ones) may be the
+    # target of a copy under way, managed ones of a kernel
+    _run(fake, f"""
+ctx = C.c_void_p(None)
+keep, cols = host_columns(5000)
+kind = dict(pageable=None, pinned=HOST, managed=MANAGED)["{lengths}"]
+if kind:
+    fake.fake_memory(C.c_void_p(cols[0]), C.c_size_t(keep[0].nbytes), kind, 0)
+new = np.full(5000, 9, np.int32)
+fake.fake_pending(C.c_void_p(cols[0]), C.c_void_p(new.ctypes.data), C.c_size_t(new.nbytes))
+assert load(ctx, 5000, cols) == 0, L.disco_last_error()
+assert fake.fake_first_packed() == 9 | 5 << 16
+""")
