@@ -1130,15 +1130,15 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     if ((e = c->F_sorted_imp.reserve(T1 * 4)) != cudaSuccess || (e = c->F_off_imp.reserve((size_t)(kMaxGroups + 1) * 4)) != cudaSuccess ||
         (e = c->sort_in.reserve(2 * ((T1 + 3) / 4 * 4) * 4 + (size_t)sort_windows((uint32_t)total, G) * 8)) != cudaSuccess)
         return fail_cuda(e, "device allocation for the tables");
-    // ticks in this device's memory are read where they are (another device's may not be mapped here); sort_in: a copy of
-    // others, the same by bin, the windows
+    // ticks in this device's memory are read where they are (another device's may not be mapped here, and a kernel cannot read
+    // words across their alignment); sort_in: a copy of others, the same by bin, the windows
     bool on_device = false;
     if (total) {
         int dev = 0;
         CU(cudaGetDevice(&dev));
         cudaPointerAttributes attr;
         if (cudaPointerGetAttributes(&attr, ticks) != cudaSuccess) cudaGetLastError();
-        else on_device = (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged) && attr.device == dev;
+        else on_device = (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged) && attr.device == dev && (uintptr_t)ticks % alignof(int32_t) == 0;
     }
     int32_t* copy = c->sort_in.as<int32_t>();
     const int32_t* in = on_device ? ticks : copy;

@@ -145,3 +145,16 @@ fake.fake_pending(C.c_void_p(cols[0]), C.c_void_p(new.ctypes.data), C.c_size_t(n
 assert load(ctx, 5000, cols) == 0, L.disco_last_error()
 assert fake.fake_first_packed() == 9 | 5 << 16
 """)
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 4, 12])
+def test_ticks_off_their_alignment_are_copied(fake, offset):
+    _run(fake, f"""
+ctx = C.c_void_p(None)
+keep, cols = host_columns(5000)
+assert load(ctx, 5000, cols) == 0, L.disco_last_error()
+ticks = unreadable(9004, DEVICE) + {offset}
+assert set_tables(ctx, 9000, ticks) == 0, L.disco_last_error()
+assert (fake.fake_last_ticks() == ticks) == {offset % 4 == 0}
+assert fake.fake_copied() == {0 if offset % 4 == 0 else 4 * 9000}
+""")
