@@ -940,10 +940,11 @@ int disco_reduce_stats(disco_ctx_t* c, disco_policy_stats_t* stats, void* stream
     if (!c->evaluated) return fail(DISCO_EINVAL, "no evaluation to reduce");
     cudaStream_t st = (cudaStream_t)stream;
     // Statistics and the error word land in pinned host memory straight from the kernel: in the caller's array if it is
-    // page-locked (from a few dozen records on, where the copy would count), else in the context's.
+    // page-locked (from a few dozen records on, where the copy would count; the kernel writes words of eight bytes), else in
+    // the context's.
     const size_t bytes = c->P * sizeof(disco_policy_stats_t);
     disco_policy_stats_t* to = nullptr;
-    if (c->P >= 64) {
+    if (c->P >= 64 && (uintptr_t)stats % 8 == 0) {
         cudaPointerAttributes attr;
         if (cudaPointerGetAttributes(&attr, stats) != cudaSuccess) cudaGetLastError();
         else if (attr.type == cudaMemoryTypeHost && attr.devicePointer) to = (disco_policy_stats_t*)attr.devicePointer;

@@ -18,7 +18,7 @@ from paper_2502_11417_b200 import api, synth
 L, fake = api.lib(), C.CDLL(os.environ["LD_PRELOAD"])
 fake.fake_memory.argtypes = [C.c_void_p, C.c_size_t, C.c_int, C.c_int]
 fake.fake_copied.restype = fake.fake_loads.restype = C.c_uint64
-fake.fake_last_ticks.restype = C.c_void_p
+fake.fake_last_ticks.restype = fake.fake_last_stats.restype = C.c_void_p
 HOST, DEVICE, MANAGED = 1, 2, 3                       # cudaMemoryType
 
 libc = C.CDLL(None)
@@ -157,4 +157,21 @@ ticks = unreadable(9004, DEVICE) + {offset}
 assert set_tables(ctx, 9000, ticks) == 0, L.disco_last_error()
 assert (fake.fake_last_ticks() == ticks) == {offset % 4 == 0}
 assert fake.fake_copied() == {0 if offset % 4 == 0 else 4 * 9000}
+""")
+
+
+@pytest.mark.parametrize("offset", [0, 4, 8, 3])
+def test_statistics_off_their_alignment_are_copied(fake, offset):
+    # from 64 policies on the kernel writes 8-byte words straight into a page-locked array
+    _run(fake, f"""
+ctx = C.c_void_p(None)
+keep, cols = host_columns(5000)
+assert load(ctx, 5000, cols) == 0, L.disco_last_error()
+pols = api.policy_array([synth.policy(k / 63) for k in range(64)])
+assert L.disco_eval_policies(ctx, pols, 64, 1, None, None) == 0, L.disco_last_error()
+room = np.zeros(64 * C.sizeof(api.PolicyStats) + 64, np.uint8)
+stats = (room.ctypes.data + 15) // 16 * 16 + {offset}
+fake.fake_memory(room.ctypes.data, room.nbytes, HOST, 0)
+assert L.disco_reduce_stats(ctx, C.c_void_p(stats), None) == 0, L.disco_last_error()
+assert (fake.fake_last_stats() == stats) == {offset % 8 == 0}
 """)
