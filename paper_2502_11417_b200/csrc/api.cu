@@ -141,6 +141,8 @@ struct disco_ctx {
     std::vector<uint64_t> F_n;         // requests per group behind F (the group's own count unless imported)
     bool fin_imported = false;         // fin_totals holds a caller's merged totals, not this trace's
     std::vector<uint64_t> fin_own;     // this trace's totals, to put back before the next evaluation
+    LargeLoad large;                   // working memory of a large trace's load
+    bool inv_there = false;            // `inv` has been written
     LoadZero* z = nullptr;
     uint32_t *cnt = nullptr, *tick_cnt = nullptr;
     uint2* windows = nullptr;
@@ -226,6 +228,8 @@ int check_profiles(const disco_trace_desc_t* d, std::vector<GroupConst>* out) {
 // How a load's inputs reach the ingestion kernel.
 enum Inputs { IN_DEVICE, IN_COPIED, IN_PLACE, IN_PACKED };
 
+bool large_load(uint32_t n, int G) { return n >= kLargeMinN && n <= kLargeMaxN && G <= kLargeMaxGroups; }
+
 cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool has_dp) {
     const size_t N = n ? n : 1, N4 = N + 3;
     const int G = c->G;
@@ -246,9 +250,23 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     } else if (in == IN_PACKED) {
         o_in[0] = lay.take(n > kPackInPlace ? packed_bytes(n) : 0);
     }
+    const bool large = large_load(n, G);
+    LargeLoad& lg = c->large;
+    std::memset(&lg, 0, sizeof lg);
+    if (large) {
+        lg.rec_share = rec_share(n); lg.tick_share = tick_share(n, (uint32_t)c->sms);
+        lg.n_rec = 2 * (n / lg.rec_share + G); lg.n_tick = 2 * (n / lg.tick_share + G);
+    }
+    const size_t o_parted = lay.take(large ? N * 16 : 0), o_rec_of = lay.take(large ? (size_t)G * (kMaxPrompt + 1) * 2 : 0);
+    const size_t o_tick_of = lay.take(large ? (size_t)G * kTickBins * 2 : 0), o_at = lay.take(large ? ((size_t)lg.n_rec + lg.n_tick + 4) * 4 : 0);
+    const size_t o_members = lay.take(large ? ((size_t)lg.n_rec + lg.n_tick) * 8 : 0);
     const cudaError_t e = c->trace_mem.reserve(lay.bytes);
     if (e) return e;
     char* base = (char*)c->trace_mem.p;
+    lg.parted = (uint4*)(base + o_parted);
+    lg.rec_bucket = (uint16_t*)(base + o_rec_of); lg.tick_bucket = (uint16_t*)(base + o_tick_of);
+    lg.rec_at = (uint32_t*)(base + o_at); lg.tick_at = lg.rec_at + lg.n_rec;
+    lg.rec_members = (uint2*)(base + o_members); lg.tick_members = lg.rec_members + lg.n_rec;
     c->req.p = base + o_req; c->sorted.p = base + o_sorted; c->binned.p = base + o_binned; c->inv.p = base + o_inv;
     c->zero.p = base + o_zero; c->len_end.p = base + o_ends; c->tick_start.p = base + o_starts; c->cum_mass.p = base + o_mass;
     c->grp_off.p = base + o_off; c->knots.p = base + o_knots; c->fin_totals.p = base + o_fin;
@@ -421,8 +439,11 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     }
     static const int32_t no_report[4] = {0, 0, 0, 2};               // what the host finds if the blocks lose each other
     std::memcpy(c->rb->err, no_report, sizeof no_report);
-    if ((e = run_load(a, c->sms, st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion kernel"));
-    g_launches += 1;
+    const bool large = large_load(n, c->G);
+    a.large = c->large;
+    c->inv_there = !large;
+    if ((e = large ? run_load_large(a, c->sms, st) : run_load(a, c->sms, st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion kernels"));
+    g_launches += large ? 6 : 1;
     // the few numbers the host needs (error word, group sizes, longest output, largest TTFT per group) are in rb
     HostReadback* rb = c->rb;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion"));
@@ -924,6 +945,11 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         }
         if (timed) CU(cudaEventRecord(c->ev[3], st));
         if (rows) {
+            if (G == 1 && !c->inv_there) {
+                CU(launch_inverse(tr, c->inv.as<uint32_t>(), st));
+                g_launches += 1;
+                c->inv_there = true;
+            }
             CU(launch_pairs_rows(tr, gc, dcc, prep, P, d_tab + lists[k].all, (uint32_t)lists[k].n_all, rec, po, k0, extras, st));
             g_launches += 1;
         }

@@ -284,6 +284,8 @@ cudaError_t launch_pairs_acc(const TraceDev& tr, const GroupConst* gc, const Cla
                              uint64_t* acc, uint64_t* hist_ttft, uint64_t* hist_tbt, uint64_t* work, uint32_t k0,
                              bool extras /* some policy routes at random or waits by Eq. 1-2 */,
                              bool wide /* some window W of the class spans several bins */, cudaStream_t st);
+// Fills tr.inv (a large trace's load leaves that to the evaluation that writes rows).
+cudaError_t launch_inverse(const TraceDev& tr, uint32_t* inv, cudaStream_t st);
 cudaError_t launch_pairs_rows(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
                               const uint32_t* pol_list, uint32_t n_list, TimelineRec rec, const disco_pair_out_t& out,
                               uint32_t k0, bool extras, cudaStream_t st);

@@ -14,52 +14,19 @@
 //      few low bits), each window by one block.  A bin of more than 8,192 ticks that spans at most 2^18 values is sorted by
 //      counting them; a trace that has a denser and wider one goes to the radix sort (radix.cu) instead.
 //
-// Bound: latency at 10^5 requests (one launch instead of eighteen), memory at 10^7: the columns are read twice (once when
-// they are in host memory: then the first pass leaves a copy), 20 bytes a request are written to scattered places, the
-// ticks are read and written once more.  16 M requests in six groups: 1,800 us by a chain of kernels, 850 now, over half
-// of it the scattered places (linear stores in their stead: 106 us for that pass instead of 470); a million: 70 us.  (The 64
-// registers that 1,024 threads leave spill 32 bytes.)
-#include "load.cuh"
-
+// Bound: latency at 10^5 requests (one launch instead of eighteen), scattered stores at 10^6: the columns are read twice (once
+// when they are in host memory: then the first pass leaves a copy), 20 bytes a request are written to scattered places, the ticks
+// are read and written once more.  A million requests: 58 us.  From 3.5 million on load_large.cu is the faster one.  (The 64
+// registers that 1,024 threads leave spill 64 bytes.)
 #include <algorithm>
 #include <cstdlib>
 #include <mutex>
 
-#include "pack.cuh"
-#include "scan.cuh"
+#include "ingest.cuh"
 
 namespace disco {
 
 namespace {
-
-constexpr int kThreads = 1024;
-constexpr int kLens = kMaxPrompt + 1;
-constexpr uint32_t FULL = 0xFFFFFFFFu;
-constexpr uint32_t kWindow = 4096;        // a window starts with the first bin behind every 4,096th tick of its group
-constexpr uint32_t kSortCap = 8192;       // ticks sorted at a time
-constexpr uint32_t kCounters = 16384;     // values counted at a time
-constexpr uint32_t kMaxRange = 1u << 18;  // values a dense bin may span
-constexpr uint32_t kMaxCount = 1u << 22;  // ticks a dense bin may hold
-constexpr int kPrivateGroups = 7;         // groups whose counters fit in shared memory (29 KB each)
-constexpr int kPrivateTickGroups = 16;    // the same, counters of tick bins alone
-static_assert(kMaxTicks + (uint64_t)kLoadBlocks * kThreads * 4 <= 1ull << 32, "a step of the loops over the ticks");
-
-enum Source { S_TRACE, S_TICKS, S_TTFT };
-enum Form { F_COLUMNS, F_STAGE, F_PACKED };   // a trace's columns; the same, with a copy left for the second pass; packed
-
-__device__ __forceinline__ uint32_t tick_bin_edge(int b) {     // smallest ticks of the bin (2^31 behind the last)
-    return b < 128 ? (uint32_t)b : (uint32_t)(128 + (b & 127)) << ((b >> 7) - 1);
-}
-
-struct SortSmem {
-    uint32_t a[kSortCap], b[kSortCap];                 // ticks of a window, twice; or kCounters counters
-    uint16_t wcnt[kThreads / 32][256];                 // keys of each digit per warp (radix sort)
-    uint32_t dig[256];
-    uint32_t wtot[32];
-    uint32_t lo, hi, n_list;
-    uint32_t bin[kTickBins];                           // of a window's bins: first place | count << 16; or the frequent values
-};
-static_assert(kCounters == 2 * kSortCap, "the counters lie over the two key arrays");
 
 // The waits between blocks are bounded.  Behind one that ran out, tables may hold what an earlier call left in them, and
 // places taken from those could lie anywhere: a block that gives up sets the flag that makes the host refuse the results
@@ -90,96 +57,6 @@ __device__ __forceinline__ bool grid_barrier(LoadZero* z, uint32_t times, uint32
         __threadfence();
     }
     return !__syncthreads_or(lost);
-}
-
-// Four neighbouring requests of the trace (or ticks of a sample) as the two passes see them.
-struct Item { uint32_t g, S, l, o; bool in; };
-
-// (LAST: read for the last time, so that the lines need not stay in L2)
-template <class T4, bool LAST, class T>
-__device__ __forceinline__ void load4(const T* p, uint32_t i0, uint32_t n, bool wide, T (&v)[4], T fill) {
-    if (wide && i0 + 4u <= n) {
-        const T4 x = LAST ? __ldcs(reinterpret_cast<const T4*>(p + i0)) : *reinterpret_cast<const T4*>(p + i0);
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-    } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = i0 + u < n ? p[i0 + u] : fill;
-    }
-}
-
-// Reads the items i0 .. i0 + 3, and in the first pass checks them.  wide: the columns are aligned for vector loads.
-// AGAIN: for counting; it will be read once more.
-template <int SRC, int FORM, bool CHECK, bool AGAIN = false>
-__device__ __forceinline__ void read_items(const LoadArgs& a, uint32_t i0, bool wide, const uint32_t* s_off, Item (&x)[4]) {
-    if (FORM == F_STAGE && !CHECK) {
-        uint32_t ln[4], S[4];
-        uint8_t g[4];
-        load4<uint4, !CHECK && !AGAIN>(a.st_ln, i0, a.n, true, ln, 0u);
-        load4<uint4, !CHECK && !AGAIN>(a.st_ticks, i0, a.n, true, S, 0u);
-        load4<uchar4, !CHECK && !AGAIN>(a.st_g, i0, a.n, true, g, (uint8_t)0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = Item{g[u], S[u], ln[u] & 0xFFFFu, ln[u] >> 16, i0 + u < a.n};
-        return;
-    }
-    if (SRC == S_TICKS) {
-        int32_t t[4];
-        load4<int4, !CHECK>(a.ticks, i0, a.n, wide, t, 0);
-        uint32_t g = 0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            x[u] = Item{0u, (uint32_t)t[u], 1u, 1u, i0 + u < a.n};
-            while ((int)g + 1 < a.G && i0 + u >= s_off[g + 1]) ++g;
-            x[u].g = g;
-            if (CHECK && t[u] < 0) {
-                if (atomicCAS(&a.z->err[0], 0, 3) == 0) a.z->err[1] = (int32_t)(i0 + u);
-                x[u].in = false;
-            }
-        }
-        return;
-    }
-    float t[4];
-    int32_t l[4] = {1, 1, 1, 1}, o[4] = {1, 1, 1, 1};
-    uint8_t sp[4] = {0, 0, 0, 0}, dp[4] = {0, 0, 0, 0};
-    constexpr bool kLast = !CHECK && !AGAIN;
-    if (FORM == F_PACKED) {
-        // (chunks are whole vectors, and a vector lies in one chunk; what lies behind item n is not used)
-        const char* c = a.packed + (size_t)(i0 / kPackChunk) * kPackBytes;
-        const uint32_t k = i0 % kPackChunk;
-        const uint4 ln = *reinterpret_cast<const uint4*>(c + (size_t)k * 4);
-        const float4 tt = *reinterpret_cast<const float4*>(c + (size_t)kPackChunk * 4 + (size_t)k * 4);
-        const uchar4 gg = *reinterpret_cast<const uchar4*>(c + (size_t)kPackChunk * 8 + k);
-        const uint32_t lns[4] = {ln.x, ln.y, ln.z, ln.w};
-        t[0] = tt.x; t[1] = tt.y; t[2] = tt.z; t[3] = tt.w;
-        dp[0] = gg.x; dp[1] = gg.y; dp[2] = gg.z; dp[3] = gg.w;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { l[u] = (int32_t)(lns[u] & 0xFFFFu); o[u] = (int32_t)(lns[u] >> 16); }
-    } else if (SRC == S_TRACE) {
-        load4<float4, kLast>(a.ttft, i0, a.n, wide, t, 1.0f);
-        load4<int4, kLast>(a.prompt, i0, a.n, wide, l, 1);
-        if (!AGAIN) load4<int4, kLast>(a.outlen, i0, a.n, wide, o, 1);
-        if (a.sp) load4<uchar4, kLast>(a.sp, i0, a.n, wide, sp, (uint8_t)0);
-        if (a.dp) load4<uchar4, kLast>(a.dp, i0, a.n, wide, dp, (uint8_t)0);
-    } else {
-        load4<float4, kLast>(a.ttft, i0, a.n, wide, t, 1.0f);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        bool in = i0 + u < a.n;
-        if (CHECK && in) {
-            int bad = 0;
-            if (l[u] < 1 || l[u] > kMaxPrompt) bad = 1;
-            else if (o[u] < 1 || o[u] > kMaxOutput) bad = 2;
-            else if (!(t[u] > 0.0f) || !(t[u] <= 2000.0f)) bad = 3;      // NaN fails both comparisons
-            else if (FORM == F_PACKED ? (int)dp[u] >= a.G : SRC == S_TRACE && (sp[u] >= a.ns || dp[u] >= a.nd)) bad = 4;
-            if (bad) {
-                if (atomicCAS(&a.z->err[0], 0, bad) == 0) a.z->err[1] = (int32_t)(i0 + u);
-                in = false;
-            }
-        }
-        // ticks = nearest integer (ties to even) of the fp64 product, as a host llrint would give
-        const uint32_t S = (uint32_t)__double2ll_rn(__dmul_rn((double)t[u], 1e6));
-        x[u] = Item{SRC == S_TRACE ? (uint32_t)sp[u] * a.nd + dp[u] : 0u, S, (uint32_t)l[u], (uint32_t)o[u], in};
-    }
 }
 
 // Waits (boundedly, as above) for a word that another block writes once; 0 if it does not come.
@@ -231,226 +108,6 @@ __device__ __forceinline__ void scan_share(const uint32_t* cnt, const Share& sh,
         carry += total;
         __syncthreads();
     }
-}
-
-// Cumulative input-token mass cum[L] = sum_{l<L} l cnt[l], L = 0 .. 4097.  All threads call.
-__device__ __forceinline__ void group_mass(const uint32_t* cnt, int64_t* cum, unsigned long long* wm) {
-    constexpr int kPer = 5;
-    const int k0 = (int)threadIdx.x * kPer;
-    uint32_t c[kPer];
-    unsigned long long m = 0, total;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) { c[k] = k0 + k < kLens ? __ldcg(&cnt[k0 + k]) : 0u; m += (unsigned long long)(k0 + k) * c[k]; }
-    unsigned long long run = block_inclusive_scan(m, wm, &total) - m;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) { if (k0 + k < kLens) cum[k0 + k] = (int64_t)run; run += (unsigned long long)(k0 + k) * c[k]; }
-    if (threadIdx.x == 0) cum[kLens] = (int64_t)total;
-    __syncthreads();
-}
-
-// Sorts the `count` <= kSortCap ticks of the bins [b0, b1] of a group from src into out: every bin has as many cells (or
-// twice as many) as ticks, evenly over its values, so that a cell holds a tick or so whatever the distribution; the ticks
-// are counted by cell, placed, and those that share a cell put in order by insertion.  Returns false, with nothing
-// written, if more than kCellCap different ticks may share a cell.
-constexpr uint32_t kCells = 8192, kCellCap = 64;
-
-__device__ __forceinline__ bool sort_window(SortSmem& sm, const uint32_t* src, uint32_t count, const uint32_t* bin_start,
-                                            const uint32_t* bin_count, int b0, int b1, int32_t* out) {
-    const int tid = threadIdx.x;
-    constexpr int kPer = kSortCap / kThreads, kCellsPer = kCells / kThreads;
-    uint32_t* cell = sm.b;                                             // counts, then starts
-    const uint32_t k0 = __ldcg(&bin_start[b0]), f = count <= kCells / 2 ? 1u : 0u, cells = count << f;
-    for (uint32_t i = tid; i < (cells + 7u) / 8u * 8u; i += kThreads) cell[i] = 0;
-    for (int b = b0 + tid; b <= b1; b += kThreads) {
-        const uint32_t c = __ldcg(&bin_count[b]);
-        sm.bin[b - b0] = (__ldcg(&bin_start[b]) - k0) | c << 16;       // (an empty bin's is not used)
-    }
-    if (tid == 0) sm.n_list = 0;
-    uint32_t key[kPer], at[kPer];                                      // at: cell | rank in it << 16
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const uint32_t i = k * kThreads + tid;
-        if (i < count) key[k] = __ldcg(&src[i]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        if ((uint32_t)k * kThreads + tid >= count) continue;
-        const int b = tick_bin(key[k]);
-        if (!DBG_OK(b - b0, b1 - b0 + 1, DBG_K_RADIX, DBG_BIN)) { at[k] = 0; continue; }
-        const uint32_t sc = sm.bin[b - b0], w = b < 128 ? 0u : (uint32_t)(b >> 7) - 1u, in = key[k] - tick_bin_edge(b);
-        const uint32_t sh = min(w, 16u);                               // (a bin spans 2^w values; 16 leading bits of the place in it)
-        uint32_t c = ((sc & 0xFFFFu) << f) + (((in >> (w - sh)) * ((sc >> 16) << f)) >> sh);
-        if (!DBG_OK(c, cells, DBG_K_RADIX, DBG_BIN)) c = 0;
-        at[k] = c | atomicAdd(&cell[c], 1u) << 16;
-    }
-    __syncthreads();
-    // the cells' starts; a thread's eight neighbouring cells (as vectors: single words would meet in four banks)
-    static_assert(kCellsPer == 8, "two vectors");
-    uint4* cell4 = reinterpret_cast<uint4*>(cell) + tid * 2;
-    uint4 u = make_uint4(0u, 0u, 0u, 0u), v = u;
-    if (tid * 8u < cells) { u = cell4[0]; v = cell4[1]; }              // (those beyond `cells` are zero)
-    const uint32_t sum = u.x + u.y + u.z + u.w + v.x + v.y + v.z + v.w;
-    uint32_t run = block_inclusive_scan(sum, sm.wtot, (uint32_t*)nullptr) - sum;
-    if (tid * 8u < cells) {
-        uint32_t t;
-        t = u.x; u.x = run; run += t; t = u.y; u.y = run; run += t; t = u.z; u.z = run; run += t; t = u.w; u.w = run; run += t;
-        t = v.x; v.x = run; run += t; t = v.y; v.y = run; run += t; t = v.z; v.z = run; run += t; t = v.w; v.w = run; run += t;
-        cell4[0] = u; cell4[1] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        if ((uint32_t)k * kThreads + tid >= count) continue;
-        const uint32_t p = cell[at[k] & 0xFFFFu] + (at[k] >> 16);
-        if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) sm.a[p] = key[k];
-    }
-    __syncthreads();
-    // a thread every 1,024th cell
-    for (uint32_t x = tid; x < cells; x += kThreads) {
-        const uint32_t from = cell[x], to = x + 1u < cells ? cell[x + 1u] : count;
-        if (to - from < 2u) continue;
-        if (to - from > 8u) {
-            // a cell of a bin with at least as many cells as values holds one value
-            const int b = tick_bin(sm.a[from]);
-            if (b < 128 || 1u << ((b >> 7) - 1) <= (sm.bin[b - b0] >> 16) << f) continue;
-            if (to - from > kCellCap) { sm.n_list = 1; continue; }
-        }
-        for (uint32_t y = from + 1u; y < to; ++y) {
-            const uint32_t v = sm.a[y];
-            uint32_t p = y;
-            while (p > from && sm.a[p - 1u] > v) { sm.a[p] = sm.a[p - 1u]; --p; }
-            sm.a[p] = v;
-        }
-    }
-    __syncthreads();
-    if (sm.n_list) return false;
-    for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)sm.a[i];
-    return true;
-}
-
-// The same whatever the ticks (all of them in [lo, lo + 2^bits)): stable counting passes of at most eight bits, a warp's 256
-// keys at a time with the ranks from ballots.  Four to six times slower.
-__device__ __noinline__ void sort_window_radix(SortSmem& sm, const uint32_t* src, uint32_t count, uint32_t lo, int bits, int32_t* out) {
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    if (bits == 0) {
-        for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)lo;
-        return;
-    }
-    uint32_t *from = sm.a, *to = sm.b;
-    for (uint32_t i = tid; i < count; i += kThreads) from[i] = __ldcg(&src[i]) - lo;
-    const int passes = (bits + 7) / 8, d_bits = (bits + passes - 1) / passes, digits = 1 << d_bits;
-    const int rounds = (int)((min(count, 256u) + 31u) / 32u), warps = (int)((count + 255u) / 256u);
-    for (int p = 0; p < passes; ++p) {
-        const int shift = p * d_bits;
-        for (int i = tid; i < warps * 256; i += kThreads) (&sm.wcnt[0][0])[i] = 0;
-        __syncthreads();
-        uint32_t key[8], place[8];                    // place: digit | rank among the warp's equal digits so far << 8
-        if (w < warps) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (j >= rounds) break;
-                const uint32_t i = w * 256u + j * 32u + lane;
-                const bool live = i < count;
-                key[j] = live ? from[i] : 0u;
-                const uint32_t d = (key[j] >> shift) & (uint32_t)(digits - 1);
-                uint32_t peers = __ballot_sync(FULL, live);
-                for (int b = 0; b < d_bits; ++b) {
-                    const uint32_t bal = __ballot_sync(FULL, (d >> b) & 1u);
-                    peers &= ((d >> b) & 1u) ? bal : ~bal;
-                }
-                const uint32_t below = __popc(peers & ((1u << lane) - 1u));
-                uint32_t before = 0;
-                if (live) before = sm.wcnt[w][d];
-                __syncwarp();
-                if (live && below == 0) sm.wcnt[w][d] = (uint16_t)(before + __popc(peers));
-                __syncwarp();
-                place[j] = d | (before + below) << 8;
-            }
-        }
-        __syncthreads();
-        // where each digit starts, and each warp's keys of it
-        uint32_t total = 0;
-        if (tid < digits) for (int k = 0; k < warps; ++k) { const uint32_t c = sm.wcnt[k][tid]; sm.wcnt[k][tid] = (uint16_t)total; total += c; }
-        const uint32_t incl = block_inclusive_scan(tid < digits ? total : 0u, sm.wtot, (uint32_t*)nullptr);
-        if (tid < digits) sm.dig[tid] = incl - total;
-        __syncthreads();
-        if (w < warps) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (j >= rounds) break;
-                const uint32_t i = w * 256u + j * 32u + lane;
-                if (i < count) {
-                    const uint32_t d = place[j] & 255u, at = sm.dig[d] + sm.wcnt[w][d] + (place[j] >> 8);
-                    if (DBG_OK(at, count, DBG_K_RADIX, DBG_ELEMENT)) to[at] = key[j];
-                }
-            }
-        }
-        __syncthreads();
-        uint32_t* t = from; from = to; to = t;
-    }
-    for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)(from[i] + lo);
-}
-
-// Sorts a dense bin by counting its values.  Returns false where that would take too long.
-__device__ __forceinline__ bool sort_dense(SortSmem& sm, const uint32_t* src, uint32_t count, int32_t* out) {
-    const int tid = threadIdx.x, lane = tid & 31;
-    if (tid == 0) { sm.lo = 0xFFFFFFFFu; sm.hi = 0u; }
-    __syncthreads();
-    uint32_t mn = 0xFFFFFFFFu, mx = 0u;
-    for (uint32_t i = tid; i < count; i += kThreads) { const uint32_t t = __ldcg(&src[i]); mn = min(mn, t); mx = max(mx, t); }
-    mn = __reduce_min_sync(FULL, mn); mx = __reduce_max_sync(FULL, mx);
-    if (lane == 0) { atomicMin(&sm.lo, mn); atomicMax(&sm.hi, mx); }
-    __syncthreads();
-    const uint32_t lo = sm.lo, range = sm.hi - lo + 1u;
-    if (range == 1u) {
-        for (uint32_t i = tid; i < count; i += kThreads) out[i] = (int32_t)lo;
-        return true;
-    }
-    if (range > kMaxRange || count > kMaxCount) return false;
-    uint32_t* at = sm.a;                                              // kCounters of them: counts, then places
-    uint32_t* often = sm.bin;                                         // values that the whole block writes: value, place, count
-    constexpr uint32_t kOften = 4096;
-    static_assert(3 * (kMaxCount / kOften) <= kTickBins, "room for the frequent values");
-    uint32_t done = 0;
-    for (uint32_t r0 = 0; r0 < range; r0 += kCounters) {
-        // a thread's neighbouring values, as few as the range needs
-        const uint32_t here = min(range - r0, kCounters), per = (here + kThreads - 1) / kThreads;
-        for (uint32_t i = tid; i < per * kThreads; i += kThreads) at[i] = 0;
-        if (tid == 0) sm.n_list = 0;
-        __syncthreads();
-#pragma unroll 4
-        for (uint32_t i = tid; i < count; i += kThreads) {
-            const uint32_t v = __ldcg(&src[i]) - lo - r0;
-            if (v < here) atomicAdd(&at[v], 1u);
-        }
-        __syncthreads();
-        uint32_t sum = 0, total;
-        for (uint32_t k = 0; k < per; ++k) sum += at[tid * per + k];
-        uint32_t run = done + block_inclusive_scan(sum, sm.wtot, &total) - sum;
-        for (uint32_t k = 0; k < per; ++k) {
-            const uint32_t v = tid * per + k, c = at[v];
-            at[v] = run;
-            if (c > kOften) {
-                const uint32_t e = atomicAdd(&sm.n_list, 1u);
-                if (DBG_OK(e, kMaxCount / kOften, DBG_K_RADIX, DBG_SLOT)) { often[3 * e] = v; often[3 * e + 1] = run; often[3 * e + 2] = c; at[v] = 0xFFFFFFFFu; }
-            }
-            run += c;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (uint32_t i = tid; i < count; i += kThreads) {
-            const uint32_t t = __ldcg(&src[i]), v = t - lo - r0;
-            if (v >= here || *(volatile uint32_t*)&at[v] == 0xFFFFFFFFu) continue;
-            const uint32_t p = atomicAdd(&at[v], 1u);                 // equal ticks in any order
-            if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) out[p] = (int32_t)t;
-        }
-        for (uint32_t e = 0; e < sm.n_list; ++e)
-            for (uint32_t j = tid; j < often[3 * e + 2]; j += kThreads) out[often[3 * e + 1] + j] = (int32_t)(lo + r0 + often[3 * e]);
-        done += total;
-        __syncthreads();
-    }
-    return true;
 }
 
 template <int SRC, bool PRIV, int FORM>
@@ -537,11 +194,7 @@ k_load(const __grid_constant__ LoadArgs a) {
                 }
             }
         }
-        if (FORM == F_STAGE) {                                                   // (the staging arrays hold whole vectors)
-            *reinterpret_cast<uint4*>(a.st_ticks + i0) = make_uint4(x[0].S, x[1].S, x[2].S, x[3].S);
-            *reinterpret_cast<uint4*>(a.st_ln + i0) = make_uint4(x[0].l | x[0].o << 16, x[1].l | x[1].o << 16, x[2].l | x[2].o << 16, x[3].l | x[3].o << 16);
-            *reinterpret_cast<uchar4*>(a.st_g + i0) = make_uchar4((uint8_t)x[0].g, (uint8_t)x[1].g, (uint8_t)x[2].g, (uint8_t)x[3].g);
-        }
+        if (FORM == F_STAGE) stage_items(a, i0, x);
     }
     if (kTrace) {
         longest = __reduce_max_sync(FULL, longest);
@@ -755,7 +408,7 @@ k_load(const __grid_constant__ LoadArgs a) {
         const uint32_t k0 = s_win[0][j & 31u], k2 = s_win[1][j & 31u], k1 = s_win[2][j & 31u];
         if (k0 >= k1) continue;                                        // (inside a large bin)
         const int g = (int)s_win[3][j & 31u] / kTickBins, b0 = (int)s_win[3][j & 31u] - g * kTickBins, b1 = (int)s_win[4][j & 31u] - g * kTickBins;
-        const uint32_t first = s_off[g], N = s_off[g + 1] - first, lo = tick_bin_edge(b0);
+        const uint32_t lo = tick_bin_edge(b0);
         auto bits_of = [](uint32_t range) { return range <= 1u ? 0 : 32 - __clz((int)(range - 1u)); };
         const uint32_t *starts = a.tick_start + (size_t)g * kTickBins, *counts = a.tick_cnt + (size_t)g * kTickBins;
         // up to kSortCap ticks; otherwise the last bin is a large one: the others first
@@ -768,20 +421,13 @@ k_load(const __grid_constant__ LoadArgs a) {
         }
         if (large) {
             __syncthreads();
-            if (!sort_dense(sm, a.binned + k2, k1 - k2, a.sorted + k2) && tid == 0) atomicMax(&z->err[3], 1);
+            const uint32_t edge = tick_bin_edge(b1);
+            if (!sort_dense<kThreads, kCounters>(sm.a, sm.wtot, sm.range, a.binned + k2, k1 - k2, edge, tick_bin_edge(b1 + 1) - edge, a.sorted + k2) &&
+                tid == 0)
+                atomicMax(&z->err[3], 1);
         }
         __syncthreads();
-        if (kTrace) {
-            // the knots K_g[k] = sorted_g[(k (N_g - 1)) / 256] that lie in the window
-            for (int k = tid; k < kNKnots; k += kThreads) {
-                const uint32_t at = first + (uint32_t)(((uint64_t)k * (N - 1)) / 256u);
-                if (at >= k0 && at < k1) {
-                    const int32_t v = __ldcg(&a.sorted[at]);
-                    a.knots[g * kNKnots + k] = v;
-                    if (k == kNKnots - 1) a.readback->knot_max[g] = v;
-                }
-            }
-        }
+        if (kTrace) write_knots<kThreads>(a, g, k0, k1, s_off[g], s_off[g + 1] - s_off[g]);
     }
     if (kTrace) {
         for (int g = 0; g < G; ++g)                                    // (the last blocks have the fewest windows)

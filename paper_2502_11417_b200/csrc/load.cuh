@@ -30,6 +30,7 @@ constexpr uint64_t kMaxTicks = (1ull << 32) - (1ull << 20);
 struct LoadZero {
     unsigned long long part[2][kLoadBlocks];      // sums over the blocks' shares of the counters: sum << 1 | 1
     uint64_t grp_sum_n[kMaxGroups];       // output tokens per group
+    uint32_t grp_n[kMaxGroups];           // requests per group (load_large.cu)
     uint32_t max_n;                       // longest output
     uint32_t barrier, done, pad;
     int32_t err[4];                       // code, request index, window flag, sort flag (1: some bin needs the fallback, 2: a
@@ -37,6 +38,27 @@ struct LoadZero {
 };
 
 __host__ __device__ constexpr uint32_t sort_windows(uint32_t n, int G) { return n / 4096u + (uint32_t)G; }
+
+// Large traces are placed in two steps, by way of buckets (load_large.cu).
+constexpr uint32_t kLargeMaxN = 1u << 24;     // (beyond, the tables of buckets no longer fit in a block's shared memory)
+constexpr uint32_t kLargeMinN = 3500000;    // (where it becomes the faster one: see load_large.cu)
+constexpr int kLargeMaxGroups = 7;            // groups whose counters fit there
+constexpr uint32_t kTickShare = 8192;         // ticks to a bucket, at most
+// Records to a bucket: 2,048, or as many as leave 1,024 buckets.  Ticks: so many that the multiprocessors sort equally many buckets.
+inline uint32_t rec_share(uint32_t n) { return n / 1024u + 1u > 2048u ? n / 1024u + 1u : 2048u; }
+inline uint32_t tick_share(uint32_t n, uint32_t sms) {
+    const uint32_t most = kTickShare - 192u, blocks = 2u * sms, each = (n + blocks * most - 1u) / (blocks * most);
+    const uint32_t share = (n + blocks * each - 1u) / (blocks * each) + 64u;                        // (the groups' last buckets are partly filled)
+    return share < 2048u ? 2048u : share;
+}
+constexpr uint32_t kRecBuckets = 2 * (1024 + kLargeMaxGroups), kTickBuckets = 2 * (kLargeMaxN / 8000 + 512 + kLargeMaxGroups);
+struct LargeLoad {
+    uint4* parted;                        // [n] records bucket by bucket
+    uint32_t rec_share, tick_share, n_rec, n_tick;    // requests or ticks to a bucket, numbers of buckets
+    uint16_t *rec_bucket, *tick_bucket;   // [G][4097], [G][kTickBins]
+    uint32_t *rec_at, *tick_at;           // cursors, [n_rec] and [n_tick]
+    uint2 *rec_members, *tick_members;    // first and last length or bin, counted through the groups (first > last: none)
+};
 
 struct LoadArgs {
     uint32_t n;
@@ -74,6 +96,7 @@ struct LoadArgs {
     uint32_t* grp_off;                    // [G + 1]
     int32_t* knots;                       // [G][257]
     uint64_t* fin_totals;                 // [2G]: output tokens per group, then requests per group
+    LargeLoad large;
     LoadReadback* readback;               // its err holds 0, 0, 0, 2 (no report) before the launch
 #ifdef DISCO_DEBUG
     uint32_t absent;                      // the wait that expects one arrival more than comes (from 1; 4: of the other blocks' sums)
@@ -81,6 +104,8 @@ struct LoadArgs {
 };
 
 cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st);          // one kernel, after a memset
+// The same for kLargeMinN to kLargeMaxN requests in at most kLargeMaxGroups groups: six kernels, after a memset.
+cudaError_t run_load_large(const LoadArgs& a, int sms, cudaStream_t st);
 cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st);    // ticks, off, G, n -> sorted
 cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st);     // ttft, n (one group) -> sorted
 

@@ -411,6 +411,15 @@ size_t acc_smem_bytes(int PL) {
     return sizeof(uint32_t) * acc_stage_offset_words(PL) + (size_t)kAccWarps * kStageReq * 2 * kStageVec * sizeof(uint4);
 }
 
+__global__ void __launch_bounds__(256)
+k_inverse(TraceDev tr, uint32_t* __restrict__ inv) {
+    grid_dependency_wait();
+    const uint32_t k = blockIdx.x * 256u + threadIdx.x;
+    if (k >= tr.n) return;
+    const uint32_t orig = tr.req[k].z;
+    if (DBG_OK(orig, tr.n, DBG_K_PAIRS_ROWS, DBG_REQUEST)) inv[orig] = k;
+}
+
 // ------------------------------------------------------------------------------------------------------
 // Per-pair arrays: lane = request, up to 16 policies per block row.
 //
@@ -595,6 +604,10 @@ cudaError_t launch_pairs_acc(const TraceDev& tr, const GroupConst* gc, const Cla
     return launch_after(acc_kernel, dim3(n_chunks * n_tiles), kAccThreads, acc_smem_bytes(PL), st, tr, gc, cc, prep, P,
                         pol_list, n_list, PL, chunks, n_tiles, list, list_count, rec, k0, (unsigned long long*)acc,
                         (unsigned long long*)hist_ttft, (unsigned long long*)hist_tbt, (unsigned long long*)work);
+}
+
+cudaError_t launch_inverse(const TraceDev& tr, uint32_t* inv, cudaStream_t st) {
+    return launch_after(k_inverse, (tr.n + 255) / 256, 256, 0, st, tr, inv);
 }
 
 cudaError_t launch_pairs_rows(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,

@@ -164,3 +164,55 @@ def test_windows_under_several_overheads(n, overheads, dearer):
     grid = [(b, t) for b in (0.0, 0.01, 0.03, 0.4, 0.8) for t in thetas]
     for how in (dict(flags=synth.FLAG_MIGRATION), dict(r_c=25.0, t_m_s=0.2), dict(r_c=30.0, t_m_s=0.3), dict(t_m_s=0.4)):
         full_parity(w, [synth.policy(b, mig_threshold=t, **how) for b, t in grid], select=False, tag=f"{n} x {overheads} {how}")
+
+
+@pytest.mark.parametrize("n,shape,kind,where", [(3_499_999, (1, 1), "spread", "device"), (3_500_000, (1, 1), "spread", "device"),
+                                                (3_500_001, (1, 1), "one", "device"), (3_508_193, (3, 2), "spread", "pinned"),
+                                                (3_600_013, (1, 7), "ties", "pageable"), (3_600_013, (2, 2), "dense", "unaligned"),
+                                                (4_000_003, (1, 2), "wide", "device"), (3_600_013, (2, 4), "spread", "device")])
+def test_large_traces_are_placed_by_way_of_buckets(n, shape, kind, where):
+    # tables and statistics of traces from 3.5 M requests in up to seven groups on, and on the other side of both limits: full
+    # and partly filled tiles and buckets, lengths and bins that take a bucket to themselves, samples left to the radix sort
+    import torch
+    from oracle import Oracle
+    from paper_2502_11417_b200 import DiscoError, Trace
+    from parity import check_stats
+    rng = np.random.default_rng(n)
+    w = synth.tiny_workload(105, n, n_servers=shape[0], n_devices=shape[1], max_prompt=4096, max_out=6)
+    if kind == "one":                              # one prompt length, one TTFT
+        w.prompt_len[:] = 77
+        w.server_ttft_s[:] = 0.25
+    elif kind != "spread":
+        w.server_ttft_s = np.clip(_sample(kind, n, rng), 1e-6, 2000.0).astype(np.float32)
+        w.prompt_len[rng.random(n) < 0.3] = 900    # (more than a bucket's share)
+    cols = [w.prompt_len, w.output_len, w.server_ttft_s, w.server_profile, w.device_profile]
+    if where == "pinned":
+        cols = [torch.from_numpy(c).pin_memory() for c in cols]
+    elif where == "device":
+        cols = [torch.from_numpy(c).cuda() for c in cols]
+    elif where == "unaligned":
+        cols = [torch.cat([torch.from_numpy(c[:1]), torch.from_numpy(c)]).cuda()[1:] for c in cols]
+    tr = Trace()
+    with pytest.raises(DiscoError) as ei:
+        bad = w.output_len.copy()
+        bad[n - 2] = 0
+        tr.load_trace(w.prompt_len, bad, *[np.asarray(c) for c in (w.server_ttft_s, w.server_profile, w.device_profile)], w.servers, w.devices)
+    assert f"at request {n - 2}" in str(ei.value)
+    tr.load_trace(*cols, w.servers, w.devices)
+    g_of = w.server_profile.astype(np.int64) * shape[1] + w.device_profile
+    ticks = np.rint(w.server_ttft_s.astype(np.float64) * 1e6).astype(np.int64)
+    for g in range(shape[0] * shape[1]):
+        cnt, knots, srt = tr.group_tables(g)
+        want = np.sort(ticks[g_of == g])
+        assert (srt == want).all() and (cnt == np.bincount(w.prompt_len[g_of == g], minlength=4097)).all()
+        assert (knots == want[np.arange(257, dtype=np.int64) * (len(want) - 1) // 256]).all()
+    pols = [synth.policy(0.4)]
+    if kind in ("spread", "one") and shape[0] * shape[1] in (1, 6):
+        orc = Oracle.from_workload(w)
+        out = tr.alloc_pair_outputs(1, ["ttft_s", "tok_server"])       # (rows: the requests' places are looked up)
+        tr.eval_policies(pols, w.seed, out)
+        stats, pairs = orc.eval(pols, w.seed, pairs=True)
+        check_stats(tr.reduce_stats(), stats, tr.histograms, f"{n}")
+        assert (out["tok_server"].cpu().numpy() == pairs["tok_server"]).all()
+        assert np.allclose(out["ttft_s"].cpu().numpy(), pairs["ttft_s"], rtol=1e-6)
+    tr.close()
