@@ -234,7 +234,7 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     const size_t N = n ? n : 1, N4 = N + 3;
     const int G = c->G;
     Layout lay;
-    const size_t o_req = lay.take(N * 16), o_sorted = lay.take(N * 4), o_binned = lay.take(N * 4), o_inv = lay.take(G == 1 ? N * 4 : 0);
+    const size_t o_req = lay.take(N * 16), o_sorted = lay.take(N * 4), o_binned = lay.take(N * 4), o_inv = lay.take(N * 4);
     // one block for everything a load clears: the flags and sums, the two histograms, the windows of the sort
     const size_t tick_bytes = (size_t)G * kTickBins * 4, cnt_bytes = ((size_t)G * (kMaxPrompt + 1) * 4 + 15) / 16 * 16;
     c->zero_bytes = sizeof(LoadZero) + tick_bytes + cnt_bytes + (size_t)sort_windows(n, G) * 8;
@@ -422,7 +422,7 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     a.z = c->z; a.zero_bytes = c->zero_bytes; a.cnt = c->cnt; a.tick_cnt = c->tick_cnt;
     a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)c->G * kTickBins;
     a.binned = c->binned.as<uint32_t>();
-    a.req = c->req.as<uint4>(); a.inv = c->G == 1 ? c->inv.as<uint32_t>() : nullptr; a.sorted = c->sorted.as<int32_t>();
+    a.req = c->req.as<uint4>(); a.inv = c->inv.as<uint32_t>(); a.sorted = c->sorted.as<int32_t>();
     a.len_end = c->len_end.as<uint32_t>(); a.cum_mass = c->cum_mass.as<int64_t>(); a.grp_off = c->grp_off.as<uint32_t>();
     a.knots = c->knots.as<int32_t>(); a.fin_totals = c->fin_totals.as<uint64_t>();
     a.windows = c->windows;
@@ -945,7 +945,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         }
         if (timed) CU(cudaEventRecord(c->ev[3], st));
         if (rows) {
-            if (G == 1 && !c->inv_there) {
+            if (!c->inv_there) {
                 CU(launch_inverse(tr, c->inv.as<uint32_t>(), st));
                 g_launches += 1;
                 c->inv_there = true;

@@ -342,7 +342,7 @@ k_load(const __grid_constant__ LoadArgs a) {
                 if (DBG_OK(tp[u], a.n, DBG_K_GATHER, DBG_ELEMENT)) a.binned[tp[u]] = y.S;
                 if (kTrace && DBG_OK(at[u], a.n, DBG_K_GATHER, DBG_REQUEST)) a.req[at[u]] = make_uint4(y.S, y.l | y.o << 16, i0 + u, 0u);
             }
-            if (kTrace && a.inv) {
+            if (kTrace) {
                 if (i0 + 4u <= a.n) *reinterpret_cast<uint4*>(a.inv + i0) = make_uint4(at[0], at[1], at[2], at[3]);
                 else for (uint32_t u = 0; i0 + u < a.n; ++u) a.inv[i0 + u] = at[u];
             }

@@ -89,7 +89,7 @@ struct LoadArgs {
     uint32_t* binned;                     // [n] ticks bin by bin
     // outputs
     uint4* req;                           // [n] internal order (by group, then by prompt length): see TraceDev
-    uint32_t* inv;                        // [n] place of each of the caller's requests (one group), or null
+    uint32_t* inv;                        // [n] place of each of the caller's requests
     int32_t* sorted;                      // [n] ticks ascending within each group
     uint32_t* len_end;                    // [G][4097]
     int64_t* cum_mass;                    // [G][4098]

@@ -423,11 +423,16 @@ k_inverse(TraceDev tr, uint32_t* __restrict__ inv) {
 // ------------------------------------------------------------------------------------------------------
 // Per-pair arrays: lane = request, up to 16 policies per block row.
 //
+// A thread takes a request in the caller's order, so that a store instruction writes 32 consecutive requests of one policy row;
+// what is read of it lies in the internal order, once per request.  What dispatch needs of a policy depends on the group: the
+// block keeps it for all groups and its policies.  (With several groups a thread per request in the internal order wrote
+// scattered words: 100,000 requests in six groups under 64 policies 448 us, now 42;
+// 1.5 million under 4 1,433, now 72.)
+//
 // What a pair writes besides its TTFT depends on the request and on which of the six outcomes it ends in.
 // Each thread therefore prices its request once per outcome (Eq. 8, token split, TBT mean and maximum of
 // the stream that applies) into a row of shared memory that only it reads; a pair then costs the decision,
-// one 16-byte row load and the nine stores.  A store instruction writes 32 consecutive requests of one
-// policy row.
+// one 16-byte row load and the nine stores.
 // ------------------------------------------------------------------------------------------------------
 constexpr int kRowThreads = 256;
 constexpr int kRowPols = 16;
@@ -436,19 +441,17 @@ constexpr int kRowVec = 7;              // uint4 per request: six outcome rows a
 // What the dispatch of one (group, policy) needs, with the mode tests folded into the thresholds: Algorithm 3
 // has no waits (l_star beyond every length), Algorithm 2 no device-only prompts (l_th = 0, as the preparation
 // kernel leaves it), and a policy or group without migration never passes the trigger (theta = +inf).
-struct __align__(8) RowPol {
+struct RowPol {
     int32_t l_th, l_star;
     uint32_t w_star, w_tail;
     float theta;
-    uint32_t pol;
 };
 
-__device__ __forceinline__ RowPol row_pol(const Prep& pr, int candidate, uint32_t p) {
+__device__ __forceinline__ RowPol row_pol(const Prep& pr, int candidate) {
     RowPol r;
     r.l_th = pr.l_th; r.l_star = pr.device_constrained ? pr.l_star : 0x7FFFFFFF;
     r.w_star = (uint32_t)pr.w_star; r.w_tail = (uint32_t)pr.w_tail;
     r.theta = (pr.mig_on && candidate != 0) ? pr.theta : __int_as_float(0x7F800000);
-    r.pol = p;
     return r;
 }
 
@@ -460,38 +463,32 @@ k_pairs_rows(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* 
              const uint32_t* __restrict__ pol_list, uint32_t n_list, TimelineRec rec, uint32_t k0,
              disco_pair_out_t out) {
     using idx_t = typename std::conditional<IDX32, uint32_t, size_t>::type;
-    __shared__ Prep s_prep[EXT ? kRowPols : 1];
-    __shared__ RowPol s_rp[kRowPols];
+    using Rule = typename std::conditional<EXT, Prep, RowPol>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Rule* s_rule = (Rule*)smem_raw;                        // [groups][kRowPols]
+    __shared__ uint32_t s_pol[kRowPols], s_end[kMaxGroups];
     __shared__ uint4 s_rows[kRowThreads * kRowVec];
     grid_dependency_wait();
     const uint32_t first = blockIdx.y * kRowPols;
-    const int npol = (int)min((uint32_t)kRowPols, n_list - first);
-    // the block's requests are consecutive in the internal order; most blocks lie inside one group
-    const uint32_t k_lo = blockIdx.x * kRowThreads, k_hi = min(tr.n, k_lo + kRowThreads) - 1;
-    int g_lo = 0, g_hi = 0;
-    while (g_lo + 1 < tr.n_groups && k_lo >= tr.grp_off[g_lo + 1]) ++g_lo;
-    g_hi = g_lo;
-    while (g_hi + 1 < tr.n_groups && k_hi >= tr.grp_off[g_hi + 1]) ++g_hi;
-    const bool one_group = g_lo == g_hi;
-    if ((int)threadIdx.x < npol) {
-        const uint32_t p = pol_list[first + threadIdx.x];
-        const Prep pr = prep[(size_t)g_lo * P + p];
-        if (EXT) s_prep[threadIdx.x] = pr;
-        s_rp[threadIdx.x] = row_pol(pr, gcs[g_lo].candidate, p);
+    const int npol = (int)min((uint32_t)kRowPols, n_list - first), G = tr.n_groups;
+    if ((int)threadIdx.x < npol) s_pol[threadIdx.x] = pol_list[first + threadIdx.x];
+    for (int g = threadIdx.x; g < G; g += kRowThreads) s_end[g] = tr.grp_off[g + 1];
+    for (int i = threadIdx.x; i < G * kRowPols; i += kRowThreads) {
+        const int g = i / kRowPols, pi = i % kRowPols;
+        if (pi >= npol) continue;
+        const Prep pr = prep[(size_t)g * P + pol_list[first + pi]];
+        if constexpr (EXT) s_rule[i] = pr; else s_rule[i] = row_pol(pr, gcs[g].candidate);
     }
     __syncthreads();
-    uint32_t k = k_lo + threadIdx.x;
+    uint32_t k = blockIdx.x * kRowThreads + threadIdx.x;
     if (k >= tr.n) return;
-    // one group: a thread per request in the caller's order, so that the rows are written side by side (the reads
-    // are scattered instead, once per request); several groups: the block's policies depend on the group, a thread
-    // per request in the internal order
-    if (tr.n_groups == 1) k = tr.inv[k];
+    k = tr.inv[k];
     if (!DBG_OK(k, tr.n, DBG_K_PAIRS_ROWS, DBG_REQUEST)) return;
     const uint4 rq = tr.req[k];
     const uint2 hand = rec.hand[k];
     const uint32_t orig = rq.z;
-    int g = g_lo;
-    while (g < g_hi && k >= tr.grp_off[g + 1]) ++g;
+    int g = 0;
+    while (g + 1 < G && k >= s_end[g]) ++g;
     const GroupConst& gc = gcs[g];
     const int candidate = gc.candidate;
     const bool dev_migrates = candidate == 2;
@@ -553,32 +550,26 @@ k_pairs_rows(TraceDev tr, const GroupConst* __restrict__ gcs, const ClassConst* 
         if (out.delayed) out.delayed[at] = (uint16_t)(migr ? dly : 0u);
         if (out.decision) out.decision[at] = (uint8_t)(dev_only ? DISCO_DEVICE_ONLY : (started ? DISCO_RACE : DISCO_SERVER_ONLY));
     };
-    auto pair = [&](const RowPol& rp, const Prep* full) {
-        const idx_t at = (idx_t)rp.pol * N + (idx_t)orig;
-        if (!DBG_OK(rp.pol, P, DBG_K_PAIRS_ROWS, DBG_POLICY) || !DBG_OK(orig, tr.n, DBG_K_PAIRS_ROWS, DBG_REQUEST)) return;
-        if (EXT) {
-            const PairOut o = decide<true>(q, *full, Td, candidate);
-            emit(at, o.dev_only, o.started, o.dev_wins, o.migr, o.ttft);
-            return;
-        }
-        // ---- dispatch (Algorithm 2's wait map / Algorithm 3's threshold) and the race
-        const bool dev_only = (int32_t)q.l < rp.l_th;
-        const uint32_t w = (int32_t)q.l < rp.l_star ? 0u : ((int32_t)q.l == rp.l_star ? rp.w_star : rp.w_tail);
-        const bool started = dev_only || q.S > w;               // the device starts after the wait
-        const uint32_t wTd = w + Td;
-        const bool dev_wins = dev_only || (started && q.S > wTd);   // a tie goes to the server
-        const uint32_t ttft = dev_only ? Td : min(q.S, wTd);
-        const bool migr = started && !dev_only && dev_wins == dev_migrates && saving_m > rp.theta;
-        emit(at, dev_only, started, dev_wins, migr, ttft);
-    };
-    if (one_group) {
+    const Rule* rules = s_rule + g * kRowPols;
 #pragma unroll 4
-        for (int pi = 0; pi < npol; ++pi) pair(s_rp[pi], EXT ? &s_prep[pi] : nullptr);
-    } else {
-        for (int pi = 0; pi < npol; ++pi) {
-            const Prep pr = prep[(size_t)g * P + s_rp[pi].pol];
-            const RowPol rp = row_pol(pr, candidate, s_rp[pi].pol);
-            pair(rp, &pr);
+    for (int pi = 0; pi < npol; ++pi) {
+        const uint32_t p = s_pol[pi];
+        const idx_t at = (idx_t)p * N + (idx_t)orig;
+        if (!DBG_OK(p, P, DBG_K_PAIRS_ROWS, DBG_POLICY) || !DBG_OK(orig, tr.n, DBG_K_PAIRS_ROWS, DBG_REQUEST)) continue;
+        if constexpr (EXT) {
+            const PairOut o = decide<true>(q, rules[pi], Td, candidate);
+            emit(at, o.dev_only, o.started, o.dev_wins, o.migr, o.ttft);
+        } else {
+            // ---- dispatch (Algorithm 2's wait map / Algorithm 3's threshold) and the race
+            const RowPol rp = rules[pi];
+            const bool dev_only = (int32_t)q.l < rp.l_th;
+            const uint32_t w = (int32_t)q.l < rp.l_star ? 0u : ((int32_t)q.l == rp.l_star ? rp.w_star : rp.w_tail);
+            const bool started = dev_only || q.S > w;               // the device starts after the wait
+            const uint32_t wTd = w + Td;
+            const bool dev_wins = dev_only || (started && q.S > wTd);   // a tie goes to the server
+            const uint32_t ttft = dev_only ? Td : min(q.S, wTd);
+            const bool migr = started && !dev_only && dev_wins == dev_migrates && saving_m > rp.theta;
+            emit(at, dev_only, started, dev_wins, migr, ttft);
         }
     }
 }
@@ -616,8 +607,10 @@ cudaError_t launch_pairs_rows(const TraceDev& tr, const GroupConst* gc, const Cl
     const bool idx32 = (uint64_t)P * tr.n <= 0xFFFFFFFFull;
     auto* row_kernel = extras ? (idx32 ? k_pairs_rows<true, true> : k_pairs_rows<true, false>)
                               : (idx32 ? k_pairs_rows<false, true> : k_pairs_rows<false, false>);
+    const size_t smem = (size_t)tr.n_groups * kRowPols * (extras ? sizeof(Prep) : sizeof(RowPol));
+    if (cudaError_t e = allow_smem((const void*)row_kernel, kMaxGroups * kRowPols * sizeof(Prep))) return e;
     dim3 grid_r((tr.n + kRowThreads - 1) / kRowThreads, (n_list + kRowPols - 1) / kRowPols);
-    return launch_after(row_kernel, grid_r, kRowThreads, 0, st, tr, gc, cc, prep, P, pol_list, n_list, rec, k0, out);
+    return launch_after(row_kernel, grid_r, kRowThreads, smem, st, tr, gc, cc, prep, P, pol_list, n_list, rec, k0, out);
 }
 
 }  // namespace disco

@@ -216,3 +216,14 @@ def test_large_traces_are_placed_by_way_of_buckets(n, shape, kind, where):
         assert (out["tok_server"].cpu().numpy() == pairs["tok_server"]).all()
         assert np.allclose(out["ttft_s"].cpu().numpy(), pairs["ttft_s"], rtol=1e-6)
     tr.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 1), (2, 3), (8, 8)])
+@pytest.mark.parametrize("n", [1, 255, 257, 1500])
+def test_rows_of_several_groups(n, shape):
+    # a block writes the rows of neighbouring requests of any groups, with the rules of up to 16 policies for each: a partly
+    # filled block and row of policies, up to 64 groups, with random routing and expected lengths among them and without
+    w = synth.tiny_workload(107, n, n_servers=shape[0], n_devices=shape[1], max_prompt=300, max_out=60)
+    plain = [synth.policy(b, mig_threshold=1e-6 * k) for k, b in enumerate(synth.budget_grid(17))]
+    full_parity(w, plain, select=False, tag=f"{n} {shape}")
+    full_parity(w, plain[:3] + [synth.policy(0.5, flags=PACED | synth.FLAG_STOCHASTIC), synth.policy(0.3, expected_len=20)], select=False, tag=f"{n} {shape} extras")
