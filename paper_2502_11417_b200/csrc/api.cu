@@ -143,6 +143,9 @@ struct disco_ctx {
     std::vector<uint64_t> fin_own;     // this trace's totals, to put back before the next evaluation
     LargeLoad large;                   // working memory of a large trace's load
     bool inv_there = false;            // `inv` has been written
+    // What a load must clear lies twice in memory where load_once.cu's kernel loads the trace: it works in one half and clears the
+    // other for the next load.  Where they lie (nowhere after any other load) and which of them is zero.
+    struct Halves { void* at = nullptr; size_t cap = 0, bytes = 0; bool zero[2] = {false, false}; int now = 0; } halves;
     LoadZero* z = nullptr;
     uint32_t *cnt = nullptr, *tick_cnt = nullptr;
     uint2* windows = nullptr;
@@ -234,11 +237,13 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     const size_t N = n ? n : 1, N4 = N + 3;
     const int G = c->G;
     Layout lay;
-    const size_t o_req = lay.take(N * 16), o_sorted = lay.take(N * 4), o_binned = lay.take(N * 4), o_inv = lay.take(N * 4);
-    // one block for everything a load clears: the flags and sums, the two histograms, the windows of the sort
+    // one block for everything a load clears, first: the flags and sums, the two histograms, the windows of the sort
+    const bool once = once_trace(n, G, (uint32_t)c->sms);
     const size_t tick_bytes = (size_t)G * kTickBins * 4, cnt_bytes = ((size_t)G * (kMaxPrompt + 1) * 4 + 15) / 16 * 16;
-    c->zero_bytes = sizeof(LoadZero) + tick_bytes + cnt_bytes + (size_t)sort_windows(n, G) * 8;
-    const size_t o_zero = lay.take(c->zero_bytes), o_ends = lay.take((size_t)G * (kMaxPrompt + 1) * 4), o_starts = lay.take(2 * tick_bytes);
+    c->zero_bytes = sizeof(LoadZero) + tick_bytes + cnt_bytes + (once ? (size_t)kOnceWindows * 16 : (size_t)sort_windows(n, G) * 8);
+    const size_t o_zero[2] = {lay.take(c->zero_bytes), once ? lay.take(c->zero_bytes) : 0};
+    const size_t o_req = lay.take(N * 16), o_sorted = lay.take(N * 4), o_binned = lay.take(N * 4), o_inv = lay.take(N * 4);
+    const size_t o_ends = lay.take((size_t)G * (kMaxPrompt + 1) * 4), o_starts = lay.take(2 * tick_bytes);
     const size_t o_mass = lay.take((size_t)G * (kMaxPrompt + 2) * 8), o_off = lay.take((kMaxGroups + 1) * 4);
     const size_t o_knots = lay.take((size_t)G * kNKnots * 4), o_fin = lay.take((size_t)2 * kMaxGroups * 8);
     size_t o_in[5] = {0, 0, 0, 0, 0};
@@ -263,12 +268,18 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     const cudaError_t e = c->trace_mem.reserve(lay.bytes);
     if (e) return e;
     char* base = (char*)c->trace_mem.p;
+    disco_ctx::Halves& hv = c->halves;
+    if (!once || hv.at != base || hv.cap != c->trace_mem.cap || hv.bytes != c->zero_bytes) {
+        hv = disco_ctx::Halves();
+        if (once) { hv.at = base; hv.cap = c->trace_mem.cap; hv.bytes = c->zero_bytes; }
+    }
+    if (once) hv.now ^= 1;
     lg.parted = (uint4*)(base + o_parted);
     lg.rec_bucket = (uint16_t*)(base + o_rec_of); lg.tick_bucket = (uint16_t*)(base + o_tick_of);
     lg.rec_at = (uint32_t*)(base + o_at); lg.tick_at = lg.rec_at + lg.n_rec;
     lg.rec_members = (uint2*)(base + o_members); lg.tick_members = lg.rec_members + lg.n_rec;
     c->req.p = base + o_req; c->sorted.p = base + o_sorted; c->binned.p = base + o_binned; c->inv.p = base + o_inv;
-    c->zero.p = base + o_zero; c->len_end.p = base + o_ends; c->tick_start.p = base + o_starts; c->cum_mass.p = base + o_mass;
+    c->zero.p = base + o_zero[hv.now]; c->len_end.p = base + o_ends; c->tick_start.p = base + o_starts; c->cum_mass.p = base + o_mass;
     c->grp_off.p = base + o_off; c->knots.p = base + o_knots; c->fin_totals.p = base + o_fin;
     c->in_prompt.p = c->st_ticks.p = c->packed.p = base + o_in[0];
     c->in_out.p = c->st_ln.p = base + o_in[1];
@@ -442,7 +453,16 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     const bool large = large_load(n, c->G);
     a.large = c->large;
     c->inv_there = !large;
-    if ((e = large ? run_load_large(a, c->sms, st) : run_load(a, c->sms, st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion kernels"));
+    disco_ctx::Halves& hv = c->halves;
+    const bool once = hv.at != nullptr;
+    if (once) {
+        a.once.windows = (unsigned long long*)c->windows;
+        a.once.zeroed = hv.zero[hv.now];
+        a.once.clear = (uint4*)((char*)c->zero.p + (hv.now ? -1 : 1) * (ptrdiff_t)((c->zero_bytes + 255) / 256 * 256));
+        a.once.clear_vecs = (uint32_t)(c->zero_bytes / 16);
+        hv.zero[0] = hv.zero[1] = false;                             // (until the load has succeeded)
+    }
+    if ((e = once ? run_load_once(a, c->sms, st) : large ? run_load_large(a, c->sms, st) : run_load(a, c->sms, st)) != cudaSuccess) return bail(fail_cuda(e, "trace ingestion kernels"));
     g_launches += large ? 6 : 1;
     // the few numbers the host needs (error word, group sizes, longest output, largest TTFT per group) are in rb
     HostReadback* rb = c->rb;
@@ -468,6 +488,7 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     }
     c->F_sorted = c->sorted.as<int32_t>(); c->F_off = c->grp_off.as<uint32_t>();
     c->F_n.assign(rb->ng, rb->ng + c->G);
+    if (once) hv.zero[hv.now ^ 1] = true;
     c->loaded = true;
     own.release();
     *pctx = c;
@@ -1155,7 +1176,7 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     const size_t T1 = (size_t)std::max<uint64_t>(total, 1);
     const size_t tick_bytes = (size_t)G * kTickBins * 4;
     if ((e = c->F_sorted_imp.reserve(T1 * 4)) != cudaSuccess || (e = c->F_off_imp.reserve((size_t)(kMaxGroups + 1) * 4)) != cudaSuccess ||
-        (e = c->sort_in.reserve(2 * ((T1 + 3) / 4 * 4) * 4 + (size_t)sort_windows((uint32_t)total, G) * 8)) != cudaSuccess)
+        (e = c->sort_in.reserve(2 * ((T1 + 3) / 4 * 4) * 4 + std::max((size_t)sort_windows((uint32_t)total, G) * 8, (size_t)kOnceWindows * 16))) != cudaSuccess)
         return fail_cuda(e, "device allocation for the tables");
     // ticks in this device's memory are read where they are (another device's may not be mapped here, and a kernel cannot read
     // words across their alignment); sort_in: a copy of others, the same by bin, the windows
@@ -1178,7 +1199,7 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     LoadArgs a = {};
     a.n = (uint32_t)total; a.G = G; a.ticks = in; a.off = c->F_off_imp.as<uint32_t>();
     a.z = c->z; a.zero_bytes = sizeof(LoadZero) + tick_bytes; a.tick_cnt = c->tick_cnt; a.tick_start = c->tick_start.as<uint32_t>(); a.tick_at = a.tick_start + (size_t)G * kTickBins;
-    a.binned = (uint32_t*)copy + T4; a.windows = (uint2*)(copy + 2 * T4); a.rounds = 1; a.sorted = c->F_sorted_imp.as<int32_t>();
+    a.binned = (uint32_t*)copy + T4; a.windows = (uint2*)(copy + 2 * T4); a.once.windows = (unsigned long long*)a.windows; a.rounds = 1; a.sorted = c->F_sorted_imp.as<int32_t>();
     if (!total) CU(cudaMemsetAsync(c->z, 0, sizeof(LoadZero), st));
     if (total) { CU(run_sort_ticks(a, c->sms, st)); g_launches += 1; }
     CU(launch_tables_imported(G, c->cnt, c->cum_mass.as<int64_t>(), c->F_sorted_imp.as<int32_t>(), c->F_off_imp.as<uint32_t>(),

@@ -39,6 +39,35 @@ struct SortSmem {
     uint32_t bin[kTickBins];                           // of a window's bins: first place | count << 16
 };
 
+// The waits between blocks are bounded.  Behind one that ran out, tables may hold what an earlier call left in them, and
+// places taken from those could lie anywhere: a block that gives up sets the flag that makes the host refuse the results
+// and kLost in the barriers' word, and leaves the kernel; so does every block that finds kLost where it waits.  A block
+// that passes a barrier has seen every block arrive there, with its part of the work in front of it done.
+constexpr uint32_t kWaitTries = 1u << 22;
+constexpr uint32_t kLost = 1u << 31;              // (the word counts at most 256 blocks three times)
+__device__ __forceinline__ void give_up(LoadZero* z) {
+    atomicMax(&z->err[3], 2);
+    atomicOr(&z->barrier, kLost);
+}
+
+// Waits until `want` blocks have arrived; false: the caller's block has to leave.
+__device__ __forceinline__ bool await_blocks(LoadZero* z, uint32_t want) {
+    uint32_t seen, tries = 0;
+    do {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&z->barrier) : "memory");
+    } while (seen < want && ++tries < kWaitTries);                     // (with kLost it is above any count)
+    if (seen < want) give_up(z);
+    __threadfence();
+    return seen >= want && !(seen & kLost);
+}
+
+// Checked build: a wait for one arrival that nobody makes (LoadArgs::absent).
+#ifdef DISCO_DEBUG
+#define ABSENT(a, wait) ((a).absent == (wait) ? 1u : 0u)
+#else
+#define ABSENT(a, wait) 0u
+#endif
+
 // Four neighbouring requests of the trace (or ticks of a sample) as the two passes see them.
 struct Item { uint32_t g, S, l, o; bool in; };
 
@@ -427,6 +456,29 @@ __device__ __forceinline__ void write_knots(const LoadArgs& a, int g, uint32_t k
             if (k == kNKnots - 1) a.readback->knot_max[g] = v;
         }
     }
+}
+
+// Sorts the bins [b0, b1] of a group, whose ticks lie in [k0, k1); ends with a barrier.
+__device__ __forceinline__ void sort_bins(const LoadArgs& a, SortSmem& sm, int g, int b0, int b1, uint32_t k0, uint32_t k1) {
+    const uint32_t lo = tick_bin_edge(b0);
+    auto bits_of = [](uint32_t range) { return range <= 1u ? 0 : 32 - __clz((int)(range - 1u)); };
+    const uint32_t *starts = a.tick_start + (size_t)g * kTickBins, *counts = a.tick_cnt + (size_t)g * kTickBins;
+    // up to kSortCap ticks; otherwise the last bin is a large one: the others first
+    const bool large = k1 - k0 > kSortCap;
+    const uint32_t to = large ? __ldcg(&starts[b1]) : k1;
+    const int last = large ? b1 - 1 : b1;
+    if (to > k0 && !sort_window(sm, a.binned + k0, to - k0, starts, counts, b0, last, a.sorted + k0)) {
+        __syncthreads();
+        sort_window_radix(sm, a.binned + k0, to - k0, lo, bits_of(tick_bin_edge(last + 1) - lo), a.sorted + k0);
+    }
+    if (large) {
+        __syncthreads();
+        const uint32_t edge = tick_bin_edge(b1);
+        if (!sort_dense<kThreads, kCounters>(sm.a, sm.wtot, sm.range, a.binned + to, k1 - to, edge, tick_bin_edge(b1 + 1) - edge, a.sorted + to) &&
+            threadIdx.x == 0)
+            atomicMax(&a.z->err[3], 1);
+    }
+    __syncthreads();
 }
 
 }  // namespace

@@ -28,17 +28,6 @@ namespace disco {
 
 namespace {
 
-// The waits between blocks are bounded.  Behind one that ran out, tables may hold what an earlier call left in them, and
-// places taken from those could lie anywhere: a block that gives up sets the flag that makes the host refuse the results
-// and kLost in the barriers' word, and leaves the kernel; so does every block that finds kLost where it waits.  A block
-// that passes a barrier has seen every block arrive there, with its part of the work in front of it done.
-constexpr uint32_t kWaitTries = 1u << 22;
-constexpr uint32_t kLost = 1u << 31;              // (the word counts at most 256 blocks three times)
-__device__ __forceinline__ void give_up(LoadZero* z) {
-    atomicMax(&z->err[3], 2);
-    atomicOr(&z->barrier, kLost);
-}
-
 // Waits until every block of the grid has come here `times` times.  False, to all threads: the block has to leave.
 __device__ __forceinline__ bool grid_barrier(LoadZero* z, uint32_t times, uint32_t absent) {
     __syncthreads();
@@ -47,14 +36,7 @@ __device__ __forceinline__ bool grid_barrier(LoadZero* z, uint32_t times, uint32
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(&z->barrier, 1u);
-        const uint32_t want = times * gridDim.x + absent;
-        uint32_t seen, tries = 0;
-        do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&z->barrier) : "memory");
-        } while (seen < want && ++tries < kWaitTries);                 // (with kLost it is above any count)
-        if (seen < want) give_up(z);
-        lost = seen < want || (seen & kLost);
-        __threadfence();
+        lost = !await_blocks(z, times * gridDim.x + absent);
     }
     return !__syncthreads_or(lost);
 }
@@ -69,13 +51,6 @@ __device__ __forceinline__ unsigned long long await_word(LoadZero* z, const unsi
     if (v == 0ull) give_up(z);
     return v;
 }
-
-// Checked build: a wait for one arrival that nobody makes (LoadArgs::absent).
-#ifdef DISCO_DEBUG
-#define ABSENT(a, wait) ((a).absent == (wait) ? 1u : 0u)
-#else
-#define ABSENT(a, wait) 0u
-#endif
 
 // Four counters from k on (16-byte aligned), those from k1 on empty.
 __device__ __forceinline__ uint4 four_counters(const uint32_t* cnt, int k, int k1) {
@@ -408,25 +383,7 @@ k_load(const __grid_constant__ LoadArgs a) {
         const uint32_t k0 = s_win[0][j & 31u], k2 = s_win[1][j & 31u], k1 = s_win[2][j & 31u];
         if (k0 >= k1) continue;                                        // (inside a large bin)
         const int g = (int)s_win[3][j & 31u] / kTickBins, b0 = (int)s_win[3][j & 31u] - g * kTickBins, b1 = (int)s_win[4][j & 31u] - g * kTickBins;
-        const uint32_t lo = tick_bin_edge(b0);
-        auto bits_of = [](uint32_t range) { return range <= 1u ? 0 : 32 - __clz((int)(range - 1u)); };
-        const uint32_t *starts = a.tick_start + (size_t)g * kTickBins, *counts = a.tick_cnt + (size_t)g * kTickBins;
-        // up to kSortCap ticks; otherwise the last bin is a large one: the others first
-        const bool large = k1 - k0 > kSortCap;
-        const uint32_t to = large ? k2 : k1;
-        const int last = large ? b1 - 1 : b1;
-        if (to > k0 && !sort_window(sm, a.binned + k0, to - k0, starts, counts, b0, last, a.sorted + k0)) {
-            __syncthreads();
-            sort_window_radix(sm, a.binned + k0, to - k0, lo, bits_of(tick_bin_edge(last + 1) - lo), a.sorted + k0);
-        }
-        if (large) {
-            __syncthreads();
-            const uint32_t edge = tick_bin_edge(b1);
-            if (!sort_dense<kThreads, kCounters>(sm.a, sm.wtot, sm.range, a.binned + k2, k1 - k2, edge, tick_bin_edge(b1 + 1) - edge, a.sorted + k2) &&
-                tid == 0)
-                atomicMax(&z->err[3], 1);
-        }
-        __syncthreads();
+        sort_bins(a, sm, g, b0, b1, k0, k1);
         if (kTrace) write_knots<kThreads>(a, g, k0, k1, s_off[g], s_off[g + 1] - s_off[g]);
     }
     if (kTrace) {
@@ -499,8 +456,9 @@ cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st) {
     if (a.packed) return launch_load<S_TRACE, F_PACKED>(a, sms, st);
     return a.st_ticks ? launch_load<S_TRACE, F_STAGE>(a, sms, st) : launch_load<S_TRACE, F_COLUMNS>(a, sms, st);
 }
-cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st) { return launch_load<S_TICKS, F_COLUMNS>(a, sms, st); }
-cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st) { return launch_load<S_TTFT, F_COLUMNS>(a, sms, st); }
+cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st) {
+    return once_ticks(a.n, a.G, (uint32_t)sms) ? run_sort_ticks_once(a, sms, st) : launch_load<S_TICKS, F_COLUMNS>(a, sms, st);
+}
 
 cudaError_t launch_tables_imported(int G, const uint32_t* cnt, int64_t* cum_mass, const int32_t* F_sorted,
                                    const uint32_t* F_off, int32_t* knots, cudaStream_t st) {
@@ -525,7 +483,7 @@ constexpr size_t kNaKeysBytes = (size_t)kNoAllocMaxN * sizeof(uint64_t);
 constexpr size_t kNaCountsBytes = (256u * ((kNoAllocMaxN + 1023u) / 1024u) + 256u) * sizeof(uint32_t);   // as radix_sort_ticks sizes its grid, plus the digit totals
 // words that must start at zero: the flags and the bins' counters; then the bins' starts and the offsets of the one group
 constexpr size_t kNaZeroOff = 2 * kNaKeysBytes + kNaCountsBytes;
-constexpr size_t kNaZeroBytes = (sizeof(LoadZero) + kTickBins * 4 + sort_windows(kNoAllocMaxN, 1) * 8 + 15) / 16 * 16;
+constexpr size_t kNaZeroBytes = (sizeof(LoadZero) + kTickBins * 4 + kOnceWindows * 16 + 15) / 16 * 16;
 constexpr size_t kNaStartOff = kNaZeroOff + kNaZeroBytes;
 constexpr size_t kNaOffOff = kNaStartOff + kTickBins * 4;
 
@@ -571,7 +529,7 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
     a.n = n; a.G = 1; a.ns = a.nd = 1;
     a.ttft = server_ttft_s;
     a.z = (LoadZero*)(base + kNaZeroOff); a.tick_cnt = (uint32_t*)(base + kNaZeroOff + sizeof(LoadZero));
-    a.windows = (uint2*)(a.tick_cnt + kTickBins); a.rounds = 1;
+    a.once.windows = (unsigned long long*)(a.tick_cnt + kTickBins);
     a.tick_start = (uint32_t*)(base + kNaStartOff);
     a.binned = (uint32_t*)base; a.sorted = sorted_ticks;
     a.zero_bytes = kNaZeroBytes;          // the array still holds the previous call's data: flags and counters must start at zero

@@ -1,6 +1,8 @@
 // Trace ingestion and the sort of server-TTFT ticks (load.cu).
 #pragma once
 
+#include <algorithm>
+
 #include "disco_internal.cuh"
 
 namespace disco {
@@ -60,6 +62,18 @@ struct LargeLoad {
     uint2 *rec_members, *tick_members;    // first and last length or bin, counted through the groups (first > last: none)
 };
 
+// Small and middling traces: a kernel whose threads read their requests once and keep them (load_once.cu).
+constexpr uint32_t kOnceAlone = 4096;         // requests of one group that a single block takes
+constexpr uint32_t kOnceWindows = 1024;       // windows of the sort, at most
+struct OnceLoad {
+    uint32_t blocks, per_block;           // blocks that read the trace, requests of each
+    int seg_shift, win_shift;             // counters added up by a warp, ticks sorted at a time (their logarithms)
+    unsigned long long* windows;          // [kOnceWindows][2]: complement of the first bin | where its ticks start, last bin + 1 | where they end
+    uint4* clear;                         // words to set to zero on the way
+    uint32_t clear_vecs;
+    bool zeroed;                          // z and what lies behind it is zero already
+};
+
 struct LoadArgs {
     uint32_t n;
     int G;
@@ -97,6 +111,7 @@ struct LoadArgs {
     int32_t* knots;                       // [G][257]
     uint64_t* fin_totals;                 // [2G]: output tokens per group, then requests per group
     LargeLoad large;
+    OnceLoad once;
     LoadReadback* readback;               // its err holds 0, 0, 0, 2 (no report) before the launch
 #ifdef DISCO_DEBUG
     uint32_t absent;                      // the wait that expects one arrival more than comes (from 1; 4: of the other blocks' sums)
@@ -106,6 +121,14 @@ struct LoadArgs {
 cudaError_t run_load(const LoadArgs& a, int sms, cudaStream_t st);          // one kernel, after a memset
 // The same for kLargeMinN to kLargeMaxN requests in at most kLargeMaxGroups groups: six kernels, after a memset.
 cudaError_t run_load_large(const LoadArgs& a, int sms, cudaStream_t st);
+// The same for as many requests as the threads can keep (eight each): one kernel, after a memset if `zeroed` is not
+// set.
+inline bool once_trace(uint32_t n, int G, uint32_t sms) {
+    return G <= kLargeMaxGroups && sms > 2u * (uint32_t)G && n <= (std::min(sms, kLoadBlocks) - (uint32_t)G) * 8192u;
+}
+inline bool once_ticks(uint32_t n, int G, uint32_t sms) { return G <= 16 && n <= std::min(sms, kLoadBlocks) * 8192u; }
+cudaError_t run_load_once(const LoadArgs& a, int sms, cudaStream_t st);
+cudaError_t run_sort_ticks_once(const LoadArgs& a, int sms, cudaStream_t st);
 cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st);    // ticks, off, G, n -> sorted
 cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st);     // ttft, n (one group) -> sorted
 
