@@ -358,7 +358,7 @@ k_load(const __grid_constant__ LoadArgs a) {
 
     // ---- 3. sort
     SortSmem& sm = *reinterpret_cast<SortSmem*>(smem_raw);
-    __shared__ uint32_t s_win[5][32];                 // of the block's next windows: first tick, last bin's first tick, end, bins
+    __shared__ uint32_t s_win[4][32];                 // of the block's next windows: first tick, end, first and last bin
     uint32_t n_win = 0;
     for (int g = 0; g < G; ++g) n_win += (s_off[g + 1] - s_off[g] + kWindow - 1) / kWindow;
 #pragma unroll 1
@@ -373,16 +373,16 @@ k_load(const __grid_constant__ LoadArgs a) {
                 if (mine < n_win) bins = __ldcg(&a.windows[mine]);
                 if (bins.y) {
                     const uint32_t first_bin = 0xFFFFFFFFu - bins.x, last_bin = bins.y - 1u;
-                    const uint32_t k2 = __ldcg(&a.tick_start[last_bin]);
-                    s_win[0][tid] = __ldcg(&a.tick_start[first_bin]); s_win[1][tid] = k2;
-                    s_win[2][tid] = k2 + __ldcg(&a.tick_cnt[last_bin]); s_win[3][tid] = first_bin; s_win[4][tid] = last_bin;
-                } else s_win[0][tid] = s_win[2][tid] = 0u;
+                    s_win[0][tid] = __ldcg(&a.tick_start[first_bin]);
+                    s_win[1][tid] = __ldcg(&a.tick_start[last_bin]) + __ldcg(&a.tick_cnt[last_bin]);
+                    s_win[2][tid] = first_bin; s_win[3][tid] = last_bin;
+                } else s_win[0][tid] = s_win[1][tid] = 0u;
             }
         }
         __syncthreads();
-        const uint32_t k0 = s_win[0][j & 31u], k2 = s_win[1][j & 31u], k1 = s_win[2][j & 31u];
+        const uint32_t k0 = s_win[0][j & 31u], k1 = s_win[1][j & 31u];
         if (k0 >= k1) continue;                                        // (inside a large bin)
-        const int g = (int)s_win[3][j & 31u] / kTickBins, b0 = (int)s_win[3][j & 31u] - g * kTickBins, b1 = (int)s_win[4][j & 31u] - g * kTickBins;
+        const int g = (int)s_win[2][j & 31u] / kTickBins, b0 = (int)s_win[2][j & 31u] - g * kTickBins, b1 = (int)s_win[3][j & 31u] - g * kTickBins;
         sort_bins(a, sm, g, b0, b1, k0, k1);
         if (kTrace) write_knots<kThreads>(a, g, k0, k1, s_off[g], s_off[g + 1] - s_off[g]);
     }

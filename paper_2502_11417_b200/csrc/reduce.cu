@@ -36,26 +36,31 @@ __device__ __forceinline__ void warp_quantile_bins(const unsigned long long* __r
         const unsigned long long up = __shfl_up_sync(0xFFFFFFFFu, incl, off);
         if (lane >= off) incl += up;
     }
+    // every rank at once, on one walk over the lane's bins: the walks of the lanes that hold them took 0.7 us a rank one after
+    // another
     const unsigned long long excl = incl - sum;
-#pragma unroll 1
+    unsigned long long rank[NQ];
+    int found[NQ];
+#pragma unroll
     for (int k = 0; k < NQ; ++k) {
-        int bin = 0;
-        if (M) {
-            unsigned long long rank = (unsigned long long)ceil(__dmul_rn(qs[k], (double)M));
-            if (rank < 1) rank = 1;
-            int found = -1;
-            if (rank > excl && rank <= incl) {
-                unsigned long long acc = excl;
-                for (int i = 0; found < 0 && i < kBinsPerLane; ++i) {
-                    acc += mine[i];
-                    if (acc >= rank) found = lane * kBinsPerLane + i;
-                }
-            }
-            const unsigned owner = __ballot_sync(0xFFFFFFFFu, found >= 0);
-            bin = owner ? __shfl_sync(0xFFFFFFFFu, found, __ffs(owner) - 1) : kNBins - 1;
-            if (!DBG_OK(bin, kNBins, DBG_K_FINALIZE, DBG_BIN)) bin = kNBins - 1;
-        }
-        out[k] = bin;
+        rank[k] = (unsigned long long)ceil(__dmul_rn(qs[k], (double)M));
+        if (rank[k] < 1) rank[k] = 1;
+        found[k] = 0;                                     // bins in front of the one that holds the rank
+    }
+    unsigned long long acc = excl;
+#pragma unroll
+    for (int i = 0; i < kBinsPerLane; ++i) {
+        acc += mine[i];
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) found[k] += acc < rank[k] ? 1 : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) {
+        const unsigned owner = __ballot_sync(0xFFFFFFFFu, rank[k] > excl && rank[k] <= incl);
+        int bin = __shfl_sync(0xFFFFFFFFu, lane * kBinsPerLane + found[k], owner ? __ffs(owner) - 1 : 0);
+        if (!owner) bin = kNBins - 1;
+        if (!DBG_OK(bin, kNBins, DBG_K_FINALIZE, DBG_BIN)) bin = kNBins - 1;
+        out[k] = M ? bin : 0;
     }
 }
 
