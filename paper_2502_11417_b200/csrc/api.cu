@@ -161,9 +161,12 @@ struct disco_ctx {
     View d_prep, d_accum, d_stats, d_tables, d_grid, d_left;
     View d_acc, d_hist_ttft, d_hist_tbt, d_work;          // regions of d_accum; d_work: the counters in front of d_grid
     View play_ticket, rec_hand, rec_u32[6], rec_win[3];      // regions of rec_mem
+    std::vector<uint4> tables_host;   // the small host->device tables where they go with a launch
     void* stage = nullptr;       // pinned staging for the small host->device tables
     size_t stage_cap = 0;
-    cudaEvent_t stage_free = nullptr;
+    cudaEvent_t stage_free = nullptr;    // behind the copies that read it
+    uint32_t stage_turn = 0;     // evaluations that have had their tables read there by a kernel, which puts their number into stage_read
+    volatile uint32_t* stage_read = nullptr;   // in the pinned block of rb
     int32_t* sel_host = nullptr; // [2], in the pinned block of rb
     uint32_t* tab_host = nullptr;   // pinned copy of the group tables: [G][4097] length counts, then [G][257] knots
     int tab_host_groups = 0;        // groups it has room for
@@ -310,10 +313,14 @@ int fetch_knots(disco_ctx* c, cudaStream_t st) {
     return 0;
 }
 
-// Pinned staging of at least that many bytes, once the copies of an earlier call no longer read it.
+// Pinned staging of at least that many bytes, once the copies or the kernel of an earlier call no longer read it.
 int reserve_stage(disco_ctx* c, size_t bytes) {
     if (c->stage_free) CU(cudaEventSynchronize(c->stage_free));
     else CU(cudaEventCreateWithFlags(&c->stage_free, cudaEventDisableTiming));
+    if (*c->stage_read != c->stage_turn) {       // (two evaluations in a row: no event behind the kernel, which would hold the next one up)
+        CU(cudaDeviceSynchronize());
+        *c->stage_read = c->stage_turn;
+    }
     if (bytes > c->stage_cap) {
         if (c->stage) cudaFreeHost(c->stage);
         c->stage = nullptr; c->stage_cap = 0;
@@ -398,6 +405,10 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     if (!c->rb && (e = cudaMallocHost((void**)&c->rb, sizeof(HostReadback) + 256)) != cudaSuccess)    // (the selection's pair behind it)
         return bail(fail_cuda(e, "cudaMallocHost"));
     c->sel_host = (int32_t*)((char*)c->rb + (sizeof(HostReadback) + 15) / 16 * 16);
+    if (!c->stage_read) {
+        c->stage_read = (uint32_t*)(c->sel_host + 4);
+        *c->stage_read = c->stage_turn;
+    }
     if ((e = reserve_trace(c, n, in, d->server_profile != nullptr, d->device_profile != nullptr)) != cudaSuccess)
         return bail(fail_cuda(e, "device allocation for the trace"));
 
@@ -649,7 +660,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     auto play_out = [&](size_t k) {
         g_launches += timeline_launches(plan[k].kinds);
         return launch_timeline(tr, gc, classes[k], c->knots.as<int32_t>(), k0, rec, c->err, c->play_ticket.as<uint32_t>(),
-                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, c->sms, st);
+                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, k == 0 && !timed, c->sms, st);
     };
     if (n != 0 && !timed) CU(play_out(0));
 
@@ -801,21 +812,21 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     // the chunks of the groups that Algorithm 1 finds device-constrained come first: Algorithm 2's wait map costs the
     // grid kernel more sweeps per chunk, and its blocks draw their work in list order, so the items drawn last (when
     // some blocks already idle) should be the cheap ones
-    auto make_chunks = [&](uint32_t CH) {
-        std::vector<Chunk> v;
-        v.reserve(N1 / CH + (size_t)G + 1);
+    TablesIn tables;
+    std::memset(&tables, 0, sizeof tables);
+    auto plan_chunks = [&](int which, uint32_t CH) {
+        uint32_t count = 0, &n_plan = tables.n_plan[which];
         for (int dear = 1; dear >= 0; --dear)
             for (int g = 0; g < G; ++g) {
-                if ((c->gc[g].auto_device_constrained != 0) != (dear != 0)) continue;
-                for (uint32_t s = rb.grp_off[g]; s < rb.grp_off[g + 1]; s += CH)
-                    v.push_back({s, std::min(CH, rb.grp_off[g + 1] - s), g, 0});
+                if ((c->gc[g].auto_device_constrained != 0) != (dear != 0) || rb.ng[g] == 0) continue;
+                tables.plan[which][n_plan++] = ChunkPlan{count, rb.grp_off[g], rb.grp_off[g + 1], g};
+                count += (rb.ng[g] - 1) / CH + 1;
             }
-        return v;
+        tables.chunk_len[which] = CH; tables.n_chunks[which] = count;
     };
     const size_t at_once = (size_t)sms * grid_blocks_per_sm(tallest);
-    const std::vector<Chunk> chunks = make_chunks(chunk_size(2 * at_once, 256));
-    std::vector<Chunk> pair_chunks;
-    if (any_pairs) pair_chunks = make_chunks(chunk_size((size_t)2 * sms, 2048));
+    plan_chunks(0, chunk_size(2 * at_once, 256));
+    if (any_pairs) plan_chunks(1, chunk_size((size_t)2 * sms, 2048));
 
     // ---- the difference tables of the slabs, laid out batch by batch: a batch's slabs have like numbers of rows and share
     //      one class; its tables are cleared, filled, added up and then belong to the next batch
@@ -861,9 +872,9 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const size_t o_accum2 = clear_accum ? o_accum : lay.take(acc_bytes + 2 * hist_bytes);
     const size_t o_left = lay.take(any_mixed ? (N1 + kMaxGroups) * 4 : 0);
     const size_t table_bytes = ((size_t)P * sizeof(PolicyConst) + 15) / 16 * 16 + (classes.size() * sizeof(ClassConst) + 15) / 16 * 16 +
-                               (tab.size() * 4 + 15) / 16 * 16 + (slabs.size() * sizeof(Slab) + 15) / 16 * 16 +
-                               (chunks.size() + pair_chunks.size()) * sizeof(Chunk);
+                               (tab.size() * 4 + 15) / 16 * 16 + (slabs.size() * sizeof(Slab) + 15) / 16 * 16;
     const size_t o_tables = lay.take(table_bytes);
+    const size_t o_chunks[2] = {lay.take(tables.n_chunks[0] * sizeof(Chunk)), lay.take(tables.n_chunks[1] * sizeof(Chunk))};
     if ((e = c->eval_mem.reserve(lay.bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
     char* mem = (char*)c->eval_mem.p;
     c->d_prep.p = mem + o_prep; c->d_accum.p = mem + o_accum2; c->d_stats.p = mem + o_stats; c->d_grid.p = mem + o_grid;
@@ -881,9 +892,11 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     }
     if (clear_apart) CU(cudaMemsetAsync(mem, 0, clear_bytes, st));
 
-    // ---- small tables to the device through pinned staging: one staging block, one copy (16-byte aligned regions)
-    if (int rc = reserve_stage(c, table_bytes)) return rc;
-    char *sp = (char*)c->stage, *dt = mem + o_tables;
+    // ---- small tables to the device with k_prep: one block, 16-byte aligned regions
+    const bool in_launch = table_bytes <= kTablesInline;
+    if (in_launch) c->tables_host.resize(kTablesInline / sizeof(uint4));
+    else if (int rc = reserve_stage(c, table_bytes)) return rc;
+    char *sp = in_launch ? (char*)c->tables_host.data() : (char*)c->stage, *dt = mem + o_tables;
     size_t off = 0;
     auto put = [&](const void* src, size_t bytes) {
         if (bytes) std::memcpy(sp + off, src, bytes);
@@ -895,14 +908,16 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const ClassConst* d_classes = (const ClassConst*)put(classes.data(), classes.size() * sizeof(ClassConst));
     const uint32_t* d_tab = (const uint32_t*)put(tab.data(), tab.size() * 4);
     const Slab* d_slabs = (const Slab*)put(slabs.data(), slabs.size() * sizeof(Slab));
-    const Chunk* d_chunks = (const Chunk*)put(chunks.data(), chunks.size() * sizeof(Chunk));
-    const Chunk* d_pair_chunks = (const Chunk*)put(pair_chunks.data(), pair_chunks.size() * sizeof(Chunk));
-    CU(cudaMemcpyAsync(dt, sp, off, cudaMemcpyHostToDevice, st));
-    CU(cudaEventRecord(c->stage_free, st));
+    const Chunk *d_chunks = (const Chunk*)(mem + o_chunks[0]), *d_pair_chunks = (const Chunk*)(mem + o_chunks[1]);
+    if (off / 16 > 0xFFFFFFFFull) return fail(DISCO_ENOMEM, "the tables of the policies are too large");
 
     // ---- Algorithms 1-3 for every (group, policy)
-    CU(launch_prep(d_pol, P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
-                   c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), mem, clear_apart ? 0 : clear_bytes, c->sms, st));
+    tables.host = sp; tables.device = dt; tables.vecs = (uint32_t)(off / 16); tables.skip = n_beta ? 0u : (uint32_t)(P * sizeof(PolicyConst) / 16);
+    for (int k = 0; k < 2; ++k) tables.chunks[k] = (Chunk*)(mem + o_chunks[k]);
+    tables.left = &c->z->tables_left; tables.read = c->stage_read; tables.turn = c->stage_turn + 1;
+    CU(launch_prep(P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
+                   c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), tables, mem, clear_apart ? 0 : clear_bytes, c->sms, st));
+    if (!in_launch) ++c->stage_turn;
     g_launches += 1;
     if (n_beta) {
         CU(launch_prep_beta(d_pol, P, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
@@ -946,21 +961,21 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
             }
             CU(launch_grid(tr, gc, dcc, prep, P, dsl, (uint32_t)b.count, b.T, wide, d_tab,
-                           d_chunks, (uint32_t)chunks.size(), rec, gt, left, k0, tickets + ticket++, work, c->sms, st));
+                           d_chunks, tables.n_chunks[0], rec, gt, left, k0, tickets + ticket++, work, c->sms, st));
             CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, wide, host_bin_of_ticks(classes[k].tau), d_tab, gt, acc,
                              h_ttft, h_tbt, st));
             g_launches += 2;
             if (mixed) {
                 const Slab& sl = slabs[b.first];
                 CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + mixed_pols[b.first], sl.policies, d_pair_chunks,
-                                    (uint32_t)pair_chunks.size(), left.list, left.count, rec, acc, h_ttft, h_tbt, work, k0,
+                                    tables.n_chunks[1], left.list, left.count, rec, acc, h_ttft, h_tbt, work, k0,
                                     sl.expected_len != 0, wide, st));
                 g_launches += 1;
             }
         }
         if (lists[k].n_ext) {
             CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + lists[k].ext, (uint32_t)lists[k].n_ext,
-                                d_pair_chunks, (uint32_t)pair_chunks.size(), nullptr, nullptr, rec, acc, h_ttft, h_tbt,
+                                d_pair_chunks, tables.n_chunks[1], nullptr, nullptr, rec, acc, h_ttft, h_tbt,
                                 work, k0, true, wide, st));
             g_launches += 1;
         }

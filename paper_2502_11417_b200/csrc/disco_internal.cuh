@@ -155,6 +155,9 @@ inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block,
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the stream start once every block of this one has come here (or ended); what it may do in front of
+// its own wait is up to it.  To be called behind this kernel's wait.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // The stream after a hand-off stores no window of its own where groups are played free without pacing: it is stream
 // x_stream's (0 the server's, 1 the device's) without the interval in front of token 2, whose bin first_bin gives.  -1: it
@@ -230,8 +233,25 @@ struct DbgRegistrar { explicit DbgRegistrar(cudaError_t (*r)(int32_t*)) { dbg_re
 #endif
 
 // ---- launch wrappers (defined in the kernel translation units) -------------------------------------------
-cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupConst* gc, const int64_t* cum_mass,
-                        const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep,
+// The small tables of an evaluation on their way to the device with k_prep: as its parameter up to kTablesInline bytes, beyond
+// it reads them in pinned host memory.
+constexpr size_t kTablesInline = 28672;      // (a launch takes 32,764 bytes of parameters, the chunk plans 2,048)
+struct ChunkPlan { uint32_t first, start, end; int32_t g; };     // a group's chunks: number of the first, requests [start, end)
+struct TablesIn {
+    const void* host;            // the policies come first; room for kTablesInline bytes where they go as a parameter
+    void* device;
+    uint32_t vecs, skip;         // of 16 bytes; how many of them (policies) no kernel behind needs
+    // chunk tables that k_prep writes out, of the grid kernel and of the pair kernel, group by group
+    ChunkPlan plan[2][kMaxGroups];
+    uint32_t n_plan[2], chunk_len[2], n_chunks[2];
+    Chunk* chunks[2];
+    // in pinned host memory only
+    uint32_t* left;              // device word, zero; blocks that have read their share (zero again when all have)
+    volatile uint32_t* read;     // pinned host word: set to `turn` once all have
+    uint32_t turn;
+};
+cudaError_t launch_prep(uint32_t P, int G, const GroupConst* gc, const int64_t* cum_mass,
+                        const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep, const TablesIn& tables,
                         void* clear, size_t clear_bytes /* a multiple of 16: set to zero on the way */, int sms, cudaStream_t st);
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off,
@@ -245,6 +265,7 @@ cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const Clas
                             const uint32_t* batches, uint32_t search /* largest ClassConst::search of a group with requests */,
                             bool long_outputs /* mean output length of 512 tokens or more */,
                             cudaEvent_t mid /* recorded between the kernels of exact groups and the others, or null */,
+                            bool early /* the preparation follows: it may start beside the last kernel */,
                             int sms /* multiprocessors of the device */, cudaStream_t st);
 uint32_t timeline_launches(uint32_t kinds);
 

@@ -34,7 +34,8 @@ struct LoadZero {
     uint64_t grp_sum_n[kMaxGroups];       // output tokens per group
     uint32_t grp_n[kMaxGroups];           // requests per group (load_large.cu)
     uint32_t max_n;                       // longest output
-    uint32_t barrier, done, pad;
+    uint32_t barrier, done;
+    uint32_t tables_left;                 // k_prep's (no load touches it)
     int32_t err[4];                       // code, request index, window flag, sort flag (1: some bin needs the fallback, 2: a
                                           // wait between blocks ran out)
 };

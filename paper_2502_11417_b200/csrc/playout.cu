@@ -285,12 +285,13 @@ __device__ __noinline__ void play_x(const GroupClass& G, Round rd, uint32_t key,
 
 __global__ void __launch_bounds__(kWarps * 32)
 k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
-          const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int32_t* err) {
+          const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int32_t* err, bool early) {
     __shared__ uint32_t ring_s[kWarps][kRing];
     __shared__ XResult xres_s[kWarps];
     extern __shared__ uint32_t s_win[];                                // [warps][W0 + W1 + W2]
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     grid_dependency_wait();
+    if (early) let_next_start();
     const int32_t tau_eff = cc.tau_eff, tau = cc.tau;
     const int W0 = cc.W[0], W1 = cc.W[1], W2 = cc.W[2];
     const uint32_t B = (uint32_t)cc.B;
@@ -512,27 +513,28 @@ k_playout(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant
 DBG_TRANSLATION_UNIT()
 
 cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots,
-                                 uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, int sms,
+                                 uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, bool early, int sms,
                                  cudaStream_t st);
 cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots,
-                                uint32_t k0, TimelineRec rec, uint32_t batches, int sms, cudaStream_t st);
+                                uint32_t k0, TimelineRec rec, uint32_t batches, bool early, int sms, cudaStream_t st);
 
 uint32_t timeline_launches(uint32_t kinds) { return (kinds & 1u) + ((kinds >> 1) & 1u) + ((kinds >> 2) & 1u); }
 
 cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0,
                             TimelineRec rec, int32_t* err, uint32_t* ticket, uint32_t kinds, const uint32_t* batches,
-                            uint32_t search, bool long_outputs, cudaEvent_t mid, int sms, cudaStream_t st) {
+                            uint32_t search, bool long_outputs, cudaEvent_t mid, bool early, int sms, cudaStream_t st) {
     cudaError_t e;
+    const auto last = [&](int kind) { return early && kinds >> (kind + 1) == 0; };
     if (kinds & (1u << G_EXACT))
-        if ((e = launch_playout_exact(tr, gc, cc, knots, k0, rec, ticket, search, long_outputs, sms, st))) return e;
+        if ((e = launch_playout_exact(tr, gc, cc, knots, k0, rec, ticket, search, long_outputs, last(G_EXACT), sms, st))) return e;
     if (mid && (e = cudaEventRecord(mid, st))) return e;
     if (kinds & (1u << G_FREE))
-        if ((e = launch_playout_free(tr, gc, cc, knots, k0, rec, batches[G_FREE], sms, st))) return e;
+        if ((e = launch_playout_free(tr, gc, cc, knots, k0, rec, batches[G_FREE], last(G_FREE), sms, st))) return e;
     if (kinds & (1u << G_GENERAL)) {
         const size_t smem = (size_t)kWarps * (cc.W[0] + cc.W[1] + cc.W[2]) * 4;
         if ((e = allow_smem((const void*)k_playout, 100 * 1024))) return e;
         const uint32_t blocks = std::min<uint32_t>((batches[G_GENERAL] + kWarps - 1) / kWarps, (uint32_t)sms * 32u);
-        return launch_after(k_playout, blocks, kWarps * 32, smem, st, tr, gc, cc, knots, k0, rec, err);
+        return launch_after(k_playout, blocks, kWarps * 32, smem, st, tr, gc, cc, knots, k0, rec, err, last(G_GENERAL));
     }
     return cudaSuccess;
 }

@@ -58,9 +58,10 @@ template <int PER>
 __global__ void __launch_bounds__(kFastWarps * 32)
 k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, uint32_t* __restrict__ tickets, int rpw,
-               uint32_t one) {
+               uint32_t one, bool early) {
     const int lane = threadIdx.x & 31;
     grid_dependency_wait();
+    if (early) let_next_start();
     const int32_t tau = cc.tau;                                   // pacing is on for every launch of this kernel
     const uint32_t B = (uint32_t)cc.B;
     const long long thr64 = (long long)(B ? B - 1 : 0) * tau;
@@ -251,12 +252,13 @@ struct ShortGroup {                      // a group under the class
 
 __global__ void __launch_bounds__(kShortThreads)
 k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
-                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int per) {
+                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int per, bool early) {
     __shared__ ShortGroup groups[kMaxGroups];
     __shared__ uint4 lag[kShortThreads * kShortPer];         // hash key, lag, output length | hand-off << 16, place | group << 16
     __shared__ uint16_t rest[kShortThreads * kShortPer];     // lags that a thread has not made up
     __shared__ int n_lag, n_long, n_rest;
     grid_dependency_wait();
+    if (early) let_next_start();
     const int32_t tau = cc.tau;
     const uint32_t B = (uint32_t)cc.B;
     const long long thr64 = (long long)(B ? B - 1 : 0) * tau;
@@ -369,13 +371,13 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
 DBG_TRANSLATION_UNIT()
 
 cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots,
-                                 uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, int sms,
+                                 uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, bool early, int sms,
                                  cudaStream_t st) {
     if (search <= kShortSearch) {
         // four requests a thread (fuller warps of lags) once that leaves several blocks to every multiprocessor
         const int per = tr.n >= (uint32_t)sms * 8u * kShortThreads * kShortPer ? kShortPer : 1;
         const uint32_t per_block = (uint32_t)(kShortThreads * per);
-        return launch_after(k_playout_short, (tr.n + per_block - 1) / per_block, kShortThreads, 0, st, tr, gc, cc, knots, k0, rec, per);
+        return launch_after(k_playout_short, (tr.n + per_block - 1) / per_block, kShortThreads, 0, st, tr, gc, cc, knots, k0, rec, per, early);
     }
     // requests per ticket: small batches spread the end of the launch evenly; large traces amortise the ticket
     int rpw = 8;
@@ -388,7 +390,7 @@ cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const
     auto* kernel = long_outputs ? k_playout_fast<4> : k_playout_fast<8>;
     // as many blocks as the GPU holds at once (at most six of these per SM); the ticket counter feeds them
     const uint32_t blocks = std::min<uint32_t>((tr.n + per_block - 1) / per_block, (uint32_t)sms * 6u);
-    return launch_after(kernel, blocks, kFastWarps * 32, 0, st, tr, gc, cc, knots, k0, rec, ticket, rpw, 1u);
+    return launch_after(kernel, blocks, kFastWarps * 32, 0, st, tr, gc, cc, knots, k0, rec, ticket, rpw, 1u, early);
 }
 
 }  // namespace disco

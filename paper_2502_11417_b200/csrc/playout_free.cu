@@ -38,10 +38,11 @@ __device__ __forceinline__ void count_in(const Counters& c, uint32_t x, uint32_t
 template <bool BOTH, bool SMALL>
 __global__ void __launch_bounds__(kFreeWarps * 32, 4)
 k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
-               const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec) {
+               const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, bool early) {
     extern __shared__ __align__(16) uint32_t s_win[];         // per warp: [W0 + W1][32] counters
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warps = blockDim.x >> 5;
     grid_dependency_wait();
+    if (early) let_next_start();
     const int W0 = cc.W[0], W1 = cc.W[1], WW = W0 + W1;
     uint32_t* win = s_win + wib * (WW * 32);
     for (int b = lane; b < WW * 32; b += 32) win[b] = 0;
@@ -151,7 +152,7 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
 
 DBG_TRANSLATION_UNIT()
 
-cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0, TimelineRec rec, uint32_t batches, int sms,
+cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0, TimelineRec rec, uint32_t batches, bool early, int sms,
                                 cudaStream_t st) {
     // as many warps to a block as the windows leave room for (wide jitter: up to 114 KB of counters a stream and warp)
     const size_t per_warp = (size_t)(cc.W[0] + cc.W[1]) * 32 * 4;
@@ -165,7 +166,7 @@ cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const 
     if ((e = allow_smem((const void*)kernel, 227 * 1024))) return e;
     // (batches counts 32 requests each; four blocks of eight warps fit a multiprocessor)
     const uint32_t blocks = std::min<uint32_t>((batches * (32 / kFreeBatch) + warps - 1) / warps, (uint32_t)sms * 4u * kFreeWarps / warps);
-    return launch_after(kernel, blocks, warps * 32, smem, st, tr, gc, cc, knots, k0, rec);
+    return launch_after(kernel, blocks, warps * 32, smem, st, tr, gc, cc, knots, k0, rec, early);
 }
 
 }  // namespace disco

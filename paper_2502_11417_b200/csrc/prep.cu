@@ -42,23 +42,21 @@ __device__ __forceinline__ int first_true(int lo, int hi, F pred) {
     return lo;
 }
 
-constexpr int kPrepThreads = 128;
+//
+// The policies and the other small tables come with the launch, as a parameter (up to kTablesInline bytes), or from the pinned
+// memory the host laid them out in: a block reads its own policies, and all blocks bring a share of the tables to the device
+// for the kernels behind, and write the chunks of requests out.  (A copy in front of this kernel stood between it and the play-out: 10 to 20 us from
+// the play-out's end to this kernel's start, 1 to 6 of them the copy.  From pinned memory this kernel takes 10 us with 1,024
+// policies, with a parameter 3 to 4.  Steps of 100,000 requests under 64 policies 154 -> 146 us, of 200,000 without pacing
+// 207 -> 197, of 4 M long ones 354 -> 341.)  Nothing here depends on the play-out, and the play-out reads nothing that is written here, so the
+// kernel runs beside it -- the load was waited for by the host, and a play-out lets this kernel start only behind its own
+// wait for what came before -- and waits for it at its end, on behalf of the kernels behind both.
+constexpr int kPrepThreads = 128, kPrepWarps = kPrepThreads / 32;
 
-__global__ void __launch_bounds__(kPrepThreads)
-k_prep(const PolicyConst* __restrict__ pol, uint32_t P, int G, const GroupConst* __restrict__ gc,
-                       const int64_t* __restrict__ cum_mass, const uint32_t* __restrict__ cnt,
-                       const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
-                       Prep* __restrict__ prep, uint4* __restrict__ clear, uint32_t clear_vecs) {
-    grid_dependency_wait();
-    // what the kernels behind this one must find zero
-    for (uint32_t i = blockIdx.x * kPrepThreads + threadIdx.x; i < clear_vecs; i += gridDim.x * kPrepThreads)
-        clear[i] = make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t idx = (blockIdx.x * kPrepThreads + threadIdx.x) >> 5;
-    if (idx >= P * (uint32_t)G) return;
-    const int g = (int)(idx / P);
-    const uint32_t p = idx % P;
-    if (!DBG_OK(g, G, DBG_K_PREP, DBG_GROUP)) return;
-    const PolicyConst pc = pol[p];
+__device__ __forceinline__ void prep_pair(const PolicyConst& pc, uint32_t p, int g, uint32_t P, const GroupConst* __restrict__ gc,
+                                          const int64_t* __restrict__ cum_mass, const uint32_t* __restrict__ cnt,
+                                          const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
+                                          Prep* __restrict__ prep) {
     const int64_t* cum = cum_mass + (size_t)g * (kMaxPrompt + 2);     // cum[L] = sum_{l<L} l*cnt[l]
     const uint32_t* c = cnt + (size_t)g * (kMaxPrompt + 1);
     const uint32_t off = grp_off[g], N = grp_off[g + 1] - off;
@@ -105,6 +103,57 @@ k_prep(const PolicyConst* __restrict__ pol, uint32_t P, int G, const GroupConst*
         }
     }
     if ((threadIdx.x & 31) == 0) prep[(size_t)g * P + p] = r;
+}
+
+template <int BYTES> struct Inline { uint4 v[BYTES / 16]; };
+template <> struct Inline<0> { };
+
+template <int BYTES>
+__global__ void __launch_bounds__(kPrepThreads)
+k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __restrict__ cum_mass,
+       const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
+       Prep* __restrict__ prep, const __grid_constant__ TablesIn in, uint4* __restrict__ clear, uint32_t clear_vecs,
+       const __grid_constant__ Inline<BYTES> given) {
+    constexpr uint32_t kVecs = sizeof(PolicyConst) / 16;
+    static_assert(sizeof(PolicyConst) % 16 == 0 && kPrepWarps * kVecs <= kPrepThreads, "a vector a thread");
+    __shared__ uint4 s_pol[kPrepWarps * kVecs];
+    auto table = [&](uint32_t i) {
+        if constexpr (BYTES != 0) return given.v[i];
+        else return static_cast<const uint4*>(in.host)[i];
+    };
+    // pairs policy by policy, so that a block needs few of them
+    const uint32_t pairs = P * (uint32_t)G, first = blockIdx.x * kPrepWarps, idx = first + (threadIdx.x >> 5), p0 = first / (uint32_t)G;
+    const uint32_t mine = first < pairs ? (min(first + kPrepWarps, pairs) - 1u) / (uint32_t)G - p0 + 1u : 0u;
+    const uint32_t at = blockIdx.x * kPrepThreads + threadIdx.x, all = gridDim.x * kPrepThreads, vec_at = in.skip + at;
+    uint4 pol, vec;
+    if (threadIdx.x < mine * kVecs) pol = table(p0 * kVecs + threadIdx.x);
+    if (vec_at < in.vecs) vec = table(vec_at);
+    // what the kernels behind this one must find zero
+    for (uint32_t i = at; i < clear_vecs; i += all) clear[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x < mine * kVecs) s_pol[threadIdx.x] = pol;
+    for (uint32_t i = vec_at; i < in.vecs; i += all) static_cast<uint4*>(in.device)[i] = i == vec_at ? vec : table(i);
+    __syncthreads();
+    if (BYTES == 0 && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicInc(in.left, gridDim.x - 1u) == gridDim.x - 1u) *in.read = in.turn;
+    }
+    if (idx < pairs) {
+        const uint32_t p = idx / (uint32_t)G;
+        const int g = (int)(idx - p * (uint32_t)G);
+        if (DBG_OK(g, G, DBG_K_PREP, DBG_GROUP) && DBG_OK(p - p0, kPrepWarps, DBG_K_PREP, DBG_POLICY))
+            prep_pair(reinterpret_cast<const PolicyConst*>(s_pol)[p - p0], p, g, P, gc, cum_mass, cnt, sorted, grp_off, prep);
+    }
+    // (the last blocks first: the others have clearing and preparing to do)
+    for (uint32_t i = (gridDim.x - 1u - blockIdx.x) * kPrepThreads + threadIdx.x; i < in.n_chunks[0] + in.n_chunks[1]; i += all) {
+        const int w = i >= in.n_chunks[0];
+        const uint32_t k = w ? i - in.n_chunks[0] : i, len = in.chunk_len[w];
+        uint32_t x = 0;
+        while (x + 1 < in.n_plan[w] && in.plan[w][x + 1].first <= k) ++x;
+        const ChunkPlan& pl = in.plan[w][x];
+        const uint32_t start = pl.start + (k - pl.first) * len;
+        in.chunks[w][k] = Chunk{start, min(len, pl.end - start), pl.g, 0};
+    }
+    grid_dependency_wait();
 }
 
 // The largest whole x with (double)x <= limit (>= 0, and below what Sum holds): sums are compared as whole numbers, since
@@ -300,13 +349,31 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
 
 DBG_TRANSLATION_UNIT()
 
-cudaError_t launch_prep(const PolicyConst* pol, uint32_t P, int G, const GroupConst* gc, const int64_t* cum_mass,
-                        const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep,
+cudaError_t launch_prep(uint32_t P, int G, const GroupConst* gc, const int64_t* cum_mass,
+                        const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep, const TablesIn& tables,
                         void* clear, size_t clear_bytes, int sms, cudaStream_t st) {
-    // a warp per pair, and blocks enough to clear at the speed of memory
-    const uint32_t per = kPrepThreads / 32, vecs = (uint32_t)(clear_bytes / 16);
-    const uint32_t blocks = std::max((P * (uint32_t)G + per - 1) / per, std::min((vecs + 4 * kPrepThreads - 1) / (4 * kPrepThreads), (uint32_t)sms * 8u));
-    return launch_after(k_prep, blocks, kPrepThreads, 0, st, pol, P, G, gc, cum_mass, cnt, sorted, grp_off, prep, (uint4*)clear, vecs);
+    // a warp per pair, and blocks enough to clear at the speed of memory and to read the tables at once
+    uint32_t vecs = (uint32_t)(clear_bytes / 16);
+    const uint32_t moved = std::max((vecs + 4 * kPrepThreads - 1) / (4 * kPrepThreads), (tables.vecs - tables.skip + kPrepThreads - 1) / kPrepThreads);
+    const uint32_t blocks = std::max((P * (uint32_t)G + kPrepWarps - 1) / kPrepWarps, std::min(moved, (uint32_t)sms * 8u));
+    auto go = [&](auto* kernel, const void* given) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = blocks; cfg.blockDim = kPrepThreads; cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        TablesIn in = tables;
+        uint4* at = (uint4*)clear;
+        void* args[] = {&P, &G, &gc, &cum_mass, &cnt, &sorted, &grp_off, &prep, &in, &at, &vecs, const_cast<void*>(given)};
+        return cudaLaunchKernelExC(&cfg, (const void*)kernel, args);
+    };
+    // (a launch copies the whole parameter: three sizes of it)
+    const size_t bytes = (size_t)tables.vecs * 16;
+    if (bytes <= 4096) return go(k_prep<4096>, tables.host);
+    if (bytes <= 12288) return go(k_prep<12288>, tables.host);
+    if (bytes <= kTablesInline) return go(k_prep<(int)kTablesInline>, tables.host);
+    return go(k_prep<0>, tables.host);
 }
 
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,

@@ -227,3 +227,29 @@ def test_rows_of_several_groups(n, shape):
     plain = [synth.policy(b, mig_threshold=1e-6 * k) for k, b in enumerate(synth.budget_grid(17))]
     full_parity(w, plain, select=False, tag=f"{n} {shape}")
     full_parity(w, plain[:3] + [synth.policy(0.5, flags=PACED | synth.FLAG_STOCHASTIC), synth.policy(0.3, expected_len=20)], select=False, tag=f"{n} {shape} extras")
+
+
+@pytest.mark.parametrize("n_policies", [1, 5, 31, 32, 150, 160, 400, 900])
+@pytest.mark.parametrize("beta", [False, True])
+def test_tables_of_the_policies_on_their_way(n_policies, beta):
+    # the small tables go with a launch in one of three sizes, or lie in page-locked memory; evaluations follow each other without
+    # a wait in between, so that the host must not write what a kernel has yet to read
+    import torch
+    from oracle import Oracle
+    from paper_2502_11417_b200 import Trace
+    from parity import check_prep, check_stats
+    w = synth.tiny_workload(109, 700, n_servers=2, n_devices=2, max_prompt=300, max_out=40)
+    rule = PACED | (synth.FLAG_BETA_RULE if beta else 0)
+    pols = [synth.policy(b, flags=rule if k % 3 == 0 else PACED, mig_threshold=1e-6 * (k % 2)) for k, b in enumerate(synth.budget_grid(n_policies))]
+    other = [synth.policy(0.9 - 0.001 * (k % 7), alpha=0.2) for k in range(n_policies)]
+    orc, tr = Oracle.from_workload(w), Trace.from_workload(w)
+    x = torch.randn(2048, 2048, device="cuda")
+    for _ in range(20):                            # (work in front: the evaluations below queue up behind it)
+        x = torch.tanh(x @ x)
+    for _ in range(3):
+        tr.eval_policies(other, 5)
+    tr.eval_policies(pols, w.seed)
+    stats = tr.reduce_stats()
+    check_stats(stats, orc.eval(pols, w.seed)[0], tr.histograms, f"{n_policies}")
+    check_prep(tr, orc, pols, f"{n_policies}")
+    tr.close()
