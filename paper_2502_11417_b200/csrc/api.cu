@@ -623,18 +623,50 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             return fail(DISCO_ENOMEM, "per-request TBT windows would exceed 48 GB");
     }
 
+    // ---- several classes are played out one after another and then reduced together (a wave of them), each into records of
+    //      its own as long as those take no more than 512 MB
+    const size_t N1 = n ? n : 1, n_classes = classes.size();
+    Layout slot;
+    const size_t o_ticket = slot.take(4), o_hand = slot.take(N1 * 8);
+    size_t o_rec[6] = {}, o_win[3] = {};
+    if (stored) {
+        for (int k = 0; k < 6; ++k) o_rec[k] = slot.take(N1 * 4);
+        for (int k = 0; k < 3; ++k) o_win[k] = slot.take(N1 * wmax[k] * 2);
+    }
+    const size_t rec_stride = (slot.bytes + 255) / 256 * 256;
+    const size_t wave = std::min(n_classes, std::max<size_t>(1, ((size_t)512 << 20) / rec_stride));
+    auto slot_of = [&](size_t k) { return k % wave; };
+    // A class whose free streams are those of an earlier class of its wave -- as generated, next to streams that keep the pace --
+    // has them played and stored by that class.
+    std::vector<uint32_t> kinds_of(n_classes);
+    std::vector<size_t> win_class(n_classes);
+    std::vector<FreeMore> more(n_classes);
+    for (size_t k = 0; k < n_classes; ++k) {
+        kinds_of[k] = plan[k].kinds;
+        win_class[k] = k;
+        more[k].n = 0;
+        const ClassConst& a = classes[k];
+        if (!a.pacing || (plan[k].kinds & (1u << G_GENERAL)) || !(plan[k].kinds & (1u << G_FREE))) continue;
+        for (size_t j = k - slot_of(k); j < k; ++j) {
+            const ClassConst& b = classes[j];
+            bool same = b.pacing && win_class[j] == j && more[j].n < kFreeMore && a.W[0] == b.W[0] && a.W[1] == b.W[1];
+            for (int g = 0; g < G && same; ++g) {
+                if (!rb.ng[g] || (a.kind[g] != G_FREE && b.kind[g] != G_FREE)) continue;
+                same = a.kind[g] == b.kind[g] && a.even[g] == b.even[g];
+                for (int s = 0; s < 2; ++s) same = same && (((a.even[g] >> s) & 1) || a.lo[g][s] == b.lo[g][s]);
+            }
+            if (!same) continue;
+            win_class[k] = j;
+            plan[k].kinds &= ~(1u << G_FREE);
+            more[j].tau[more[j].n] = a.tau;
+            more[j].off[more[j].n++] = (ptrdiff_t)((slot_of(k) - slot_of(j)) * rec_stride);
+            break;
+        }
+    }
     // ---- the first class's play-out needs no more than this: it runs while the host lays out the policies
     cudaError_t e;
-    const size_t N1 = n ? n : 1;
     {
-        Layout lay;
-        const size_t o_ticket = lay.take(4), o_hand = lay.take(N1 * 8);
-        size_t o_rec[6] = {}, o_win[3] = {};
-        if (stored) {
-            for (int k = 0; k < 6; ++k) o_rec[k] = lay.take(N1 * 4);
-            for (int k = 0; k < 3; ++k) o_win[k] = lay.take(N1 * wmax[k] * 2);
-        }
-        if ((e = c->rec_mem.reserve(lay.bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
+        if ((e = c->rec_mem.reserve(wave * rec_stride)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
         char* mem = (char*)c->rec_mem.p;
         c->play_ticket.p = mem + o_ticket; c->rec_hand.p = mem + o_hand;
         for (int k = 0; k < 6; ++k) c->rec_u32[k].p = mem + o_rec[k];
@@ -649,6 +681,16 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         rec.sum[k] = c->rec_u32[2 * k].as<uint32_t>(); rec.max[k] = c->rec_u32[2 * k + 1].as<uint32_t>();
         rec.win[k] = c->rec_win[k].as<uint16_t>();
     }
+    auto rec_of = [&](size_t k) {                  // a class's records
+        TimelineRec r = rec;
+        const size_t at = slot_of(k) * rec_stride, win_at = slot_of(win_class[k]) * rec_stride;
+        r.hand = (uint2*)((char*)r.hand + at);
+        for (int s = 0; s < 3; ++s) {
+            r.sum[s] = (uint32_t*)((char*)r.sum[s] + at); r.max[s] = (uint32_t*)((char*)r.max[s] + at);
+            r.win[s] = (uint16_t*)((char*)r.win[s] + win_at);
+        }
+        return r;
+    };
     const GroupConst* gc = c->d_gc.as<GroupConst>();
     uint64_t out_tokens = 0;
     for (int g = 0; g < G; ++g) out_tokens += rb.grp_sum_n[g];
@@ -659,8 +701,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const bool timed = c->timing && classes.size() == 1;
     auto play_out = [&](size_t k) {
         g_launches += timeline_launches(plan[k].kinds);
-        return launch_timeline(tr, gc, classes[k], c->knots.as<int32_t>(), k0, rec, c->err, c->play_ticket.as<uint32_t>(),
-                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, k == 0 && !timed, c->sms, st);
+        return launch_timeline(tr, gc, classes[k], c->knots.as<int32_t>(), k0, rec_of(k), c->err, c->play_ticket.as<uint32_t>(),
+                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, more[k], k == 0 && !timed, c->sms, st);
     };
     if (n != 0 && !timed) CU(play_out(0));
 
@@ -670,7 +712,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     tab.reserve((size_t)4 * P + 64);
     std::vector<Slab> slabs;
     std::vector<uint32_t> mixed_pols;              // per slab: where its policies are listed for the pair kernel (mixed slabs)
-    struct ClassLists { size_t all, n_all, ext, n_ext, slab0, slab1; };
+    struct ClassLists { size_t all, n_all, ext, n_ext; };
     std::vector<ClassLists> lists(classes.size());
     bool any_mixed = false, any_pairs = false;
     constexpr uint32_t kNone = 0xFFFFFFFFu;
@@ -692,7 +734,12 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             if ((pc[p].flags & DISCO_FLAG_BETA_RULE) && (pc[p].mode == 1 || (pc[p].mode == 0 && c->gc[g].auto_device_constrained)))
                 tab.push_back((uint32_t)g * P + p);
     const uint32_t n_beta = (uint32_t)(tab.size() - beta_at);
-    for (size_t k = 0; k < classes.size(); ++k) {
+    // (in a wave, the classes without windows first: their slabs go through the grid kernel together)
+    auto wide_class = [&](size_t k) { return (kinds_of[k] & ~(1u << G_EXACT)) != 0; };
+    std::vector<size_t> order(n_classes);
+    std::iota(order.begin(), order.end(), (size_t)0);
+    std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) { return x / wave != y / wave ? x / wave < y / wave : wide_class(x) < wide_class(y); });
+    for (size_t k : order) {
         ClassLists& L = lists[k];
         L.all = tab.size();
         if (classes.size() == 1) {
@@ -703,7 +750,6 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         }
         L.n_all = tab.size() - L.all;
         L.ext = tab.size();
-        L.slab0 = slabs.size();
         grids.clear();
         Grid* last = nullptr;
         for (size_t i = L.all; i < L.all + L.n_all; ++i) {
@@ -730,6 +776,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             auto open = [&](int T, bool mixed) {
                 Slab sl;
                 std::memset(&sl, 0, sizeof sl);
+                sl.cls = (uint32_t)k; sl.slot = (uint32_t)slot_of(k); sl.win_slot = (uint32_t)slot_of(win_class[k]);
+                sl.bin_tau = host_bin_of_ticks(classes[k].tau);
                 sl.T = T; sl.expected_len = gr.expected_len; sl.mixed = mixed ? 1 : 0;
                 sl.mig = (gr.flags & DISCO_FLAG_MIGRATION) ? 1 : 0;
                 return sl;
@@ -795,8 +843,33 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 for (size_t c0 = 0; c0 < cols; c0 += kGridCols) close(sl, c0, std::min(cols, c0 + (size_t)kGridCols), 0u);
             }
         }
-        L.slab1 = slabs.size();
     }
+
+    // ---- the difference tables of the slabs, laid out batch by batch: a batch's slabs have like numbers of rows, and windows or
+    //      none.  Small ones lie side by side and are cleared by k_prep; beyond 64 MB a batch's tables are cleared, filled,
+    //      added up and then belong to the next batch
+    struct Batch { size_t first, count, wave; int T; bool wide; uint64_t ttft, tbt, sums, at; };
+    std::vector<Batch> batches;
+    auto batch_bytes = [&](const Batch& b) { return (b.sums * 8 + b.tbt * (b.wide ? 8 : 4) + b.ttft * 4 + 15) / 16 * 16; };
+    size_t most_slabs = 1;
+    for (size_t x = 0; x < slabs.size(); ++x) {
+        Slab& sl = slabs[x];
+        const bool wide_tables = wide_class(sl.cls);
+        if (batches.empty() || batch_bytes(batches.back()) > (256ull << 20) || grid_rows(batches.back().T) != grid_rows(sl.T) || sl.mixed ||
+            slabs[x - 1].mixed || batches.back().wave != sl.cls / wave || batches.back().wide != wide_tables)
+            batches.push_back(Batch{x, 0, sl.cls / wave, 1, wide_tables, 0, 0, 0, 0});
+        Batch& b = batches.back();
+        sl.ttft = b.ttft; sl.tbt = b.tbt; sl.sums = b.sums;
+        b.ttft += grid_ttft_words(sl.K); b.tbt += grid_tbt_words(sl.K, sl.T); b.sums += grid_sum_words(sl.K, sl.T, G);
+        ++b.count;
+        b.T = std::max(b.T, sl.T);
+        most_slabs = std::max(most_slabs, b.count);
+    }
+    uint64_t grid_bytes = 0, all_bytes = 0;
+    for (Batch& b : batches) { b.at = all_bytes; all_bytes += batch_bytes(b); grid_bytes = std::max(grid_bytes, batch_bytes(b)); }
+    const bool side_by_side = all_bytes <= (64ull << 20);
+    if (side_by_side) grid_bytes = all_bytes;
+    else for (Batch& b : batches) b.at = 0;
 
     // ---- request chunks, of one group each: of the grid kernel, about two to each block that fits the GPU at once, 256
     //      requests (one a thread) or more (three to a block: k_grid and k_spread for 16 M requests in six groups under 128
@@ -825,45 +898,17 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         tables.chunk_len[which] = CH; tables.n_chunks[which] = count;
     };
     const size_t at_once = (size_t)sms * grid_blocks_per_sm(tallest);
-    plan_chunks(0, chunk_size(2 * at_once, 256));
+    plan_chunks(0, chunk_size(std::max<size_t>(2 * at_once / std::min<size_t>(most_slabs, 4), 1), 256));
     if (any_pairs) plan_chunks(1, chunk_size((size_t)2 * sms, 2048));
-
-    // ---- the difference tables of the slabs, laid out batch by batch: a batch's slabs have like numbers of rows and share
-    //      one class; its tables are cleared, filled, added up and then belong to the next batch
-    struct Batch { size_t first, count; int T; uint64_t ttft, tbt, sums; };
-    std::vector<std::vector<Batch>> batches(classes.size());
-    uint64_t grid_bytes = 0;
-    auto wide_class = [&](size_t k) { return (plan[k].kinds & ~(1u << G_EXACT)) != 0; };
-    uint32_t n_tickets = 0;
-    for (size_t k = 0; k < classes.size(); ++k) {
-        const uint64_t tbt_word = wide_class(k) ? 8 : 4;
-        for (size_t x = lists[k].slab0; x < lists[k].slab1; ++x) {
-            Slab& sl = slabs[x];
-            auto bytes = [&](const Batch& b) { return b.ttft * 4 + b.tbt * tbt_word + b.sums * 8; };
-            std::vector<Batch>& bs = batches[k];
-            if (bs.empty() || bytes(bs.back()) > (256ull << 20) || grid_rows(bs.back().T) != grid_rows(sl.T) || sl.mixed || slabs[x - 1].mixed)
-                bs.push_back(Batch{x, 0, 1, 0, 0, 0});
-            Batch& b = bs.back();
-            sl.ttft = b.ttft; sl.tbt = b.tbt; sl.sums = b.sums;
-            b.ttft += grid_ttft_words(sl.K); b.tbt += grid_tbt_words(sl.K, sl.T); b.sums += grid_sum_words(sl.K, sl.T, G);
-            ++b.count;
-            b.T = std::max(b.T, sl.T);
-            grid_bytes = std::max(grid_bytes, bytes(b) + 64);
-        }
-        n_tickets += (uint32_t)batches[k].size();
-    }
 
     // ---- device memory: what must be clear comes first and together -- the work counters and tickets, the difference
     //      tables of the first batch, and the accumulators if some pairs are added to them one by one (k_spread writes those
     //      of all other policies)
     const size_t acc_bytes = (size_t)P * G * kNAcc * 8, hist_bytes = (size_t)P * kNBins * 8;
-    auto batch_bytes = [&](const Batch& b, bool wide) { return b.sums * 8 + b.tbt * (wide ? 8 : 4) + b.ttft * 4; };
-    size_t first_bytes = 0;
-    for (size_t k = 0; k < classes.size() && first_bytes == 0; ++k)
-        if (!batches[k].empty()) first_bytes = batch_bytes(batches[k][0], wide_class(k));
+    const size_t first_bytes = side_by_side ? all_bytes : batches.empty() ? 0 : batch_bytes(batches[0]);
     const bool clear_accum = any_pairs || n == 0;
     Layout lay;
-    const size_t o_work = lay.take(32 + (size_t)n_tickets * 4), o_accum = clear_accum ? lay.take(acc_bytes + 2 * hist_bytes) : 0;
+    const size_t o_work = lay.take(32 + batches.size() * 4), o_accum = clear_accum ? lay.take(acc_bytes + 2 * hist_bytes) : 0;
     const size_t o_grid = lay.bytes;
     lay.take(grid_bytes);
     const size_t clear_bytes = n == 0 ? o_grid : (o_grid + first_bytes + 15) / 16 * 16;      // (k_prep clears them)
@@ -936,57 +981,55 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const Prep* prep = c->d_prep.as<Prep>();
     uint64_t *acc = c->d_acc.as<uint64_t>(), *h_ttft = c->d_hist_ttft.as<uint64_t>(), *h_tbt = c->d_hist_tbt.as<uint64_t>(),
              *work = c->d_work.as<uint64_t>();
-    bool first_batch = true;
-    // ---- per timeline class: play every request out, then evaluate the class's policies on the summaries
-    for (size_t k = 0; k < classes.size() && n != 0; ++k) {
-        const ClassConst* dcc = d_classes + k;
-        const bool wide = wide_class(k);
+    size_t next = 0;                               // batch
+    // ---- wave by wave: play every request out under the wave's classes, then evaluate their policies on the summaries
+    for (size_t first = 0; first < n_classes && n != 0; first += wave) {
+        const size_t last = std::min(n_classes, first + wave);
         if (timed) CU(cudaEventRecord(c->ev[0], st));
-        if (k != 0 || timed) CU(play_out(k));
+        for (size_t k = first; k < last; ++k)
+            if (k != 0 || timed) CU(play_out(k));
         if (timed) CU(cudaEventRecord(c->ev[2], st));
-        for (const Batch& b : batches[k]) {
+        for (; next < batches.size() && batches[next].wave == first / wave; ++next) {
+            const Batch& b = batches[next];
             GridTables gt;
-            const size_t tbt_word = wide ? 8 : 4;
-            char* base = (char*)c->d_grid.p;
+            char* base = (char*)c->d_grid.p + b.at;
             gt.sums = (unsigned long long*)base;
             gt.tbt = base + b.sums * 8;
-            gt.ttft = (uint32_t*)(base + b.sums * 8 + b.tbt * tbt_word);
-            if (!first_batch) CU(cudaMemsetAsync(base, 0, batch_bytes(b, wide), st));
-            first_batch = false;
+            gt.ttft = (uint32_t*)(base + b.sums * 8 + b.tbt * (b.wide ? 8 : 4));
+            if (!side_by_side && next != 0) CU(cudaMemsetAsync(base, 0, batch_bytes(b), st));
             const Slab* dsl = d_slabs + b.first;
-            const bool mixed = slabs[b.first].mixed != 0;
+            const Slab& sl = slabs[b.first];
             LeftLists left = {nullptr, nullptr};
-            if (mixed) {
+            if (sl.mixed) {
                 left.list = c->d_left.as<uint32_t>(); left.count = left.list + N1;
                 CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
             }
-            CU(launch_grid(tr, gc, dcc, prep, P, dsl, (uint32_t)b.count, b.T, wide, d_tab,
-                           d_chunks, tables.n_chunks[0], rec, gt, left, k0, tickets + ticket++, work, c->sms, st));
-            CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, wide, host_bin_of_ticks(classes[k].tau), d_tab, gt, acc,
-                             h_ttft, h_tbt, st));
+            CU(launch_grid(tr, gc, d_classes, prep, P, dsl, (uint32_t)b.count, b.T, b.wide, d_tab,
+                           d_chunks, tables.n_chunks[0], rec, rec_stride, gt, left, k0, tickets + ticket++, work, c->sms, st));
+            CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, b.wide, d_tab, gt, acc, h_ttft, h_tbt, st));
             g_launches += 2;
-            if (mixed) {
-                const Slab& sl = slabs[b.first];
-                CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + mixed_pols[b.first], sl.policies, d_pair_chunks,
-                                    tables.n_chunks[1], left.list, left.count, rec, acc, h_ttft, h_tbt, work, k0,
-                                    sl.expected_len != 0, wide, st));
+            if (sl.mixed) {
+                CU(launch_pairs_acc(tr, gc, d_classes + sl.cls, prep, P, d_tab + mixed_pols[b.first], sl.policies, d_pair_chunks,
+                                    tables.n_chunks[1], left.list, left.count, rec_of(sl.cls), acc, h_ttft, h_tbt, work, k0,
+                                    sl.expected_len != 0, b.wide, st));
                 g_launches += 1;
             }
         }
-        if (lists[k].n_ext) {
-            CU(launch_pairs_acc(tr, gc, dcc, prep, P, d_tab + lists[k].ext, (uint32_t)lists[k].n_ext,
-                                d_pair_chunks, tables.n_chunks[1], nullptr, nullptr, rec, acc, h_ttft, h_tbt,
-                                work, k0, true, wide, st));
+        for (size_t k = first; k < last; ++k) {
+            if (!lists[k].n_ext) continue;
+            CU(launch_pairs_acc(tr, gc, d_classes + k, prep, P, d_tab + lists[k].ext, (uint32_t)lists[k].n_ext,
+                                d_pair_chunks, tables.n_chunks[1], nullptr, nullptr, rec_of(k), acc, h_ttft, h_tbt,
+                                work, k0, true, wide_class(k), st));
             g_launches += 1;
         }
         if (timed) CU(cudaEventRecord(c->ev[3], st));
-        if (rows) {
+        for (size_t k = first; k < last && rows; ++k) {
             if (!c->inv_there) {
                 CU(launch_inverse(tr, c->inv.as<uint32_t>(), st));
                 g_launches += 1;
                 c->inv_there = true;
             }
-            CU(launch_pairs_rows(tr, gc, dcc, prep, P, d_tab + lists[k].all, (uint32_t)lists[k].n_all, rec, po, k0, extras, st));
+            CU(launch_pairs_rows(tr, gc, d_classes + k, prep, P, d_tab + lists[k].all, (uint32_t)lists[k].n_all, rec_of(k), po, k0, extras, st));
             g_launches += 1;
         }
         if (timed) CU(cudaEventRecord(c->ev[4], st));

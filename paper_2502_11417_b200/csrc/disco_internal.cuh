@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "disco.h"
@@ -258,6 +259,9 @@ cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* 
                              const uint32_t* tick_start, const uint32_t* tick_cnt /* [G][kTickBins], of the sorted ticks */,
                              const uint32_t* pairs /* [n_pairs]: g P + p */, uint32_t n_pairs,
                              uint64_t most /* ticks of a group, at most */, Prep* prep, cudaStream_t st);
+// Further classes whose free streams are the same (api.cu): the play-out writes their summaries as well, so many bytes from its own.
+constexpr int kFreeMore = 8;
+struct FreeMore { int n; int32_t tau[kFreeMore]; ptrdiff_t off[kFreeMore]; };
 // Plays every request under one class.  `kinds`: bit k set if some group with requests is of GroupKind k; `batches[k]`:
 // batches of 32 requests of the groups of kind k.
 cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0 /* hash key base: seed_key(seed) + first_index * kHashReq */,
@@ -265,7 +269,7 @@ cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const Clas
                             const uint32_t* batches, uint32_t search /* largest ClassConst::search of a group with requests */,
                             bool long_outputs /* mean output length of 512 tokens or more */,
                             cudaEvent_t mid /* recorded between the kernels of exact groups and the others, or null */,
-                            bool early /* the preparation follows: it may start beside the last kernel */,
+                            const FreeMore& more, bool early /* the preparation follows: it may start beside the last kernel */,
                             int sms /* multiprocessors of the device */, cudaStream_t st);
 uint32_t timeline_launches(uint32_t kinds);
 
@@ -281,6 +285,8 @@ struct Slab {
     uint32_t policies;           // how many they are
     int32_t mixed;               // a column per policy, whose overheads lie between theta[0] and theta[1] (T = 1):
                                  // requests whose saving lies between the two are left to the pair kernel
+    uint32_t cls, slot, win_slot;  // its class, where the class's records lie, and its windows (both in places of rec_stride bytes)
+    int32_t bin_tau;             // the bin of the class's pace
     float theta[kGridRows];
     // 32- or 64-bit words in front of the slab's difference tables, see grid.cu
     uint64_t ttft, tbt, sums;
@@ -290,13 +296,13 @@ struct LeftLists { uint32_t* list; uint32_t* count; };   // [slabs][n] places in
 uint64_t grid_ttft_words(int K), grid_tbt_words(int K, int T), grid_sum_words(int K, int T, int G);
 uint32_t grid_blocks_per_sm(int T);
 int grid_rows(int T);            // rows the kernel that takes such a slab is built for
-cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
-                        const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide,
-                        const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt,
+cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* classes, const Prep* prep, uint32_t P,
+                        const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide /* of all of them */,
+                        const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec /* of slot 0 */, size_t rec_stride, GridTables gt,
                         LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t k0, uint32_t* ticket /* zero */,
                         uint64_t* work /* [4], added to */, int sms, cudaStream_t st);
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
-                          bool wide, int bin_tau, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
+                          bool wide, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
                           uint64_t* hist_tbt, cudaStream_t st);
 // Pair by pair: `n_list` policies under the chunks' requests, or (list not null) under the listed ones.
 cudaError_t launch_pairs_acc(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,

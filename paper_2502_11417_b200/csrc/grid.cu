@@ -92,13 +92,17 @@ struct Ctx {                                           // a (chunk, slab)
     float th_lo;                                       // mixed: smallest overhead
     int E0, x_from;
     uint32_t even;
+    const ClassConst* cc;
+    const uint2* hand;
+    size_t win_at;                                     // bytes from the windows of slot 0
 };
 
 struct Args {
     TraceDev tr;
     TimelineRec rec;
     const GroupConst* gcs;
-    const ClassConst* cc;
+    size_t rec_stride;
+    const ClassConst* classes;
     const Prep* prep;
     uint32_t P;
     const Slab* slabs;
@@ -161,21 +165,22 @@ __device__ __forceinline__ void add_rows(const uint16_t* __restrict__ win, int W
 // every row of the grid but those that migrate, [0, t), which get the stream after the hand-off.
 __device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_t* tbt, bool valid, uint32_t kk, bool device, int t,
                                             uint32_t orig) {
-    const ClassConst& cc = *a.cc;
+    const ClassConst& cc = *c.cc;
+    const auto win = [&](int s) { return reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(a.rec.win[s]) + c.win_at); };
     uint32_t* all = tbt + (c.T - 1) * kNBins;
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
         if ((c.even >> s) & 1u) continue;
         const bool mine = valid && (int)device == s;
         const int W = cc.W[s], lo = cc.lo[c.g][s];
-        add_rows(a.rec.win[s], W, lo, __ballot_sync(FULL, mine && t < c.T), kk, false, all);
+        add_rows(win(s), W, lo, __ballot_sync(FULL, mine && t < c.T), kk, false, all);
         for (int r = 1; r < c.T; ++r)
-            add_rows(a.rec.win[s], W, lo, __ballot_sync(FULL, mine && t == r), kk, true, tbt + (r - 1) * kNBins);
+            add_rows(win(s), W, lo, __ballot_sync(FULL, mine && t == r), kk, true, tbt + (r - 1) * kNBins);
     }
     if (c.even & 4u) return;
     const int from = c.x_from >= 0 ? c.x_from : 2;
     for (int r = 1; r <= c.T; ++r)
-        add_rows(a.rec.win[from], cc.W[from], cc.lo[c.g][from], __ballot_sync(FULL, valid && t == r), kk, false, tbt + (r - 1) * kNBins);
+        add_rows(win(from), cc.W[from], cc.lo[c.g][from], __ballot_sync(FULL, valid && t == r), kk, false, tbt + (r - 1) * kNBins);
     if (c.x_from >= 0 && valid && t > 0) {
         const int bin = first_bin(a.gcs[c.g], c.x_from, a.k0, orig);
         if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) atomicSub(&tbt[(t - 1) * kNBins + bin], 1u);
@@ -202,7 +207,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
         const uint32_t i = min(i0 + lane, pb - 1);
         at = list ? (uint32_t)sm.list[i] : i;
         to = a.tr.req[c.start + at];
-        to_hand = c.may_migrate ? a.rec.hand[c.start + at] : make_uint2(0u, 0u);
+        to_hand = c.may_migrate ? c.hand[c.start + at] : make_uint2(0u, 0u);
     };
     const uint32_t first = pa + (threadIdx.x & ~31u);
     if (kAhead && first < pb) fetch(first, ahead, q_ahead, hand_ahead);
@@ -231,7 +236,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
                 } else if (valid) hist_add(sm.only_ttft, bin);
                 if (!WIDE && valid) o.bins |= 1u << (bin >> 5);
                 if (valid) { o.cnt += 1u; o.n += n; o.l += l; o.tt += Td; o.tau += (!WIDE || (c.even & 2u)) ? n - 1u : 0u; }
-                if (WIDE && !(c.even & 2u)) add_rows(a.rec.win[1], a.cc->W[1], a.cc->lo[c.g][1], live, kk, false, tbt + NT * kNBins);
+                if (WIDE && !(c.even & 2u)) add_rows(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(a.rec.win[1]) + c.win_at), c.cc->W[1], c.cc->lo[c.g][1], live, kk, false, tbt + NT * kNBins);
             }
             if (!race) continue;
         }
@@ -455,7 +460,7 @@ __device__ __noinline__ void enter_requests(const Args& a, const Ctx& c, const f
     for (uint32_t i = threadIdx.x; i < c.len; i += kThreads) {
         const uint32_t kk = c.start + i;
         const uint4 q = a.tr.req[kk];
-        const uint2 hand = c.may_migrate ? a.rec.hand[kk] : make_uint2(0u, 0u);
+        const uint2 hand = c.may_migrate ? c.hand[kk] : make_uint2(0u, 0u);
         const uint32_t S = q.x, l = q.y & 0xFFFFu, n = q.y >> 16, m = hand.x & 0xFFFFu, dly = hand.x >> 16;
         const uint32_t Td = c.kappa * l + c.c0;
         const float saving = m ? c.delta_c * (float)(c.E0 ? max(c.E0 - (int)m, 0) : (int)(n - m)) : -1.0f;
@@ -543,8 +548,11 @@ k_grid(const __grid_constant__ Args a) {
         c.delta_c = gc.delta_c; c.cand = gc.candidate; c.g = g; c.K = sl.K; c.T = sl.T;
         c.may_migrate = sl.mig && gc.candidate != 0;
         c.mixed = sl.mixed && c.may_migrate;
-        c.E0 = (int)sl.expected_len; c.even = a.cc->even[g];
-        c.x_from = x_stream(*a.cc, gc);
+        c.cc = a.classes + sl.cls;
+        c.hand = reinterpret_cast<const uint2*>(reinterpret_cast<const char*>(a.rec.hand) + sl.slot * a.rec_stride);
+        c.win_at = sl.win_slot * a.rec_stride;
+        c.E0 = (int)sl.expected_len; c.even = c.cc->even[g];
+        c.x_from = x_stream(*c.cc, gc);
         float th[NT];                                                  // rows beyond the slab's never migrate
 #pragma unroll
         for (int r = 0; r < NT; ++r) th[r] = (c.may_migrate && r < c.T) ? sl.theta[sl.mixed ? 1 : r] : __int_as_float(0x7F800000);
@@ -567,7 +575,7 @@ k_grid(const __grid_constant__ Args a) {
             for (uint32_t i0 = threadIdx.x & ~31u; i0 < ch.len; i0 += kThreads) {
                 const uint32_t i = min(i0 + (threadIdx.x & 31), ch.len - 1), kk = ch.start + i;
                 const uint4 q = a.tr.req[kk];
-                const uint32_t m = a.rec.hand[kk].x & 0xFFFFu, n = q.y >> 16;
+                const uint32_t m = c.hand[kk].x & 0xFFFFu, n = q.y >> 16;
                 const float saving = m ? c.delta_c * (float)(c.E0 ? max(c.E0 - (int)m, 0) : (int)(n - m)) : -1.0f;
                 const bool out = i0 + (threadIdx.x & 31) < ch.len && saving > c.th_lo && !(saving > th[0]);
                 const uint32_t all = __ballot_sync(FULL, out);
@@ -750,13 +758,13 @@ __device__ __forceinline__ void spread_columns(unsigned long long* s_part, int K
 
 template <bool WIDE>
 __global__ void __launch_bounds__(kSpreadWarps * 32)
-k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict__ slabs, int bin_tau,
+k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict__ slabs,
          const uint32_t* __restrict__ tab, GridTables gt, unsigned long long* __restrict__ acc,
          unsigned long long* __restrict__ hist_ttft, unsigned long long* __restrict__ hist_tbt) {
     __shared__ unsigned long long s_part[kSpreadWarps * 33];
     grid_dependency_wait();
     const Slab& sl = slabs[blockIdx.y];
-    const int K = sl.K, T = sl.T, lane = threadIdx.x & 31;
+    const int K = sl.K, T = sl.T, bin_tau = sl.bin_tau, lane = threadIdx.x & 31;
     const Tables<WIDE> tb(gt, sl, tr.n_groups);
     using word = typename Tables<WIDE>::word;
     const uint32_t* cells = tab + sl.cells;
@@ -840,13 +848,13 @@ uint64_t grid_sum_words(int K, int T, int G) { return (uint64_t)G * K * sum_fiel
 uint32_t grid_blocks_per_sm(int T) { return (uint32_t)blocks_for(rows_for(T), false); }
 int grid_rows(int T) { return rows_for(T); }
 
-cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
+cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* classes, const Prep* prep, uint32_t P,
                         const Slab* slabs, uint32_t n_slabs, int T, bool wide, const uint32_t* tab,
-                        const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, GridTables gt, LeftLists left,
+                        const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, size_t rec_stride, GridTables gt, LeftLists left,
                         uint32_t k0, uint32_t* ticket, uint64_t* work, int sms, cudaStream_t st) {
     if (n_chunks == 0 || n_slabs == 0) return cudaSuccess;
     if ((uint64_t)n_chunks * n_slabs > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    const Args a = {tr, rec, gc, cc, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, k0, ticket,
+    const Args a = {tr, rec, gc, rec_stride, classes, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, k0, ticket,
                     (unsigned long long*)work};
     switch (rows_for(T)) {
         case 1: return wide ? launch_one<1, true>(a, sms, st) : launch_one<1, false>(a, sms, st);
@@ -857,12 +865,12 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
 }
 
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
-                          bool wide, int bin_tau, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
+                          bool wide, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
                           uint64_t* hist_tbt, cudaStream_t st) {
     if (n_slabs == 0) return cudaSuccess;
     const dim3 grid((uint32_t)(2 * T * (kNBins / 32) + (tr.n_groups * T * kNAcc + 31) / 32), n_slabs);
     auto* kernel = wide ? k_spread<true> : k_spread<false>;
-    return launch_after(kernel, grid, kSpreadWarps * 32, 0, st, tr, gc, slabs, bin_tau, tab, gt, (unsigned long long*)acc,
+    return launch_after(kernel, grid, kSpreadWarps * 32, 0, st, tr, gc, slabs, tab, gt, (unsigned long long*)acc,
                         (unsigned long long*)hist_ttft, (unsigned long long*)hist_tbt);
 }
 

@@ -38,7 +38,7 @@ __device__ __forceinline__ void count_in(const Counters& c, uint32_t x, uint32_t
 template <bool BOTH, bool SMALL>
 __global__ void __launch_bounds__(kFreeWarps * 32, 4)
 k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
-               const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, bool early) {
+               const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, const __grid_constant__ FreeMore more, bool early) {
     extern __shared__ __align__(16) uint32_t s_win[];         // per warp: [W0 + W1][32] counters
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warps = blockDim.x >> 5;
     grid_dependency_wait();
@@ -143,6 +143,14 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
             rec.sum[0][k] = sum0; rec.sum[1][k] = sum1; rec.sum[2][k] = sumX;
             rec.max[0][k] = nI ? (on0 ? most0 : tau) : 0u; rec.max[1][k] = nI ? (on1 ? most1 : tau) : 0u;
             rec.max[2][k] = maxX;
+            // classes that differ in the pace alone: the same intervals, another pace beside them, and no hand-off either
+            for (int c = 0; !BOTH && c < more.n; ++c) {
+                const uint32_t pace = (uint32_t)more.tau[c];
+                auto put = [&](uint32_t* at, uint32_t v) { *reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(at + k) + more.off[c]) = v; };
+                *reinterpret_cast<uint2*>(reinterpret_cast<char*>(rec.hand + k) + more.off[c]) = make_uint2(0u, 0u);
+                put(rec.sum[0], on0 ? sum0 : nI * pace); put(rec.sum[1], on1 ? sum1 : nI * pace); put(rec.sum[2], 0u);
+                put(rec.max[0], nI ? (on0 ? most0 : pace) : 0u); put(rec.max[1], nI ? (on1 ? most1 : pace) : 0u); put(rec.max[2], 0u);
+            }
         }
         __syncwarp();
     }
@@ -152,7 +160,7 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
 
 DBG_TRANSLATION_UNIT()
 
-cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0, TimelineRec rec, uint32_t batches, bool early, int sms,
+cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0, TimelineRec rec, const FreeMore& more, uint32_t batches, bool early, int sms,
                                 cudaStream_t st) {
     // as many warps to a block as the windows leave room for (wide jitter: up to 114 KB of counters a stream and warp)
     const size_t per_warp = (size_t)(cc.W[0] + cc.W[1]) * 32 * 4;
@@ -166,7 +174,7 @@ cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const 
     if ((e = allow_smem((const void*)kernel, 227 * 1024))) return e;
     // (batches counts 32 requests each; four blocks of eight warps fit a multiprocessor)
     const uint32_t blocks = std::min<uint32_t>((batches * (32 / kFreeBatch) + warps - 1) / warps, (uint32_t)sms * 4u * kFreeWarps / warps);
-    return launch_after(kernel, blocks, warps * 32, smem, st, tr, gc, cc, knots, k0, rec, early);
+    return launch_after(kernel, blocks, warps * 32, smem, st, tr, gc, cc, knots, k0, rec, more, early);
 }
 
 }  // namespace disco
