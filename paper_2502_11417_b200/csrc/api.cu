@@ -702,7 +702,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     auto play_out = [&](size_t k) {
         g_launches += timeline_launches(plan[k].kinds);
         return launch_timeline(tr, gc, classes[k], c->knots.as<int32_t>(), k0, rec_of(k), c->err, c->play_ticket.as<uint32_t>(),
-                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, more[k], k == 0 && !timed, c->sms, st);
+                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, more[k], &c->z->free_ticket, rb.ng, k == 0 && !timed, c->sms, st);
     };
     if (n != 0 && !timed) CU(play_out(0));
 

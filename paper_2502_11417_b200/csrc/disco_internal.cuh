@@ -269,7 +269,7 @@ cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const Clas
                             const uint32_t* batches, uint32_t search /* largest ClassConst::search of a group with requests */,
                             bool long_outputs /* mean output length of 512 tokens or more */,
                             cudaEvent_t mid /* recorded between the kernels of exact groups and the others, or null */,
-                            const FreeMore& more, bool early /* the preparation follows: it may start beside the last kernel */,
+                            const FreeMore& more, uint32_t* free_ticket /* one word, zero before and after */, const uint32_t* grp_n /* requests per group, on the host */, bool early /* the preparation follows: it may start beside the last kernel */,
                             int sms /* multiprocessors of the device */, cudaStream_t st);
 uint32_t timeline_launches(uint32_t kinds);
 

@@ -35,7 +35,7 @@ struct LoadZero {
     uint32_t grp_n[kMaxGroups];           // requests per group (load_large.cu)
     uint32_t max_n;                       // longest output
     uint32_t barrier, done;
-    uint32_t tables_left;                 // k_prep's (no load touches it)
+    uint32_t tables_left, free_ticket, pad[3];    // k_prep's and k_playout_free's, zero between their launches (no load touches them)
     int32_t err[4];                       // code, request index, window flag, sort flag (1: some bin needs the fallback, 2: a
                                           // wait between blocks ran out)
 };

@@ -269,3 +269,17 @@ def test_classes_that_are_reduced_together(n, rates):
     more = [synth.policy(0.4, r_c=rates[0], flags=synth.FLAG_MIGRATION), synth.policy(0.4, r_c=rates[-1], flags=PACED | synth.FLAG_STOCHASTIC),
             synth.policy(0.6, r_c=rates[-1], flags=synth.FLAG_PACING), synth.policy(0.6, r_c=rates[1], flags=PACED | synth.FLAG_BETA_RULE, l_immediate=64)]
     full_parity(w, pols[::-1] + more, select=False, tag=f"{rates} and others")
+
+
+@pytest.mark.parametrize("n", [1, 3, 9000, 30001])
+@pytest.mark.parametrize("jitter", [0.0, 0.2])
+@pytest.mark.parametrize("rate", [None, 12.0, 40.0])
+def test_streams_delivered_as_they_are_generated(n, jitter, rate):
+    # without pacing, with a slow device beside a server that keeps the pace, and with both endpoints slower than the reader or one of
+    # them by groups: batches of two requests and more, partly filled, groups that are not played here between others
+    w = synth.tiny_workload(127 + n, n, n_servers=2, n_devices=2, max_prompt=200, max_out=70)
+    w.output_len[::17] = 900                       # (several rounds of a warp)
+    w.servers = [synth.server(tbt_s=0.03, jitter=jitter), synth.server(tbt_s=0.045, jitter=jitter / 4)]
+    w.devices = [synth.device(1500.0, 40.0, jitter=0.05), synth.device(200.0, 10.0, jitter=jitter / 2, c_prefill=5e-3, c_decode=5e-3)]
+    flags = synth.FLAG_MIGRATION | (synth.FLAG_PACING if rate else 0)
+    full_parity(w, [synth.policy(b, r_c=rate or 5.0, flags=flags) for b in (0.3, 0.8)], select=False, tag=f"{n} {jitter} {rate}")
