@@ -964,10 +964,12 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                    c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), tables, mem, clear_apart ? 0 : clear_bytes, c->sms, st));
     if (!in_launch) ++c->stage_turn;
     g_launches += 1;
+    // (one class, played out already, and a grid: the search's results are not needed before the pair kernel)
+    const bool beside = n_beta && n_classes == 1 && n != 0 && !timed && !batches.empty() && !slabs[0].mixed;
     if (n_beta) {
         CU(launch_prep_beta(d_pol, P, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
                             c->F_off, c->tick_start.as<uint32_t>(), c->tick_cnt, d_tab + beta_at, n_beta,
-                            *std::max_element(c->F_n.begin(), c->F_n.end()), c->d_prep.as<Prep>(), st));
+                            *std::max_element(c->F_n.begin(), c->F_n.end()), c->d_prep.as<Prep>(), beside, st));
         g_launches += 1;
     }
 
@@ -1005,7 +1007,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
             }
             CU(launch_grid(tr, gc, d_classes, prep, P, dsl, (uint32_t)b.count, b.T, b.wide, d_tab,
-                           d_chunks, tables.n_chunks[0], rec, rec_stride, gt, left, k0, tickets + ticket++, work, c->sms, st));
+                           d_chunks, tables.n_chunks[0], rec, rec_stride, gt, left, k0, tickets + ticket, work, beside && ticket == 0, c->sms, st));
+            ++ticket;
             CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, b.wide, d_tab, gt, acc, h_ttft, h_tbt, st));
             g_launches += 2;
             if (sl.mixed) {

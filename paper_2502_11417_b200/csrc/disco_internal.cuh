@@ -258,7 +258,8 @@ cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* 
                              const int32_t* sorted, const uint32_t* grp_off,
                              const uint32_t* tick_start, const uint32_t* tick_cnt /* [G][kTickBins], of the sorted ticks */,
                              const uint32_t* pairs /* [n_pairs]: g P + p */, uint32_t n_pairs,
-                             uint64_t most /* ticks of a group, at most */, Prep* prep, cudaStream_t st);
+                             uint64_t most /* ticks of a group, at most */, Prep* prep, bool early /* the grid kernel follows: it may start beside */,
+                             cudaStream_t st);
 // Further classes whose free streams are the same (api.cu): the play-out writes their summaries as well, so many bytes from its own.
 constexpr int kFreeMore = 8;
 struct FreeMore { int n; int32_t tau[kFreeMore]; ptrdiff_t off[kFreeMore]; };
@@ -300,7 +301,7 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
                         const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide /* of all of them */,
                         const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec /* of slot 0 */, size_t rec_stride, GridTables gt,
                         LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t k0, uint32_t* ticket /* zero */,
-                        uint64_t* work /* [4], added to */, int sms, cudaStream_t st);
+                        uint64_t* work /* [4], added to */, bool beside /* runs beside its predecessor, whose own it has complete */, int sms, cudaStream_t st);
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
                           bool wide, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
                           uint64_t* hist_tbt, cudaStream_t st);

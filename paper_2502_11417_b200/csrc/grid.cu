@@ -115,6 +115,7 @@ struct Args {
     uint32_t k0;
     uint32_t* ticket;
     unsigned long long* work;
+    bool beside;
 };
 
 __device__ __forceinline__ void hist_add(uint32_t* h, int bin) {
@@ -521,7 +522,10 @@ k_grid(const __grid_constant__ Args a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
     uint32_t* tbt = (uint32_t*)(smem_raw + sizeof(Smem));
-    grid_dependency_wait();
+    // Beside the slope search of Eq. 1-2 (k_prep_beta), which no plain policy needs: what this kernel reads was complete before that
+    // one let it start.  It then waits at its end, for the kernels behind.  (Under 48 such searches, 79 us on 48
+    // multiprocessors, 300,000 requests by 16 budgets take 27.)
+    if (!a.beside) grid_dependency_wait();
     for (int i = threadIdx.x; i < (int)(offsetof(Smem, key) / 4); i += kThreads) ((uint32_t*)&sm)[i] = 0;
     for (int i = threadIdx.x; i < (NT + (WIDE ? 1 : 0)) * kNBins; i += kThreads) tbt[i] = 0;
 
@@ -717,6 +721,7 @@ k_grid(const __grid_constant__ Args a) {
             atomicAdd(&a.work[3], (unsigned long long)passes);         // sweeps over segments
         }
     }
+    if (a.beside) grid_dependency_wait();
 }
 
 // Adds up the difference rows: what a policy gets is the sum of the rows up to its column.  A block takes 32 histogram
@@ -851,11 +856,11 @@ int grid_rows(int T) { return rows_for(T); }
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* classes, const Prep* prep, uint32_t P,
                         const Slab* slabs, uint32_t n_slabs, int T, bool wide, const uint32_t* tab,
                         const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, size_t rec_stride, GridTables gt, LeftLists left,
-                        uint32_t k0, uint32_t* ticket, uint64_t* work, int sms, cudaStream_t st) {
+                        uint32_t k0, uint32_t* ticket, uint64_t* work, bool beside, int sms, cudaStream_t st) {
     if (n_chunks == 0 || n_slabs == 0) return cudaSuccess;
     if ((uint64_t)n_chunks * n_slabs > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
     const Args a = {tr, rec, gc, rec_stride, classes, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, k0, ticket,
-                    (unsigned long long*)work};
+                    (unsigned long long*)work, beside};
     switch (rows_for(T)) {
         case 1: return wide ? launch_one<1, true>(a, sms, st) : launch_one<1, false>(a, sms, st);
         case 2: return wide ? launch_one<2, true>(a, sms, st) : launch_one<2, false>(a, sms, st);

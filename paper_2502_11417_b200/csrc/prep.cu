@@ -189,11 +189,12 @@ __global__ void __launch_bounds__(kBetaThreads)
 k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __restrict__ cum_mass,
             const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
             const uint32_t* __restrict__ tick_start, const uint32_t* __restrict__ tick_cnt, const uint32_t* __restrict__ pairs,
-            Prep* __restrict__ prep) {
+            Prep* __restrict__ prep, bool early) {
     __shared__ uint32_t s_end[kTickBins];                             // ticks of the group up to the bin's last
     __shared__ long long part[8][32], total[6];
     using Sum = typename std::conditional<LARGE, __int128, long long>::type;
     grid_dependency_wait();
+    if (early) let_next_start();
     const uint32_t pair = pairs[blockIdx.x], p = pair % P;
     const int g = (int)(pair / P);
     Prep& out = prep[(size_t)g * P + p];
@@ -378,10 +379,10 @@ cudaError_t launch_prep(uint32_t P, int G, const GroupConst* gc, const int64_t* 
 
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off, const uint32_t* tick_start,
-                             const uint32_t* tick_cnt, const uint32_t* pairs, uint32_t n_pairs, uint64_t most, Prep* prep, cudaStream_t st) {
+                             const uint32_t* tick_cnt, const uint32_t* pairs, uint32_t n_pairs, uint64_t most, Prep* prep, bool early, cudaStream_t st) {
     auto* kernel = most > kBetaLargeN ? k_prep_beta<true> : k_prep_beta<false>;
     return launch_after(kernel, n_pairs, kBetaThreads, 0, st, pol, P, cum_mass, cnt, sorted, grp_off, tick_start,
-                        tick_cnt, pairs, prep);
+                        tick_cnt, pairs, prep, early);
 }
 
 }  // namespace disco

@@ -283,3 +283,16 @@ def test_streams_delivered_as_they_are_generated(n, jitter, rate):
     w.devices = [synth.device(1500.0, 40.0, jitter=0.05), synth.device(200.0, 10.0, jitter=jitter / 2, c_prefill=5e-3, c_decode=5e-3)]
     flags = synth.FLAG_MIGRATION | (synth.FLAG_PACING if rate else 0)
     full_parity(w, [synth.policy(b, r_c=rate or 5.0, flags=flags) for b in (0.3, 0.8)], select=False, tag=f"{n} {jitter} {rate}")
+
+
+@pytest.mark.parametrize("n", [1, 700, 20001])
+@pytest.mark.parametrize("shape", [(1, 1), (3, 2)])
+@pytest.mark.parametrize("plain", [0, 1, 9])
+def test_grids_beside_the_slope_search(n, shape, plain):
+    # plain policies are reduced while the slopes of the others are searched for: no plain ones, one, several rows, a column a policy
+    # with overheads of its own, and searches that outlast or do not outlast the grid
+    w = synth.tiny_workload(131 + n, n, n_servers=shape[0], n_devices=shape[1], max_prompt=2000, max_out=40)
+    slopes = [synth.policy(b, flags=PACED | synth.FLAG_BETA_RULE | synth.MODE_DEVICE_CONSTRAINED, l_immediate=64) for b in (0.2, 0.5, 0.9)]
+    rows = [synth.policy(b, mig_threshold=th) for b in synth.budget_grid(plain) for th in (0.0, 1e-5)]
+    full_parity(w, slopes + rows, select=False, tag=f"{n} {shape} {plain}")
+    full_parity(w, slopes[:1] + [synth.policy(b, mig_threshold=1e-6 * k) for k, b in enumerate(synth.budget_grid(plain))], select=False, tag="columns")
