@@ -20,6 +20,7 @@
 // registers that 1,024 threads leave spill 64 bytes.)
 #include <algorithm>
 #include <cstdlib>
+#include <cstring>
 #include <mutex>
 
 #include "ingest.cuh"
@@ -482,9 +483,10 @@ constexpr uint32_t kNoAllocMaxN = DISCO_NOALLOC_MAX_N;
 constexpr size_t kNaKeysBytes = (size_t)kNoAllocMaxN * sizeof(uint64_t);
 constexpr size_t kNaCountsBytes = (256u * ((kNoAllocMaxN + 1023u) / 1024u) + 256u) * sizeof(uint32_t);   // as radix_sort_ticks sizes its grid, plus the digit totals
 // words that must start at zero: the flags and the bins' counters; then the bins' starts and the offsets of the one group
+// (they lie there twice: a call clears the half that the next one uses)
 constexpr size_t kNaZeroOff = 2 * kNaKeysBytes + kNaCountsBytes;
 constexpr size_t kNaZeroBytes = (sizeof(LoadZero) + kTickBins * 4 + kOnceWindows * 16 + 15) / 16 * 16;
-constexpr size_t kNaStartOff = kNaZeroOff + kNaZeroBytes;
+constexpr size_t kNaStartOff = kNaZeroOff + 2 * kNaZeroBytes;
 constexpr size_t kNaOffOff = kNaStartOff + kTickBins * 4;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaOffOff + 256];
@@ -492,6 +494,12 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaOffOff + 256
 std::mutex g_na_mutex;
 unsigned char* g_na_base[64] = {};        // device address of the scratch array, per device ordinal
 int g_na_sms[64] = {};                    // multiprocessors, per device ordinal
+struct { bool zero[2]; int now; } g_na_half[64] = {};   // which halves are known to be zero, and which was used last
+// Where the kernel reports its flags: a page of the library's own, page-locked by the first call, 64 bytes a device ordinal.  (A
+// copy into pageable memory behind the kernel took 7 us of a call, the clearing in front of it 5: 100,000 values 35 us, now 27.)
+alignas(4096) unsigned char g_na_report[4096];
+int g_na_locked = 0;                      // 1: it is, -1: it cannot be
+void* g_na_report_dev[64] = {};           // its address on the device, per device ordinal
 
 }  // namespace
 }  // namespace disco
@@ -510,7 +518,10 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
     if (e != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
     if (dev < 0 || dev >= 64) return set_error(DISCO_EINVAL, "device ordinal above 63");
     unsigned char* base;
-    int sms;
+    int sms, half;
+    bool zeroed;
+    int32_t* report = nullptr;
+    void* report_dev = nullptr;
     {
         // In host code the array's name is only a handle; its address on the current device has to be asked for.
         std::lock_guard<std::mutex> lock(g_na_mutex);
@@ -524,11 +535,28 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
         }
         base = g_na_base[dev];
         sms = g_na_sms[dev];
+        if (!g_na_locked) {
+            g_na_locked = cudaHostRegister(g_na_report, sizeof g_na_report, cudaHostRegisterPortable | cudaHostRegisterMapped) == cudaSuccess ? 1 : -1;
+            if (g_na_locked < 0) cudaGetLastError();
+        }
+        if (g_na_locked > 0 && !g_na_report_dev[dev] && cudaHostGetDevicePointer(&g_na_report_dev[dev], g_na_report + 64 * dev, 0) != cudaSuccess) {
+            g_na_report_dev[dev] = nullptr;
+            cudaGetLastError();
+        }
+        report_dev = g_na_report_dev[dev];
+        if (report_dev) report = (int32_t*)(g_na_report + 64 * dev);
+        auto& h = g_na_half[dev];
+        half = h.now ^= 1;
+        zeroed = h.zero[half];
+        h.zero[0] = h.zero[1] = false;    // (until the call has succeeded)
     }
     LoadArgs a = {};
     a.n = n; a.G = 1; a.ns = a.nd = 1;
     a.ttft = server_ttft_s;
-    a.z = (LoadZero*)(base + kNaZeroOff); a.tick_cnt = (uint32_t*)(base + kNaZeroOff + sizeof(LoadZero));
+    unsigned char *mine = base + kNaZeroOff + half * kNaZeroBytes, *next = base + kNaZeroOff + (half ^ 1) * kNaZeroBytes;
+    a.z = (LoadZero*)mine; a.tick_cnt = (uint32_t*)(mine + sizeof(LoadZero));
+    a.once.zeroed = zeroed; a.once.clear = (uint4*)next; a.once.clear_vecs = (uint32_t)(kNaZeroBytes / 16);
+    a.readback = (LoadReadback*)report_dev;                          // (its flags alone)
     a.once.windows = (unsigned long long*)(a.tick_cnt + kTickBins);
     a.tick_start = (uint32_t*)(base + kNaStartOff);
     a.binned = (uint32_t*)base; a.sorted = sorted_ticks;
@@ -539,10 +567,16 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
         cudaStreamSynchronize(st);
         return set_error(DISCO_ECUDA, cudaGetErrorString(err_code));
     };
+    int32_t h_err[4] = {0, 0, 0, 2};      // what stands where the blocks lose each other
+    if (report) std::memcpy(report, h_err, sizeof h_err);
     if ((e = run_sort_ttft(a, sms, st)) != cudaSuccess) return fail_after_launch(e);
-    int32_t h_err[4] = {0, 0, 0, 0};
-    if ((e = cudaMemcpyAsync(h_err, a.z->err, sizeof h_err, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return fail_after_launch(e);
+    if (!report && (e = cudaMemcpyAsync(h_err, a.z->err, sizeof h_err, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return fail_after_launch(e);
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
+    if (report) std::memcpy(h_err, report, sizeof h_err);
+    if (h_err[3] != 2) {
+        std::lock_guard<std::mutex> lock(g_na_mutex);
+        g_na_half[dev].zero[half ^ 1] = true;
+    }
     if (int rc = check_debug_record()) return rc;
     if (h_err[0]) return set_error(DISCO_EINVAL, "server TTFT not finite, not positive or above 2000 s");
     if (h_err[3] == 2) return set_error(DISCO_ECUDA, "internal error: the blocks of the sort lost each other");

@@ -217,7 +217,7 @@ k_load_once(const __grid_constant__ LoadArgs a) {
             __syncthreads();
         }
         if (refused) {                                 // a rejected trace: nothing is placed
-            if (kTrace && block == 0 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
+            if (SRC != S_TICKS && block == 0 && tid < 4 && a.readback) a.readback->err[tid] = __ldcg(&z->err[tid]);
             return;
         }
         auto start = [&](uint32_t k) { return s[k] + s_base[k >> shift]; };     // (of a length: behind the n ticks)
@@ -305,7 +305,7 @@ k_load_once(const __grid_constant__ LoadArgs a) {
                 if ((uint32_t)(G - 1 - g) % blocks == blocks - 1 - block) group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
         }
     }
-    if (kTrace) {
+    if (kTrace || (SRC == S_TTFT && a.readback)) {
         // the last block to come here reports the flags (where a block has left, none does: what the host put there stands)
         if (tid == 0) { __threadfence(); s_item = atomicAdd(&z->done, 1u); }
         __syncthreads();
