@@ -160,6 +160,13 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 // its own wait is up to it.  To be called behind this kernel's wait.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// add + ((h * mul) >> 32) in one instruction
+__device__ __forceinline__ uint32_t mad_hi(uint32_t h, uint32_t mul, uint32_t add) {
+    uint32_t x;
+    asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(x) : "r"(h), "r"(mul), "r"(add));
+    return x;
+}
+
 // The stream after a hand-off stores no window of its own where groups are played free without pacing: it is stream
 // x_stream's (0 the server's, 1 the device's) without the interval in front of token 2, whose bin first_bin gives.  -1: it
 // stores one, if it has any.

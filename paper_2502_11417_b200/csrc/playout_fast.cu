@@ -235,7 +235,9 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
 // what is left of the longer ones is made up by a warp each, 32 tokens at a time, so that the longest (thousands of
 // tokens) does not hold the block for as many dependent steps.  A thread draws 32 tokens, or 256 where most of the block's
 // requests have longer lags (prompts that take a device long to read: those lags are alike).  (Without the collection:
-// 513 us for the 16 M requests of three server profiles and two devices, 43 us for 250,000 of them; now 304 and 12.)
+// 513 us for the 16 M requests of three server profiles and two devices, 43 us for 250,000 of them; with it 304 and 12, and
+// 248 and 10 with the tokens that can neither fill the buffer nor make up the lag drawn without a test each; 4 M requests of long
+// outputs on a slow device 97 us, now 59, most of it because the blocks with the longest lags come first.)
 constexpr uint32_t kShortSearch = 64;
 constexpr int kShortThreads = 256;
 constexpr int kShortPer = 4;             // requests a thread may play
@@ -248,7 +250,16 @@ struct ShortGroup {                      // a group under the class
     uint32_t end;                        // where the group's requests end
     int exact;                           // played here
     int32_t cT_mean;
+    uint32_t sure;                       // tokens that cannot fill the buffer, whatever their jitter
 };
+
+// (h * mul) >> 32 of so many tokens behind hin, added up: no test a token, so that several are under way at once.
+__device__ __forceinline__ uint32_t sum_jitter(uint32_t& hin, uint32_t count, uint32_t mul) {
+    uint32_t sum = 0;
+#pragma unroll 4
+    for (uint32_t t = 0; t < count; ++t) { hin += kHashTok; sum = mad_hi(mix32(hin), mul, sum); }
+    return sum;
+}
 
 __global__ void __launch_bounds__(kShortThreads)
 k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
@@ -276,14 +287,17 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
         G.end = tr.grp_off[g + 1];
         G.exact = cc.kind[g] == G_EXACT;
         G.cT_mean = G.cT - (int32_t)(G.mulT >> 1);
+        G.sure = G.cC > 0 ? (uint32_t)(thr / G.cC) : (uint32_t)kMaxOutput;     // (a token adds at most cC)
         groups[g] = G;
     }
     __syncthreads();
-    const uint32_t first = blockIdx.x * (uint32_t)(kShortThreads * per);
+    // (the last blocks first: lags of a device that reads slowly grow with the prompt, and the requests are stored by it)
+    const uint32_t first = (gridDim.x - 1u - blockIdx.x) * (uint32_t)(kShortThreads * per);
+    int g = 0;
+    while (g + 1 < tr.n_groups && first >= groups[g].end) ++g;
     for (int k = 0; k < per; ++k) {
         const uint32_t kk = first + k * kShortThreads + threadIdx.x;
         if (kk >= tr.n) break;
-        int g = 0;
         while (g + 1 < tr.n_groups && kk >= groups[g].end) ++g;
         const ShortGroup& G = groups[g];
         if (!G.exact) continue;
@@ -296,7 +310,9 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
             if (B == 0) m = 1;                                         // nothing to fill: hand off after token 1
             else {
                 uint32_t hin = key + kHashTok;
-                for (uint32_t j = 2; j < n; ++j) {                     // (the hand-off needs a token left to generate)
+                const uint32_t sure = min(G.sure, n - 2u);
+                e_m = (int32_t)(sure * (uint32_t)G.cC - sum_jitter(hin, sure, G.mulC));
+                for (uint32_t j = 2 + sure; j < n; ++j) {              // (the hand-off needs a token left to generate)
                     hin += kHashTok;
                     e_m += G.cC - (int32_t)__umulhi(mix32(hin), G.mulC);
                     if (e_m > thr) { m = j; break; }
@@ -333,9 +349,12 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
         const ShortGroup& G = groups[x.w >> 16];
         const int32_t need = (int32_t)x.y, cT = G.cT;
         const uint32_t n = x.z & 0xFFFFu, m = x.z >> 16, mulT = G.mulT, end = min(n, m + 1 + most);
-        int32_t run = 0;
-        uint32_t j = m + 2;
-        for (uint32_t hin = x.x + j * kHashTok; j <= end; ++j, hin += kHashTok) {
+        uint32_t j = m + 2, hin = x.x + (m + 1) * kHashTok;
+        // so many tokens are late for sure, each making up cT at most (the quotient is rounded down by more than its error)
+        const uint32_t sure = min(end + 1u - j, (uint32_t)(__fdividef((float)(need - 1), (float)max(cT, 1)) * 0.99999f));
+        int32_t run = (int32_t)(sure * (uint32_t)cT - sum_jitter(hin, sure, mulT));
+        j += sure;
+        for (hin += kHashTok; j <= end; ++j, hin += kHashTok) {
             run += cT - (int32_t)__umulhi(mix32(hin), mulT);
             if (run >= need) break;
         }

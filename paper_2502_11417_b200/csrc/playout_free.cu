@@ -35,13 +35,6 @@ __device__ __forceinline__ void count_in(const Counters& c, uint32_t x, uint32_t
     const int b = (SMALL ? bin_of_ticks(x) : (int)(__float_as_uint(__uint2float_rz(x)) >> 18) - ((127 + 4) << 5)) - c.lo;
     if (DBG_OK(b, c.W, DBG_K_PLAYOUT, DBG_WINDOW)) atomicAdd(&c.at[b * kCols], inc);
 }
-// base + ((h * mul) >> 32) in one instruction
-__device__ __forceinline__ uint32_t draw(uint32_t h, uint32_t mul, uint32_t base) {
-    uint32_t x;
-    asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(x) : "r"(h), "r"(mul), "r"(base));
-    return x;
-}
-
 // PLAY: which streams are played.  P_BOTH: pacing is off, both, and a hand-off may follow the first token.  Otherwise pacing is
 // on, a stream or two clamp at every token and no buffer fills: the server's or the device's in all groups, or what a group's
 // are.  (Kernels of their own: in one kernel for all cases the warps waited for instructions four cycles of every ten.)
@@ -100,8 +93,8 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
                 auto token = [&]() {
                     const uint32_t h = mix32(hin);
                     hin += 32u * kHashTok;
-                    if (on0) { const uint32_t x = draw(h, mul0, base0); s0 += x; count_in<SMALL>(ct0, x, inc); }
-                    if (on1) { const uint32_t x = draw(h, mul1, base1); s1 += x; count_in<SMALL>(ct1, x, inc); }
+                    if (on0) { const uint32_t x = mad_hi(h, mul0, base0); s0 += x; count_in<SMALL>(ct0, x, inc); }
+                    if (on1) { const uint32_t x = mad_hi(h, mul1, base1); s1 += x; count_in<SMALL>(ct1, x, inc); }
                     return h;
                 };
                 if (j <= n) {
@@ -151,10 +144,10 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
                     if (DBG_OK(ki + 1, kNKnots, DBG_K_PLAYOUT, DBG_KNOT))
                         M = (uint32_t)(K[ki] + (int32_t)(((int64_t)(K[ki + 1] - K[ki]) * (int64_t)fr) >> 16));
                 }
-                sumX = M + (to_dev ? sum1 - draw(h2, mul1, base1) : sum0 - draw(h2, mul0, base0));
-                maxX = max(M, nI > 1u ? (to_dev ? draw(o_h, mul1, base1) : draw(o_h, mul0, base0)) : 0u);
+                sumX = M + (to_dev ? sum1 - mad_hi(h2, mul1, base1) : sum0 - mad_hi(h2, mul0, base0));
+                maxX = max(M, nI > 1u ? (to_dev ? mad_hi(o_h, mul1, base1) : mad_hi(o_h, mul0, base0)) : 0u);
             }
-            const uint32_t most0 = draw(max(o_h, h2), mul0, base0), most1 = draw(max(o_h, h2), mul1, base1);
+            const uint32_t most0 = mad_hi(max(o_h, h2), mul0, base0), most1 = mad_hi(max(o_h, h2), mul1, base1);
             rec.hand[k] = make_uint2(m, M);
             rec.sum[0][k] = sum0; rec.sum[1][k] = sum1; rec.sum[2][k] = sumX;
             rec.max[0][k] = nI ? (on0 ? most0 : tau) : 0u; rec.max[1][k] = nI ? (on1 ? most1 : tau) : 0u;

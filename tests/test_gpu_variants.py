@@ -296,3 +296,16 @@ def test_grids_beside_the_slope_search(n, shape, plain):
     rows = [synth.policy(b, mig_threshold=th) for b in synth.budget_grid(plain) for th in (0.0, 1e-5)]
     full_parity(w, slopes + rows, select=False, tag=f"{n} {shape} {plain}")
     full_parity(w, slopes[:1] + [synth.policy(b, mig_threshold=1e-6 * k) for k, b in enumerate(synth.budget_grid(plain))], select=False, tag="columns")
+
+
+@pytest.mark.parametrize("n", [2, 1023, 1025, 5000])
+@pytest.mark.parametrize("tbt", [0.0, 0.01, 0.0499, 0.05])
+def test_tokens_that_are_certain_not_to_decide(n, tbt):
+    # the tokens in front of the first that can fill a buffer or make a lag up are added up without a test: without jitter, where that
+    # is all but the last, an interval of the reader's own pace, where none does, outputs that end among them, lags of one tick
+    w = synth.tiny_workload(137 + n, n, n_servers=2, n_devices=2, max_prompt=1500, max_out=40)
+    w.output_len[::5] = np.arange(len(w.output_len[::5])) % 9 + 1
+    w.output_len[3::11] = 700
+    w.servers = [synth.server(tbt_s=max(tbt, 1e-6), jitter=0.0), synth.server(tbt_s=0.04, jitter=0.2)]
+    w.devices = [synth.device(20.0, 1.0 / max(tbt, 1e-6), jitter=0.0), synth.device(300.0, 25.0, jitter=0.2, c_prefill=5e-3, c_decode=5e-3)]
+    full_parity(w, [synth.policy(b, r_c=20.0, t_m_s=t, flags=PACED) for b in (0.4, 1.0) for t in (0.05, 0.1, 0.4)], select=False, tag=f"{n} {tbt}")
