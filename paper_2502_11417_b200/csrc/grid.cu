@@ -525,26 +525,31 @@ k_grid(const __grid_constant__ Args a) {
     // Beside the slope search of Eq. 1-2 (k_prep_beta), which no plain policy needs: what this kernel reads was complete before that
     // one let it start.  It then waits at its end, for the kernels behind.  (Under 48 such searches, 79 us on 48
     // multiprocessors, 300,000 requests by 16 budgets take 27.)
-    if (!a.beside) grid_dependency_wait();
     for (int i = threadIdx.x; i < (int)(offsetof(Smem, key) / 4); i += kThreads) ((uint32_t*)&sm)[i] = 0;
     for (int i = threadIdx.x; i < (NT + (WIDE ? 1 : 0)) * kNBins; i += kThreads) tbt[i] = 0;
+    if (!a.beside) grid_dependency_wait();
 
     int turn = 0;                                                     // which of the two sets of used bins is in use
     const uint32_t direct = a.n_chunks * a.n_slabs <= gridDim.x ? kDirectAlone : kDirectMany;
-    // the blocks draw (chunk, slab) items from a counter (zero at launch): items differ in cost
-    for (;;) {
+    // A block starts with a (chunk, slab) item of its own and then draws the next ones from a counter (zero at launch): items
+    // differ in cost.  (Drawn ahead, when the one in front begins, they are no longer dealt to who is free: 16 M requests by
+    // 128 and 8 policies 348 -> 385 us.  Beside another kernel not all blocks are there at once: all items are drawn.)
+    const uint32_t n_items = a.n_chunks * a.n_slabs, dealt = a.beside ? 0u : gridDim.x;
+    uint32_t item = blockIdx.x;
+    __syncthreads();
+    if (a.beside) {
+        if (threadIdx.x == 0) sm.ticket = atomicAdd(a.ticket, 1u);
         __syncthreads();
-        if (threadIdx.x == 0) { sm.ticket = atomicAdd(a.ticket, 1u); sm.n_seg = 0; sm.n_runs = 0; sm.n_list = 0; sm.flagged = 0; }
-        __syncthreads();
-        const uint32_t item = sm.ticket;
-        if (item >= a.n_chunks * a.n_slabs) break;
+        item = sm.ticket;
+    }
+    for (; item < n_items; item = sm.ticket) {
         const uint32_t slab_id = item % a.n_slabs;
         const Slab& sl = a.slabs[slab_id];
         const Chunk ch = a.chunks[item / a.n_slabs];
         const int g = ch.g;
         if (!DBG_OK(g, a.tr.n_groups, DBG_K_GRID, DBG_GROUP) ||
             (ch.len && !DBG_OK((unsigned long long)ch.start + ch.len - 1, a.tr.n, DBG_K_GRID, DBG_REQUEST)))
-            continue;
+            break;
         const GroupConst& gc = a.gcs[g];
         const Tables<WIDE> tb(a.gt, sl, a.tr.n_groups);
         Ctx c;
@@ -720,6 +725,13 @@ k_grid(const __grid_constant__ Args a) {
             atomicAdd(&a.work[2], settled);                            // requests settled, per slab
             atomicAdd(&a.work[3], (unsigned long long)passes);         // sweeps over segments
         }
+        if (n_items <= dealt) break;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            sm.n_seg = 0; sm.n_runs = 0; sm.n_list = 0; sm.flagged = 0;
+            sm.ticket = dealt + atomicAdd(a.ticket, 1u);
+        }
+        __syncthreads();
     }
     if (a.beside) grid_dependency_wait();
 }
