@@ -988,8 +988,19 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     for (size_t first = 0; first < n_classes && n != 0; first += wave) {
         const size_t last = std::min(n_classes, first + wave);
         if (timed) CU(cudaEventRecord(c->ev[0], st));
+        ShortMany many;
+        many.classes = d_classes; many.rec_stride = rec_stride; many.count = 0;
+        for (size_t k = std::max<size_t>(first, 1); k < last && last - first > 1 && many.count < kShortMany; ++k) {
+            if (!(plan[k].kinds & (1u << G_EXACT)) || !short_search(plan[k].search)) continue;
+            plan[k].kinds &= ~(1u << G_EXACT);
+            many.cls[many.count] = (uint32_t)k; many.slot[many.count++] = (uint32_t)slot_of(k);
+        }
+        if (many.count) {
+            CU(launch_playout_many(tr, gc, c->knots.as<int32_t>(), k0, rec, many, c->sms, st));
+            g_launches += 1;
+        }
         for (size_t k = first; k < last; ++k)
-            if (k != 0 || timed) CU(play_out(k));
+            if ((k != 0 || timed) && plan[k].kinds) CU(play_out(k));
         if (timed) CU(cudaEventRecord(c->ev[2], st));
         for (; next < batches.size() && batches[next].wave == first / wave; ++next) {
             const Batch& b = batches[next];

@@ -280,6 +280,12 @@ cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const Clas
                             const FreeMore& more, uint32_t* free_ticket /* one word, zero before and after */, const uint32_t* grp_n /* requests per group, on the host */, bool early /* the preparation follows: it may start beside the last kernel */,
                             int sms /* multiprocessors of the device */, cudaStream_t st);
 uint32_t timeline_launches(uint32_t kinds);
+// The exact groups of several classes whose searches are short, in one launch.
+constexpr int kShortMany = 16;
+struct ShortMany { const ClassConst* classes; size_t rec_stride; uint32_t count, cls[kShortMany], slot[kShortMany]; };
+bool short_search(uint32_t search);
+cudaError_t launch_playout_many(const TraceDev& tr, const GroupConst* gc, const int32_t* knots, uint32_t k0, TimelineRec rec /* of slot 0 */,
+                                const ShortMany& many, int sms, cudaStream_t st);
 
 // Reductions over a grid of plain policies, budget by overhead (grid.cu).
 constexpr int kGridRows = 8;     // overheads a slab may have

@@ -261,9 +261,13 @@ __device__ __forceinline__ uint32_t sum_jitter(uint32_t& hin, uint32_t count, ui
     return sum;
 }
 
+// MANY: several classes, a row of blocks each (250,000 requests under five paces one after another 42 us; the last four together 23, and 8 for the first).
+template <bool MANY>
 __global__ void __launch_bounds__(kShortThreads)
-k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
-                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int per, bool early) {
+k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst given,
+                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, int per, bool early, const __grid_constant__ ShortMany many) {
+    const ClassConst& cc = MANY ? many.classes[many.cls[blockIdx.y]] : given;
+    if (MANY) rec.hand = reinterpret_cast<uint2*>(reinterpret_cast<char*>(rec.hand) + many.slot[blockIdx.y] * many.rec_stride);
     __shared__ ShortGroup groups[kMaxGroups];
     __shared__ uint4 lag[kShortThreads * kShortPer];         // hash key, lag, output length | hand-off << 16, place | group << 16
     __shared__ uint16_t rest[kShortThreads * kShortPer];     // lags that a thread has not made up
@@ -389,14 +393,26 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
 
 DBG_TRANSLATION_UNIT()
 
+// four requests a thread (fuller warps of lags) once that leaves several blocks to every multiprocessor
+static int short_per(uint32_t n, int sms) { return n >= (uint32_t)sms * 8u * kShortThreads * kShortPer ? kShortPer : 1; }
+
+bool short_search(uint32_t search) { return search <= kShortSearch; }
+
+cudaError_t launch_playout_many(const TraceDev& tr, const GroupConst* gc, const int32_t* knots, uint32_t k0, TimelineRec rec, const ShortMany& many, int sms,
+                                cudaStream_t st) {
+    const int per = short_per(tr.n, sms);
+    const uint32_t per_block = (uint32_t)(kShortThreads * per);
+    return launch_after(k_playout_short<true>, dim3((tr.n + per_block - 1) / per_block, many.count), kShortThreads, 0, st, tr, gc, ClassConst{}, knots, k0,
+                        rec, per, false, many);
+}
+
 cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots,
                                  uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, bool early, int sms,
                                  cudaStream_t st) {
-    if (search <= kShortSearch) {
-        // four requests a thread (fuller warps of lags) once that leaves several blocks to every multiprocessor
-        const int per = tr.n >= (uint32_t)sms * 8u * kShortThreads * kShortPer ? kShortPer : 1;
+    if (short_search(search)) {
+        const int per = short_per(tr.n, sms);
         const uint32_t per_block = (uint32_t)(kShortThreads * per);
-        return launch_after(k_playout_short, (tr.n + per_block - 1) / per_block, kShortThreads, 0, st, tr, gc, cc, knots, k0, rec, per, early);
+        return launch_after(k_playout_short<false>, (tr.n + per_block - 1) / per_block, kShortThreads, 0, st, tr, gc, cc, knots, k0, rec, per, early, ShortMany{});
     }
     // requests per ticket: small batches spread the end of the launch evenly; large traces amortise the ticket
     int rpw = 8;

@@ -256,11 +256,12 @@ def test_tables_of_the_policies_on_their_way(n_policies, beta):
 
 
 @pytest.mark.parametrize("n", [1, 300, 4000])
-@pytest.mark.parametrize("rates", [(12.0, 20.0), (20.0, 5.0, 12.0), (5.0, 30.0, 12.0, 4.0, 20.0, 11.0), (12.0, 33.0, 20.0), tuple(12.0 + 0.4 * k for k in range(12))])
+@pytest.mark.parametrize("rates", [(12.0, 20.0), (20.0, 5.0, 12.0), (5.0, 30.0, 12.0, 4.0, 20.0, 11.0), (12.0, 33.0, 20.0), tuple(12.0 + 0.4 * k for k in range(12)),
+                                   tuple(3.0 + 0.2 * k for k in range(20))])
 def test_classes_that_are_reduced_together(n, rates):
     # a slow device whose streams are delivered as they are generated at most of these rates, beside a server and a device that keep
-    # the pace at some: such streams are played once for several classes (up to nine), classes without windows share a launch, and
-    # classes of any kind lie between them
+    # the pace at some: such streams are played once for several classes (up to nine), classes without windows share a launch, sixteen
+    # play-outs up to the hand-off do, and classes of any kind lie between them
     w = synth.tiny_workload(113 + n, n, n_servers=2, n_devices=2, max_prompt=300, max_out=200)
     w.servers = [synth.server(tbt_s=0.03, jitter=0.2), synth.server(tbt_s=0.03, jitter=0.0)]
     w.devices = [synth.device(1500.0, 40.0, jitter=0.05), synth.device(200.0, 10.0, jitter=0.05, c_prefill=5e-3, c_decode=5e-3)]
