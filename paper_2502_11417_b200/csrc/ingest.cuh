@@ -64,8 +64,11 @@ __device__ __forceinline__ bool await_blocks(LoadZero* z, uint32_t want) {
 // Checked build: a wait for one arrival that nobody makes (LoadArgs::absent).
 #ifdef DISCO_DEBUG
 #define ABSENT(a, wait) ((a).absent == (wait) ? 1u : 0u)
+// A block that is some two milliseconds late with what it has to do next (LoadArgs::absent = 5).
+#define LATE(a, block) do { if ((a).absent == 5u && (block)) for (const long long t0 = clock64(); clock64() - t0 < 4000000ll;) { } } while (0)
 #else
 #define ABSENT(a, wait) 0u
+#define LATE(a, block) do { } while (0)
 #endif
 
 // Four neighbouring requests of the trace (or ticks of a sample) as the two passes see them.

@@ -115,7 +115,8 @@ struct LoadArgs {
     OnceLoad once;
     LoadReadback* readback;               // its err holds 0, 0, 0, 2 (no report) before the launch
 #ifdef DISCO_DEBUG
-    uint32_t absent;                      // the wait that expects one arrival more than comes (from 1; 4: of the other blocks' sums)
+    uint32_t absent;                      // the wait that expects one arrival more than comes (from 1; 4: of the other blocks' sums);
+                                          // 5: k_load_once's last block is late with its totals
 #endif
 };
 

@@ -14,7 +14,7 @@
 // Bound: latency, some fifteen dependent steps, and from half a million requests on the scattered stores.  Against k_load, which
 // reads the requests twice and waits three times (with the memset in front of it, kernels and gaps): 100,000 requests in one group
 // 42 us -> 21, in six 56 -> 34; a million 64 -> 45 and 76 -> 57; 1,000 in one block 23 -> 17; 100,000 ticks 25 -> 15.  Where the
-// threads cannot keep their requests (8,192 a block) k_load is left.  (Eight requests a thread spill 160 bytes, four 76.)
+// threads cannot keep their requests (8,192 a block) k_load is left.  (Eight requests a thread spill 172 bytes, four 48.)
 #include <algorithm>
 #include <cstdlib>
 
@@ -144,6 +144,7 @@ k_load_once(const __grid_constant__ LoadArgs a) {
                 pt[k] += s[tick_at(k)];
                 if constexpr (kTrace) pl[k] += s[len_at(k)];
             }
+            LATE(a, block == blocks - 1u);
             totals();
             if (!wait_for<false>(z, blocks + ABSENT(a, 1u) + ABSENT(a, 4u))) return;
         } else if (kTrace) {
@@ -271,17 +272,25 @@ k_load_once(const __grid_constant__ LoadArgs a) {
         if (kTrace && block == 0) {
             for (int g = tid; g < G; g += kThreads) {
                 const uint32_t N = s_off[g + 1] - s_off[g];
-                const uint64_t sum = __ldcg((const unsigned long long*)&z->grp_sum_n[g]);
-                a.readback->ng[g] = N; a.readback->grp_sum_n[g] = sum; a.readback->grp_off[g] = s_off[g];
+                a.readback->ng[g] = N; a.readback->grp_off[g] = s_off[g];
                 a.grp_off[g] = s_off[g];
-                a.fin_totals[g] = sum; a.fin_totals[G + g] = N;        // what the final reductions' totals refer to
+                a.fin_totals[G + g] = N;                               // what the final reductions' totals refer to
                 if (N == 0) a.readback->knot_max[g] = 0;
             }
-            if (tid == 0) { a.grp_off[G] = s_off[G]; a.readback->grp_off[G] = s_off[G]; a.readback->max_n = __ldcg(&z->max_n); }
+            if (tid == 0) { a.grp_off[G] = s_off[G]; a.readback->grp_off[G] = s_off[G]; }
             for (int k = tid; k < G * kNKnots; k += kThreads)
                 if (s_off[k / kNKnots + 1] == s_off[k / kNKnots]) a.knots[k] = 0;
         }
         if (!alone && !wait_for<true>(z, 2 * blocks + ABSENT(a, 2u) + ABSENT(a, 3u))) return;
+        // A block announces itself at the first wait before it adds its share of these, and at the second behind it.  (The last
+        // block has the fewest windows.)
+        if (kTrace && block == blocks - 1u) {
+            for (int g = tid; g < G; g += kThreads) {
+                const uint64_t sum = __ldcg((const unsigned long long*)&z->grp_sum_n[g]);
+                a.readback->grp_sum_n[g] = sum; a.fin_totals[g] = sum;
+            }
+            if (tid == 0) a.readback->max_n = __ldcg(&z->max_n);
+        }
 
         // ---- 3. sort
         SortSmem& sm = *reinterpret_cast<SortSmem*>(smem_raw);

@@ -102,6 +102,38 @@ def test_blocks_leave_when_a_wait_runs_out():
     assert r.returncode == 0 and "waited" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
 
 
+LATE = """
+import os, sys
+sys.path[:0] = [os.getcwd(), os.path.join(os.getcwd(), "tests")]
+import numpy as np, torch
+from paper_2502_11417_b200 import DiscoError, Trace, synth
+for n, shape in ((5000, (1, 1)), (5000, (3, 2)), (40001, (1, 7)), (500009, (1, 1)), (1150000, (3, 2))):
+    w = synth.tiny_workload(n, n, n_servers=shape[0], n_devices=shape[1], max_prompt=4096, max_out=60)
+    w.output_len[n - 3] = 4000                      # (the longest output is the last block's)
+    cols = [torch.from_numpy(getattr(w, f)).cuda() for f in ("prompt_len", "output_len", "server_ttft_s", "server_profile", "device_profile")]
+    t = Trace()
+    for _ in range(2):
+        t.load_trace(*cols, w.servers, w.devices)
+        t.eval_policies([synth.policy(0.4), synth.policy(0.0)], 1)
+        for s in t.reduce_stats():
+            assert s.tok_server + s.tok_device == w.output_len.sum(dtype=np.int64), (n, shape)
+            assert s.n_intervals == w.output_len.sum(dtype=np.int64) - n and s.n_requests == n, (n, shape)
+        try:                                        # 4,000 tokens at one a second would outlast 2^31 ticks, 60 would not
+            t.eval_policies([synth.policy(0.4, r_c=1.0)], 1)
+            raise AssertionError("the longest output was overlooked")
+        except DiscoError as e:
+            assert e.code == -1 and "outlast" in str(e)
+    t.close()
+print("late")
+"""
+
+
+def test_totals_of_a_block_that_is_late():
+    # the last block of a load adds its output tokens and its longest output long behind the others
+    r = _run(["-c", LATE], DISCO_DEBUG_ABSENT="5")
+    assert r.returncode == 0 and "late" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
+
+
 def test_the_ordinary_build_has_no_selftest():
     from paper_2502_11417_b200 import api
     if os.environ.get("DISCO_CHECKED_BUILD") == "1":
