@@ -384,11 +384,12 @@ struct BigSort {
     uint32_t a[kBigCap + 2 * kSortPad];                // the ticks; or counters
     uint32_t cell[kBigCap / 2];                        // counts, then starts, then ends, two to a word
     uint32_t bin[kTickBins];                           // first place | count << 16
+    uint32_t mixed[kBigCap / 32];                      // a bit a cell: it holds different ticks
     uint32_t wtot[32], range[2], most;
 };
 static_assert(2 * (sizeof(BigSort) + 1024 + 16) <= 227 * 1024, "two blocks to a multiprocessor");
 
-__device__ __forceinline__ bool sort_bucket(BigSort& sm, const uint32_t* src, uint32_t count, const uint32_t* bin_start,
+__device__ __forceinline__ void sort_bucket(BigSort& sm, const uint32_t* src, uint32_t count, const uint32_t* bin_start,
                                             const uint32_t* bin_count, int b0, int b1, int32_t* out) {
     const int tid = threadIdx.x;
     constexpr int kVecs = kBigCap / 2 / kSortThreads / 4;              // vectors of cells a thread has
@@ -465,17 +466,45 @@ __device__ __forceinline__ bool sort_bucket(BigSort& sm, const uint32_t* src, ui
     __syncthreads();
     if (most <= kSortPad) {
         order_by_neighbours<kSortThreads>(a, count, (int)most - 1, out);
-        return true;
+        return;
     }
+    // Cells reach further: mostly a clock coarser than a microsecond, whose ticks share a cell with their like alone and need no
+    // order among themselves.  (A load of 4 M requests by a millisecond's clock: 189 us, by a microsecond's 184; with a trace that
+    // has one such cell of 256 left to the radix sort 454, of 16 M 1,213 and now 565.)
+    for (uint32_t i = tid; i < kBigCap / 32; i += kSortThreads) sm.mixed[i] = 0;
+    __syncthreads();
+    for (uint32_t i = tid; i + 1u < count; i += kSortThreads) {
+        const uint32_t v = a[i];
+        if (a[i + 1u] == v) continue;
+        const uint32_t c = cell_of(v);
+        if (i + 1u < half_of(c, sm.cell[c >> 1])) atomicOr(&sm.mixed[c >> 5], 1u << (c & 31u));
+    }
+    __syncthreads();
     uint32_t full = 0;
     for (uint32_t i = tid; i < count; i += kSortThreads) {
-        const uint32_t v = a[i], c = cell_of(v), from = c ? half_of(c - 1u, sm.cell[(c - 1u) >> 1]) : 0u, to = half_of(c, sm.cell[c >> 1]);
-        if (single) { out[i] = (int32_t)v; continue; }
+        const uint32_t v = a[i], c = cell_of(v);
+        if (!(sm.mixed[c >> 5] >> (c & 31u) & 1u)) { out[i] = (int32_t)v; continue; }
+        const uint32_t from = c ? half_of(c - 1u, sm.cell[(c - 1u) >> 1]) : 0u, to = half_of(c, sm.cell[c >> 1]);
         if (to - from > 4u * kCellCap) { full = 1u; continue; }
         const uint32_t p = place_in_cell(a, i, v, from, to);
         if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) out[p] = (int32_t)v;
     }
-    return !__syncthreads_or((int)full);
+    if (!__syncthreads_or((int)full)) return;
+    // Hundreds of ticks of a few neighbouring values in a cell: the whole bucket by a bitonic network, padded with the largest word
+    // (a power of two is at most kBigCap).
+    uint32_t whole = 2;
+    while (whole < count) whole <<= 1;
+    for (uint32_t i = count + tid; i < whole; i += kSortThreads) a[i] = 0xFFFFFFFFu;
+    for (uint32_t size = 2; size <= whole; size <<= 1)
+        for (uint32_t gap = size >> 1; gap > 0; gap >>= 1) {
+            __syncthreads();
+            for (uint32_t k = tid; k < whole / 2; k += kSortThreads) {
+                const uint32_t i = (k & ~(gap - 1u)) << 1 | (k & (gap - 1u)), x = a[i], y = a[i + gap];
+                if ((x > y) == ((i & size) == 0u)) { a[i] = y; a[i + gap] = x; }
+            }
+        }
+    __syncthreads();
+    for (uint32_t i = tid; i < count; i += kSortThreads) out[i] = (int32_t)a[i];
 }
 
 __global__ void __launch_bounds__(kSortThreads, 2)
@@ -492,10 +521,12 @@ k_sort(const __grid_constant__ LoadArgs a) {
         const int g = (int)members.x / kTickBins, b0 = (int)members.x - g * kTickBins, b1 = (int)members.y - g * kTickBins;
         const uint32_t k0 = __ldcg(&a.tick_start[members.x]), k1 = __ldcg(&a.tick_start[members.y]) + __ldcg(&a.tick_cnt[members.y]);
         const uint32_t first = __ldcg(&a.grp_off[g]), N = __ldcg(&a.grp_off[g + 1]) - first, edge = tick_bin_edge(b0);
-        const bool done = k1 - k0 > kBigCap
-                              ? sort_dense<kSortThreads, kBigCap>(sm.a, sm.wtot, sm.range, a.binned + k0, k1 - k0, edge, tick_bin_edge(b1 + 1) - edge, a.sorted + k0)
-                              : sort_bucket(sm, a.binned + k0, k1 - k0, a.tick_start + (size_t)g * kTickBins, a.tick_cnt + (size_t)g * kTickBins, b0, b1, a.sorted + k0);
-        if (!done && threadIdx.x == 0) atomicMax(&a.z->err[3], 1);     // (the radix sort, then)
+        if (k1 - k0 <= kBigCap) {
+            sort_bucket(sm, a.binned + k0, k1 - k0, a.tick_start + (size_t)g * kTickBins, a.tick_cnt + (size_t)g * kTickBins, b0, b1, a.sorted + k0);
+        } else if (!sort_dense<kSortThreads, kBigCap>(sm.a, sm.wtot, sm.range, a.binned + k0, k1 - k0, edge, tick_bin_edge(b1 + 1) - edge, a.sorted + k0) &&
+                   threadIdx.x == 0) {
+            atomicMax(&a.z->err[3], 1);                                // (the radix sort, then)
+        }
         __syncthreads();
         write_knots<kSortThreads>(a, g, k0, k1, first, N);
     }

@@ -218,6 +218,41 @@ def test_large_traces_are_placed_by_way_of_buckets(n, shape, kind, where):
     tr.close()
 
 
+def _crowded(kind, n, rng):
+    x = np.exp(rng.normal(-0.5, 0.9, n))
+    if kind == "pairs":                        # two neighbouring microseconds, thousands of each, in bins 8,192 and more wide
+        at = (2 ** 20 * 2 ** (rng.permutation(3 * 128)[:300] / 128.0) + rng.integers(0, 4000, 300)).astype(np.int64)
+        ticks = at[rng.integers(0, 300, n)] + rng.integers(0, 2, n)
+        return np.where(rng.random(n) < 0.3, ticks * 1e-6, x)
+    step = {"1ms": 1e-3, "10ms": 1e-2, "0.1ms": 1e-4}[kind]
+    return np.maximum(np.rint(x / step), 1) * step
+
+
+@pytest.mark.parametrize("n,shape,kind", [(3_500_000, (1, 1), "1ms"), (4_000_003, (3, 2), "1ms"), (4_000_003, (1, 1), "10ms"), (4_000_003, (3, 2), "10ms"),
+                                          (4_000_003, (1, 1), "0.1ms"), (4_000_003, (1, 1), "pairs"), (4_000_003, (1, 2), "pairs"), (16_000_000, (1, 1), "1ms"),
+                                          (16_000_000, (3, 2), "10ms")])
+def test_large_traces_by_a_coarse_clock(n, shape, kind):
+    # buckets of ticks in which hundreds are equal, or take a few neighbouring values: sorted where they are, without further launches
+    import torch
+    from paper_2502_11417_b200 import Trace, api
+    rng = np.random.default_rng(n + len(kind))
+    x = np.clip(_crowded(kind, n, rng), 1e-6, 2000.0).astype(np.float32)
+    g_of = rng.integers(0, shape[0] * shape[1], n).astype(np.uint8)
+    cols = [np.full(n, 7, np.int32), np.full(n, 5, np.int32), x, g_of // shape[1], g_of % shape[1]]
+    dev = [torch.from_numpy(c).cuda() for c in cols]
+    ticks = np.rint(x.astype(np.float64) * 1e6).astype(np.int64)
+    tr = Trace()
+    before = api.lib().disco_kernel_launch_count()
+    tr.load_trace(*dev, [synth.server()] * shape[0], [synth.device(500.0, 20.0)] * shape[1])
+    assert api.lib().disco_kernel_launch_count() == before + 6
+    for g in range(tr.n_groups):
+        want = np.sort(ticks[g_of == g])
+        cnt, knots, got = tr.group_tables(g)
+        assert (got == want).all() and cnt[7] == len(want)
+        assert (knots == want[np.arange(257, dtype=np.int64) * (len(want) - 1) // 256]).all()
+    tr.close()
+
+
 @pytest.mark.parametrize("shape", [(1, 1), (2, 3), (8, 8)])
 @pytest.mark.parametrize("n", [1, 255, 257, 1500])
 def test_rows_of_several_groups(n, shape):
