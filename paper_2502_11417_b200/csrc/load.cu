@@ -200,7 +200,7 @@ k_load(const __grid_constant__ LoadArgs a) {
 
     // ---- 2. place
     if (__ldcg(&z->err[0])) {                          // a rejected trace: nothing is placed
-        if (kTrace && blockIdx.x == 0 && tid < 4) a.readback->err[tid] = __ldcg(&z->err[tid]);
+        if (SRC != S_TICKS && blockIdx.x == 0 && tid < 4 && a.readback) a.readback->err[tid] = __ldcg(&z->err[tid]);
         return;
     }
     // where every bucket starts: the groups one after another, so one running sum over all groups' counters each
@@ -391,6 +391,8 @@ k_load(const __grid_constant__ LoadArgs a) {
         for (int g = 0; g < G; ++g)                                    // (the last blocks have the fewest windows)
             if ((uint32_t)(G - 1 - g) % gridDim.x == gridDim.x - 1 - blockIdx.x)
                 group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
+    }
+    if (kTrace || (SRC == S_TTFT && a.readback)) {
         // the last block to come here reports the flags (where a block has left, none does: what the host put there stands)
         if (tid == 0) { __threadfence(); s_item = atomicAdd(&z->done, 1u); }
         __syncthreads();
@@ -461,6 +463,10 @@ cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st) {
     return once_ticks(a.n, a.G, (uint32_t)sms) ? run_sort_ticks_once(a, sms, st) : launch_load<S_TICKS, F_COLUMNS>(a, sms, st);
 }
 
+cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st) {
+    return once_ticks(a.n, a.G, (uint32_t)sms) ? run_sort_ttft_once(a, sms, st) : launch_load<S_TTFT, F_COLUMNS>(a, sms, st);
+}
+
 cudaError_t launch_tables_imported(int G, const uint32_t* cnt, int64_t* cum_mass, const int32_t* F_sorted,
                                    const uint32_t* F_off, int32_t* knots, cudaStream_t st) {
     k_tables_imported<<<G, kThreads, 0, st>>>(cnt, cum_mass, F_sorted, F_off, knots);
@@ -486,6 +492,7 @@ constexpr size_t kNaCountsBytes = (256u * ((kNoAllocMaxN + 1023u) / 1024u) + 256
 // (they lie there twice: a call clears the half that the next one uses)
 constexpr size_t kNaZeroOff = 2 * kNaKeysBytes + kNaCountsBytes;
 constexpr size_t kNaZeroBytes = (sizeof(LoadZero) + kTickBins * 4 + kOnceWindows * 16 + 15) / 16 * 16;
+static_assert(sort_windows(kNoAllocMaxN, 1) * 8 <= kOnceWindows * 16, "k_load's windows");
 constexpr size_t kNaStartOff = kNaZeroOff + 2 * kNaZeroBytes;
 constexpr size_t kNaOffOff = kNaStartOff + kTickBins * 4;
 
@@ -550,6 +557,9 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
         zeroed = h.zero[half];
         h.zero[0] = h.zero[1] = false;    // (until the call has succeeded)
     }
+#ifdef DISCO_DEBUG
+    if (const char* few = std::getenv("DISCO_DEBUG_MULTIPROCESSORS")) sms = std::max(1, std::min(sms, std::atoi(few)));
+#endif
     LoadArgs a = {};
     a.n = n; a.G = 1; a.ns = a.nd = 1;
     a.ttft = server_ttft_s;
@@ -558,6 +568,7 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
     a.once.zeroed = zeroed; a.once.clear = (uint4*)next; a.once.clear_vecs = (uint32_t)(kNaZeroBytes / 16);
     a.readback = (LoadReadback*)report_dev;                          // (its flags alone)
     a.once.windows = (unsigned long long*)(a.tick_cnt + kTickBins);
+    a.windows = (uint2*)a.once.windows;
     a.tick_start = (uint32_t*)(base + kNaStartOff);
     a.binned = (uint32_t*)base; a.sorted = sorted_ticks;
     a.zero_bytes = kNaZeroBytes;          // the array still holds the previous call's data: flags and counters must start at zero
@@ -573,7 +584,7 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
     if (!report && (e = cudaMemcpyAsync(h_err, a.z->err, sizeof h_err, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return fail_after_launch(e);
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
     if (report) std::memcpy(h_err, report, sizeof h_err);
-    if (h_err[3] != 2) {
+    if (h_err[3] != 2 && once_ticks(n, 1, (uint32_t)sms)) {          // (k_load clears its own half alone)
         std::lock_guard<std::mutex> lock(g_na_mutex);
         g_na_half[dev].zero[half ^ 1] = true;
     }

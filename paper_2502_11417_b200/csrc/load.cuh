@@ -131,6 +131,7 @@ inline bool once_trace(uint32_t n, int G, uint32_t sms) {
 inline bool once_ticks(uint32_t n, int G, uint32_t sms) { return G <= 16 && n <= std::min(sms, kLoadBlocks) * 8192u; }
 cudaError_t run_load_once(const LoadArgs& a, int sms, cudaStream_t st);
 cudaError_t run_sort_ticks_once(const LoadArgs& a, int sms, cudaStream_t st);
+cudaError_t run_sort_ttft_once(const LoadArgs& a, int sms, cudaStream_t st);
 cudaError_t run_sort_ticks(const LoadArgs& a, int sms, cudaStream_t st);    // ticks, off, G, n -> sorted
 cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st);     // ttft, n (one group) -> sorted
 

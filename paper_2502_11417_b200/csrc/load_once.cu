@@ -384,6 +384,6 @@ DBG_TRANSLATION_UNIT()
 
 cudaError_t run_load_once(const LoadArgs& a, int sms, cudaStream_t st) { return plan_and_launch<S_TRACE>(a, sms, st); }
 cudaError_t run_sort_ticks_once(const LoadArgs& a, int sms, cudaStream_t st) { return plan_and_launch<S_TICKS>(a, sms, st); }
-cudaError_t run_sort_ttft(const LoadArgs& a, int sms, cudaStream_t st) { return plan_and_launch<S_TTFT>(a, sms, st); }
+cudaError_t run_sort_ttft_once(const LoadArgs& a, int sms, cudaStream_t st) { return plan_and_launch<S_TTFT>(a, sms, st); }
 
 }  // namespace disco

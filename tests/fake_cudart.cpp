@@ -19,6 +19,9 @@ uint64_t copied = 0, loads = 0;                 // bytes copied out of the range
 const void* last_ticks = nullptr;               // what the last of them was given
 const void* last_stats = nullptr;               // where the statistics' kernel was to write on the host
 uint32_t first_packed = 0;                      // ... and the lengths of the first request, if it was given a packed trace
+unsigned last_blocks = 0;                       // ... its grid, and whether its words were said to be zero
+bool last_zeroed = false;
+int multiprocessors = 148;
 struct Write { void* to; const void* from; size_t bytes; };
 std::vector<Write> pending;                     // work that a stream still holds
 void finish() {
@@ -30,12 +33,14 @@ const Range* range_of(const void* p) {
     for (const Range& r : ranges) if ((const char*)p >= r.at && (const char*)p < r.at + r.bytes) return &r;
     return nullptr;
 }
-cudaError_t launch(const void* f, void** args) {
+cudaError_t launch(const void* f, dim3 grid, void** args) {
     if (kernels[f].find("k_finalize") != std::string::npos) last_stats = *(const void**)args[8];
     if (kernels[f].find("k_load") == std::string::npos) return cudaSuccess;
     const disco::LoadArgs& a = *(const disco::LoadArgs*)args[0];
     ++loads;
     last_ticks = a.ticks;
+    last_blocks = grid.x;
+    last_zeroed = a.once.zeroed;
     if (a.packed) first_packed = *(const uint32_t*)a.packed;
     if (a.readback) {
         std::memset(a.readback, 0, sizeof *a.readback);
@@ -54,6 +59,9 @@ uint64_t fake_loads(void) { return loads; }
 const void* fake_last_ticks(void) { return last_ticks; }
 const void* fake_last_stats(void) { return last_stats; }
 uint32_t fake_first_packed(void) { return first_packed; }
+unsigned fake_last_blocks(void) { return last_blocks; }
+int fake_last_zeroed(void) { return last_zeroed; }
+void fake_multiprocessors(int n) { multiprocessors = n; }
 void fake_pending(void* to, const void* from, size_t bytes) { pending.push_back({to, from, bytes}); }
 
 // ---- what the library calls
@@ -64,10 +72,10 @@ void __cudaRegisterFunction(void**, const char* f, char*, const char* name, int,
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, struct CUstream_st*) { return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3*, dim3*, size_t* smem, void* stream) { *smem = 0; *(void**)stream = nullptr; return cudaSuccess; }
-cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t, cudaStream_t) { return launch(f, args); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* f, void** args) { return launch(f, args); }
+cudaError_t cudaLaunchKernel(const void* f, dim3 grid, dim3, void** args, size_t, cudaStream_t) { return launch(f, grid, args); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) { return launch(f, c->gridDim, args); }
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
-cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = multiprocessors; return cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 1; return cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t n) {
@@ -94,7 +102,14 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
     a->hostPointer = r && r->type != cudaMemoryTypeDevice ? (void*)p : nullptr;
     return cudaSuccess;
 }
-cudaError_t cudaGetSymbolAddress(void**, const void*) { return cudaErrorInvalidValue; }
+cudaError_t cudaGetSymbolAddress(void** p, const void*) {
+    static void* at = nullptr;
+    if (!at) cudaMalloc(&at, 16 << 20);
+    *p = at;
+    return cudaSuccess;
+}
+cudaError_t cudaHostRegister(void*, size_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaHostGetDevicePointer(void** p, void* host, unsigned) { *p = host; return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { finish(); return cudaSuccess; }
 cudaError_t cudaStreamQuery(cudaStream_t) { return pending.empty() ? cudaSuccess : cudaErrorNotReady; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)&ranges; return cudaSuccess; }

@@ -134,6 +134,33 @@ def test_totals_of_a_block_that_is_late():
     assert r.returncode == 0 and "late" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
 
 
+FEW = """
+import numpy as np, torch
+from paper_2502_11417_b200 import DiscoError
+from paper_2502_11417_b200.api import sort_ttft_ticks_noalloc
+rng = np.random.default_rng(3)
+for n in (5000, 131072, 131073, 5000, 200001, 262144, 9000, 262143):
+    for wide in (False, True):                      # (the second: left to the radix sort)
+        x = (1000.0 + 100.0 * rng.random(n) if wide else np.exp(rng.normal(-0.5, 0.9, n))).astype(np.float32)
+        out = torch.empty(n, dtype=torch.int32, device="cuda")
+        got = sort_ttft_ticks_noalloc(torch.from_numpy(x).cuda(), out).cpu().numpy()
+        assert (got == np.sort(np.rint(x.astype(np.float64) * 1e6))).all(), (n, wide)
+    x[n // 2] = float("nan")
+    try:
+        sort_ttft_ticks_noalloc(torch.from_numpy(x).cuda(), out)
+        raise AssertionError("a value out of range was taken")
+    except DiscoError as e:
+        assert e.code == -1
+print("few")
+"""
+
+
+def test_allocation_free_sort_on_few_multiprocessors():
+    # more than 8,192 values a multiprocessor: a kernel that reads them twice
+    r = _run(["-c", FEW], DISCO_DEBUG_MULTIPROCESSORS="16")
+    assert r.returncode == 0 and "few" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
+
+
 def test_the_ordinary_build_has_no_selftest():
     from paper_2502_11417_b200 import api
     if os.environ.get("DISCO_CHECKED_BUILD") == "1":

@@ -175,3 +175,24 @@ fake.fake_memory(room.ctypes.data, room.nbytes, HOST, 0)
 assert L.disco_reduce_stats(ctx, C.c_void_p(stats), None) == 0, L.disco_last_error()
 assert (fake.fake_last_stats() == stats) == {offset % 8 == 0}
 """)
+
+
+@pytest.mark.parametrize("sms", [1, 16, 31, 32, 148])
+def test_allocation_free_sort_whatever_the_multiprocessors(fake, sms):
+    # the kernel whose threads keep their values takes 8,192 a multiprocessor; the other one takes the rest, and clears what it
+    # needs alone
+    _run(fake, f"""
+fake.fake_multiprocessors({sms})
+x, out = np.full(262144, 0.5, np.float32), np.zeros(262144, np.int32)
+fits = 8192 * {sms}
+clear = False
+for n in (5000, 1, 5000, fits, fits + 1, 5000, 262144, 262144, 5000, 5000):
+    n = min(n, 262144)
+    loads = fake.fake_loads()
+    rc = L.disco_sort_ttft_ticks_noalloc(C.c_void_p(x.ctypes.data), n, C.c_void_p(out.ctypes.data), None)
+    assert rc == 0, (n, L.disco_last_error())
+    assert fake.fake_loads() == loads + 1 and 1 <= fake.fake_last_blocks() <= {sms}
+    if n <= fits:
+        assert bool(fake.fake_last_zeroed()) == clear, n
+    clear = n <= fits
+""")
