@@ -268,10 +268,10 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     const size_t o_parted = lay.take(large ? N * 16 : 0), o_rec_of = lay.take(large ? (size_t)G * (kMaxPrompt + 1) * 2 : 0);
     const size_t o_tick_of = lay.take(large ? (size_t)G * kTickBins * 2 : 0), o_at = lay.take(large ? ((size_t)lg.n_rec + lg.n_tick + 4) * 4 : 0);
     const size_t o_members = lay.take(large ? ((size_t)lg.n_rec + lg.n_tick) * 8 : 0);
-    const cudaError_t e = c->trace_mem.reserve(lay.bytes);
-    if (e) return e;
-    char* base = (char*)c->trace_mem.p;
     disco_ctx::Halves& hv = c->halves;
+    const cudaError_t e = c->trace_mem.reserve(lay.bytes);
+    if (e) { hv = disco_ctx::Halves(); return e; }                   // (a later buffer may lie where the one that was given back did)
+    char* base = (char*)c->trace_mem.p;
     if (!once || hv.at != base || hv.cap != c->trace_mem.cap || hv.bytes != c->zero_bytes) {
         hv = disco_ctx::Halves();
         if (once) { hv.at = base; hv.cap = c->trace_mem.cap; hv.bytes = c->zero_bytes; }

@@ -22,6 +22,10 @@ uint32_t first_packed = 0;                      // ... and the lengths of the fi
 unsigned last_blocks = 0;                       // ... its grid, and whether its words were said to be zero
 bool last_zeroed = false;
 int multiprocessors = 148;
+size_t device_left = ~(size_t)0;                // bytes that cudaMalloc gives out
+std::map<void*, size_t> device;                 // what it has given out
+std::vector<std::pair<void*, size_t>> given_back;
+cudaError_t last_error = cudaSuccess;
 struct Write { void* to; const void* from; size_t bytes; };
 std::vector<Write> pending;                     // work that a stream still holds
 void finish() {
@@ -62,6 +66,7 @@ uint32_t fake_first_packed(void) { return first_packed; }
 unsigned fake_last_blocks(void) { return last_blocks; }
 int fake_last_zeroed(void) { return last_zeroed; }
 void fake_multiprocessors(int n) { multiprocessors = n; }
+void fake_device_left(uint64_t bytes) { device_left = bytes; }
 void fake_pending(void* to, const void* from, size_t bytes) { pending.push_back({to, from, bytes}); }
 
 // ---- what the library calls
@@ -78,13 +83,28 @@ cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = multiprocessors; return cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 1; return cudaSuccess; }
-cudaError_t cudaMalloc(void** p, size_t n) {
+cudaError_t cudaMallocHost(void** p, size_t n) {
     // (a mapping: large sizes cost nothing until they are touched; not given back, a case is a short process)
     *p = mmap(nullptr, n, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
     return *p != MAP_FAILED ? cudaSuccess : cudaErrorMemoryAllocation;
 }
-cudaError_t cudaMallocHost(void** p, size_t n) { return cudaMalloc(p, n); }
-cudaError_t cudaFree(void*) { return cudaSuccess; }
+cudaError_t cudaMalloc(void** p, size_t n) {
+    if (n > device_left) { last_error = cudaErrorMemoryAllocation; return last_error; }
+    // what was given back is given out again, with what has been written there
+    for (auto f = given_back.begin(); f != given_back.end(); ++f)
+        if (f->second == n) { *p = f->first; given_back.erase(f); device[*p] = n; device_left -= n; return cudaSuccess; }
+    const cudaError_t e = cudaMallocHost(p, n);
+    if (e == cudaSuccess) { device[*p] = n; device_left -= n; }
+    return e;
+}
+cudaError_t cudaFree(void* p) {
+    const auto f = device.find(p);
+    if (f == device.end()) return cudaSuccess;
+    device_left += f->second;
+    given_back.push_back(*f);
+    device.erase(f);
+    return cudaSuccess;
+}
 cudaError_t cudaFreeHost(void*) { return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* to, const void* from, size_t n, cudaMemcpyKind, cudaStream_t) {
     finish();                                     // (in stream order)
@@ -119,6 +139,6 @@ cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0.
 cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaGetLastError(void) { return cudaSuccess; }
+cudaError_t cudaGetLastError(void) { const cudaError_t e = last_error; last_error = cudaSuccess; return e; }
 const char* cudaGetErrorString(cudaError_t) { return "an error of the fake runtime"; }
 }

@@ -196,3 +196,20 @@ for n in (5000, 1, 5000, fits, fits + 1, 5000, 262144, 262144, 5000, 5000):
         assert bool(fake.fake_last_zeroed()) == clear, n
     clear = n <= fits
 """)
+
+
+def test_a_load_behind_one_that_found_no_memory(fake):
+    # a context remembers which of its words the last load has cleared for the next one: not when their memory was given back in
+    # between, though the next buffer may lie in the same place
+    _run(fake, """
+fake.fake_device_left.argtypes = [C.c_uint64]
+ctx = C.c_void_p(None)
+keep, cols = host_columns(50000)
+for known in (0, 1, 1):
+    assert load(ctx, 50000, cols) == 0 and fake.fake_last_zeroed() == known, L.disco_last_error()
+more, many = host_columns(100000)
+fake.fake_device_left(1 << 20)
+assert load(ctx, 100000, many) == -2 and b"device allocation" in L.disco_last_error()
+assert load(ctx, 50000, cols) == 0 and fake.fake_last_zeroed() == 0, L.disco_last_error()
+assert load(ctx, 50000, cols) == 0 and fake.fake_last_zeroed() == 1, L.disco_last_error()
+""")
