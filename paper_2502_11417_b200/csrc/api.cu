@@ -314,11 +314,18 @@ int fetch_knots(disco_ctx* c, cudaStream_t st) {
 }
 
 // Pinned staging of at least that many bytes, once the copies or the kernel of an earlier call no longer read it.
-int reserve_stage(disco_ctx* c, size_t bytes) {
+int reserve_stage(disco_ctx* c, size_t bytes, cudaStream_t st) {
     if (c->stage_free) CU(cudaEventSynchronize(c->stage_free));
     else CU(cudaEventCreateWithFlags(&c->stage_free, cudaEventDisableTiming));
-    if (*c->stage_read != c->stage_turn) {       // (two evaluations in a row: no event behind the kernel, which would hold the next one up)
-        CU(cudaDeviceSynchronize());
+    // Two evaluations in a row: the first one's kernel puts its number into stage_read.  (An event behind that kernel would hold the
+    // next one up.)  The stream is asked as well, since what the earlier evaluation launched lies in front of this one: nothing
+    // else on the device is waited for.
+    while (*c->stage_read != c->stage_turn) {
+        const cudaError_t e = cudaStreamQuery(st);
+        if (e == cudaErrorNotReady) { cudaGetLastError(); continue; }
+        CU(e);
+        if (*c->stage_read == c->stage_turn) break;
+        CU(cudaDeviceSynchronize());                                 // (it lay on another stream, against the rules)
         *c->stage_read = c->stage_turn;
     }
     if (bytes > c->stage_cap) {
@@ -940,7 +947,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     // ---- small tables to the device with k_prep: one block, 16-byte aligned regions
     const bool in_launch = table_bytes <= kTablesInline;
     if (in_launch) c->tables_host.resize(kTablesInline / sizeof(uint4));
-    else if (int rc = reserve_stage(c, table_bytes)) return rc;
+    else if (int rc = reserve_stage(c, table_bytes, st)) return rc;
     char *sp = in_launch ? (char*)c->tables_host.data() : (char*)c->stage, *dt = mem + o_tables;
     size_t off = 0;
     auto put = [&](const void* src, size_t bytes) {
@@ -1224,7 +1231,7 @@ int disco_set_group_tables(disco_ctx_t* c, const int64_t* cnt, const int32_t* ti
     const int G = c->G;
     const size_t L = kLengths;
     uint64_t total = 0;
-    if (int rc = reserve_stage(c, ((size_t)G * L + kMaxGroups + 1) * 4)) return rc;
+    if (int rc = reserve_stage(c, ((size_t)G * L + kMaxGroups + 1) * 4, st)) return rc;
     uint32_t *cnt32 = (uint32_t*)c->stage, *off = cnt32 + (size_t)G * L;      // counts of all groups, then the groups' offsets
     off[0] = 0;
     for (int g = 0; g < G; ++g) {

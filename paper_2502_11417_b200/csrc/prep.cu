@@ -135,7 +135,7 @@ k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __re
     __syncthreads();
     if (BYTES == 0 && threadIdx.x == 0) {
         __threadfence();
-        if (atomicInc(in.left, gridDim.x - 1u) == gridDim.x - 1u) *in.read = in.turn;
+        if (atomicInc(in.left, gridDim.x - 1u) == gridDim.x - 1u) { __threadfence_system(); *in.read = in.turn; }
     }
     if (idx < pairs) {
         const uint32_t p = idx / (uint32_t)G;

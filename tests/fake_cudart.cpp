@@ -28,9 +28,14 @@ std::vector<std::pair<void*, size_t>> given_back;
 cudaError_t last_error = cudaSuccess;
 struct Write { void* to; const void* from; size_t bytes; };
 std::vector<Write> pending;                     // work that a stream still holds
+struct Word { volatile uint32_t* to; uint32_t value; };
+std::vector<Word> reports;                      // words that kernels under way will write
+uint64_t device_waits = 0;
 void finish() {
     for (const Write& w : pending) std::memcpy(w.to, w.from, w.bytes);
+    for (const Word& w : reports) *w.to = w.value;
     pending.clear();
+    reports.clear();
 }
 
 const Range* range_of(const void* p) {
@@ -39,6 +44,10 @@ const Range* range_of(const void* p) {
 }
 cudaError_t launch(const void* f, dim3 grid, void** args) {
     if (kernels[f].find("k_finalize") != std::string::npos) last_stats = *(const void**)args[8];
+    if (kernels[f].find("k_prep") != std::string::npos && kernels[f].find("k_prep_beta") == std::string::npos) {
+        const disco::TablesIn& in = *(const disco::TablesIn*)args[8];
+        if ((size_t)in.vecs * 16 > disco::kTablesInline) reports.push_back({in.read, in.turn});
+    }
     if (kernels[f].find("k_load") == std::string::npos) return cudaSuccess;
     const disco::LoadArgs& a = *(const disco::LoadArgs*)args[0];
     ++loads;
@@ -67,6 +76,7 @@ unsigned fake_last_blocks(void) { return last_blocks; }
 int fake_last_zeroed(void) { return last_zeroed; }
 void fake_multiprocessors(int n) { multiprocessors = n; }
 void fake_device_left(uint64_t bytes) { device_left = bytes; }
+uint64_t fake_device_waits(void) { return device_waits; }
 void fake_pending(void* to, const void* from, size_t bytes) { pending.push_back({to, from, bytes}); }
 
 // ---- what the library calls
@@ -131,7 +141,12 @@ cudaError_t cudaGetSymbolAddress(void** p, const void*) {
 cudaError_t cudaHostRegister(void*, size_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaHostGetDevicePointer(void** p, void* host, unsigned) { *p = host; return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { finish(); return cudaSuccess; }
-cudaError_t cudaStreamQuery(cudaStream_t) { return pending.empty() ? cudaSuccess : cudaErrorNotReady; }
+cudaError_t cudaStreamQuery(cudaStream_t) {
+    if (pending.empty() && reports.empty()) return cudaSuccess;
+    if (pending.empty()) finish();                // (kernels get on meanwhile)
+    return cudaErrorNotReady;
+}
+cudaError_t cudaDeviceSynchronize(void) { ++device_waits; finish(); return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)&ranges; return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }

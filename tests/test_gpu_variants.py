@@ -352,3 +352,29 @@ def test_tokens_that_are_certain_not_to_decide(n, tbt):
     w.servers = [synth.server(tbt_s=max(tbt, 1e-6), jitter=0.0), synth.server(tbt_s=0.04, jitter=0.2)]
     w.devices = [synth.device(20.0, 1.0 / max(tbt, 1e-6), jitter=0.0), synth.device(300.0, 25.0, jitter=0.2, c_prefill=5e-3, c_decode=5e-3)]
     full_parity(w, [synth.policy(b, r_c=20.0, t_m_s=t, flags=PACED) for b in (0.4, 1.0) for t in (0.05, 0.1, 0.4)], select=False, tag=f"{n} {tbt}")
+
+
+@pytest.mark.parametrize("policies", [64, 1024])
+def test_evaluations_in_a_row_wait_for_no_other_stream(policies):
+    # beyond some 430 policies their tables are read from page-locked memory, which the next evaluation writes again
+    import torch
+    from paper_2502_11417_b200 import Trace
+    w = synth.tiny_workload(3, 5000)
+    pols = [[synth.policy(top * k / (policies - 1)) for k in range(policies)] for top in (1.0, 0.5)]
+    mine, other, done = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Event()
+    t = Trace.from_workload(w, stream=mine)
+    with torch.cuda.stream(mine):
+        want = []
+        for p in pols:
+            t.eval_policies(p, 1)
+            want.append([bytes(s) for s in t.reduce_stats()])
+        with torch.cuda.stream(other):
+            torch.cuda._sleep(1_000_000_000)                   # about half a second
+            done.record()
+        torch.cuda._sleep(20_000_000)                          # (the first evaluation's tables have not been read when the next one comes)
+        for turn in range(8):
+            t.eval_policies(pols[turn % 2], 1)
+        got = [bytes(s) for s in t.reduce_stats()]
+        assert not done.query()
+        assert got == want[1] and got != want[0]
+    done.synchronize()
