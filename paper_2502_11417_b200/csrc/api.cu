@@ -142,6 +142,8 @@ struct disco_ctx {
     bool fin_imported = false;         // fin_totals holds a caller's merged totals, not this trace's
     std::vector<uint64_t> fin_own;     // this trace's totals, to put back before the next evaluation
     LargeLoad large;                   // working memory of a large trace's load
+    bool large_now = false;            // this trace is loaded by load_large.cu's kernels
+    size_t trace_too_much = ~(size_t)0, rec_too_much = ~(size_t)0;   // bytes that trace_mem and rec_mem could not get, at least
     bool inv_there = false;            // `inv` has been written
     // What a load must clear lies twice in memory where load_once.cu's kernel loads the trace: it works in one half and clears the
     // other for the next load.  Where they lie (nowhere after any other load) and which of them is zero.
@@ -258,6 +260,7 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     } else if (in == IN_PACKED) {
         o_in[0] = lay.take(n > kPackInPlace ? packed_bytes(n) : 0);
     }
+    const size_t without = lay.bytes;
     const bool large = large_load(n, G);
     LargeLoad& lg = c->large;
     std::memset(&lg, 0, sizeof lg);
@@ -269,7 +272,15 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     const size_t o_tick_of = lay.take(large ? (size_t)G * kTickBins * 2 : 0), o_at = lay.take(large ? ((size_t)lg.n_rec + lg.n_tick + 4) * 4 : 0);
     const size_t o_members = lay.take(large ? ((size_t)lg.n_rec + lg.n_tick) * 8 : 0);
     disco_ctx::Halves& hv = c->halves;
-    const cudaError_t e = c->trace_mem.reserve(lay.bytes);
+    // (a large load works without its buckets, by k_load, where there is no room for them: 16 bytes a request)
+    c->large_now = large && lay.bytes < c->trace_too_much;
+    cudaError_t e = c->trace_mem.reserve(c->large_now ? lay.bytes : without);
+    if (e == cudaErrorMemoryAllocation && c->large_now) {
+        cudaGetLastError();
+        c->large_now = false;
+        c->trace_too_much = lay.bytes;
+        e = c->trace_mem.reserve(without);
+    }
     if (e) { hv = disco_ctx::Halves(); return e; }                   // (a later buffer may lie where the one that was given back did)
     char* base = (char*)c->trace_mem.p;
     if (!once || hv.at != base || hv.cap != c->trace_mem.cap || hv.bytes != c->zero_bytes) {
@@ -468,7 +479,7 @@ int disco_load_trace(disco_ctx_t** pctx, const disco_trace_desc_t* d, void* stre
     }
     static const int32_t no_report[4] = {0, 0, 0, 2};               // what the host finds if the blocks lose each other
     std::memcpy(c->rb->err, no_report, sizeof no_report);
-    const bool large = large_load(n, c->G);
+    const bool large = c->large_now;
     a.large = c->large;
     c->inv_there = !large;
     disco_ctx::Halves& hv = c->halves;
@@ -641,7 +652,15 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         for (int k = 0; k < 3; ++k) o_win[k] = slot.take(N1 * wmax[k] * 2);
     }
     const size_t rec_stride = (slot.bytes + 255) / 256 * 256;
-    const size_t wave = std::min(n_classes, std::max<size_t>(1, ((size_t)512 << 20) / rec_stride));
+    size_t wave = std::min(n_classes, std::max<size_t>(1, ((size_t)512 << 20) / rec_stride));
+    cudaError_t e;
+    while (wave > 1 && wave * rec_stride >= c->rec_too_much) wave = (wave + 1) / 2;
+    while ((e = c->rec_mem.reserve(wave * rec_stride)) == cudaErrorMemoryAllocation && wave > 1) {      // (smaller waves, then)
+        cudaGetLastError();
+        c->rec_too_much = wave * rec_stride;
+        wave = (wave + 1) / 2;
+    }
+    if (e != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
     auto slot_of = [&](size_t k) { return k % wave; };
     // A class whose free streams are those of an earlier class of its wave -- as generated, next to streams that keep the pace --
     // has them played and stored by that class.
@@ -671,9 +690,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         }
     }
     // ---- the first class's play-out needs no more than this: it runs while the host lays out the policies
-    cudaError_t e;
     {
-        if ((e = c->rec_mem.reserve(wave * rec_stride)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
         char* mem = (char*)c->rec_mem.p;
         c->play_ticket.p = mem + o_ticket; c->rec_hand.p = mem + o_hand;
         for (int k = 0; k < 6; ++k) c->rec_u32[k].p = mem + o_rec[k];
@@ -927,7 +944,13 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                                (tab.size() * 4 + 15) / 16 * 16 + (slabs.size() * sizeof(Slab) + 15) / 16 * 16;
     const size_t o_tables = lay.take(table_bytes);
     const size_t o_chunks[2] = {lay.take(tables.n_chunks[0] * sizeof(Chunk)), lay.take(tables.n_chunks[1] * sizeof(Chunk))};
-    if ((e = c->eval_mem.reserve(lay.bytes)) != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
+    if ((e = c->eval_mem.reserve(lay.bytes)) == cudaErrorMemoryAllocation && wave > 1) {
+        cudaGetLastError();                                          // (again in smaller waves, which leave more room)
+        c->rec_too_much = wave * rec_stride;
+        c->rec_mem.release();
+        return disco_eval_policies(c, pol, P, seed, out, stream);
+    }
+    if (e != cudaSuccess) return fail_cuda(e, "device allocation for the evaluation");
     char* mem = (char*)c->eval_mem.p;
     c->d_prep.p = mem + o_prep; c->d_accum.p = mem + o_accum2; c->d_stats.p = mem + o_stats; c->d_grid.p = mem + o_grid;
     c->d_left.p = mem + o_left; c->d_tables.p = mem + o_tables;

@@ -227,3 +227,38 @@ for turn in range(4):
     assert L.disco_eval_policies(ctx, pols, 1024, 1, None, None) == 0, L.disco_last_error()
     assert fake.fake_device_waits() == 0
 """)
+
+
+def test_a_large_load_without_room_for_its_buckets(fake):
+    # 4 M requests: 28 bytes each and 16 more for the buckets, which k_load does without
+    _run(fake, """
+fake.fake_device_left.argtypes = [C.c_uint64]
+L.disco_kernel_launch_count.restype = C.c_uint64
+ctx = C.c_void_p(None)
+n = 4_000_000
+cols = [unreadable(n, DEVICE) for _ in range(5)]
+fake.fake_device_left(n * 36)
+for again in range(2):
+    launches = L.disco_kernel_launch_count()
+    assert load(ctx, n, cols, 1) == 0, L.disco_last_error()
+    assert L.disco_kernel_launch_count() == launches + 1
+fake.fake_device_left(n * 20)
+c2 = C.c_void_p(None)
+assert load(c2, n, cols, 1) == -2 and b"device allocation" in L.disco_last_error()
+""")
+
+
+@pytest.mark.parametrize("room", [9 << 20, 8_001_300, 6 << 20, 3 << 20])
+def test_paces_without_room_for_all_records(fake, room):
+    # five paces are played out into records of their own, of 1.6 MB here; with less room (or what follows without any) in
+    # smaller waves
+    _run(fake, f"""
+fake.fake_device_left.argtypes = [C.c_uint64]
+ctx = C.c_void_p(None)
+keep, cols = host_columns(200000)
+assert load(ctx, 200000, cols) == 0, L.disco_last_error()
+pols = api.policy_array([synth.policy(0.5, r_c=r) for r in (2.0, 3.0, 4.0, 5.0, 6.0)])
+fake.fake_device_left({room})
+for again in range(2):
+    assert L.disco_eval_policies(ctx, pols, 5, 1, None, None) == 0, L.disco_last_error()
+""")
