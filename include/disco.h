@@ -283,8 +283,8 @@ int disco_measure_alu_peak(double* lane_instr_per_s, double* token_steps_per_s, 
  *  - n > DISCO_NOALLOC_MAX_N is refused with DISCO_EINVAL (use disco_load_trace); a TTFT that is not
  *    finite, not positive or above 2000 s gives DISCO_EINVAL after the kernels have run.
  *  - The first call on each device looks up the device address of the working array, and the first of all
- *    page-locks one page of the library's own, where the kernel reports errors; make that first
- *    call during start-up, on the device you will use (cudaSetDevice first) and before any stream
+ *    page-locks one page of the library's own, where the kernel reports errors (the first one behind a
+ *    cudaDeviceReset does so again); make that first call during start-up, on the device you will use (cudaSetDevice first) and before any stream
  *    capture begins.
  *  - All calls on a device share the one working array, which still holds the previous call's data
  *    (the call clears what it needs cleared).  Two calls whose kernels could run at the same time on

@@ -499,14 +499,12 @@ constexpr size_t kNaOffOff = kNaStartOff + kTickBins * 4;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaOffOff + 256];
 
 std::mutex g_na_mutex;
-unsigned char* g_na_base[64] = {};        // device address of the scratch array, per device ordinal
 int g_na_sms[64] = {};                    // multiprocessors, per device ordinal
 struct { bool zero[2]; int now; } g_na_half[64] = {};   // which halves are known to be zero, and which was used last
 // Where the kernel reports its flags: a page of the library's own, page-locked by the first call, 64 bytes a device ordinal.  (A
 // copy into pageable memory behind the kernel took 7 us of a call, the clearing in front of it 5: 100,000 values 35 us, now 27.)
 alignas(4096) unsigned char g_na_report[4096];
-int g_na_locked = 0;                      // 1: it is, -1: it cannot be
-void* g_na_report_dev[64] = {};           // its address on the device, per device ordinal
+bool g_na_unlockable = false;
 
 }  // namespace
 }  // namespace disco
@@ -530,28 +528,28 @@ extern "C" int disco_sort_ttft_ticks_noalloc(const float* server_ttft_s, uint32_
     int32_t* report = nullptr;
     void* report_dev = nullptr;
     {
-        // In host code the array's name is only a handle; its address on the current device has to be asked for.
+        // In host code the array's name is only a handle; its address on the current device has to be asked for, and so has the
+        // page's.  On every call: a reset of the device may move the one and takes the other away.
         std::lock_guard<std::mutex> lock(g_na_mutex);
-        if (!g_na_base[dev]) {
+        if ((e = cudaGetSymbolAddress((void**)&base, g_noalloc_scratch)) != cudaSuccess) return set_error(DISCO_ECUDA, cudaGetErrorString(e));
+        if (!g_na_sms[dev]) {
             int count = 0;
             if ((e = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess || count < 1)
                 return set_error(DISCO_ECUDA, "cannot read the multiprocessor count of the current device");
-            e = cudaGetSymbolAddress((void**)&g_na_base[dev], g_noalloc_scratch);
-            if (e != cudaSuccess) { g_na_base[dev] = nullptr; return set_error(DISCO_ECUDA, cudaGetErrorString(e)); }
             g_na_sms[dev] = count;
         }
-        base = g_na_base[dev];
         sms = g_na_sms[dev];
-        if (!g_na_locked) {
-            g_na_locked = cudaHostRegister(g_na_report, sizeof g_na_report, cudaHostRegisterPortable | cudaHostRegisterMapped) == cudaSuccess ? 1 : -1;
-            if (g_na_locked < 0) cudaGetLastError();
-        }
-        if (g_na_locked > 0 && !g_na_report_dev[dev] && cudaHostGetDevicePointer(&g_na_report_dev[dev], g_na_report + 64 * dev, 0) != cudaSuccess) {
-            g_na_report_dev[dev] = nullptr;
+        unsigned char* page = g_na_report + 64 * dev;
+        for (int locked = 0; !report && !g_na_unlockable; ++locked) {
+            if (cudaHostGetDevicePointer(&report_dev, page, 0) == cudaSuccess) { report = (int32_t*)page; break; }
             cudaGetLastError();
+            report_dev = nullptr;
+            if (locked) break;
+            if (cudaHostRegister(g_na_report, sizeof g_na_report, cudaHostRegisterPortable | cudaHostRegisterMapped) != cudaSuccess) {
+                cudaGetLastError();
+                g_na_unlockable = true;
+            }
         }
-        report_dev = g_na_report_dev[dev];
-        if (report_dev) report = (int32_t*)(g_na_report + 64 * dev);
         auto& h = g_na_half[dev];
         half = h.now ^= 1;
         zeroed = h.zero[half];

@@ -26,6 +26,9 @@ size_t device_left = ~(size_t)0;                // bytes that cudaMalloc gives o
 std::map<void*, size_t> device;                 // what it has given out
 std::vector<std::pair<void*, size_t>> given_back;
 cudaError_t last_error = cudaSuccess;
+void* symbol = nullptr;                         // where the library's device array lies
+std::map<const char*, size_t> locked;           // host memory that the library has page-locked
+const void *last_words = nullptr, *last_report = nullptr;
 struct Write { void* to; const void* from; size_t bytes; };
 std::vector<Write> pending;                     // work that a stream still holds
 struct Word { volatile uint32_t* to; uint32_t value; };
@@ -54,6 +57,8 @@ cudaError_t launch(const void* f, dim3 grid, void** args) {
     last_ticks = a.ticks;
     last_blocks = grid.x;
     last_zeroed = a.once.zeroed;
+    last_words = a.z;
+    last_report = a.readback;
     if (a.packed) first_packed = *(const uint32_t*)a.packed;
     if (a.readback) {
         std::memset(a.readback, 0, sizeof *a.readback);
@@ -76,6 +81,9 @@ unsigned fake_last_blocks(void) { return last_blocks; }
 int fake_last_zeroed(void) { return last_zeroed; }
 void fake_multiprocessors(int n) { multiprocessors = n; }
 void fake_device_left(uint64_t bytes) { device_left = bytes; }
+void fake_reset_device(void) { symbol = nullptr; locked.clear(); }
+int fake_last_words_in_place(void) { return last_words >= symbol && (const char*)last_words < (const char*)symbol + (16 << 20); }
+int fake_last_report_locked(void) { void* p; return cudaHostGetDevicePointer(&p, (void*)last_report, 0) == cudaSuccess; }
 uint64_t fake_device_waits(void) { return device_waits; }
 void fake_pending(void* to, const void* from, size_t bytes) { pending.push_back({to, from, bytes}); }
 
@@ -133,13 +141,15 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
     return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) {
-    static void* at = nullptr;
-    if (!at) cudaMalloc(&at, 16 << 20);
-    *p = at;
+    if (!symbol) cudaMallocHost(&symbol, 16 << 20);
+    *p = symbol;
     return cudaSuccess;
 }
-cudaError_t cudaHostRegister(void*, size_t, unsigned) { return cudaSuccess; }
-cudaError_t cudaHostGetDevicePointer(void** p, void* host, unsigned) { *p = host; return cudaSuccess; }
+cudaError_t cudaHostRegister(void* p, size_t n, unsigned) { locked[(const char*)p] = n; return cudaSuccess; }
+cudaError_t cudaHostGetDevicePointer(void** p, void* host, unsigned) {
+    for (const auto& r : locked) if ((const char*)host >= r.first && (const char*)host < r.first + r.second) { *p = host; return cudaSuccess; }
+    return last_error = cudaErrorInvalidValue;
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t) { finish(); return cudaSuccess; }
 cudaError_t cudaStreamQuery(cudaStream_t) {
     if (pending.empty() && reports.empty()) return cudaSuccess;

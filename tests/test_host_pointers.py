@@ -262,3 +262,16 @@ fake.fake_device_left({room})
 for again in range(2):
     assert L.disco_eval_policies(ctx, pols, 5, 1, None, None) == 0, L.disco_last_error()
 """)
+
+
+def test_allocation_free_sort_after_a_device_reset(fake):
+    # a reset moves the library's array and takes the page away where the kernel reports
+    _run(fake, """
+x, out = np.full(9000, 0.5, np.float32), np.zeros(9000, np.int32)
+for reset in (False, False, True, False, True):
+    if reset:
+        fake.fake_reset_device()
+    rc = L.disco_sort_ttft_ticks_noalloc(C.c_void_p(x.ctypes.data), 9000, C.c_void_p(out.ctypes.data), None)
+    assert rc == 0, L.disco_last_error()
+    assert fake.fake_last_words_in_place() and fake.fake_last_report_locked()
+""")
