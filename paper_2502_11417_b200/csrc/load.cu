@@ -1,6 +1,8 @@
-// Trace ingestion on the device in one kernel: tick conversion and validation, per-group prompt-length histogram,
-// internal request order (by group, then by prompt length), sort of the server-TTFT ticks (the empirical F of
-// Algorithm 1), cumulative input-token mass (Eq. 3) and the quantile knots of F.
+// Trace ingestion on the device in one kernel, for the traces that load_once.cu and load_large.cu do not take (1.2 to 3.5 million
+// requests, more than seven groups, beyond 2^24 requests, or without room for load_large.cu's buckets), and the sort of as many
+// ticks: tick conversion and validation, per-group prompt-length histogram, internal request order (by group, then by prompt
+// length), sort of the server-TTFT ticks (the empirical F of Algorithm 1), cumulative input-token mass (Eq. 3) and the quantile
+// knots of F.
 //
 // One block of 1024 threads per multiprocessor, all resident at once (a cooperative launch), works in three passes with a
 // wait for all blocks between them:
@@ -14,10 +16,10 @@
 //      few low bits), each window by one block.  A bin of more than 8,192 ticks that spans at most 2^18 values is sorted by
 //      counting them; a trace that has a denser and wider one goes to the radix sort (radix.cu) instead.
 //
-// Bound: latency at 10^5 requests (one launch instead of eighteen), scattered stores at 10^6: the columns are read twice (once
-// when they are in host memory: then the first pass leaves a copy), 20 bytes a request are written to scattered places, the ticks
-// are read and written once more.  A million requests: 58 us.  From 3.5 million on load_large.cu is the faster one.  (The 64
-// registers that 1,024 threads leave spill 64 bytes.)
+// Bound: latency up to some 10^5 requests, then scattered stores: the columns are read twice (once when they are in host memory:
+// then the first pass leaves a copy), 20 bytes a request are written to scattered places, the ticks are read and written once
+// more.  2 million requests in one group: 84 us, 3 million 120, a million in twenty groups 115.  From 3.5 million on load_large.cu is
+// the faster one.  (The 64 registers that 1,024 threads leave spill 64 bytes.)
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
@@ -32,7 +34,6 @@ namespace {
 // Waits until every block of the grid has come here `times` times.  False, to all threads: the block has to leave.
 __device__ __forceinline__ bool grid_barrier(LoadZero* z, uint32_t times, uint32_t absent) {
     __syncthreads();
-    if (gridDim.x == 1) return true;
     bool lost = false;
     if (threadIdx.x == 0) {
         __threadfence();
@@ -103,11 +104,7 @@ k_load(const __grid_constant__ LoadArgs a) {
     uint32_t waits = 0;
 
     // the block's counters join the global ones; what it finds there is where its own requests go within the bucket
-    auto join = [&](uint32_t* mine, uint32_t* all, int count, bool store) {
-        if (store) {
-            for (int i = tid; i < count; i += kThreads) { all[i] = mine[i]; mine[i] = 0; }
-            return;
-        }
+    auto join = [&](uint32_t* mine, uint32_t* all, int count) {
 #pragma unroll 1
         for (int i0 = tid; i0 < count; i0 += 4 * kThreads) {
             uint32_t c[4];
@@ -121,15 +118,6 @@ k_load(const __grid_constant__ LoadArgs a) {
     };
 
     // ---- 1. count
-    const bool alone = gridDim.x == 1;                                 // then nothing has been cleared, and nothing is shared
-    if (alone) {
-        for (int i = tid; i < (int)(sizeof(LoadZero) / 4); i += kThreads) ((uint32_t*)z)[i] = 0;
-        for (int i = tid; i < (int)sort_windows(a.n, G); i += kThreads) a.windows[i] = make_uint2(0u, 0u);
-        if (!PRIV) {
-            for (int i = tid; i < G * kTickBins; i += kThreads) a.tick_cnt[i] = 0;
-            if (kTrace) for (int i = tid; i < G * kLens; i += kThreads) a.cnt[i] = 0;
-        }
-    }
     if (PRIV) for (int i = tid; i < (kTrace ? G * kLens : 0) + G * kTickBins; i += kThreads) s_tick[i] = 0;
     if (SRC == S_TICKS) for (int g = tid; g <= G; g += kThreads) s_off[g] = a.off[g];
     for (int g = tid; g < G; g += kThreads) s_sum[g] = 0;
@@ -192,8 +180,8 @@ k_load(const __grid_constant__ LoadArgs a) {
         if (tid == 0 && s_max) atomicMax(&z->max_n, s_max);
     }
     if (PRIV) {
-        if (kTrace) join(s_len, a.cnt, G * kLens, alone);
-        join(s_tick, a.tick_cnt, G * kTickBins, alone);
+        if (kTrace) join(s_len, a.cnt, G * kLens);
+        join(s_tick, a.tick_cnt, G * kTickBins);
     }
     ++waits;
     if (!grid_barrier(z, waits, ABSENT(a, waits))) return;
@@ -210,34 +198,32 @@ k_load(const __grid_constant__ LoadArgs a) {
         const Share st = share_of(G * kTickBins), sl = share_of(kTrace ? G * kLens : 0);
         const uint4 ft = four_counters(a.tick_cnt, st.k0 + tid * 4, st.k1);
         const uint4 fl = kTrace ? four_counters(a.cnt, sl.k0 + tid * 4, sl.k1) : make_uint4(0u, 0u, 0u, 0u);
-        if (!alone) {
-            uint32_t sum[2] = {ft.x + ft.y + ft.z + ft.w, fl.x + fl.y + fl.z + fl.w};
-            for (int k = st.k0 + (tid + kThreads) * 4; k < st.k1; k += 4 * kThreads) { const uint4 c = four_counters(a.tick_cnt, k, st.k1); sum[0] += c.x + c.y + c.z + c.w; }
-            if (kTrace) for (int k = sl.k0 + (tid + kThreads) * 4; k < sl.k1; k += 4 * kThreads) { const uint4 c = four_counters(a.cnt, k, sl.k1); sum[1] += c.x + c.y + c.z + c.w; }
-            if (tid < 2) s_carry[tid] = 0;
-            __syncthreads();
+        uint32_t sum[2] = {ft.x + ft.y + ft.z + ft.w, fl.x + fl.y + fl.z + fl.w};
+        for (int k = st.k0 + (tid + kThreads) * 4; k < st.k1; k += 4 * kThreads) { const uint4 c = four_counters(a.tick_cnt, k, st.k1); sum[0] += c.x + c.y + c.z + c.w; }
+        if (kTrace) for (int k = sl.k0 + (tid + kThreads) * 4; k < sl.k1; k += 4 * kThreads) { const uint4 c = four_counters(a.cnt, k, sl.k1); sum[1] += c.x + c.y + c.z + c.w; }
+        if (tid < 2) s_carry[tid] = 0;
+        __syncthreads();
 #pragma unroll
-            for (int j = 0; j < (kTrace ? 2 : 1); ++j) {
-                const uint32_t v = __reduce_add_sync(FULL, sum[j]);
-                if (lane == 0 && v) atomicAdd(&s_carry[j], v);
+        for (int j = 0; j < (kTrace ? 2 : 1); ++j) {
+            const uint32_t v = __reduce_add_sync(FULL, sum[j]);
+            if (lane == 0 && v) atomicAdd(&s_carry[j], v);
+        }
+        __syncthreads();
+        // a warp for each of the two sums: tells the other blocks, and adds up those in front
+        const int j = tid >> 5;
+        if (j < (kTrace ? 2 : 1)) {
+            if (lane == 0)
+                asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&z->part[j][blockIdx.x]), "l"(((unsigned long long)s_carry[j] << 1) | 1ull) : "memory");
+            uint32_t before = 0;
+            for (uint32_t b = lane; b < blockIdx.x && !lost; b += 32) {
+                const unsigned long long word = await_word(z, &z->part[j][b]);
+                lost = word == 0ull;
+                before += (uint32_t)(word >> 1);
             }
-            __syncthreads();
-            // a warp for each of the two sums: tells the other blocks, and adds up those in front
-            const int j = tid >> 5;
-            if (j < (kTrace ? 2 : 1)) {
-                if (lane == 0)
-                    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&z->part[j][blockIdx.x]), "l"(((unsigned long long)s_carry[j] << 1) | 1ull) : "memory");
-                uint32_t before = 0;
-                for (uint32_t b = lane; b < blockIdx.x && !lost; b += 32) {
-                    const unsigned long long word = await_word(z, &z->part[j][b]);
-                    lost = word == 0ull;
-                    before += (uint32_t)(word >> 1);
-                }
-                if (ABSENT(a, 4u) && lane == 0) lost = await_word(z, &z->part[j][kLoadBlocks - 1]) == 0ull;
-                before = __reduce_add_sync(FULL, before);
-                if (lane == 0) s_carry[j] = before;
-            }
-        } else if (tid < 2) s_carry[tid] = 0;
+            if (ABSENT(a, 4u) && lane == 0) lost = await_word(z, &z->part[j][kLoadBlocks - 1]) == 0ull;
+            before = __reduce_add_sync(FULL, before);
+            if (lane == 0) s_carry[j] = before;
+        }
         if (__syncthreads_or(lost)) return;                            // (some block's sum did not come)
         scan_share(a.tick_cnt, st, ft, s_carry[0], s_wtot, [&](int k, const uint4&, const uint4& start) {
             *reinterpret_cast<uint4*>(a.tick_start + k) = start;
@@ -345,8 +331,8 @@ k_load(const __grid_constant__ LoadArgs a) {
                     }
             }
             __syncthreads();
-            join(s_len, a.len_end, G * kLens, false);
-            join(s_tick, a.tick_at, G * kTickBins, false);
+            join(s_len, a.len_end, G * kLens);
+            join(s_tick, a.tick_at, G * kTickBins);
             __syncthreads();
             place(i_end);
             __syncthreads();
@@ -409,24 +395,20 @@ cudaError_t launch_load(const LoadArgs& a, int sms, cudaStream_t st) {
     auto* kernel = priv ? k_load<SRC, true, FORM> : k_load<SRC, false, FORM>;
     cudaError_t e = allow_smem((const void*)kernel, 220 * 1024);
     if (e) return e;
-    // One group: four requests a thread (and about a window a block) until the multiprocessors are full.  Several: each has
-    // counters, a window and a table of its own whatever the number of requests, so at least four blocks a group share that
-    // work (1,000 requests in six groups 92 -> 53 us a load, in twenty 235 -> 54), and beyond, twice as many blocks as for
-    // one group (300,000 in six groups 83 -> 76 us).
+    // One group: four requests a thread until the multiprocessors are full.  Several: each has counters, a window and a table of
+    // its own whatever the number of requests, so at least four blocks a group share that work (1,000 requests in twenty groups
+    // 235 -> 54 us a load), and beyond, twice as many blocks as for one group.
     const uint32_t per_block = (a.G > 1 ? 2u : 4u) * kThreads, least = a.G > 1 ? 4u * (uint32_t)a.G : 1u;
     const uint32_t blocks = std::min(std::max((a.n + per_block - 1) / per_block, least), std::min((uint32_t)sms, kLoadBlocks));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = blocks; cfg.blockDim = kThreads; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[1];
-    if (blocks > 1) {
-        // (one block clears its words itself and waits for nobody)
-        if ((e = cudaMemsetAsync(a.z, 0, a.zero_bytes, st))) return e;
-        if (((char*)a.windows < (char*)a.z || (char*)a.windows >= (char*)a.z + a.zero_bytes) &&
-            (e = cudaMemsetAsync(a.windows, 0, sort_windows(a.n, a.G) * sizeof(uint2), st))) return e;
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-    }
+    if ((e = cudaMemsetAsync(a.z, 0, a.zero_bytes, st))) return e;
+    if (((char*)a.windows < (char*)a.z || (char*)a.windows >= (char*)a.z + a.zero_bytes) &&
+        (e = cudaMemsetAsync(a.windows, 0, sort_windows(a.n, a.G) * sizeof(uint2), st))) return e;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
 #ifdef DISCO_DEBUG
     LoadArgs b = a;
     if (const char* wait = std::getenv("DISCO_DEBUG_ABSENT")) b.absent = (uint32_t)std::atoi(wait);

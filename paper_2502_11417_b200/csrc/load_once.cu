@@ -14,7 +14,7 @@
 // Bound: latency, some fifteen dependent steps, and from half a million requests on the scattered stores.  Against k_load, which
 // reads the requests twice and waits three times (with the memset in front of it, kernels and gaps): 100,000 requests in one group
 // 42 us -> 21, in six 56 -> 34; a million 64 -> 45 and 76 -> 57; 1,000 in one block 23 -> 17; 100,000 ticks 25 -> 15.  Where the
-// threads cannot keep their requests (8,192 a block) k_load is left.  (Eight requests a thread spill 172 bytes, four 48.)
+// threads cannot keep their requests (8,192 a block) k_load is left.  (Eight requests a thread spill 168 bytes, four 48.)
 #include <algorithm>
 #include <cstdlib>
 
@@ -308,11 +308,6 @@ k_load_once(const __grid_constant__ LoadArgs a) {
             sort_bins(a, sm, g, (int)first - g * kTickBins, (int)last - g * kTickBins, k0, k1);
             if (kTrace) write_knots<kThreads>(a, g, k0, k1, s_off[g], s_off[g + 1] - s_off[g]);
         }
-        if (kTrace && !alone && gridDim.x == blocks) {                 // no blocks to spare for the masses
-            __syncthreads();
-            for (int g = 0; g < G; ++g)
-                if ((uint32_t)(G - 1 - g) % blocks == blocks - 1 - block) group_mass(a.cnt + (size_t)g * kLens, a.cum_mass + (size_t)g * (kLens + 1), s_wide);
-        }
     }
     if (kTrace || (SRC == S_TTFT && a.readback)) {
         // the last block to come here reports the flags (where a block has left, none does: what the host put there stands)
@@ -355,7 +350,7 @@ cudaError_t plan_and_launch(const LoadArgs& args, int sms, cudaStream_t st) {
     LoadArgs a = args;
     constexpr bool kTrace = SRC == S_TRACE;
     const bool single = a.G == 1 && a.n <= kOnceAlone;
-    const uint32_t spare = kTrace && !single && (uint32_t)sms > 2u * (uint32_t)a.G ? (uint32_t)a.G : 0u;
+    const uint32_t spare = kTrace && !single ? (uint32_t)a.G : 0u;   // (once_trace has seen that there are as many)
     const uint32_t most = std::min((uint32_t)sms, kLoadBlocks) - spare;
     // a request a thread until the multiprocessors are full, and some blocks whatever the number of requests
     const uint32_t least = a.G > 1 ? 4u * (uint32_t)a.G : 2u;
