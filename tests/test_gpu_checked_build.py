@@ -69,7 +69,9 @@ def load(t, w):
     return t.load_trace(w.prompt_len, w.output_len, w.server_ttft_s, w.server_profile, w.device_profile, w.servers, w.devices)
 
 waits = os.environ["WAITS"].split()
-large, small = synth.make_workload(4, n=40000, n_budgets=2), synth.make_workload(4, n=9000, n_budgets=2)
+large = synth.make_workload(4, n=40000, n_budgets=2)
+small = {"once": lambda: synth.make_workload(4, n=9000, n_budgets=2),
+         "groups": lambda: synth.tiny_workload(4, 9000, n_servers=4, n_devices=5, max_prompt=4096, policies=[synth.policy(0.3)])}[os.environ["TRACE"]]()
 x = torch.from_numpy(large.server_ttft_s).cuda()
 out = torch.full((large.n,), -7, dtype=torch.int32, device="cuda")
 t, u = load(Trace(), large), load(Trace(), small)
@@ -95,11 +97,22 @@ print("waited")
 """
 
 
-def test_blocks_leave_when_a_wait_runs_out():
-    # each of the ingestion kernel's waits in turn (three barriers, the blocks' sums) expects an arrival that nobody makes:
-    # the call fails, nothing has been placed or sorted, and the context takes the next load
-    r = _run(["-c", WAITS], WAITS="1 2 3 4")
+@pytest.mark.parametrize("trace", ["once", "groups"])
+def test_blocks_leave_when_a_wait_runs_out(trace):
+    # each of the ingestion kernels' waits in turn expects an arrival that nobody makes: the call fails, nothing has been placed or
+    # sorted, and the context takes the next load.  Six groups are loaded, and their ticks imported, by k_load_once with its two
+    # waits (4 is the first again, 3 the second), as are the ticks of the allocation-free sort; twenty groups by k_load (three
+    # barriers, and the blocks' sums as 4).
+    r = _run(["-c", WAITS], WAITS="1 2 3 4", TRACE=trace)
     assert r.returncode == 0 and "waited" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
+
+
+def test_large_traces_with_every_index_checked():
+    # the kernels of large traces (with rows, whose requests' places are looked up, from device and page-locked memory), buckets that
+    # are crowded or left to the radix sort, and a trace that k_load places in rounds
+    r = _run(["-m", "pytest", "tests/test_gpu_variants.py", "-x", "-q", "-m", "gpu", "-k",
+              "by_way_of_buckets and (3500000 or 3508193 or 4000003 or 16777) or coarse_clock and 4000003 and pairs"])
+    assert r.returncode == 0 and " passed" in r.stdout, r.stdout[-3000:] + r.stderr[-2000:]
 
 
 LATE = """

@@ -171,10 +171,12 @@ def test_windows_under_several_overheads(n, overheads, dearer):
 @pytest.mark.parametrize("n,shape,kind,where", [(3_499_999, (1, 1), "spread", "device"), (3_500_000, (1, 1), "spread", "device"),
                                                 (3_500_001, (1, 1), "one", "device"), (3_508_193, (3, 2), "spread", "pinned"),
                                                 (3_600_013, (1, 7), "ties", "pageable"), (3_600_013, (2, 2), "dense", "unaligned"),
-                                                (4_000_003, (1, 2), "wide", "device"), (3_600_013, (2, 4), "spread", "device")])
+                                                (4_000_003, (1, 2), "wide", "device"), (3_600_013, (2, 4), "spread", "device"),
+                                                (2 ** 24 + 17, (3, 2), "spread", "device")])
 def test_large_traces_are_placed_by_way_of_buckets(n, shape, kind, where):
     # tables and statistics of traces from 3.5 M requests in up to seven groups on, and on the other side of both limits: full
-    # and partly filled tiles and buckets, lengths and bins that take a bucket to themselves, samples left to the radix sort
+    # and partly filled tiles and buckets, lengths and bins that take a bucket to themselves, samples left to the radix sort; beyond
+    # 2^24 requests k_load places them in rounds
     import torch
     from oracle import Oracle
     from paper_2502_11417_b200 import DiscoError, Trace
