@@ -46,7 +46,7 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, const __grid_constant__ FreeMore more,
                uint32_t* __restrict__ ticket, uint32_t batches, uint32_t size, bool early) {
     constexpr bool BOTH = PLAY == P_BOTH;
-    extern __shared__ __align__(16) uint32_t s_win[];         // per warp: [W0 + W1][32] counters
+    extern __shared__ __align__(16) uint32_t s_win[];         // per warp: [W0 + W1][kCols] counters
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warps = blockDim.x >> 5;
     grid_dependency_wait();
     if (early) let_next_start();
@@ -172,7 +172,7 @@ DBG_TRANSLATION_UNIT()
 
 cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0, TimelineRec rec,
                                 const FreeMore& more, uint32_t* ticket, const uint32_t* grp_n, bool early, int sms, cudaStream_t st) {
-    // as many warps to a block as the windows leave room for (wide jitter: up to 114 KB of counters a stream and warp)
+    // as many warps to a block as the windows leave room for (wide jitter: up to 27 KB of counters a stream and warp)
     const size_t per_warp = (size_t)(cc.W[0] + cc.W[1]) * kCols * 4;
     const uint32_t warps = std::max<uint32_t>(1u, std::min<uint32_t>(kFreeWarps, (uint32_t)(100 * 1024 / per_warp)));
     const size_t smem = per_warp * warps;
