@@ -389,6 +389,53 @@ struct BigSort {
 };
 static_assert(2 * (sizeof(BigSort) + 1024 + 16) <= 227 * 1024, "two blocks to a multiprocessor");
 
+// A bucket whose ticks lie in their cells (sm.cell: where each ends), where cells of different ticks reach further than kSortPad: mostly
+// a clock coarser than a microsecond, whose ticks share a cell with their like alone and need no order among themselves.  (A load of
+// 4 M requests by a millisecond's clock: 189 us, by a microsecond's 184; with a trace that has one such cell of 256 left to the
+// radix sort 454, of 16 M 1,213 and now 565.  Called, not inlined: k_sort of 16 M microsecond ticks in six groups, which do not come
+// here, 124.5 us and 125.8; sort_dense called as well 128.9.)
+__device__ __noinline__ void sort_crowded(BigSort& sm, uint32_t count, int b0, int b1, uint32_t down, uint32_t cells, int32_t* out) {
+    const int tid = threadIdx.x;
+    uint32_t* const a = sm.a + kSortPad;
+    bool single;
+    auto cell_of = [&](uint32_t t) { return tick_cell(sm.bin, b0, b1, down, cells, t, single); };
+    auto end_of = [&](uint32_t c) { const uint32_t w = sm.cell[c >> 1]; return c & 1u ? w >> 16 : w & 0xFFFFu; };
+    for (uint32_t i = tid; i < kBigCap / 32; i += kSortThreads) sm.mixed[i] = 0;
+    __syncthreads();
+    for (uint32_t i = tid; i + 1u < count; i += kSortThreads) {
+        const uint32_t v = a[i];
+        if (a[i + 1u] == v) continue;
+        const uint32_t c = cell_of(v);
+        if (i + 1u < end_of(c)) atomicOr(&sm.mixed[c >> 5], 1u << (c & 31u));
+    }
+    __syncthreads();
+    uint32_t full = 0;
+    for (uint32_t i = tid; i < count; i += kSortThreads) {
+        const uint32_t v = a[i], c = cell_of(v);
+        if (!(sm.mixed[c >> 5] >> (c & 31u) & 1u)) { out[i] = (int32_t)v; continue; }
+        const uint32_t from = c ? end_of(c - 1u) : 0u, to = end_of(c);
+        if (to - from > 4u * kCellCap) { full = 1u; continue; }
+        const uint32_t p = place_in_cell(a, i, v, from, to);
+        if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) out[p] = (int32_t)v;
+    }
+    if (!__syncthreads_or((int)full)) return;
+    // Hundreds of ticks of a few neighbouring values in a cell: the whole bucket by a bitonic network, padded with the largest word
+    // (a power of two is at most kBigCap).
+    uint32_t whole = 2;
+    while (whole < count) whole <<= 1;
+    for (uint32_t i = count + tid; i < whole; i += kSortThreads) a[i] = 0xFFFFFFFFu;
+    for (uint32_t size = 2; size <= whole; size <<= 1)
+        for (uint32_t gap = size >> 1; gap > 0; gap >>= 1) {
+            __syncthreads();
+            for (uint32_t k = tid; k < whole / 2; k += kSortThreads) {
+                const uint32_t i = (k & ~(gap - 1u)) << 1 | (k & (gap - 1u)), x = a[i], y = a[i + gap];
+                if ((x > y) == ((i & size) == 0u)) { a[i] = y; a[i + gap] = x; }
+            }
+        }
+    __syncthreads();
+    for (uint32_t i = tid; i < count; i += kSortThreads) out[i] = (int32_t)a[i];
+}
+
 __device__ __forceinline__ void sort_bucket(BigSort& sm, const uint32_t* src, uint32_t count, const uint32_t* bin_start,
                                             const uint32_t* bin_count, int b0, int b1, int32_t* out) {
     const int tid = threadIdx.x;
@@ -468,43 +515,7 @@ __device__ __forceinline__ void sort_bucket(BigSort& sm, const uint32_t* src, ui
         order_by_neighbours<kSortThreads>(a, count, (int)most - 1, out);
         return;
     }
-    // Cells reach further: mostly a clock coarser than a microsecond, whose ticks share a cell with their like alone and need no
-    // order among themselves.  (A load of 4 M requests by a millisecond's clock: 189 us, by a microsecond's 184; with a trace that
-    // has one such cell of 256 left to the radix sort 454, of 16 M 1,213 and now 565.)
-    for (uint32_t i = tid; i < kBigCap / 32; i += kSortThreads) sm.mixed[i] = 0;
-    __syncthreads();
-    for (uint32_t i = tid; i + 1u < count; i += kSortThreads) {
-        const uint32_t v = a[i];
-        if (a[i + 1u] == v) continue;
-        const uint32_t c = cell_of(v);
-        if (i + 1u < half_of(c, sm.cell[c >> 1])) atomicOr(&sm.mixed[c >> 5], 1u << (c & 31u));
-    }
-    __syncthreads();
-    uint32_t full = 0;
-    for (uint32_t i = tid; i < count; i += kSortThreads) {
-        const uint32_t v = a[i], c = cell_of(v);
-        if (!(sm.mixed[c >> 5] >> (c & 31u) & 1u)) { out[i] = (int32_t)v; continue; }
-        const uint32_t from = c ? half_of(c - 1u, sm.cell[(c - 1u) >> 1]) : 0u, to = half_of(c, sm.cell[c >> 1]);
-        if (to - from > 4u * kCellCap) { full = 1u; continue; }
-        const uint32_t p = place_in_cell(a, i, v, from, to);
-        if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) out[p] = (int32_t)v;
-    }
-    if (!__syncthreads_or((int)full)) return;
-    // Hundreds of ticks of a few neighbouring values in a cell: the whole bucket by a bitonic network, padded with the largest word
-    // (a power of two is at most kBigCap).
-    uint32_t whole = 2;
-    while (whole < count) whole <<= 1;
-    for (uint32_t i = count + tid; i < whole; i += kSortThreads) a[i] = 0xFFFFFFFFu;
-    for (uint32_t size = 2; size <= whole; size <<= 1)
-        for (uint32_t gap = size >> 1; gap > 0; gap >>= 1) {
-            __syncthreads();
-            for (uint32_t k = tid; k < whole / 2; k += kSortThreads) {
-                const uint32_t i = (k & ~(gap - 1u)) << 1 | (k & (gap - 1u)), x = a[i], y = a[i + gap];
-                if ((x > y) == ((i & size) == 0u)) { a[i] = y; a[i + gap] = x; }
-            }
-        }
-    __syncthreads();
-    for (uint32_t i = tid; i < count; i += kSortThreads) out[i] = (int32_t)a[i];
+    sort_crowded(sm, count, b0, b1, down, cells, out);
 }
 
 __global__ void __launch_bounds__(kSortThreads, 2)
