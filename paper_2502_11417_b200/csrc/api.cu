@@ -270,7 +270,7 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     }
     const size_t o_parted = lay.take(large ? N * 16 : 0), o_rec_of = lay.take(large ? (size_t)G * (kMaxPrompt + 1) * 2 : 0);
     const size_t o_tick_of = lay.take(large ? (size_t)G * kTickBins * 2 : 0), o_at = lay.take(large ? ((size_t)lg.n_rec + lg.n_tick + 4) * 4 : 0);
-    const size_t o_members = lay.take(large ? ((size_t)lg.n_rec + lg.n_tick) * 8 : 0);
+    const size_t o_members = lay.take(large ? (size_t)lg.n_rec * 8 + (size_t)lg.n_tick * 16 : 0);
     disco_ctx::Halves& hv = c->halves;
     // (a large load works without its buckets, by k_load, where there is no room for them: 16 bytes a request)
     c->large_now = large && lay.bytes < c->trace_too_much;
@@ -291,7 +291,7 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
     lg.parted = (uint4*)(base + o_parted);
     lg.rec_bucket = (uint16_t*)(base + o_rec_of); lg.tick_bucket = (uint16_t*)(base + o_tick_of);
     lg.rec_at = (uint32_t*)(base + o_at); lg.tick_at = lg.rec_at + lg.n_rec;
-    lg.rec_members = (uint2*)(base + o_members); lg.tick_members = lg.rec_members + lg.n_rec;
+    lg.rec_members = (uint2*)(base + o_members); lg.tick_jobs = (uint4*)(lg.rec_members + lg.n_rec);     // (an even number)
     c->req.p = base + o_req; c->sorted.p = base + o_sorted; c->binned.p = base + o_binned; c->inv.p = base + o_inv;
     c->zero.p = base + o_zero[hv.now]; c->len_end.p = base + o_ends; c->tick_start.p = base + o_starts; c->cum_mass.p = base + o_mass;
     c->grp_off.p = base + o_off; c->knots.p = base + o_knots; c->fin_totals.p = base + o_fin;

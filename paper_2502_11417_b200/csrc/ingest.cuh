@@ -170,7 +170,7 @@ __device__ __forceinline__ void to_items(const LoadArgs& a, uint32_t i0, const R
             }
         }
         // ticks = nearest integer (ties to even) of the fp64 product, as a host llrint would give
-        const uint32_t S = (uint32_t)__double2ll_rn(__dmul_rn((double)t, 1e6));
+        const uint32_t S = __double2uint_rn(__dmul_rn((double)t, 1e6));      // (2e9 at most)
         x[u] = Item{SRC == S_TRACE ? sp * a.nd + dp : 0u, S, (uint32_t)l, (uint32_t)o, in};
     }
 }
@@ -204,20 +204,23 @@ __device__ __forceinline__ void group_mass(const uint32_t* cnt, int64_t* cum, un
     __syncthreads();
 }
 
-// The cell of a tick among those of the bins [b0, b1]: every bin has as many cells (`down` = 1), or twice as many, as ticks,
-// evenly over its values; bins: first place | count << 16.  single: the cell holds one value (a bin with at least as many cells
-// as values has a cell for each).
-__device__ __forceinline__ uint32_t tick_cell(const uint32_t* bins, int b0, int b1, uint32_t down, uint32_t cells, uint32_t t, bool& single) {
-    const int b = tick_bin(t);
-    single = false;
+// Where a bin's ticks go: every bin has as many cells (`down` = 1), or twice as many, as ticks, evenly over its values.  A word a
+// bin: its first cell, its cells << 14, and 1 << 31 if each of them holds one value (as many cells as values, or more).
+__device__ __forceinline__ uint32_t bin_cells(uint32_t first, uint32_t count, int b, uint32_t down) {
+    const uint32_t w = b < 128 ? 0u : (uint32_t)(b >> 7) - 1u, cells = count << 1 >> down;              // (a bin spans 2^w values)
+    return (first << 1 >> down & 0x3FFFu) | cells << 14 | (1u << w <= cells ? 1u << 31 : 0u);
+}
+// The cell of a tick of the bins from b0 on, by the 16 bits of its float that follow the bin's; `bin`: its bin's word.
+__device__ __forceinline__ uint32_t tick_cell(const uint32_t* bins, int b0, int b1, uint32_t cells, uint32_t t, uint32_t& bin) {
+    const uint32_t f = __float_as_uint(__uint2float_rz(t));
+    const int b = t < 128u ? (int)t : (int)(f >> 16) - ((127 + 7) << 7) + 128;
+    bin = 0;
     if (!DBG_OK(b - b0, b1 - b0 + 1, DBG_K_RADIX, DBG_BIN)) return 0u;
-    const uint32_t sc = bins[b - b0], w = b < 128 ? 0u : (uint32_t)(b >> 7) - 1u, in = t - tick_bin_edge(b);
-    const uint32_t sh = min(w, 16u);                                   // (a bin spans 2^w values; 16 leading bits of the place in it)
-    const uint32_t of_bin = sc >> 16 << 1;
-    const uint32_t c = (((sc & 0xFFFFu) << 1) + ((in >> (w - sh)) * of_bin >> sh)) >> down;
-    single = 1u << w <= of_bin >> down;
+    bin = bins[b - b0];
+    const uint32_t c = mad_hi(f << 16, bin >> 14 & 0x7FFFu, bin & 0x3FFFu);
     return DBG_OK(c, cells, DBG_K_RADIX, DBG_BIN) ? c : 0u;
 }
+__device__ __forceinline__ bool one_value(uint32_t bin) { return (int32_t)bin < 0; }
 
 // Ticks placed cell by cell into their order, found by comparing with neighbours as far as cells of different ticks reach
 // (`reach` <= kSortPad; a tick moves up by those behind it that are smaller, and down by those in front that are larger).  A
@@ -248,43 +251,43 @@ __device__ __forceinline__ uint32_t place_in_cell(const uint32_t* a, uint32_t i,
 // placed, and compared with their neighbours as far as cells reach.  Returns false if more than kCellCap different ticks may
 // share a cell (what it has written is to be written again).
 // Bound: instruction issue.  (Of the 14 us of a window of 8,192 ticks cells put in order by insertion, a thread a cell, took 5.6,
-// each tick compared with its cell's as long; with its neighbours 1.5.)
+// each tick compared with its cell's as long; with its neighbours 1.5.  A thread keeps its ticks, their cells and their ranks there: counted once
+// more to be placed, and cells worked out from the ticks' places in their bins, k_load_once took 48 us for a million requests of one group,
+// now 44, 35 and 33 for 100,000 of six.)
 constexpr uint32_t kCellCap = 64;
 
 __device__ __forceinline__ bool sort_window(SortSmem& sm, const uint32_t* src, uint32_t count, const uint32_t* bin_start,
                                             const uint32_t* bin_count, int b0, int b1, int32_t* out) {
     const int tid = threadIdx.x;
-    constexpr int kKeep = kWindow / kThreads, kVecs = kSortCap / kThreads / 4;      // ticks a thread keeps (others are read again), vectors of cells it has
-    uint32_t* cell = sm.b;                                             // counts, then starts, then ends
+    constexpr int kKeep = kSortCap / kThreads, kVecs = kSortCap / kThreads / 4;     // ticks a thread keeps, vectors of cells it has
+    uint32_t* cell = sm.b;                                             // counts, then starts
     uint32_t* const a = sm.a + kSortPad;
     // twice as many cells as ticks, or as many
     const uint32_t k0 = __ldcg(&bin_start[b0]), down = count <= kSortCap / 2 ? 0u : 1u, cells = 2u * count >> down;
     for (uint32_t i = tid; i < (cells + kVecs * 4u - 1u) / (kVecs * 4u) * (kVecs * 4u); i += kThreads) cell[i] = 0;
     for (int b = b0 + tid; b <= b1; b += kThreads) {
         const uint32_t c = __ldcg(&bin_count[b]);
-        sm.bin[b - b0] = (__ldcg(&bin_start[b]) - k0) | c << 16;       // (an empty bin's is not used)
+        sm.bin[b - b0] = bin_cells(__ldcg(&bin_start[b]) - k0, c, b, down);           // (an empty bin's is not used)
     }
     if (tid < (int)kSortPad) { sm.a[tid] = 0u; a[count + tid] = 0xFFFFFFFFu; }
     if (tid == 0) sm.most = 0;
-    uint32_t key[kKeep], at[kKeep];                                    // at: the cells
+    uint32_t key[kKeep], at[kKeep];                                    // at: cell | rank among the cell's ticks << 14
 #pragma unroll
     for (int k = 0; k < kKeep; ++k) {
         const uint32_t i = k * kThreads + tid;
         if (i < count) key[k] = __ldcg(&src[i]);
     }
     __syncthreads();
-    bool single;
-    auto cell_of = [&](uint32_t t) { return tick_cell(sm.bin, b0, b1, down, cells, t, single); };
+    auto cell_of = [&](uint32_t t, uint32_t& bin) { return tick_cell(sm.bin, b0, b1, cells, t, bin); };
     uint32_t most = 1;                                                 // ticks of a cell that may hold different ones
-    auto count_in = [&](uint32_t t) {
-        const uint32_t c = cell_of(t), rank = atomicAdd(&cell[c], 1u);
-        if (!single) most = max(most, rank + 1u);
-        return c;
-    };
 #pragma unroll
-    for (int k = 0; k < kKeep; ++k) if ((uint32_t)k * kThreads + tid < count) at[k] = count_in(key[k]);
-#pragma unroll 2
-    for (uint32_t i = kWindow + tid; i < count; i += kThreads) count_in(__ldcg(&src[i]));
+    for (int k = 0; k < kKeep; ++k) {
+        if ((uint32_t)k * kThreads + tid >= count) break;
+        uint32_t bin;
+        const uint32_t c = cell_of(key[k], bin), rank = atomicAdd(&cell[c], 1u);
+        if (!one_value(bin)) most = max(most, rank + 1u);
+        at[k] = c | rank << 14;
+    }
     most = __reduce_max_sync(FULL, most);
     if ((tid & 31) == 0) atomicMax(&sm.most, most);
     __syncthreads();
@@ -313,28 +316,25 @@ __device__ __forceinline__ bool sort_window(SortSmem& sm, const uint32_t* src, u
         }
     }
     __syncthreads();
-    auto put = [&](uint32_t t, uint32_t c) {
-        const uint32_t p = atomicAdd(&cell[c], 1u);
-        if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) a[p] = t;
-    };
 #pragma unroll
-    for (int k = 0; k < kKeep; ++k) if ((uint32_t)k * kThreads + tid < count) put(key[k], at[k]);
-#pragma unroll 2
-    for (uint32_t i = kWindow + tid; i < count; i += kThreads) { const uint32_t t = __ldcg(&src[i]); put(t, cell_of(t)); }
+    for (int k = 0; k < kKeep; ++k) {
+        if ((uint32_t)k * kThreads + tid >= count) break;
+        const uint32_t p = cell[at[k] & 0x3FFFu] + (at[k] >> 14);
+        if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) a[p] = key[k];
+    }
     __syncthreads();
     if (most <= kSortPad) {
         order_by_neighbours<kThreads>(a, count, (int)most - 1, out);
         return true;
     }
-    uint32_t full = 0;
+    if (most > kCellCap) return false;
     for (uint32_t i = tid; i < count; i += kThreads) {
-        const uint32_t v = a[i], c = cell_of(v), from = c ? cell[c - 1u] : 0u, to = cell[c];
-        if (single) { out[i] = (int32_t)v; continue; }
-        if (to - from > kCellCap) { full = 1u; continue; }
-        const uint32_t p = place_in_cell(a, i, v, from, to);
+        uint32_t bin;
+        const uint32_t v = a[i], c = cell_of(v, bin), from = cell[c], to = c + 1u < cells ? cell[c + 1u] : count;
+        const uint32_t p = one_value(bin) ? i : place_in_cell(a, i, v, from, to);
         if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) out[p] = (int32_t)v;
     }
-    return !__syncthreads_or((int)full);
+    return true;
 }
 
 // The same whatever the ticks (all of them in [lo, lo + 2^bits)): stable counting passes of at most eight bits, a warp's share

@@ -60,7 +60,8 @@ struct LargeLoad {
     uint32_t rec_share, tick_share, n_rec, n_tick;    // requests or ticks to a bucket, numbers of buckets
     uint16_t *rec_bucket, *tick_bucket;   // [G][4097], [G][kTickBins]
     uint32_t *rec_at, *tick_at;           // cursors, [n_rec] and [n_tick]
-    uint2 *rec_members, *tick_members;    // first and last length or bin, counted through the groups (first > last: none)
+    uint2* rec_members;                   // first and last length, counted through the groups (first > last: none)
+    uint4* tick_jobs;                     // where the bucket's ticks start and end, first and last bin, counted through the groups (0, 0: none)
 };
 
 // Small and middling traces: a kernel whose threads read their requests once and keep them (load_once.cu).

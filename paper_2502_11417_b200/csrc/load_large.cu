@@ -14,8 +14,8 @@
 //   k_sort     the ticks of a bucket ascending.
 // Nothing waits for another block.
 //
-// Bound: memory and shared-memory atomics.  16 M requests in six groups: k_load 855 us, these 560 (count 57, plan 14, records 150,
-// ticks 111, order 105, sort 122); 4 M in one group 213 and 161, in six 209 and 189.  At 3 M k_load wins (127 and 136 in one group,
+// Bound: memory and shared-memory atomics.  16 M requests in six groups: k_load 855 us, these 550 (count 58, plan 13, records 149,
+// ticks 109, order 105, sort 114); 4 M in one group 213 and 157, in six 209 and 183.  At 3 M k_load wins (127 and 136 in one group,
 // 137 and 155 in six): its scattered stores still meet their lines in L2, and it has one launch.  Above 2^24 requests the tables
 // of buckets do not fit in a block's shared memory, above seven groups the counters.
 #include <algorithm>
@@ -150,18 +150,20 @@ k_plan(const __grid_constant__ LoadArgs a) {
     }
     if (!ticks && tid == 0) a.len_end[(size_t)g * kLens] = off;
     __syncthreads();
-    for (uint32_t i = tid; i < ids; i += kThreads) {
-        (ticks ? a.large.tick_members : a.large.rec_members)[id0 + i] =
-            s_first[i] <= s_last[i] ? make_uint2((uint32_t)(g * width) + s_first[i], (uint32_t)(g * width) + s_last[i]) : make_uint2(1u, 0u);
+    // where the buckets start, at their first member (written above by a thread of this block), and what they hold
+    const uint32_t last_id = g == G - 1 ? (ticks ? a.large.n_tick : a.large.n_rec) - id0 : ids;        // (the last are buckets that no group has)
+    for (uint32_t i = tid; i < last_id; i += kThreads) {
+        const bool some = i < ids && s_first[i] <= s_last[i];
+        const uint32_t m0 = (uint32_t)(g * width) + s_first[i], m1 = (uint32_t)(g * width) + s_last[i];
+        if (ticks) {
+            const uint32_t start = some ? a.tick_start[m0] : 0u;
+            if (some) a.large.tick_at[id0 + i] = start;
+            a.large.tick_jobs[id0 + i] = some ? make_uint4(start, a.tick_start[m1] + __ldcg(&a.tick_cnt[m1]), m0, m1) : make_uint4(0u, 0u, 0u, 0u);
+        } else {
+            if (some) a.large.rec_at[id0 + i] = a.len_end[m0 - 1];
+            a.large.rec_members[id0 + i] = some ? make_uint2(m0, m1) : make_uint2(1u, 0u);
+        }
     }
-    // where the buckets start: at their first member (written above by a thread of this block)
-    for (uint32_t i = tid; i < ids; i += kThreads)
-        if (s_first[i] <= s_last[i])
-            (ticks ? a.large.tick_at : a.large.rec_at)[id0 + i] = ticks ? a.tick_start[(size_t)g * kTickBins + s_first[i]]
-                                                                        : a.len_end[(size_t)g * kLens + s_first[i] - 1];
-    if (g == G - 1)                                                    // buckets that no group has
-        for (uint32_t i = id0 + ids + tid; i < (ticks ? a.large.n_tick : a.large.n_rec); i += kThreads)
-            (ticks ? a.large.tick_members : a.large.rec_members)[i] = make_uint2(1u, 0u);
     if (ticks) return;
     // cumulative input-token mass cum[L] = sum_{l<L} l cnt[l], L = 0 .. 4097
     unsigned long long mass = 0, total;
@@ -186,16 +188,22 @@ k_plan(const __grid_constant__ LoadArgs a) {
 }
 
 // Tiles to buckets.  (Straight from the registers, a store of 16 bytes a lane, the records took 366 us instead of 150 at 16 M;
-// tiles of 4,096 ticks, two blocks to a multiprocessor, 141 instead of 111: half the ticks to a run.)  A tile's requests are counted by bucket in shared memory, its shares of the buckets taken from global
+// tiles of 4,096 ticks, two blocks to a multiprocessor, 141 instead of 111: half the ticks to a run; of 16,384, 110.)  A tile's requests are counted by bucket in shared memory, its shares of the buckets taken from global
 // cursors, and what goes to one bucket is brought side by side in shared memory before it leaves.  The next tile is read while
 // one leaves.
 template <int FORM>
-__device__ __forceinline__ void read_tile(const LoadArgs& a, uint32_t t0, bool wide, Raw (&r)[kPer / 4]) {
+__device__ __forceinline__ void read_tile(const LoadArgs& a, uint32_t t0, uint32_t end, bool wide, Raw (&r)[kPer / 4]) {
 #pragma unroll
     for (int q = 0; q < kPer / 4; ++q) {
         const uint32_t i0 = t0 + (uint32_t)(q * kThreads + (int)threadIdx.x) * 4u;
-        if (i0 < a.n) read_raw<S_TRACE, FORM, false>(a, i0, wide, r[q]);
+        if (i0 < end) read_raw<S_TRACE, FORM, false>(a, i0, wide, r[q]);
     }
+}
+// Ticks of a tile, whole vectors: as many to each block (4 M in one group 29.4 us -> 26.5, in six 31.3 -> 28.3, 16 M 112 -> 109; the same for
+// records, whose kernel then spills more: 16 M 149 -> 156).
+__device__ __forceinline__ uint32_t even_tile(uint32_t n) {
+    const uint32_t tiles = gridDim.x * ((n - 1u) / (gridDim.x * kTile) + 1u);
+    return ((n - 1u) / tiles + 4u) / 4u * 4u;
 }
 
 // Exclusive prefix sums over `count` counters, vectors of four (those behind the last are zero), and the tile's shares from the
@@ -240,7 +248,7 @@ k_records(const __grid_constant__ LoadArgs a) {
     const bool wide = columns_aligned(a);
     uint32_t t0 = blockIdx.x * kTile;
     Raw raw[kPer / 4];
-    if (t0 < a.n) read_tile<FORM>(a, t0, wide, raw);
+    if (t0 < a.n) read_tile<FORM>(a, t0, a.n, wide, raw);
 #pragma unroll 1
     for (; t0 < a.n; t0 += gridDim.x * kTile) {
         for (uint32_t i = tid; i < n_rec; i += kThreads) s_start[i] = 0;
@@ -270,7 +278,7 @@ k_records(const __grid_constant__ LoadArgs a) {
             const uint32_t slot = s_start[rec[k] & 0xFFFFu] + (rec[k] >> 16), i = t0 + (uint32_t)(k / 4 * kThreads + tid) * 4u + k % 4;
             if (DBG_OK(slot, kTile, DBG_K_GATHER, DBG_SLOT)) s_req[slot] = make_uint4(S[k], ln[k], i, rec[k] & 0xFFFFu);
         }
-        if (t0 + gridDim.x * kTile < a.n) read_tile<FORM>(a, t0 + gridDim.x * kTile, wide, raw);
+        if (t0 + gridDim.x * kTile < a.n) read_tile<FORM>(a, t0 + gridDim.x * kTile, a.n, wide, raw);
         __syncthreads();
         const uint32_t here = min(kTile, a.n - t0);
 #pragma unroll 2
@@ -301,29 +309,31 @@ k_ticks(const __grid_constant__ LoadArgs a) {
     if (refused(a)) return;
     for (int i = tid; i < G * kTickBins; i += kThreads) s_of[i] = a.large.tick_bucket[i];
     const bool wide = columns_aligned(a);
-    uint32_t t0 = blockIdx.x * kTile;
+    const uint32_t tile = even_tile(a.n), stride = gridDim.x * tile;
+    uint32_t t0 = blockIdx.x * tile, end = min(a.n, t0 + tile);
     Raw raw[kPer / 4];
-    if (t0 < a.n) read_tile<FORM>(a, t0, wide, raw);
+    if (t0 < a.n) read_tile<FORM>(a, t0, end, wide, raw);
 #pragma unroll 1
-    for (; t0 < a.n; t0 += gridDim.x * kTile) {
+    for (; t0 < a.n; t0 += stride, end = min(a.n, t0 + tile)) {
         for (uint32_t i = tid; i < n_tick; i += kThreads) s_start[i] = 0;
         __syncthreads();
         uint32_t S[kPer], tick[kPer];
 #pragma unroll
         for (int q = 0; q < kPer / 4; ++q) {
             Item x[4];
-            to_items<S_TRACE, FORM, false>(a, t0 + (uint32_t)(q * kThreads + tid) * 4u, raw[q], nullptr, x);
+            const uint32_t i0 = t0 + (uint32_t)(q * kThreads + tid) * 4u;
+            to_items<S_TRACE, FORM, false>(a, i0, raw[q], nullptr, x);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int k = q * 4 + u;
                 tick[k] = 0xFFFFFFFFu;
-                if (!x[u].in || !DBG_OK(x[u].g, G, DBG_K_GATHER, DBG_GROUP)) continue;
+                if (i0 + u >= end || !DBG_OK(x[u].g, G, DBG_K_GATHER, DBG_GROUP)) continue;
                 S[k] = x[u].S;
                 const uint32_t t = s_of[x[u].g * kTickBins + tick_bin(x[u].S)];
                 if (DBG_OK(t, n_tick, DBG_K_GATHER, DBG_TABLE)) tick[k] = t | atomicAdd(&s_start[t], 1u) << 16;
             }
         }
-        if (t0 + gridDim.x * kTile < a.n) read_tile<FORM>(a, t0 + gridDim.x * kTile, wide, raw);
+        if (t0 + stride < a.n) read_tile<FORM>(a, t0 + stride, min(a.n, t0 + stride + tile), wide, raw);
         __syncthreads();
         take_shares(s_start, s_to, n_tick, a.large.tick_at, s_wtot);
         __syncthreads();
@@ -334,7 +344,7 @@ k_ticks(const __grid_constant__ LoadArgs a) {
             if (DBG_OK(slot, kTile, DBG_K_GATHER, DBG_SLOT)) { s_tick[slot] = S[k]; s_in[slot] = (uint16_t)tick[k]; }
         }
         __syncthreads();
-        const uint32_t here = min(kTile, a.n - t0);
+        const uint32_t here = end - t0;
 #pragma unroll 4
         for (uint32_t slot = tid; slot < here; slot += kThreads) {
             const uint32_t to = s_to[s_in[slot]] + slot;
@@ -377,29 +387,34 @@ k_order(const __grid_constant__ LoadArgs a) {
 }
 
 // A block per pair of buckets (the ones of odd numbers are mostly empty), two of 512 threads to a multiprocessor: one sorts while
-// the other waits (16 M ticks 122 us; one of 1,024 threads 167).  As sort_window in ingest.cuh, but that the cells are counted in halves of words, and that the ticks are read
-// again to be placed (a thread has too many to keep).
+// the other waits (16 M ticks 114 us; one of 1,024 threads 167 where two of 512 took 122).  As sort_window in ingest.cuh, but that the cells are counted in halves
+// of words, and that the ticks are read and counted again to be placed: a thread has too many to keep them, or their ranks (121 us with cell
+// and rank in a word, 121 with the rank in half a one).  Blocks that stay and draw their pairs were held up behind dense ones: 16 M ticks of
+// one group 138 us -> 217.
 constexpr int kSortThreads = 512;
 struct BigSort {
     uint32_t a[kBigCap + 2 * kSortPad];                // the ticks; or counters
     uint32_t cell[kBigCap / 2];                        // counts, then starts, then ends, two to a word
-    uint32_t bin[kTickBins];                           // first place | count << 16
+    uint32_t bin[kTickBins];                           // bin_cells()
     uint32_t mixed[kBigCap / 32];                      // a bit a cell: it holds different ticks
     uint32_t wtot[32], range[2], most;
 };
 static_assert(2 * (sizeof(BigSort) + 1024 + 16) <= 227 * 1024, "two blocks to a multiprocessor");
+
+__device__ __forceinline__ uint32_t half_of(uint32_t c, uint32_t w) { return c & 1u ? w >> 16 : w & 0xFFFFu; }
 
 // A bucket whose ticks lie in their cells (sm.cell: where each ends), where cells of different ticks reach further than kSortPad: mostly
 // a clock coarser than a microsecond, whose ticks share a cell with their like alone and need no order among themselves.  (A load of
 // 4 M requests by a millisecond's clock: 189 us, by a microsecond's 184; with a trace that has one such cell of 256 left to the
 // radix sort 454, of 16 M 1,213 and now 565.  Called, not inlined: k_sort of 16 M microsecond ticks in six groups, which do not come
 // here, 124.5 us and 125.8; sort_dense called as well 128.9.)
-__device__ __noinline__ void sort_crowded(BigSort& sm, uint32_t count, int b0, int b1, uint32_t down, uint32_t cells, int32_t* out) {
+__device__ __noinline__ void sort_crowded(BigSort& sm, uint32_t count, int b0, int b1, uint32_t cells, int32_t* out) {
     const int tid = threadIdx.x;
     uint32_t* const a = sm.a + kSortPad;
-    bool single;
-    auto cell_of = [&](uint32_t t) { return tick_cell(sm.bin, b0, b1, down, cells, t, single); };
-    auto end_of = [&](uint32_t c) { const uint32_t w = sm.cell[c >> 1]; return c & 1u ? w >> 16 : w & 0xFFFFu; };
+    uint32_t bin;
+    auto cell_of = [&](uint32_t t) { return tick_cell(sm.bin, b0, b1, cells, t, bin); };
+    auto end_of = [&](uint32_t c) { return half_of(c, sm.cell[c >> 1]); };
+    auto start_of = [&](uint32_t c) { return c ? end_of(c - 1u) : 0u; };
     for (uint32_t i = tid; i < kBigCap / 32; i += kSortThreads) sm.mixed[i] = 0;
     __syncthreads();
     for (uint32_t i = tid; i + 1u < count; i += kSortThreads) {
@@ -413,7 +428,7 @@ __device__ __noinline__ void sort_crowded(BigSort& sm, uint32_t count, int b0, i
     for (uint32_t i = tid; i < count; i += kSortThreads) {
         const uint32_t v = a[i], c = cell_of(v);
         if (!(sm.mixed[c >> 5] >> (c & 31u) & 1u)) { out[i] = (int32_t)v; continue; }
-        const uint32_t from = c ? end_of(c - 1u) : 0u, to = end_of(c);
+        const uint32_t from = start_of(c), to = end_of(c);
         if (to - from > 4u * kCellCap) { full = 1u; continue; }
         const uint32_t p = place_in_cell(a, i, v, from, to);
         if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) out[p] = (int32_t)v;
@@ -437,22 +452,17 @@ __device__ __noinline__ void sort_crowded(BigSort& sm, uint32_t count, int b0, i
 }
 
 __device__ __forceinline__ void sort_bucket(BigSort& sm, const uint32_t* src, uint32_t count, const uint32_t* bin_start,
-                                            const uint32_t* bin_count, int b0, int b1, int32_t* out) {
+                                            const uint32_t* bin_count, int b0, int b1, uint32_t k0, int32_t* out) {
     const int tid = threadIdx.x;
     constexpr int kVecs = kBigCap / 2 / kSortThreads / 4;              // vectors of cells a thread has
     uint32_t* const a = sm.a + kSortPad;
-    const uint32_t k0 = __ldcg(&bin_start[b0]), down = count <= kBigCap / 2 ? 0u : 1u, cells = 2u * count >> down, words = (cells + 1u) / 2u;
+    const uint32_t down = count <= kBigCap / 2 ? 0u : 1u, cells = 2u * count >> down, words = (cells + 1u) / 2u;
     for (uint32_t i = tid; i < (words + kVecs * 4u - 1u) / (kVecs * 4u) * (kVecs * 4u); i += kSortThreads) sm.cell[i] = 0;
-    for (int b = b0 + tid; b <= b1; b += kSortThreads) {
-        const uint32_t c = __ldcg(&bin_count[b]);
-        sm.bin[b - b0] = (__ldcg(&bin_start[b]) - k0) | c << 16;       // (an empty bin's is not used)
-    }
+    for (int b = b0 + tid; b <= b1; b += kSortThreads)
+        sm.bin[b - b0] = bin_cells(__ldcg(&bin_start[b]) - k0, __ldcg(&bin_count[b]), b, down);         // (an empty bin's is not used)
     if (tid < (int)kSortPad) { sm.a[tid] = 0u; a[count + tid] = 0xFFFFFFFFu; }
     if (tid == 0) sm.most = 0;
     __syncthreads();
-    bool single;
-    auto cell_of = [&](uint32_t t) { return tick_cell(sm.bin, b0, b1, down, cells, t, single); };
-    auto half_of = [&](uint32_t c, uint32_t w) { return c & 1u ? w >> 16 : w & 0xFFFFu; };
     constexpr int kAhead = 8;
     uint32_t most = 1;                                                 // ticks of a cell that may hold different ones
 #pragma unroll 1
@@ -463,8 +473,9 @@ __device__ __forceinline__ void sort_bucket(BigSort& sm, const uint32_t* src, ui
 #pragma unroll
         for (int k = 0; k < kAhead; ++k) {
             if (i0 + k * kSortThreads >= count) continue;
-            const uint32_t c = cell_of(key[k]), rank = half_of(c, atomicAdd(&sm.cell[c >> 1], c & 1u ? 65536u : 1u));
-            if (!single) most = max(most, rank + 1u);
+            uint32_t bin;
+            const uint32_t c = tick_cell(sm.bin, b0, b1, cells, key[k], bin), rank = half_of(c, atomicAdd(&sm.cell[c >> 1], c & 1u ? 65536u : 1u));
+            if (!one_value(bin)) most = max(most, rank + 1u);
         }
     }
     most = __reduce_max_sync(FULL, most);
@@ -506,7 +517,8 @@ __device__ __forceinline__ void sort_bucket(BigSort& sm, const uint32_t* src, ui
 #pragma unroll
         for (int k = 0; k < kAhead; ++k) {
             if (i0 + k * kSortThreads >= count) continue;
-            const uint32_t c = cell_of(key[k]), p = half_of(c, atomicAdd(&sm.cell[c >> 1], c & 1u ? 65536u : 1u));
+            uint32_t bin;
+            const uint32_t c = tick_cell(sm.bin, b0, b1, cells, key[k], bin), p = half_of(c, atomicAdd(&sm.cell[c >> 1], c & 1u ? 65536u : 1u));
             if (DBG_OK(p, count, DBG_K_RADIX, DBG_ELEMENT)) a[p] = key[k];
         }
     }
@@ -515,7 +527,7 @@ __device__ __forceinline__ void sort_bucket(BigSort& sm, const uint32_t* src, ui
         order_by_neighbours<kSortThreads>(a, count, (int)most - 1, out);
         return;
     }
-    sort_crowded(sm, count, b0, b1, down, cells, out);
+    sort_crowded(sm, count, b0, b1, cells, out);
 }
 
 __global__ void __launch_bounds__(kSortThreads, 2)
@@ -527,13 +539,13 @@ k_sort(const __grid_constant__ LoadArgs a) {
     if (refused(a)) return;
 #pragma unroll 1
     for (uint32_t bucket = blockIdx.x * 2u; bucket <= blockIdx.x * 2u + 1u; ++bucket) {
-        const uint2 members = __ldcg(&a.large.tick_members[bucket]);
-        if (members.x > members.y) continue;
-        const int g = (int)members.x / kTickBins, b0 = (int)members.x - g * kTickBins, b1 = (int)members.y - g * kTickBins;
-        const uint32_t k0 = __ldcg(&a.tick_start[members.x]), k1 = __ldcg(&a.tick_start[members.y]) + __ldcg(&a.tick_cnt[members.y]);
-        const uint32_t first = __ldcg(&a.grp_off[g]), N = __ldcg(&a.grp_off[g + 1]) - first, edge = tick_bin_edge(b0);
+        const uint4 j = __ldcg(&a.large.tick_jobs[bucket]);            // ticks [x, y) of the bins z .. w, counted through the groups
+        if (j.x >= j.y) continue;
+        const int g = (int)j.z / kTickBins, b0 = (int)j.z - g * kTickBins, b1 = (int)j.w - g * kTickBins;
+        const uint32_t k0 = j.x, k1 = j.y, edge = tick_bin_edge(b0);
+        const uint32_t first = __ldcg(&a.grp_off[g]), N = __ldcg(&a.grp_off[g + 1]) - first;
         if (k1 - k0 <= kBigCap) {
-            sort_bucket(sm, a.binned + k0, k1 - k0, a.tick_start + (size_t)g * kTickBins, a.tick_cnt + (size_t)g * kTickBins, b0, b1, a.sorted + k0);
+            sort_bucket(sm, a.binned + k0, k1 - k0, a.tick_start + (size_t)g * kTickBins, a.tick_cnt + (size_t)g * kTickBins, b0, b1, k0, a.sorted + k0);
         } else if (!sort_dense<kSortThreads, kBigCap>(sm.a, sm.wtot, sm.range, a.binned + k0, k1 - k0, edge, tick_bin_edge(b1 + 1) - edge, a.sorted + k0) &&
                    threadIdx.x == 0) {
             atomicMax(&a.z->err[3], 1);                                // (the radix sort, then)

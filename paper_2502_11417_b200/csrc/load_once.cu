@@ -13,7 +13,7 @@
 //
 // Bound: latency, some fifteen dependent steps, and from half a million requests on the scattered stores.  Against k_load, which
 // reads the requests twice and waits three times (with the memset in front of it, kernels and gaps): 100,000 requests in one group
-// 42 us -> 21, in six 56 -> 34; a million 64 -> 45 and 76 -> 57; 1,000 in one block 23 -> 17; 100,000 ticks 25 -> 15.  Where the
+// 42 us -> 19, in six 56 -> 33; a million 64 -> 44 and 76 -> 55; 1,000 in one block 23 -> 17; 100,000 ticks 25 -> 15.  Where the
 // threads cannot keep their requests (8,192 a block) k_load is left.  (Eight requests a thread spill 168 bytes, four 48.)
 #include <algorithm>
 #include <cstdlib>
