@@ -237,7 +237,10 @@ k_playout_fast(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
 // requests have longer lags (prompts that take a device long to read: those lags are alike).  (Without the collection:
 // 513 us for the 16 M requests of three server profiles and two devices, 43 us for 250,000 of them; with it 304 and 12, and
 // 248 and 10 with the tokens that can neither fill the buffer nor make up the lag drawn without a test each; 4 M requests of long
-// outputs on a slow device 97 us, now 59, most of it because the blocks with the longest lags come first.)
+// outputs on a slow device 97 us, now 60, most of it because the blocks with the longest lags come first.)  Of those 248 us the lags took
+// 100, since a warp draws as long as the longest of its 32: put in order by their lengths first they take 50 (4 M in six groups 66 us ->
+// 54).  That pays where they are lags behind a server's TTFT; a device's, 4 M requests in one group, take 60 us as they come and 64
+// put in order.
 constexpr uint32_t kShortSearch = 64;
 constexpr int kShortThreads = 256;
 constexpr int kShortPer = 4;             // requests a thread may play
@@ -251,7 +254,13 @@ struct ShortGroup {                      // a group under the class
     int exact;                           // played here
     int32_t cT_mean;
     uint32_t sure;                       // tokens that cannot fill the buffer, whatever their jitter
+    // so many tokens are late for sure, each making up cT at most (the quotient is rounded down by more than its error)
+    __device__ uint32_t sure_late(int32_t need) const { return (uint32_t)(__fdividef((float)(need - 1), (float)max(cT, 1)) * 0.99999f); }
 };
+
+// The lags of a block are put in order by what they take at least, in 64 steps: a token each, and from 32 on eight.
+constexpr int kLagLengths = 64;
+__device__ __forceinline__ uint32_t lag_length(uint32_t tokens) { return tokens < 32u ? tokens : min(28u + tokens / 8u, (uint32_t)kLagLengths - 1u); }
 
 // (h * mul) >> 32 of so many tokens behind hin, added up: no test a token, so that several are under way at once.
 __device__ __forceinline__ uint32_t sum_jitter(uint32_t& hin, uint32_t count, uint32_t mul) {
@@ -270,7 +279,8 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
     if (MANY) rec.hand = reinterpret_cast<uint2*>(reinterpret_cast<char*>(rec.hand) + many.slot[blockIdx.y] * many.rec_stride);
     __shared__ ShortGroup groups[kMaxGroups];
     __shared__ uint4 lag[kShortThreads * kShortPer];         // hash key, lag, output length | hand-off << 16, place | group << 16
-    __shared__ uint16_t rest[kShortThreads * kShortPer];     // lags that a thread has not made up
+    __shared__ uint16_t rest[kShortThreads * kShortPer];     // the lags by their lengths, then those that a thread has not made up
+    __shared__ int of_length[kLagLengths];                   // how many, then where they start
     __shared__ int n_lag, n_long, n_rest;
     grid_dependency_wait();
     if (early) let_next_start();
@@ -279,6 +289,7 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
     const long long thr64 = (long long)(B ? B - 1 : 0) * tau;
     const int32_t thr = thr64 > 0x7FFFFFFFLL ? 0x7FFFFFFF : (int32_t)thr64;
     if (threadIdx.x == 0) { n_lag = 0; n_long = 0; n_rest = 0; }
+    if (threadIdx.x < kLagLengths) of_length[threadIdx.x] = 0;
     for (int g = threadIdx.x; g < tr.n_groups; g += kShortThreads) {
         const GroupConst& gc = gcs[g];
         ShortGroup G;
@@ -346,16 +357,53 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
         rec.hand[kk] = make_uint2(m, stall);
     }
     __syncthreads();
-    // ---- tokens m+2.. stay late while the target's sum of c from there on is below the lag (c >= 0: a prefix)
     const uint32_t most = n_long > kShortThreads / 4 ? 256u : 32u;
-    for (int i = threadIdx.x; i < n_lag; i += kShortThreads) {
+    // ---- many lags as widely spread as the server's TTFT: by their lengths, the longest first, so that the lanes of a warp have about
+    //      the same to draw (a device's are alike among neighbours)
+    uint64_t mine = 0;                                         // the thread's lags, 16 bits each; in order of place unless they are sorted
+#pragma unroll
+    for (int k = 0; k < kShortPer; ++k) mine |= (uint64_t)(k * kShortThreads + threadIdx.x) << (16 * k);
+    static_assert(kShortPer <= 4, "16 bits each");
+    if (n_lag > kShortThreads / 2 && groups[lag[0].w >> 16].cand == 2) {
+        uint32_t at[kShortPer];                                    // length | rank << 8
+#pragma unroll
+        for (int k = 0; k < kShortPer; ++k) {
+            const int i = k * kShortThreads + threadIdx.x;
+            if (i >= n_lag) break;
+            const uint4 x = lag[i];
+            const uint32_t length = lag_length(min((x.z & 0xFFFFu) - (x.z >> 16), groups[x.w >> 16].sure_late((int32_t)x.y)));
+            at[k] = length | (uint32_t)atomicAdd(&of_length[length], 1) << 8;
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            static_assert(kLagLengths == 64, "two a lane");
+            const int a = of_length[63 - 2 * threadIdx.x], b = of_length[62 - 2 * threadIdx.x];
+            const int before = team_inclusive_sum(a + b, threadIdx.x) - a - b;
+            of_length[63 - 2 * threadIdx.x] = before; of_length[62 - 2 * threadIdx.x] = before + a;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kShortPer; ++k) {
+            const int i = k * kShortThreads + threadIdx.x;
+            if (i >= n_lag) break;
+            const int to = of_length[at[k] & 255u] + (int)(at[k] >> 8);
+            if (DBG_OK(to, kShortThreads * kShortPer, DBG_K_PLAYOUT_FAST, DBG_SLOT)) rest[to] = (uint16_t)i;
+        }
+        __syncthreads();
+        mine = 0;
+#pragma unroll
+        for (int k = 0; k < kShortPer; ++k) mine |= (uint64_t)rest[k * kShortThreads + threadIdx.x] << (16 * k);     // (those behind the last are not used)
+        __syncthreads();
+    }
+    // ---- tokens m+2.. stay late while the target's sum of c from there on is below the lag (c >= 0: a prefix)
+    for (int j0 = threadIdx.x; j0 < n_lag; j0 += kShortThreads, mine >>= 16) {
+        const int i = (int)(mine & 0xFFFFu);
         const uint4 x = lag[i];
         const ShortGroup& G = groups[x.w >> 16];
         const int32_t need = (int32_t)x.y, cT = G.cT;
         const uint32_t n = x.z & 0xFFFFu, m = x.z >> 16, mulT = G.mulT, end = min(n, m + 1 + most);
         uint32_t j = m + 2, hin = x.x + (m + 1) * kHashTok;
-        // so many tokens are late for sure, each making up cT at most (the quotient is rounded down by more than its error)
-        const uint32_t sure = min(end + 1u - j, (uint32_t)(__fdividef((float)(need - 1), (float)max(cT, 1)) * 0.99999f));
+        const uint32_t sure = min(end + 1u - j, G.sure_late(need));
         int32_t run = (int32_t)(sure * (uint32_t)cT - sum_jitter(hin, sure, mulT));
         j += sure;
         for (hin += kHashTok; j <= end; ++j, hin += kHashTok) {
@@ -363,7 +411,7 @@ k_playout_short(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_co
             if (run >= need) break;
         }
         if (run < need && j <= n) { lag[i].y = (uint32_t)(need - run); rest[atomicAdd(&n_rest, 1)] = (uint16_t)i; continue; }
-        rec.hand[first + (x.w & 0xFFFFu)].x = m | (j - m - 1) << 16;           // tokens m+1 .. j-1 are late
+        rec.hand[first + (x.w & 0xFFFFu)].x = m | (j - m - 1) << 16;             // tokens m+1 .. j-1 are late
     }
     __syncthreads();
     const int lane = threadIdx.x & 31;

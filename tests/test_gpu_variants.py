@@ -380,3 +380,24 @@ def test_evaluations_in_a_row_wait_for_no_other_stream(policies):
         assert not done.query()
         assert got == want[1] and got != want[0]
     done.synchronize()
+
+
+@pytest.mark.parametrize("n", [1, 129, 700, 20001, 1_300_001])
+@pytest.mark.parametrize("tbt", [0.03, 0.1999, 0.2])
+def test_lags_behind_a_handoff_to_the_server(n, tbt):
+    # many lags of a block are put in order by their lengths before they are made up: lags as widely spread as the server's TTFT, of no
+    # token and of all that are left, intervals that make up hardly anything or nothing of them; a request a thread, and four
+    w = synth.tiny_workload(139 + n, n, n_servers=2, max_prompt=300, max_out=500, device_dearer=True)
+    w.server_ttft_s = np.clip(np.exp(np.random.default_rng(n).normal(0.0, 1.5, n)), 1e-3, 100.0).astype(np.float32)
+    w.servers = [synth.server(jitter=0.2), synth.server(tbt_s=tbt, jitter=0.0)]
+    pols = [synth.policy(b, flags=PACED) for b in (0.3, 1.0)]
+    if n <= 20001:
+        full_parity(w, pols, select=False, tag=f"{n} {tbt}")
+        return
+    from oracle import Oracle
+    from paper_2502_11417_b200 import Trace
+    from parity import check_stats
+    tr = Trace.from_workload(w)
+    tr.eval_policies(pols[1:], w.seed)
+    check_stats(tr.reduce_stats(), Oracle.from_workload(w).eval(pols[1:], w.seed)[0], tr.histograms, f"{n} {tbt}")
+    tr.close()
