@@ -3,6 +3,7 @@
 #include <type_traits>
 
 #include "load.cuh"
+#include "scan.cuh"
 
 namespace disco {
 
@@ -172,26 +173,33 @@ __device__ Sum last_within(double limit) {
 // token) with  sum_l l cnt[l] #{S > w(l)} <= b Total N,  w(l) = 0 for l <= l_immediate, min(beta l, w_tail) above.
 // The sum is exact: it is at most Total N <= 4,096 N^2, which 64 bits hold up to kBetaLargeN requests in the group, and 128
 // (LARGE) beyond.  It does not grow with beta, so beta is found by search: three slopes a
-// round, which cut the range to a quarter.  A thread keeps four prompt lengths and, for each, the two positions in the
+// round, which cut the range to a quarter.  A thread keeps up to four of the prompt lengths that occur and, for each, the two positions in the
 // sorted ticks that belong to the ends of the range, between which the positions of the slopes in between lie; the first
-// and last positions come from the bins' starts in shared memory.  Bound: latency (two barriers and a few dependent loads a
-// round, some fourteen rounds).  (300,000 requests in six groups under sixteen such policies: 437 us with a bisection whose
-// every step searched all the ticks for every length, 79 us now.  Four blocks a pair gave 4 us with few pairs and lost 15
-// once the pairs outnumbered the multiprocessors; three searches in step gave nothing.)
+// and last positions come from the bins' starts in shared memory.  Bound: issue and latency of one block (some eleven rounds by bins of
+// two barriers and up to a dozen products a thread, two by ticks).  (300,000 requests in six groups under sixteen such policies: 437 us
+// with a bisection whose every step searched all the ticks for every length, 82 with every length and products of 64 by 64 bits, 31 of
+// them the rounds by bins, 60 now.  Four blocks a pair gave 4 us with few pairs and lost 15 once the pairs outnumbered the
+// multiprocessors; three searches in step gave nothing.)
 constexpr int kBetaThreads = 1024;
 constexpr int kBetaLens = kMaxPrompt / kBetaThreads;                  // prompt lengths a thread has
 static_assert(kBetaLens * kBetaThreads == kMaxPrompt, "lengths 1 .. 4096");
 constexpr uint64_t kBetaLargeN = 47453132;
 static_assert(kMaxPrompt * kBetaLargeN < (1ull << 63) / kBetaLargeN && kMaxPrompt * (kBetaLargeN + 1) >= (1ull << 63) / (kBetaLargeN + 1), "the last N");
 
-template <bool LARGE>
+// SMALL: a group has fewer than 2^20 requests, so that a length's tokens fit in 32 bits.
+constexpr uint64_t kBetaSmallN = 1u << 20;
+static_assert(kMaxPrompt * kBetaSmallN <= 1ull << 32, "a length's tokens");
+template <bool LARGE, bool SMALL>
 __global__ void __launch_bounds__(kBetaThreads)
 k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __restrict__ cum_mass,
             const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
             const uint32_t* __restrict__ tick_start, const uint32_t* __restrict__ tick_cnt, const uint32_t* __restrict__ pairs,
             Prep* __restrict__ prep, bool early) {
     __shared__ uint32_t s_end[kTickBins];                             // ticks of the group up to the bin's last
+    __shared__ uint16_t s_len[kMaxPrompt];                            // the lengths that requests have
+    __shared__ uint32_t s_wtot[32];
     __shared__ long long part[8][32], total[6];
+    using Mass = typename std::conditional<SMALL, uint32_t, unsigned long long>::type;
     using Sum = typename std::conditional<LARGE, __int128, long long>::type;
     grid_dependency_wait();
     if (early) let_next_start();
@@ -206,31 +214,46 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
     const int32_t* srt = sorted + off;
     const double Total = (double)cum_mass[(size_t)g * (kMaxPrompt + 2) + kMaxPrompt + 1];
     const Sum limit = last_within<Sum>(__dmul_rn(__dmul_rn((double)pc.budget, Total), (double)N));
-    const long long w_tail = pr.w_tail, l_imm = pr.l_star;
+    const uint32_t w_tail = (uint32_t)pr.w_tail, l_imm = (uint32_t)pr.l_star;
     for (int k = threadIdx.x; k < kTickBins; k += kBetaThreads)
         s_end[k] = tick_start[(size_t)g * kTickBins + k] + tick_cnt[(size_t)g * kTickBins + k] - off;
+    // a thread's four lengths, and from then on every 1,024th of those that requests have: each of these costs a round as much, and the
+    // long ones are few
+    uint32_t lengths, own = 0;
+    {
+        uint32_t c[kBetaLens];
+#pragma unroll
+        for (int i = 0; i < kBetaLens; ++i) {
+            c[i] = cnt[(size_t)g * (kMaxPrompt + 1) + 1 + threadIdx.x * kBetaLens + i];
+            own += c[i] ? 1u : 0u;
+        }
+        uint32_t at = block_inclusive_scan(own, s_wtot, &lengths) - own;
+#pragma unroll
+        for (int i = 0; i < kBetaLens; ++i) if (c[i]) s_len[at++] = (uint16_t)(1 + threadIdx.x * kBetaLens + i);
+    }
     __syncthreads();
 
     // ticks at or below w, known to be between lo and hi of them
-    auto position = [&](long long w, uint32_t lo, uint32_t hi) {
+    auto position = [&](uint32_t w, uint32_t lo, uint32_t hi) {
         if (lo < hi) {
-            const int bin = tick_bin((uint32_t)w);
+            const int bin = tick_bin(w);
             if (bin > 0) lo = max(lo, s_end[bin - 1]);
             hi = min(hi, s_end[bin]);
         }
         while (lo < hi) {
             const uint32_t mid = LARGE ? lo + ((hi - lo) >> 1) : (lo + hi) >> 1;       // (their sum may pass 2^32)
             if (!DBG_OK(mid, N, DBG_K_PREP, DBG_ELEMENT)) break;
-            if ((long long)srt[mid] <= w) lo = mid + 1; else hi = mid;
+            if ((uint32_t)srt[mid] <= w) lo = mid + 1; else hi = mid;
         }
         return lo;
     };
-    uint32_t k[kBetaLens], at_lo[kBetaLens], at_hi[kBetaLens];        // requests of the length; positions at the range's ends
-    int len[kBetaLens];
+    Mass tokens[kBetaLens];                                           // of the requests of the length (0: there is no such length)
+    uint32_t len[kBetaLens], at_lo[kBetaLens], at_hi[kBetaLens];      // positions at the range's ends
 #pragma unroll
     for (int i = 0; i < kBetaLens; ++i) {
-        len[i] = 1 + (int)threadIdx.x + i * kBetaThreads;
-        k[i] = cnt[(size_t)g * (kMaxPrompt + 1) + len[i]];
+        const uint32_t x = threadIdx.x + i * kBetaThreads;
+        len[i] = x < lengths ? s_len[x] : 1u;
+        tokens[i] = x < lengths ? (Mass)len[i] * cnt[(size_t)g * (kMaxPrompt + 1) + len[i]] : (Mass)0;
     }
     // the block's sums of the values, the same to all threads.  Over a warp the lanes halve what they add up at every step
     // (nine exchanges for six values, not thirty); a warp then adds up the warps' parts of one value for all.
@@ -273,8 +296,13 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
             for (int j = 0; j < kValues; ++j) v[j] = ((Sum)high[j] << 48) + low[j];
         }
     };
-    auto wait = [&](long long beta, int l) { return l <= l_imm ? 0ll : min(beta * (long long)l, w_tail); };
-    long long lo = 0, hi = w_tail + 1;                                // beyond hi every wait is w_tail
+    // (a slope is at most w_tail + 1)
+    auto wait = [&](long long beta, uint32_t l) {
+        const unsigned long long w = (unsigned long long)(uint32_t)beta * l;
+        return l <= l_imm ? 0u : w < w_tail ? (uint32_t)w : w_tail;
+    };
+    auto mass = [&](Mass t, uint32_t requests) { return LARGE ? (Sum)t * (Sum)requests : (Sum)((unsigned long long)t * requests); };
+    long long lo = 0, hi = (long long)w_tail + 1;                     // beyond hi every wait is w_tail
     // ---- first by whole bins: the ticks up to a bin's first and last bound the sum from both sides, which settles most of
     //      the range without a look at the ticks
     while (hi - lo > 1) {
@@ -283,13 +311,12 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
         Sum v[6] = {0, 0, 0, 0, 0, 0};                                // at least, at most
 #pragma unroll
         for (int i = 0; i < kBetaLens; ++i) {
-            if (k[i] == 0) continue;
-            const Sum mass = (long long)len[i] * (long long)k[i];
+            if (tokens[i] == 0) continue;
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                const int bin = tick_bin((uint32_t)wait(m[j], len[i]));
-                v[j] += mass * (long long)(N - s_end[bin]);
-                v[3 + j] += mass * (long long)(N - (bin ? s_end[bin - 1] : 0u));
+                const int bin = tick_bin(wait(m[j], len[i]));
+                v[j] += mass(tokens[i], N - s_end[bin]);
+                v[3 + j] += mass(tokens[i], N - (bin ? s_end[bin - 1] : 0u));
             }
         }
         totals(v);
@@ -306,12 +333,11 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
 #pragma unroll
         for (int i = 0; i < kBetaLens; ++i) {
             at_lo[i] = at_hi[i] = 0;
-            if (k[i] == 0) continue;
+            if (tokens[i] == 0) continue;
             at_lo[i] = position(wait(lo, len[i]), 0u, N);
             at_hi[i] = len[i] <= l_imm ? at_lo[i] : position(wait(hi, len[i]), at_lo[i], N);
-            const Sum mass = (long long)len[i] * (long long)k[i];
-            v[0] += mass * (long long)(N - at_lo[i]);
-            v[1] += mass * (long long)(N - at_hi[i]);
+            v[0] += mass(tokens[i], N - at_lo[i]);
+            v[1] += mass(tokens[i], N - at_hi[i]);
         }
         totals(v);
         if (lo == 0 && v[0] <= limit) hi = lo;                // (no waits at all fit)
@@ -328,8 +354,8 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 at[j][i] = at_lo[i];
-                if (k[i] != 0 && at_lo[i] < at_hi[i]) at[j][i] = position(wait(m[j], len[i]), at_lo[i], at_hi[i]);
-                v[j] += (Sum)((long long)len[i] * (long long)k[i]) * (long long)(N - at[j][i]);
+                if (at_lo[i] < at_hi[i]) at[j][i] = position(wait(m[j], len[i]), at_lo[i], at_hi[i]);
+                v[j] += mass(tokens[i], N - at[j][i]);
             }
         }
         totals(v);
@@ -380,7 +406,7 @@ cudaError_t launch_prep(uint32_t P, int G, const GroupConst* gc, const int64_t* 
 cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off, const uint32_t* tick_start,
                              const uint32_t* tick_cnt, const uint32_t* pairs, uint32_t n_pairs, uint64_t most, Prep* prep, bool early, cudaStream_t st) {
-    auto* kernel = most > kBetaLargeN ? k_prep_beta<true> : k_prep_beta<false>;
+    auto* kernel = most > kBetaLargeN ? k_prep_beta<true, false> : most < kBetaSmallN ? k_prep_beta<false, true> : k_prep_beta<false, false>;
     return launch_after(kernel, n_pairs, kBetaThreads, 0, st, pol, P, cum_mass, cnt, sorted, grp_off, tick_start,
                         tick_cnt, pairs, prep, early);
 }

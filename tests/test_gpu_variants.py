@@ -401,3 +401,21 @@ def test_lags_behind_a_handoff_to_the_server(n, tbt):
     tr.eval_policies(pols[1:], w.seed)
     check_stats(tr.reduce_stats(), Oracle.from_workload(w).eval(pols[1:], w.seed)[0], tr.histograms, f"{n} {tbt}")
     tr.close()
+
+
+@pytest.mark.parametrize("n", [(1 << 20) - 1, 1 << 20, (1 << 20) + 1])
+@pytest.mark.parametrize("lengths", [1, 900, 4096])
+def test_linear_wait_rule_of_many_requests(n, lengths):
+    # the slope search multiplies in 32 bits below 2^20 requests of a group, and takes the prompt lengths that occur
+    from oracle import Oracle
+    from paper_2502_11417_b200 import Trace
+    from parity import check_prep
+    w = synth.tiny_workload(149, n, max_prompt=lengths, max_out=4, device_dearer=True)
+    w.prompt_len[:3] = 4096                        # (tokens of a length close to 2^32 where all but these have one)
+    if lengths == 1:
+        w.prompt_len[3:] = 4095
+    pols = [synth.policy(b, flags=PACED | synth.FLAG_BETA_RULE | synth.MODE_DEVICE_CONSTRAINED, l_immediate=li) for b in (0.06, 0.5, 1.0) for li in (0, 100)]
+    tr = Trace.from_workload(w)
+    tr.eval_policies(pols, 1)
+    check_prep(tr, Oracle.from_workload(w), pols, f"{n} {lengths}")
+    tr.close()
