@@ -1,7 +1,10 @@
 // Traces in pageable host memory: packed to nine bytes a request in page-locked slots by several threads, while the calling
 // thread copies to the device what is packed, several neighbouring chunks at a time (a copy costs some 5 us besides its
-// bytes, and copies issued by several threads wait for one another).  Bound: reading the caller's columns (14 bytes a
-// request, 10 GB/s a thread, 54 GB/s eight) and the link (9 bytes a request).
+// bytes, 2 of them behind the one in front, and copies issued by several threads wait for one another), and packs itself while there
+// is nothing to copy.  Bound: reading the caller's columns (14 bytes a request, 11 GB/s a thread, 55 GB/s eight, 74 twelve, 77 sixteen of
+// 16 cores; with prefetches half of that) and the link (9 bytes a request).
+// (Loads from pageable arrays, us, with chunks of 32,768 requests, eight threads and a calling thread that only copies, and now: 50,000
+// requests 119 and 90, 100,000 131 and 101, 200,000 151 and 126, 2 million 652 and 597, 16 million 5,030 and 4,170.)
 #include "pack.cuh"
 
 #include <algorithm>
@@ -78,27 +81,30 @@ cudaError_t Packer::reserve_slots(uint32_t slots) {
         if ((e = cudaMallocHost((void**)&slots_, slots * kPackBytes))) { slots_ = nullptr; return e; }
         have_ = slots;
     }
-    for (uint32_t k = 0; k < slots; ++k)
+    for (uint32_t k = 0; k < std::min(slots, kCopies); ++k)
         if (!copied_[k] && (e = cudaEventCreateWithFlags(&copied_[k], cudaEventDisableTiming))) { copied_[k] = nullptr; return e; }
     return cudaSuccess;
 }
 
+void Packer::pack_chunk(uint32_t c) {
+    const uint32_t lo = c * kPackChunk;
+    pack_range(*d_, lo, std::min(kPackChunk, (uint32_t)d_->n - lo), slots_ + (c % have_) * kPackBytes);
+    packed_[c % have_].store(c + 1, std::memory_order_release);
+}
+
 // A packing thread: takes chunks until there are none left.
 void Packer::run() {
-    uint64_t seen = 0;
     for (;;) {
         {
             std::unique_lock<std::mutex> lock(m_);
-            wake_.wait(lock, [&] { return stop_ || job_ != seen; });
+            wake_.wait(lock, [&] { return stop_ || calls_ != 0; });
             if (stop_) return;
-            seen = job_;
+            --calls_;
         }
-        const uint32_t n = (uint32_t)d_->n, chunks = (n + kPackChunk - 1) / kPackChunk;
+        const uint32_t chunks = ((uint32_t)d_->n + kPackChunk - 1) / kPackChunk;
         for (uint32_t c; (c = chunk_.fetch_add(1)) < chunks;) {
             while (c >= freed_.load(std::memory_order_acquire) + have_) std::this_thread::yield();   // (ends: the caller counts a failed copy as done)
-            const uint32_t lo = c * kPackChunk;
-            pack_range(*d_, lo, std::min(kPackChunk, n - lo), slots_ + (c % have_) * kPackBytes);
-            packed_[c % have_].store(c + 1, std::memory_order_release);
+            pack_chunk(c);
         }
         {
             std::lock_guard<std::mutex> lock(m_);
@@ -108,34 +114,36 @@ void Packer::run() {
     }
 }
 
-// The calling thread: copies what the others have packed, in order.
+// The calling thread: copies what has been packed, in order, and packs while there is nothing to copy.
 cudaError_t Packer::copy_runs(uint32_t chunks, char* dev, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    uint32_t issued = 0, freed = 0, ends[kSlots];                     // of the copies under way, where they end
-    uint32_t first = 0, last = 0;
+    uint32_t issued = 0, freed = 0, ends[kCopies];                    // of the copies under way, where they end
+    uint32_t first = 0, last = 0, mine = chunks;                      // mine: a chunk taken whose slot is not free yet
+    auto ready = [&](uint32_t c) { return packed_[c % have_].load(std::memory_order_acquire) == c + 1; };
     while (issued < chunks) {
         uint32_t k = issued;
-        while (k < chunks && k - issued < kRun && k % have_ >= issued % have_ && packed_[k % have_].load(std::memory_order_acquire) == k + 1) ++k;
-        if (k > issued) {
+        while (k < chunks && k - issued < kRun && k % have_ >= issued % have_ && ready(k)) ++k;
+        // (a few chunks at a time, but for the last ones and those in front of the ring's end)
+        if (last - first < kCopies && (k - issued >= kRunMin || (k > issued && (k == chunks || k % have_ == 0)))) {
             if (!e) {
                 const uint32_t s = issued % have_;
                 e = cudaMemcpyAsync(dev + (size_t)issued * kPackBytes, slots_ + s * kPackBytes, (k - issued) * kPackBytes, cudaMemcpyHostToDevice, st);
-                if (!e) e = cudaEventRecord(copied_[(k - 1) % have_], st);
+                if (!e) e = cudaEventRecord(copied_[last % kCopies], st);
             }
-            ends[last++ % kSlots] = k;
+            ends[last++ % kCopies] = k;
             issued = k;
-        } else if (first != last && issued - freed > have_ / 2) {
+        } else if (first != last && (issued - freed > have_ / 2 || last - first == kCopies)) {
             // the packers may soon want the slots
-            const uint32_t end = ends[first % kSlots];
-            const cudaError_t q = e ? cudaSuccess : cudaEventQuery(copied_[(end - 1) % have_]);
+            const cudaError_t q = e ? cudaSuccess : cudaEventQuery(copied_[first % kCopies]);
             if (q != cudaErrorNotReady) {
                 if (q) e = q;
-                ++first;
-                freed_.store(freed = end, std::memory_order_release);
+                freed_.store(freed = ends[first++ % kCopies], std::memory_order_release);
+                continue;
             }
-        } else {
-            std::this_thread::yield();
         }
+        if (mine == chunks && chunk_.load(std::memory_order_relaxed) < chunks) mine = std::min(chunks, chunk_.fetch_add(1));
+        if (mine < chunks && mine < freed + have_) { pack_chunk(mine); mine = chunks; }
+        else std::this_thread::yield();
     }
     return e;
 }
@@ -151,33 +159,25 @@ cudaError_t Packer::pack(const disco_trace_desc_t& d, char* dev, cudaStream_t st
         return cudaSuccess;
     }
     *at = dev;
-    // two chunks or more to each thread that is started; at most eight, and half the host's cores
-    const size_t want = std::min<size_t>({chunks / 2, (size_t)std::thread::hardware_concurrency() / 2, 8});
+    // two chunks or more to each thread that is started; at most twelve, and three quarters of the host's cores
+    const size_t want = std::min<size_t>({chunks / 2, (size_t)std::thread::hardware_concurrency() * 3 / 4, kThreadsMost});
     d_ = &d;
     chunk_.store(0);
     freed_.store(0);
     for (auto& p : packed_) p.store(0);
+    size_t called = 0;
     if (want > 1) {
         std::lock_guard<std::mutex> lock(m_);
         try {
             while (threads_.size() < want) threads_.emplace_back(&Packer::run, this);
         } catch (...) {}                                               // fewer threads, then
-        running_ = threads_.size();
-        if (running_) ++job_;
+        called = calls_ = running_ = std::min(want, threads_.size());
     }
-    if (want <= 1 || threads_.empty()) {
-        for (uint32_t c = 0; c < chunks; ++c) {
-            const uint32_t s = c % have_, lo = c * kPackChunk;
-            if (c >= have_ && (e = cudaEventSynchronize(copied_[s]))) return e;
-            pack_range(d, lo, std::min(kPackChunk, n - lo), slots_ + s * kPackBytes);
-            if ((e = cudaMemcpyAsync(dev + (size_t)c * kPackBytes, slots_ + s * kPackBytes, kPackBytes, cudaMemcpyHostToDevice, st)) ||
-                (e = cudaEventRecord(copied_[s], st))) return e;
-        }
-        return cudaSuccess;
-    }
-    wake_.notify_all();
+    for (size_t k = 0; k < called; ++k) wake_.notify_one();
     e = copy_runs(chunks, dev, st);
     std::unique_lock<std::mutex> lock(m_);
+    running_ -= calls_;                                                // (who has not come by now is not needed)
+    calls_ = 0;
     done_.wait(lock, [&] { return running_ == 0; });
     return e;
 }

@@ -11,9 +11,9 @@
 
 namespace disco {
 
-// Packed requests, a chunk of 32,768 after another: lengths (prompt | output << 16), TTFTs, groups (a byte each).  A length
+// Packed requests, a chunk of 8,192 after another: lengths (prompt | output << 16), TTFTs, groups (a byte each).  A length
 // or profile out of range is packed as 0 or 255, which the ingestion kernel refuses with the same error.
-constexpr uint32_t kPackChunk = 32768;
+constexpr uint32_t kPackChunk = 8192;
 constexpr size_t kPackBytes = (size_t)kPackChunk * 9;
 constexpr uint32_t kPackInPlace = 8192;       // traces up to this size are read from the pinned slots, without a copy
 inline size_t packed_bytes(uint32_t n) { return ((size_t)n + kPackChunk - 1) / kPackChunk * kPackBytes; }
@@ -31,20 +31,23 @@ public:
     cudaError_t pack(const disco_trace_desc_t& d, char* dev, cudaStream_t st, const char** at);
 
 private:
-    static constexpr uint32_t kSlots = 32;    // chunks in page-locked memory at a time (9 MB)
-    static constexpr uint32_t kRun = 8;       // chunks that go with one copy, at most
+    static constexpr uint32_t kSlots = 128;   // chunks in page-locked memory at a time (9 MB)
+    static constexpr uint32_t kCopies = 32;   // copies under way, at most
+    static constexpr uint32_t kRunMin = 8, kRun = 32;   // chunks that go with one copy
+    static constexpr size_t kThreadsMost = 12;
     cudaError_t reserve_slots(uint32_t slots);
     cudaError_t copy_runs(uint32_t chunks, char* dev, cudaStream_t st);
+    void pack_chunk(uint32_t c);
     void run();
 
     char* slots_ = nullptr;
     uint32_t have_ = 0;
-    cudaEvent_t copied_[kSlots] = {};         // after the copy that ends with the slot
+    cudaEvent_t copied_[kCopies] = {};        // after each copy, by turns
     std::vector<std::thread> threads_;
     std::mutex m_;
     std::condition_variable wake_, done_;
-    uint64_t job_ = 0;
-    size_t running_ = 0;
+    size_t calls_ = 0;                        // threads the job in work still asks for
+    size_t running_ = 0;                      // ... and those that have not ended their part
     bool stop_ = false;
     const disco_trace_desc_t* d_ = nullptr;   // the job in work
     std::atomic<uint32_t> chunk_{0};          // next chunk to pack
