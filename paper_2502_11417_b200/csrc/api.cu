@@ -4,6 +4,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <memory>
 #include <new>
@@ -539,6 +540,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     std::vector<ClassConst> classes;
     bool any_beta = false;                // some policy uses the Eq. 1-2 wait rule
     bool extras = false;                  // some policy routes at random or triggers on an expected length
+    bool any_waits = false;               // Algorithm 2 decides for some policy in some group
+    const bool any_constrained = std::any_of(c->gc.begin(), c->gc.end(), [](const GroupConst& g) { return g.auto_device_constrained != 0; });
     int64_t tau = 0, t_m = 0;
     for (uint32_t p = 0; p < P; ++p) {
         const disco_policy_t& q = pol[p];
@@ -562,6 +565,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         o.tau = (int32_t)tau; o.B = (int32_t)B; o.mode = (int32_t)mode;
         o.expected_len = q.expected_len; o.l_immediate = q.l_immediate;
         if (q.flags & DISCO_FLAG_BETA_RULE) any_beta = true;
+        any_waits = any_waits || mode == 1 || (mode == 0 && any_constrained);
         o.route_all = q.budget >= 1.0f ? 1 : 0;
         o.route_thr = o.route_all ? 0xFFFFFFFFu : (uint32_t)std::floor((double)q.budget * 4294967296.0);
         if ((q.flags & (DISCO_FLAG_STOCHASTIC | DISCO_FLAG_BETA_RULE)) || q.expected_len) extras = true;
@@ -922,7 +926,15 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         tables.chunk_len[which] = CH; tables.n_chunks[which] = count;
     };
     const size_t at_once = (size_t)sms * grid_blocks_per_sm(tallest);
-    plan_chunks(0, chunk_size(std::max<size_t>(2 * at_once / std::min<size_t>(most_slabs, 4), 1), 256));
+    // (requests side by side: a chunk is a thread's request or a few)
+    int widest = 1, groups = 0;
+    for (const Slab& sl : slabs) widest = std::max(widest, sl.K);
+    for (int g = 0; g < G; ++g) groups += rb.ng[g] != 0;
+    bool joined = grid_joins(n, groups, widest, tallest);
+#ifdef DISCO_DEBUG
+    if (std::getenv("DISCO_DEBUG_RUNS")) joined = false;
+#endif
+    plan_chunks(0, joined && !stored ? chunk_size((size_t)sms * 8, 256) : chunk_size(std::max<size_t>(2 * at_once / std::min<size_t>(most_slabs, 4), 1), 256));
     if (any_pairs) plan_chunks(1, chunk_size((size_t)2 * sms, 2048));
 
     // ---- device memory: what must be clear comes first and together -- the work counters and tickets, the difference
@@ -1048,7 +1060,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
             }
             CU(launch_grid(tr, gc, d_classes, prep, P, dsl, (uint32_t)b.count, b.T, b.wide, d_tab,
-                           d_chunks, tables.n_chunks[0], rec, rec_stride, gt, left, k0, tickets + ticket, work, beside && ticket == 0, c->sms, st));
+                           d_chunks, tables.n_chunks[0], rec, rec_stride, gt, left, k0, tickets + ticket, work, beside && ticket == 0, any_waits, joined, c->sms, st));
             ++ticket;
             CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, b.wide, d_tab, gt, acc, h_ttft, h_tbt, st));
             g_launches += 2;

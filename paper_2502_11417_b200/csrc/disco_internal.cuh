@@ -309,12 +309,14 @@ struct GridTables { uint32_t* ttft; void* tbt; unsigned long long* sums; };
 struct LeftLists { uint32_t* list; uint32_t* count; };   // [slabs][n] places in the internal order, [slabs][G]
 uint64_t grid_ttft_words(int K), grid_tbt_words(int K, int T), grid_sum_words(int K, int T, int G);
 uint32_t grid_blocks_per_sm(int T);
+bool grid_joins(uint32_t n, int groups /* that have requests */, int K, int T);   // small traces under many policies: requests side by side
 int grid_rows(int T);            // rows the kernel that takes such a slab is built for
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* classes, const Prep* prep, uint32_t P,
                         const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide /* of all of them */,
                         const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec /* of slot 0 */, size_t rec_stride, GridTables gt,
                         LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t k0, uint32_t* ticket /* zero */,
-                        uint64_t* work /* [4], added to */, bool beside /* runs beside its predecessor, whose own it has complete */, int sms, cudaStream_t st);
+                        uint64_t* work /* [4], added to */, bool beside /* runs beside its predecessor, whose own it has complete */,
+                        bool waits /* Algorithm 2 decides in some group */, bool joined /* requests side by side, not run by run */, int sms, cudaStream_t st);
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
                           bool wide, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
                           uint64_t* hist_tbt, cudaStream_t st);

@@ -9,24 +9,24 @@
 //   Algorithm 2:  columns [0, k1) have l* < l   -> wait w_tail;     [k1, k2) have l* = l -> wait their own w*;
 //                 [k2, K) have l* > l           -> wait 0.
 // k, k1, k2 depend on the prompt length alone, and the requests of a group are stored by prompt length: a chunk of
-// requests splits into a few SEGMENTS of consecutive requests that share them.  A block sweeps a segment once per run
-// with a lane per request, sums up what the requests come to in registers and shared-memory histograms, and enters the
-// run's totals ONCE into a table of differences along the columns (row q is carried to the columns from q on: a run of the
-// columns [a, b) is entered into row a and taken back in row b).  k_spread adds the rows up and writes every policy's
-// sums and histograms.
-// Under Algorithm 2 the first columns (budgets below the tail ratio) may wait longer than the others: for the few
-// requests that the common w_tail does not cover (at most a share alpha of them) the block keeps a list, and each of
-// those columns gets the list's totals under its own wait in place of the common one.
+// requests splits into a few SEGMENTS of consecutive requests that share them.  A block sweeps a segment with a lane per
+// request, sums up what the requests come to in registers and shared-memory histograms, and enters a run's totals ONCE into a
+// table of differences along the columns (row q is carried to the columns from q on: a run of the columns [a, b) is entered
+// into row a and taken back in row b).  k_spread adds the rows up and writes every policy's sums and histograms.
+// The last run of a segment and the first are swept together: where the device runs alone, or where the common w_tail covers a
+// request (S <= w_tail: the server answers alone), the first run adds little to what is read.  The requests that w_tail does not
+// cover (at most a share alpha of them) go on a list of the block's, swept again for the first run, and once for each of the
+// columns that wait longer (budgets below the tail ratio).
+// Small traces leave a run few requests: there a lane takes a request with all its runs (see below).
 //
 // The rows differ in the hand-off alone: a race won by the endpoint that may hand over migrates in the rows whose
 // overhead is below the request's saving.  Every sweep adds what migration changes to each row whose overhead it passes
-// (three additions a row); the hand-off stall is counted at the level of the last such row, and the levels are summed
-// up when the run is entered.
+// (three additions a row), or, with eight rows, to the last of them; the hand-off stall is counted at the level of the last such
+// row, and the levels are summed up when the run is entered.
 //
-// Bound: integer issue.  Against one sweep per 128 policies of one overhead, with what differs between neighbouring
-// policies entered into their histograms one by one, a request is visited once per run instead of once per run and
-// overhead: 16 M requests in six groups under 128 budgets by 8 overheads took 2,300 us (and 450 more pair by pair), now
-// 349 and k_spread 18; a million in one group under 256 by 4 took 220 us, now 35 and 15.
+// Bound: integer issue, and a run's latency.  16 M requests in six groups under 128 budgets by 8 overheads: 347 us with a sweep for
+// each run and every row's sums in registers (122 of them, two blocks to a multiprocessor), 247 now (80, three); 5 M under 40 by 8
+// 113 -> 85; a million in one group under 256 by 4 32 -> 28.  (Kernels that also held the way of small traces had to spill: 283 and 99.)
 #include <algorithm>
 #include <cstddef>
 #include <type_traits>
@@ -38,16 +38,20 @@ namespace disco {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kListCap = 8192;           // requests a block lists for the columns with longer waits
-constexpr int kListStep = 4096;          // ... and looks after the list's room every so many requests
+constexpr int kListCap = 4096;           // requests a block lists whose TTFT the common wait does not cover
+// ... of a segment that are entered by warps, a wait each: a handful is not worth a run for every column that waits longer (600,000 requests
+// in six groups under 32 by 2 34 us, now 30).  Not with more rows: the additions to their histograms are as many as the rows, and the call
+// costs registers.
+__host__ __device__ constexpr int list_few(int NT) { return NT > 2 ? 0 : 256 / (1 + NT); }
 constexpr int kMaxSeg = 2 * kGridCols + 2;
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr uint32_t kNoPolicy = 0xFFFFFFFFu;
 static_assert(kNBins % 32 == 0 && kNBins / 32 < 32, "a bit for each group of bins");
 
-// Blocks to a multiprocessor by the rows a kernel is built for: as many as its registers allow with few spills (64 registers:
-// 136 bytes in k_grid<1, true>, 16 in <2, false>; 80: 8 in <2, true>, 20 in <4, true>; the others none).
-__host__ __device__ constexpr int blocks_for(int rows, bool wide) { return rows == 1 || (rows == 2 && !wide) ? 4 : rows <= 4 ? 3 : 2; }
+// Blocks to a multiprocessor by the rows a kernel is built for: as many as its registers allow with few spills (with windows up to
+// 76 bytes, without up to 20).
+enum GridMode { M_RACES = 0, M_WAITS, M_JOINED };
+__host__ __device__ constexpr int blocks_for(int rows, bool wide, int mode) { return mode == M_JOINED ? (rows <= 2 ? 4 : 3) : rows <= (wide ? 1 : 2) ? 4 : rows <= 4 || !wide ? 3 : 2; }
 // The rows of the kernel that takes a slab of T.
 constexpr int rows_for(int T) { return T <= 1 ? 1 : T <= 2 ? 2 : T <= 4 ? 4 : 8; }
 
@@ -58,29 +62,8 @@ __host__ __device__ constexpr int sum_fields(int T) { return kBase + T * kLev; }
 
 struct Seg { uint16_t pa, pb, k1, k2; };               // requests [pa, pb) of the chunk
 
-struct Smem {                                          // fixed part; the TBT histograms [T][kNBins] follow, and one more for
-                                                       // the device-only run where windows are counted
-    uint32_t sum[kBase + kGridRows * kLev];            // totals of the run in work
-    uint32_t only_sum[4];                              // ... of the device-only run: requests, tokens, prompt tokens, TBTs in tau's bin
-    uint32_t tt[3], only_tt[3];                        // ... and the sums of TTFTs, in parts of 20 bits
-    uint32_t ttft[kNBins], only_ttft[kNBins];
-    uint32_t used[2][3];                               // groups of bins with counts: TTFT, stall, device only; by turns
-    uint32_t n_seg, n_runs, n_list, flagged, ticket;
-    int32_t key[kGridCols];                            // the columns' length thresholds
-    uint32_t w_star[kGridCols], w_tail[kGridCols];
-    Seg seg[kMaxSeg];
-    uint16_t list[kListCap];
-};
-
-template <int NT>
-struct Acc {                                           // a lane's share of a run
-    uint32_t td, ps, pd, tau, race, dw;
-    unsigned long long tt;
-    uint32_t bins, stalls;                             // groups of 32 bins with counts: of the TTFTs, of the hand-off stalls
-    uint32_t a[NT], b[NT], cn[NT], tx[NT];             // cn: delayed tokens | requests << 22 (at most 255 requests a lane)
-};
-
-struct Only { uint32_t cnt, n, l, tau, bins; unsigned long long tt; };   // ... of a device-only run
+// Whether a lane's shares of what migration changes lie in shared memory, level by level (see Levels).
+__host__ __device__ constexpr bool has_levels(int NT, bool wide) { return NT >= 8 && !wide; }
 
 struct Ctx {                                           // a (chunk, slab)
     uint32_t start, len;
@@ -96,6 +79,55 @@ struct Ctx {                                           // a (chunk, slab)
     const uint2* hand;
     size_t win_at;                                     // bytes from the windows of slot 0
 };
+
+// Whether the bins of the TTFTs that a run has counts in are remembered: not where windows may lie anywhere, nor in the kernel of eight
+// rows, which has no registers left for it.
+__host__ __device__ constexpr bool knows_bins(int NT, bool wide) { return !wide && !has_levels(NT, wide); }
+
+struct __align__(16) Smem {                            // fixed part; the TBT histograms [T][kNBins] follow, and one more for
+                                                       // the run beside where windows are counted, or the warps' levels
+    uint32_t sum[2][kBase + kGridRows * kLev];         // totals of the run in work; by turns
+    uint32_t side_sum[4];                              // ... of the run beside it: requests, tokens, prompt tokens, TBTs in tau's bin
+    uint32_t tt[3], side_tt[3];                        // ... and the sums of TTFTs, in parts of 20 bits
+    uint32_t ttft[kNBins], side_ttft[kNBins];
+    uint32_t used[2][3];                               // groups of bins with counts: TTFT, stall, TTFT of the run beside; by turns
+    uint32_t n_seg, n_list, flagged, ticket;
+    int32_t key[kGridCols];                            // the columns' length thresholds
+    uint32_t w_star[kGridCols], w_tail[kGridCols];
+    Seg seg[kMaxSeg];
+    uint16_t list[kListCap];
+    Ctx ctx;                                           // of the item, and its overheads, for what is called and not inlined
+    float rows[kGridRows];
+    uint32_t slab;
+};
+
+static_assert(sizeof(Smem) % 16 == 0 && kNBins % 2 == 0, "the levels are read in words of eight bytes");
+
+template <int NT, bool WIDE>
+struct Acc {                                           // a lane's share of a run
+    static constexpr int kRows = has_levels(NT, WIDE) ? 0 : NT;
+    uint32_t td, ps, pd, tau, race, dw;
+    unsigned long long tt;
+    uint32_t bins, stalls;                             // groups of 32 bins with counts: of the TTFTs, of the hand-off stalls
+    uint32_t levels;                                   // a bit a level with requests
+    uint32_t a[kRows + 1], b[kRows + 1], cn[kRows + 1], tx[kRows + 1];   // cn: delayed tokens | requests << 22 (at most 255 requests a lane)
+};
+
+struct Side { uint32_t cnt, n, l, tau, bins; unsigned long long tt; };   // ... of the run beside it
+
+// With eight rows a request does not go to every row that it migrates in but to the last of them, its level, and the levels are
+// added up when the run is entered.  (With four, registers do: a million requests under 256 by 4 28 us, by levels 36.)  A lane's shares lie in shared memory, a column of the warp's for each lane, which nobody else
+// touches: handed-over tokens and prefill side by side, then delayed tokens | requests << 22.
+template <int NT>
+struct Levels {
+    uint2* ab;                                         // [NT][32]
+    uint32_t* cn;                                      // [NT][32]
+    static constexpr int kWords = NT * 96;             // of a warp
+    __device__ explicit Levels(uint32_t* at) : ab(reinterpret_cast<uint2*>(at)), cn(at + NT * 64) {}
+};
+
+// Words behind the fixed part: the TBT histograms and what follows them.
+__host__ __device__ constexpr int tbt_words(int NT, bool wide) { return (NT + (wide ? 1 : 0)) * kNBins + (has_levels(NT, wide) ? kThreads / 32 * NT * 96 : 0); }
 
 struct Args {
     TraceDev tr;
@@ -189,24 +221,27 @@ __device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_
 }
 
 // One sweep over the requests [pa, pb) of the chunk, or (list) of the block's list: what they come to when the device
-// starts after the wait w, added up in `s` and in the shared histograms.  push: requests with S > w go on the list.
-// ONLY: the segment is Algorithm 3's; `race` says whether some columns race (w = 0), `only` whether some run the device
-// alone, which is added up in `o` and histograms of its own.
-template <int NT, bool WIDE, bool ONLY>
-__device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (&th)[NT], Smem& sm, uint32_t* tbt, uint32_t pa,
-                                      uint32_t pb, uint32_t w, bool list, bool push, bool race, bool only, Acc<NT>& s, Only& o) {
+// starts after the wait w, added up in `s` and in the shared histograms.
+// SIDE: a segment's requests under its last columns, which wait 0 (`race`: there are such columns), and beside them under its first
+// ones (`side`), added up in `o` and histograms of its own: Algorithm 3's, where the device runs alone, or (S_EITHER, `waits`) Algorithm
+// 2's, which wait w: there the server alone answers the requests with S <= w, and the others go on the list.
+// push: requests with S > w go on the list (without a run beside).
+enum SideKind { S_NONE = 0, S_DEVICE, S_EITHER };
+template <int NT, bool WIDE, int SIDE>
+__device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (&th)[NT], Smem& sm, uint32_t* tbt, const Levels<NT>& lv,
+                                      uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, bool given_waits, bool race, bool side, Acc<NT, WIDE>& s, Side& o) {
+    const bool waits = SIDE == S_EITHER && given_waits;
     const int lane = threadIdx.x & 31;
-    // The kernel of eight rows has too few warps a multiprocessor to hide the loads' latency: there they run an iteration
-    // ahead (16 M requests under 128 budgets by 8 overheads, with k_spread, 369 us instead of 435; the others have the
-    // warps, and no registers left: 3 % slower).
+    // The kernel of eight rows has too few warps a multiprocessor to hide the loads' latency: there they run an iteration ahead.
     constexpr bool kAhead = NT == 8 && !WIDE;
+    constexpr bool kLevels = has_levels(NT, WIDE);
     uint32_t pos;
     uint4 q, q_ahead;
     uint2 hand, hand_ahead;
     uint32_t ahead;
     auto fetch = [&](uint32_t i0, uint32_t& at, uint4& to, uint2& to_hand) {
         const uint32_t i = min(i0 + lane, pb - 1);
-        at = list ? (uint32_t)sm.list[i] : i;
+        at = !SIDE && list ? (uint32_t)sm.list[i] : i;
         to = a.tr.req[c.start + at];
         to_hand = c.may_migrate ? c.hand[c.start + at] : make_uint2(0u, 0u);
     };
@@ -226,23 +261,36 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
         // Eq. 4's projected saving, on the true remainder or on what is left of the expected length; a request may only
         // hand over if its buffer filled (m != 0)
         float saving = m ? c.delta_c * (float)(c.E0 ? max(c.E0 - (int)m, 0) : (int)(n - m)) : -1.0f;
-        if (c.mixed) valid = valid && !(saving > c.th_lo && !(saving > th[0]));       // left to the pair kernel
-        if (ONLY) {
-            if (only) {
-                const int bin = bin_of_ticks(Td);
-                const uint32_t live = __ballot_sync(FULL, valid);
-                // requests of one prompt length share the device's TTFT: mostly the whole warp counts in one bin
-                if (__shfl_sync(FULL, l, 0) == __shfl_sync(FULL, l, 31)) {
-                    if (lane == 0 && live && DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) atomicAdd(&sm.only_ttft[bin], (uint32_t)__popc(live));
-                } else if (valid) hist_add(sm.only_ttft, bin);
-                if (!WIDE && valid) o.bins |= 1u << (bin >> 5);
-                if (valid) { o.cnt += 1u; o.n += n; o.l += l; o.tt += Td; o.tau += (!WIDE || (c.even & 2u)) ? n - 1u : 0u; }
-                if (WIDE && !(c.even & 2u)) add_rows(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(a.rec.win[1]) + c.win_at), c.cc->W[1], c.cc->lo[c.g][1], live, kk, false, tbt + NT * kNBins);
-            }
-            if (!race) continue;
+        if (NT == 1 && c.mixed) valid = valid && !(saving > c.th_lo && !(saving > th[0]));       // left to the pair kernel
+        if (SIDE && side) {
+            constexpr int stream = 1;                                 // (with windows a run beside is the device's)
+            const bool mine = valid && !(waits && S > w);
+            const uint32_t tt = waits ? S : Td;
+            const uint32_t live = __ballot_sync(FULL, mine);
+            const int bin = bin_of_ticks(tt);
+            // requests of one prompt length share the device's TTFT: mostly the whole warp counts in one bin
+            if (!waits && __shfl_sync(FULL, l, 0) == __shfl_sync(FULL, l, 31)) {
+                if (lane == 0 && live && DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) atomicAdd(&sm.side_ttft[bin], (uint32_t)__popc(live));
+            } else if (mine) hist_add(sm.side_ttft, bin);
+            if (knows_bins(NT, WIDE) && mine) o.bins |= 1u << (bin >> 5);
+            if (mine) { o.cnt += 1u; o.n += n; o.l += l; o.tt += tt; o.tau += (!WIDE || ((c.even >> stream) & 1u)) ? n - 1u : 0u; }
+            if (WIDE && !((c.even >> stream) & 1u))
+                add_rows(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(a.rec.win[stream]) + c.win_at), c.cc->W[stream], c.cc->lo[c.g][stream], live, kk, false, tbt + NT * kNBins);
         }
-        const bool started = S > w, dev_wins = S > w + Td;            // the device starts after the wait; a tie goes to the server
-        const uint32_t tt = min(S, w + Td);
+        if (SIDE == S_EITHER ? waits && side : WIDE && push) {
+            const bool longer = valid && S > w;
+            const uint32_t all = __ballot_sync(FULL, longer);
+            if (all) {
+                uint32_t at = 0;
+                if (lane == 0) at = atomicAdd(&sm.n_list, (uint32_t)__popc(all));
+                at = __shfl_sync(FULL, at, 0) + __popc(all & ((1u << lane) - 1u));
+                if (longer && DBG_OK(at, kListCap, DBG_K_GRID, DBG_SLOT)) sm.list[at] = (uint16_t)pos;
+            }
+        }
+        if (SIDE && !race) continue;
+        const uint32_t wait = SIDE ? 0u : w;
+        const bool started = S > wait, dev_wins = S > wait + Td;      // the device starts after the wait; a tie goes to the server
+        const uint32_t tt = min(S, wait + Td);
         const bool pace = ((c.even >> (dev_wins ? 1 : 0)) & 1u) != 0; // the base stream's intervals are all tau
         if (valid) {
             s.td += dev_wins ? n : 0u; s.ps += l; s.pd += started ? l : 0u;
@@ -251,32 +299,44 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
             s.tau += (!WIDE || pace) ? n - 1u : 0u;
             const int bin = bin_of_ticks(tt);
             hist_add(sm.ttft, bin);
-            if (!WIDE) s.bins |= 1u << (bin >> 5);
-        }
-        if (!ONLY && push) {
-            const bool mine = valid && S > w;
-            const uint32_t all = __ballot_sync(FULL, mine);
-            if (all) {
-                uint32_t at = 0;
-                if (lane == 0) at = atomicAdd(&sm.n_list, (uint32_t)__popc(all));
-                at = __shfl_sync(FULL, at, 0) + __popc(all & ((1u << lane) - 1u));
-                if (mine && DBG_OK(at, kListCap, DBG_K_GRID, DBG_SLOT)) sm.list[at] = (uint16_t)pos;
-            }
+            if (knows_bins(NT, WIDE)) s.bins |= 1u << (bin >> 5);
         }
         if (!(valid && started && (dev_wins ? 2 : 1) == c.cand)) saving = -1.0f;      // not won by the endpoint that may hand over
         const uint32_t handed = n - m, refill = l + m, cn = dly | 1u << 22;
         const uint32_t tx = WIDE ? ((c.even & 4u) ? n - 2u : 0u) - (pace ? n - 1u : 0u) : 0u;
         int t = 0;                                                    // rows that migrate: [0, t)
-#pragma unroll
-        for (int r = 0; r < NT; ++r)
-            if (saving > th[r]) {
-                s.a[r] += handed; s.b[r] += refill; s.cn[r] += cn; ++t;
-                if (WIDE) s.tx[r] += tx;
+        if constexpr (kLevels) {
+            if (saving > th[0]) {
+                static_assert(NT == 4 || NT == 8, "a search in steps of two and one, or four, two and one");
+                if constexpr (NT == 8) {
+                    const bool p4 = saving > th[4], p2 = saving > (p4 ? th[6] : th[2]);
+                    t = (p4 ? 5 : 1) + (p2 ? 2 : 0) + (saving > (p4 ? (p2 ? th[7] : th[5]) : (p2 ? th[3] : th[1])) ? 1 : 0);
+                } else {
+                    const bool p2 = saving > th[2];
+                    t = (p2 ? 3 : 1) + (saving > (p2 ? th[3] : th[1]) ? 1 : 0);
+                }
+                const int at = (t - 1) * 32 + lane;
+                uint2 v = lv.ab[at];
+                v.x += handed; v.y += refill;
+                lv.ab[at] = v;
+                lv.cn[at] += cn;
+                s.levels |= 1u << (t - 1);
+                const int bin = bin_of_ticks(hand.y);
+                hist_add(tbt + (t - 1) * kNBins, bin);
+                s.stalls |= 1u << (bin >> 5);
             }
-        if (t > 0) {
-            const int bin = bin_of_ticks(hand.y);
-            hist_add(tbt + (t - 1) * kNBins, bin);
-            if (!WIDE) s.stalls |= 1u << (bin >> 5);
+        } else {
+#pragma unroll
+            for (int r = 0; r < NT; ++r)
+                if (saving > th[r]) {
+                    s.a[r] += handed; s.b[r] += refill; s.cn[r] += cn; ++t;
+                    if (WIDE) s.tx[r] += tx;
+                }
+            if (t > 0) {
+                const int bin = bin_of_ticks(hand.y);
+                hist_add(tbt + (t - 1) * kNBins, bin);
+                if (!WIDE) s.stalls |= 1u << (bin >> 5);
+            }
         }
         if (WIDE) add_windows(a, c, tbt, valid, kk, dev_wins, t, q.z);
     }
@@ -302,10 +362,10 @@ __device__ __forceinline__ unsigned long long take_wide(uint32_t (&from)[3]) {
 // The lanes' shares of a run go to the block's totals (32-bit: at most 65,280 requests of at most 12,288 tokens).  Lane f
 // of a warp adds field f.
 template <int NT, bool WIDE>
-__device__ __forceinline__ void share_out(Smem& sm, const Acc<NT>& s, int turn) {
+__device__ __forceinline__ void share_out(Smem& sm, const Acc<NT, WIDE>& s, const Levels<NT>& lv, int turn) {
     const int lane = threadIdx.x & 31;
     if (!WIDE) {
-        const uint32_t bins = __reduce_or_sync(FULL, s.bins), stalls = __reduce_or_sync(FULL, s.stalls);
+        const uint32_t bins = knows_bins(NT, WIDE) ? __reduce_or_sync(FULL, s.bins) : 0u, stalls = __reduce_or_sync(FULL, s.stalls);
         if (lane == 0 && bins) atomicOr(&sm.used[turn][0], bins);
         if (lane == 0 && stalls) atomicOr(&sm.used[turn][1], stalls);
     }
@@ -315,24 +375,41 @@ __device__ __forceinline__ void share_out(Smem& sm, const Acc<NT>& s, int turn) 
         if (f < 32) { if (lane == f) lo = v; } else if (lane == f - 32) hi = v;
     };
     put(B_TD, s.td); put(B_PS, s.ps); put(B_PD, s.pd); put(B_RACE, s.race); put(B_DW, s.dw); put(B_TAU, s.tau);
+    if constexpr (has_levels(NT, WIDE)) {
+#pragma unroll 1
+        for (uint32_t left = __reduce_or_sync(FULL, s.levels); left; left &= left - 1u) {
+            const int r = __ffs(left) - 1, at = r * 32 + lane;
+            const uint2 v = lv.ab[at];
+            const uint32_t cn = lv.cn[at];
+            lv.ab[at] = make_uint2(0u, 0u); lv.cn[at] = 0u;
+            const uint32_t x = __reduce_add_sync(FULL, v.x), y = __reduce_add_sync(FULL, v.y), dly = __reduce_add_sync(FULL, cn & 0x3FFFFFu), num = __reduce_add_sync(FULL, cn >> 22);
+            const uint32_t z = lane == V_A ? x : lane == V_B ? y : lane == V_C ? dly : num;
+            if (lane < V_TAU && z) atomicAdd(&sm.sum[turn][kBase + r * kLev + lane], z);
+        }
+    } else {
 #pragma unroll
-    for (int r = 0; r < NT; ++r) {
-        const int f = kBase + r * kLev;
-        put(f + V_A, s.a[r]); put(f + V_B, s.b[r]); put(f + V_C, s.cn[r] & 0x3FFFFFu); put(f + V_N, s.cn[r] >> 22);
-        if (WIDE) put(f + V_TAU, s.tx[r]);
+        for (int r = 0; r < NT; ++r) {
+            const int f = kBase + r * kLev;
+            put(f + V_A, s.a[r]); put(f + V_B, s.b[r]); put(f + V_C, s.cn[r] & 0x3FFFFFu); put(f + V_N, s.cn[r] >> 22);
+            if (WIDE) put(f + V_TAU, s.tx[r]);
+        }
     }
-    if (lo) atomicAdd(&sm.sum[lane], lo);
-    if (NT * kLev + kBase > 32 && hi) atomicAdd(&sm.sum[32 + lane], hi);
+    if (lo) atomicAdd(&sm.sum[turn][lane], lo);
+    if (!has_levels(NT, WIDE) && NT * kLev + kBase > 32 && hi) atomicAdd(&sm.sum[turn][32 + lane], hi);
     add_wide(sm.tt, s.tt);
 }
-__device__ __forceinline__ void share_only(Smem& sm, const Only& o, int turn) {
-    const uint32_t bins = __reduce_or_sync(FULL, o.bins);
-    if ((threadIdx.x & 31) == 0 && bins) atomicOr(&sm.used[turn][2], bins);
+static_assert(V_A == 0 && V_B == 1 && V_C == 2 && V_N == 3 && V_TAU == 4, "a lane a field of a level");
+template <int NT, bool WIDE>
+__device__ __forceinline__ void share_side(Smem& sm, const Side& o, int turn) {
+    if (knows_bins(NT, WIDE)) {
+        const uint32_t bins = __reduce_or_sync(FULL, o.bins);
+        if ((threadIdx.x & 31) == 0 && bins) atomicOr(&sm.used[turn][2], bins);
+    }
     const uint32_t c = __reduce_add_sync(FULL, o.cnt), n = __reduce_add_sync(FULL, o.n), l = __reduce_add_sync(FULL, o.l),
                    tau = __reduce_add_sync(FULL, o.tau);
-    add_wide(sm.only_tt, o.tt);
+    add_wide(sm.side_tt, o.tt);
     if ((threadIdx.x & 31) == 0 && c) {
-        atomicAdd(&sm.only_sum[0], c); atomicAdd(&sm.only_sum[1], n); atomicAdd(&sm.only_sum[2], l); atomicAdd(&sm.only_sum[3], tau);
+        atomicAdd(&sm.side_sum[0], c); atomicAdd(&sm.side_sum[1], n); atomicAdd(&sm.side_sum[2], l); atomicAdd(&sm.side_sum[3], tau);
     }
 }
 
@@ -363,6 +440,12 @@ __device__ __forceinline__ void each_bin(uint32_t groups, F f) {
         if (k % (kThreads / 32) == w) f((__ffs(groups) - 1) * 32 + lane);
 }
 
+// What the run before used is clear for the next one (all have read it).
+__device__ __forceinline__ void clear_before(Smem& sm, int turn) {
+    for (int f = threadIdx.x; f < kBase + kGridRows * kLev; f += kThreads) sm.sum[turn ^ 1][f] = 0;
+    if (threadIdx.x < 3) sm.used[turn ^ 1][threadIdx.x] = 0;
+}
+
 // Enters what the block has totalled for a run of the columns [q0, q1), or takes it from them (neg), and clears it.  All
 // threads call; barriers before and after.  Only groups of 32 bins that the run has counts in are looked at (a run over all
 // bins of nine histograms took longer than the sweep of a few hundred requests).
@@ -370,7 +453,7 @@ template <int NT, bool WIDE>
 __device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE>& tb, int g, int q0, int q1, bool neg, int turn) {
     using word = typename Tables<WIDE>::word;
     const bool back = q1 < tb.K;
-    each_bin<WIDE>(sm.used[turn][0], [&](int b) {
+    each_bin<!knows_bins(NT, WIDE)>(sm.used[turn][0], [&](int b) {
         const uint32_t x = sm.ttft[b];
         if (x) {
             sm.ttft[b] = 0;
@@ -395,33 +478,35 @@ __device__ __forceinline__ void enter(Smem& sm, uint32_t* tbt, const Tables<WIDE
     });
     const int F = sum_fields(tb.T);
     for (int f = threadIdx.x; f < F; f += kThreads) {
-        unsigned long long x = (f >= kBase && (f - kBase) % kLev == V_TAU) ? (unsigned long long)(long long)(int32_t)sm.sum[f] : sm.sum[f];
-        sm.sum[f] = 0;
+        const uint32_t* sum = sm.sum[turn];
+        unsigned long long x = (f >= kBase && (f - kBase) % kLev == V_TAU) ? (unsigned long long)(long long)(int32_t)sum[f] : sum[f];
+        if (has_levels(NT, WIDE) && f >= kBase)
+            for (int h = f + kLev; h < F; h += kLev) x += sum[h];      // (so do these)
         if (f == B_TT) x = take_wide(sm.tt);
         if (!x) continue;
         if (neg) x = 0ull - x;
         atomicAdd(&tb.sum_row(g, q0)[f], x);
         if (back) atomicAdd(&tb.sum_row(g, q1)[f], 0ull - x);
     }
-    if (threadIdx.x < 3) sm.used[turn ^ 1][threadIdx.x] = 0;          // (of the run before; all have read them)
+    clear_before(sm, turn);
 }
 
-// The same for a device-only run of the columns below q1.
-template <bool WIDE>
-__device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const Tables<WIDE>& tb, int g, int q1, int turn) {
+// The same for the run beside it, of the columns below q1: the device alone, or the server.
+template <int NT, bool WIDE>
+__device__ __forceinline__ void enter_side(Smem& sm, uint32_t* side_tbt, const Tables<WIDE>& tb, int g, int q1, bool server, int turn) {
     using word = typename Tables<WIDE>::word;
     const bool back = q1 < tb.K;
-    each_bin<WIDE>(sm.used[turn][2], [&](int b) {
-        const uint32_t x = sm.only_ttft[b];
+    each_bin<!knows_bins(NT, WIDE)>(sm.used[turn][2], [&](int b) {
+        const uint32_t x = sm.side_ttft[b];
         if (x) {
-            sm.only_ttft[b] = 0;
+            sm.side_ttft[b] = 0;
             atomicAdd(&tb.ttft_row(0)[b], x);
             if (back) atomicAdd(&tb.ttft_row(q1)[b], 0u - x);
         }
         if (WIDE) {
-            const word y = only_tbt[b];
+            const word y = side_tbt[b];
             if (y) {
-                only_tbt[b] = 0;
+                side_tbt[b] = 0;
                 for (int r = 0; r < tb.T; ++r) {
                     atomicAdd(&tb.tbt_row(0, r)[b], y);
                     if (back) atomicAdd(&tb.tbt_row(q1, r)[b], (word)0 - y);
@@ -429,108 +514,221 @@ __device__ __forceinline__ void enter_only(Smem& sm, uint32_t* only_tbt, const T
             }
         }
     });
-    if (threadIdx.x < 3) sm.used[turn ^ 1][threadIdx.x] = 0;
     if (threadIdx.x < 5) {
         const int k = threadIdx.x;
-        const unsigned long long x = k < 4 ? (unsigned long long)sm.only_sum[k] : take_wide(sm.only_tt);
-        if (k < 4) sm.only_sum[k] = 0;
-        const int f = k == 0 ? B_DO : k == 1 ? B_TD : k == 2 ? B_PD : k == 3 ? B_TAU : B_TT;
-        if (x) {
+        const unsigned long long x = k < 4 ? (unsigned long long)sm.side_sum[k] : take_wide(sm.side_tt);
+        if (k < 4) sm.side_sum[k] = 0;
+        const int f = k == 0 ? B_DO : k == 1 ? B_TD : k == 2 ? (server ? B_PS : B_PD) : k == 3 ? B_TAU : B_TT;
+        if (x && !(server && k < 2)) {                                 // (none of these requests runs on the device)
             atomicAdd(&tb.sum_row(g, 0)[f], x);
             if (back) atomicAdd(&tb.sum_row(g, q1)[f], 0ull - x);
         }
     }
+    clear_before(sm, turn);
 }
 
-// A chunk whose runs have few requests each, request by request: a thread enters what its request comes to in every run by
-// itself.  A run swept by the whole block costs its barriers and a walk over all bins (a microsecond or more), which pays
-// only with enough requests to share it.  Bound: the chain of atomics per request, and, with many of them, the L2 slices
-// that the hottest sums live in (lanes that add up first were tried: shorter there, but longer where the lanes' columns
-// differ).  A step of 1,000 requests under 256 budgets 465 -> 114 us, of 10,000 requests under 256 policies with
-// migration 785 -> 185 us.
-//
-// Taken below so many requests to a run: where every block has at most one item the step waits for the slowest item, and
-// the runs' latency decides (64; nothing changes beyond); with more items than blocks the atomics' rate does, and at 24
-// requests to a run 300,000 requests under 128 policies with migration already lose (286 us against 230, 202 at 16).
-constexpr uint32_t kDirectAlone = 64, kDirectMany = 16;
+// ---- side by side: a lane a request, with what it comes to in all its runs.  A run swept by a block costs its barriers, its first
+// loads' latency and a walk over its histograms, some 2.5 us, which pays only with enough requests to share it.  Here the lanes of
+// a warp whose requests have the same runs -- neighbours do, the requests are stored by length -- enter each run together: the sums
+// are added up over the lanes and entered by a lane a field, the histograms by a lane a request (one for all in the same bin).  What is
+// left of a warp enters its runs lane by lane.  Bound: latency for small traces, then the atomic additions (some 250 a nanosecond on
+// all of the GPU).  With every sum entered by every lane 20,000 requests in six groups under 64 budgets took some 40 us, run by run
+// 147, together 11; 100,000 under 32 by 4 80 us, now 20.
+constexpr int kJoin = 8;                               // lanes that join, at least
 
+// Adds to the tables of a slab: a count to a histogram of the columns [q0, q1), a value to a sum.
+struct Adder {
+    unsigned long long* sums;
+    size_t F;
+    int K;
+    __device__ __forceinline__ void count(uint32_t* at, int q0, int q1, uint32_t x) const {
+        atomicAdd(at + (size_t)q0 * kNBins, x);
+        if (q1 < K) atomicAdd(at + (size_t)q1 * kNBins, 0u - x);
+    }
+    __device__ __forceinline__ void add(int f, unsigned long long v, int q0, int q1) const {
+        atomicAdd(sums + q0 * F + f, v);
+        if (q1 < K) atomicAdd(sums + q1 * F + f, 0ull - v);
+    }
+};
+struct Request {                                       // a lane's; level: rows that migrate where the winner may hand over, [0, level)
+    uint32_t S, l, n, m, dly, Td;
+    int stall, level;
+};
 template <int NT>
-__device__ __noinline__ void enter_requests(const Args& a, const Ctx& c, const float (&th)[NT], const Smem& sm,
-                                            const Tables<false>& tb, bool waits, uint32_t wt_min, int n_low) {
-    const int K = c.K;
-    for (uint32_t i = threadIdx.x; i < c.len; i += kThreads) {
-        const uint32_t kk = c.start + i;
-        const uint4 q = a.tr.req[kk];
-        const uint2 hand = c.may_migrate ? c.hand[kk] : make_uint2(0u, 0u);
-        const uint32_t S = q.x, l = q.y & 0xFFFFu, n = q.y >> 16, m = hand.x & 0xFFFFu, dly = hand.x >> 16;
-        const uint32_t Td = c.kappa * l + c.c0;
-        const float saving = m ? c.delta_c * (float)(c.E0 ? max(c.E0 - (int)m, 0) : (int)(n - m)) : -1.0f;
-        if (c.mixed && saving > c.th_lo && !(saving > th[0])) continue;               // left to the pair kernel
-        // adds (or takes) a count to a histogram of the columns [q0, q1), a value to a sum
-        auto count = [&](uint32_t* at, int q0, int q1) {
-            atomicAdd(at + (size_t)q0 * kNBins, 1u);
-            if (q1 < K) atomicAdd(at + (size_t)q1 * kNBins, ~0u);
-        };
-        const size_t F = sum_fields(c.T);
-        auto add = [&](int f, unsigned long long v, int q0, int q1) {
-            unsigned long long* at = tb.sum_row(c.g, 0) + f;
-            atomicAdd(at + q0 * F, v);
-            if (q1 < K) atomicAdd(at + q1 * F, 0ull - v);
-        };
-        // what the request comes to under the columns [q0, q1), which start the device after w
-        auto enter_run = [&](uint32_t w, int q0, int q1) {
-            const bool started = S > w, dev_wins = S > w + Td;
-            const uint32_t tt = min(S, w + Td);
-            const int bin = bin_of_ticks(tt);
-            if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) count(tb.ttft + bin, q0, q1);
-            if (dev_wins) { add(B_TD, n, q0, q1); add(B_DW, 1ull, q0, q1); }
-            add(B_PS, l, q0, q1);
-            if (started) { add(B_PD, l, q0, q1); add(B_RACE, 1ull, q0, q1); }
-            add(B_TAU, n - 1u, q0, q1); add(B_TT, tt, q0, q1);
-            if (!started || (dev_wins ? 2 : 1) != c.cand) return;
-            const int stall = bin_of_ticks(hand.y);
+__device__ __forceinline__ Request request_of(const Ctx& c, const float* th, const uint4& q, const uint2& hand, float& saving) {
+    Request r;
+    r.S = q.x; r.l = q.y & 0xFFFFu; r.n = q.y >> 16; r.m = hand.x & 0xFFFFu; r.dly = hand.x >> 16;
+    r.Td = c.kappa * r.l + c.c0;
+    r.stall = bin_of_ticks(hand.y);
+    saving = r.m ? c.delta_c * (float)(c.E0 ? max(c.E0 - (int)r.m, 0) : (int)(r.n - r.m)) : -1.0f;
+    r.level = 0;
 #pragma unroll
-            for (int r = 0; r < NT; ++r) {
-                if (!(saving > th[r])) break;                                          // (overheads ascend)
-                const int f = kBase + r * kLev;
-                add(f + V_A, n - m, q0, q1); add(f + V_B, l + m, q0, q1); add(f + V_N, 1ull, q0, q1);
-                if (dly) add(f + V_C, dly, q0, q1);
-                if (DBG_OK(stall, kNBins, DBG_K_GRID, DBG_BIN)) count(tb.tbt + (size_t)r * K * kNBins + stall, q0, q1);
-            }
-        };
-        // the columns on either side of the request's length
-        int k1 = 0, k2;
-        for (int hi = K; k1 < hi;) { const int mid = (k1 + hi) >> 1; if (waits ? sm.key[mid] < (int)l : sm.key[mid] > (int)l) k1 = mid + 1; else hi = mid; }
-        k2 = k1;
-        if (waits) {
-            while (k2 < K && sm.key[k2] == (int)l) { enter_run(sm.w_star[k2], k2, k2 + 1); ++k2; }
-            const int low = S > wt_min ? min(n_low, k1) : 0;
-            for (int p = 0; p < low; ++p) enter_run(sm.w_tail[p], p, p + 1);
-            if (low < k1) enter_run(wt_min, low, k1);
-        } else if (k1 > 0) {                                                           // the device alone
-            const int bin = bin_of_ticks(Td);
-            if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) count(tb.ttft + bin, 0, k1);
-            add(B_DO, 1ull, 0, k1); add(B_TD, n, 0, k1); add(B_PD, l, 0, k1); add(B_TAU, n - 1u, 0, k1); add(B_TT, Td, 0, k1);
+    for (int k = 0; k < NT; ++k) r.level += saving > th[k] ? 1 : 0;
+    return r;
+}
+// What a request comes to under the columns [q0, q1), which start the device after w, entered by its lane alone.
+__device__ __forceinline__ void enter_run(const Adder& t, const Tables<false>& tb, const Request& r, int cand, uint32_t w, int q0, int q1) {
+    const bool started = r.S > w, dev_wins = r.S > w + r.Td;
+    const uint32_t tt = min(r.S, w + r.Td);
+    const int bin = bin_of_ticks(tt);
+    if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) t.count(tb.ttft + bin, q0, q1, 1u);
+    if (dev_wins) { t.add(B_TD, r.n, q0, q1); t.add(B_DW, 1ull, q0, q1); }
+    t.add(B_PS, r.l, q0, q1);
+    if (started) { t.add(B_PD, r.l, q0, q1); t.add(B_RACE, 1ull, q0, q1); }
+    t.add(B_TAU, r.n - 1u, q0, q1); t.add(B_TT, tt, q0, q1);
+    if (!started || (dev_wins ? 2 : 1) != cand) return;
+#pragma unroll 1
+    for (int k = 0; k < r.level; ++k) {
+        const int f = kBase + k * kLev;
+        t.add(f + V_A, r.n - r.m, q0, q1); t.add(f + V_B, r.l + r.m, q0, q1); t.add(f + V_N, 1ull, q0, q1);
+        if (r.dly) t.add(f + V_C, r.dly, q0, q1);
+        if (DBG_OK(r.stall, kNBins, DBG_K_GRID, DBG_BIN)) t.count(tb.tbt + (size_t)k * t.K * kNBins + r.stall, q0, q1, 1u);
+    }
+}
+// What the requests of the lanes `mine` come to under the columns [q0, q1), which start the device after w, together: the sums are added
+// up over the lanes and entered once, a lane a field.  alone: the device alone answers.
+template <int NT>
+__device__ __forceinline__ void join_run(const Adder& t, const Tables<false>& tb, const Request& r, int cand, bool mine, bool alone, uint32_t w, int q0, int q1) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t all = __ballot_sync(FULL, mine);
+    if (!all) return;
+    const bool started = mine && !alone && r.S > w, dev_wins = mine && (alone || r.S > w + r.Td);
+    const uint32_t tt = alone ? r.Td : min(r.S, w + r.Td);
+    const int bin = bin_of_ticks(tt), first = __shfl_sync(FULL, bin, __ffs(all) - 1);
+    const uint32_t like = __ballot_sync(FULL, mine && bin == first);     // (one prompt length, one TTFT of the device)
+    if (mine && (bin != first || lane == __ffs(all) - 1) && DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN))
+        t.count(tb.ttft + bin, q0, q1, bin == first ? (uint32_t)__popc(like) : 1u);
+    uint32_t lo = 0, hi = 0;
+    auto put = [&](int f, uint32_t v) { if (f < 32) { if (lane == f) lo = v; } else if (lane == f - 32) hi = v; };
+    const uint32_t sum_l = __reduce_add_sync(FULL, mine ? r.l : 0u);
+    put(B_TD, __reduce_add_sync(FULL, dev_wins ? r.n : 0u));
+    put(B_TAU, __reduce_add_sync(FULL, mine ? r.n - 1u : 0u));
+    if (alone) { put(B_PD, sum_l); put(B_DO, (uint32_t)__popc(all)); }
+    else {
+        put(B_PS, sum_l);
+        put(B_PD, __reduce_add_sync(FULL, started ? r.l : 0u));
+        put(B_RACE, (uint32_t)__popc(__ballot_sync(FULL, started)));
+        put(B_DW, (uint32_t)__popc(__ballot_sync(FULL, dev_wins)));
+    }
+    const unsigned long long tt_sum = __reduce_add_sync(FULL, mine ? tt & 0xFFFFu : 0u) + ((unsigned long long)__reduce_add_sync(FULL, mine ? tt >> 16 : 0u) << 16);
+    const int level = started && (dev_wins ? 2 : 1) == cand ? r.level : 0;
+    const uint32_t movers = __ballot_sync(FULL, level > 0);
+    const int leader = movers ? __ffs(movers) - 1 : 0, stall_0 = __shfl_sync(FULL, r.stall, leader);     // (mostly tau, where none stalls)
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+        const uint32_t go = __ballot_sync(FULL, level > k), alike = __ballot_sync(FULL, level > k && r.stall == stall_0);
+        if (!go) break;
+        const int f = kBase + k * kLev;
+        put(f + V_A, __reduce_add_sync(FULL, level > k ? r.n - r.m : 0u)); put(f + V_B, __reduce_add_sync(FULL, level > k ? r.l + r.m : 0u));
+        put(f + V_C, __reduce_add_sync(FULL, level > k ? r.dly : 0u)); put(f + V_N, (uint32_t)__popc(go));
+        const bool by_one = alike != 0u && lane == __ffs(alike) - 1;
+        if (level > k && (r.stall != stall_0 || by_one) && DBG_OK(r.stall, kNBins, DBG_K_GRID, DBG_BIN))
+            t.count(tb.tbt + (size_t)k * t.K * kNBins + r.stall, q0, q1, by_one ? (uint32_t)__popc(alike) : 1u);
+    }
+    const unsigned long long x = lane == B_TT ? tt_sum : lo;
+    if (x) t.add(lane, x, q0, q1);
+    if (NT * kLev + kBase > 32 && hi) t.add(lane + 32, hi, q0, q1);
+}
+
+// The requests [from, to) of the block's list, a segment's, for the columns [0, k1).
+// A warp a wait: the common one, and those of the columns that wait longer.
+template <int NT>
+__device__ __noinline__ void enter_listed(const Args& a, const Smem& sm, uint32_t from, uint32_t to, uint32_t wt_min, int n_low, int k1) {
+    const Ctx& c = sm.ctx;
+    const Tables<false> tb(a.gt, a.slabs[sm.slab], a.tr.n_groups);
+    const Adder t = {tb.sum_row(c.g, 0), (size_t)sum_fields(c.T), c.K};
+    const int lane = threadIdx.x & 31;
+    for (int p = threadIdx.x >> 5; p <= n_low; p += kThreads / 32) {
+        const uint32_t w = p < n_low ? sm.w_tail[p] : wt_min;
+        const int q1 = p < n_low ? p + 1 : k1;
+        if (p >= q1) continue;                                         // (every column waits longer)
+#pragma unroll 1
+        for (uint32_t i0 = from; i0 < to; i0 += 32) {
+            const uint32_t i = min(i0 + lane, to - 1), kk = c.start + sm.list[i];
+            if (!DBG_OK(kk, a.tr.n, DBG_K_GRID, DBG_REQUEST)) break;
+            float saving;
+            const Request r = request_of<NT>(c, sm.rows, a.tr.req[kk], c.may_migrate ? c.hand[kk] : make_uint2(0u, 0u), saving);
+            join_run<NT>(t, tb, r, c.cand, i0 + lane < to, false, w, p, q1);
         }
-        if (k2 < K) enter_run(0u, k2, K);
     }
 }
 
-template <int NT, bool WIDE>
-__global__ void __launch_bounds__(kThreads, blocks_for(NT, WIDE))
+template <int NT>
+__device__ __forceinline__ void enter_requests(const Args& a, const Ctx& c, const float (&th)[NT], const Smem& sm, const Tables<false>& tb,
+                                               bool waits, uint32_t wt_min, int n_low) {
+    const int K = c.K, lane = threadIdx.x & 31;
+    const Adder t_ = {tb.sum_row(c.g, 0), (size_t)sum_fields(c.T), K};
+#pragma unroll 1
+    for (uint32_t i0 = threadIdx.x & ~31u; i0 < c.len; i0 += kThreads) {
+        const uint32_t kk = c.start + min(i0 + lane, c.len - 1);
+        float saving;
+        const Request r = request_of<NT>(c, th, a.tr.req[kk], c.may_migrate ? c.hand[kk] : make_uint2(0u, 0u), saving);
+        const uint32_t S = r.S, l = r.l, n = r.n, Td = r.Td;
+        const bool valid = i0 + lane < c.len && !(c.mixed && saving > c.th_lo && !(saving > th[0]));       // (else left to the pair kernel)
+        // the columns on either side of the request's length
+        int k1 = 0;
+        for (int hi = K; k1 < hi;) { const int mid = (k1 + hi) >> 1; if (waits ? sm.key[mid] < (int)l : sm.key[mid] > (int)l) k1 = mid + 1; else hi = mid; }
+        int k2 = k1;
+        if (waits) while (k2 < K && sm.key[k2] == (int)l) ++k2;
+        const bool longer = waits && valid && S > wt_min && n_low > 0;         // (not covered by the common wait)
+        bool joined = false;
+        uint32_t todo = __ballot_sync(FULL, valid);
+#pragma unroll 1
+        while (todo) {
+            const int lead = __ffs(todo) - 1, a1 = __shfl_sync(FULL, k1, lead), a2 = __shfl_sync(FULL, k2, lead);
+            const uint32_t same = __ballot_sync(FULL, valid && k1 == a1 && k2 == a2);
+            todo &= ~same;
+            if (__popc(same) < kJoin) continue;
+            const bool mine = (same >> lane) & 1u;
+            joined = joined || mine;
+            if (waits) {
+#pragma unroll 1
+                for (int p = a1; p < a2; ++p) join_run<NT>(t_, tb, r, c.cand, mine, false, sm.w_star[p], p, p + 1);
+            }
+            if (a1 > 0) join_run<NT>(t_, tb, r, c.cand, mine && !longer, !waits, waits ? wt_min : 0u, 0, a1);
+            if (a1 > n_low) join_run<NT>(t_, tb, r, c.cand, mine && longer, false, wt_min, n_low, a1);
+            if (a2 < K) join_run<NT>(t_, tb, r, c.cand, mine, false, 0u, a2, K);
+        }
+        // (the columns that wait longer have l* = 0: they are in front of every request's k1)
+        if (__any_sync(FULL, longer)) {
+#pragma unroll 1
+            for (int p = 0; p < n_low; ++p) join_run<NT>(t_, tb, r, c.cand, longer, false, sm.w_tail[p], p, p + 1);
+        }
+        if (valid && !joined) {
+            const int low = longer ? n_low : 0;
+            for (int p = k1; p < k2; ++p) enter_run(t_, tb, r, c.cand, sm.w_star[p], p, p + 1);
+            if (k2 < K) enter_run(t_, tb, r, c.cand, 0u, k2, K);
+            if (waits) {
+                if (low < k1) enter_run(t_, tb, r, c.cand, wt_min, low, k1);
+            } else if (k1 > 0) {                                           // the device alone
+                const int bin = bin_of_ticks(Td);
+                if (DBG_OK(bin, kNBins, DBG_K_GRID, DBG_BIN)) t_.count(tb.ttft + bin, 0, k1, 1u);
+                t_.add(B_DO, 1ull, 0, k1); t_.add(B_TD, n, 0, k1); t_.add(B_PD, l, 0, k1); t_.add(B_TAU, n - 1u, 0, k1); t_.add(B_TT, Td, 0, k1);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// MODE: run by run, where no group of the slabs is Algorithm 2's, or where some are (kernels of their own: the second has no registers
+// to spare); or a chunk's requests side by side.
+template <int NT, bool WIDE, int MODE>
+__global__ void __launch_bounds__(kThreads, blocks_for(NT, WIDE, MODE))
 k_grid(const __grid_constant__ Args a) {
+    constexpr bool WAITS = MODE != M_RACES, JOINED = MODE == M_JOINED;
+    static_assert(!(WIDE && JOINED), "windows are added up by runs");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
     uint32_t* tbt = (uint32_t*)(smem_raw + sizeof(Smem));
+    const Levels<NT> lv(tbt + NT * kNBins + (has_levels(NT, WIDE) ? (threadIdx.x >> 5) * Levels<NT>::kWords : 0));
     // Beside the slope search of Eq. 1-2 (k_prep_beta), which no plain policy needs: what this kernel reads was complete before that
     // one let it start.  It then waits at its end, for the kernels behind.  (Under 48 such searches, 79 us on 48
     // multiprocessors, 300,000 requests by 16 budgets take 27.)
     for (int i = threadIdx.x; i < (int)(offsetof(Smem, key) / 4); i += kThreads) ((uint32_t*)&sm)[i] = 0;
-    for (int i = threadIdx.x; i < (NT + (WIDE ? 1 : 0)) * kNBins; i += kThreads) tbt[i] = 0;
+    if (!JOINED) for (int i = threadIdx.x; i < tbt_words(NT, WIDE); i += kThreads) tbt[i] = 0;
     if (!a.beside) grid_dependency_wait();
 
     int turn = 0;                                                     // which of the two sets of used bins is in use
-    const uint32_t direct = a.n_chunks * a.n_slabs <= gridDim.x ? kDirectAlone : kDirectMany;
     // A block starts with a (chunk, slab) item of its own and then draws the next ones from a counter (zero at launch): items
     // differ in cost.  (Drawn ahead, when the one in front begins, they are no longer dealt to who is free: 16 M requests by
     // 128 and 8 policies 348 -> 385 us.  Beside another kernel not all blocks are there at once: all items are drawn.)
@@ -566,10 +764,15 @@ k_grid(const __grid_constant__ Args a) {
 #pragma unroll
         for (int r = 0; r < NT; ++r) th[r] = (c.may_migrate && r < c.T) ? sl.theta[sl.mixed ? 1 : r] : __int_as_float(0x7F800000);
         c.th_lo = sl.theta[0];
+        if (!WIDE && MODE == M_WAITS && list_few(NT) != 0 && threadIdx.x == 0) {
+            sm.ctx = c; sm.slab = slab_id;
+#pragma unroll
+            for (int r = 0; r < NT; ++r) sm.rows[r] = th[r];
+        }
         bool waits = false;
         {
             const Prep& pr = a.prep[(size_t)g * a.P + a.tab[sl.cols]];
-            waits = pr.device_constrained != 0;
+            waits = WAITS && pr.device_constrained != 0;
         }
         for (int p = threadIdx.x; p < c.K; p += kThreads) {
             if (!DBG_OK(a.tab[sl.cols + p], a.P, DBG_K_GRID, DBG_POLICY)) continue;
@@ -602,7 +805,7 @@ k_grid(const __grid_constant__ Args a) {
         // ---- the segments: stretches of prompt lengths between two thresholds and (Algorithm 2) the thresholds
         //      themselves; a thread per candidate looks up where its lengths lie in the chunk
         const int K = c.K;
-        for (int q = threadIdx.x; q < (waits ? 2 * K + 1 : K + 1); q += kThreads) {
+        for (int q = threadIdx.x; !JOINED && q < (waits ? 2 * K + 1 : K + 1); q += kThreads) {
             auto cl = [](int x) { return min(max(x, 0), kMaxPrompt + 1); };
             int la, lb, k1, k2;
             bool any = true;
@@ -628,7 +831,6 @@ k_grid(const __grid_constant__ Args a) {
                 const uint32_t pa = min(max(at_a, lo), hi) - lo, pb = min(max(at_b, lo), hi) - lo;
                 if (pa < pb) {
                     const uint32_t at = atomicAdd(&sm.n_seg, 1u);
-                    atomicAdd(&sm.n_runs, waits ? (uint32_t)(k2 - k1) + (k1 > 0) + (k2 < K) : 1u);
                     if (DBG_OK(at, kMaxSeg, DBG_K_GRID, DBG_SLOT))
                         sm.seg[at] = Seg{(uint16_t)pa, (uint16_t)pb, (uint16_t)k1, (uint16_t)k2};
                 }
@@ -644,79 +846,120 @@ k_grid(const __grid_constant__ Args a) {
         const int n_seg = (int)min(sm.n_seg, (uint32_t)kMaxSeg);
         uint32_t passes = 0;
 
-        // one run: sweep and enter; `list` and `push` as in sweep
-        auto run = [&](uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, int q0, int q1, bool neg) {
-            Acc<NT> s = {};
-            Only none = {};
-            sweep<NT, WIDE, false>(a, c, th, sm, tbt, pa, pb, w, list, push, true, false, s, none);
-            share_out<NT, WIDE>(sm, s, turn);
-            __syncthreads();
-            enter<NT, WIDE>(sm, tbt, tb, g, q0, q1, neg, turn);
-            __syncthreads();
-            ++passes; turn ^= 1;
-        };
-        bool by_request = false;
-        if constexpr (!WIDE) {
-            by_request = c.len < (sm.n_runs + (n_low ? (uint32_t)n_low + 1u : 0u)) * direct;
-            if (by_request) {
-                const Ctx its = c;                                    // (copies: what is handed over by address lives in memory)
-                const Tables<false> tables = tb;
-                float rows[NT];
-#pragma unroll
-                for (int r = 0; r < NT; ++r) rows[r] = th[r];
-                enter_requests<NT>(a, its, rows, sm, tables, waits, wt_min, n_low);
-                passes = 1;
-            }
+        if constexpr (JOINED) {
+            enter_requests<NT>(a, c, th, sm, tb, waits, wt_min, n_low);
+            passes = 1;
         }
-        if (by_request) {
-        } else if (!waits) {
+        // a segment's last columns, which wait 0, and beside them its first ones: the device alone
+        if constexpr (MODE == M_RACES) {
             for (int si = 0; si < n_seg; ++si) {
                 const Seg sg = sm.seg[si];
-                const bool race = (int)sg.k2 < K, only = sg.k1 > 0;
-                Acc<NT> s = {};
-                Only o = {};
-                sweep<NT, WIDE, true>(a, c, th, sm, tbt, sg.pa, sg.pb, 0u, false, false, race, only, s, o);
-                if (race) share_out<NT, WIDE>(sm, s, turn);
-                if (only) share_only(sm, o, turn);
+                const bool race = (int)sg.k2 < K, side = sg.k1 > 0;
+                Acc<NT, WIDE> s = {};
+                Side o = {};
+                sweep<NT, WIDE, S_DEVICE>(a, c, th, sm, tbt, lv, sg.pa, sg.pb, 0u, false, false, false, race, side, s, o);
+                if (race) share_out<NT, WIDE>(sm, s, lv, turn);
+                if (side) share_side<NT, WIDE>(sm, o, turn);
                 __syncthreads();
                 if (race) enter<NT, WIDE>(sm, tbt, tb, g, sg.k2, K, false, turn);
-                if (only) enter_only<WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1, turn);
+                if (side) enter_side<NT, WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1, false, turn);
                 __syncthreads();
                 ++passes; turn ^= 1;
             }
-        } else {
-            // segment by segment, run by run: [k2, K) waits 0, each column of [k1, k2) its own w*, [0, k1) w_tail -- and,
-            // when the list is full or the chunk is done, the list for the columns that wait longer
-            uint32_t pa = 0;                                          // (of the segment in work: where the sweep goes on)
-            int si = 0, ri = 0;
+        } else if constexpr (MODE == M_WAITS) {
+            // Segment by segment: each column of [k1, k2) under its own w*; then [k2, K), which waits 0, in one sweep with [0, k1), where the
+            // device runs alone or (Algorithm 2) waits w_tail.  The few requests that w_tail does not cover have been listed.  A handful is
+            // entered request by request; more are entered for [0, k1) from the list, and when it is half full or the chunk is done,
+            // the columns that wait longer get what they come to there under their own wait in place of the common one.
+            enum { POINTS, MAIN, ALONE, LISTED, LONGER } at = POINTS;
+            constexpr int kFirst = WIDE ? -1 : 0;                      // of the columns that wait longer (-1: the common wait's totals are taken back)
+            uint32_t pos = 0, listed = 0, n_list = 0;                  // where the segment's sweep goes on; the list: entered for [0, k1), all
+            int si = 0, ri = 0;                                       // segment, point or column
+#pragma unroll 1
             for (;;) {
                 uint32_t from = 0, to = 0, w = 0;
                 int q0 = 0, q1 = 0;
-                bool push = false;
-                const bool done = si >= n_seg;
-                if (!done) {
-                    const Seg sg = sm.seg[si];
-                    const int n_pts = (int)sg.k2 - (int)sg.k1;
-                    if (ri == 0) pa = sg.pa;
-                    if (ri == 0 && (int)sg.k2 >= K) { ++ri; continue; }
-                    if (ri > n_pts && sg.k1 == 0) { ri = 0; ++si; continue; }
-                    from = pa; to = sg.pb;
-                    if (ri == 0) { q0 = sg.k2; q1 = K; ++ri; }
-                    else if (ri <= n_pts) { q0 = (int)sg.k1 + ri - 1; q1 = q0 + 1; w = sm.w_star[q0]; ++ri; }
-                    else {
-                        w = wt_min; q1 = sg.k1; push = n_low > 0;
-                        if (push && to - from > (uint32_t)kListStep) { to = from + kListStep; pa = to; }
-                        else { ri = 0; ++si; }
+                bool neg = false, list = false, push = false;
+                if (at == POINTS) {
+                    if (si >= n_seg) {
+                        if (n_list == 0) break;
+                        at = LONGER; ri = kFirst;
+                        continue;
                     }
-                    run(from, to, w, false, push, q0, q1, false);
-                } else if (sm.n_list == 0) break;
-                if (done || (push && sm.n_list > (uint32_t)(kListCap - kListStep))) {
-                    const uint32_t k = sm.n_list;                     // (barriers inside run: all threads agree)
+                    const Seg sg = sm.seg[si];
+                    if (ri >= (int)sg.k2 - (int)sg.k1 || !waits) { at = MAIN; pos = sg.pa; continue; }
+                    from = sg.pa; to = sg.pb; q0 = (int)sg.k1 + ri; q1 = q0 + 1; w = sm.w_star[q0];
+                    ++ri;
+                } else if (at == MAIN) {
+                    const Seg sg = sm.seg[min(si, kMaxSeg - 1)];
+                    const bool race = (int)sg.k2 < K, side = sg.k1 > 0;
+                    if (pos >= sg.pb || !(race || side)) { at = POINTS; ri = 0; ++si; continue; }
+                    if (WIDE && waits) { at = ALONE; ri = race ? 0 : 1; continue; }
+                    Acc<NT, WIDE> s = {};
+                    Side o = {};
+                    for (;;) {
+                        uint32_t end = sg.pb;
+                        if (!WIDE && waits && side) end = min(end, pos + (uint32_t)kListCap - n_list);
+                        sweep<NT, WIDE, WIDE ? S_DEVICE : S_EITHER>(a, c, th, sm, tbt, lv, pos, end, wt_min, false, false, waits, race, side, s, o);
+                        pos = end;
+                        if (WIDE || !waits || !side) break;
+                        __syncthreads();
+                        n_list = sm.n_list;
+                        __syncthreads();
+                        if (pos >= sg.pb || n_list > (uint32_t)(kListCap - kThreads)) break;
+                    }
+                    if (race) share_out<NT, WIDE>(sm, s, lv, turn);
+                    if (side) share_side<NT, WIDE>(sm, o, turn);
+                    if constexpr (!WIDE && list_few(NT) != 0) {
+                        if (n_list > listed && n_list - listed <= (uint32_t)list_few(NT)) {
+                            enter_listed<NT>(a, sm, listed, n_list, wt_min, n_low, sg.k1);
+                            n_list = listed;
+                        }
+                    }
                     __syncthreads();
-                    if (threadIdx.x == 0) sm.n_list = 0;
-                    for (int p = -1; p < n_low; ++p)                  // the common wait's totals go, each column's own come
-                        run(0u, k, p < 0 ? wt_min : sm.w_tail[p], true, false, max(p, 0), p < 0 ? n_low : p + 1, p < 0);
+                    if (!WIDE && threadIdx.x == 0) sm.n_list = n_list;
+                    if (race) enter<NT, WIDE>(sm, tbt, tb, g, sg.k2, K, false, turn);
+                    if (side) enter_side<NT, WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1, waits, turn);
+                    __syncthreads();
+                    ++passes; turn ^= 1;
+                    if (!WIDE && n_list > listed) at = LISTED;
+                    continue;
+                } else if (WIDE && at == ALONE) {
+                    // (windows: the sweep for [k2, K), then those for [0, k1), whose requests that w_tail does not cover are listed for the
+                    // columns that wait longer)
+                    const Seg sg = sm.seg[si];
+                    if (ri == 0) { from = sg.pa; to = sg.pb; q0 = sg.k2; q1 = K; ri = 1; }
+                    else if (pos >= sg.pb || sg.k1 == 0) { pos = sg.pb; at = MAIN; continue; }
+                    else if (n_list > (uint32_t)kListCap / 2) { at = LONGER; ri = kFirst; continue; }
+                    else {
+                        push = n_low > 0;
+                        from = pos; to = push ? min((uint32_t)sg.pb, pos + (uint32_t)kListCap / 2) : sg.pb; w = wt_min; q1 = sg.k1;
+                        pos = to;
+                    }
+                } else if (!WIDE && at == LISTED) {
+                    const int k1 = sm.seg[si].k1;
+                    list = true; from = listed; to = n_list; w = wt_min; q0 = n_low; q1 = k1;
+                    listed = n_list;
+                    at = MAIN;
+                    if (n_low == 0) listed = n_list = 0;
+                    else if (n_list > (uint32_t)kListCap / 2) { at = LONGER; ri = kFirst; }
+                    if (q0 >= k1) continue;                            // (every column waits longer)
+                } else {
+                    list = true; to = n_list; neg = WIDE && ri < 0;
+                    w = neg ? wt_min : sm.w_tail[ri];
+                    q0 = neg ? 0 : ri; q1 = neg ? n_low : ri + 1;
+                    if (++ri == n_low) { listed = n_list = 0; at = si >= n_seg ? POINTS : WIDE ? ALONE : MAIN; }
                 }
+                Acc<NT, WIDE> s = {};
+                Side none = {};
+                sweep<NT, WIDE, S_NONE>(a, c, th, sm, tbt, lv, from, to, w, list, push, false, true, false, s, none);
+                share_out<NT, WIDE>(sm, s, lv, turn);
+                __syncthreads();
+                if (n_list == 0 && threadIdx.x == 0 && !push) sm.n_list = 0;
+                if (WIDE && push) n_list = sm.n_list;
+                enter<NT, WIDE>(sm, tbt, tb, g, q0, q1, neg, turn);
+                __syncthreads();
+                ++passes; turn ^= 1;
             }
         }
         if (threadIdx.x == 0 && a.work) {
@@ -728,7 +971,7 @@ k_grid(const __grid_constant__ Args a) {
         if (n_items <= dealt) break;
         __syncthreads();
         if (threadIdx.x == 0) {
-            sm.n_seg = 0; sm.n_runs = 0; sm.n_list = 0; sm.flagged = 0;
+            sm.n_seg = 0; sm.n_list = 0; sm.flagged = 0;
             sm.ticket = dealt + atomicAdd(a.ticket, 1u);
         }
         __syncthreads();
@@ -843,41 +1086,54 @@ k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict
     });
 }
 
-size_t grid_smem(int NT, bool wide) { return sizeof(Smem) + (size_t)(NT + (wide ? 1 : 0)) * kNBins * 4; }
+size_t grid_smem(int NT, bool wide) { return sizeof(Smem) + (size_t)tbt_words(NT, wide) * 4; }
 
-template <int NT, bool WIDE>
+template <int NT, bool WIDE, int MODE>
 cudaError_t launch_one(const Args& a, int sms, cudaStream_t st) {
-    const size_t smem = grid_smem(NT, WIDE);
-    cudaError_t e = allow_smem((const void*)k_grid<NT, WIDE>, smem);
+    const size_t smem = MODE == M_JOINED ? sizeof(Smem) : grid_smem(NT, WIDE);
+    auto* kernel = k_grid<NT, WIDE, MODE>;
+    cudaError_t e = allow_smem((const void*)kernel, smem);
     if (e) return e;
     const uint64_t items = (uint64_t)a.n_chunks * a.n_slabs;
-    const uint32_t blocks = (uint32_t)std::min<uint64_t>(items, (uint64_t)sms * blocks_for(NT, WIDE));
-    return launch_after(k_grid<NT, WIDE>, dim3(blocks), kThreads, smem, st, a);
+    const uint32_t blocks = (uint32_t)std::min<uint64_t>(items, (uint64_t)sms * blocks_for(NT, WIDE, MODE));
+    return launch_after(kernel, dim3(blocks), kThreads, smem, st, a);
+}
+template <int NT>
+cudaError_t launch_rows(const Args& a, bool wide, int mode, int sms, cudaStream_t st) {
+    if (wide) return mode == M_RACES ? launch_one<NT, true, M_RACES>(a, sms, st) : launch_one<NT, true, M_WAITS>(a, sms, st);
+    return mode == M_RACES ? launch_one<NT, false, M_RACES>(a, sms, st) : mode == M_WAITS ? launch_one<NT, false, M_WAITS>(a, sms, st)
+                                                                                         : launch_one<NT, false, M_JOINED>(a, sms, st);
 }
 
 }  // namespace
 
 DBG_TRANSLATION_UNIT()
 
+// Side by side or run by run: the first takes some 0.1 us for a thousand requests, the second a run's latency for every threshold of every
+// group.  (us, run by run and side by side: one group, 150,000 requests under 64 10 and 11, 256 by 4 24 and 15, 400,000 21 and 25 under 256;
+// six groups, 60,000 under one 12 and 9, 150,000 under 16 by 2 23 and 20, under 64 45 and 22, 400,000 42 and 43, under 64 by 4 59 and 46,
+// a million under 256 125 and 117, under 128 by 8 116 and 126.)
+bool grid_joins(uint32_t n, int groups, int K, int T) { return n <= (80000.0 + 650.0 * K * groups) * (1.0 + T / 16.0); }
 uint64_t grid_ttft_words(int K) { return (uint64_t)K * kNBins; }
 uint64_t grid_tbt_words(int K, int T) { return (uint64_t)K * T * kNBins; }
 uint64_t grid_sum_words(int K, int T, int G) { return (uint64_t)G * K * sum_fields(T); }
-uint32_t grid_blocks_per_sm(int T) { return (uint32_t)blocks_for(rows_for(T), false); }
+uint32_t grid_blocks_per_sm(int T) { return (uint32_t)blocks_for(rows_for(T), false, M_WAITS); }
 int grid_rows(int T) { return rows_for(T); }
 
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* classes, const Prep* prep, uint32_t P,
                         const Slab* slabs, uint32_t n_slabs, int T, bool wide, const uint32_t* tab,
                         const Chunk* chunks, uint32_t n_chunks, TimelineRec rec, size_t rec_stride, GridTables gt, LeftLists left,
-                        uint32_t k0, uint32_t* ticket, uint64_t* work, bool beside, int sms, cudaStream_t st) {
+                        uint32_t k0, uint32_t* ticket, uint64_t* work, bool beside, bool waits, bool joined, int sms, cudaStream_t st) {
     if (n_chunks == 0 || n_slabs == 0) return cudaSuccess;
     if ((uint64_t)n_chunks * n_slabs > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
     const Args a = {tr, rec, gc, rec_stride, classes, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, k0, ticket,
                     (unsigned long long*)work, beside};
+    const int mode = joined && !wide ? M_JOINED : waits ? M_WAITS : M_RACES;
     switch (rows_for(T)) {
-        case 1: return wide ? launch_one<1, true>(a, sms, st) : launch_one<1, false>(a, sms, st);
-        case 2: return wide ? launch_one<2, true>(a, sms, st) : launch_one<2, false>(a, sms, st);
-        case 4: return wide ? launch_one<4, true>(a, sms, st) : launch_one<4, false>(a, sms, st);
-        default: return wide ? launch_one<8, true>(a, sms, st) : launch_one<8, false>(a, sms, st);
+        case 1: return launch_rows<1>(a, wide, mode, sms, st);
+        case 2: return launch_rows<2>(a, wide, mode, sms, st);
+        case 4: return launch_rows<4>(a, wide, mode, sms, st);
+        default: return launch_rows<8>(a, wide, mode, sms, st);
     }
 }
 

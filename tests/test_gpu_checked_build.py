@@ -30,6 +30,14 @@ def test_parity_cases_pass_with_every_index_checked():
     assert " passed" in r.stdout and "failed" not in r.stdout
 
 
+def test_small_traces_run_by_run():
+    # the grid kernels of large traces, which small ones do not reach: the same cases, and those made for runs, against the oracle
+    r = _run(["-m", "pytest", "tests/test_gpu_parity.py", "tests/test_gpu_variants.py", "-x", "-q", "-m", "gpu", "-k",
+              CASES + " or few_requests or eight_overheads or several_overheads or reduced_together or beside_the_slope or many_kinds"], DISCO_DEBUG_RUNS="1")
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
+    assert " passed" in r.stdout and "failed" not in r.stdout
+
+
 def test_the_checks_are_live():
     code = (
         "import ctypes\n"
