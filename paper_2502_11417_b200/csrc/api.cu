@@ -952,7 +952,19 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const size_t o_prep = lay.take((size_t)G * P * sizeof(Prep)), o_stats = lay.take(P * sizeof(disco_policy_stats_t) + 16);
     const size_t o_accum2 = clear_accum ? o_accum : lay.take(acc_bytes + 2 * hist_bytes);
     const size_t o_left = lay.take(any_mixed ? (N1 + kMaxGroups) * 4 : 0);
-    const size_t table_bytes = ((size_t)P * sizeof(PolicyConst) + 15) / 16 * 16 + (classes.size() * sizeof(ClassConst) + 15) / 16 * 16 +
+    std::vector<PolicyIn> policies_in(P);
+    std::vector<PolicyKind> kinds;
+    for (uint32_t p = 0, k = 0; p < P; ++p) {
+        const PolicyConst& q = pc[p];
+        auto like = [&](const PolicyKind& x) { return x.alpha == q.alpha && x.flags == q.flags && x.mode == q.mode && x.expected_len == q.expected_len && x.l_immediate == q.l_immediate; };
+        if (k >= kinds.size() || !like(kinds[k])) {                  // (mostly that of the policy before; else one of the last few, or another)
+            const size_t from = kinds.size() > 16 ? kinds.size() - 16 : 0;
+            for (k = (uint32_t)from; k < kinds.size() && !like(kinds[k]);) ++k;
+            if (k == kinds.size()) kinds.push_back(PolicyKind{q.alpha, q.flags, q.mode, q.expected_len, q.l_immediate, {0, 0, 0}});
+        }
+        policies_in[p] = PolicyIn{q.budget, q.theta, k, q.route_thr};
+    }
+    const size_t table_bytes = (size_t)P * sizeof(PolicyIn) + kinds.size() * sizeof(PolicyKind) + (classes.size() * sizeof(ClassConst) + 15) / 16 * 16 +
                                (tab.size() * 4 + 15) / 16 * 16 + (slabs.size() * sizeof(Slab) + 15) / 16 * 16;
     const size_t o_tables = lay.take(table_bytes);
     const size_t o_chunks[2] = {lay.take(tables.n_chunks[0] * sizeof(Chunk)), lay.take(tables.n_chunks[1] * sizeof(Chunk))};
@@ -991,7 +1003,9 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         off += (bytes + 15) / 16 * 16;
         return at;
     };
-    const PolicyConst* d_pol = (const PolicyConst*)put(pc.data(), P * sizeof(PolicyConst));
+    const PolicyIn* d_pol = (const PolicyIn*)put(policies_in.data(), P * sizeof(PolicyIn));
+    const PolicyKind* d_kinds = (const PolicyKind*)put(kinds.data(), kinds.size() * sizeof(PolicyKind));
+    const uint32_t policy_vecs = (uint32_t)(off / 16);
     const ClassConst* d_classes = (const ClassConst*)put(classes.data(), classes.size() * sizeof(ClassConst));
     const uint32_t* d_tab = (const uint32_t*)put(tab.data(), tab.size() * 4);
     const Slab* d_slabs = (const Slab*)put(slabs.data(), slabs.size() * sizeof(Slab));
@@ -999,7 +1013,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     if (off / 16 > 0xFFFFFFFFull) return fail(DISCO_ENOMEM, "the tables of the policies are too large");
 
     // ---- Algorithms 1-3 for every (group, policy)
-    tables.host = sp; tables.device = dt; tables.vecs = (uint32_t)(off / 16); tables.skip = n_beta ? 0u : (uint32_t)(P * sizeof(PolicyConst) / 16);
+    tables.host = sp; tables.device = dt; tables.vecs = (uint32_t)(off / 16); tables.skip = n_beta ? 0u : policy_vecs;
+    tables.kinds = (uint32_t)kinds.size();
     for (int k = 0; k < 2; ++k) tables.chunks[k] = (Chunk*)(mem + o_chunks[k]);
     tables.left = &c->z->tables_left; tables.read = c->stage_read; tables.turn = c->stage_turn + 1;
     CU(launch_prep(P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
@@ -1009,7 +1024,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     // (one class, played out already, and a grid: the search's results are not needed before the pair kernel)
     const bool beside = n_beta && n_classes == 1 && n != 0 && !timed && !batches.empty() && !slabs[0].mixed;
     if (n_beta) {
-        CU(launch_prep_beta(d_pol, P, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
+        CU(launch_prep_beta(d_pol, d_kinds, P, c->cum_mass.as<int64_t>(), c->cnt, c->F_sorted,
                             c->F_off, c->tick_start.as<uint32_t>(), c->tick_cnt, d_tab + beta_at, n_beta,
                             *std::max_element(c->F_n.begin(), c->F_n.end()), c->d_prep.as<Prep>(), beside, st));
         g_launches += 1;

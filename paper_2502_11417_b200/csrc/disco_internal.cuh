@@ -40,6 +40,16 @@ struct PolicyConst {
     uint32_t l_immediate;        // Eq. 1's immediate-start threshold (beta rule)
 };
 
+// ---- the same for the preparation: what differs from policy to policy, and the rest, which most of them share (a thousand
+//      policies then go with a launch, 28 KB at most, that took 57 KB) ----
+struct PolicyIn { float budget, theta; uint32_t kind, route_thr; };
+struct PolicyKind {
+    float alpha;
+    uint32_t flags;
+    int32_t mode;
+    uint32_t expected_len, l_immediate, pad[3];
+};
+
 // ---- what Algorithms 1-3 produce for one (group, policy) ----
 struct Prep {
     int32_t device_constrained;
@@ -246,9 +256,10 @@ struct DbgRegistrar { explicit DbgRegistrar(cudaError_t (*r)(int32_t*)) { dbg_re
 constexpr size_t kTablesInline = 28672;      // (a launch takes 32,764 bytes of parameters, the chunk plans 2,048)
 struct ChunkPlan { uint32_t first, start, end; int32_t g; };     // a group's chunks: number of the first, requests [start, end)
 struct TablesIn {
-    const void* host;            // the policies come first; room for kTablesInline bytes where they go as a parameter
+    const void* host;            // the policies come first, then their kinds; room for kTablesInline bytes where they go as a parameter
     void* device;
-    uint32_t vecs, skip;         // of 16 bytes; how many of them (policies) no kernel behind needs
+    uint32_t vecs, skip;         // of 16 bytes; how many of them (policies and kinds) no kernel behind needs
+    uint32_t kinds;
     // chunk tables that k_prep writes out, of the grid kernel and of the pair kernel, group by group
     ChunkPlan plan[2][kMaxGroups];
     uint32_t n_plan[2], chunk_len[2], n_chunks[2];
@@ -261,7 +272,7 @@ struct TablesIn {
 cudaError_t launch_prep(uint32_t P, int G, const GroupConst* gc, const int64_t* cum_mass,
                         const uint32_t* cnt, const int32_t* sorted, const uint32_t* grp_off, Prep* prep, const TablesIn& tables,
                         void* clear, size_t clear_bytes /* a multiple of 16: set to zero on the way */, int sms, cudaStream_t st);
-cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
+cudaError_t launch_prep_beta(const PolicyIn* pol, const PolicyKind* kinds, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off,
                              const uint32_t* tick_start, const uint32_t* tick_cnt /* [G][kTickBins], of the sorted ticks */,
                              const uint32_t* pairs /* [n_pairs]: g P + p */, uint32_t n_pairs,

@@ -54,7 +54,7 @@ __device__ __forceinline__ int first_true(int lo, int hi, F pred) {
 // wait for what came before -- and waits for it at its end, on behalf of the kernels behind both.
 constexpr int kPrepThreads = 128, kPrepWarps = kPrepThreads / 32;
 
-__device__ __forceinline__ void prep_pair(const PolicyConst& pc, uint32_t p, int g, uint32_t P, const GroupConst* __restrict__ gc,
+__device__ __forceinline__ void prep_pair(const PolicyIn& pi, const PolicyKind& pc, uint32_t p, int g, uint32_t P, const GroupConst* __restrict__ gc,
                                           const int64_t* __restrict__ cum_mass, const uint32_t* __restrict__ cnt,
                                           const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
                                           Prep* __restrict__ prep) {
@@ -62,16 +62,16 @@ __device__ __forceinline__ void prep_pair(const PolicyConst& pc, uint32_t p, int
     const uint32_t* c = cnt + (size_t)g * (kMaxPrompt + 1);
     const uint32_t off = grp_off[g], N = grp_off[g + 1] - off;
     const int32_t* srt = sorted + off;
-    const double b = (double)pc.budget, alpha = (double)pc.alpha;
+    const double b = (double)pi.budget, alpha = (double)pc.alpha;
     const double Total = (double)cum[kMaxPrompt + 1];
 
     Prep r;
     r.device_constrained = pc.mode == 1 ? 1 : pc.mode == 2 ? 0 : gc[g].auto_device_constrained;
     r.l_th = 0; r.l_star = 0; r.w_star = 0; r.w_tail = 0;
-    r.theta = pc.theta;
+    r.theta = pi.theta;
     r.mig_on = (pc.flags & DISCO_FLAG_MIGRATION) ? 1 : 0;
     r.stochastic = (pc.flags & DISCO_FLAG_STOCHASTIC) ? 1 : 0;
-    r.expected_len = pc.expected_len; r.route_thr = pc.route_thr; r.route_all = pc.route_all;
+    r.expected_len = pc.expected_len; r.route_thr = pi.route_thr; r.route_all = pi.budget >= 1.0f ? 1 : 0;
     r.beta_rule = 0;
 
     if (!r.device_constrained) {
@@ -115,9 +115,9 @@ k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __re
        const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
        Prep* __restrict__ prep, const __grid_constant__ TablesIn in, uint4* __restrict__ clear, uint32_t clear_vecs,
        const __grid_constant__ Inline<BYTES> given) {
-    constexpr uint32_t kVecs = sizeof(PolicyConst) / 16;
-    static_assert(sizeof(PolicyConst) % 16 == 0 && kPrepWarps * kVecs <= kPrepThreads, "a vector a thread");
-    __shared__ uint4 s_pol[kPrepWarps * kVecs];
+    constexpr uint32_t kVecs = sizeof(PolicyIn) / 16, kKindVecs = sizeof(PolicyKind) / 16, kNear = kPrepThreads / kKindVecs;
+    static_assert(sizeof(PolicyIn) % 16 == 0 && sizeof(PolicyKind) % 16 == 0 && kPrepWarps * kVecs <= kPrepThreads, "a vector a thread");
+    __shared__ uint4 s_pol[kPrepWarps * kVecs], s_kind[kPrepThreads];     // the block's policies, and the first kinds
     auto table = [&](uint32_t i) {
         if constexpr (BYTES != 0) return given.v[i];
         else return static_cast<const uint4*>(in.host)[i];
@@ -126,12 +126,15 @@ k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __re
     const uint32_t pairs = P * (uint32_t)G, first = blockIdx.x * kPrepWarps, idx = first + (threadIdx.x >> 5), p0 = first / (uint32_t)G;
     const uint32_t mine = first < pairs ? (min(first + kPrepWarps, pairs) - 1u) / (uint32_t)G - p0 + 1u : 0u;
     const uint32_t at = blockIdx.x * kPrepThreads + threadIdx.x, all = gridDim.x * kPrepThreads, vec_at = in.skip + at;
-    uint4 pol, vec;
+    uint4 pol, kind, vec;
+    const bool has_kind = mine != 0 && threadIdx.x < in.kinds * kKindVecs;
     if (threadIdx.x < mine * kVecs) pol = table(p0 * kVecs + threadIdx.x);
+    if (has_kind) kind = table(P * kVecs + threadIdx.x);
     if (vec_at < in.vecs) vec = table(vec_at);
     // what the kernels behind this one must find zero
     for (uint32_t i = at; i < clear_vecs; i += all) clear[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x < mine * kVecs) s_pol[threadIdx.x] = pol;
+    if (has_kind) s_kind[threadIdx.x] = kind;
     for (uint32_t i = vec_at; i < in.vecs; i += all) static_cast<uint4*>(in.device)[i] = i == vec_at ? vec : table(i);
     __syncthreads();
     if (BYTES == 0 && threadIdx.x == 0) {
@@ -142,7 +145,16 @@ k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __re
         const uint32_t p = idx / (uint32_t)G;
         const int g = (int)(idx - p * (uint32_t)G);
         if (DBG_OK(g, G, DBG_K_PREP, DBG_GROUP) && DBG_OK(p - p0, kPrepWarps, DBG_K_PREP, DBG_POLICY))
-            prep_pair(reinterpret_cast<const PolicyConst*>(s_pol)[p - p0], p, g, P, gc, cum_mass, cnt, sorted, grp_off, prep);
+        {
+            const PolicyIn pi = reinterpret_cast<const PolicyIn*>(s_pol)[p - p0];
+            PolicyKind pk;
+            if (pi.kind < kNear) pk = reinterpret_cast<const PolicyKind*>(s_kind)[pi.kind];
+            else {
+#pragma unroll
+                for (uint32_t k = 0; k < kKindVecs; ++k) reinterpret_cast<uint4*>(&pk)[k] = table(P * kVecs + pi.kind * kKindVecs + k);
+            }
+            prep_pair(pi, pk, p, g, P, gc, cum_mass, cnt, sorted, grp_off, prep);
+        }
     }
     // (the last blocks first: the others have clearing and preparing to do)
     for (uint32_t i = (gridDim.x - 1u - blockIdx.x) * kPrepThreads + threadIdx.x; i < in.n_chunks[0] + in.n_chunks[1]; i += all) {
@@ -191,7 +203,7 @@ constexpr uint64_t kBetaSmallN = 1u << 20;
 static_assert(kMaxPrompt * kBetaSmallN <= 1ull << 32, "a length's tokens");
 template <bool LARGE, bool SMALL>
 __global__ void __launch_bounds__(kBetaThreads)
-k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __restrict__ cum_mass,
+k_prep_beta(const PolicyIn* __restrict__ pol, const PolicyKind* __restrict__ kinds, uint32_t P, const int64_t* __restrict__ cum_mass,
             const uint32_t* __restrict__ cnt, const int32_t* __restrict__ sorted, const uint32_t* __restrict__ grp_off,
             const uint32_t* __restrict__ tick_start, const uint32_t* __restrict__ tick_cnt, const uint32_t* __restrict__ pairs,
             Prep* __restrict__ prep, bool early) {
@@ -207,8 +219,8 @@ k_prep_beta(const PolicyConst* __restrict__ pol, uint32_t P, const int64_t* __re
     const int g = (int)(pair / P);
     Prep& out = prep[(size_t)g * P + p];
     const Prep pr = out;
-    const PolicyConst pc = pol[p];
-    if (!pr.beta_rule || !pr.device_constrained || (double)pc.budget <= (double)pc.alpha) return;   // block-uniform
+    const PolicyIn pc = pol[p];
+    if (!pr.beta_rule || !pr.device_constrained || (double)pc.budget <= (double)kinds[pc.kind].alpha) return;   // block-uniform
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const uint32_t off = grp_off[g], N = grp_off[g + 1] - off;
     const int32_t* srt = sorted + off;
@@ -403,11 +415,11 @@ cudaError_t launch_prep(uint32_t P, int G, const GroupConst* gc, const int64_t* 
     return go(k_prep<0>, tables.host);
 }
 
-cudaError_t launch_prep_beta(const PolicyConst* pol, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
+cudaError_t launch_prep_beta(const PolicyIn* pol, const PolicyKind* kinds, uint32_t P, const int64_t* cum_mass, const uint32_t* cnt,
                              const int32_t* sorted, const uint32_t* grp_off, const uint32_t* tick_start,
                              const uint32_t* tick_cnt, const uint32_t* pairs, uint32_t n_pairs, uint64_t most, Prep* prep, bool early, cudaStream_t st) {
     auto* kernel = most > kBetaLargeN ? k_prep_beta<true, false> : most < kBetaSmallN ? k_prep_beta<false, true> : k_prep_beta<false, false>;
-    return launch_after(kernel, n_pairs, kBetaThreads, 0, st, pol, P, cum_mass, cnt, sorted, grp_off, tick_start,
+    return launch_after(kernel, n_pairs, kBetaThreads, 0, st, pol, kinds, P, cum_mass, cnt, sorted, grp_off, tick_start,
                         tick_cnt, pairs, prep, early);
 }
 

@@ -419,3 +419,12 @@ def test_linear_wait_rule_of_many_requests(n, lengths):
     tr.eval_policies(pols, 1)
     check_prep(tr, Oracle.from_workload(w), pols, f"{n} {lengths}")
     tr.close()
+
+
+@pytest.mark.parametrize("kinds", [1, 16, 17, 64, 65, 700])
+def test_policies_of_many_kinds(kinds):
+    # what policies share goes to the preparation once: kinds that come back, more of them than are looked up or lie close at hand,
+    # with the launch and in page-locked memory
+    w = synth.tiny_workload(151, 300, n_servers=2, max_prompt=300, max_out=30, device_dearer=True)
+    pols = [synth.policy(0.001 * (k % 997), alpha=0.01 + 0.001 * (k % kinds), expected_len=k % 2 * 20) for k in range(max(kinds, 3))]
+    full_parity(w, pols + pols[::2], select=False, tag=f"{kinds}")
