@@ -187,10 +187,10 @@ __device__ Sum last_within(double limit) {
 // (LARGE) beyond.  It does not grow with beta, so beta is found by search: three slopes a
 // round, which cut the range to a quarter.  A thread keeps up to four of the prompt lengths that occur and, for each, the two positions in the
 // sorted ticks that belong to the ends of the range, between which the positions of the slopes in between lie; the first
-// and last positions come from the bins' starts in shared memory.  Bound: issue and latency of one block (some eleven rounds by bins of
-// two barriers and up to a dozen products a thread, two by ticks).  (300,000 requests in six groups under sixteen such policies: 437 us
+// and last positions come from the bins' starts in shared memory.  Bound: issue and latency of one block (rounds by bins of
+// two barriers and up to a dozen products a thread, then two by ticks).  (300,000 requests in six groups under sixteen such policies: 437 us
 // with a bisection whose every step searched all the ticks for every length, 82 with every length and products of 64 by 64 bits, 31 of
-// them the rounds by bins, 60 now.  Four blocks a pair gave 4 us with few pairs and lost 15 once the pairs outnumbered the
+// them the rounds by bins, 60 with these kept short, 50 now that they part octaves.  Four blocks a pair gave 4 us with few pairs and lost 15 once the pairs outnumbered the
 // multiprocessors; three searches in step gave nothing.)
 constexpr int kBetaThreads = 1024;
 constexpr int kBetaLens = kMaxPrompt / kBetaThreads;                  // prompt lengths a thread has
@@ -319,7 +319,13 @@ k_prep_beta(const PolicyIn* __restrict__ pol, const PolicyKind* __restrict__ kin
     //      the range without a look at the ticks
     while (hi - lo > 1) {
         const long long d = hi - lo;
-        const long long m[3] = {lo + (d + 3) / 4, lo + (d + 1) / 2, lo + (3 * d + 3) / 4};
+        long long m[3] = {lo + (d + 3) / 4, lo + (d + 1) / 2, lo + (3 * d + 3) / 4};
+        if (hi > 8 * (lo + 1)) {
+            // The bins part octaves: while the ends are octaves apart so are the slopes in between.  (w_tail is far above the slope that fits,
+            // which even parts of the range approach by two bits a round; any three in between will do, to whatever digits.)
+            const float at = (float)(lo + 1), by = sqrtf(sqrtf((float)hi / at));
+            m[0] = min((long long)(at * by), hi - 1); m[1] = min((long long)(at * by * by), hi - 1); m[2] = min((long long)(at * by * by * by), hi - 1);
+        }
         Sum v[6] = {0, 0, 0, 0, 0, 0};                                // at least, at most
 #pragma unroll
         for (int i = 0; i < kBetaLens; ++i) {
