@@ -902,7 +902,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     // ---- request chunks, of one group each: of the grid kernel, about two to each block that fits the GPU at once, 256
     //      requests (one a thread) or more (three to a block: k_grid and k_spread for 16 M requests in six groups under 128
     //      budgets by 8 overheads 369 us either way, under 16 by 2 218 instead of 205, in one group under 64 budgets 139
-    //      instead of 133, a million 34 instead of 30); of the pair kernel, two to a multiprocessor, 2,048 requests or more
+    //      instead of 133, a million 34 instead of 30)
     const uint32_t sms = (uint32_t)c->sms, kMaxChunk = 65280;
     int tallest = 1;
     for (const Slab& sl : slabs) tallest = std::max(tallest, sl.T);
@@ -935,7 +935,27 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     if (std::getenv("DISCO_DEBUG_RUNS")) joined = false;
 #endif
     plan_chunks(0, joined && !stored ? chunk_size((size_t)sms * 8, 256) : chunk_size(std::max<size_t>(2 * at_once / std::min<size_t>(most_slabs, 4), 1), 256));
-    if (any_pairs) plan_chunks(1, chunk_size((size_t)2 * sms, 2048));
+    if (any_pairs) {
+        // of the pair kernel, whose blocks (a chunk and 32 policies each) take a multiprocessor's shared memory: the fewest whole rounds
+        // of them, where a block costs as much as some 800 requests besides its own.  (300,000 requests in six groups under 32
+        // policies, k_pairs_acc 56.7 us in chunks of 2,048 -- 150, two more than a round -- 50.7 in chunks of 1,024, 50.0 of 2,304.)
+        size_t listed = 1;
+        for (const ClassLists& L : lists) listed = std::max(listed, L.n_ext);
+        for (const Slab& sl : slabs) if (sl.mixed) listed = std::max<size_t>(listed, sl.policies);
+        const size_t tiles = (listed + 31) / 32;
+        auto blocks = [&](size_t ch) { size_t k = 0; for (int g = 0; g < G; ++g) if (rb.ng[g]) k += (rb.ng[g] - 1) / ch + 1; return k * tiles; };
+        uint32_t best = kMaxChunk;
+        size_t least = ~(size_t)0;
+        for (size_t rounds = 1; rounds <= 8; ++rounds) {
+            const size_t at_most = rounds * sms;
+            if ((size_t)groups * tiles > at_most) continue;
+            size_t ch = chunk_size((at_most + tiles - 1) / tiles, 256);
+            while (ch <= kMaxChunk && blocks(ch) > at_most) ch += 256;
+            if (ch > kMaxChunk || rounds * (ch + 800) >= least) continue;
+            best = (uint32_t)ch; least = rounds * (ch + 800);
+        }
+        plan_chunks(1, best);
+    }
 
     // ---- device memory: what must be clear comes first and together -- the work counters and tickets, the difference
     //      tables of the first batch, and the accumulators if some pairs are added to them one by one (k_spread writes those

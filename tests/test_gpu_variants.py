@@ -428,3 +428,19 @@ def test_policies_of_many_kinds(kinds):
     w = synth.tiny_workload(151, 300, n_servers=2, max_prompt=300, max_out=30, device_dearer=True)
     pols = [synth.policy(0.001 * (k % 997), alpha=0.01 + 0.001 * (k % kinds), expected_len=k % 2 * 20) for k in range(max(kinds, 3))]
     full_parity(w, pols + pols[::2], select=False, tag=f"{kinds}")
+
+
+@pytest.mark.parametrize("n", [1, 256, 148 * 256, 148 * 256 + 1, 100_001])
+@pytest.mark.parametrize("shape,policies", [((1, 1), 3), ((2, 3), 33), ((3, 3), 200)])
+def test_pairs_in_whole_rounds_of_blocks(n, shape, policies):
+    # policies with random routing take the pair kernel: a request to a multiprocessor's thread or one more, several tiles of
+    # policies, and more groups times tiles than a round has blocks
+    from oracle import Oracle
+    from paper_2502_11417_b200 import Trace
+    from parity import check_stats
+    w = synth.tiny_workload(157, n, n_servers=shape[0], n_devices=shape[1], max_prompt=300, max_out=30)
+    pols = [synth.policy(b, mig_threshold=1e-6 * (k % 2), flags=PACED | synth.FLAG_STOCHASTIC) for k, b in enumerate(synth.budget_grid(policies))]
+    tr = Trace.from_workload(w)
+    tr.eval_policies(pols, w.seed)
+    check_stats(tr.reduce_stats(), Oracle.from_workload(w).eval(pols, w.seed)[0], tr.histograms, f"{n} {shape} {policies}")
+    tr.close()
