@@ -43,6 +43,9 @@ constexpr int kListCap = 4096;           // requests a block lists whose TTFT th
 // in six groups under 32 by 2 34 us, now 30).  Not with more rows: the additions to their histograms are as many as the rows, and the call
 // costs registers.
 __host__ __device__ constexpr int list_few(int NT) { return NT > 2 ? 0 : 256 / (1 + NT); }
+// Requests that may be swept at once where any may be listed: whole rounds of the block, so that what a lane takes of a chunk in several
+// sweeps is no more than in one.
+__device__ __forceinline__ uint32_t list_room(uint32_t listed) { return ((uint32_t)kListCap - listed) / kThreads * kThreads; }
 constexpr int kMaxSeg = 2 * kGridCols + 2;
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr uint32_t kNoPolicy = 0xFFFFFFFFu;
@@ -851,7 +854,7 @@ k_grid(const __grid_constant__ Args a) {
             passes = 1;
         }
         // a segment's last columns, which wait 0, and beside them its first ones: the device alone
-        if constexpr (MODE == M_RACES) {
+        if (MODE == M_RACES || (WIDE && !waits)) {
             for (int si = 0; si < n_seg; ++si) {
                 const Seg sg = sm.seg[si];
                 const bool race = (int)sg.k2 < K, side = sg.k1 > 0;
@@ -866,24 +869,70 @@ k_grid(const __grid_constant__ Args a) {
                 __syncthreads();
                 ++passes; turn ^= 1;
             }
+        } else if constexpr (WIDE) {
+            // Windows: run by run, [k2, K), each column of [k1, k2), [0, k1), and, when the list is half full or the chunk is done, the list
+            // for the columns that wait longer, with the common wait's totals taken back from them.  (A sweep for two runs, and the
+            // turns of the kernels below, cost registers that are short here: 250,000 requests in five classes, those with windows 46.7 us
+            // instead of 42.0.)
+            auto run = [&](uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, int q0, int q1, bool neg) {
+                Acc<NT, WIDE> s = {};
+                Side none = {};
+                sweep<NT, WIDE, S_NONE>(a, c, th, sm, tbt, lv, pa, pb, w, list, push, false, true, false, s, none);
+                share_out<NT, WIDE>(sm, s, lv, turn);
+                __syncthreads();
+                enter<NT, WIDE>(sm, tbt, tb, g, q0, q1, neg, turn);
+                __syncthreads();
+                ++passes; turn ^= 1;
+            };
+            constexpr uint32_t kListStep = kListCap / 2;
+            uint32_t pa = 0;                                          // (of the segment in work: where the sweep goes on)
+            int si = 0, ri = 0;
+            for (;;) {
+                uint32_t from = 0, to = 0, w = 0;
+                int q0 = 0, q1 = 0;
+                bool push = false;
+                const bool done = si >= n_seg;
+                if (!done) {
+                    const Seg sg = sm.seg[si];
+                    const int n_pts = (int)sg.k2 - (int)sg.k1;
+                    if (ri == 0) pa = sg.pa;
+                    if (ri == 0 && (int)sg.k2 >= K) { ++ri; continue; }
+                    if (ri > n_pts && sg.k1 == 0) { ri = 0; ++si; continue; }
+                    from = pa; to = sg.pb;
+                    if (ri == 0) { q0 = sg.k2; q1 = K; ++ri; }
+                    else if (ri <= n_pts) { q0 = (int)sg.k1 + ri - 1; q1 = q0 + 1; w = sm.w_star[q0]; ++ri; }
+                    else {
+                        w = wt_min; q1 = sg.k1; push = n_low > 0;
+                        if (push && to - from > (uint32_t)kListStep) { to = from + kListStep; pa = to; }
+                        else { ri = 0; ++si; }
+                    }
+                    run(from, to, w, false, push, q0, q1, false);
+                } else if (sm.n_list == 0) break;
+                if (done || (push && sm.n_list > (uint32_t)(kListCap - kListStep))) {
+                    const uint32_t k = sm.n_list;                     // (barriers inside run: all threads agree)
+                    __syncthreads();
+                    if (threadIdx.x == 0) sm.n_list = 0;
+                    for (int p = -1; p < n_low; ++p)                  // the common wait's totals go, each column's own come
+                        run(0u, k, p < 0 ? wt_min : sm.w_tail[p], true, false, max(p, 0), p < 0 ? n_low : p + 1, p < 0);
+                }
+            }
         } else if constexpr (MODE == M_WAITS) {
             // Segment by segment: each column of [k1, k2) under its own w*; then [k2, K), which waits 0, in one sweep with [0, k1), where the
             // device runs alone or (Algorithm 2) waits w_tail.  The few requests that w_tail does not cover have been listed.  A handful is
             // entered request by request; more are entered for [0, k1) from the list, and when it is half full or the chunk is done,
             // the columns that wait longer get what they come to there under their own wait in place of the common one.
-            enum { POINTS, MAIN, ALONE, LISTED, LONGER } at = POINTS;
-            constexpr int kFirst = WIDE ? -1 : 0;                      // of the columns that wait longer (-1: the common wait's totals are taken back)
+            enum { POINTS, MAIN, LISTED, LONGER } at = POINTS;
             uint32_t pos = 0, listed = 0, n_list = 0;                  // where the segment's sweep goes on; the list: entered for [0, k1), all
             int si = 0, ri = 0;                                       // segment, point or column
 #pragma unroll 1
             for (;;) {
                 uint32_t from = 0, to = 0, w = 0;
                 int q0 = 0, q1 = 0;
-                bool neg = false, list = false, push = false;
+                bool list = false;
                 if (at == POINTS) {
                     if (si >= n_seg) {
                         if (n_list == 0) break;
-                        at = LONGER; ri = kFirst;
+                        at = LONGER; ri = 0;
                         continue;
                     }
                     const Seg sg = sm.seg[si];
@@ -894,70 +943,54 @@ k_grid(const __grid_constant__ Args a) {
                     const Seg sg = sm.seg[min(si, kMaxSeg - 1)];
                     const bool race = (int)sg.k2 < K, side = sg.k1 > 0;
                     if (pos >= sg.pb || !(race || side)) { at = POINTS; ri = 0; ++si; continue; }
-                    if (WIDE && waits) { at = ALONE; ri = race ? 0 : 1; continue; }
                     Acc<NT, WIDE> s = {};
                     Side o = {};
                     for (;;) {
                         uint32_t end = sg.pb;
-                        if (!WIDE && waits && side) end = min(end, pos + (uint32_t)kListCap - n_list);
-                        sweep<NT, WIDE, WIDE ? S_DEVICE : S_EITHER>(a, c, th, sm, tbt, lv, pos, end, wt_min, false, false, waits, race, side, s, o);
+                        if (waits && side) end = min(end, pos + list_room(n_list));
+                        sweep<NT, WIDE, S_EITHER>(a, c, th, sm, tbt, lv, pos, end, wt_min, false, false, waits, race, side, s, o);
                         pos = end;
-                        if (WIDE || !waits || !side) break;
+                        if (!waits || !side) break;
                         __syncthreads();
                         n_list = sm.n_list;
                         __syncthreads();
-                        if (pos >= sg.pb || n_list > (uint32_t)(kListCap - kThreads)) break;
+                        if (pos >= sg.pb || list_room(n_list) == 0u) break;
                     }
                     if (race) share_out<NT, WIDE>(sm, s, lv, turn);
                     if (side) share_side<NT, WIDE>(sm, o, turn);
-                    if constexpr (!WIDE && list_few(NT) != 0) {
+                    if constexpr (list_few(NT) != 0) {
                         if (n_list > listed && n_list - listed <= (uint32_t)list_few(NT)) {
                             enter_listed<NT>(a, sm, listed, n_list, wt_min, n_low, sg.k1);
                             n_list = listed;
                         }
                     }
                     __syncthreads();
-                    if (!WIDE && threadIdx.x == 0) sm.n_list = n_list;
+                    if (threadIdx.x == 0) sm.n_list = n_list;
                     if (race) enter<NT, WIDE>(sm, tbt, tb, g, sg.k2, K, false, turn);
                     if (side) enter_side<NT, WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1, waits, turn);
                     __syncthreads();
                     ++passes; turn ^= 1;
-                    if (!WIDE && n_list > listed) at = LISTED;
+                    if (n_list > listed) at = LISTED;
                     continue;
-                } else if (WIDE && at == ALONE) {
-                    // (windows: the sweep for [k2, K), then those for [0, k1), whose requests that w_tail does not cover are listed for the
-                    // columns that wait longer)
-                    const Seg sg = sm.seg[si];
-                    if (ri == 0) { from = sg.pa; to = sg.pb; q0 = sg.k2; q1 = K; ri = 1; }
-                    else if (pos >= sg.pb || sg.k1 == 0) { pos = sg.pb; at = MAIN; continue; }
-                    else if (n_list > (uint32_t)kListCap / 2) { at = LONGER; ri = kFirst; continue; }
-                    else {
-                        push = n_low > 0;
-                        from = pos; to = push ? min((uint32_t)sg.pb, pos + (uint32_t)kListCap / 2) : sg.pb; w = wt_min; q1 = sg.k1;
-                        pos = to;
-                    }
-                } else if (!WIDE && at == LISTED) {
+                } else if (at == LISTED) {
                     const int k1 = sm.seg[si].k1;
                     list = true; from = listed; to = n_list; w = wt_min; q0 = n_low; q1 = k1;
                     listed = n_list;
                     at = MAIN;
                     if (n_low == 0) listed = n_list = 0;
-                    else if (n_list > (uint32_t)kListCap / 2) { at = LONGER; ri = kFirst; }
+                    else if (n_list > (uint32_t)kListCap / 2) { at = LONGER; ri = 0; }
                     if (q0 >= k1) continue;                            // (every column waits longer)
                 } else {
-                    list = true; to = n_list; neg = WIDE && ri < 0;
-                    w = neg ? wt_min : sm.w_tail[ri];
-                    q0 = neg ? 0 : ri; q1 = neg ? n_low : ri + 1;
-                    if (++ri == n_low) { listed = n_list = 0; at = si >= n_seg ? POINTS : WIDE ? ALONE : MAIN; }
+                    list = true; to = n_list; w = sm.w_tail[ri]; q0 = ri; q1 = ri + 1;
+                    if (++ri == n_low) { listed = n_list = 0; at = si >= n_seg ? POINTS : MAIN; }
                 }
                 Acc<NT, WIDE> s = {};
                 Side none = {};
-                sweep<NT, WIDE, S_NONE>(a, c, th, sm, tbt, lv, from, to, w, list, push, false, true, false, s, none);
+                sweep<NT, WIDE, S_NONE>(a, c, th, sm, tbt, lv, from, to, w, list, false, false, true, false, s, none);
                 share_out<NT, WIDE>(sm, s, lv, turn);
                 __syncthreads();
-                if (n_list == 0 && threadIdx.x == 0 && !push) sm.n_list = 0;
-                if (WIDE && push) n_list = sm.n_list;
-                enter<NT, WIDE>(sm, tbt, tb, g, q0, q1, neg, turn);
+                if (n_list == 0 && threadIdx.x == 0) sm.n_list = 0;
+                enter<NT, WIDE>(sm, tbt, tb, g, q0, q1, false, turn);
                 __syncthreads();
                 ++passes; turn ^= 1;
             }
