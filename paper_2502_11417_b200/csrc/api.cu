@@ -1079,32 +1079,42 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         for (size_t k = first; k < last; ++k)
             if ((k != 0 || timed) && plan[k].kinds) CU(play_out(k));
         if (timed) CU(cudaEventRecord(c->ev[2], st));
-        for (; next < batches.size() && batches[next].wave == first / wave; ++next) {
-            const Batch& b = batches[next];
-            GridTables gt;
-            char* base = (char*)c->d_grid.p + b.at;
-            gt.sums = (unsigned long long*)base;
-            gt.tbt = base + b.sums * 8;
-            gt.ttft = (uint32_t*)(base + b.sums * 8 + b.tbt * (b.wide ? 8 : 4));
-            if (!side_by_side && next != 0) CU(cudaMemsetAsync(base, 0, batch_bytes(b), st));
-            const Slab* dsl = d_slabs + b.first;
-            const Slab& sl = slabs[b.first];
+        while (next < batches.size() && batches[next].wave == first / wave) {
+            // grids with tables of their own run beside each other (the one behind needs nothing of the one in front), then k_spread each
+            size_t end = next + 1;
+            const Slab& sl = slabs[batches[next].first];
+            if (side_by_side && !sl.mixed)
+                while (end < batches.size() && batches[end].wave == first / wave && !slabs[batches[end].first].mixed) ++end;
+            auto tables_of = [&](const Batch& b) {
+                char* base = (char*)c->d_grid.p + b.at;
+                return GridTables{(uint32_t*)(base + b.sums * 8 + b.tbt * (b.wide ? 8 : 4)), base + b.sums * 8, (unsigned long long*)base};
+            };
             LeftLists left = {nullptr, nullptr};
             if (sl.mixed) {
                 left.list = c->d_left.as<uint32_t>(); left.count = left.list + N1;
                 CU(cudaMemsetAsync(left.count, 0, (size_t)G * 4, st));
             }
-            CU(launch_grid(tr, gc, d_classes, prep, P, dsl, (uint32_t)b.count, b.T, b.wide, d_tab,
-                           d_chunks, tables.n_chunks[0], rec, rec_stride, gt, left, k0, tickets + ticket, work, beside && ticket == 0, any_waits, joined, c->sms, st));
-            ++ticket;
-            CU(launch_spread(tr, gc, dsl, (uint32_t)b.count, b.T, b.wide, d_tab, gt, acc, h_ttft, h_tbt, st));
-            g_launches += 2;
+            for (size_t k = next; k < end; ++k) {
+                const Batch& b = batches[k];
+                if (!side_by_side && k != 0) CU(cudaMemsetAsync((char*)c->d_grid.p + b.at, 0, batch_bytes(b), st));
+                CU(launch_grid(tr, gc, d_classes, prep, P, d_slabs + b.first, (uint32_t)b.count, b.T, b.wide, d_tab, d_chunks, tables.n_chunks[0], rec,
+                               rec_stride, tables_of(b), left, k0, tickets + ticket, work, k > next || (beside && ticket == 0), k + 1 < end, any_waits,
+                               joined, c->sms, st));
+                ++ticket;
+            }
+            for (size_t k = next; k < end; ++k) {
+                const Batch& b = batches[k];
+                CU(launch_spread(tr, gc, d_slabs + b.first, (uint32_t)b.count, b.T, b.wide, d_tab, tables_of(b), acc, h_ttft, h_tbt, st));
+                g_launches += 2;
+            }
             if (sl.mixed) {
+                const Batch& b = batches[next];
                 CU(launch_pairs_acc(tr, gc, d_classes + sl.cls, prep, P, d_tab + mixed_pols[b.first], sl.policies, d_pair_chunks,
                                     tables.n_chunks[1], left.list, left.count, rec_of(sl.cls), acc, h_ttft, h_tbt, work, k0,
                                     sl.expected_len != 0, b.wide, st));
                 g_launches += 1;
             }
+            next = end;
         }
         for (size_t k = first; k < last; ++k) {
             if (!lists[k].n_ext) continue;

@@ -327,6 +327,7 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
                         const uint32_t* tab, const Chunk* chunks, uint32_t n_chunks, TimelineRec rec /* of slot 0 */, size_t rec_stride, GridTables gt,
                         LeftLists left /* of these slabs, or nulls: none is mixed */, uint32_t k0, uint32_t* ticket /* zero */,
                         uint64_t* work /* [4], added to */, bool beside /* runs beside its predecessor, whose own it has complete */,
+                        bool early /* its successor runs beside it */,
                         bool waits /* Algorithm 2 decides in some group */, bool joined /* requests side by side, not run by run */, int sms, cudaStream_t st);
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
                           bool wide, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,

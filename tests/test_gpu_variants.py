@@ -444,3 +444,15 @@ def test_pairs_in_whole_rounds_of_blocks(n, shape, policies):
     tr.eval_policies(pols, w.seed)
     check_stats(tr.reduce_stats(), Oracle.from_workload(w).eval(pols, w.seed)[0], tr.histograms, f"{n} {shape} {policies}")
     tr.close()
+
+
+@pytest.mark.parametrize("n", [1, 700, 20_001, 60_000])
+@pytest.mark.parametrize("shape", [(1, 1), (2, 3)])
+def test_grids_beside_each_other(n, shape):
+    # grids of one, five and two rows, with windows and without, and between them one whose overheads differ by budget (which runs
+    # by itself)
+    w = synth.tiny_workload(163 + n, n, n_servers=shape[0], n_devices=shape[1], max_prompt=500, max_out=60, device_dearer=True)
+    of = lambda rate, rows: [synth.policy(b, r_c=rate, flags=PACED, mig_threshold=1e-6 * k) for b in (0.02, 0.2, 0.7) for k in range(rows)]
+    full_parity(w, of(5.0, 1) + of(6.0, 5) + of(40.0, 2), select=False, tag=f"{n} {shape}")
+    by_budget = [synth.policy(b, r_c=7.0, flags=PACED, mig_threshold=1e-6 * k) for k, b in enumerate(synth.budget_grid(9))]
+    full_parity(w, of(40.0, 1) + by_budget + of(6.0, 1) + of(5.0, 3), select=False, tag=f"{n} {shape} and one apart")
