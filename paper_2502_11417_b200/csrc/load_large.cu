@@ -12,7 +12,9 @@
 //   k_ticks    the same for the ticks;
 //   k_order    the records of a bucket by length;
 //   k_sort     the ticks of a bucket ascending.
-// Nothing waits for another block.
+// Nothing waits for another block.  Records and ticks need nothing of each other: k_ticks begins where a block of k_records has ended, and
+// so do k_order behind k_ticks and k_sort behind k_order, each of which waits for the kernel in front before it ends (a step of 4 M requests
+// 297 -> 283 us, of 16 M in six groups 1,090 -> 1,057: the last tiles and buckets of a kernel leave most multiprocessors idle).
 //
 // Bound: memory and shared-memory atomics.  16 M requests in six groups: k_load 855 us, these 550 (count 58, plan 13, records 149,
 // ticks 109, order 105, sort 114); 4 M in one group 213 and 157, in six 209 and 183.  At 3 M k_load wins (127 and 136 in one group,
@@ -243,6 +245,7 @@ k_records(const __grid_constant__ LoadArgs a) {
     uint32_t* s_to = s_start + n_rec;                                  // [n_rec] place in the bucket less place in s_req
     uint16_t* s_of = (uint16_t*)(s_to + n_rec);                        // [G][kLens]
     grid_dependency_wait();
+    let_next_start();
     if (refused(a)) return;
     for (int i = tid; i < G * kLens; i += kThreads) s_of[i] = a.large.rec_bucket[i];
     const bool wide = columns_aligned(a);
@@ -305,8 +308,8 @@ k_ticks(const __grid_constant__ LoadArgs a) {
     uint32_t* s_to = s_start + n_tick;
     uint16_t* s_in = (uint16_t*)(s_to + n_tick);                       // [kTile] the ticks' buckets
     uint16_t* s_of = s_in + kTile;                                     // [G][kTickBins]
-    grid_dependency_wait();
-    if (refused(a)) return;
+    // (beside k_records, which began when k_plan was complete)
+    if (refused(a)) { grid_dependency_wait(); return; }
     for (int i = tid; i < G * kTickBins; i += kThreads) s_of[i] = a.large.tick_bucket[i];
     const bool wide = columns_aligned(a);
     const uint32_t tile = even_tile(a.n), stride = gridDim.x * tile;
@@ -315,6 +318,8 @@ k_ticks(const __grid_constant__ LoadArgs a) {
     if (t0 < a.n) read_tile<FORM>(a, t0, end, wide, raw);
 #pragma unroll 1
     for (; t0 < a.n; t0 += stride, end = min(a.n, t0 + tile)) {
+        // (with the last tile; k_order reads what k_records has written.  The first block has a tile.)
+        if (t0 + stride >= a.n) { grid_dependency_wait(); let_next_start(); }
         for (uint32_t i = tid; i < n_tick; i += kThreads) s_start[i] = 0;
         __syncthreads();
         uint32_t S[kPer], tick[kPer];
@@ -359,7 +364,9 @@ constexpr int kOrderThreads = 512;
 __global__ void __launch_bounds__(kOrderThreads)
 k_order(const __grid_constant__ LoadArgs a) {
     __shared__ uint32_t s_at[kLens];
-    grid_dependency_wait();
+    // (beside k_ticks, which let it begin when k_records was complete; and k_sort beside this one, when k_ticks is: the last block, for all)
+    if (blockIdx.x == gridDim.x - 1) grid_dependency_wait();
+    let_next_start();
     if (refused(a)) return;
     const uint2 members = __ldcg(&a.large.rec_members[blockIdx.x]);
     if (members.x > members.y) return;
@@ -535,8 +542,7 @@ k_sort(const __grid_constant__ LoadArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t s_item;
     BigSort& sm = *reinterpret_cast<BigSort*>(smem_raw);
-    grid_dependency_wait();
-    if (refused(a)) return;
+    if (refused(a)) { grid_dependency_wait(); return; }                // (beside k_order)
 #pragma unroll 1
     for (uint32_t bucket = blockIdx.x * 2u; bucket <= blockIdx.x * 2u + 1u; ++bucket) {
         const uint4 j = __ldcg(&a.large.tick_jobs[bucket]);            // ticks [x, y) of the bins z .. w, counted through the groups
@@ -556,7 +562,9 @@ k_sort(const __grid_constant__ LoadArgs a) {
     // the last block to come here reports the flags
     if (threadIdx.x == 0) { __threadfence(); s_item = atomicAdd(&a.z->done, 1u); }
     __syncthreads();
-    if (s_item == gridDim.x - 1 && threadIdx.x < 4) a.readback->err[threadIdx.x] = __ldcg(&a.z->err[threadIdx.x]);
+    if (s_item != gridDim.x - 1) return;
+    grid_dependency_wait();
+    if (threadIdx.x < 4) a.readback->err[threadIdx.x] = __ldcg(&a.z->err[threadIdx.x]);
 }
 
 size_t records_smem(const LoadArgs& a) { return (size_t)kTile * 16 + (size_t)whole_vectors(a.large.n_rec) * 8 + (size_t)a.G * kLens * 2; }
