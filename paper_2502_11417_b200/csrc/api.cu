@@ -727,12 +727,12 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const uint32_t k0 = seed_key(seed) + (uint32_t)c->first_index * kHashReq;
     c->timing_valid = false;
     const bool timed = c->timing && classes.size() == 1;
-    auto play_out = [&](size_t k) {
+    auto play_out = [&](size_t k, bool beside) {
         g_launches += timeline_launches(plan[k].kinds);
         return launch_timeline(tr, gc, classes[k], c->knots.as<int32_t>(), k0, rec_of(k), c->err, c->play_ticket.as<uint32_t>(),
-                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, more[k], &c->z->free_ticket, rb.ng, k == 0 && !timed, c->sms, st);
+                               plan[k].kinds, plan[k].batches, plan[k].search, long_outputs, timed ? c->ev[1] : nullptr, more[k], &c->z->free_ticket, rb.ng, beside, k == 0 && !timed, c->sms, st);
     };
-    if (n != 0 && !timed) CU(play_out(0));
+    if (n != 0 && !timed) CU(play_out(0, false));
 
     // ---- the policies of a class: plain ones form grids of budgets by overheads (grid.cu), at most kGridCols by kGridRows
     //      to a slab; random routing and the Eq. 1-2 rule go pair by pair
@@ -1072,12 +1072,19 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             plan[k].kinds &= ~(1u << G_EXACT);
             many.cls[many.count] = (uint32_t)k; many.slot[many.count++] = (uint32_t)slot_of(k);
         }
+        // (free streams of other classes are played out beside these: nobody needs the others' results)
+        size_t free_class = last;
+        for (size_t k = std::max<size_t>(first, 1); k < last && many.count && !timed; ++k) {
+            if (!plan[k].kinds) continue;
+            if ((plan[k].kinds & (1u << G_FREE)) && !(plan[k].kinds & (1u << G_EXACT))) free_class = k;
+            break;
+        }
         if (many.count) {
-            CU(launch_playout_many(tr, gc, c->knots.as<int32_t>(), k0, rec, many, c->sms, st));
+            CU(launch_playout_many(tr, gc, c->knots.as<int32_t>(), k0, rec, many, free_class < last, c->sms, st));
             g_launches += 1;
         }
         for (size_t k = first; k < last; ++k)
-            if ((k != 0 || timed) && plan[k].kinds) CU(play_out(k));
+            if ((k != 0 || timed) && plan[k].kinds) CU(play_out(k, k == free_class));
         if (timed) CU(cudaEventRecord(c->ev[2], st));
         while (next < batches.size() && batches[next].wave == first / wave) {
             // grids with tables of their own run beside each other (the one behind needs nothing of the one in front), then k_spread each
@@ -1104,7 +1111,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             }
             for (size_t k = next; k < end; ++k) {
                 const Batch& b = batches[k];
-                CU(launch_spread(tr, gc, d_slabs + b.first, (uint32_t)b.count, b.T, b.wide, d_tab, tables_of(b), acc, h_ttft, h_tbt, st));
+                CU(launch_spread(tr, gc, d_slabs + b.first, (uint32_t)b.count, b.T, b.wide, d_tab, tables_of(b), acc, h_ttft, h_tbt, k > next, k + 1 < end, st));
                 g_launches += 2;
             }
             if (sl.mixed) {

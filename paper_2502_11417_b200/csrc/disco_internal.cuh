@@ -288,7 +288,8 @@ cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const Clas
                             const uint32_t* batches, uint32_t search /* largest ClassConst::search of a group with requests */,
                             bool long_outputs /* mean output length of 512 tokens or more */,
                             cudaEvent_t mid /* recorded between the kernels of exact groups and the others, or null */,
-                            const FreeMore& more, uint32_t* free_ticket /* one word, zero before and after */, const uint32_t* grp_n /* requests per group, on the host */, bool early /* the preparation follows: it may start beside the last kernel */,
+                            const FreeMore& more, uint32_t* free_ticket /* one word, zero before and after */, const uint32_t* grp_n /* requests per group, on the host */,
+                            bool beside /* the first kernel runs beside its predecessor (only one of streams that never wait for the reader) */, bool early /* the preparation follows: it may start beside the last kernel */,
                             int sms /* multiprocessors of the device */, cudaStream_t st);
 uint32_t timeline_launches(uint32_t kinds);
 // The exact groups of several classes whose searches are short, in one launch.
@@ -296,7 +297,7 @@ constexpr int kShortMany = 16;
 struct ShortMany { const ClassConst* classes; size_t rec_stride; uint32_t count, cls[kShortMany], slot[kShortMany]; };
 bool short_search(uint32_t search);
 cudaError_t launch_playout_many(const TraceDev& tr, const GroupConst* gc, const int32_t* knots, uint32_t k0, TimelineRec rec /* of slot 0 */,
-                                const ShortMany& many, int sms, cudaStream_t st);
+                                const ShortMany& many, bool early /* its successor runs beside it */, int sms, cudaStream_t st);
 
 // Reductions over a grid of plain policies, budget by overhead (grid.cu).
 constexpr int kGridRows = 8;     // overheads a slab may have
@@ -331,7 +332,7 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
                         bool waits /* Algorithm 2 decides in some group */, bool joined /* requests side by side, not run by run */, int sms, cudaStream_t st);
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
                           bool wide, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
-                          uint64_t* hist_tbt, cudaStream_t st);
+                          uint64_t* hist_tbt, bool beside, bool early /* as above */, cudaStream_t st);
 // Pair by pair: `n_list` policies under the chunks' requests, or (list not null) under the listed ones.
 cudaError_t launch_pairs_acc(const TraceDev& tr, const GroupConst* gc, const ClassConst* cc, const Prep* prep, uint32_t P,
                              const uint32_t* pol_list, uint32_t n_list, const Chunk* chunks, uint32_t n_chunks,

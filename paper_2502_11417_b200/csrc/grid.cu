@@ -1056,9 +1056,11 @@ template <bool WIDE>
 __global__ void __launch_bounds__(kSpreadWarps * 32)
 k_spread(TraceDev tr, const GroupConst* __restrict__ gcs, const Slab* __restrict__ slabs,
          const uint32_t* __restrict__ tab, GridTables gt, unsigned long long* __restrict__ acc,
-         unsigned long long* __restrict__ hist_ttft, unsigned long long* __restrict__ hist_tbt) {
+         unsigned long long* __restrict__ hist_ttft, unsigned long long* __restrict__ hist_tbt, bool beside, bool early) {
     __shared__ unsigned long long s_part[kSpreadWarps * 33];
-    grid_dependency_wait();
+    // (beside another such kernel, which began when the tables were complete: the last block waits for it)
+    if (!beside || (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1)) grid_dependency_wait();
+    if (early) let_next_start();
     const Slab& sl = slabs[blockIdx.y];
     const int K = sl.K, T = sl.T, bin_tau = sl.bin_tau, lane = threadIdx.x & 31;
     const Tables<WIDE> tb(gt, sl, tr.n_groups);
@@ -1175,12 +1177,12 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
 
 cudaError_t launch_spread(const TraceDev& tr, const GroupConst* gc, const Slab* slabs, uint32_t n_slabs, int T,
                           bool wide, const uint32_t* tab, GridTables gt, uint64_t* acc, uint64_t* hist_ttft,
-                          uint64_t* hist_tbt, cudaStream_t st) {
+                          uint64_t* hist_tbt, bool beside, bool early, cudaStream_t st) {
     if (n_slabs == 0) return cudaSuccess;
     const dim3 grid((uint32_t)(2 * T * (kNBins / 32) + (tr.n_groups * T * kNAcc + 31) / 32), n_slabs);
     auto* kernel = wide ? k_spread<true> : k_spread<false>;
     return launch_after(kernel, grid, kSpreadWarps * 32, 0, st, tr, gc, slabs, tab, gt, (unsigned long long*)acc,
-                        (unsigned long long*)hist_ttft, (unsigned long long*)hist_tbt);
+                        (unsigned long long*)hist_ttft, (unsigned long long*)hist_tbt, beside, early);
 }
 
 }  // namespace disco

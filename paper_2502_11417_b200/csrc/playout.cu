@@ -516,21 +516,21 @@ cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const
                                  uint32_t k0, TimelineRec rec, uint32_t* ticket, uint32_t search, bool long_outputs, bool early, int sms,
                                  cudaStream_t st);
 cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots,
-                                uint32_t k0, TimelineRec rec, const FreeMore& more, uint32_t* ticket, const uint32_t* grp_n, bool early,
+                                uint32_t k0, TimelineRec rec, const FreeMore& more, uint32_t* ticket, const uint32_t* grp_n, bool beside, bool early,
                                 int sms, cudaStream_t st);
 
 uint32_t timeline_launches(uint32_t kinds) { return (kinds & 1u) + ((kinds >> 1) & 1u) + ((kinds >> 2) & 1u); }
 
 cudaError_t launch_timeline(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0,
                             TimelineRec rec, int32_t* err, uint32_t* ticket, uint32_t kinds, const uint32_t* batches,
-                            uint32_t search, bool long_outputs, cudaEvent_t mid, const FreeMore& more, uint32_t* free_ticket, const uint32_t* grp_n, bool early, int sms, cudaStream_t st) {
+                            uint32_t search, bool long_outputs, cudaEvent_t mid, const FreeMore& more, uint32_t* free_ticket, const uint32_t* grp_n, bool beside, bool early, int sms, cudaStream_t st) {
     cudaError_t e;
     const auto last = [&](int kind) { return early && kinds >> (kind + 1) == 0; };
     if (kinds & (1u << G_EXACT))
         if ((e = launch_playout_exact(tr, gc, cc, knots, k0, rec, ticket, search, long_outputs, last(G_EXACT), sms, st))) return e;
     if (mid && (e = cudaEventRecord(mid, st))) return e;
     if (kinds & (1u << G_FREE))
-        if ((e = launch_playout_free(tr, gc, cc, knots, k0, rec, more, free_ticket, grp_n, last(G_FREE), sms, st))) return e;
+        if ((e = launch_playout_free(tr, gc, cc, knots, k0, rec, more, free_ticket, grp_n, beside && !(kinds & (1u << G_EXACT)), last(G_FREE), sms, st))) return e;
     if (kinds & (1u << G_GENERAL)) {
         const size_t smem = (size_t)kWarps * (cc.W[0] + cc.W[1] + cc.W[2]) * 4;
         if ((e = allow_smem((const void*)k_playout, 100 * 1024))) return e;

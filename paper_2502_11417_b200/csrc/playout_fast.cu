@@ -446,12 +446,12 @@ static int short_per(uint32_t n, int sms) { return n >= (uint32_t)sms * 8u * kSh
 
 bool short_search(uint32_t search) { return search <= kShortSearch; }
 
-cudaError_t launch_playout_many(const TraceDev& tr, const GroupConst* gc, const int32_t* knots, uint32_t k0, TimelineRec rec, const ShortMany& many, int sms,
+cudaError_t launch_playout_many(const TraceDev& tr, const GroupConst* gc, const int32_t* knots, uint32_t k0, TimelineRec rec, const ShortMany& many, bool early, int sms,
                                 cudaStream_t st) {
     const int per = short_per(tr.n, sms);
     const uint32_t per_block = (uint32_t)(kShortThreads * per);
     return launch_after(k_playout_short<true>, dim3((tr.n + per_block - 1) / per_block, many.count), kShortThreads, 0, st, tr, gc, ClassConst{}, knots, k0,
-                        rec, per, false, many);
+                        rec, per, early, many);
 }
 
 cudaError_t launch_playout_exact(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots,

@@ -44,11 +44,12 @@ template <int PLAY, bool SMALL>
 __global__ void __launch_bounds__(kFreeWarps * 32, kFreeBlocks)
 k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_constant__ ClassConst cc,
                const int32_t* __restrict__ knots, uint32_t k0, TimelineRec rec, const __grid_constant__ FreeMore more,
-               uint32_t* __restrict__ ticket, uint32_t batches, uint32_t size, bool early) {
+               uint32_t* __restrict__ ticket, uint32_t batches, uint32_t size, bool beside, bool early) {
     constexpr bool BOTH = PLAY == P_BOTH;
     extern __shared__ __align__(16) uint32_t s_win[];         // per warp: [W0 + W1][kCols] counters
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    grid_dependency_wait();
+    // (beside the play-out of other classes, which began when the load was complete: the last block waits for it)
+    if (!beside || blockIdx.x == gridDim.x - 1) grid_dependency_wait();
     if (early) let_next_start();
     const int W0 = cc.W[0], W1 = cc.W[1], WW = W0 + W1;
     uint32_t* win = s_win + wib * (WW * kCols);
@@ -171,7 +172,7 @@ k_playout_free(TraceDev tr, const GroupConst* __restrict__ gcs, const __grid_con
 DBG_TRANSLATION_UNIT()
 
 cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const ClassConst& cc, const int32_t* knots, uint32_t k0, TimelineRec rec,
-                                const FreeMore& more, uint32_t* ticket, const uint32_t* grp_n, bool early, int sms, cudaStream_t st) {
+                                const FreeMore& more, uint32_t* ticket, const uint32_t* grp_n, bool beside, bool early, int sms, cudaStream_t st) {
     // as many warps to a block as the windows leave room for (wide jitter: up to 27 KB of counters a stream and warp)
     const size_t per_warp = (size_t)(cc.W[0] + cc.W[1]) * kCols * 4;
     const uint32_t warps = std::max<uint32_t>(1u, std::min<uint32_t>(kFreeWarps, (uint32_t)(100 * 1024 / per_warp)));
@@ -199,7 +200,7 @@ cudaError_t launch_playout_free(const TraceDev& tr, const GroupConst* gc, const 
     cudaError_t e;
     if ((e = allow_smem((const void*)kernel, 227 * 1024))) return e;
     const uint32_t blocks = std::min<uint32_t>((batches + warps - 1) / warps, at_once / warps);
-    return launch_after(kernel, blocks, warps * 32, smem, st, tr, gc, cc, knots, k0, rec, more, ticket, batches, size, early);
+    return launch_after(kernel, blocks, warps * 32, smem, st, tr, gc, cc, knots, k0, rec, more, ticket, batches, size, beside, early);
 }
 
 }  // namespace disco
