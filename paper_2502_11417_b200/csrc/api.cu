@@ -237,7 +237,7 @@ int check_profiles(const disco_trace_desc_t* d, std::vector<GroupConst>* out) {
 // How a load's inputs reach the ingestion kernel.
 enum Inputs { IN_DEVICE, IN_COPIED, IN_PLACE, IN_PACKED };
 
-bool large_load(uint32_t n, int G) { return n >= kLargeMinN && n <= kLargeMaxN && G <= kLargeMaxGroups; }
+bool large_load(uint32_t n, int G, Inputs in) { return n >= (in == IN_PLACE ? kLargeMinInPlace : kLargeMinN) && n <= kLargeMaxN && G <= kLargeMaxGroups; }
 
 cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool has_dp) {
     const size_t N = n ? n : 1, N4 = N + 3;
@@ -262,7 +262,7 @@ cudaError_t reserve_trace(disco_ctx* c, uint32_t n, Inputs in, bool has_sp, bool
         o_in[0] = lay.take(n > kPackInPlace ? packed_bytes(n) : 0);
     }
     const size_t without = lay.bytes;
-    const bool large = large_load(n, G);
+    const bool large = large_load(n, G, in);
     LargeLoad& lg = c->large;
     std::memset(&lg, 0, sizeof lg);
     if (large) {

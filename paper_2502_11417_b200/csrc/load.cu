@@ -1,4 +1,4 @@
-// Trace ingestion on the device in one kernel, for the traces that load_once.cu and load_large.cu do not take (1.2 to 3.5 million
+// Trace ingestion on the device in one kernel, for the traces that load_once.cu and load_large.cu do not take (1.2 to 2.2 million
 // requests, more than seven groups, beyond 2^24 requests, or without room for load_large.cu's buckets), and the sort of as many
 // ticks: tick conversion and validation, per-group prompt-length histogram, internal request order (by group, then by prompt
 // length), sort of the server-TTFT ticks (the empirical F of Algorithm 1), cumulative input-token mass (Eq. 3) and the quantile
@@ -18,7 +18,7 @@
 //
 // Bound: latency up to some 10^5 requests, then scattered stores: the columns are read twice (once when they are in host memory:
 // then the first pass leaves a copy), 20 bytes a request are written to scattered places, the ticks are read and written once
-// more.  2 million requests in one group: 84 us, 3 million 120, a million in twenty groups 115.  From 3.5 million on load_large.cu is
+// more.  2 million requests in one group: 84 us, 3 million 120, a million in twenty groups 115.  From 2.2 million on load_large.cu is
 // the faster one.  (The 64 registers that 1,024 threads leave spill 64 bytes.)
 #include <algorithm>
 #include <cstdlib>

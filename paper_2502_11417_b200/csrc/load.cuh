@@ -44,7 +44,8 @@ __host__ __device__ constexpr uint32_t sort_windows(uint32_t n, int G) { return 
 
 // Large traces are placed in two steps, by way of buckets (load_large.cu).
 constexpr uint32_t kLargeMaxN = 1u << 24;     // (beyond, the tables of buckets no longer fit in a block's shared memory)
-constexpr uint32_t kLargeMinN = 3500000;    // (where it becomes the faster one: see load_large.cu)
+constexpr uint32_t kLargeMinN = 2200000;    // (where it becomes the faster one: see load_large.cu)
+constexpr uint32_t kLargeMinInPlace = 3000000;   // ... where columns are read in place, over the link
 constexpr int kLargeMaxGroups = 7;            // groups whose counters fit there
 constexpr uint32_t kTickShare = 8192;         // ticks to a bucket, at most
 // Records to a bucket: 2,048, or as many as leave 1,024 buckets.  Ticks: so many that the multiprocessors sort equally many buckets.

@@ -456,3 +456,14 @@ def test_grids_beside_each_other(n, shape):
     full_parity(w, of(5.0, 1) + of(6.0, 5) + of(40.0, 2), select=False, tag=f"{n} {shape}")
     by_budget = [synth.policy(b, r_c=7.0, flags=PACED, mig_threshold=1e-6 * k) for k, b in enumerate(synth.budget_grid(9))]
     full_parity(w, of(40.0, 1) + by_budget + of(6.0, 1) + of(5.0, 3), select=False, tag=f"{n} {shape} and one apart")
+
+
+@pytest.mark.parametrize("n,shape,kind,where", [(2_199_999, (3, 2), "spread", "device"), (2_200_000, (3, 2), "spread", "device"), (2_200_001, (1, 1), "one", "pageable"),
+                                                (2_300_017, (1, 7), "ties", "unaligned"), (2_999_999, (1, 1), "spread", "pinned"), (3_000_000, (1, 2), "dense", "pinned")])
+def test_where_buckets_begin(n, shape, kind, where):
+    test_large_traces_are_placed_by_way_of_buckets(n, shape, kind, where)
+
+
+@pytest.mark.parametrize("shape,kind", [((1, 1), "10ms"), ((3, 2), "pairs"), ((3, 2), "narrow")])
+def test_smallest_traces_by_way_of_buckets_by_a_coarse_clock(shape, kind):
+    test_large_traces_by_a_coarse_clock(2_200_000, shape, kind)
