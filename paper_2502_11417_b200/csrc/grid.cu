@@ -16,7 +16,7 @@
 // The last run of a segment and the first are swept together: where the device runs alone, or where the common w_tail covers a
 // request (S <= w_tail: the server answers alone), the first run adds little to what is read.  The requests that w_tail does not
 // cover (at most a share alpha of them) go on a list of the block's, swept again for the first run, and once for each of the
-// columns that wait longer (budgets below the tail ratio).
+// columns that wait longer (budgets below the tail ratio).  With windows Algorithm 2's segments are swept run by run.
 // Small traces leave a run few requests: there a lane takes a request with all its runs (see below).
 //
 // The rows differ in the hand-off alone: a race won by the endpoint that may hand over migrates in the rows whose
@@ -52,7 +52,7 @@ constexpr uint32_t kNoPolicy = 0xFFFFFFFFu;
 static_assert(kNBins % 32 == 0 && kNBins / 32 < 32, "a bit for each group of bins");
 
 // Blocks to a multiprocessor by the rows a kernel is built for: as many as its registers allow with few spills (with windows up to
-// 76 bytes, without up to 20).
+// 44 bytes, without up to 20).
 enum GridMode { M_RACES = 0, M_WAITS, M_JOINED };
 __host__ __device__ constexpr int blocks_for(int rows, bool wide, int mode) { return mode == M_JOINED ? (rows <= 2 ? 4 : 3) : rows <= (wide ? 1 : 2) ? 4 : rows <= 4 || !wide ? 3 : 2; }
 // The rows of the kernel that takes a slab of T.
