@@ -16,8 +16,8 @@
 // so do k_order behind k_ticks and k_sort behind k_order, each of which waits for the kernel in front before it ends (a step of 4 M requests
 // 297 -> 283 us, of 16 M in six groups 1,090 -> 1,057: the last tiles and buckets of a kernel leave most multiprocessors idle).
 //
-// Bound: memory and shared-memory atomics.  16 M requests in six groups: k_load 855 us, these 550 (count 58, plan 13, records 149,
-// ticks 109, order 105, sort 114; 520 as they overlap); 4 M in one group 213 and 143, in six 209 and 170.  Below, k_load's scattered stores
+// Bound: memory and shared-memory atomics.  16 M requests in six groups: k_load 855 us, these, one after another, 550 (count 58, plan 13, records 149,
+// ticks 109, order 105, sort 114; 527 as they overlap); 4 M in one group 213 and 138.  Below, k_load's scattered stores
 // still meet their lines in L2, and it has one launch: steps with either, in one group, 1.5 M requests 177 us and 178, 2 M 199 and 199,
 // 2.5 M 228 and 216, 3 M 261 and 231, 3.4 M 292 and 234; in six 205 and 208, 234 and 229, 268 and 261, 297 and 278, 338 and 290; from pageable
 // arrays 2 M 738 and 737, 3.4 M 1,142 and 1,107.  From page-locked columns, which k_count reads, 2 M 767 and 808, 3 M 1,100 and 1,098, 3.4 M 1,244
