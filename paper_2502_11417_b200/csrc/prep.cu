@@ -118,6 +118,7 @@ k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __re
     constexpr uint32_t kVecs = sizeof(PolicyIn) / 16, kKindVecs = sizeof(PolicyKind) / 16, kNear = kPrepThreads / kKindVecs;
     static_assert(sizeof(PolicyIn) % 16 == 0 && sizeof(PolicyKind) % 16 == 0 && kPrepWarps * kVecs <= kPrepThreads, "a vector a thread");
     __shared__ uint4 s_pol[kPrepWarps * kVecs], s_kind[kPrepThreads];     // the block's policies, and the first kinds
+    __shared__ uint4 s_far[kPrepWarps * kKindVecs];                       // the warps' kinds that are not among these
     auto table = [&](uint32_t i) {
         if constexpr (BYTES != 0) return given.v[i];
         else return static_cast<const uint4*>(in.host)[i];
@@ -137,25 +138,26 @@ k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __re
     if (has_kind) s_kind[threadIdx.x] = kind;
     for (uint32_t i = vec_at; i < in.vecs; i += all) static_cast<uint4*>(in.device)[i] = i == vec_at ? vec : table(i);
     __syncthreads();
-    if (BYTES == 0 && threadIdx.x == 0) {
-        __threadfence();
-        if (atomicInc(in.left, gridDim.x - 1u) == gridDim.x - 1u) { __threadfence_system(); *in.read = in.turn; }
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, g = (int)(idx % (uint32_t)G);
+    const uint32_t p = idx / (uint32_t)G;
+    const bool own = idx < pairs && DBG_OK(g, G, DBG_K_PREP, DBG_GROUP) && DBG_OK(p - p0, kPrepWarps, DBG_K_PREP, DBG_POLICY) &&
+                     DBG_OK(reinterpret_cast<const PolicyIn*>(s_pol)[p - p0].kind, in.kinds, DBG_K_PREP, DBG_TABLE);
+    const PolicyKind* pk = nullptr;
+    if (own) {
+        const uint32_t k = reinterpret_cast<const PolicyIn*>(s_pol)[p - p0].kind;
+        pk = reinterpret_cast<const PolicyKind*>(k < kNear ? s_kind + k * kKindVecs : s_far + wi * kKindVecs);
+        if (k >= kNear && lane < (int)kKindVecs) s_far[wi * kKindVecs + lane] = table(P * kVecs + k * kKindVecs + lane);
+        __syncwarp();
     }
-    if (idx < pairs) {
-        const uint32_t p = idx / (uint32_t)G;
-        const int g = (int)(idx - p * (uint32_t)G);
-        if (DBG_OK(g, G, DBG_K_PREP, DBG_GROUP) && DBG_OK(p - p0, kPrepWarps, DBG_K_PREP, DBG_POLICY))
-        {
-            const PolicyIn pi = reinterpret_cast<const PolicyIn*>(s_pol)[p - p0];
-            PolicyKind pk;
-            if (pi.kind < kNear) pk = reinterpret_cast<const PolicyKind*>(s_kind)[pi.kind];
-            else {
-#pragma unroll
-                for (uint32_t k = 0; k < kKindVecs; ++k) reinterpret_cast<uint4*>(&pk)[k] = table(P * kVecs + pi.kind * kKindVecs + k);
-            }
-            prep_pair(pi, pk, p, g, P, gc, cum_mass, cnt, sorted, grp_off, prep);
+    if constexpr (BYTES == 0) {
+        // Behind the last of the block's reads: the host may write the memory anew, or give it back, once all blocks have been here.
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            if (atomicInc(in.left, gridDim.x - 1u) == gridDim.x - 1u) { __threadfence_system(); *in.read = in.turn; }
         }
     }
+    if (own) prep_pair(reinterpret_cast<const PolicyIn*>(s_pol)[p - p0], *pk, p, g, P, gc, cum_mass, cnt, sorted, grp_off, prep);
     // (the last blocks first: the others have clearing and preparing to do)
     for (uint32_t i = (gridDim.x - 1u - blockIdx.x) * kPrepThreads + threadIdx.x; i < in.n_chunks[0] + in.n_chunks[1]; i += all) {
         const int w = i >= in.n_chunks[0];

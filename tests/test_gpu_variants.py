@@ -430,6 +430,39 @@ def test_policies_of_many_kinds(kinds):
     full_parity(w, pols + pols[::2], select=False, tag=f"{kinds}")
 
 
+def test_evaluations_in_a_row_of_many_kinds():
+    # Tables read from page-locked memory, with more kinds than a block of the preparation keeps: the call behind writes that memory
+    # again (or gives it back for a larger piece) as soon as the last of it has been read.  Nothing is waited for between the calls.
+    import torch
+    from oracle import Oracle
+    from paper_2502_11417_b200 import Trace
+    from paper_2502_11417_b200.api import policy_array
+    from parity import check_pairs, check_stats
+    w = synth.tiny_workload(167, 300, n_servers=2, n_devices=3, max_prompt=300, max_out=30, device_dearer=True)
+    t, orc = Trace.from_workload(w), Oracle.from_workload(w)
+    cnt = np.stack([t.group_tables(g)[0] for g in range(t.n_groups)])
+    ticks = torch.cat([t.sorted_ticks_device(g) for g in range(t.n_groups)])
+    sizes = cnt.sum(axis=1).astype(np.uint64)
+    kind = lambda k, e: dict(alpha=0.01 + 0.007 * ((k * (3 + 2 * e)) % 131), expected_len=(k + e) % 2 * 20)
+    sets = [[synth.policy(0.001 * ((k * 7 + e) % 997), **kind(k, e)) for k in range(n)][::1 - 2 * (e % 2)] for e, n in enumerate([900, 700, 1300, 900, 1800, 1000])]
+    arrays, outs = [policy_array(p) for p in sets], [t.alloc_pair_outputs(len(p)) for p in sets]
+    again = [t.alloc_pair_outputs(len(p)) for p in sets]
+    for tables in (False, True):
+        torch.cuda.synchronize()
+        for a, o in zip(arrays, again if tables else outs):
+            t.eval_policies(a, w.seed, o)
+            if tables:
+                t.set_group_tables(cnt, ticks, sizes)
+    t.eval_policies(arrays[-1], w.seed)
+    stats = t.reduce_stats()
+    for e, p in enumerate(sets):
+        want, pairs = orc.eval(p, w.seed, pairs=True)
+        check_pairs(outs[e], pairs, tag=f"evaluation {e}")
+        check_pairs(again[e], pairs, tag=f"evaluation {e} in front of tables")
+    check_stats(stats, want, t.histograms, "the last")
+    t.close()
+
+
 @pytest.mark.parametrize("n", [1, 256, 148 * 256, 148 * 256 + 1, 100_001])
 @pytest.mark.parametrize("shape,policies", [((1, 1), 3), ((2, 3), 33), ((3, 3), 200)])
 def test_pairs_in_whole_rounds_of_blocks(n, shape, policies):
