@@ -911,8 +911,13 @@ k_grid(const __grid_constant__ Args a) {
                     }
                     run(from, to, w, false, push, q0, q1, false);
                 } else if (sm.n_list == 0) break;
-                if (done || (push && sm.n_list > (uint32_t)(kListCap - kListStep))) {
-                    const uint32_t k = sm.n_list;                     // (barriers inside run: all threads agree)
+                bool full = done;
+                if (push) {                                           // all threads see the same, and only then may the next run add to it
+                    full = sm.n_list > (uint32_t)(kListCap - kListStep);
+                    __syncthreads();
+                }
+                if (full) {
+                    const uint32_t k = sm.n_list;                     // (nobody adds to it from here to the runs' end)
                     __syncthreads();
                     if (threadIdx.x == 0) sm.n_list = 0;
                     for (int p = -1; p < n_low; ++p)                  // the common wait's totals go, each column's own come

@@ -430,6 +430,24 @@ def test_policies_of_many_kinds(kinds):
     full_parity(w, pols + pols[::2], select=False, tag=f"{kinds}")
 
 
+@pytest.mark.parametrize("rate", [5.0, 40.0])
+@pytest.mark.parametrize("rows", [1, 2])
+def test_lists_that_fill_within_a_segment(rate, rows):
+    # Algorithm 2 with a tail ratio so large that most requests of a segment wait longer in its first columns than the common wait
+    # covers: chunks of some 4,800 requests and a few prompt lengths, whose lists are added to by run after run, fill and begin anew;
+    # without windows and (a reader faster than either endpoint) with
+    from oracle import Oracle
+    from paper_2502_11417_b200 import Trace
+    from parity import check_stats
+    n = 1_400_001
+    w = synth.tiny_workload(173, n, max_prompt=4, max_out=6, device_dearer=True)
+    pols = [synth.policy(b, alpha=a, r_c=rate, flags=PACED, mig_threshold=1e-3 * k) for a in (0.55, 0.6, 0.65, 0.7) for b in (0.2, 0.5, 0.9) for k in range(rows)]
+    tr = Trace.from_workload(w)
+    tr.eval_policies(pols, w.seed)
+    check_stats(tr.reduce_stats(), Oracle.from_workload(w).eval(pols, w.seed)[0], tr.histograms, f"{rate} {rows}")
+    tr.close()
+
+
 def test_evaluations_in_a_row_of_many_kinds():
     # Tables read from page-locked memory, with more kinds than a block of the preparation keeps: the call behind writes that memory
     # again (or gives it back for a larger piece) as soon as the last of it has been read.  Nothing is waited for between the calls.
