@@ -739,7 +739,6 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     std::vector<uint32_t> tab;                     // lists of policy indices, one after the other
     tab.reserve((size_t)4 * P + 64);
     std::vector<Slab> slabs;
-    std::vector<uint32_t> mixed_pols;              // per slab: where its policies are listed for the pair kernel (mixed slabs)
     struct ClassLists { size_t all, n_all, ext, n_ext; };
     std::vector<ClassLists> lists(classes.size());
     bool any_mixed = false, any_pairs = false;
@@ -811,7 +810,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 return sl;
             };
             // closes a slab of the columns [c0, c1) of `cells` (T policies each, kNone for none)
-            auto close = [&](Slab sl, size_t c0, size_t c1, uint32_t listed) {
+            auto close = [&](Slab sl, size_t c0, size_t c1) {
                 const size_t T = (size_t)sl.T;
                 sl.K = (int32_t)(c1 - c0);
                 sl.cols = (uint32_t)tab.size();
@@ -824,7 +823,6 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 tab.insert(tab.end(), cells.begin() + c0 * T, cells.begin() + c1 * T);
                 sl.policies = (uint32_t)((c1 - c0) * T - std::count(cells.begin() + c0 * T, cells.begin() + c1 * T, kNone));
                 slabs.push_back(sl);
-                mixed_pols.push_back(listed);
             };
             if (n_t > 1 && 2 * n_p <= n_b * n_t) {
                 // Most (budget, overhead) combinations are no policy: a column per policy instead, and what the overheads
@@ -834,13 +832,11 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 for (size_t x0 = 0; x0 < n_p; x0 += kGridCols) {
                     const size_t x1 = std::min(n_p, x0 + (size_t)kGridCols);
                     Slab sl = open(1, true);
-                    const uint32_t listed = (uint32_t)tab.size();
-                    tab.insert(tab.end(), cells.begin() + x0, cells.begin() + x1);
                     sl.theta[0] = sl.theta[1] = theta_of(cells[x0]);
                     for (size_t x = x0; x < x1; ++x) {
                         sl.theta[0] = std::min(sl.theta[0], theta_of(cells[x])); sl.theta[1] = std::max(sl.theta[1], theta_of(cells[x]));
                     }
-                    close(sl, x0, x1, listed);
+                    close(sl, x0, x1);
                     any_mixed = any_pairs = true;
                 }
                 continue;
@@ -868,30 +864,46 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
                 used.assign(n_b * kGridRows, 0);
                 for (size_t x = 0; x < n_p; ++x)
                     if (cell_of[x] != kNone) cells[(wide[cell_of[x] / kGridRows] + used[cell_of[x]]++) * T + cell_of[x] % kGridRows] = gr.pols[x];
-                for (size_t c0 = 0; c0 < cols; c0 += kGridCols) close(sl, c0, std::min(cols, c0 + (size_t)kGridCols), 0u);
+                for (size_t c0 = 0; c0 < cols; c0 += kGridCols) close(sl, c0, std::min(cols, c0 + (size_t)kGridCols));
             }
         }
     }
 
-    // ---- the difference tables of the slabs, laid out batch by batch: a batch's slabs have like numbers of rows, and windows or
-    //      none.  Small ones lie side by side and are cleared by k_prep; beyond 64 MB a batch's tables are cleared, filled,
+    // ---- requests run by run or side by side: slab by slab, and within a wave's slabs with windows or without those of one way together
+    int groups = 0;                                // that have requests
+    for (int g = 0; g < G; ++g) groups += rb.ng[g] != 0;
+    auto joins = [&](const Slab& sl) {
+#ifdef DISCO_DEBUG
+        if (std::getenv("DISCO_DEBUG_RUNS")) return false;
+#endif
+        return !wide_class(sl.cls) && grid_joins(n, groups, sl.K, sl.T);
+    };
+    for (size_t x = 0, end; x < slabs.size(); x = end) {
+        auto like = [&](const Slab& sl) { return sl.cls / wave == slabs[x].cls / wave && wide_class(sl.cls) == wide_class(slabs[x].cls); };
+        for (end = x + 1; end < slabs.size() && like(slabs[end]);) ++end;
+        std::stable_partition(slabs.begin() + x, slabs.begin() + end, [&](const Slab& sl) { return !joins(sl); });
+    }
+
+    // ---- the difference tables of the slabs, laid out batch by batch: a batch's slabs have like numbers of rows, windows or
+    //      none, and go one way.  Small ones lie side by side and are cleared by k_prep; beyond 64 MB a batch's tables are cleared, filled,
     //      added up and then belong to the next batch
-    struct Batch { size_t first, count, wave; int T; bool wide; uint64_t ttft, tbt, sums, at; };
+    struct Batch { size_t first, count, wave; int T; bool wide, joined; uint64_t ttft, tbt, sums, at; };
     std::vector<Batch> batches;
     auto batch_bytes = [&](const Batch& b) { return (b.sums * 8 + b.tbt * (b.wide ? 8 : 4) + b.ttft * 4 + 15) / 16 * 16; };
-    size_t most_slabs = 1;
+    size_t most_slabs = 0;                         // of a batch that goes run by run
+    int tallest = 1;
     for (size_t x = 0; x < slabs.size(); ++x) {
         Slab& sl = slabs[x];
-        const bool wide_tables = wide_class(sl.cls);
+        const bool wide_tables = wide_class(sl.cls), joined = joins(sl);
         if (batches.empty() || batch_bytes(batches.back()) > (256ull << 20) || grid_rows(batches.back().T) != grid_rows(sl.T) || sl.mixed ||
-            slabs[x - 1].mixed || batches.back().wave != sl.cls / wave || batches.back().wide != wide_tables)
-            batches.push_back(Batch{x, 0, sl.cls / wave, 1, wide_tables, 0, 0, 0, 0});
+            slabs[x - 1].mixed || batches.back().wave != sl.cls / wave || batches.back().wide != wide_tables || batches.back().joined != joined)
+            batches.push_back(Batch{x, 0, sl.cls / wave, 1, wide_tables, joined, 0, 0, 0, 0});
         Batch& b = batches.back();
         sl.ttft = b.ttft; sl.tbt = b.tbt; sl.sums = b.sums;
         b.ttft += grid_ttft_words(sl.K); b.tbt += grid_tbt_words(sl.K, sl.T); b.sums += grid_sum_words(sl.K, sl.T, G);
         ++b.count;
         b.T = std::max(b.T, sl.T);
-        most_slabs = std::max(most_slabs, b.count);
+        if (!joined) { most_slabs = std::max(most_slabs, b.count); tallest = std::max(tallest, sl.T); }
     }
     uint64_t grid_bytes = 0, all_bytes = 0;
     for (Batch& b : batches) { b.at = all_bytes; all_bytes += batch_bytes(b); grid_bytes = std::max(grid_bytes, batch_bytes(b)); }
@@ -904,8 +916,6 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     //      budgets by 8 overheads 369 us either way, under 16 by 2 218 instead of 205, in one group under 64 budgets 139
     //      instead of 133, a million 34 instead of 30)
     const uint32_t sms = (uint32_t)c->sms, kMaxChunk = 65280;
-    int tallest = 1;
-    for (const Slab& sl : slabs) tallest = std::max(tallest, sl.T);
     auto chunk_size = [&](size_t want, uint32_t least) {
         const size_t ch = ((N1 + want - 1) / want + 255) / 256 * 256;
         return (uint32_t)std::min<size_t>(std::max<size_t>(ch, least), kMaxChunk);
@@ -926,15 +936,9 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         tables.chunk_len[which] = CH; tables.n_chunks[which] = count;
     };
     const size_t at_once = (size_t)sms * grid_blocks_per_sm(tallest);
+    if (most_slabs) plan_chunks(CHUNKS_RUNS, chunk_size(std::max<size_t>(2 * at_once / std::min<size_t>(most_slabs, 4), 1), 256));
     // (requests side by side: a chunk is a thread's request or a few)
-    int widest = 1, groups = 0;
-    for (const Slab& sl : slabs) widest = std::max(widest, sl.K);
-    for (int g = 0; g < G; ++g) groups += rb.ng[g] != 0;
-    bool joined = grid_joins(n, groups, widest, tallest);
-#ifdef DISCO_DEBUG
-    if (std::getenv("DISCO_DEBUG_RUNS")) joined = false;
-#endif
-    plan_chunks(0, joined && !stored ? chunk_size((size_t)sms * 8, 256) : chunk_size(std::max<size_t>(2 * at_once / std::min<size_t>(most_slabs, 4), 1), 256));
+    if (std::any_of(batches.begin(), batches.end(), [](const Batch& b) { return b.joined; })) plan_chunks(CHUNKS_JOINED, chunk_size((size_t)sms * 8, 256));
     if (any_pairs) {
         // of the pair kernel, whose blocks (a chunk and 32 policies each) take a multiprocessor's shared memory: the fewest whole rounds
         // of them, where a block costs as much as some 800 requests besides its own.  (300,000 requests in six groups under 32
@@ -954,7 +958,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             if (ch > kMaxChunk || rounds * (ch + 800) >= least) continue;
             best = (uint32_t)ch; least = rounds * (ch + 800);
         }
-        plan_chunks(1, best);
+        plan_chunks(CHUNKS_PAIRS, best);
     }
 
     // ---- device memory: what must be clear comes first and together -- the work counters and tickets, the difference
@@ -987,7 +991,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const size_t table_bytes = (size_t)P * sizeof(PolicyIn) + kinds.size() * sizeof(PolicyKind) + (classes.size() * sizeof(ClassConst) + 15) / 16 * 16 +
                                (tab.size() * 4 + 15) / 16 * 16 + (slabs.size() * sizeof(Slab) + 15) / 16 * 16;
     const size_t o_tables = lay.take(table_bytes);
-    const size_t o_chunks[2] = {lay.take(tables.n_chunks[0] * sizeof(Chunk)), lay.take(tables.n_chunks[1] * sizeof(Chunk))};
+    size_t o_chunks[kChunkTables];
+    for (int k = 0; k < kChunkTables; ++k) o_chunks[k] = lay.take(tables.n_chunks[k] * sizeof(Chunk));
     if ((e = c->eval_mem.reserve(lay.bytes)) == cudaErrorMemoryAllocation && wave > 1) {
         cudaGetLastError();                                          // (again in smaller waves, which leave more room)
         c->rec_too_much = wave * rec_stride;
@@ -1029,13 +1034,13 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
     const ClassConst* d_classes = (const ClassConst*)put(classes.data(), classes.size() * sizeof(ClassConst));
     const uint32_t* d_tab = (const uint32_t*)put(tab.data(), tab.size() * 4);
     const Slab* d_slabs = (const Slab*)put(slabs.data(), slabs.size() * sizeof(Slab));
-    const Chunk *d_chunks = (const Chunk*)(mem + o_chunks[0]), *d_pair_chunks = (const Chunk*)(mem + o_chunks[1]);
+    const Chunk* d_pair_chunks = (const Chunk*)(mem + o_chunks[CHUNKS_PAIRS]);
     if (off / 16 > 0xFFFFFFFFull) return fail(DISCO_ENOMEM, "the tables of the policies are too large");
 
     // ---- Algorithms 1-3 for every (group, policy)
     tables.host = sp; tables.device = dt; tables.vecs = (uint32_t)(off / 16); tables.skip = n_beta ? 0u : policy_vecs;
     tables.kinds = (uint32_t)kinds.size();
-    for (int k = 0; k < 2; ++k) tables.chunks[k] = (Chunk*)(mem + o_chunks[k]);
+    for (int k = 0; k < kChunkTables; ++k) tables.chunks[k] = (Chunk*)(mem + o_chunks[k]);
     tables.left = &c->z->tables_left; tables.read = c->stage_read; tables.turn = c->stage_turn + 1;
     CU(launch_prep(P, G, c->d_gc.as<GroupConst>(), c->cum_mass.as<int64_t>(),
                    c->cnt, c->F_sorted, c->F_off, c->d_prep.as<Prep>(), tables, mem, clear_apart ? 0 : clear_bytes, c->sms, st));
@@ -1104,9 +1109,10 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             for (size_t k = next; k < end; ++k) {
                 const Batch& b = batches[k];
                 if (!side_by_side && k != 0) CU(cudaMemsetAsync((char*)c->d_grid.p + b.at, 0, batch_bytes(b), st));
-                CU(launch_grid(tr, gc, d_classes, prep, P, d_slabs + b.first, (uint32_t)b.count, b.T, b.wide, d_tab, d_chunks, tables.n_chunks[0], rec,
+                const int which = b.joined ? CHUNKS_JOINED : CHUNKS_RUNS;
+                CU(launch_grid(tr, gc, d_classes, prep, P, d_slabs + b.first, (uint32_t)b.count, b.T, b.wide, d_tab, tables.chunks[which], tables.n_chunks[which], rec,
                                rec_stride, tables_of(b), left, k0, tickets + ticket, work, k > next || (beside && ticket == 0), k + 1 < end, any_waits,
-                               joined, c->sms, st));
+                               b.joined, c->sms, st));
                 ++ticket;
             }
             for (size_t k = next; k < end; ++k) {
@@ -1116,8 +1122,8 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
             }
             if (sl.mixed) {
                 const Batch& b = batches[next];
-                CU(launch_pairs_acc(tr, gc, d_classes + sl.cls, prep, P, d_tab + mixed_pols[b.first], sl.policies, d_pair_chunks,
-                                    tables.n_chunks[1], left.list, left.count, rec_of(sl.cls), acc, h_ttft, h_tbt, work, k0,
+                CU(launch_pairs_acc(tr, gc, d_classes + sl.cls, prep, P, d_tab + sl.cells, sl.policies, d_pair_chunks,
+                                    tables.n_chunks[CHUNKS_PAIRS], left.list, left.count, rec_of(sl.cls), acc, h_ttft, h_tbt, work, k0,
                                     sl.expected_len != 0, b.wide, st));
                 g_launches += 1;
             }
@@ -1126,7 +1132,7 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
         for (size_t k = first; k < last; ++k) {
             if (!lists[k].n_ext) continue;
             CU(launch_pairs_acc(tr, gc, d_classes + k, prep, P, d_tab + lists[k].ext, (uint32_t)lists[k].n_ext,
-                                d_pair_chunks, tables.n_chunks[1], nullptr, nullptr, rec_of(k), acc, h_ttft, h_tbt,
+                                d_pair_chunks, tables.n_chunks[CHUNKS_PAIRS], nullptr, nullptr, rec_of(k), acc, h_ttft, h_tbt,
                                 work, k0, true, wide_class(k), st));
             g_launches += 1;
         }

@@ -253,17 +253,18 @@ struct DbgRegistrar { explicit DbgRegistrar(cudaError_t (*r)(int32_t*)) { dbg_re
 // ---- launch wrappers (defined in the kernel translation units) -------------------------------------------
 // The small tables of an evaluation on their way to the device with k_prep: as its parameter up to kTablesInline bytes, beyond
 // it reads them in pinned host memory.
-constexpr size_t kTablesInline = 28672;      // (a launch takes 32,764 bytes of parameters, the chunk plans 2,048)
+constexpr size_t kTablesInline = 28672;      // (a launch takes 32,764 bytes of parameters, the chunk plans 3,072)
 struct ChunkPlan { uint32_t first, start, end; int32_t g; };     // a group's chunks: number of the first, requests [start, end)
+enum { CHUNKS_RUNS, CHUNKS_PAIRS, CHUNKS_JOINED, kChunkTables };   // of the grid kernel run by run, of the pair kernel, of the grid kernel side by side
 struct TablesIn {
     const void* host;            // the policies come first, then their kinds; room for kTablesInline bytes where they go as a parameter
     void* device;
     uint32_t vecs, skip;         // of 16 bytes; how many of them (policies and kinds) no kernel behind needs
     uint32_t kinds;
-    // chunk tables that k_prep writes out, of the grid kernel and of the pair kernel, group by group
-    ChunkPlan plan[2][kMaxGroups];
-    uint32_t n_plan[2], chunk_len[2], n_chunks[2];
-    Chunk* chunks[2];
+    // chunk tables that k_prep writes out, group by group
+    ChunkPlan plan[kChunkTables][kMaxGroups];
+    uint32_t n_plan[kChunkTables], chunk_len[kChunkTables], n_chunks[kChunkTables];
+    Chunk* chunks[kChunkTables];
     // in pinned host memory only
     uint32_t* left;              // device word, zero; blocks that have read their share (zero again when all have)
     volatile uint32_t* read;     // pinned host word: set to `turn` once all have

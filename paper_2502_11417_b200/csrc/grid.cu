@@ -28,6 +28,7 @@
 // each run and every row's sums in registers (122 of them, two blocks to a multiprocessor), 247 now (80, three); 5 M under 40 by 8
 // 113 -> 85; a million in one group under 256 by 4 32 -> 28.  (Kernels that also held the way of small traces had to spill: 283 and 99.)
 #include <algorithm>
+#include <cmath>
 #include <cstddef>
 #include <type_traits>
 
@@ -1152,11 +1153,16 @@ cudaError_t launch_rows(const Args& a, bool wide, int mode, int sms, cudaStream_
 
 DBG_TRANSLATION_UNIT()
 
-// Side by side or run by run: the first takes some 0.1 us for a thousand requests, the second a run's latency for every threshold of every
-// group.  (us, run by run and side by side: one group, 150,000 requests under 64 10 and 11, 256 by 4 24 and 15, 400,000 21 and 25 under 256;
-// six groups, 60,000 under one 12 and 9, 150,000 under 16 by 2 23 and 20, under 64 45 and 22, 400,000 42 and 43, under 64 by 4 59 and 46,
-// a million under 256 125 and 117, under 128 by 8 116 and 126.)
-bool grid_joins(uint32_t n, int groups, int K, int T) { return n <= (80000.0 + 650.0 * K * groups) * (1.0 + T / 16.0); }
+// Side by side or run by run.  Run by run a threshold of a group costs a run's latency, in the chunks that it falls into; side by side the
+// requests add to the same rows of the tables, two runs each (under one policy setting one), and the fewer columns there are the more
+// of them meet.  (Evaluation and reduction, us, run by run and side by side: one group, 60,000 requests under 2 policies 31 and 40, under 4 34 and 36,
+// 130,000 under 64 40 and 41, 220,000 under 256 62 and 58, 400,000 63 and 68; six groups, 60,000 under 2 36 and 49, under one 80,000 37 and 39,
+// 130,000 under 16 51 and 47, 220,000 53 and 55, 400,000 under 64 75 and 77, under 128 113 and 91, 550,000 101 and 117, 750,000 under 256 175 and 142,
+// 1.3 million 194 and 216, under 16 by 8 170,000 72 and 64, 400,000 74 and 86, under 128 by 8 750,000 174 and 172.  Up to 15 % between the GPUs.)
+// It is asked slab by slab: a narrow grid beside a wide one goes its own way (six groups, a million requests under 256 by 4, and sixteen times 2 by 4
+// of other expected lengths, 779 us all side by side, now 484; under 256 by 4 and one 300, now 248; one group, 150,000 under 128 by 8 and eight
+// times 4 164, now 141).
+bool grid_joins(uint32_t n, int groups, int K, int T) { return n <= (K == 1 ? 70000.0 : 12000.0 * std::pow((double)K * groups, 0.6)) * (1.0 + T / 16.0); }
 uint64_t grid_ttft_words(int K) { return (uint64_t)K * kNBins; }
 uint64_t grid_tbt_words(int K, int T) { return (uint64_t)K * T * kNBins; }
 uint64_t grid_sum_words(int K, int T, int G) { return (uint64_t)G * K * sum_fields(T); }
@@ -1171,7 +1177,7 @@ cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassCon
     if ((uint64_t)n_chunks * n_slabs > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
     const Args a = {tr, rec, gc, rec_stride, classes, prep, P, slabs, n_slabs, tab, chunks, n_chunks, gt, left, k0, ticket,
                     (unsigned long long*)work, beside, early};
-    const int mode = joined && !wide ? M_JOINED : waits ? M_WAITS : M_RACES;
+    const int mode = joined ? M_JOINED : waits ? M_WAITS : M_RACES;
     switch (rows_for(T)) {
         case 1: return launch_rows<1>(a, wide, mode, sms, st);
         case 2: return launch_rows<2>(a, wide, mode, sms, st);

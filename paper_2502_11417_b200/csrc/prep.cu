@@ -116,6 +116,7 @@ k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __re
        Prep* __restrict__ prep, const __grid_constant__ TablesIn in, uint4* __restrict__ clear, uint32_t clear_vecs,
        const __grid_constant__ Inline<BYTES> given) {
     constexpr uint32_t kVecs = sizeof(PolicyIn) / 16, kKindVecs = sizeof(PolicyKind) / 16, kNear = kPrepThreads / kKindVecs;
+    static_assert(kChunkTables == 3, "three to write out");
     static_assert(sizeof(PolicyIn) % 16 == 0 && sizeof(PolicyKind) % 16 == 0 && kPrepWarps * kVecs <= kPrepThreads, "a vector a thread");
     __shared__ uint4 s_pol[kPrepWarps * kVecs], s_kind[kPrepThreads];     // the block's policies, and the first kinds
     __shared__ uint4 s_far[kPrepWarps * kKindVecs];                       // the warps' kinds that are not among these
@@ -159,9 +160,11 @@ k_prep(uint32_t P, int G, const GroupConst* __restrict__ gc, const int64_t* __re
     }
     if (own) prep_pair(reinterpret_cast<const PolicyIn*>(s_pol)[p - p0], *pk, p, g, P, gc, cum_mass, cnt, sorted, grp_off, prep);
     // (the last blocks first: the others have clearing and preparing to do)
-    for (uint32_t i = (gridDim.x - 1u - blockIdx.x) * kPrepThreads + threadIdx.x; i < in.n_chunks[0] + in.n_chunks[1]; i += all) {
-        const int w = i >= in.n_chunks[0];
-        const uint32_t k = w ? i - in.n_chunks[0] : i, len = in.chunk_len[w];
+    for (uint32_t i = (gridDim.x - 1u - blockIdx.x) * kPrepThreads + threadIdx.x; i < in.n_chunks[0] + in.n_chunks[1] + in.n_chunks[2]; i += all) {
+        uint32_t k = i;
+        int w = 0;
+        while (w + 1 < kChunkTables && k >= in.n_chunks[w]) k -= in.n_chunks[w++];
+        const uint32_t len = in.chunk_len[w];
         uint32_t x = 0;
         while (x + 1 < in.n_plan[w] && in.plan[w][x + 1].first <= k) ++x;
         const ChunkPlan& pl = in.plan[w][x];

@@ -34,6 +34,7 @@ std::vector<Write> pending;                     // work that a stream still hold
 struct Word { volatile uint32_t* to; uint32_t value; };
 std::vector<Word> reports;                      // words that kernels under way will write
 uint64_t device_waits = 0;
+std::map<std::string, uint64_t> launched;       // by (mangled) name
 void finish() {
     for (const Write& w : pending) std::memcpy(w.to, w.from, w.bytes);
     for (const Word& w : reports) *w.to = w.value;
@@ -46,6 +47,7 @@ const Range* range_of(const void* p) {
     return nullptr;
 }
 cudaError_t launch(const void* f, dim3 grid, void** args) {
+    ++launched[kernels[f]];
     if (kernels[f].find("k_finalize") != std::string::npos) last_stats = *(const void**)args[8];
     if (kernels[f].find("k_prep") != std::string::npos && kernels[f].find("k_prep_beta") == std::string::npos) {
         const disco::TablesIn& in = *(const disco::TablesIn*)args[8];
@@ -85,6 +87,11 @@ void fake_reset_device(void) { symbol = nullptr; locked.clear(); }
 int fake_last_words_in_place(void) { return last_words >= symbol && (const char*)last_words < (const char*)symbol + (16 << 20); }
 int fake_last_report_locked(void) { void* p; return cudaHostGetDevicePointer(&p, (void*)last_report, 0) == cudaSuccess; }
 uint64_t fake_device_waits(void) { return device_waits; }
+uint64_t fake_launched(const char* part) {      // kernels launched whose names hold `part`
+    uint64_t n = 0;
+    for (const auto& k : launched) if (k.first.find(part) != std::string::npos) n += k.second;
+    return n;
+}
 void fake_pending(void* to, const void* from, size_t bytes) { pending.push_back({to, from, bytes}); }
 
 // ---- what the library calls

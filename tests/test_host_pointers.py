@@ -275,3 +275,27 @@ for reset in (False, False, True, False, True):
     assert rc == 0, L.disco_last_error()
     assert fake.fake_last_words_in_place() and fake.fake_last_report_locked()
 """)
+
+
+@pytest.mark.parametrize("n,policies,runs,joined", [
+    (10_000, "grid(2)", 0, 1), (60_000, "grid(2)", 1, 0),             # few columns: side by side up to some 20,000 requests
+    (60_000, "grid(1)", 0, 1), (90_000, "grid(1)", 1, 0),             # one: a run a request
+    (150_000, "grid(256, 4)", 0, 1), (500_000, "grid(256, 4)", 1, 0),
+    # a wide grid and narrow ones beside it: each its own way, in the same launch where the ways are the same
+    (150_000, "grid(256, 4) + grid(2, 4, 7) + grid(2, 4, 8)", 1, 1), (150_000, "grid(2, 4, 7) + grid(256, 4) + grid(2, 4, 8)", 1, 1),
+    (10_000, "grid(2, 4, 7) + grid(256, 4) + grid(2, 4, 8)", 0, 1), (500_000, "grid(2, 4, 7) + grid(256, 4) + grid(2, 4, 8)", 1, 0)])
+def test_grids_go_run_by_run_or_side_by_side(fake, n, policies, runs, joined):
+    # k_grid<rows, windows, way>: ways 0 and 1 run by run, 2 side by side
+    _run(fake, f"""
+fake.fake_launched.restype = C.c_uint64
+ctx = C.c_void_p(None)
+keep, cols = host_columns({n})
+assert load(ctx, {n}, cols) == 0, L.disco_last_error()
+def grid(K, T=1, E=0):
+    return [synth.policy(b, mig_threshold=1e-6 * k, expected_len=E) for k in range(T) for b in synth.budget_grid(K)]
+pols = api.policy_array({policies})
+assert L.disco_eval_policies(ctx, pols, len(pols), 1, None, None) == 0, L.disco_last_error()
+rows = min(4, max(p.mig_threshold for p in pols) * 1e6 + 1)
+ways = [fake.fake_launched(b"k_gridILi%dELb0ELi%dE" % (rows, way)) for way in range(3)]
+assert (ways[0] + ways[1], ways[2]) == ({runs}, {joined}), ways
+""")
