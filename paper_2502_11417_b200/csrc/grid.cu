@@ -227,14 +227,14 @@ __device__ __forceinline__ void add_windows(const Args& a, const Ctx& c, uint32_
 // One sweep over the requests [pa, pb) of the chunk, or (list) of the block's list: what they come to when the device
 // starts after the wait w, added up in `s` and in the shared histograms.
 // SIDE: a segment's requests under its last columns, which wait 0 (`race`: there are such columns), and beside them under its first
-// ones (`side`), added up in `o` and histograms of its own: Algorithm 3's, where the device runs alone, or (S_EITHER, `waits`) Algorithm
-// 2's, which wait w: there the server alone answers the requests with S <= w, and the others go on the list.
+// ones (`side`), added up in `o` and histograms of its own: Algorithm 3's, where the device runs alone (S_DEVICE), or Algorithm 2's
+// (S_SERVER), which wait w: there the server alone answers the requests with S <= w, and the others go on the list.
 // push: requests with S > w go on the list (without a run beside).
-enum SideKind { S_NONE = 0, S_DEVICE, S_EITHER };
+enum SideKind { S_NONE = 0, S_DEVICE, S_SERVER };
 template <int NT, bool WIDE, int SIDE>
 __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (&th)[NT], Smem& sm, uint32_t* tbt, const Levels<NT>& lv,
-                                      uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, bool given_waits, bool race, bool side, Acc<NT, WIDE>& s, Side& o) {
-    const bool waits = SIDE == S_EITHER && given_waits;
+                                      uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, bool race, bool side, Acc<NT, WIDE>& s, Side& o) {
+    constexpr bool waits = SIDE == S_SERVER;
     const int lane = threadIdx.x & 31;
     // The kernel of eight rows has too few warps a multiprocessor to hide the loads' latency: there they run an iteration ahead.
     constexpr bool kAhead = NT == 8 && !WIDE;
@@ -281,7 +281,7 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
             if (WIDE && !((c.even >> stream) & 1u))
                 add_rows(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(a.rec.win[stream]) + c.win_at), c.cc->W[stream], c.cc->lo[c.g][stream], live, kk, false, tbt + NT * kNBins);
         }
-        if (SIDE == S_EITHER ? waits && side : WIDE && push) {
+        if (waits || (WIDE && push)) {
             const bool longer = valid && S > w;
             const uint32_t all = __ballot_sync(FULL, longer);
             if (all) {
@@ -858,13 +858,13 @@ k_grid(const __grid_constant__ Args a) {
             passes = 1;
         }
         // a segment's last columns, which wait 0, and beside them its first ones: the device alone
-        if (MODE == M_RACES || (WIDE && !waits)) {
+        if (MODE == M_RACES || (MODE == M_WAITS && !waits)) {
             for (int si = 0; si < n_seg; ++si) {
                 const Seg sg = sm.seg[si];
                 const bool race = (int)sg.k2 < K, side = sg.k1 > 0;
                 Acc<NT, WIDE> s = {};
                 Side o = {};
-                sweep<NT, WIDE, S_DEVICE>(a, c, th, sm, tbt, lv, sg.pa, sg.pb, 0u, false, false, false, race, side, s, o);
+                sweep<NT, WIDE, S_DEVICE>(a, c, th, sm, tbt, lv, sg.pa, sg.pb, 0u, false, false, race, side, s, o);
                 if (race) share_out<NT, WIDE>(sm, s, lv, turn);
                 if (side) share_side<NT, WIDE>(sm, o, turn);
                 __syncthreads();
@@ -881,7 +881,7 @@ k_grid(const __grid_constant__ Args a) {
             auto run = [&](uint32_t pa, uint32_t pb, uint32_t w, bool list, bool push, int q0, int q1, bool neg) {
                 Acc<NT, WIDE> s = {};
                 Side none = {};
-                sweep<NT, WIDE, S_NONE>(a, c, th, sm, tbt, lv, pa, pb, w, list, push, false, true, false, s, none);
+                sweep<NT, WIDE, S_NONE>(a, c, th, sm, tbt, lv, pa, pb, w, list, push, true, false, s, none);
                 share_out<NT, WIDE>(sm, s, lv, turn);
                 __syncthreads();
                 enter<NT, WIDE>(sm, tbt, tb, g, q0, q1, neg, turn);
@@ -926,8 +926,9 @@ k_grid(const __grid_constant__ Args a) {
                 }
             }
         } else if constexpr (MODE == M_WAITS) {
-            // Segment by segment: each column of [k1, k2) under its own w*; then [k2, K), which waits 0, in one sweep with [0, k1), where the
-            // device runs alone or (Algorithm 2) waits w_tail.  The few requests that w_tail does not cover have been listed.  A handful is
+            // Algorithm 2, segment by segment: each column of [k1, k2) under its own w*; then [k2, K), which waits 0, in one sweep with [0, k1),
+            // which waits w_tail.  (Groups of Algorithm 3 have the way above: with one for both 300,000 requests of six groups under 32 policies took
+            // 26.1 us instead of 24.8, 600,000 under 32 by 2 30.0 instead of 28.4, 2 M under 64 by 2 48.8 instead of 47.0.)  The few requests that w_tail does not cover have been listed.  A handful is
             // entered request by request; more are entered for [0, k1) from the list, and when it is half full or the chunk is done,
             // the columns that wait longer get what they come to there under their own wait in place of the common one.
             enum { POINTS, MAIN, LISTED, LONGER } at = POINTS;
@@ -945,14 +946,14 @@ k_grid(const __grid_constant__ Args a) {
                         continue;
                     }
                     const Seg sg = sm.seg[si];
-                    if (ri >= (int)sg.k2 - (int)sg.k1 || !waits) { at = MAIN; pos = sg.pa; continue; }
+                    if (ri >= (int)sg.k2 - (int)sg.k1) { at = MAIN; pos = sg.pa; continue; }
                     from = sg.pa; to = sg.pb; q0 = (int)sg.k1 + ri; q1 = q0 + 1; w = sm.w_star[q0];
                     ++ri;
                 } else if (at == MAIN) {
                     const Seg sg = sm.seg[min(si, kMaxSeg - 1)];
                     const bool race = (int)sg.k2 < K, side = sg.k1 > 0;
                     if (pos >= sg.pb || !(race || side)) { at = POINTS; ri = 0; ++si; continue; }
-                    if (!side || (waits && !race && n_low == 0)) {
+                    if (!side || (!race && n_low == 0)) {
                         // no two runs to sweep at once, and no column that wants the list: a run of its own, without one (six groups under one policy,
                         // evaluation and reduction: 100,000 requests 39.4 us -> 38.1, a million 57.9 -> 57.0, under 1 by 8 300,000 51.1 -> 48.9)
                         from = sg.pa; to = sg.pb;
@@ -962,18 +963,16 @@ k_grid(const __grid_constant__ Args a) {
                         Acc<NT, WIDE> s = {};
                         Side o = {};
                         for (;;) {
-                            uint32_t end = sg.pb;
-                            if (waits && side) end = min(end, pos + list_room(n_list));
-                            sweep<NT, WIDE, S_EITHER>(a, c, th, sm, tbt, lv, pos, end, wt_min, false, false, waits, race, side, s, o);
+                            const uint32_t end = min((uint32_t)sg.pb, pos + list_room(n_list));
+                            sweep<NT, WIDE, S_SERVER>(a, c, th, sm, tbt, lv, pos, end, wt_min, false, false, race, true, s, o);
                             pos = end;
-                            if (!waits || !side) break;
                             __syncthreads();
                             n_list = sm.n_list;
                             __syncthreads();
                             if (pos >= sg.pb || list_room(n_list) == 0u) break;
                         }
                         if (race) share_out<NT, WIDE>(sm, s, lv, turn);
-                        if (side) share_side<NT, WIDE>(sm, o, turn);
+                        share_side<NT, WIDE>(sm, o, turn);
                         if constexpr (list_few(NT) != 0) {
                             if (n_list > listed && n_list - listed <= (uint32_t)list_few(NT)) {
                                 enter_listed<NT>(a, sm, listed, n_list, wt_min, n_low, sg.k1);
@@ -983,7 +982,7 @@ k_grid(const __grid_constant__ Args a) {
                         __syncthreads();
                         if (threadIdx.x == 0) sm.n_list = n_list;
                         if (race) enter<NT, WIDE>(sm, tbt, tb, g, sg.k2, K, false, turn);
-                        if (side) enter_side<NT, WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1, waits, turn);
+                        enter_side<NT, WIDE>(sm, tbt + NT * kNBins, tb, g, sg.k1, true, turn);
                         __syncthreads();
                         ++passes; turn ^= 1;
                         if (n_list > listed) at = LISTED;
@@ -1003,7 +1002,7 @@ k_grid(const __grid_constant__ Args a) {
                 }
                 Acc<NT, WIDE> s = {};
                 Side none = {};
-                sweep<NT, WIDE, S_NONE>(a, c, th, sm, tbt, lv, from, to, w, list, false, false, true, false, s, none);
+                sweep<NT, WIDE, S_NONE>(a, c, th, sm, tbt, lv, from, to, w, list, false, true, false, s, none);
                 share_out<NT, WIDE>(sm, s, lv, turn);
                 __syncthreads();
                 if (n_list == 0 && threadIdx.x == 0) sm.n_list = 0;
