@@ -216,15 +216,15 @@ assert load(ctx, 50000, cols) == 0 and fake.fake_last_zeroed() == 1, L.disco_las
 
 
 def test_evaluations_in_a_row_wait_for_their_own_stream_alone(fake):
-    # the tables of 1,024 policies lie in page-locked memory until a kernel has read them; other streams may be busy for long
+    # the tables of 2,048 policies lie in page-locked memory until a kernel has read them; other streams may be busy for long
     _run(fake, """
 fake.fake_device_waits.restype = C.c_uint64
 ctx = C.c_void_p(None)
 keep, cols = host_columns(5000)
 assert load(ctx, 5000, cols) == 0, L.disco_last_error()
-pols = api.policy_array([synth.policy(k / 1023) for k in range(1024)])
+pols = api.policy_array([synth.policy(k / 2047) for k in range(2048)])
 for turn in range(4):
-    assert L.disco_eval_policies(ctx, pols, 1024, 1, None, None) == 0, L.disco_last_error()
+    assert L.disco_eval_policies(ctx, pols, 2048, 1, None, None) == 0, L.disco_last_error()
     assert fake.fake_device_waits() == 0
 """)
 
