@@ -152,8 +152,12 @@ inline int64_t host_bin_edge_ticks(int b) {
 
 #ifdef __CUDACC__
 // Launch that lets the grid be scheduled while its predecessor in the stream is still draining (programmatic
-// stream serialisation).  Every kernel launched this way calls grid_dependency_wait() before it reads or
-// writes global memory; the wait returns once the preceding grids have completed and their writes are visible.
+// stream serialisation).  grid_dependency_wait() returns once the predecessor has completed, its own waits included, and its writes are
+// visible.  The rule: a kernel waits before it reads or writes global memory -- unless all that it touches (what it reads, what it
+// writes and who else may write there) was complete before the blocks of its predecessor let it start; then at least one of its
+// blocks waits before it ends, and before it lets a successor start that needs the predecessor's results.  So a kernel's completion
+// always means that of all in front of it.  Who goes in front of its wait, and why it may, is said at each such kernel: k_prep, k_ticks, k_order,
+// k_sort, k_grid, k_spread, k_playout_free.
 template <class... KArgs, class... Args>
 inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                 Args&&... args) {
@@ -167,7 +171,8 @@ inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block,
 }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the stream start once every block of this one has come here (or ended); what it may do in front of
-// its own wait is up to it.  To be called behind this kernel's wait.
+// its own wait is up to it.  To be called behind this kernel's wait, or where the successor touches nothing that a kernel in front of this
+// one may still work on (k_order's other blocks, k_grid beside its predecessor).
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // add + ((h * mul) >> 32) in one instruction

@@ -311,14 +311,9 @@ __device__ __forceinline__ void sweep(const Args& a, const Ctx& c, const float (
         int t = 0;                                                    // rows that migrate: [0, t)
         if constexpr (kLevels) {
             if (saving > th[0]) {
-                static_assert(NT == 4 || NT == 8, "a search in steps of two and one, or four, two and one");
-                if constexpr (NT == 8) {
-                    const bool p4 = saving > th[4], p2 = saving > (p4 ? th[6] : th[2]);
-                    t = (p4 ? 5 : 1) + (p2 ? 2 : 0) + (saving > (p4 ? (p2 ? th[7] : th[5]) : (p2 ? th[3] : th[1])) ? 1 : 0);
-                } else {
-                    const bool p2 = saving > th[2];
-                    t = (p2 ? 3 : 1) + (saving > (p2 ? th[3] : th[1]) ? 1 : 0);
-                }
+                static_assert(NT == 8, "a search in steps of four, two and one");
+                const bool p4 = saving > th[4], p2 = saving > (p4 ? th[6] : th[2]);
+                t = (p4 ? 5 : 1) + (p2 ? 2 : 0) + (saving > (p4 ? (p2 ? th[7] : th[5]) : (p2 ? th[3] : th[1])) ? 1 : 0);
                 const int at = (t - 1) * 32 + lane;
                 uint2 v = lv.ab[at];
                 v.x += handed; v.y += refill;
@@ -1166,7 +1161,8 @@ DBG_TRANSLATION_UNIT()
 // 130,000 under 64 40 and 41, 220,000 under 256 62 and 58, 400,000 63 and 68; six groups, 60,000 under 2 36 and 49, under one 80,000 37 and 39,
 // 130,000 under 16 51 and 47, 220,000 53 and 55, 400,000 under 64 75 and 77, under 128 113 and 91, 550,000 101 and 117, 750,000 under 256 175 and 142,
 // 1.3 million 194 and 216, under 16 by 8 170,000 72 and 64, 400,000 74 and 86, under 128 by 8 750,000 174 and 172.  How fast the rows are
-// added to depends on where they lie -- 400,000 of six groups under 64 by 2 80 us or 97, run by run 80 --: the line lies in front of where both meet.)
+// added to depends on where they lie -- k_grid of 400,000 requests of six groups under 64 by 2 took 59 us in one context, run by run 44 there, and as
+// long as run by run in others --: the line lies in front of where both meet.)
 // It is asked slab by slab: a narrow grid beside a wide one goes its own way (six groups, a million requests under 256 by 4, and sixteen times 2 by 4
 // of other expected lengths, 779 us all side by side, now 484; under 256 by 4 and one 300, now 248; one group, 150,000 under 128 by 8 and eight
 // times 4 164, now 141).

@@ -1,5 +1,5 @@
 // Trace ingestion on the device in one kernel, for the traces that load_once.cu and load_large.cu do not take (1.2 to 2.2 million
-// requests, more than seven groups, beyond 2^24 requests, or without room for load_large.cu's buckets), and the sort of as many
+// requests, to 3.0 million where columns are read in place from page-locked memory, more than seven groups, beyond 2^24 requests, or without room for load_large.cu's buckets), and the sort of as many
 // ticks: tick conversion and validation, per-group prompt-length histogram, internal request order (by group, then by prompt
 // length), sort of the server-TTFT ticks (the empirical F of Algorithm 1), cumulative input-token mass (Eq. 3) and the quantile
 // knots of F.
