@@ -24,9 +24,9 @@
 // (three additions a row), or, with eight rows, to the last of them; the hand-off stall is counted at the level of the last such
 // row, and the levels are summed up when the run is entered.
 //
-// Bound: integer issue, and a run's latency.  16 M requests in six groups under 128 budgets by 8 overheads: 347 us with a sweep for
-// each run and every row's sums in registers (122 of them, two blocks to a multiprocessor), 247 now (80, three); 5 M under 40 by 8
-// 113 -> 85; a million in one group under 256 by 4 32 -> 28.  (Kernels that also held the way of small traces had to spill: 283 and 99.)
+// Bound: a run's barriers and its latency, then integer issue (half of the slots).  16 M requests in six groups under 128 budgets by 8
+// overheads: 347 us with a sweep for each run and every row's sums in registers (122 of them, two blocks to a multiprocessor), 240 now
+// (80, three); 5 M under 40 by 8 113 -> 85; a million in one group under 256 by 4 32 -> 28.  (Kernels that also held the way of small traces had to spill: 283 and 99.)
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
