@@ -430,6 +430,17 @@ def test_policies_of_many_kinds(kinds):
     full_parity(w, pols + pols[::2], select=False, tag=f"{kinds}")
 
 
+@pytest.mark.parametrize("n", [5000, 30_001, 60_001])
+@pytest.mark.parametrize("shape", [(1, 1), (2, 3)])
+def test_narrow_grids_beside_wide_ones(n, shape):
+    # a wide grid goes side by side, narrow ones run by run, and between them one whose overheads differ by budget (either): all in one
+    # evaluation, with chunks of their own
+    w = synth.tiny_workload(179 + n, n, n_servers=shape[0], n_devices=shape[1], max_prompt=700, max_out=40, device_dearer=True)
+    of = lambda columns, rows, E: [synth.policy(b, flags=PACED, mig_threshold=1e-6 * k, expected_len=E) for b in synth.budget_grid(columns) for k in range(rows)]
+    by_budget = [synth.policy(b, flags=PACED, mig_threshold=1e-6 * k, expected_len=3) for k, b in enumerate(synth.budget_grid(9))]
+    full_parity(w, of(2, 1, 5) + of(48, 1, 0) + by_budget + of(2, 3, 7) + of(20, 3, 9) + of(1, 1, 11), select=False, tag=f"{n} {shape}")
+
+
 @pytest.mark.parametrize("rate", [5.0, 40.0])
 @pytest.mark.parametrize("rows", [1, 2])
 def test_lists_that_fill_within_a_segment(rate, rows):
