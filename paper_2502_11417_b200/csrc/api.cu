@@ -876,7 +876,9 @@ int disco_eval_policies(disco_ctx_t* c, const disco_policy_t* pol, uint32_t P, u
 #ifdef DISCO_DEBUG
         if (std::getenv("DISCO_DEBUG_RUNS")) return false;
 #endif
-        return !wide_class(sl.cls) && grid_joins(n, groups, sl.K, sl.T);
+        bool inner = false;                                          // some budget parts the requests (0 and 1 do not)
+        for (int x = 0; x < sl.K && !inner; ++x) { const float b = pc[tab[sl.cols + x]].budget; inner = b > 0.0f && b < 1.0f; }
+        return !wide_class(sl.cls) && grid_joins(n, groups, sl.K, sl.T, inner);
     };
     for (size_t x = 0, end; x < slabs.size(); x = end) {
         auto like = [&](const Slab& sl) { return sl.cls / wave == slabs[x].cls / wave && wide_class(sl.cls) == wide_class(slabs[x].cls); };

@@ -327,7 +327,7 @@ struct GridTables { uint32_t* ttft; void* tbt; unsigned long long* sums; };
 struct LeftLists { uint32_t* list; uint32_t* count; };   // [slabs][n] places in the internal order, [slabs][G]
 uint64_t grid_ttft_words(int K), grid_tbt_words(int K, int T), grid_sum_words(int K, int T, int G);
 uint32_t grid_blocks_per_sm(int T);
-bool grid_joins(uint32_t n, int groups /* that have requests */, int K, int T);   // small traces under many policies: requests side by side
+bool grid_joins(uint32_t n, int groups /* that have requests */, int K, int T, bool inner /* a budget lies between 0 and 1 */);   // small traces under many policies: requests side by side
 int grid_rows(int T);            // rows the kernel that takes such a slab is built for
 cudaError_t launch_grid(const TraceDev& tr, const GroupConst* gc, const ClassConst* classes, const Prep* prep, uint32_t P,
                         const Slab* slabs, uint32_t n_slabs, int T /* most rows of a slab */, bool wide /* of all of them */,

@@ -1157,8 +1157,8 @@ DBG_TRANSLATION_UNIT()
 
 // Side by side or run by run.  Run by run a threshold of a group costs a run's latency, in the chunks that it falls into; side by side the
 // requests add to the same rows of the tables, two runs each (under one policy setting one), and the fewer columns there are the more
-// of them meet.  (Evaluation and reduction, us, run by run and side by side: one group, 60,000 requests under 2 policies 31 and 40, under 4 34 and 36,
-// 130,000 under 64 40 and 41, 220,000 under 256 62 and 58, 400,000 63 and 68; six groups, 60,000 under 2 36 and 49, under one 80,000 37 and 39,
+// of them meet.  (Evaluation and reduction, us, run by run and side by side: one group, 60,000 requests under budgets of 0 and 1 31 and 40, under 4 34 and 36,
+// 130,000 under 64 40 and 41, 220,000 under 256 62 and 58, 400,000 63 and 68; six groups, 60,000 under 0 and 1 36 and 49, under one 80,000 37 and 39,
 // 130,000 under 16 51 and 47, 220,000 53 and 55, 400,000 under 64 75 and 77, under 128 113 and 91, 550,000 101 and 117, 750,000 under 256 175 and 142,
 // 1.3 million 194 and 216, under 16 by 8 170,000 72 and 64, 400,000 74 and 86, under 128 by 8 750,000 174 and 172.  How fast the rows are
 // added to depends on where they lie -- k_grid of 400,000 requests of six groups under 64 by 2 took 59 us in one context, run by run 44 there, and as
@@ -1166,7 +1166,10 @@ DBG_TRANSLATION_UNIT()
 // It is asked slab by slab: a narrow grid beside a wide one goes its own way (six groups, a million requests under 256 by 4, and sixteen times 2 by 4
 // of other expected lengths, 779 us all side by side, now 484; under 256 by 4 and one 300, now 248; one group, 150,000 under 128 by 8 and eight
 // times 4 164, now 141).
-bool grid_joins(uint32_t n, int groups, int K, int T) { return n <= (K == 1 ? 60000.0 : 10000.0 * std::pow((double)K * groups, 0.6)) * (1.0 + T / 16.0); }
+// Budgets of 0 and 1 alone part no requests: a chunk is one run or two, and side by side all requests meet in the same rows.
+bool grid_joins(uint32_t n, int groups, int K, int T, bool inner) {
+    return n <= (K == 1 ? 60000.0 : !inner ? 16000.0 : 10000.0 * std::pow((double)K * groups, 0.6)) * (1.0 + T / 16.0);
+}
 uint64_t grid_ttft_words(int K) { return (uint64_t)K * kNBins; }
 uint64_t grid_tbt_words(int K, int T) { return (uint64_t)K * T * kNBins; }
 uint64_t grid_sum_words(int K, int T, int G) { return (uint64_t)G * K * sum_fields(T); }

@@ -278,7 +278,8 @@ for reset in (False, False, True, False, True):
 
 
 @pytest.mark.parametrize("n,policies,runs,joined", [
-    (10_000, "grid(2)", 0, 1), (60_000, "grid(2)", 1, 0),             # few columns: side by side up to some 20,000 requests
+    (10_000, "grid(2)", 0, 1), (18_000, "grid(2)", 1, 0), (60_000, "grid(2)", 1, 0),     # budgets of 0 and 1 part no requests
+    (24_000, "grid(2) * 4", 1, 0), (24_000, "grid(8)", 0, 1), (24_000, "grid(4)", 0, 1), (25_000, "grid(4)", 1, 0),
     (60_000, "grid(1)", 0, 1), (90_000, "grid(1)", 1, 0),             # one: a run a request
     (150_000, "grid(256, 4)", 0, 1), (500_000, "grid(256, 4)", 1, 0),
     # a wide grid and narrow ones beside it: each its own way, in the same launch where the ways are the same
